@@ -99,11 +99,16 @@ struct RefWeights {            // fp32 device copies in PyTorch layouts
     float *whead, *bhead;      // [A+1,512], [A+1]: policy rows then the value row
 };
 struct RefWorkspace { float *a1, *a2, *a3, *h; };   // NCHW fp32 activations, [n,512]
+struct RefPlanes {             // the hidden convolution outputs once more, as three bf16 planes of pixel-major rows
+    __nv_bfloat16 *a1, *a2, *a3;
+    size_t p1, p2, p3;         // elements between planes
+};
 
 hts_status ref_convert_weights(const Geometry& g, int dtype, const hts_weights& src,
                                const RefWeights& dst, cudaStream_t s);
 hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspace& ws,
-                       const uint8_t* obs, const Indexing& ix, int* status, int n, Profiler& prof, cudaStream_t s);
+                       const uint8_t* obs, const Indexing& ix, int* status, int n, Profiler& prof, cudaStream_t s,
+                       const RefPlanes* planes = nullptr);
 
 // ---- gradient of the learner objective on the fp32 path (backward.cu) ---------------------------
 constexpr int kBackwardChunks = 64;      // batch chunks whose partial weight gradients are added in index order
