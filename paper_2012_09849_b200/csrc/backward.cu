@@ -6,295 +6,597 @@
 // S_i = log pi(a_i|s_i) A_i (actor-critic; the advantage is data) or the clipped surrogate
 // min(rho_i A_i, clip(rho_i, 1-clip, 1+clip) A_i), rho_i = exp(log pi(a_i|s_i) - logp_old_i) (PPO).
 //
-// fp32 CUDA-core kernels on the activations of the fp32 check path (NCHW), layer by layer through the network
-// of Appendix F.1 / F.2.  Every sum runs in a fixed order (no atomics): weight gradients of the convolutions
-// are summed per batch chunk and the chunks are then added in index order.  These kernels are written for
-// correctness and a reproducible result, not tuned: they are not part of the actor's hot path.
+// The forward pass is that of the fp32 actor step: a ReLU passes the gradient exactly where the step's output is
+// positive.  The data and weight gradients of the four hidden layers run on the tensor cores at fp32 accuracy
+// (x3_gemm.cuh); the two heads, less than half a percent of the work, are fp32 CUDA-core kernels.
+// Every sum runs in an order fixed by the batch size (no atomics): a weight gradient is summed per range of rows and
+// the ranges are then added in index order.
+#include <new>
 #include "common.cuh"
+#include "x3_gemm.cuh"
 
 namespace hts {
 namespace {
 
-constexpr int kOTile = 8;       // outputs per thread in the dense weight gradient
+typedef __nv_bfloat16 bf16;
 
-// d J / d logits and d J / d value of each sample.  dhead[i][0..A-1] = d/d logit_j, dhead[i][A] = d/d V.
-__global__ void head_grad_kernel(const float* __restrict__ logits, const float* __restrict__ values,
-                                 const int32_t* __restrict__ actions, const float* __restrict__ adv,
-                                 const float* __restrict__ ret, const float* __restrict__ logp_old, float value_coef,
-                                 float entropy_coef, float clip, int n, int A, int* __restrict__ status,
-                                 float* __restrict__ dhead)
+// ---- frames as the first convolution's operand -----------------------------------------------------------------
+// uint8 [n,C,H,W] -> bf16 [n * (H/4)(W/4)][16 Cp], column c*16 + uy*4 + ux = x[c][4Y+uy][4X+ux] (a byte is exact);
+// Cp = C rounded up to a multiple of 4, the added channels are zero.
+__global__ void __launch_bounds__(256)
+frames_kernel(const uint8_t* __restrict__ obs, int C, int Cp, int H, int W, size_t items, bool words, bf16* __restrict__ x0)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float* lg = logits + (size_t)i * A;
-    float* out = dhead + (size_t)i * (A + 1);
-    const int a = actions[i];
-    if ((unsigned)a >= (unsigned)A) {                    // not used as an index: the row contributes nothing
-        if (status) atomicCAS(status, 0, kStatusBadAction);
-        for (int j = 0; j <= A; ++j) out[j] = 0.f;
+    pdl_wait();
+    pdl_trigger();
+    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;       // (position, channel), channel fastest
+    if (idx >= items) return;
+    const int c = (int)(idx % Cp);
+    const size_t pos = idx / Cp;
+    const int W0 = W / 4, G0 = W0 * (H / 4);
+    const size_t e = pos / G0;
+    const int cell = (int)(pos - e * G0), Y = cell / W0, X = cell - Y * W0;
+    uint32_t out[8];
+#pragma unroll
+    for (int uy = 0; uy < 4; ++uy) {
+        uint32_t w = 0;
+        if (c < C) {
+            const uint8_t* src = obs + ((e * C + c) * H + 4 * Y + uy) * W + 4 * X;
+            if (words) w = *reinterpret_cast<const uint32_t*>(src);
+            else w = src[0] | (uint32_t)src[1] << 8 | (uint32_t)src[2] << 16 | (uint32_t)src[3] << 24;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float lo = (float)((w >> (16 * h)) & 0xffu), hi = (float)((w >> (16 * h + 8)) & 0xffu);
+            out[2 * uy + h] = (__float_as_uint(lo) >> 16) | (__float_as_uint(hi) & 0xffff0000u);
+        }
+    }
+    uint4* dst = reinterpret_cast<uint4*>(x0 + idx * 16);
+    dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
+    dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
+}
+
+// ---- fp32 weights as three bf16 planes in the layouts of the contractions ---------------------------------------
+//   w2p [3][64][tap * 128 + (uy*2+ux)*32 + c]    value w2[o][c][2dy+uy][2dx+ux]
+//   w3p [3][64][tap * 64 + c]                    value w3[o][c][dy][dx]
+//   wfp [3][512][pixel * 64 + c]                 value wfc[o][c * P3 + pixel]
+__device__ __forceinline__ void put3(bf16* dst, size_t plane, size_t i, float v)
+{
+    uint32_t a, b, c;
+    x3_split2(v, 0.f, a, b, c);
+    uint16_t* d = reinterpret_cast<uint16_t*>(dst);
+    d[i] = (uint16_t)a; d[plane + i] = (uint16_t)b; d[2 * plane + i] = (uint16_t)c;
+}
+constexpr int kPackFloats = 8192;
+// Blocks 0..511 turn one row of the dense layer each through shared memory; the rest take the convolutions.
+__global__ void __launch_bounds__(256)
+pack_x3_kernel(const float* __restrict__ w2, const float* __restrict__ w3, const float* __restrict__ wf, int P3,
+               bf16* __restrict__ w2p, bf16* __restrict__ w3p, bf16* __restrict__ wfp)
+{
+    __shared__ float s_row[kPackFloats];
+    const int F = 64 * P3;
+    if (blockIdx.x < 512) {
+        const int o = blockIdx.x;
+        const int cstep = P3 > kPackFloats ? 1 : kPackFloats / P3 > 64 ? 64 : kPackFloats / P3;      // channels per pass
+        for (int c0 = 0; c0 < 64; c0 += cstep) {
+            const int nc = c0 + cstep > 64 ? 64 - c0 : cstep;
+            const float* src = wf + (size_t)o * F + (size_t)c0 * P3;
+            if (P3 <= kPackFloats) {
+                for (int i = threadIdx.x; i < nc * P3; i += 256) s_row[i] = src[i];
+                __syncthreads();
+                src = s_row;
+            }
+            for (int i = threadIdx.x; i < nc * P3; i += 256) {
+                const int pix = i / nc, c = i - pix * nc;
+                put3(wfp, (size_t)512 * F, (size_t)o * F + (size_t)pix * 64 + c0 + c, src[c * P3 + pix]);
+            }
+            __syncthreads();
+        }
         return;
     }
-    float m = -INFINITY;
-    for (int j = 0; j < A; ++j) m = fmaxf(m, lg[j]);
-    float z = 0.f;
-    for (int j = 0; j < A; ++j) z += expf(lg[j] - m);
-    const float lse = m + logf(z);
-    float ent = 0.f;
-    for (int j = 0; j < A; ++j) { const float lp = lg[j] - lse; ent -= expf(lp) * lp; }
-    const float inv_n = 1.0f / (float)n;
-    float ds = adv[i];                                   // d S_i / d log pi(a_i)
-    if (logp_old && clip > 0.f) {
-        const float rho = expf((lg[a] - lse) - logp_old[i]);
-        const float clipped = fminf(fmaxf(rho, 1.f - clip), 1.f + clip);
-        ds = (rho * adv[i] <= clipped * adv[i]) ? rho * adv[i] : 0.f;       // the min takes its first argument
+    int i = (blockIdx.x - 512) * 256 + threadIdx.x;
+    if (i < 64 * 512) {
+        const int o = i >> 9, k = i & 511, tap = k >> 7, cp = k & 127;
+        const int dy = tap >> 1, dx = tap & 1, uy = cp >> 6, ux = (cp >> 5) & 1, c = cp & 31;
+        put3(w2p, 64 * 512, i, w2[((o * 32 + c) * 4 + 2 * dy + uy) * 4 + 2 * dx + ux]);
+        return;
     }
-    for (int j = 0; j < A; ++j) {
-        const float lp = lg[j] - lse, p = expf(lp);
-        // d log pi(a) / d logit_j = [j == a] - p_j ;   d H / d logit_j = -p_j (log p_j + H)
-        out[j] = (ds * ((j == a ? 1.f : 0.f) - p) - entropy_coef * p * (lp + ent)) * inv_n;
-    }
-    out[A] = 2.f * value_coef * (ret[i] - values[i]) * inv_n;
-}
-
-// dW[o][k] = sum_i dout[i][o] * in[i][k]   (dout [n][ldo], in [n][K]);  thread = (k, tile of kOTile outputs)
-__global__ void dense_wgrad_kernel(const float* __restrict__ dout, int ldo, int O, const float* __restrict__ in, int K,
-                                   int n, float* __restrict__ dW)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int o0 = blockIdx.y * kOTile;
-    if (k >= K) return;
-    float acc[kOTile];
-#pragma unroll
-    for (int j = 0; j < kOTile; ++j) acc[j] = 0.f;
-    for (int i = 0; i < n; ++i) {
-        const float x = in[(size_t)i * K + k];
-        const float* d = dout + (size_t)i * ldo + o0;
-#pragma unroll
-        for (int j = 0; j < kOTile; ++j) if (o0 + j < O) acc[j] = fmaf(d[j], x, acc[j]);
-    }
-#pragma unroll
-    for (int j = 0; j < kOTile; ++j) if (o0 + j < O) dW[(size_t)(o0 + j) * K + k] = acc[j];
-}
-
-// db[o] = sum_i dout[i][o]
-__global__ void dense_bgrad_kernel(const float* __restrict__ dout, int ldo, int O, int n, float* __restrict__ db)
-{
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= O) return;
-    float acc = 0.f;
-    for (int i = 0; i < n; ++i) acc += dout[(size_t)i * ldo + o];
-    db[o] = acc;
-}
-
-// din[i][k] = (act[i][k] > 0) * sum_o dout[i][o] * W[o][k]     (the ReLU of the layer that produced act)
-__global__ void dense_dgrad_kernel(const float* __restrict__ dout, int ldo, int O, const float* __restrict__ W, int K,
-                                   const float* __restrict__ act, int n, float* __restrict__ din)
-{
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (size_t)n * K) return;
-    const int k = (int)(idx % K);
-    const size_t i = idx / K;
-    float acc = 0.f;
-    if (act[idx] > 0.f) {
-        const float* d = dout + i * ldo;
-        for (int o = 0; o < O; ++o) acc = fmaf(d[o], W[(size_t)o * K + k], acc);
-    }
-    din[idx] = acc;
-}
-
-// Partial weight and bias gradients of a convolution over one chunk of the batch:
-//   part[chunk][p]  p < O C k k : sum_{i in chunk, y, x} dy[i][o][y][x] * in[i][c][y s + u][x s + v]
-//                   p >= O C k k: bias o = p - O C k k : sum dy[i][o][y][x]
-// A thread owns one (c, u, v) and kWgradOB output channels: one input load feeds that many independent
-// accumulators (the dy loads are the same address across most of a warp).  Each element is still summed over
-// (i, y, x) in ascending order.
-constexpr int kWgradOB = 8;
-template <typename TIn>
-__global__ void conv_wgrad_kernel(const float* __restrict__ dy, const TIn* __restrict__ in, int n, int C, int H, int W,
-                                  int O, int k, int s, int Ho, int Wo, int per_chunk, float* __restrict__ part)
-{
-    const int per_o = C * k * k, nW = O * per_o, total = nW + O;
-    const int nT = nW / kWgradOB;                      // threads that own weights; O more own one bias each
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= nT + O) return;
-    const int i0 = blockIdx.y * per_chunk;
-    int i1 = i0 + per_chunk; i1 = i1 > n ? n : i1;
-    float* out = part + (size_t)blockIdx.y * total;
-    const size_t plane = (size_t)Ho * Wo;
-    if (q < nT) {
-        const int r = q % per_o, o0 = (q / per_o) * kWgradOB;
-        const int v = r % k, u = (r / k) % k, c = r / (k * k);
-        float acc[kWgradOB];
-#pragma unroll
-        for (int j = 0; j < kWgradOB; ++j) acc[j] = 0.f;
-        for (int i = i0; i < i1; ++i) {
-            const float* d = dy + ((size_t)i * O + o0) * plane;
-            const TIn* x = in + ((size_t)i * C + c) * H * W + (size_t)u * W + v;
-            for (int y = 0; y < Ho; ++y)
-                for (int xx = 0; xx < Wo; ++xx) {
-                    const float xv = (float)x[(size_t)(y * s) * W + xx * s];
-#pragma unroll
-                    for (int j = 0; j < kWgradOB; ++j) acc[j] = fmaf(d[j * plane + y * Wo + xx], xv, acc[j]);
-                }
-        }
-#pragma unroll
-        for (int j = 0; j < kWgradOB; ++j) out[(size_t)(o0 + j) * per_o + r] = acc[j];
-    } else {
-        const int o = q - nT;
-        float acc = 0.f;
-        for (int i = i0; i < i1; ++i) {
-            const float* d = dy + ((size_t)i * O + o) * plane;
-            for (int t = 0; t < Ho * Wo; ++t) acc += d[t];
-        }
-        out[nW + o] = acc;
+    i -= 64 * 512;
+    if (i < 64 * 576) {
+        const int o = i / 576, k = i - o * 576, tap = k >> 6, c = k & 63;
+        put3(w3p, 64 * 576, i, w3[(o * 64 + c) * 9 + tap]);
     }
 }
 
-// dW / db = in_scale * (chunk partials added in index order)
-__global__ void conv_wgrad_reduce_kernel(const float* __restrict__ part, int chunks, int nW, int O, float in_scale,
-                                         float* __restrict__ dW, float* __restrict__ db)
+// ---- heads ---------------------------------------------------------------------------------------------------
+__device__ __forceinline__ float warp_sum(float v)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    const int total = nW + O;
-    if (p >= total) return;
-    float acc = 0.f;
-    for (int b = 0; b < chunks; ++b) acc += part[(size_t)b * total + p];
-    if (p < nW) dW[p] = acc * in_scale; else db[p - nW] = acc;
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
+    return v;
 }
 
-// dx[i][c][Y][X] = (x[i][c][Y][X] > 0) * sum_{o,u,v : Y = y s + u, X = x s + v} dy[i][o][y][x] * w[o][c][u][v]
-// A thread owns one input position and kDgradCB channels: every dy value it loads feeds that many independent
-// accumulators, and the block's slice of the filter sits in shared memory as [u][v][o][channel], so the inner loop
-// is one global load and two shared 16-byte loads per eight multiply-adds.  Taps are visited in ascending (u, v),
-// outputs in ascending o: the order of the sum of one element does not depend on the blocking.
-constexpr int kDgradCB = 8;
+// One warp per sample: d J / d logits and d J / d value (dhead[i][0..A-1], dhead[i][A]), then the gradient of the
+// hidden layer, dh[i][k] = (h[i][k] > 0) * sum_o dhead[i][o] whead[o][k], as three planes [n][512].
 __global__ void __launch_bounds__(256)
-conv_dgrad_kernel(const float* __restrict__ dy, const float* __restrict__ w, const float* __restrict__ x,
-                  int n, int C, int H, int W, int O, int k, int s, int Ho, int Wo, float* __restrict__ dx)
+head_backward_kernel(const float* __restrict__ logits, const float* __restrict__ values, const int32_t* __restrict__ actions,
+                     const float* __restrict__ adv, const float* __restrict__ ret, const float* __restrict__ logp_old,
+                     const float* __restrict__ whead, const float* __restrict__ h, float value_coef, float entropy_coef,
+                     float clip, int n, int A, int* __restrict__ status, float* __restrict__ dhead, bf16* __restrict__ dh,
+                     size_t dh_plane)
 {
-    extern __shared__ float4 s_w4[];                   // [k*k][O][kDgradCB]
-    float* s_w = reinterpret_cast<float*>(s_w4);
-    const int c0 = blockIdx.y * kDgradCB;
-    for (int idx = threadIdx.x; idx < k * k * O * kDgradCB; idx += blockDim.x) {
-        const int cc = idx % kDgradCB, o = (idx / kDgradCB) % O, t = idx / (kDgradCB * O);
-        const int c = c0 + cc;
-        s_w[idx] = c < C ? w[((size_t)o * C + c) * k * k + t] : 0.f;
-    }
+    extern __shared__ float4 s_w4[];                    // [A+1][512] head weights
+    __shared__ float s_d[8][65];
+    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < (A + 1) * 128; i += 256) s_w4[i] = reinterpret_cast<const float4*>(whead)[i];
+    pdl_wait();
+    pdl_trigger();
     __syncthreads();
-    const size_t pos = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (pos >= (size_t)n * H * W) return;
-    const int X = (int)(pos % W), Y = (int)((pos / W) % H);
-    const size_t i = pos / ((size_t)W * H);
-    float acc[kDgradCB];
+    const float inv_n = 1.0f / (float)n;
+    for (int i = blockIdx.x * 8 + wib; i < n; i += gridDim.x * 8) {
+        const int a = actions[i];
+        const bool bad = (unsigned)a >= (unsigned)A;     // not used as an index: the row contributes nothing
+        if (bad && lane == 0 && status) atomicCAS(status, 0, kStatusBadAction);
+        float lg[2];
 #pragma unroll
-    for (int cc = 0; cc < kDgradCB; ++cc) acc[cc] = 0.f;
-    const size_t plane = (size_t)Ho * Wo;
-    for (int u = Y % s; u < k && u <= Y; u += s) {
-        const int y = (Y - u) / s;
-        if (y >= Ho) continue;
-        for (int v = X % s; v < k && v <= X; v += s) {
-            const int xo = (X - v) / s;
-            if (xo >= Wo) continue;
-            const float* d = dy + i * O * plane + (size_t)y * Wo + xo;
-            const float4* wp = s_w4 + (size_t)(u * k + v) * O * (kDgradCB / 4);
-#pragma unroll 4
-            for (int o = 0; o < O; ++o) {
-                const float dv = d[(size_t)o * plane];
-                const float4 w0 = wp[2 * o], w1 = wp[2 * o + 1];
-                acc[0] = fmaf(dv, w0.x, acc[0]); acc[1] = fmaf(dv, w0.y, acc[1]);
-                acc[2] = fmaf(dv, w0.z, acc[2]); acc[3] = fmaf(dv, w0.w, acc[3]);
-                acc[4] = fmaf(dv, w1.x, acc[4]); acc[5] = fmaf(dv, w1.y, acc[5]);
-                acc[6] = fmaf(dv, w1.z, acc[6]); acc[7] = fmaf(dv, w1.w, acc[7]);
+        for (int k = 0; k < 2; ++k) lg[k] = lane + 32 * k < A ? logits[(size_t)i * A + lane + 32 * k] : -INFINITY;
+        float m = fmaxf(lg[0], lg[1]);
+#pragma unroll
+        for (int k = 16; k > 0; k >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, k));
+        float z = 0.f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) z += lane + 32 * k < A ? expf(lg[k] - m) : 0.f;
+        const float lse = m + logf(warp_sum(z));
+        float lp[2], p[2], ent = 0.f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const bool in = lane + 32 * k < A;
+            lp[k] = in ? lg[k] - lse : 0.f;
+            p[k] = in ? expf(lp[k]) : 0.f;
+            ent -= p[k] * lp[k];
+        }
+        ent = warp_sum(ent);
+        float ds = adv[i];                               // d S_i / d log pi(a_i)
+        if (logp_old && clip > 0.f && !bad) {
+            const float lpa = __shfl_sync(0xffffffffu, a < 32 ? lp[0] : lp[1], a & 31);
+            const float rho = expf(lpa - logp_old[i]);
+            const float clipped = fminf(fmaxf(rho, 1.f - clip), 1.f + clip);
+            ds = (rho * ds <= clipped * ds) ? rho * ds : 0.f;                  // the min takes its first argument
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int j = lane + 32 * k;
+            // d log pi(a) / d logit_j = [j == a] - p_j ;   d H / d logit_j = -p_j (log p_j + H)
+            if (j < A) s_d[wib][j] = bad ? 0.f : (ds * ((j == a ? 1.f : 0.f) - p[k]) - entropy_coef * p[k] * (lp[k] + ent)) * inv_n;
+        }
+        if (lane == 0) s_d[wib][A] = bad ? 0.f : 2.f * value_coef * (ret[i] - values[i]) * inv_n;
+        __syncwarp();
+        for (int j = lane; j <= A; j += 32) dhead[(size_t)i * (A + 1) + j] = s_d[wib][j];
+        float acc[16];                                   // hidden units 128*q + 4*lane + {0..3}
+#pragma unroll
+        for (int k = 0; k < 16; ++k) acc[k] = 0.f;
+        for (int o = 0; o <= A; ++o) {
+            const float d = s_d[wib][o];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 w = s_w4[o * 128 + 32 * q + lane];
+                acc[4 * q] = fmaf(d, w.x, acc[4 * q]); acc[4 * q + 1] = fmaf(d, w.y, acc[4 * q + 1]);
+                acc[4 * q + 2] = fmaf(d, w.z, acc[4 * q + 2]); acc[4 * q + 3] = fmaf(d, w.w, acc[4 * q + 3]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 hv = reinterpret_cast<const float4*>(h + (size_t)i * 512)[32 * q + lane];
+            uint2 pl[3];
+            x3_split2(hv.x > 0.f ? acc[4 * q] : 0.f, hv.y > 0.f ? acc[4 * q + 1] : 0.f, pl[0].x, pl[1].x, pl[2].x);
+            x3_split2(hv.z > 0.f ? acc[4 * q + 2] : 0.f, hv.w > 0.f ? acc[4 * q + 3] : 0.f, pl[0].y, pl[1].y, pl[2].y);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) reinterpret_cast<uint2*>(dh + k * dh_plane + (size_t)i * 512)[32 * q + lane] = pl[k];
+        }
+        __syncwarp();
+    }
+}
+
+// Partial sums over a range of samples: row o <= A of the block's tile of outputs is sum_i dhead[i][o] h[i][k], row
+// A + 1 is sum_i dh[i][k] (the dense bias); the head biases sum_i dhead[i][o] follow the 512 columns.
+//   part [range][A + 2][513]
+constexpr size_t kHeadRanges = 18;
+constexpr int kHeadTile = 11;                            // outputs per block
+__global__ void __launch_bounds__(256)
+head_wgrad_kernel(const float* __restrict__ dhead, const float* __restrict__ h, const bf16* __restrict__ dh, size_t dh_plane,
+                  int n, int A, int per_range, float* __restrict__ part)
+{
+    __shared__ float s_acc[4][64];
+    const int k = blockIdx.x * 64 + (threadIdx.x & 63), sub = threadIdx.x >> 6;
+    const int o0 = blockIdx.z * kHeadTile;
+    const int i0 = blockIdx.y * per_range, i1 = min(n, i0 + per_range);
+    pdl_wait();
+    pdl_trigger();
+    float acc[kHeadTile];
+#pragma unroll
+    for (int j = 0; j < kHeadTile; ++j) acc[j] = 0.f;
+    for (int i = i0 + sub; i < i1; i += 4) {
+        const float x = h[(size_t)i * 512 + k];
+        const float* d = dhead + (size_t)i * (A + 1) + o0;
+#pragma unroll
+        for (int j = 0; j < kHeadTile; ++j) {
+            if (o0 + j <= A) acc[j] = fmaf(d[j], x, acc[j]);
+            else if (o0 + j == A + 1) {
+                const bf16* g = dh + (size_t)i * 512 + k;
+                acc[j] += __bfloat162float(g[0]) + (__bfloat162float(g[dh_plane]) + __bfloat162float(g[2 * dh_plane]));
             }
         }
     }
+    float* out = part + ((size_t)blockIdx.y * (A + 2) + o0) * 513 + blockIdx.x * 64;
 #pragma unroll
-    for (int cc = 0; cc < kDgradCB; ++cc) {
-        const int c = c0 + cc;
-        if (c < C) {
-            const size_t idx = ((i * C + c) * H + Y) * W + X;
-            dx[idx] = x[idx] > 0.f ? acc[cc] : 0.f;
-        }
+    for (int j = 0; j < kHeadTile; ++j) {
+        if (o0 + j >= A + 2) break;
+        s_acc[sub][threadIdx.x & 63] = acc[j];
+        __syncthreads();
+        if (threadIdx.x < 64) out[j * 513 + threadIdx.x] = (s_acc[0][threadIdx.x] + s_acc[1][threadIdx.x]) + (s_acc[2][threadIdx.x] + s_acc[3][threadIdx.x]);
+        __syncthreads();
     }
+    if (blockIdx.x == 0 && threadIdx.x < kHeadTile && o0 + threadIdx.x <= A) {
+        float t = 0.f;
+        for (int i = i0; i < i1; ++i) t += dhead[(size_t)i * (A + 1) + o0 + threadIdx.x];
+        part[((size_t)blockIdx.y * (A + 2) + o0 + threadIdx.x) * 513 + 512] = t;
+    }
+}
+
+// ---- sums over the ranges, in index order, into the caller's tensors -----------------------------------------------
+struct ReduceParams {
+    const float *c1, *c2, *c3, *b1, *b2, *b3, *head;     // partials
+    int r1, r2, r3, r3_last, rh;                         // ranges (r3_last: of conv3's last tap)
+    size_t g1, g2, g3;                                   // floats between group indices
+    int C, Cp, A;
+    hts_grads out;
+};
+__device__ __forceinline__ float sum_ranges(const float* p, int ranges, size_t stride)
+{
+    float acc = 0.f;
+    int r = 0;
+    for (; r + 8 <= ranges; r += 8) {
+        float v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = p[(size_t)(r + i) * stride];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc += v[i];
+    }
+    for (; r < ranges; ++r) acc += p[(size_t)r * stride];
+    return acc;
+}
+__global__ void __launch_bounds__(256) reduce_kernel(const ReduceParams p)
+{
+    pdl_wait();
+    pdl_trigger();
+    int i = blockIdx.x * 256 + threadIdx.x;
+    const int n3 = 5 * 8192, n2 = 4 * 8192, n1 = p.Cp / 2 * 4096, nh = (p.A + 2) * 513;
+    if (i < n3) {                                        // [tap pair][tap of the pair, c][o]
+        const int gi = i >> 13, e = i & 8191, m = e >> 6, o = e & 63, b = m >> 6, c = m & 63;
+        const int tap = gi < 4 ? 2 * gi + b : 7 + b;
+        if (gi == 4 && b == 0) return;                   // tap 7 belongs to pair 3
+        p.out.conv3_w[(o * 64 + c) * 9 + tap] = sum_ranges(p.c3 + gi * p.g3 + e, gi == 4 ? p.r3_last : p.r3, 8192);
+        return;
+    }
+    i -= n3;
+    if (i < n2) {                                        // [tap][(uy, ux, c)][o]
+        const int tap = i >> 13, e = i & 8191, cp = e >> 6, o = e & 63;
+        const int dy = tap >> 1, dx = tap & 1, uy = cp >> 6, ux = (cp >> 5) & 1, c = cp & 31;
+        p.out.conv2_w[((o * 32 + c) * 4 + 2 * dy + uy) * 4 + 2 * dx + ux] = sum_ranges(p.c2 + tap * p.g2 + e, p.r2, 8192);
+        return;
+    }
+    i -= n2;
+    if (i < n1) {                                        // [64 columns of the cell, tap pair][tap, column][o]
+        const int gi = i >> 12, e = i & 4095, m = e >> 5, o = e & 31;
+        const int tap = (gi & 1) * 2 + (m >> 6), k = (gi >> 1) * 64 + (m & 63);
+        const int c = k >> 4, uy = (k >> 2) & 3, ux = k & 3, dy = tap >> 1, dx = tap & 1;
+        if (c < p.C)
+            p.out.conv1_w[((o * p.C + c) * 8 + 4 * dy + uy) * 8 + 4 * dx + ux] =
+                sum_ranges(p.c1 + gi * p.g1 + e, p.r1, 4096) * (1.0f / 255.0f);
+        return;
+    }
+    i -= n1;
+    if (i < nh) {
+        const int o = i / 513, k = i - o * 513;
+        if (o == p.A + 1 && k == 512) return;
+        const float v = sum_ranges(p.head + i, p.rh, (size_t)nh);
+        if (o == p.A + 1) p.out.fc_b[k] = v;
+        else if (k == 512) *(o < p.A ? p.out.pi_b + o : p.out.v_b) = v;
+        else *(o < p.A ? p.out.pi_w + o * 512 + k : p.out.v_w + k) = v;
+        return;
+    }
+    i -= nh;
+    if (i < 64) p.out.conv3_b[i] = sum_ranges(p.b3 + i, p.r3, 64);
+    else if (i < 128) p.out.conv2_b[i - 64] = sum_ranges(p.b2 + i - 64, p.r2, 64);
+    else if (i < 160) p.out.conv1_b[i - 128] = sum_ranges(p.b1 + i - 128, p.r1, 32);
 }
 
 inline unsigned nblk(size_t total, int th) { return (unsigned)((total + th - 1) / th); }
 
 }  // namespace
 
-size_t backward_workspace_floats(const Geometry& g, int max_batch)
+// Packed weights, workspace and tensor maps of the fp32-accurate network passes of one context.
+struct X3State {
+    Geometry g;
+    int max_batch, Cp, H0, W0, G0, H1s, W1s, P1s, P2, P3;
+    int sms;
+    int* status;
+    bf16 *w2p, *w3p, *wfp;
+    // workspace
+    bf16 *x0 = nullptr, *a1, *a2, *a3, *dh, *dz3, *dz2, *dz1;
+    float *logits, *logp, *val, *ent, *dhead, *part1, *part2, *part3, *bias1, *bias2, *bias3, *headp;
+    X3TapParams bfc, bc3, bc2;                           // batch-independent parts
+    X3WgradParams wfc, wc3, wc2, wc1;
+    CUtensorMap mW2, mW3, mWf;
+    int mapped_n = 0;                                    // batch size the maps below were made for
+    CUtensorMap mDh, mDz3, mDz2, vX0, vA1, vA2, vA3, vDh, vDz3, vDz2, vDz1;
+};
+
+namespace {
+
+// A tap groups' slabs: one slab read at every tap's row offset, or, on very wide grids, a slab per tap.
+bool wgrad_rings(X3WgradParams* p, int apl, int b_planes, int kr, int spread, int shared_slabs, int own_slabs, bool* shared)
 {
-    const size_t nb = (size_t)max_batch;
-    const size_t part = (size_t)kBackwardChunks * ((size_t)64 * 64 * 9 + 64 > (size_t)32 * g.C * 64 + 32
-                                                        ? (size_t)64 * 64 * 9 + 64 : (size_t)32 * g.C * 64 + 32);
-    return nb * (g.A + 1) + nb * 512 + nb * g.F + nb * 64 * g.H2 * g.W2 + nb * 32 * g.H1 * g.W1 + part;
+    p->kr = kr;
+    const int room = 227 * 1024 - 4 * 1024;
+    for (int sh = 1; sh >= 0; --sh) {
+        *shared = sh != 0;
+        p->a_rows = sh ? kr + spread : kr;
+        p->n_a = sh ? shared_slabs : own_slabs;
+        if (p->a_rows > 256) continue;
+        const int stage = p->n_a * ((apl * p->a_rows * 128 + 1023) & ~1023) + p->n_b * b_planes * kr * 128;
+        p->stages = room / stage > 8 ? 8 : room / stage;
+        if (p->stages >= (sh ? 2 : 1)) return true;
+    }
+    return false;
 }
 
-hts_status ref_backward(const Geometry& g, const RefWeights& w, const RefWorkspace& act, const uint8_t* obs, float* ws,
-                        const float* logits, const float* values, const int32_t* actions, const float* adv,
-                        const float* ret, const float* logp_old, float value_coef, float entropy_coef, float clip,
-                        int n, int max_batch, int* status, const hts_grads& out, cudaStream_t s)
+bool x3_plan(X3State* t)
 {
-    const size_t nb = (size_t)max_batch;
-    const int A = g.A, th = 256;
-    float* dhead = ws;                                   // [n][A+1]
-    float* dh = dhead + nb * (A + 1);                    // [n][512]
-    float* da3 = dh + nb * 512;                          // [n][F]    (NCHW, as the FC sees it)
-    float* da2 = da3 + nb * g.F;                         // [n][64][H2][W2]
-    float* da1 = da2 + nb * 64 * g.H2 * g.W2;            // [n][32][H1][W1]
-    float* part = da1 + nb * 32 * g.H1 * g.W1;           // chunk partials of one convolution's weight gradient
+    const Geometry& g = t->g;
+    const int s1[4] = {0, 1, t->W0, t->W0 + 1}, s2[4] = {0, 1, t->W1s, t->W1s + 1}, n2[4] = {0, -1, -t->W1s, -t->W1s - 1};
+    int s3[9], n3[9];
+    const int zero = 0;
+    for (int i = 0; i < 9; ++i) { s3[i] = (i / 3) * g.W2 + i % 3; n3[i] = -s3[i]; }
+    auto tap = [&](X3TapParams& p, int mode, int chunks, int taps, const int* shift, int tap_cols, int n_tiles, int P, int W, int H_out,
+                   int W_out, int P_dst, int W_dst, int pitch) {
+        p = X3TapParams{};
+        p.mode = mode; p.n_tiles = n_tiles; p.tap_cols = tap_cols; p.P = P; p.W = W; p.H_out = H_out; p.W_out = W_out;
+        p.P_dst = P_dst; p.W_dst = W_dst; p.dst_pitch = pitch; p.status = t->status;
+        return x3_taps_plan(&p, chunks, taps, shift);
+    };
+    if (!(tap(t->bfc, X3_DGRAD_FC, 8, 1, &zero, 0, t->P3, 1, 1, g.H3, g.W3, t->P2, g.W2, 64) &&
+          tap(t->bc3, X3_DGRAD, 1, 9, n3, 64, 1, t->P2, g.W2, g.H2, g.W2, t->P1s, t->W1s, 64) &&
+          tap(t->bc2, X3_DGRAD_S2D, 1, 4, n2, 128, 2, t->P1s, t->W1s, g.H1, g.W1, t->G0, t->W0, 128)))
+        return false;
 
-    head_grad_kernel<<<nblk(n, 128), 128, 0, s>>>(logits, values, actions, adv, ret, logp_old, value_coef, entropy_coef,
-                                                   clip, n, A, status, dhead);
-    HTS_LAUNCH_CHECK("head_grad_kernel");
-    // heads: rows 0..A-1 of the stacked head are the policy, row A the value
-    dense_wgrad_kernel<<<dim3(nblk(512, th), nblk(A, kOTile)), th, 0, s>>>(dhead, A + 1, A, act.h, 512, n, out.pi_w);
-    HTS_LAUNCH_CHECK("dense_wgrad(pi)");
-    dense_wgrad_kernel<<<dim3(nblk(512, th), 1), th, 0, s>>>(dhead + A, A + 1, 1, act.h, 512, n, out.v_w);
-    HTS_LAUNCH_CHECK("dense_wgrad(v)");
-    dense_bgrad_kernel<<<nblk(A, 64), 64, 0, s>>>(dhead, A + 1, A, n, out.pi_b);
-    HTS_LAUNCH_CHECK("dense_bgrad(pi)");
-    dense_bgrad_kernel<<<1, 64, 0, s>>>(dhead + A, A + 1, 1, n, out.v_b);
-    HTS_LAUNCH_CHECK("dense_bgrad(v)");
-    dense_dgrad_kernel<<<nblk((size_t)n * 512, th), th, 0, s>>>(dhead, A + 1, A + 1, w.whead, 512, act.h, n, dh);
-    HTS_LAUNCH_CHECK("dense_dgrad(heads)");
-    // FC
-    dense_wgrad_kernel<<<dim3(nblk(g.F, th), nblk(512, kOTile)), th, 0, s>>>(dh, 512, 512, act.a3, g.F, n, out.fc_w);
-    HTS_LAUNCH_CHECK("dense_wgrad(fc)");
-    dense_bgrad_kernel<<<nblk(512, 64), 64, 0, s>>>(dh, 512, 512, n, out.fc_b);
-    HTS_LAUNCH_CHECK("dense_bgrad(fc)");
-    dense_dgrad_kernel<<<nblk((size_t)n * g.F, th), th, 0, s>>>(dh, 512, 512, w.wfc, g.F, act.a3, n, da3);
-    HTS_LAUNCH_CHECK("dense_dgrad(fc)");
-    // the three convolutions, last to first
-    const int chunks = n < kBackwardChunks ? n : kBackwardChunks;
-    const int per_chunk = (n + chunks - 1) / chunks;
-    const int used = (n + per_chunk - 1) / per_chunk;
-    struct Layer { const float* dy; const void* in; bool u8; int C, H, W, O, k, s, Ho, Wo; const float* wt; float *dW, *db, *dx; const float* x_act; };
-    const Layer layers[3] = {
-        {da3, act.a2, false, 64, g.H2, g.W2, 64, 3, 1, g.H3, g.W3, w.w3, out.conv3_w, out.conv3_b, da2, act.a2},
-        {da2, act.a1, false, 32, g.H1, g.W1, 64, 4, 2, g.H2, g.W2, w.w2, out.conv2_w, out.conv2_b, da1, act.a1},
-        {da1, obs, true, g.C, g.H, g.W, 32, 8, 4, g.H1, g.W1, w.w1, out.conv1_w, out.conv1_b, nullptr, nullptr}};
-    for (const Layer& L : layers) {
-        const int nW = L.O * L.C * L.k * L.k, total = nW + L.O;
-        if (L.O % kWgradOB) return HTS_ERR_SHAPE;
-        const int wthreads = nW / kWgradOB + L.O;
-        if (L.u8)
-            conv_wgrad_kernel<uint8_t><<<dim3(nblk(wthreads, 128), used), 128, 0, s>>>(
-                L.dy, static_cast<const uint8_t*>(L.in), n, L.C, L.H, L.W, L.O, L.k, L.s, L.Ho, L.Wo, per_chunk, part);
-        else
-            conv_wgrad_kernel<float><<<dim3(nblk(wthreads, 128), used), 128, 0, s>>>(
-                L.dy, static_cast<const float*>(L.in), n, L.C, L.H, L.W, L.O, L.k, L.s, L.Ho, L.Wo, per_chunk, part);
-        HTS_LAUNCH_CHECK("conv_wgrad_kernel");
-        conv_wgrad_reduce_kernel<<<nblk(total, th), th, 0, s>>>(part, used, nW, L.O, L.u8 ? 1.0f / 255.0f : 1.0f, L.dW, L.db);
-        HTS_LAUNCH_CHECK("conv_wgrad_reduce_kernel");
-        if (L.dx) {
-            const size_t w_smem = (size_t)L.k * L.k * L.O * kDgradCB * sizeof(float);
-            if (w_smem > 48 * 1024) return HTS_ERR_SHAPE;
-            conv_dgrad_kernel<<<dim3(nblk((size_t)n * L.H * L.W, 256), nblk(L.C, kDgradCB)), 256, w_smem, s>>>(
-                L.dy, L.wt, L.x_act, n, L.C, L.H, L.W, L.O, L.k, L.s, L.Ho, L.Wo, L.dx);
-            HTS_LAUNCH_CHECK("conv_dgrad_kernel");
-        }
+    bool sh;
+    auto slab = [](const X3WgradParams& p, int apl) { return (apl * p.a_rows * 128 + 1023) & ~1023; };
+    {   // dense layer: kind = (128 outputs, two pixels)
+        X3WgradParams& p = t->wfc; p = X3WgradParams{};
+        p.n_b = 2;
+        if (!wgrad_rings(&p, 3, 3, 64, 0, 2, 2, &sh)) return false;
+        p.ka = 4; p.a_step = 128; p.b_step = 128; p.slab_col[1] = 64;
+        p.groups = 2; p.group_cap = 2; p.kinds = 4 * ((t->P3 + 1) / 2); p.ranges = p.last_ranges = 1;
+        p.a_lbo[0] = p.a_lbo[1] = slab(p, 3); p.b_off[1] = 3 * p.kr * 128; p.P3 = t->P3;
     }
+    {   // conv3: five pairs of taps (0,1) (2,3) (4,5) (6,7) (7,8)
+        X3WgradParams& p = t->wc3; p = X3WgradParams{};
+        p.n_b = 1;
+        if (!wgrad_rings(&p, 3, 3, 64, s3[8], 1, 4, &sh)) return false;
+        p.ka = 1; p.kinds = 3; p.group_mul = 2; p.groups = 2; p.group_cap = 5;
+        for (int gi = 0; gi < 5; ++gi) {
+            const int t0 = gi < 4 ? 2 * gi : 7;
+            p.a_off[gi] = sh ? s3[t0] * 128 : (gi & 1) * 2 * slab(p, 3);
+            p.a_lbo[gi] = sh ? (s3[t0 + 1] - s3[t0]) * 128 : slab(p, 3);
+            if (!sh) for (int b = 0; b < 2; ++b) p.slab_row[2 * gi + b] = s3[t0 + b];
+        }
+        if (!sh) p.slab_mul = 4;
+    }
+    {   // conv2: a group = one tap, its two 64-channel slabs
+        X3WgradParams& p = t->wc2; p = X3WgradParams{};
+        p.n_b = 1;
+        if (!wgrad_rings(&p, 3, 3, 64, s2[3], 2, 4, &sh)) return false;
+        p.ka = 1; p.kinds = 2; p.group_mul = 2; p.groups = 2; p.group_cap = 4;
+        for (int gi = 0; gi < 4; ++gi) {
+            p.a_off[gi] = sh ? s2[gi] * 128 : (gi & 1) * 2 * slab(p, 3);
+            p.a_lbo[gi] = slab(p, 3);
+            if (!sh) for (int b = 0; b < 2; ++b) { p.slab_col[2 * gi + b] = 64 * b; p.slab_row[2 * gi + b] = s2[gi]; }
+        }
+        if (sh) p.slab_col[1] = 64; else p.slab_mul = 4;
+    }
+    {   // conv1: kind = 64 columns of a cell, groups = the tap pairs (0,1) (2,3)
+        X3WgradParams& p = t->wc1; p = X3WgradParams{};
+        p.n_b = 2;
+        if (!wgrad_rings(&p, 1, 1, 128, s1[3], 1, 4, &sh)) return false;
+        p.ka = p.kinds = t->Cp / 4; p.a_step = 64; p.group_mul = 2; p.groups = 2; p.group_cap = 2 * p.kinds;
+        for (int gi = 0; gi < p.group_cap; ++gi) {
+            p.a_off[gi] = sh ? s1[2 * (gi & 1)] * 128 : (gi & 1) * 2 * slab(p, 1);
+            p.a_lbo[gi] = sh ? 128 : slab(p, 1);
+        }
+        if (!sh) for (int i = 0; i < 4; ++i) p.slab_row[i] = s1[i];
+    }
+    for (X3WgradParams* p : {&t->wfc, &t->wc3, &t->wc2, &t->wc1}) p->status = t->status;
+    return true;
+}
+
+}  // namespace
+
+hts_status x3_create(const Geometry& g, int max_batch, int* status, X3State** out,
+                     bool (*alloc)(void* ctx, void** p, size_t bytes), void* alloc_ctx)
+{
+    X3State* t = new (std::nothrow) X3State();
+    if (!t) return HTS_ERR_ALLOC;
+    t->g = g; t->max_batch = max_batch; t->status = status;
+    t->Cp = (g.C + 3) / 4 * 4; t->H0 = g.H / 4; t->W0 = g.W / 4; t->G0 = t->H0 * t->W0;
+    t->H1s = (g.H1 + 1) / 2; t->W1s = (g.W1 + 1) / 2; t->P1s = t->H1s * t->W1s; t->P2 = g.H2 * g.W2; t->P3 = g.H3 * g.W3;
+    t->sms = device_sm_count(device_slot());
+    if (!x3_plan(t)) { delete t; return HTS_ERR_SHAPE; }
+    const size_t n2 = 64 * 512, n3 = 64 * 576, nf = (size_t)512 * g.F;
+    void* base = nullptr;
+    if (!alloc(alloc_ctx, &base, 2 * 3 * (n2 + n3 + nf))) { delete t; return HTS_ERR_ALLOC; }
+    t->w2p = static_cast<bf16*>(base); t->w3p = t->w2p + 3 * n2; t->wfp = t->w3p + 3 * n3;
+    if (!(x3_make_map(&t->mW2, t->w2p, 512, 64, 3, 512, n2, 64, 3) && x3_make_map(&t->mW3, t->w3p, 576, 64, 3, 576, n3, 64, 3) &&
+          x3_make_map(&t->mWf, t->wfp, g.F, 512, 3, g.F, nf, 64, 3))) {
+        delete t;
+        return HTS_ERR_CUDA;
+    }
+    *out = t;
+    return HTS_OK;
+}
+
+void x3_destroy(X3State* t) { delete t; }
+
+hts_status x3_pack_weights(X3State* t, const RefWeights& w, cudaStream_t s)
+{
+    pack_x3_kernel<<<512 + nblk(64 * 512 + 64 * 576, 256), 256, 0, s>>>(w.w2, w.w3, w.wfc, t->P3, t->w2p, t->w3p, t->wfp);
+    HTS_LAUNCH_CHECK("pack_x3");
+    return HTS_OK;
+}
+
+namespace {
+
+// One allocation for everything the passes keep between kernels.  Zeroed once: positions of a grid outside a layer's
+// output extent and channels added to the frames are never written and have to read as zero.
+hts_status x3_workspace(X3State* t, bool (*alloc)(void* ctx, void** p, size_t bytes), void* alloc_ctx, cudaStream_t s)
+{
+    if (t->x0) return HTS_OK;
+    const Geometry& g = t->g;
+    const size_t nb = (size_t)t->max_batch, A = g.A;
+    const int r1 = t->sms / t->wc1.kinds < 1 ? 1 : t->sms / t->wc1.kinds;
+    size_t total = 0;
+    auto room = [&](size_t bytes) { const size_t at = total; total += (bytes + 1023) & ~(size_t)1023; return at; };
+    const size_t o_x0 = room(2 * nb * t->G0 * 16 * t->Cp), o_a1 = room(6 * nb * t->P1s * 128), o_a2 = room(6 * nb * t->P2 * 64),
+                 o_a3 = room(6 * nb * g.F), o_dh = room(6 * nb * 512), o_dz3 = room(6 * nb * t->P2 * 64), o_dz2 = room(6 * nb * t->P1s * 64),
+                 o_dz1 = room(2 * nb * t->G0 * 128), zeroed = total;
+    const size_t o_lg = room(4 * nb * A), o_lp = room(4 * nb), o_v = room(4 * nb),
+                 o_e = room(4 * nb), o_dhead = room(4 * nb * (A + 1)), o_p1 = room(4 * (size_t)2 * t->wc1.kinds * r1 * 4096),
+                 o_p2 = room(4 * (size_t)4 * (t->sms / 2 + 1) * 8192), o_p3 = room(4 * (size_t)5 * (t->sms * 2 / 5 + 1) * 8192), o_b1 = room(4 * (size_t)t->sms * 32),
+                 o_b2 = room(4 * (size_t)t->sms * 64), o_b3 = room(4 * (size_t)t->sms * 64), o_hd = room(4 * kHeadRanges * (A + 2) * 513);
+    void* q = nullptr;
+    if (!alloc(alloc_ctx, &q, total + 1024)) return HTS_ERR_ALLOC;
+    uint8_t* b = reinterpret_cast<uint8_t*>(((uintptr_t)q + 1023) & ~(uintptr_t)1023);
+    HTS_CUDA(cudaMemsetAsync(b, 0, zeroed, s));
+    auto H = [&](size_t o) { return reinterpret_cast<bf16*>(b + o); };
+    auto Fl = [&](size_t o) { return reinterpret_cast<float*>(b + o); };
+    t->x0 = H(o_x0); t->a1 = H(o_a1); t->a2 = H(o_a2); t->a3 = H(o_a3); t->dh = H(o_dh); t->dz3 = H(o_dz3); t->dz2 = H(o_dz2); t->dz1 = H(o_dz1);
+    t->logits = Fl(o_lg); t->logp = Fl(o_lp); t->val = Fl(o_v); t->ent = Fl(o_e); t->dhead = Fl(o_dhead);
+    t->part1 = Fl(o_p1); t->part2 = Fl(o_p2); t->part3 = Fl(o_p3); t->bias1 = Fl(o_b1); t->bias2 = Fl(o_b2); t->bias3 = Fl(o_b3); t->headp = Fl(o_hd);
+    return HTS_OK;
+}
+
+// Tensor maps end with the rows of this batch: what an earlier, larger batch left behind reads as zero.
+bool x3_map_batch(X3State* t, int n)
+{
+    if (t->mapped_n == n) return true;
+    const Geometry& g = t->g;
+    const size_t nb = (size_t)t->max_batch, N = (size_t)n;
+    auto map = [](CUtensorMap* m, const bf16* p, uint64_t cols, uint64_t rows, uint64_t planes, uint64_t plane, int box, int box_planes) {
+        return x3_make_map(m, p, cols, rows, planes, cols, plane, (uint32_t)box, (uint32_t)box_planes);
+    };
+    const size_t p1 = nb * t->P1s * 128, p2 = nb * t->P2 * 64, p3 = nb * g.F, ph = nb * 512, pz2 = nb * t->P1s * 64, x = nb * t->G0 * 16 * t->Cp;
+    const bool ok =
+        map(&t->vX0, t->x0, 16 * t->Cp, N * t->G0, 1, x, t->wc1.a_rows, 1) &&
+        map(&t->vA1, t->a1, 128, N * t->P1s, 3, p1, t->wc2.a_rows, 3) &&
+        map(&t->vA2, t->a2, 64, N * t->P2, 3, p2, t->wc3.a_rows, 3) &&
+        map(&t->vA3, t->a3, g.F, N, 3, p3, t->wfc.kr, 3) &&
+        map(&t->mDh, t->dh, 512, N, 3, ph, t->bfc.entry_rows, 3) && map(&t->vDh, t->dh, 512, N, 3, ph, t->wfc.a_rows, 3) &&
+        map(&t->mDz3, t->dz3, 64, N * t->P2, 3, p2, t->bc3.entry_rows, 3) && map(&t->vDz3, t->dz3, 64, N * t->P2, 3, p2, t->wc3.kr, 3) &&
+        map(&t->mDz2, t->dz2, 64, N * t->P1s, 3, pz2, t->bc2.entry_rows, 3) && map(&t->vDz2, t->dz2, 64, N * t->P1s, 3, pz2, t->wc2.kr, 3) &&
+        map(&t->vDz1, t->dz1, 128, N * t->G0, 1, nb * t->G0 * 128, t->wc1.kr, 1);
+    t->mapped_n = ok ? n : 0;
+    return ok;
+}
+
+inline int tiles_of(size_t rows) { return (int)((rows + 127) / 128); }
+
+}  // namespace
+
+hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, Profiler& prof, const uint8_t* obs, const int32_t* actions, const float* adv, const float* ret,
+                       const float* logp_old, float value_coef, float entropy_coef, float clip, int n, const hts_grads& out,
+                       bool (*alloc)(void* ctx, void** p, size_t bytes), void* alloc_ctx, cudaStream_t s)
+{
+    const Geometry& g = t->g;
+    hts_status st = x3_workspace(t, alloc, alloc_ctx, s);
+    if (st != HTS_OK) return st;
+    if (!x3_map_batch(t, n)) return HTS_ERR_CUDA;
+    const size_t nb = (size_t)t->max_batch, N = (size_t)n;
+    const size_t p1 = nb * t->P1s * 128, p2 = nb * t->P2 * 64, p3 = nb * g.F, ph = nb * 512, pz2 = nb * t->P1s * 64;
+
+    const size_t items = N * t->G0 * t->Cp;
+    HTS_CUDA(launch_pdl(frames_kernel, dim3(nblk(items, 256)), dim3(256), 0, s, obs, g.C, t->Cp, g.H, g.W, items, ((uintptr_t)obs & 3) == 0,
+                        t->x0));
+    note_launch();
+    const RefPlanes planes{t->a1, t->a2, t->a3, p1, p2, p3};
+    st = ref_forward(g, w, ws, obs, Indexing{}, t->status, n, prof, s, &planes);
+    if (st != HTS_OK) return st;
+    st = launch_heads(ws.h, 1, 0, nullptr, w.whead, w.bhead, g.A, nullptr, nullptr, 0, 0, n, Indexing{}, t->status, nullptr, t->logp, t->val,
+                      t->ent, t->logits, nullptr, s, actions);
+    if (st != HTS_OK) return st;
+    auto run = [&](X3TapParams p, size_t rows, bf16* dst, size_t dst_plane, const bf16* mask, int mask_pitch) {
+        p.m_tiles = tiles_of(rows); p.n = n; p.dst = dst; p.dst_plane = dst_plane; p.mask = mask; p.mask_pitch = mask_pitch;
+        return p;
+    };
+
+    // ---- heads and data gradients
+    const int sms = t->sms;
+    {
+        const size_t smem = (size_t)(g.A + 1) * 2048;
+        static size_t smem_set_by_device[kDeviceSlots] = {};
+        size_t& smem_set = smem_set_by_device[device_slot()];
+        if (smem > 40 * 1024 && smem > smem_set) {
+            HTS_CUDA(cudaFuncSetAttribute(head_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            smem_set = smem;
+        }
+        const int blocks = n < sms ? n : (int)nblk(N, 8) < sms ? sms : (int)nblk(N, 8) < 4 * sms ? (int)nblk(N, 8) : 4 * sms;
+        HTS_CUDA(launch_pdl(head_backward_kernel, dim3(blocks), dim3(256), smem, s, t->logits, t->val, actions, adv, ret, logp_old, w.whead, ws.h,
+                            value_coef, entropy_coef, clip, n, g.A, t->status, t->dhead, t->dh, ph));
+        note_launch();
+    }
+    int per_range = (n + (int)kHeadRanges - 1) / (int)kHeadRanges;
+    if (per_range < 16) per_range = 16;
+    const int rh = (n + per_range - 1) / per_range;
+    HTS_CUDA(launch_pdl(head_wgrad_kernel, dim3(8, rh, nblk(g.A + 2, kHeadTile)), dim3(256), 0, s, t->dhead, ws.h, t->dh, ph, n, g.A, per_range,
+                        t->headp));
+    note_launch();
+    st = x3_dgrad_launch(t->mDh, t->mWf, run(t->bfc, N, t->dz3, p2, t->a3, g.F), s);
+    if (st != HTS_OK) return st;
+    st = x3_dgrad_launch(t->mDz3, t->mW3, run(t->bc3, N * t->P2, t->dz2, pz2, t->a2, 64), s);
+    if (st != HTS_OK) return st;
+    st = x3_dgrad_launch(t->mDz2, t->mW2, run(t->bc2, N * t->P1s, t->dz1, 32, t->a1, 128), s);
+    if (st != HTS_OK) return st;
+
+    // ---- weight gradients: as many ranges of rows as SMs, each with at least one stage of rows
+    auto cut = [&](X3WgradParams p, size_t rows, int ranges, int last) {
+        p.row_chunks = (int)((rows + p.kr - 1) / p.kr);
+        p.ranges = ranges < p.row_chunks ? ranges : p.row_chunks;
+        p.last_ranges = last < p.row_chunks ? last : p.row_chunks;
+        return p;
+    };
+    X3WgradParams q = cut(t->wfc, N, 1, 1);
+    q.fc_w = out.fc_w;
+    st = x3_wgrad_launch<3, 64>(t->vDh, t->vA3, q, s);
+    if (st != HTS_OK) return st;
+    ReduceParams r{};
+    X3WgradParams q3 = cut(t->wc3, N * t->P2, sms * 2 / 5 < 1 ? 1 : sms * 2 / 5, sms / 5 < 1 ? 1 : sms / 5);   // the last kind has one group of five
+    q3.part = t->part3; q3.group_stride = (size_t)q3.ranges * 8192; q3.bias_part = t->bias3;
+    st = x3_wgrad_launch<3, 64>(t->vA2, t->vDz3, q3, s);
+    if (st != HTS_OK) return st;
+    X3WgradParams q2 = cut(t->wc2, N * t->P1s, sms / 2 < 1 ? 1 : sms / 2, sms / 2 < 1 ? 1 : sms / 2);
+    q2.part = t->part2; q2.group_stride = (size_t)q2.ranges * 8192; q2.bias_part = t->bias2;
+    st = x3_wgrad_launch<3, 64>(t->vA1, t->vDz2, q2, s);
+    if (st != HTS_OK) return st;
+    const int r1 = sms / t->wc1.kinds < 1 ? 1 : sms / t->wc1.kinds;
+    X3WgradParams q1 = cut(t->wc1, N * t->G0, r1, r1);
+    q1.part = t->part1; q1.group_stride = (size_t)q1.ranges * 4096; q1.bias_part = t->bias1;
+    st = x3_wgrad_launch<1, 32>(t->vX0, t->vDz1, q1, s);
+    if (st != HTS_OK) return st;
+    r.c1 = t->part1; r.c2 = t->part2; r.c3 = t->part3; r.b1 = t->bias1; r.b2 = t->bias2; r.b3 = t->bias3; r.head = t->headp;
+    r.r1 = q1.ranges; r.r2 = q2.ranges; r.r3 = q3.ranges; r.r3_last = q3.last_ranges; r.rh = rh;
+    r.g1 = q1.group_stride; r.g2 = q2.group_stride; r.g3 = q3.group_stride;
+    r.C = g.C; r.Cp = t->Cp; r.A = g.A; r.out = out;
+    const size_t total = (size_t)9 * 8192 + (size_t)t->Cp / 2 * 4096 + (size_t)(g.A + 2) * 513 + 160;
+    HTS_CUDA(launch_pdl(reduce_kernel, dim3(nblk(total, 256)), dim3(256), 0, s, r));
+    note_launch();
     return HTS_OK;
 }
 

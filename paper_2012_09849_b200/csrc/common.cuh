@@ -110,13 +110,16 @@ hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspac
                        const uint8_t* obs, const Indexing& ix, int* status, int n, Profiler& prof, cudaStream_t s,
                        const RefPlanes* planes = nullptr);
 
-// ---- gradient of the learner objective on the fp32 path (backward.cu) ---------------------------
-constexpr int kBackwardChunks = 64;      // batch chunks whose partial weight gradients are added in index order
-size_t backward_workspace_floats(const Geometry& g, int max_batch);
-hts_status ref_backward(const Geometry& g, const RefWeights& w, const RefWorkspace& act, const uint8_t* obs, float* ws,
-                        const float* logits, const float* values, const int32_t* actions, const float* adv,
-                        const float* ret, const float* logp_old, float value_coef, float entropy_coef, float clip,
-                        int n, int max_batch, int* status, const hts_grads& out, cudaStream_t s);
+// ---- gradient of the learner objective: fp32-accurate passes on the tensor cores (backward.cu) -------
+struct X3State;
+hts_status x3_create(const Geometry& g, int max_batch, int* status, X3State** out,
+                     bool (*alloc)(void* ctx, void** p, size_t bytes), void* alloc_ctx);
+void x3_destroy(X3State* t);
+hts_status x3_pack_weights(X3State* t, const RefWeights& w, cudaStream_t s);
+// The workspace is allocated by the first call on a state.
+hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, Profiler& prof, const uint8_t* obs, const int32_t* actions, const float* adv, const float* ret,
+                       const float* logp_old, float value_coef, float entropy_coef, float clip, int n, const hts_grads& out,
+                       bool (*alloc)(void* ctx, void** p, size_t bytes), void* alloc_ctx, cudaStream_t s);
 
 // ---- the tensor-core path (bf16 weights) -------------------------------------------------------
 struct TcState;

@@ -35,8 +35,7 @@ struct hts_ctx {
     uint8_t* s_obs = nullptr;
     int32_t *s_ids = nullptr, *s_t = nullptr, *s_act = nullptr;
     float *s_logp = nullptr, *s_val = nullptr, *s_ent = nullptr, *s_logits = nullptr;
-    float* bw_ws = nullptr;       // backward workspace (allocated by the first hts_policy_gradient)
-    float *bw_logits = nullptr, *bw_logp = nullptr, *bw_val = nullptr, *bw_ent = nullptr;
+    X3State* x3 = nullptr;        // packed weights and workspace of the gradient (weight_dtype fp32)
     int* status = nullptr;        // device status word
     Profiler prof;
     void* allocs[112];
@@ -167,6 +166,10 @@ hts_status hts_policy_create(const hts_net_desc* d, hts_ctx** out)
         ok = ok && dev_alloc(c, &c->rw.whead, (size_t)(A + 1) * 512) && dev_alloc(c, &c->rw.bhead, (size_t)A + 1);
         ok = ok && dev_alloc(c, &c->rws.a1, nb * 32 * g.H1 * g.W1) && dev_alloc(c, &c->rws.a2, nb * 64 * g.H2 * g.W2);
         ok = ok && dev_alloc(c, &c->rws.a3, nb * g.F) && dev_alloc(c, &c->rws.h, nb * 512);
+        if (ok) {
+            const hts_status st = x3_create(g, d->max_batch, c->status, &c->x3, raw_alloc, c);
+            if (st != HTS_OK) { hts_policy_destroy(c); return st; }
+        }
     }
     ok = ok && dev_alloc(c, &c->s_obs, nb * g.C * g.H * g.W);
     ok = ok && dev_alloc(c, &c->s_ids, nb) && dev_alloc(c, &c->s_t, nb) && dev_alloc(c, &c->s_act, nb);
@@ -190,6 +193,7 @@ hts_status hts_policy_load_weights(hts_ctx* ctx, const hts_weights* w, void* cud
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     hts_status st = ctx->tc ? tc_load_weights(ctx->tc, *w, s)
                             : ref_convert_weights(ctx->g, ctx->desc.weight_dtype, *w, ctx->rw, s);
+    if (st == HTS_OK && ctx->x3) st = x3_pack_weights(ctx->x3, ctx->rw, s);
     if (st != HTS_OK) return st;
     ctx->loaded = true;
     return HTS_OK;
@@ -256,19 +260,10 @@ hts_status hts_policy_gradient(hts_ctx* ctx, const uint8_t* obs, const int32_t* 
     if (!(clip >= 0.f) || !std::isfinite(clip) || !std::isfinite(value_coef) || !std::isfinite(entropy_coef)) return HTS_ERR_INVALID_ARG;
     if (ctx->tc) return HTS_ERR_UNSUPPORTED;
     if (!ctx->loaded) return HTS_ERR_UNSUPPORTED;
-    const size_t nb = (size_t)ctx->desc.max_batch;
-    if (!ctx->bw_ws) {
-        bool ok = dev_alloc(ctx, &ctx->bw_ws, backward_workspace_floats(ctx->g, ctx->desc.max_batch));
-        ok = ok && dev_alloc(ctx, &ctx->bw_logits, nb * ctx->g.A) && dev_alloc(ctx, &ctx->bw_logp, nb);
-        ok = ok && dev_alloc(ctx, &ctx->bw_val, nb) && dev_alloc(ctx, &ctx->bw_ent, nb);
-        if (!ok) { ctx->bw_ws = nullptr; return HTS_ERR_ALLOC; }
-    }
-    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    hts_status st = run_step(ctx, obs, Indexing{}, nullptr, nullptr, 0, 0, n, nullptr, ctx->bw_logp, ctx->bw_val, ctx->bw_ent,
-                             ctx->bw_logits, s, actions);
-    if (st != HTS_OK) return st;
-    return ref_backward(ctx->g, ctx->rw, ctx->rws, obs, ctx->bw_ws, ctx->bw_logits, ctx->bw_val, actions, advantages, returns,
-                        logp_old_or_null, value_coef, entropy_coef, clip, n, ctx->desc.max_batch, ctx->status, *grads, s);
+    const hts_status st = x3_gradient(ctx->x3, ctx->rw, ctx->rws, ctx->prof, obs, actions, advantages, returns, logp_old_or_null,
+                                      value_coef, entropy_coef, clip, n, *grads, raw_alloc, ctx, static_cast<cudaStream_t>(cuda_stream));
+    if (st == HTS_OK) ctx->last_n = n;
+    return st;
 }
 
 hts_status hts_policy_step_host(hts_ctx* ctx, const uint8_t* obs, const int32_t* env_ids,
@@ -385,6 +380,7 @@ void hts_policy_destroy(hts_ctx* ctx)
         if (ctx->prof.stop[k]) { for (int i = 0; i < Profiler::kCap; ++i) cudaEventDestroy(ctx->prof.stop[k][i]); delete[] ctx->prof.stop[k]; }
     }
     if (ctx->tc) tc_destroy(ctx->tc);
+    if (ctx->x3) x3_destroy(ctx->x3);
     for (int i = 0; i < ctx->nalloc; ++i) cudaFree(ctx->allocs[i]);
     delete ctx;
 }

@@ -1,0 +1,467 @@
+// The two tensor-core kernels of the fp32-accurate path (see x3_gemm.cuh for the arithmetic and the layouts).
+#include "x3_gemm.cuh"
+#include "tc_ptx.cuh"
+#include "tc_host.cuh"
+
+namespace hts {
+using namespace tc;
+
+namespace {
+
+constexpr int kSmemMax = 227 * 1024;
+constexpr int kMaxEntries = 4, kMaxStages = 8;
+
+// bf16 operands, fp32 accumulation; `mn_a` / `mn_b`: the operand's tile has its M / N index along the 128-byte rows
+__host__ __device__ constexpr uint32_t idesc_x3(uint32_t N, uint32_t mn_a, uint32_t mn_b)
+{
+    return instr_desc_f16(1, 128, N) | (mn_a << 15) | (mn_b << 16);
+}
+// Tile with K along the rows (128 bytes of M or N per row, 128-byte swizzle): groups of eight K rows are 1024 bytes
+// apart, blocks of 64 M / N elements `lbo_bytes`.
+__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr, uint32_t lbo_bytes)
+{
+    return (smem_desc_sw128(addr) & ~((uint64_t)0x3FFF << 16)) | ((uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16);
+}
+__device__ __forceinline__ void tma_load_3d(uint32_t smem_dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar)
+{
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 ::"r"(smem_dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void st_v8(void* ptr, const uint32_t* v)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 ::"l"(ptr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
+// One K step of 16: the six products, each weight class into its own accumulator columns [0, NB), [NB, 2 NB), [2 NB, 3 NB).
+// With the planes of B stacked along N, plane i of A meets planes 0 .. 2 - i of B in one instruction.
+template <int APL, int NB>
+__device__ __forceinline__ void mma_x3(uint32_t d, uint64_t a, uint64_t a_plane, uint64_t b, uint32_t mn_a, uint32_t mn_b, bool first)
+{
+    mma_f16_ss(d, a, b, idesc_x3(3 * NB, 0, 0) | (mn_a << 15) | (mn_b << 16), !first);
+    if (APL == 3) {
+        mma_f16_ss(d + NB, a + a_plane, b, idesc_x3(2 * NB, 0, 0) | (mn_a << 15) | (mn_b << 16), 1);
+        mma_f16_ss(d + 2 * NB, a + 2 * a_plane, b, idesc_x3(NB, 0, 0) | (mn_a << 15) | (mn_b << 16), 1);
+    }
+}
+template <int NB>
+__device__ __forceinline__ void acc_load32(uint32_t taddr, int c0, float (&v)[32], bool last, uint64_t* empty_bar)
+{
+    uint32_t p0[32], p1[32];
+    tmem_ld_32x32(taddr + NB + c0, p0);
+    tmem_ld_32x32(taddr + 2 * NB + c0, p1);
+    tmem_ld_wait();
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(p0[j]) + __uint_as_float(p1[j]);
+    tmem_ld_32x32(taddr + c0, p0);
+    tmem_ld_wait();
+    if (last && empty_bar) {                            // everything is in registers: hand the accumulator back
+        tc_fence_before();
+        mbar_arrive(empty_bar);
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(p0[j]) + v[j];
+}
+
+// Persistent: CTA b takes tiles b, b + gridDim.x, ...  Warp 0 copies (A entries and B stages in two rings), warp 1
+// issues, then two groups of four epilogue warps, one accumulator of 192 columns each.
+// Bound: the tensor core, which spends (128 + N) / 4 clocks (shared-memory operand fetch) or N / 2 on an
+// instruction: 96 + 64 + 48 = 208 clocks per 16 of K for 64 output columns, against 288 for six separate
+// 128 x 64 instructions.  An A entry (all planes, rows 128 + spread) is loaded once per tile and every tap reads it
+// shifted; B is streamed.
+constexpr int EG = 2, kDgradThreads = 64 + 128 * EG;
+__global__ void __launch_bounds__(kDgradThreads)
+x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const X3TapParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t a_full[kMaxEntries], a_empty[kMaxEntries], b_full[kMaxStages], b_empty[kMaxStages], d_full[EG], d_empty[EG];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+    volatile int* abortp = &abort_flag;
+    constexpr int BB = 3 * 8192;                        // bytes of a B stage: [plane][64 K rows][64 columns]
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const int plane_bytes = p.entry_rows * 128;
+    const int a_bytes = 3 * plane_bytes, a_pitch = (a_bytes + 1023) & ~1023;
+    const uint32_t b_base = base + p.entries * a_pitch;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tiles = p.m_tiles * p.n_tiles;
+    const int groups = p.taps / p.tpe;                  // A entries per chunk
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kMaxEntries; ++i) { mbar_init(&a_full[i], 1); mbar_init(&a_empty[i], 1); }
+        for (int i = 0; i < kMaxStages; ++i) { mbar_init(&b_full[i], 1); mbar_init(&b_empty[i], 1); }
+        for (int i = 0; i < EG; ++i) { mbar_init(&d_full[i], 1); mbar_init(&d_empty[i], 128); }
+        abort_flag = 0;
+        fence_barrier_init();
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+    }
+    if (warp == 1) tmem_alloc(&tmem_slot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_d = tmem_slot;
+    pdl_wait();
+    pdl_trigger();
+
+    // tile -> (M tile, N tile): M fastest, so that CTAs running together share B through L2
+    if (warp == 0) {
+        if (lane == 0) {
+            int ea = 0, sb = 0;
+            uint32_t pa = 1, pb = 1;                    // parity of the "empty" phase waited for
+            bool alive = true;
+            for (int t = blockIdx.x; alive && t < tiles; t += gridDim.x) {
+                const int mt = t % p.m_tiles, nt = t / p.m_tiles;
+                for (int c = 0; alive && c < p.chunks; ++c) {
+                    const int kc = c * 64;
+                    for (int g = 0; alive && g < groups; ++g) {
+                        if (!mbar_wait(&a_empty[ea], pa, abortp, p.status, 81)) { alive = false; break; }
+                        mbar_arrive_expect_tx(&a_full[ea], (uint32_t)a_bytes);
+                        tma_load_3d(base + ea * a_pitch, &tmA, kc, mt * 128 + (p.tpe == 1 ? p.shift[g] : p.lo), 0, &a_full[ea]);
+                        if (++ea == p.entries) { ea = 0; pa ^= 1u; }
+                        for (int j = 0; j < p.tpe; ++j) {
+                            if (!mbar_wait(&b_empty[sb], pb, abortp, p.status, 82)) { alive = false; break; }
+                            mbar_arrive_expect_tx(&b_full[sb], BB);
+                            tma_load_3d(b_base + sb * BB, &tmB, (g + j) * p.tap_cols + nt * 64, kc, 0, &b_full[sb]);
+                            if (++sb == p.b_stages) { sb = 0; pb ^= 1u; }
+                        }
+                    }
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            int ea = 0, sb = 0, it = 0;
+            uint32_t pa = 0, pb = 0;
+            bool alive = true;
+            const uint64_t a_plane = (uint64_t)(plane_bytes >> 4);
+            for (int t = blockIdx.x; alive && t < tiles; t += gridDim.x, ++it) {
+                const int acc = it % EG;
+                if (!mbar_wait(&d_empty[acc], (((uint32_t)(it / EG)) & 1u) ^ 1u, abortp, p.status, 83)) break;
+                tc_fence_after();
+                const uint32_t d = tmem_d + acc * 192;
+                bool first = true;
+                for (int c = 0; alive && c < p.chunks; ++c)
+                    for (int g = 0; alive && g < groups; ++g) {
+                        if (!mbar_wait(&a_full[ea], pa, abortp, p.status, 84)) { alive = false; break; }
+                        for (int j = 0; j < p.tpe; ++j) {
+                            if (!mbar_wait(&b_full[sb], pb, abortp, p.status, 85)) { alive = false; break; }
+                            tc_fence_after();
+                            const uint32_t row = p.tpe == 1 ? 0 : (uint32_t)(p.shift[j] - p.lo);
+                            const uint64_t a = smem_desc_sw128(base + ea * a_pitch + row * 128);
+                            const uint64_t b = smem_desc_mn(b_base + sb * BB, BB / 3);
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                mma_x3<3, 64>(d, a + 2 * k, a_plane, b + 128 * k, 0, 1, first);   // 32 bytes along A's rows, 16 rows of B
+                                first = false;
+                            }
+                            mma_commit(&b_empty[sb]);
+                            if (++sb == p.b_stages) { sb = 0; pb ^= 1u; }
+                        }
+                        mma_commit(&a_empty[ea]);
+                        if (++ea == p.entries) { ea = 0; pa ^= 1u; }
+                    }
+                if (alive) mma_commit(&d_full[acc]);
+            }
+        }
+    } else {
+        const int grp = (warp - 2) >> 2, q = warp & 3;  // TMEM lane quarter of this warp
+        const int row = q * 32 + lane;
+        int it = grp;
+        for (int t = blockIdx.x + grp * gridDim.x; t < tiles; t += EG * gridDim.x, it += EG) {
+            const int mt = t % p.m_tiles, nt = t / p.m_tiles;
+            const int m = mt * 128 + row;
+            int env = m / p.P, pix = m - env * p.P;
+            int y = pix / p.W, x = pix - y * p.W;
+            if (p.mode == X3_DGRAD_FC) { y = nt / p.W_out; x = nt - y * p.W_out; }
+            if (!mbar_wait_warp(&d_full[grp], ((uint32_t)(it / EG)) & 1u, abortp, p.status, 86)) break;
+            tc_fence_after();
+            const uint32_t taddr = tmem_d + grp * 192 + ((uint32_t)(q * 32) << 16);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                __syncwarp();                           // rows without a destination have left the previous half early
+                bool ok = env < p.n && y < p.H_out && x < p.W_out;
+                size_t off;
+                if (p.mode == X3_DGRAD_S2D) {
+                    const int yy = 2 * y + nt, xx = 2 * x + j;
+                    ok = env < p.n && yy < p.H_out && xx < p.W_out;
+                    off = ((size_t)env * p.P_dst + (size_t)yy * p.W_dst + xx) * p.dst_pitch;
+                } else
+                    off = ((size_t)env * p.P_dst + (size_t)y * p.W_dst + x) * p.dst_pitch + j * 32;
+                uint32_t mk[16];
+                if (ok) {
+                    const uint4* src = reinterpret_cast<const uint4*>(p.mask + (size_t)m * p.mask_pitch + nt * 64 + j * 32);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) reinterpret_cast<uint4*>(mk)[i] = src[i];
+                }
+                float v[32];
+                acc_load32<64>(taddr, j * 32, v, j == 2 - 1, &d_empty[grp]);
+                if (!ok) continue;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {           // positive bf16: sign clear, not zero
+                    if ((int16_t)(mk[i] & 0xffffu) <= 0) v[2 * i] = 0.f;
+                    if ((int16_t)(mk[i] >> 16) <= 0) v[2 * i + 1] = 0.f;
+                }
+                __nv_bfloat16* dst = p.dst + off;
+#pragma unroll
+                for (int h = 0; h < 32; h += 16) {
+                    uint32_t o0[8], o1[8], o2[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) x3_split2(v[h + 2 * i], v[h + 2 * i + 1], o0[i], o1[i], o2[i]);
+                    st_v8(dst + h, o0);
+                    st_v8(dst + p.dst_plane + h, o1);
+                    st_v8(dst + 2 * p.dst_plane + h, o2);
+                }
+            }
+        }
+    }
+    if (*abortp) {                                      // give copies still in flight time to land
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000) { }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(tmem_d, 512);
+}
+
+// One CTA = (kind, range of row chunks).  Warp 0 copies, warp 1 issues, warps 2..5 sum the columns of B while the
+// main loop runs (bias gradient) and write the accumulators at the end.
+// Both operands have the contracted index along their rows (pixels), so tiles go from global memory to the tensor
+// core without a transposition; a tap is a row offset into the slab, and the two taps (or slabs) of a group are two
+// 64-row blocks of M at a free distance (the leading byte offset).  Bound: the tensor core, 208 clocks per 16 rows and
+// group (56 for frames).
+template <int APL, int NB>
+__global__ void __launch_bounds__(192)
+x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const X3WgradParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t full[kMaxStages], empty[kMaxStages], done;
+    __shared__ float s_sum[128][2];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+    volatile int* abortp = &abort_flag;
+    constexpr int BPL = NB == 64 ? 3 : 1;               // NB = 32: the planes are 32-column blocks of one row
+    constexpr int ACC = 3 * NB;
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint8_t* sm = smem_raw + (base - smem_u32(smem_raw));
+    const int a_slab = (APL * p.a_rows * 128 + 1023) & ~1023, b_plane = p.kr * 128, b_slab = BPL * b_plane;
+    const int a_tx = APL * p.a_rows * 128;
+    const int stage_bytes = p.n_a * a_slab + p.n_b * b_slab;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int kind = (int)blockIdx.x / p.ranges;
+    if (kind > p.kinds - 1) kind = p.kinds - 1;
+    const int range = (int)blockIdx.x - kind * p.ranges;
+    const int nr = kind == p.kinds - 1 ? p.last_ranges : p.ranges;
+    const int c0 = (int)((long)p.row_chunks * range / nr), c1 = (int)((long)p.row_chunks * (range + 1) / nr);
+    const int gi0 = kind * p.group_mul;
+    int groups = p.groups;
+    if (gi0 + groups > p.group_cap) groups = p.group_cap - gi0;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kMaxStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], p.bias_part ? 5 : 1); }
+        mbar_init(&done, 1);
+        abort_flag = 0;
+        fence_barrier_init();
+        tma_prefetch_desc(&tmA);
+        tma_prefetch_desc(&tmB);
+    }
+    if (warp == 1) tmem_alloc(&tmem_slot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_d = tmem_slot;
+    pdl_wait();
+    pdl_trigger();
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int s = 0;
+            uint32_t ph = 1;
+            const int a_col = (kind % p.ka) * p.a_step, b_col = (kind / p.ka) * p.b_step;
+            for (int c = c0; c < c1; ++c) {
+                if (!mbar_wait(&empty[s], ph, abortp, p.status, 91)) break;
+                mbar_arrive_expect_tx(&full[s], (uint32_t)(p.n_a * a_tx + p.n_b * b_slab));
+                const uint32_t dst = base + s * stage_bytes;
+                for (int i = 0; i < p.n_a; ++i) {
+                    const int k = kind * p.slab_mul + i;
+                    tma_load_3d(dst + i * a_slab, &tmA, a_col + p.slab_col[k], c * p.kr + p.slab_row[k], 0, &full[s]);
+                }
+                for (int i = 0; i < p.n_b; ++i)
+                    tma_load_3d(dst + p.n_a * a_slab + i * b_slab, &tmB, b_col + 64 * i, c * p.kr, 0, &full[s]);
+                if (++s == p.stages) { s = 0; ph ^= 1u; }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            int s = 0;
+            uint32_t ph = 0;
+            bool alive = true;
+            const uint64_t a_plane = (uint64_t)((p.a_rows * 128) >> 4);
+            const uint32_t b_lbo = NB == 64 ? (uint32_t)b_plane : (uint32_t)b_slab;
+            for (int c = c0; c < c1; ++c) {
+                if (!mbar_wait(&full[s], ph, abortp, p.status, 92)) { alive = false; break; }
+                tc_fence_after();
+                const uint32_t a0 = base + s * stage_bytes, b0 = a0 + p.n_a * a_slab;
+                for (int g = 0; g < groups; ++g) {
+                    const uint64_t a = smem_desc_mn(a0 + p.a_off[gi0 + g], p.a_lbo[gi0 + g]);
+                    const uint64_t b = smem_desc_mn(b0 + p.b_off[g], b_lbo);
+                    for (int k = 0; k < p.kr / 16; ++k)
+                        mma_x3<APL, NB>(tmem_d + g * ACC, a + 128 * k, a_plane, b + 128 * k, 1, 1, c == c0 && k == 0);
+                }
+                mma_commit(&empty[s]);
+                if (++s == p.stages) { s = 0; ph ^= 1u; }
+            }
+            if (alive) mma_commit(&done);
+        }
+    } else {
+        const int wt = threadIdx.x - 64;
+        bool ok = true;
+        if (p.bias_part) {                              // all four warps arrive on each stage; those of kind 0 sum
+            int s = 0;
+            uint32_t ph = 0;
+            float s0 = 0.f, s1 = 0.f;
+            constexpr int TC = NB / 2;                  // threads along the columns (two columns each)
+            const int cp = wt % TC, r0 = wt / TC;
+            for (int c = c0; ok && c < c1; ++c) {
+                ok = mbar_wait_warp(&full[s], ph, abortp, p.status, 93);
+                if (ok && kind == 0) {
+                    const uint8_t* b = sm + s * stage_bytes + p.n_a * a_slab;
+                    for (int r = r0; r < p.kr; r += 128 / TC) {
+                        float t0 = 0.f, t1 = 0.f;
+#pragma unroll
+                        for (int pl = 2; pl >= 0; --pl) {
+                            // byte of the pair inside its 128-byte row, and the row's place (address-based swizzle)
+                            const int col = NB == 64 ? cp * 4 : (pl & 1) * 64 + cp * 4;
+                            const int blk = NB == 64 ? pl : pl >> 1;
+                            const uint32_t off = (uint32_t)(blk * b_plane + r * 128 + (col ^ ((r & 7) << 4)));
+                            const uint32_t w = *reinterpret_cast<const uint32_t*>(b + off);
+                            t0 += __uint_as_float(w << 16); t1 += __uint_as_float(w & 0xffff0000u);
+                        }
+                        s0 += t0; s1 += t1;
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&empty[s]);
+                if (++s == p.stages) { s = 0; ph ^= 1u; }
+            }
+            if (kind == 0) {
+                s_sum[wt][0] = s0; s_sum[wt][1] = s1;
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                if (wt < NB) {
+                    float t = 0.f;
+                    for (int r = 0; r < 128 / TC; ++r) t += s_sum[r * TC + wt / 2][wt & 1];
+                    p.bias_part[range * NB + wt] = t;
+                }
+            }
+        }
+        const int q = warp & 3, m = q * 32 + lane;
+        ok = ok && mbar_wait_warp(&done, 0, abortp, p.status, 94);
+        tc_fence_after();
+        if (ok) {
+            for (int g = 0; g < groups; ++g) {
+                const uint32_t taddr = tmem_d + g * ACC + ((uint32_t)(q * 32) << 16);
+#pragma unroll
+                for (int j = 0; j < NB / 32; ++j) {
+                    float v[32];
+                    acc_load32<NB>(taddr, j * 32, v, false, nullptr);
+                    if (p.fc_w) {
+                        const int o = (kind % p.ka) * 128 + m, pix = (kind / p.ka) * 2 + g;
+                        if (pix < p.P3) {
+                            float* dst = p.fc_w + (size_t)o * 64 * p.P3 + (size_t)(j * 32) * p.P3 + pix;
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) dst[(size_t)i * p.P3] = v[i];
+                        }
+                    } else {
+                        float* dst = p.part + (gi0 + g) * p.group_stride + ((size_t)range * 128 + m) * NB + j * 32;
+#pragma unroll
+                        for (int i = 0; i < 32; i += 8) st_v8(dst + i, reinterpret_cast<const uint32_t*>(v) + i);
+                    }
+                }
+            }
+        }
+    }
+    if (*abortp) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000) { }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(tmem_d, 512);
+}
+
+}  // namespace
+
+bool x3_make_map(CUtensorMap* m, const void* ptr, uint64_t cols, uint64_t rows, uint64_t planes, uint64_t pitch_elems,
+                 uint64_t plane_elems, uint32_t box_rows, uint32_t box_planes)
+{
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[3] = {cols, rows, planes};
+    const cuuint64_t strides[2] = {pitch_elems * 2, plane_elems * 2};
+    const cuuint32_t box[3] = {64, box_rows, box_planes};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool x3_taps_plan(X3TapParams* p, int chunks, int taps, const int* shift)
+{
+    int lo = shift[0], hi = shift[0];
+    for (int i = 0; i < taps; ++i) { lo = shift[i] < lo ? shift[i] : lo; hi = shift[i] > hi ? shift[i] : hi; p->shift[i] = shift[i]; }
+    p->taps = taps; p->lo = lo; p->chunks = chunks;
+    const int bb = 3 * 8192;
+    // every tap reads one A entry shifted; on grids too wide for that (rows of one TMA box, shared memory) each tap
+    // loads its own 128 rows
+    for (int shared = 1; shared >= 0; --shared) {
+        p->tpe = shared ? taps : 1;
+        p->entry_rows = shared ? 128 + hi - lo : 128;
+        if (p->entry_rows > 256) continue;
+        const int a = (3 * p->entry_rows * 128 + 1023) & ~1023;
+        p->entries = taps == 1 ? 3 : 2;
+        int room = kSmemMax - 3 * 1024 - p->entries * a;
+        if (room < 2 * bb) { p->entries = 2; room = kSmemMax - 3 * 1024 - p->entries * a; }
+        if (room < 2 * bb) continue;
+        p->b_stages = room / bb > kMaxStages ? kMaxStages : room / bb;
+        return true;
+    }
+    return false;
+}
+
+hts_status x3_dgrad_launch(const CUtensorMap& a, const CUtensorMap& b, const X3TapParams& p, cudaStream_t s)
+{
+    const int dev = device_slot();
+    static bool attr_set[kDeviceSlots] = {};
+    if (!attr_set[dev]) {
+        HTS_CUDA(cudaFuncSetAttribute(x3_dgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 2048));
+        HTS_CUDA(cudaFuncSetAttribute(x3_dgrad_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+        attr_set[dev] = true;
+    }
+    const int smem = 1024 + p.entries * ((3 * p.entry_rows * 128 + 1023) & ~1023) + p.b_stages * 3 * 8192;
+    const int tiles = p.m_tiles * p.n_tiles, sms = device_sm_count(dev);
+    HTS_CUDA(launch_pdl(x3_dgrad_kernel, dim3(tiles < sms ? tiles : sms), dim3(kDgradThreads), (size_t)smem, s, a, b, p));
+    note_launch();
+    return HTS_OK;
+}
+
+template <int APL, int NB>
+hts_status x3_wgrad_launch(const CUtensorMap& a, const CUtensorMap& b, const X3WgradParams& p, cudaStream_t s)
+{
+    const int dev = device_slot();
+    static bool attr_set[kDeviceSlots] = {};
+    if (!attr_set[dev]) {
+        HTS_CUDA(cudaFuncSetAttribute(x3_wgrad_kernel<APL, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 2048));
+        HTS_CUDA(cudaFuncSetAttribute(x3_wgrad_kernel<APL, NB>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+        attr_set[dev] = true;
+    }
+    const int a_slab = (APL * p.a_rows * 128 + 1023) & ~1023, b_slab = (NB == 64 ? 3 : 1) * p.kr * 128;
+    const int smem = 1024 + p.stages * (p.n_a * a_slab + p.n_b * b_slab);
+    if (smem > kSmemMax - 2048) return HTS_ERR_SHAPE;
+    const int grid = p.ranges * (p.kinds - 1) + p.last_ranges;
+    HTS_CUDA(launch_pdl(x3_wgrad_kernel<APL, NB>, dim3(grid), dim3(192), (size_t)smem, s, a, b, p));
+    note_launch();
+    return HTS_OK;
+}
+template hts_status x3_wgrad_launch<3, 64>(const CUtensorMap&, const CUtensorMap&, const X3WgradParams&, cudaStream_t);
+template hts_status x3_wgrad_launch<1, 32>(const CUtensorMap&, const CUtensorMap&, const X3WgradParams&, cudaStream_t);
+
+}  // namespace hts
