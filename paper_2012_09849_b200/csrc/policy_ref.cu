@@ -21,12 +21,26 @@ __device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b)
 {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
+__device__ __forceinline__ f32x2 pair(float lo, float hi)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ f32x2 both(float v) { return pair(v, v); }
 __device__ __forceinline__ float lane_of(f32x2 v, int i) { return __uint_as_float(i ? (uint32_t)(v >> 32) : (uint32_t)v); }
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
 __device__ __forceinline__ float4 load4(const float* p, bool vec)
 {
     return vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
@@ -48,30 +62,49 @@ struct ConvParams {
     bool s2d;
 };
 
+// Frame of batch row e: e itself, or its slot in the pool (a slot outside it is reported and reads frame 0).
+__device__ __forceinline__ size_t frame_of(const ConvParams& p, int e)
+{
+    if (!p.slots) return (size_t)e;
+    const int sl = p.slots[e];
+    if ((unsigned)sl >= (unsigned)p.pool) { atomicCAS(p.status, 0, kStatusBadSlot); return 0; }
+    return (size_t)sl;
+}
+// Where pixel r of row e starts in the planes.
+__device__ __forceinline__ size_t plane_row(const ConvParams& p, int e, int r)
+{
+    const int i = r / p.Wo, x = r - i * p.Wo;
+    return p.s2d ? ((size_t)e * p.P_rows + (size_t)(i >> 1) * p.W_rows + (x >> 1)) * 128 + ((i & 1) * 2 + (x & 1)) * 32
+                 : ((size_t)e * p.P_rows + r) * 64;
+}
+
 // y[e,o,i,j] = relu(b[o] + in_scale * sum_{c,u,v} w[o,c,u,v] x[e,c,i s+u,j s+v]), summed over (c, u, v) in ascending
-// order.  Implicit GEMM: a block owns PX consecutive output pixels of the batch and OC channels, gathers PX x KC inputs
-// and OC x KC weights per step into shared memory (double-buffered; weights stored twice, as both lanes of a packed
-// multiply-add), a thread owns PP pixel pairs x OT channels.  Bound: the fp32 pipes.  Packed multiply-adds reach
-// 64 TFLOP/s in this pattern where scalar ones stop at 49 (three distinct registers per operation).
-template <typename TIn, int PP, int OT, int WP, int WO, int KC, int PER_SM>
-__global__ void __launch_bounds__(128, PER_SM)
+// order.  Implicit GEMM: a block owns PX consecutive output pixels of the batch and OC channels and gathers PX x KC
+// inputs and OC x KC weights per step into shared memory, one step ahead; a thread owns PXT pixels x OT channels.
+// Bound: the 128 bytes per clock at which shared memory reaches registers (a thread loads 4 (PXT + OT) bytes per
+// PXT x OT multiply-adds) and the fp32 pipes alike.  Packed multiply-adds (two channels each, the input in both lanes)
+// reach 64 TFLOP/s in this pattern where scalar ones stop at 49 (three distinct registers per operation).  8 x 16 per
+// thread loads less but leaves two warps per scheduler: 206 against 171 us (conv2, n = 1024); copying input rows
+// instead of gathering per tap makes the reads scattered: 278 us.
+template <typename TIn, int PXT, int OT, int WPX, int WO, int KC, int PER_SM>
+__global__ void __launch_bounds__(32 * WPX * WO, PER_SM)
 conv_tile_kernel(const ConvParams p)
 {
-    constexpr int PX = WP * 16 * PP, OC = WO * 4 * OT;
+    constexpr int NT = 32 * WPX * WO, PX = WPX * 8 * PXT, OC = WO * 4 * OT;
     constexpr bool U8 = std::is_same<TIn, uint8_t>::value;
-    constexpr int NPX = PX > 128 ? PX / 128 : 1, KL = PX > 128 ? 1 : 128 / PX;   // pixels of a loading thread, threads along k
+    constexpr int NPX = PX > NT ? PX / NT : 1, KL = PX > NT ? 1 : NT / PX;       // pixels of a loading thread, threads along k
     constexpr int UNIT = U8 ? 4 : 1;                                              // inputs per load
     constexpr int NA = KC / UNIT / KL;                                            // loads per pixel of a loading thread
-    constexpr int NW = OC * KC / 4 / 128;
-    static_assert(WP * WO == 4 && NA * UNIT * KL == KC && NW * 512 == OC * KC, "block shape");
+    constexpr int NW = OC * KC / 4 / NT;
+    static_assert(NPX * NT == PX * KL && NA * UNIT * KL == KC && NW * 4 * NT == OC * KC, "block shape");
     extern __shared__ __align__(16) float s_mem[];
     float* sA = s_mem;                                  // [2][KC][PX]
-    float2* sW = reinterpret_cast<float2*>(s_mem + 2 * KC * PX);   // [2][KC][OC]
-    int* s_off = reinterpret_cast<int*>(sW + 2 * KC * OC);         // input offset of each load unit
+    float* sW = s_mem + 2 * KC * PX;                    // [2][KC][OC]
+    int* s_off = reinterpret_cast<int*>(sW + 2 * KC * OC);   // input offset of each load unit
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int K = p.C * p.k * p.k, P = p.Ho * p.Wo;
     const int total = p.n * P, o_base = blockIdx.y * OC;
-    for (int u = tid; u < K / UNIT; u += 128) {
+    for (int u = tid; u < K / UNIT; u += NT) {
         const int kk = u * UNIT, c = kk / (p.k * p.k), r = kk - c * p.k * p.k, uu = r / p.k;
         s_off[u] = (c * p.H + uu) * p.W + (r - uu * p.k);
     }
@@ -80,37 +113,35 @@ conv_tile_kernel(const ConvParams p)
     const TIn* src[NPX];
 #pragma unroll
     for (int q = 0; q < NPX; ++q) {
-        int px = blockIdx.x * PX + (NPX > 1 ? tid + 128 * q : tid % PX);
+        int px = blockIdx.x * PX + (NPX > 1 ? tid + NT * q : tid % PX);
         px = px < total ? px : total - 1;
         const int e = px / P, r = px - e * P, i = r / p.Wo, j = r - i * p.Wo;
-        size_t frame = (size_t)e;
-        if (p.slots) {
-            const int sl = p.slots[e];
-            if ((unsigned)sl >= (unsigned)p.pool) { atomicCAS(p.status, 0, kStatusBadSlot); frame = 0; }
-            else frame = (size_t)sl;
-        }
-        src[q] = static_cast<const TIn*>(p.x) + frame * p.C * p.H * p.W + (size_t)(i * p.s) * p.W + j * p.s;
+        src[q] = static_cast<const TIn*>(p.x) + frame_of(p, e) * p.C * p.H * p.W + (size_t)(i * p.s) * p.W + j * p.s;
     }
     __syncthreads();
-    const int kl = NPX > 1 ? 0 : tid / PX, pl = tid % PX;
+    const int kl = NPX > 1 ? 0 : tid / PX, pl = NPX > 1 ? tid : tid % PX;
     uint32_t ra[U8 ? NPX * NA : 1];
     float4 rw[NW];
     auto fetch = [&](int k0, int buf) {
+        int off[NA];                                    // all of them first: a copy may not be moved across another one
 #pragma unroll
-        for (int q = 0; q < NPX; ++q)
+        for (int a = 0; a < NA; ++a) off[a] = s_off[k0 / UNIT + kl * NA + a];
 #pragma unroll
-            for (int a = 0; a < NA; ++a) {
-                const int u = a * KL + kl;
-                const TIn* s = src[q] + s_off[k0 / UNIT + u];
+        for (int a = 0; a < NA; ++a) {
+            const int u = kl * NA + a;
+#pragma unroll
+            for (int q = 0; q < NPX; ++q) {
+                const TIn* s = src[q] + off[a];
                 if constexpr (U8) {
                     if (p.words) ra[q * NA + a] = *reinterpret_cast<const uint32_t*>(s);
                     else ra[q * NA + a] = s[0] | (uint32_t)s[1] << 8 | (uint32_t)s[2] << 16 | (uint32_t)s[3] << 24;
                 } else
-                    cp_async4((uint32_t)__cvta_generic_to_shared(sA + (buf * KC + u) * PX + pl + 128 * q), s);
+                    cp_async4((uint32_t)__cvta_generic_to_shared(sA + (buf * KC + u) * PX + pl + NT * q), s);
             }
+        }
 #pragma unroll
         for (int a = 0; a < NW; ++a) {
-            const int u = a * 128 + tid, o = u % OC, kq = u / OC;
+            const int u = a * NT + tid, o = u % OC, kq = u / OC;
             rw[a] = load4(p.w + (size_t)(o_base + o) * K + k0 + 4 * kq, p.w_vec);
         }
     };
@@ -122,262 +153,346 @@ conv_tile_kernel(const ConvParams p)
                 for (int a = 0; a < NA; ++a)
 #pragma unroll
                     for (int b = 0; b < 4; ++b)
-                        sA[(buf * KC + (a * KL + kl) * 4 + b) * PX + pl + 128 * q] = (float)((ra[q * NA + a] >> (8 * b)) & 0xffu);
+                        sA[(buf * KC + (kl * NA + a) * 4 + b) * PX + pl + NT * q] = (float)((ra[q * NA + a] >> (8 * b)) & 0xffu);
         }
 #pragma unroll
         for (int a = 0; a < NW; ++a) {
-            const int u = a * 128 + tid, o = u % OC, kq = u / OC;
-            float2* d = sW + (buf * KC + 4 * kq) * OC + o;
-            d[0] = make_float2(rw[a].x, rw[a].x); d[OC] = make_float2(rw[a].y, rw[a].y);
-            d[2 * OC] = make_float2(rw[a].z, rw[a].z); d[3 * OC] = make_float2(rw[a].w, rw[a].w);
+            const int u = a * NT + tid, o = u % OC, kq = u / OC;
+            float* d = sW + (buf * KC + 4 * kq) * OC + o;
+            d[0] = rw[a].x; d[OC] = rw[a].y; d[2 * OC] = rw[a].z; d[3 * OC] = rw[a].w;
         }
     };
-    const int wp = warp % WP, wo = warp / WP, g = lane & 7, og = lane >> 3;
-    const int px_t = wp * 16 * PP + 2 * g, o_t = wo * 4 * OT + og * OT;   // pairs at px_t + 16 q
-    f32x2 acc[PP][OT];
+    const int wp = warp % WPX, wo = warp / WPX, g = lane & 7, og = lane >> 3;
+    const int px_t = wp * 8 * PXT + g, o_t = wo * 4 * OT + og * OT;              // pixels px_t + 8 q
+    f32x2 acc[PXT][OT / 2];
 #pragma unroll
-    for (int q = 0; q < PP; ++q)
+    for (int q = 0; q < PXT; ++q)
 #pragma unroll
-        for (int j = 0; j < OT; ++j) acc[q][j] = 0;
+        for (int j = 0; j < OT / 2; ++j) acc[q][j] = 0;
+    const int chunks = K / KC;
     fetch(0, 0);
     store(0);
-    cp_async_wait();
+    cp_async_wait_all();
     __syncthreads();
-    int buf = 0;
-    for (int k0 = 0; k0 < K; k0 += KC, buf ^= 1) {
-        const bool more = k0 + KC < K;
-        if (more) fetch(k0 + KC, buf ^ 1);
-#pragma unroll 8
+    for (int c = 0; c < chunks; ++c) {
+        const int buf = c & 1;
+        if (c + 1 < chunks) fetch((c + 1) * KC, buf ^ 1);
+#pragma unroll 16
         for (int kk = 0; kk < KC; ++kk) {
-            f32x2 xv[PP], wv[OT];
             const float* a = sA + (buf * KC + kk) * PX + px_t;
-            const float2* w = sW + (buf * KC + kk) * OC + o_t;
+            const float* w = sW + (buf * KC + kk) * OC + o_t;
+            f32x2 wv[OT / 2];
 #pragma unroll
-            for (int q = 0; q < PP; ++q) xv[q] = *reinterpret_cast<const f32x2*>(a + 16 * q);
-#pragma unroll
-            for (int j = 0; j < OT; j += 2) {
-                const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(w + j);
+            for (int j = 0; j < OT / 2; j += 2) {
+                const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(w + 2 * j);
                 wv[j] = t.x; wv[j + 1] = t.y;
             }
 #pragma unroll
-            for (int q = 0; q < PP; ++q)
+            for (int q = 0; q < PXT; ++q) {
+                const f32x2 xx = both(a[8 * q]);
 #pragma unroll
-                for (int j = 0; j < OT; ++j) fma2(acc[q][j], xv[q], wv[j]);
+                for (int j = 0; j < OT / 2; ++j) fma2(acc[q][j], xx, wv[j]);
+            }
         }
-        if (more) {
+        if (c + 1 < chunks) {
             store(buf ^ 1);
-            cp_async_wait();
+            cp_async_wait_all();
             __syncthreads();
         }
     }
 #pragma unroll
-    for (int q = 0; q < PP; ++q)
+    for (int q = 0; q < PXT; ++q) {
+        const int px = blockIdx.x * PX + px_t + 8 * q;
+        if (px >= total) continue;
+        const int e = px / P, r = px - e * P;
+        float v[OT];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int px = blockIdx.x * PX + px_t + 16 * q + h;
-            if (px >= total) continue;
-            const int e = px / P, r = px - e * P;
-            float v[OT];
+        for (int j = 0; j < OT; ++j) {
+            const float t = fmaf(lane_of(acc[q][j / 2], j & 1), p.in_scale, p.b[o_base + o_t + j]);
+            v[j] = t > 0.f ? t : 0.f;
+            p.y[((size_t)e * p.O + o_base + o_t + j) * P + r] = v[j];
+        }
+        if (p.planes) {
+            __nv_bfloat16* d = p.planes + plane_row(p, e, r) + o_base + o_t;
 #pragma unroll
-            for (int j = 0; j < OT; ++j) {
-                const float t = fmaf(lane_of(acc[q][j], h), p.in_scale, p.b[o_base + o_t + j]);
-                v[j] = t > 0.f ? t : 0.f;
-                p.y[((size_t)e * p.O + o_base + o_t + j) * P + r] = v[j];
-            }
-            if (p.planes) {
-                const int i = r / p.Wo, x = r - i * p.Wo;
-                const size_t at = p.s2d ? ((size_t)e * p.P_rows + (size_t)(i >> 1) * p.W_rows + (x >> 1)) * 128 + ((i & 1) * 2 + (x & 1)) * 32
-                                        : ((size_t)e * p.P_rows + r) * 64;
-                uint32_t o0[OT / 2], o1[OT / 2], o2[OT / 2];
-#pragma unroll
-                for (int j = 0; j < OT / 2; ++j) x3_split2(v[2 * j], v[2 * j + 1], o0[j], o1[j], o2[j]);
-                __nv_bfloat16* d = p.planes + at + o_base + o_t;
-                if constexpr (OT == 8) {
-                    *reinterpret_cast<uint4*>(d) = make_uint4(o0[0], o0[1], o0[2], o0[3]);
-                    *reinterpret_cast<uint4*>(d + p.plane) = make_uint4(o1[0], o1[1], o1[2], o1[3]);
-                    *reinterpret_cast<uint4*>(d + 2 * p.plane) = make_uint4(o2[0], o2[1], o2[2], o2[3]);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < OT / 2; ++j) {
-                        reinterpret_cast<uint32_t*>(d)[j] = o0[j];
-                        reinterpret_cast<uint32_t*>(d + p.plane)[j] = o1[j];
-                        reinterpret_cast<uint32_t*>(d + 2 * p.plane)[j] = o2[j];
-                    }
-                }
+            for (int j = 0; j < OT; j += 4) {
+                uint2 o0, o1, o2;
+                x3_split2(v[j], v[j + 1], o0.x, o1.x, o2.x);
+                x3_split2(v[j + 2], v[j + 3], o0.y, o1.y, o2.y);
+                *reinterpret_cast<uint2*>(d + j) = o0;
+                *reinterpret_cast<uint2*>(d + p.plane + j) = o1;
+                *reinterpret_cast<uint2*>(d + 2 * p.plane + j) = o2;
             }
         }
-}
-
-template <typename TIn, int PP, int OT, int WP, int WO, int KC, int PER_SM>
-hts_status launch_conv_tile(const ConvParams& p, cudaStream_t s)
-{
-    constexpr int PX = WP * 16 * PP, OC = WO * 4 * OT;
-    const int K = p.C * p.k * p.k;
-    const size_t smem = sizeof(float) * (2 * KC * PX + 4 * KC * OC) + sizeof(int) * (size_t)(K / (std::is_same<TIn, uint8_t>::value ? 4 : 1));
-    auto kernel = conv_tile_kernel<TIn, PP, OT, WP, WO, KC, PER_SM>;
-    static size_t smem_set_by_device[kDeviceSlots] = {};
-    size_t& smem_set = smem_set_by_device[device_slot()];
-    if (!smem_set || smem > smem_set) {
-        HTS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        HTS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        smem_set = smem;
     }
-    const size_t px = (size_t)p.n * p.Ho * p.Wo;
-    HTS_CUDA(launch_pdl(kernel, dim3((unsigned)((px + PX - 1) / PX), (unsigned)(p.O / OC)), dim3(128), smem, s, p));
-    note_launch();
-    return HTS_OK;
 }
 
-// The largest tile that still gives every SM two blocks: larger tiles load less per multiply-add, smaller ones
-// spread a small batch over the device.
+// The same sums for batches too small to fill the device with tiles: 16 pixels x 32 channels per block of 128 threads,
+// 2 x 2 per thread, K in groups of 64 that are all requested at once (up to kSmallRing of them) and multiplied as they
+// arrive.  Inputs and weights stay in K order, four of it per load.  Bound: latency, about one warp per scheduler.
+constexpr int kSmallK = 64, kSmallPitch = kSmallK + 4, kSmallPx = 16, kSmallOc = 32, kSmallRing = 12;
 template <typename TIn>
-hts_status launch_conv(const ConvParams& p, cudaStream_t s)
+__global__ void __launch_bounds__(128)
+conv_small_kernel(const ConvParams p, int ring)
 {
-    const size_t px = (size_t)p.n * p.Ho * p.Wo, want = 2 * (size_t)device_sm_count(device_slot());
-    if (p.O == 64 && px >= 128 * want) return launch_conv_tile<TIn, 4, 8, 2, 2, 16, 4>(p, s);
-    if (p.O == 32 && px >= 256 * want) return launch_conv_tile<TIn, 4, 8, 4, 1, 16, 4>(p, s);
-    if (px * p.O >= 64 * 32 * want) return launch_conv_tile<TIn, 2, 4, 2, 2, 32, 4>(p, s);
-    return launch_conv_tile<TIn, 1, 2, 1, 4, 64, 4>(p, s);
-}
-
-// h[e,o] = relu(b[o] + sum over lanes l of (chain of f = l, l+32, l+64, ...)), the 32 chains added as a binary tree
-// over the lane number (halves first).  512 threads: warp q runs chain q and then chain q + 16 for the block's whole
-// TE x TO tile (a thread: PP row pairs x OT outputs), keeping the first result in shared memory; the tree closes
-// across the warps.  Bound: the fp32 pipes for large batches, the weights' L2 traffic (block rows x 6.4 MB) below.
-template <int PP, int OT, int PER_SM>
-__global__ void __launch_bounds__(512, PER_SM)
-fc_tile_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ b,
-               float* __restrict__ h, int n, int F, int O, bool w_vec)
-{
-    constexpr int TE = 16 * PP, TO = 4 * OT, NT = PP * OT * 2;
-    constexpr int UX = TE * 8, UW = TO * 8;             // float4 loads per step of two chain elements (2 x 16 lanes)
-    constexpr int NX = (UX + 511) / 512, NWL = (UW + 511) / 512;
-    extern __shared__ __align__(16) float s_mem[];
-    float* sX = s_mem;                                  // [2][32][TE], rows (element, lane), columns swizzled
-    float2* sW = reinterpret_cast<float2*>(s_mem + 2 * 32 * TE);   // [2][32][TO]
-    float* sH = reinterpret_cast<float*>(sW + 2 * 32 * TO);        // [NT][512], later [16][TE * TO]
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane & 7, og = lane >> 3;
-    const int e0 = blockIdx.y * TE, o0 = blockIdx.x * TO;
-    constexpr int SX = TE >= 32 ? 3 : 1, SW = TO >= 32 ? 3 : 0;   // swizzle by groups of 8 columns
-    float4 rx[NX], rw[NWL];
-    // unit u: row r = u / 8, four lanes l4 = u % 4 of element (u / 4) % 2
-    auto fetch = [&](int f0) {
+    constexpr bool U8 = std::is_same<TIn, uint8_t>::value;
+    extern __shared__ __align__(16) float s_mem[];      // [ring][16 + 32][pitch]
+    __shared__ const TIn* s_src[kSmallPx];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int kk2 = p.k * p.k, K = p.C * kk2, P = p.Ho * p.Wo, groups = K / kSmallK;
+    const int total = p.n * P, px0 = blockIdx.x * kSmallPx, o_base = blockIdx.y * kSmallOc;
+    auto fetch_w = [&](int gr, int slot) {
+        float* dst = s_mem + (slot * (kSmallPx + kSmallOc) + kSmallPx) * kSmallPitch;
 #pragma unroll
-        for (int a = 0; a < NX; ++a) {
-            const int u = a * 512 + tid, r = u >> 3;
-            if (UX % 512 == 0 || u < UX) rx[a] = *reinterpret_cast<const float4*>(x + (size_t)min(e0 + r, n - 1) * F + f0 + ((u >> 2) & 1) * 32 + (u & 3) * 4);
-        }
-#pragma unroll
-        for (int a = 0; a < NWL; ++a) {
-            const int u = a * 512 + tid, r = u >> 3;
-            if (UW % 512 == 0 || u < UW) rw[a] = load4(w + (size_t)(o0 + r) * F + f0 + ((u >> 2) & 1) * 32 + (u & 3) * 4, w_vec);
+        for (int a = 0; a < kSmallOc * kSmallK / 4 / 128; ++a) {
+            const int u = a * 128 + tid, o = u >> 4, q = (u & 15) * 4;
+            const float* src = p.w + (size_t)(o_base + o) * K + gr * kSmallK + q;
+            const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + o * kSmallPitch + q);
+            if (p.w_vec) cp_async16(d, src);
+            else
+                for (int i = 0; i < 4; ++i) cp_async4(d + 4 * i, src + i);
         }
     };
-    auto store = [&](int buf) {
+    auto fetch_x = [&](int gr, int slot) {
+        float* dst = s_mem + slot * (kSmallPx + kSmallOc) * kSmallPitch;
+        if constexpr (U8) {
 #pragma unroll
-        for (int a = 0; a < NX; ++a) {
-            const int u = a * 512 + tid, r = u >> 3, row = ((u >> 2) & 1) * 16 + (u & 3) * 4;
-            if (UX % 512 == 0 || u < UX) {
-                float* d = sX + (buf * 32 + row) * TE + (r ^ ((u & SX) << 3));
-                d[0] = rx[a].x; d[TE] = rx[a].y; d[2 * TE] = rx[a].z; d[3 * TE] = rx[a].w;
+            for (int a = 0; a < kSmallPx * kSmallK / 4 / 128; ++a) {
+                const int u = a * 128 + tid, px = u >> 4, k = gr * kSmallK + (u & 15) * 4;
+                const int c = k / kk2, r = k - c * kk2, uu = r / p.k;
+                const TIn* s = s_src[px] + (c * p.H + uu) * p.W + (r - uu * p.k);
+                uint32_t w;
+                if (p.words) w = *reinterpret_cast<const uint32_t*>(s);
+                else w = s[0] | (uint32_t)s[1] << 8 | (uint32_t)s[2] << 16 | (uint32_t)s[3] << 24;
+                *reinterpret_cast<float4*>(dst + px * kSmallPitch + (u & 15) * 4) =
+                    make_float4((float)(w & 0xffu), (float)((w >> 8) & 0xffu), (float)((w >> 16) & 0xffu), (float)(w >> 24));
             }
-        }
+        } else {
+            const int k = gr * kSmallK + (tid & 63), c = k / kk2, r = k - c * kk2, uu = r / p.k;
+            const int off = (c * p.H + uu) * p.W + (r - uu * p.k);
 #pragma unroll
-        for (int a = 0; a < NWL; ++a) {
-            const int u = a * 512 + tid, r = u >> 3, row = ((u >> 2) & 1) * 16 + (u & 3) * 4;
-            if (UW % 512 == 0 || u < UW) {
-                float2* d = sW + (buf * 32 + row) * TO + (r ^ ((u & SW) << 3));
-                d[0] = make_float2(rw[a].x, rw[a].x); d[TO] = make_float2(rw[a].y, rw[a].y);
-                d[2 * TO] = make_float2(rw[a].z, rw[a].z); d[3 * TO] = make_float2(rw[a].w, rw[a].w);
+            for (int a = 0; a < kSmallPx / 2; ++a) {
+                const int px = 2 * a + (tid >> 6);
+                cp_async4((uint32_t)__cvta_generic_to_shared(dst + px * kSmallPitch + (tid & 63)), s_src[px] + off);
             }
         }
     };
     pdl_wait();
     pdl_trigger();
-    const int steps = F / 64;
-    const int xs = ((warp >> 2) & SX) << 3, ws = ((warp >> 2) & SW) << 3;   // this warp's rows: lane group warp / 4
-    f32x2 acc[PP][OT];
-    for (int half = 0; half < 2; ++half) {
-#pragma unroll
-        for (int q = 0; q < PP; ++q)
-#pragma unroll
-            for (int j = 0; j < OT; ++j) acc[q][j] = 0;
-        fetch(half * 16);
-        __syncthreads();
-        store(0);
-        __syncthreads();
-        for (int s = 0; s < steps; ++s) {
-            if (s + 1 < steps) fetch((s + 1) * 64 + half * 16);
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                f32x2 xv[PP], wv[OT];
-                const float* xr = sX + ((s & 1) * 32 + i * 16 + warp) * TE;
-                const float2* wr = sW + ((s & 1) * 32 + i * 16 + warp) * TO;
-#pragma unroll
-                for (int q = 0; q < PP; ++q) xv[q] = *reinterpret_cast<const f32x2*>(xr + ((16 * q + 2 * g) ^ xs));
-#pragma unroll
-                for (int j = 0; j < OT; j += 2) {
-                    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(wr + ((og * OT + j) ^ ws));
-                    wv[j] = t.x; wv[j + 1] = t.y;
-                }
-#pragma unroll
-                for (int q = 0; q < PP; ++q)
-#pragma unroll
-                    for (int j = 0; j < OT; ++j) fma2(acc[q][j], xv[q], wv[j]);
-            }
-            if (s + 1 < steps) store((s + 1) & 1);
-            __syncthreads();
-        }
-        if (half == 0) {
-#pragma unroll
-            for (int q = 0; q < PP; ++q)
-#pragma unroll
-                for (int j = 0; j < OT; ++j) {
-                    sH[(2 * (q * OT + j)) * 512 + tid] = lane_of(acc[q][j], 0);
-                    sH[(2 * (q * OT + j) + 1) * 512 + tid] = lane_of(acc[q][j], 1);
-                }
-        }
+    for (int g = 0; g < ring; ++g) fetch_w(g, g);
+    if (tid < kSmallPx) {
+        int px = px0 + tid;
+        px = px < total ? px : total - 1;
+        const int e = px / P, r = px - e * P, i = r / p.Wo, j = r - i * p.Wo;
+        s_src[tid] = static_cast<const TIn*>(p.x) + frame_of(p, e) * p.C * p.H * p.W + (size_t)(i * p.s) * p.W + j * p.s;
     }
-    // level 16: chains q and q + 16, both of this thread; then one plane per warp for the levels 8, 4, 2, 1
-    float v[NT];
+    __syncthreads();
+    for (int g = 0; g < ring; ++g) {
+        fetch_x(g, g);
+        cp_async_commit();
+    }
+    const int g8 = lane & 7, og = lane >> 3, o_t = warp * 8 + og * 2;            // pixels g8, g8 + 8; channels o_t, o_t + 1
+    float a00 = 0.f, a01 = 0.f, a10 = 0.f, a11 = 0.f;                            // [pixel][channel]
+    for (int gr = 0, slot = 0; gr < groups; ++gr) {
+        // groups still in flight may be as many as were requested after this one
+        const int later = groups - 1 - gr < ring - 1 ? groups - 1 - gr : ring - 1;
+        if (later >= 8) cp_async_wait<8>(); else if (later >= 4) cp_async_wait<4>(); else if (later >= 2) cp_async_wait<2>();
+        else if (later == 1) cp_async_wait<1>(); else cp_async_wait<0>();
+        __syncthreads();
+        const float* x = s_mem + (slot * (kSmallPx + kSmallOc) + g8) * kSmallPitch;
+        const float* w = s_mem + (slot * (kSmallPx + kSmallOc) + kSmallPx + o_t) * kSmallPitch;
 #pragma unroll
-    for (int q = 0; q < PP; ++q)
-#pragma unroll
-        for (int j = 0; j < OT; ++j) {
-            const int i = 2 * (q * OT + j);
-            v[i] = sH[i * 512 + tid] + lane_of(acc[q][j], 0);
-            v[i + 1] = sH[(i + 1) * 512 + tid] + lane_of(acc[q][j], 1);
+        for (int k = 0; k < kSmallK; k += 4) {
+            const float4 x0 = *reinterpret_cast<const float4*>(x + k), x1 = *reinterpret_cast<const float4*>(x + 8 * kSmallPitch + k);
+            const float4 w0 = *reinterpret_cast<const float4*>(w + k), w1 = *reinterpret_cast<const float4*>(w + kSmallPitch + k);
+            a00 = fmaf(w0.x, x0.x, a00); a01 = fmaf(w1.x, x0.x, a01); a10 = fmaf(w0.x, x1.x, a10); a11 = fmaf(w1.x, x1.x, a11);
+            a00 = fmaf(w0.y, x0.y, a00); a01 = fmaf(w1.y, x0.y, a01); a10 = fmaf(w0.y, x1.y, a10); a11 = fmaf(w1.y, x1.y, a11);
+            a00 = fmaf(w0.z, x0.z, a00); a01 = fmaf(w1.z, x0.z, a01); a10 = fmaf(w0.z, x1.z, a10); a11 = fmaf(w1.z, x1.z, a11);
+            a00 = fmaf(w0.w, x0.w, a00); a01 = fmaf(w1.w, x0.w, a01); a10 = fmaf(w0.w, x1.w, a10); a11 = fmaf(w1.w, x1.w, a11);
         }
-    __syncthreads();
+        if (gr + ring < groups) {
+            __syncthreads();
+            fetch_w(gr + ring, slot);
+            fetch_x(gr + ring, slot);
+        }
+        cp_async_commit();
+        slot = slot + 1 == ring ? 0 : slot + 1;
+    }
 #pragma unroll
-    for (int q = 0; q < PP; ++q)
+    for (int q = 0; q < 2; ++q) {
+        const int px = px0 + g8 + 8 * q;
+        if (px >= total) continue;
+        const int e = px / P, r = px - e * P, o = o_base + o_t;
+        float v[2];
 #pragma unroll
-        for (int j = 0; j < OT; ++j)
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh)
-                sH[warp * (TE * TO) + (16 * q + 2 * g + hh) * TO + og * OT + j] = v[2 * (q * OT + j) + hh];
-    __syncthreads();
-    for (int i = tid; i < TE * TO; i += 512) {
-        const int e = e0 + i / TO, o = o0 + i % TO;
-        if (e >= n) break;
-        float t[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) t[q] = sH[q * (TE * TO) + i];
-#pragma unroll
-        for (int m = 8; m > 0; m >>= 1)
-#pragma unroll
-            for (int q = 0; q < m; ++q) t[q] = t[q] + t[q + m];
-        const float r = t[0] + b[o];
-        h[(size_t)e * O + o] = r > 0.f ? r : 0.f;
+        for (int j = 0; j < 2; ++j) {
+            const float t = fmaf(q ? (j ? a11 : a10) : (j ? a01 : a00), p.in_scale, p.b[o + j]);
+            v[j] = t > 0.f ? t : 0.f;
+            p.y[((size_t)e * p.O + o + j) * P + r] = v[j];
+        }
+        if (p.planes) {
+            uint32_t o0, o1, o2;
+            x3_split2(v[0], v[1], o0, o1, o2);
+            uint32_t* d = reinterpret_cast<uint32_t*>(p.planes + plane_row(p, e, r) + o);
+            d[0] = o0; d[p.plane / 2] = o1; d[p.plane] = o2;
+        }
     }
 }
 
-template <int PP, int OT, int PER_SM>
-hts_status launch_fc_tile(const float* x, const float* w, const float* b, float* h, int n, int F, cudaStream_t s)
+template <typename TIn>
+hts_status launch_conv_small(const ConvParams& p, cudaStream_t s)
 {
-    constexpr int TE = 16 * PP, TO = 4 * OT;
-    constexpr int smem = (2 * 32 * TE + 4 * 32 * TO + PP * OT * 2 * 512) * (int)sizeof(float);
-    auto kernel = fc_tile_kernel<PP, OT, PER_SM>;
+    const int groups = p.C * p.k * p.k / kSmallK, ring = groups < kSmallRing ? groups : kSmallRing;
+    const int smem = ring * (kSmallPx + kSmallOc) * kSmallPitch * (int)sizeof(float);
+    static int smem_set_by_device[kDeviceSlots] = {};
+    int& smem_set = smem_set_by_device[device_slot()];
+    if (smem > smem_set) {
+        HTS_CUDA(cudaFuncSetAttribute(conv_small_kernel<TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        HTS_CUDA(cudaFuncSetAttribute(conv_small_kernel<TIn>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+        smem_set = smem;
+    }
+    const size_t px = (size_t)p.n * p.Ho * p.Wo;
+    HTS_CUDA(launch_pdl(conv_small_kernel<TIn>, dim3((unsigned)((px + kSmallPx - 1) / kSmallPx), (unsigned)(p.O / kSmallOc)), dim3(128),
+                        (size_t)smem, s, p, ring));
+    note_launch();
+    return HTS_OK;
+}
+
+template <typename TIn, int PXT, int OT, int WPX, int WO, int KC, int PER_SM>
+hts_status launch_conv_tile(const ConvParams& p, cudaStream_t s)
+{
+    constexpr int NT = 32 * WPX * WO, PX = WPX * 8 * PXT, OC = WO * 4 * OT;
+    const int K = p.C * p.k * p.k;
+    const size_t smem = sizeof(float) * (2 * KC * PX + 2 * KC * OC) + sizeof(int) * (size_t)(K / (std::is_same<TIn, uint8_t>::value ? 4 : 1));
+    auto kernel = conv_tile_kernel<TIn, PXT, OT, WPX, WO, KC, PER_SM>;
+    static size_t smem_set_by_device[kDeviceSlots] = {};
+    size_t& smem_set = smem_set_by_device[device_slot()];
+    if (smem > smem_set) {
+        HTS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        HTS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+        smem_set = smem;
+    }
+    const size_t px = (size_t)p.n * p.Ho * p.Wo;
+    HTS_CUDA(launch_pdl(kernel, dim3((unsigned)((px + PX - 1) / PX), (unsigned)(p.O / OC)), dim3(NT), smem, s, p));
+    note_launch();
+    return HTS_OK;
+}
+
+// 128 x 64 (256 x 32) tiles from two per SM on: they load least per multiply-add.  Below, 64 x 32 tiles of four warps
+// while every second SM gets one (n = 256: 229 us per step, 266 with two warps of 4 x 8 per tile), else the latency form.
+template <typename TIn>
+hts_status launch_conv(const ConvParams& p, cudaStream_t s)
+{
+    const size_t px = (size_t)p.n * p.Ho * p.Wo, sms = (size_t)device_sm_count(device_slot());
+    if (p.O == 64 && px >= 128 * 2 * sms) return launch_conv_tile<TIn, 8, 8, 2, 2, 16, 4>(p, s);
+    if (p.O == 32 && px >= 256 * 2 * sms) return launch_conv_tile<TIn, 8, 8, 4, 1, 16, 4>(p, s);
+    if (px * p.O >= 64 * 16 * sms) return launch_conv_tile<TIn, 4, 4, 2, 2, 32, 5>(p, s);
+    return launch_conv_small<TIn>(p, s);
+}
+
+// h[e,o] = relu(b[o] + sum over lanes l of (chain of f = l, l+32, l+64, ...)), the 32 chains added as a binary tree
+// over the lane number (halves first).  A warp owns TE rows x TO outputs and lane l runs chain l of all of them: both
+// operands are contiguous across the lanes, so neither needs a transposition, and one transposing reduction closes
+// the tree (at each level a lane keeps half of its values and gets its partner's share of them).
+// The block's rows of x and w go through a ring in shared memory, 64 columns at a time.  Bound: large batches by
+// shared memory and the fp32 pipes (8 x 8 per warp: one byte per multiply-add, 128 of each per clock; 8 x 16 leaves too
+// few warps, 149 against 115 us at n = 1024), small ones by the latency of the weights: narrow tiles, deep ring.
+template <int TE, int TO, int WE, int WO, int STAGES>
+__global__ void __launch_bounds__(32 * WE * WO)
+fc_chain_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ b,
+                float* __restrict__ h, int n, int F, bool w_vec)
+{
+    constexpr int NV = TE * TO, RX = TE * WE, RW = TO * WO, NT = 32 * WE * WO, UNITS = (RX + RW) * 16;   // 16-byte pieces of a stage
+    extern __shared__ __align__(16) float s_mem[];      // [STAGES][RX + RW][64]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int we = warp % WE, wo = warp / WE;
+    const int e0 = (blockIdx.y * WE + we) * TE, o0 = (blockIdx.x * WO + wo) * TO;
+    pdl_wait();
+    pdl_trigger();
+    f32x2 acc[TE][TO / 2];
+#pragma unroll
+    for (int i = 0; i < TE; ++i)
+#pragma unroll
+        for (int j = 0; j < TO / 2; ++j) acc[i][j] = 0;
+    auto fetch = [&](int f, int st) {
+        float* dst = s_mem + st * (RX + RW) * 64;
+#pragma unroll
+        for (int a = 0; a < (UNITS + NT - 1) / NT; ++a) {
+            const int u = a * NT + threadIdx.x, r = u >> 4, q = (u & 15) * 4;
+            if (UNITS % NT && u >= UNITS) break;
+            const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + r * 64 + q);
+            if (r < RX) cp_async16(d, x + (size_t)min((int)(blockIdx.y * RX) + r, n - 1) * F + f + q);
+            else {
+                const float* src = w + (size_t)(blockIdx.x * RW + r - RX) * F + f + q;
+                if (w_vec) cp_async16(d, src);
+                else
+                    for (int i = 0; i < 4; ++i) cp_async4(d + 4 * i, src + i);
+            }
+        }
+    };
+    const int steps = F / 64;
+#pragma unroll
+    for (int s = 0; s < STAGES - 1; ++s) {
+        if (s < steps) fetch(64 * s, s);
+        cp_async_commit();
+    }
+    for (int s = 0; s < steps; ++s) {
+        cp_async_wait<STAGES - 2>();
+        __syncthreads();                                // stage s has landed for every thread; stage s - 1 is free
+        if (s + STAGES - 1 < steps) fetch(64 * (s + STAGES - 1), (s + STAGES - 1) % STAGES);
+        cp_async_commit();
+        const float* xr = s_mem + (s % STAGES) * (RX + RW) * 64 + we * TE * 64 + lane;
+        const float* wr = s_mem + (s % STAGES) * (RX + RW) * 64 + (RX + wo * TO) * 64 + lane;
+        float xv[2][TE], wv[2][TO];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+#pragma unroll
+            for (int j = 0; j < TO; ++j) wv[k][j] = wr[64 * j + 32 * k];
+#pragma unroll
+            for (int i = 0; i < TE; ++i) xv[k][i] = xr[64 * i + 32 * k];
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int i = 0; i < TE; ++i) {
+                const f32x2 xx = both(xv[k][i]);
+#pragma unroll
+                for (int j = 0; j < TO / 2; ++j) fma2(acc[i][j], xx, pair(wv[k][2 * j], wv[k][2 * j + 1]));
+            }
+    }
+    float v[NV];
+#pragma unroll
+    for (int i = 0; i < TE; ++i)
+#pragma unroll
+        for (int j = 0; j < TO; ++j) v[i * TO + j] = lane_of(acc[i][j / 2], j & 1);
+    int id = 0;                                         // (row, output) of v[0]
+#pragma unroll
+    for (int m = 16, len = NV / 2; m > 0; m >>= 1, len >>= 1) {
+        if (len >= 1) {
+            const bool up = lane & m;
+#pragma unroll
+            for (int k = 0; k < len; ++k) {
+                const float send = up ? v[k] : v[k + len], keep = up ? v[k + len] : v[k];
+                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+            }
+            id += up ? len : 0;
+        } else
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], m);
+    }
+    constexpr int LEFT = NV >= 32 ? NV / 32 : 1;
+#pragma unroll
+    for (int k = 0; k < LEFT; ++k) {
+        const int e = e0 + (id + k) / TO, o = o0 + (id + k) % TO;
+        const float r = v[k] + b[o];
+        if (e < n && (NV >= 32 || (lane & (32 / NV - 1)) == 0)) h[(size_t)e * 512 + o] = r > 0.f ? r : 0.f;
+    }
+}
+
+template <int TE, int TO, int WE, int WO, int STAGES>
+hts_status launch_fc_chain(const float* x, const float* w, const float* b, float* h, int n, int F, cudaStream_t s)
+{
+    constexpr int smem = STAGES * (TE * WE + TO * WO) * 256;
+    auto kernel = fc_chain_kernel<TE, TO, WE, WO, STAGES>;
     static bool set_by_device[kDeviceSlots] = {};
     bool& set = set_by_device[device_slot()];
     if (!set) {
@@ -385,16 +500,15 @@ hts_status launch_fc_tile(const float* x, const float* w, const float* b, float*
         HTS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
         set = true;
     }
-    HTS_CUDA(launch_pdl(kernel, dim3(512 / TO, (unsigned)((n + TE - 1) / TE)), dim3(512), (size_t)smem, s, x, w, b, h, n, F, 512,
-                        ((uintptr_t)w & 15) == 0));
+    HTS_CUDA(launch_pdl(kernel, dim3(512 / (TO * WO), (unsigned)((n + TE * WE - 1) / (TE * WE))), dim3(32 * WE * WO), (size_t)smem, s,
+                        x, w, b, h, n, F, ((uintptr_t)w & 15) == 0));
     note_launch();
     return HTS_OK;
 }
 hts_status launch_fc(const float* x, const float* w, const float* b, float* h, int n, int F, cudaStream_t s)
 {
-    if (n > 384) return launch_fc_tile<4, 8, 1>(x, w, b, h, n, F, s);
-    if (n > 96) return launch_fc_tile<2, 4, 2>(x, w, b, h, n, F, s);
-    return launch_fc_tile<1, 2, 2>(x, w, b, h, n, F, s);
+    if (n > 128) return launch_fc_chain<8, 8, 4, 2, 4>(x, w, b, h, n, F, s);
+    return launch_fc_chain<4, 4, 4, 1, 8>(x, w, b, h, n, F, s);
 }
 
 inline unsigned blocks_for(size_t total, int threads) { return (unsigned)((total + threads - 1) / threads); }
