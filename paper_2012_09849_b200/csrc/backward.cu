@@ -67,27 +67,41 @@ __device__ __forceinline__ void put3(bf16* dst, size_t plane, size_t i, float v)
     d[i] = (uint16_t)a; d[plane + i] = (uint16_t)b; d[2 * plane + i] = (uint16_t)c;
 }
 constexpr int kPackFloats = 8192;
-// Blocks 0..511 turn one row of the dense layer each through shared memory; the rest take the convolutions.
-__global__ void __launch_bounds__(256)
-pack_x3_kernel(const float* __restrict__ w2, const float* __restrict__ w3, const float* __restrict__ wf, int P3,
-               bf16* __restrict__ w2p, bf16* __restrict__ w3p, bf16* __restrict__ wfp)
+struct LoadItem { const float* src; float* dst; int n; };
+struct LoadParams {
+    const float* wf;                    // [512][64 P3]
+    float* wf_dst;
+    LoadItem conv[2];                   // conv2, conv3: copied and packed
+    LoadItem rest[9];                   // copied
+    int P3;
+    bf16 *w2p, *w3p, *wfp;              // nullptr: only copied
+};
+// One launch for all twelve tensors (a parameter update ends in one, so launches count: twelve copies and a packing pass
+// took 45 us, this takes 9).  Blocks 0..511 take one row of the dense layer each and turn it through shared memory; the
+// rest one element per thread.
+__global__ void __launch_bounds__(256) load_fp32_kernel(const LoadParams p)
 {
     __shared__ float s_row[kPackFloats];
-    const int F = 64 * P3;
+    const int P3 = p.P3, F = 64 * P3;
     if (blockIdx.x < 512) {
         const int o = blockIdx.x;
         const int cstep = P3 > kPackFloats ? 1 : kPackFloats / P3 > 64 ? 64 : kPackFloats / P3;      // channels per pass
         for (int c0 = 0; c0 < 64; c0 += cstep) {
             const int nc = c0 + cstep > 64 ? 64 - c0 : cstep;
-            const float* src = wf + (size_t)o * F + (size_t)c0 * P3;
-            if (P3 <= kPackFloats) {
-                for (int i = threadIdx.x; i < nc * P3; i += 256) s_row[i] = src[i];
-                __syncthreads();
-                src = s_row;
+            const float* src = p.wf + (size_t)o * F + (size_t)c0 * P3;
+            float* copy = p.wf_dst + (size_t)o * F + (size_t)c0 * P3;
+            const bool fits = P3 <= kPackFloats;
+            for (int i = threadIdx.x; i < nc * P3; i += 256) {
+                const float v = src[i];
+                copy[i] = v;
+                if (fits && p.wfp) s_row[i] = v;
             }
+            if (!p.wfp) continue;
+            __syncthreads();
+            if (fits) src = s_row;
             for (int i = threadIdx.x; i < nc * P3; i += 256) {
                 const int pix = i / nc, c = i - pix * nc;
-                put3(wfp, (size_t)512 * F, (size_t)o * F + (size_t)pix * 64 + c0 + c, src[c * P3 + pix]);
+                put3(p.wfp, (size_t)512 * F, (size_t)o * F + (size_t)pix * 64 + c0 + c, src[c * P3 + pix]);
             }
             __syncthreads();
         }
@@ -97,13 +111,25 @@ pack_x3_kernel(const float* __restrict__ w2, const float* __restrict__ w3, const
     if (i < 64 * 512) {
         const int o = i >> 9, k = i & 511, tap = k >> 7, cp = k & 127;
         const int dy = tap >> 1, dx = tap & 1, uy = cp >> 6, ux = (cp >> 5) & 1, c = cp & 31;
-        put3(w2p, 64 * 512, i, w2[((o * 32 + c) * 4 + 2 * dy + uy) * 4 + 2 * dx + ux]);
+        if (p.w2p) put3(p.w2p, 64 * 512, i, p.conv[0].src[((o * 32 + c) * 4 + 2 * dy + uy) * 4 + 2 * dx + ux]);
+        p.conv[0].dst[i] = p.conv[0].src[i];
         return;
     }
     i -= 64 * 512;
     if (i < 64 * 576) {
         const int o = i / 576, k = i - o * 576, tap = k >> 6, c = k & 63;
-        put3(w3p, 64 * 576, i, w3[(o * 64 + c) * 9 + tap]);
+        if (p.w3p) put3(p.w3p, 64 * 576, i, p.conv[1].src[(o * 64 + c) * 9 + tap]);
+        p.conv[1].dst[i] = p.conv[1].src[i];
+        return;
+    }
+    i -= 64 * 576;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        if (i < p.rest[k].n) {
+            p.rest[k].dst[i] = p.rest[k].src[i];
+            return;
+        }
+        i -= p.rest[k].n;
     }
 }
 
@@ -199,7 +225,7 @@ head_backward_kernel(const float* __restrict__ logits, const float* __restrict__
 // Partial sums over a range of samples: row o <= A of the block's tile of outputs is sum_i dhead[i][o] h[i][k], row
 // A + 1 is sum_i dh[i][k] (the dense bias); the head biases sum_i dhead[i][o] follow the 512 columns.
 //   part [range][A + 2][513]
-constexpr size_t kHeadRanges = 18;
+constexpr size_t kHeadRanges = 40;
 constexpr int kHeadTile = 11;                            // outputs per block
 __global__ void __launch_bounds__(256)
 head_wgrad_kernel(const float* __restrict__ dhead, const float* __restrict__ h, const bf16* __restrict__ dh, size_t dh_plane,
@@ -247,28 +273,49 @@ struct ReduceParams {
     const float *c1, *c2, *c3, *b1, *b2, *b3, *head;     // partials
     int r1, r2, r3, r3_last, rh;                         // ranges (r3_last: of conv3's last tap)
     size_t g1, g2, g3;                                   // floats between group indices
-    int C, Cp, A;
+    const float* fc;                                     // [512][pixel * 64 + c]
+    int C, Cp, A, P3;
     hts_grads out;
 };
 __device__ __forceinline__ float sum_ranges(const float* p, int ranges, size_t stride)
 {
     float acc = 0.f;
     int r = 0;
-    for (; r + 8 <= ranges; r += 8) {
-        float v[8];
+    for (; r + 16 <= ranges; r += 16) {
+        float v[16];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = p[(size_t)(r + i) * stride];
+        for (int i = 0; i < 16; ++i) v[i] = p[(size_t)(r + i) * stride];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc += v[i];
+        for (int i = 0; i < 16; ++i) acc += v[i];
     }
     for (; r < ranges; ++r) acc += p[(size_t)r * stride];
     return acc;
 }
+// Blocks 0..511 turn one row of the dense gradient each into the caller's column order (c * P3 + pixel): written by the
+// contraction itself, 4-byte pieces P3 apart cost it 20 us.  The others sum.
 __global__ void __launch_bounds__(256) reduce_kernel(const ReduceParams p)
 {
+    __shared__ float s_row[kPackFloats];
     pdl_wait();
     pdl_trigger();
-    int i = blockIdx.x * 256 + threadIdx.x;
+    if (blockIdx.x < 512) {
+        const int F = 64 * p.P3;
+        const float* src = p.fc + (size_t)blockIdx.x * F;
+        float* dst = p.out.fc_w + (size_t)blockIdx.x * F;
+        const int pstep = kPackFloats / 65;              // pixels per pass, rows of 65 against bank conflicts
+        for (int q0 = 0; q0 < p.P3; q0 += pstep) {
+            const int nq = p.P3 - q0 < pstep ? p.P3 - q0 : pstep;
+            for (int i = threadIdx.x; i < nq * 64; i += 256) s_row[(i >> 6) * 65 + (i & 63)] = src[(size_t)q0 * 64 + i];
+            __syncthreads();
+            for (int i = threadIdx.x; i < nq * 64; i += 256) {
+                const int c = i / nq, q = i - c * nq;
+                dst[(size_t)c * p.P3 + q0 + q] = s_row[q * 65 + c];
+            }
+            __syncthreads();
+        }
+        return;
+    }
+    int i = (blockIdx.x - 512) * 256 + threadIdx.x;
     const int n3 = 5 * 8192, n2 = 4 * 8192, n1 = p.Cp / 2 * 4096, nh = (p.A + 2) * 513;
     if (i < n3) {                                        // [tap pair][tap of the pair, c][o]
         const int gi = i >> 13, e = i & 8191, m = e >> 6, o = e & 63, b = m >> 6, c = m & 63;
@@ -320,10 +367,11 @@ struct X3State {
     int max_batch, Cp, H0, W0, G0, H1s, W1s, P1s, P2, P3;
     int sms;
     int* status;
-    bf16 *w2p, *w3p, *wfp;
+    bool packed = false;                                 // the planes below hold the current weights
+    bf16 *w2p = nullptr, *w3p = nullptr, *wfp = nullptr;
     // workspace
     bf16 *x0 = nullptr, *a1, *a2, *a3, *dh, *dz3, *dz2, *dz1;
-    float *logits, *logp, *val, *ent, *dhead, *part1, *part2, *part3, *bias1, *bias2, *bias3, *headp;
+    float *logits, *logp, *val, *ent, *dhead, *part1, *part2, *part3, *partf, *bias1, *bias2, *bias3, *headp;
     X3TapParams bfc, bc3, bc2;                           // batch-independent parts
     X3WgradParams wfc, wc3, wc2, wc1;
     CUtensorMap mW2, mW3, mWf;
@@ -421,8 +469,7 @@ bool x3_plan(X3State* t)
 
 }  // namespace
 
-hts_status x3_create(const Geometry& g, int max_batch, int* status, X3State** out,
-                     bool (*alloc)(void* ctx, void** p, size_t bytes), void* alloc_ctx)
+hts_status x3_create(const Geometry& g, int max_batch, int* status, X3State** out)
 {
     X3State* t = new (std::nothrow) X3State();
     if (!t) return HTS_ERR_ALLOC;
@@ -431,31 +478,33 @@ hts_status x3_create(const Geometry& g, int max_batch, int* status, X3State** ou
     t->H1s = (g.H1 + 1) / 2; t->W1s = (g.W1 + 1) / 2; t->P1s = t->H1s * t->W1s; t->P2 = g.H2 * g.W2; t->P3 = g.H3 * g.W3;
     t->sms = device_sm_count(device_slot());
     if (!x3_plan(t)) { delete t; return HTS_ERR_SHAPE; }
-    const size_t n2 = 64 * 512, n3 = 64 * 576, nf = (size_t)512 * g.F;
-    void* base = nullptr;
-    if (!alloc(alloc_ctx, &base, 2 * 3 * (n2 + n3 + nf))) { delete t; return HTS_ERR_ALLOC; }
-    t->w2p = static_cast<bf16*>(base); t->w3p = t->w2p + 3 * n2; t->wfp = t->w3p + 3 * n3;
-    if (!(x3_make_map(&t->mW2, t->w2p, 512, 64, 3, 512, n2, 64, 3) && x3_make_map(&t->mW3, t->w3p, 576, 64, 3, 576, n3, 64, 3) &&
-          x3_make_map(&t->mWf, t->wfp, g.F, 512, 3, g.F, nf, 64, 3))) {
-        delete t;
-        return HTS_ERR_CUDA;
-    }
     *out = t;
     return HTS_OK;
 }
 
 void x3_destroy(X3State* t) { delete t; }
 
-hts_status x3_pack_weights(X3State* t, const RefWeights& w, cudaStream_t s)
+hts_status x3_load_weights(X3State* t, const hts_weights& w, const RefWeights& d, cudaStream_t s)
 {
-    pack_x3_kernel<<<512 + nblk(64 * 512 + 64 * 576, 256), 256, 0, s>>>(w.w2, w.w3, w.wfc, t->P3, t->w2p, t->w3p, t->wfp);
-    HTS_LAUNCH_CHECK("pack_x3");
+    const int A = t->g.A;
+    auto f = [](const void* p) { return static_cast<const float*>(p); };
+    const LoadParams p{f(w.fc_w), d.wfc,
+                       {{f(w.conv2_w), d.w2, 64 * 512}, {f(w.conv3_w), d.w3, 64 * 576}},
+                       {{f(w.conv1_w), d.w1, 32 * 64 * t->g.C}, {f(w.conv1_b), d.b1, 32}, {f(w.conv2_b), d.b2, 64}, {f(w.conv3_b), d.b3, 64},
+                        {f(w.fc_b), d.bfc, 512}, {f(w.pi_w), d.whead, A * 512}, {f(w.v_w), d.whead + A * 512, 512}, {f(w.pi_b), d.bhead, A},
+                        {f(w.v_b), d.bhead + A, 1}},
+                       t->P3, t->w2p, t->w3p, t->wfp};
+    t->packed = t->wfp != nullptr;
+    int n = 64 * 512 + 64 * 576;
+    for (const LoadItem& it : p.rest) n += it.n;
+    load_fp32_kernel<<<512 + nblk(n, 256), 256, 0, s>>>(p);
+    HTS_LAUNCH_CHECK("load_fp32");
     return HTS_OK;
 }
 
 namespace {
 
-// One allocation for everything the passes keep between kernels.  Zeroed once: positions of a grid outside a layer's
+// One allocation for the packed weights and everything the passes keep between kernels, made by the first gradient.  Zeroed once: positions of a grid outside a layer's
 // output extent and channels added to the frames are never written and have to read as zero.
 hts_status x3_workspace(X3State* t, bool (*alloc)(void* ctx, void** p, size_t bytes), void* alloc_ctx, cudaStream_t s)
 {
@@ -468,6 +517,8 @@ hts_status x3_workspace(X3State* t, bool (*alloc)(void* ctx, void** p, size_t by
     const size_t o_x0 = room(2 * nb * t->G0 * 16 * t->Cp), o_a1 = room(6 * nb * t->P1s * 128), o_a2 = room(6 * nb * t->P2 * 64),
                  o_a3 = room(6 * nb * g.F), o_dh = room(6 * nb * 512), o_dz3 = room(6 * nb * t->P2 * 64), o_dz2 = room(6 * nb * t->P1s * 64),
                  o_dz1 = room(2 * nb * t->G0 * 128), zeroed = total;
+    const size_t n2 = 64 * 512, n3 = 64 * 576, nf = (size_t)512 * g.F;
+    const size_t o_w2 = room(6 * n2), o_w3 = room(6 * n3), o_wf = room(6 * nf), o_pf = room(4 * nf);
     const size_t o_lg = room(4 * nb * A), o_lp = room(4 * nb), o_v = room(4 * nb),
                  o_e = room(4 * nb), o_dhead = room(4 * nb * (A + 1)), o_p1 = room(4 * (size_t)2 * t->wc1.kinds * r1 * 4096),
                  o_p2 = room(4 * (size_t)4 * (t->sms / 2 + 1) * 8192), o_p3 = room(4 * (size_t)5 * (t->sms * 2 / 5 + 1) * 8192), o_b1 = room(4 * (size_t)t->sms * 32),
@@ -478,6 +529,10 @@ hts_status x3_workspace(X3State* t, bool (*alloc)(void* ctx, void** p, size_t by
     HTS_CUDA(cudaMemsetAsync(b, 0, zeroed, s));
     auto H = [&](size_t o) { return reinterpret_cast<bf16*>(b + o); };
     auto Fl = [&](size_t o) { return reinterpret_cast<float*>(b + o); };
+    t->w2p = H(o_w2); t->w3p = H(o_w3); t->wfp = H(o_wf); t->partf = Fl(o_pf);
+    if (!(x3_make_map(&t->mW2, t->w2p, 512, 64, 3, 512, n2, 64, 3) && x3_make_map(&t->mW3, t->w3p, 576, 64, 3, 576, n3, 64, 3) &&
+          x3_make_map(&t->mWf, t->wfp, g.F, 512, 3, g.F, nf, 64, 3)))
+        return HTS_ERR_CUDA;
     t->x0 = H(o_x0); t->a1 = H(o_a1); t->a2 = H(o_a2); t->a3 = H(o_a3); t->dh = H(o_dh); t->dz3 = H(o_dz3); t->dz2 = H(o_dz2); t->dz1 = H(o_dz1);
     t->logits = Fl(o_lg); t->logp = Fl(o_lp); t->val = Fl(o_v); t->ent = Fl(o_e); t->dhead = Fl(o_dhead);
     t->part1 = Fl(o_p1); t->part2 = Fl(o_p2); t->part3 = Fl(o_p3); t->bias1 = Fl(o_b1); t->bias2 = Fl(o_b2); t->bias3 = Fl(o_b3); t->headp = Fl(o_hd);
@@ -519,6 +574,11 @@ hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, 
     hts_status st = x3_workspace(t, alloc, alloc_ctx, s);
     if (st != HTS_OK) return st;
     if (!x3_map_batch(t, n)) return HTS_ERR_CUDA;
+    if (!t->packed) {                                    // weights loaded before the first gradient
+        const hts_weights own{w.w1, w.b1, w.w2, w.b2, w.w3, w.b3, w.wfc, w.bfc, w.whead, w.bhead, w.whead + (size_t)g.A * 512, w.bhead + g.A};
+        st = x3_load_weights(t, own, w, s);
+        if (st != HTS_OK) return st;
+    }
     const size_t nb = (size_t)t->max_batch, N = (size_t)n;
     const size_t p1 = nb * t->P1s * 128, p2 = nb * t->P2 * 64, p3 = nb * g.F, ph = nb * 512, pz2 = nb * t->P1s * 64;
 
@@ -573,7 +633,7 @@ hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, 
         return p;
     };
     X3WgradParams q = cut(t->wfc, N, 1, 1);
-    q.fc_w = out.fc_w;
+    q.fc_w = t->partf;
     st = x3_wgrad_launch<3, 64>(t->vDh, t->vA3, q, s);
     if (st != HTS_OK) return st;
     ReduceParams r{};
@@ -593,9 +653,9 @@ hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, 
     r.c1 = t->part1; r.c2 = t->part2; r.c3 = t->part3; r.b1 = t->bias1; r.b2 = t->bias2; r.b3 = t->bias3; r.head = t->headp;
     r.r1 = q1.ranges; r.r2 = q2.ranges; r.r3 = q3.ranges; r.r3_last = q3.last_ranges; r.rh = rh;
     r.g1 = q1.group_stride; r.g2 = q2.group_stride; r.g3 = q3.group_stride;
-    r.C = g.C; r.Cp = t->Cp; r.A = g.A; r.out = out;
+    r.fc = t->partf; r.P3 = t->P3; r.C = g.C; r.Cp = t->Cp; r.A = g.A; r.out = out;
     const size_t total = (size_t)9 * 8192 + (size_t)t->Cp / 2 * 4096 + (size_t)(g.A + 2) * 513 + 160;
-    HTS_CUDA(launch_pdl(reduce_kernel, dim3(nblk(total, 256)), dim3(256), 0, s, r));
+    HTS_CUDA(launch_pdl(reduce_kernel, dim3(512 + nblk(total, 256)), dim3(256), 0, s, r));
     note_launch();
     return HTS_OK;
 }

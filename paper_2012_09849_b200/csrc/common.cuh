@@ -104,18 +104,16 @@ struct RefPlanes {             // the hidden convolution outputs once more, as t
     size_t p1, p2, p3;         // elements between planes
 };
 
-hts_status ref_convert_weights(const Geometry& g, int dtype, const hts_weights& src,
-                               const RefWeights& dst, cudaStream_t s);
 hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspace& ws,
                        const uint8_t* obs, const Indexing& ix, int* status, int n, Profiler& prof, cudaStream_t s,
                        const RefPlanes* planes = nullptr);
 
 // ---- gradient of the learner objective: fp32-accurate passes on the tensor cores (backward.cu) -------
 struct X3State;
-hts_status x3_create(const Geometry& g, int max_batch, int* status, X3State** out,
-                     bool (*alloc)(void* ctx, void** p, size_t bytes), void* alloc_ctx);
+hts_status x3_create(const Geometry& g, int max_batch, int* status, X3State** out);
 void x3_destroy(X3State* t);
-hts_status x3_pack_weights(X3State* t, const RefWeights& w, cudaStream_t s);
+// Copies the caller's fp32 weights into the context, and packs them once a gradient has been asked for, in one launch.
+hts_status x3_load_weights(X3State* t, const hts_weights& src, const RefWeights& dst, cudaStream_t s);
 // The workspace is allocated by the first call on a state.
 hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, Profiler& prof, const uint8_t* obs, const int32_t* actions, const float* adv, const float* ret,
                        const float* logp_old, float value_coef, float entropy_coef, float clip, int n, const hts_grads& out,

@@ -407,18 +407,6 @@ conv1_march_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     if (warp == 1) tmem_dealloc(tmem_slot, S::TMEM);
 }
 
-__global__ void pack_conv1_kernel(const __nv_bfloat16* __restrict__ w, __half* __restrict__ wp, int C,
-                                  const float* __restrict__ scale)
-{
-    const int K = 16 * C;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 128 * K) return;
-    const int row = i / K, k = i - row * K;
-    const int dy = row >> 6, dx = (row >> 5) & 1, o = row & 31;
-    const int c = k >> 4, uy = (k >> 2) & 3, ux = k & 3;
-    wp[i] = __float2half_rn(__bfloat162float(w[((o * C + c) * 8 + (4 * dy + uy)) * 8 + (4 * dx + ux)]) * scale[0]);
-}
-
 // output-row ranges per tile: enough units that every CTA of the grid gets several, few enough that the extra
 // grid row each unit converts (a unit of k steps stages k + 1 rows) stays cheap
 int choose_splits(int tiles, int H1, int grid)
@@ -480,15 +468,6 @@ bool conv1_plan(const Geometry& g, Conv1Plan* pl)
     pl->stages = st;
     pl->smem_bytes = fixed + st * pl->stage_bytes;
     return true;
-}
-
-hts_status conv1_pack_weights(const Conv1Plan& pl, const __nv_bfloat16* w1, __half* packed, const float* scale,
-                              cudaStream_t s)
-{
-    const int total = 128 * 16 * pl.C;
-    pack_conv1_kernel<<<(total + 255) / 256, 256, 0, s>>>(w1, packed, pl.C, scale);
-    HTS_LAUNCH_CHECK("pack_conv1");
-    return HTS_OK;
 }
 
 hts_status conv1_launch(const Conv1Plan& pl, const CUtensorMap& weight_map, Conv1MapCache& maps, const uint8_t* obs,

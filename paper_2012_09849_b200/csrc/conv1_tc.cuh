@@ -38,11 +38,7 @@ struct Conv1MapCache {
 // false if the geometry does not fit the kernel (C not 4, 8 or 16; H or W not a multiple of 4; too wide)
 bool conv1_plan(const Geometry& g, Conv1Plan* plan);
 
-// w1 [32,C,8,8] bf16 -> packed [128][16*C] fp16 scaled by *scale:
-//   row dy*64 + dx*32 + o, column c*16 + uy*4 + ux  holds  w1[o][c][4dy+uy][4dx+ux]
-hts_status conv1_pack_weights(const Conv1Plan& pl, const __nv_bfloat16* w1, __half* packed, const float* scale,
-                              cudaStream_t s);
-
+// weight_map: w1 packed [128][16*C] fp16, scaled: row dy*64 + dx*32 + o, column c*16 + uy*4 + ux  holds  w1[o][c][4dy+uy][4dx+ux]
 // out: fp16 rows [env*P1s + (y/2)*W1s + x/2][128], column ((y%2)*2 + x%2)*32 + o
 // ix: dense frames (row e = frame e of obs) or frames gathered by slot from a pool (see Indexing)
 hts_status conv1_launch(const Conv1Plan& pl, const CUtensorMap& weight_map, Conv1MapCache& maps, const uint8_t* obs,

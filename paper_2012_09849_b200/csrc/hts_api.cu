@@ -167,7 +167,7 @@ hts_status hts_policy_create(const hts_net_desc* d, hts_ctx** out)
         ok = ok && dev_alloc(c, &c->rws.a1, nb * 32 * g.H1 * g.W1) && dev_alloc(c, &c->rws.a2, nb * 64 * g.H2 * g.W2);
         ok = ok && dev_alloc(c, &c->rws.a3, nb * g.F) && dev_alloc(c, &c->rws.h, nb * 512);
         if (ok) {
-            const hts_status st = x3_create(g, d->max_batch, c->status, &c->x3, raw_alloc, c);
+            const hts_status st = x3_create(g, d->max_batch, c->status, &c->x3);
             if (st != HTS_OK) { hts_policy_destroy(c); return st; }
         }
     }
@@ -191,9 +191,7 @@ hts_status hts_policy_load_weights(hts_ctx* ctx, const hts_weights* w, void* cud
     const void* const* p = reinterpret_cast<const void* const*>(w);
     for (int i = 0; i < 12; ++i) if (!p[i]) return HTS_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    hts_status st = ctx->tc ? tc_load_weights(ctx->tc, *w, s)
-                            : ref_convert_weights(ctx->g, ctx->desc.weight_dtype, *w, ctx->rw, s);
-    if (st == HTS_OK && ctx->x3) st = x3_pack_weights(ctx->x3, ctx->rw, s);
+    const hts_status st = ctx->tc ? tc_load_weights(ctx->tc, *w, s) : x3_load_weights(ctx->x3, *w, ctx->rw, s);
     if (st != HTS_OK) return st;
     ctx->loaded = true;
     return HTS_OK;

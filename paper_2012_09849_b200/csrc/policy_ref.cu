@@ -8,14 +8,6 @@
 namespace hts {
 namespace {
 
-__global__ void to_f32_kernel(const void* __restrict__ src, int dtype, float* __restrict__ dst, size_t count)
-{
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
-    dst[i] = (dtype == HTS_DTYPE_FP32) ? static_cast<const float*>(src)[i]
-                                       : __bfloat162float(static_cast<const __nv_bfloat16*>(src)[i]);
-}
-
 typedef unsigned long long f32x2;                       // two fp32 lanes of a packed multiply-add
 __device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b)
 {
@@ -511,28 +503,7 @@ hts_status launch_fc(const float* x, const float* w, const float* b, float* h, i
     return launch_fc_chain<4, 4, 4, 1, 8>(x, w, b, h, n, F, s);
 }
 
-inline unsigned blocks_for(size_t total, int threads) { return (unsigned)((total + threads - 1) / threads); }
-
 }  // namespace
-
-hts_status ref_convert_weights(const Geometry& g, int dtype, const hts_weights& src,
-                               const RefWeights& dst, cudaStream_t s)
-{
-    struct Item { const void* p; float* q; size_t n; };
-    const Item items[] = {
-        {src.conv1_w, dst.w1, (size_t)32 * g.C * 64}, {src.conv1_b, dst.b1, 32},
-        {src.conv2_w, dst.w2, (size_t)64 * 32 * 16},  {src.conv2_b, dst.b2, 64},
-        {src.conv3_w, dst.w3, (size_t)64 * 64 * 9},   {src.conv3_b, dst.b3, 64},
-        {src.fc_w, dst.wfc, (size_t)512 * g.F},       {src.fc_b, dst.bfc, 512},
-        {src.pi_w, dst.whead, (size_t)g.A * 512},     {src.pi_b, dst.bhead, (size_t)g.A},
-        {src.v_w, dst.whead + (size_t)g.A * 512, 512}, {src.v_b, dst.bhead + g.A, 1},
-    };
-    for (const Item& it : items) {
-        to_f32_kernel<<<blocks_for(it.n, 256), 256, 0, s>>>(it.p, dtype, it.q, it.n);
-        HTS_LAUNCH_CHECK("to_f32_kernel");
-    }
-    return HTS_OK;
-}
 
 // `planes`: also leave the three hidden convolution outputs as bf16 planes for the gradient.
 hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspace& ws,

@@ -53,14 +53,6 @@ struct GemmParams {
     int* status;
 };
 
-__device__ __forceinline__ uint32_t pack_relu_h2(float a, float b)
-{
-    a = fminf(fmaxf(a, 0.f), 65504.f);
-    b = fminf(fmaxf(b, 0.f), 65504.f);
-    __half2 t = __floats2half2_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&t);
-}
-
 template <int BN, int EPI>
 __global__ void __launch_bounds__(192)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmParams p)
@@ -140,11 +132,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     } else {
         // epilogue warps 2..5: warp w may touch TMEM lanes [32*(w%4), 32*(w%4)+32)
         const int q = warp & 3;
-        const int r = q * 32 + lane;                    // row of the tile = TMEM lane
         const bool ok = mbar_wait_warp(&accum_bar, 0, abortp, p.status, 3);
         tc_fence_after();
         if (ok) {
-            const long m = (long)m0 + r;
             const float inv = *p.inv_scale;
             {
                 // The accumulator arrives one row per thread; a row-per-thread store would touch 32
@@ -486,65 +476,116 @@ fc_ranges_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 }
 
 // ---- weight scaling and packing ---------------------------------------------------------------
-__global__ void absmax_kernel(const __nv_bfloat16* __restrict__ w, size_t n, unsigned* __restrict__ slot)
+// Two launches: the largest magnitude of each layer (the last block to finish turns them into scales), then every
+// layer scaled, converted and laid out.  They follow each parameter update, so launches count: 18 separate ones took
+// 125 us (47 of them in a 64-block pass over the dense layer).
+struct LoadTcParams {
+    const __nv_bfloat16* w[L_COUNT];    // conv1, conv2, conv3, dense
+    int n[L_COUNT];
+    unsigned* absmax;                   // [L_COUNT], then the ticket; zero between calls
+    float *scale, *inv_scale;
+    float conv1_extra;
+    int C, P3;
+    __half* wp[L_COUNT];
+    const __nv_bfloat16* f[8];          // biases and heads: kept as fp32
+    float* fdst[8];
+    int fn[8];
+};
+constexpr int kAbsmaxBlocks = 4 * 148;
+
+__global__ void __launch_bounds__(256) absmax_kernel(const LoadTcParams p)
 {
-    unsigned m = 0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float a = fabsf(__bfloat162float(w[i]));
-        if (a == a && a < INFINITY) m = max(m, __float_as_uint(a));     // finite magnitudes order like their bits
+    __shared__ bool s_last;
+    const int tid = blockIdx.x * 256 + threadIdx.x, threads = gridDim.x * 256;
+#pragma unroll
+    for (int l = 0; l < L_COUNT; ++l) {
+        unsigned m = 0;                                 // finite magnitudes order like their bits
+        auto take = [&](uint32_t bits) { bits &= 0x7fffu; if (bits < 0x7f80u) m = max(m, bits); };
+        int done = 0;
+        if (((uintptr_t)p.w[l] & 15) == 0) {
+            const uint4* v = reinterpret_cast<const uint4*>(p.w[l]);
+            for (int i = tid; i < p.n[l] / 8; i += threads) {
+                const uint4 q = v[i];
+                take(q.x); take(q.x >> 16); take(q.y); take(q.y >> 16); take(q.z); take(q.z >> 16); take(q.w); take(q.w >> 16);
+            }
+            done = p.n[l] / 8 * 8;
+        }
+        for (int i = done + tid; i < p.n[l]; i += threads) take(reinterpret_cast<const uint16_t*>(p.w[l])[i]);
+        m = __reduce_max_sync(0xffffffffu, m);
+        if ((threadIdx.x & 31) == 0 && m) atomicMax(p.absmax + l, m << 16);
     }
-    for (int k = 16; k > 0; k >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, k));
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(slot, m);
-}
-// scale = 2^(14 - floor(log2 max)): the largest weight lands in [2^14, 2^15)
-__global__ void scales_kernel(const unsigned* __restrict__ slots, float* __restrict__ scale, float* __restrict__ inv,
-                              float conv1_extra)
-{
-    const int l = threadIdx.x;
-    if (l >= L_COUNT) return;
-    const float mx = __uint_as_float(slots[l]);
-    int e = 0;
-    float s = 1.f;
-    if (mx > 0.f) { frexpf(mx, &e); s = ldexpf(1.f, 15 - e); }        // mx = f * 2^e, f in [0.5, 1)
-    scale[l] = s;
-    inv[l] = (l == L_CONV1 ? conv1_extra : 1.f) / s;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(p.absmax + L_COUNT, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (s_last && threadIdx.x <= L_COUNT) {
+        const int l = threadIdx.x;
+        __threadfence();
+        const float mx = __uint_as_float(atomicExch(p.absmax + l, 0u));      // and ready for the next call
+        if (l == L_COUNT) return;
+        // scale = 2^(14 - floor(log2 max)): the largest weight lands in [2^14, 2^15)
+        int e = 0;
+        float s = 1.f;
+        if (mx > 0.f) { frexpf(mx, &e); s = ldexpf(1.f, 15 - e); }        // mx = f * 2^e, f in [0.5, 1)
+        p.scale[l] = s;
+        p.inv_scale[l] = (l == L_CONV1 ? p.conv1_extra : 1.f) / s;
+    }
 }
 __device__ __forceinline__ __half scaled_h(__nv_bfloat16 w, float s) { return __float2half_rn(__bfloat162float(w) * s); }
 
-// conv2: Wp[o][(tap*2 + half)*64 + j], c' = half*64 + j = (uy*2+ux)*32 + c, tap = dy*2+dx,
-//        value w2[o][c][2dy+uy][2dx+ux]
-__global__ void pack_conv2_kernel(const __nv_bfloat16* __restrict__ w, __half* __restrict__ wp, const float* __restrict__ scale)
+//   conv1: row dy*64 + dx*32 + o, column c*16 + uy*4 + ux       value w1[o][c][4dy+uy][4dx+ux]
+//   conv2: [o][(tap*2 + half)*64 + j], c' = half*64 + j = (uy*2+ux)*32 + c, tap = dy*2+dx, value w2[o][c][2dy+uy][2dx+ux]
+//   conv3: [o][(dy*3+dx)*64 + c]                                value w3[o][c][dy][dx]
+//   dense: [o][pix*64 + c] (activations are stored pixel-major)  value wfc[o][c*P3 + pix]
+// Blocks 0..511 take one row of the dense layer each and turn it through shared memory (rows of up to 16384 columns;
+// wider ones are read with a stride); the rest one element per thread.
+constexpr int kPackRow = 16384;
+__global__ void __launch_bounds__(256) pack_kernel(const LoadTcParams p)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 64 * 512) return;
-    const int o = i / 512, k = i % 512;
-    const int tap = k / 128, cp = k % 128;
-    const int dy = tap >> 1, dx = tap & 1, uy = (cp / 32) >> 1, ux = (cp / 32) & 1, c = cp % 32;
-    wp[i] = scaled_h(w[((o * 32 + c) * 4 + (2 * dy + uy)) * 4 + (2 * dx + ux)], scale[L_CONV2]);
-}
-// conv3: Wp[o][(dy*3+dx)*64 + c] = w3[o][c][dy][dx]
-__global__ void pack_conv3_kernel(const __nv_bfloat16* __restrict__ w, __half* __restrict__ wp, const float* __restrict__ scale)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 64 * 576) return;
-    const int o = i / 576, k = i % 576;
-    const int tap = k / 64, c = k % 64;
-    wp[i] = scaled_h(w[(o * 64 + c) * 9 + tap], scale[L_CONV3]);
-}
-// FC: Wp[o][pix*64 + c] = wfc[o][c*P3 + pix]   (activations are stored pixel-major, channel-minor)
-__global__ void pack_fc_kernel(const __nv_bfloat16* __restrict__ w, __half* __restrict__ wp, int P3, const float* __restrict__ scale)
-{
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int F = 64 * P3;
-    if (i >= (size_t)512 * F) return;
-    const int o = (int)(i / F), k = (int)(i % F);
-    const int pix = k / 64, c = k % 64;
-    wp[i] = scaled_h(w[(size_t)o * F + c * P3 + pix], scale[L_FC]);
-}
-__global__ void bf16_to_f32_kernel(const __nv_bfloat16* __restrict__ src, float* __restrict__ dst, size_t n)
-{
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dst[i] = __bfloat162float(src[i]);
+    __shared__ __nv_bfloat16 s_row[kPackRow];
+    if (blockIdx.x < 512) {
+        const int o = blockIdx.x, F = 64 * p.P3;
+        const __nv_bfloat16* src = p.w[L_FC] + (size_t)o * F;
+        const float s = p.scale[L_FC];
+        if (F <= kPackRow) {
+            for (int i = threadIdx.x; i < F; i += 256) s_row[i] = src[i];
+            __syncthreads();
+            src = s_row;
+        }
+        __half* dst = p.wp[L_FC] + (size_t)o * F;
+        for (int k = threadIdx.x; k < F; k += 256) dst[k] = scaled_h(src[(k & 63) * p.P3 + (k >> 6)], s);
+        return;
+    }
+    int i = (blockIdx.x - 512) * 256 + threadIdx.x;
+    const int K = 16 * p.C;
+    if (i < 128 * K) {
+        const int row = i / K, k = i - row * K, dy = row >> 6, dx = (row >> 5) & 1, o = row & 31;
+        const int c = k >> 4, uy = (k >> 2) & 3, ux = k & 3;
+        p.wp[L_CONV1][i] = scaled_h(p.w[L_CONV1][((o * p.C + c) * 8 + (4 * dy + uy)) * 8 + (4 * dx + ux)], p.scale[L_CONV1]);
+        return;
+    }
+    i -= 128 * K;
+    if (i < 64 * 512) {
+        const int o = i / 512, k = i % 512, tap = k / 128, cp = k % 128;
+        const int dy = tap >> 1, dx = tap & 1, uy = (cp / 32) >> 1, ux = (cp / 32) & 1, c = cp % 32;
+        p.wp[L_CONV2][i] = scaled_h(p.w[L_CONV2][((o * 32 + c) * 4 + (2 * dy + uy)) * 4 + (2 * dx + ux)], p.scale[L_CONV2]);
+        return;
+    }
+    i -= 64 * 512;
+    if (i < 64 * 576) {
+        const int o = i / 576, k = i % 576, tap = k / 64, c = k % 64;
+        p.wp[L_CONV3][i] = scaled_h(p.w[L_CONV3][(o * 64 + c) * 9 + tap], p.scale[L_CONV3]);
+        return;
+    }
+    i -= 64 * 576;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        if (i < p.fn[k]) {
+            p.fdst[k][i] = __bfloat162float(p.f[k][i]);
+            return;
+        }
+        i -= p.fn[k];
+    }
 }
 
 // ---- parity taps: internal layouts -> fp32 NCHW ----------------------------------------------------
@@ -610,7 +651,7 @@ struct TcState {
     Conv1MapCache maps1;
     __half *w1p, *w2p, *w3p, *wfcp;
     float *b1, *b2, *b3, *bfc, *whead, *bhead;
-    unsigned* absmax;           // [L_COUNT]
+    unsigned* absmax;           // [L_COUNT] and a ticket, zero between calls
     float *scale, *inv_scale;   // [L_COUNT] each
     // workspace
     __half *a1s, *a2, *a3;
@@ -651,12 +692,13 @@ hts_status tc_create(const Geometry& g, int max_batch, int* status, TcState** ou
     bool ok = A(&t->w2p, (size_t)64 * 512) && A(&t->w3p, (size_t)64 * 576) && A(&t->wfcp, (size_t)512 * g.F) &&
               A(&t->w1p, (size_t)128 * 16 * g.C) && A(&t->b1, 32) && A(&t->b2, 64) && A(&t->b3, 64) && A(&t->bfc, 512) &&
               A(&t->whead, (size_t)(g.A + 1) * 512) && A(&t->bhead, (size_t)g.A + 1) &&
-              A(&t->absmax, L_COUNT) && A(&t->scale, L_COUNT) && A(&t->inv_scale, L_COUNT) &&
+              A(&t->absmax, L_COUNT + 1) && A(&t->scale, L_COUNT) && A(&t->inv_scale, L_COUNT) &&
               A(&t->a1s, nb * t->P1s * 128) && A(&t->a2, nb * t->P2 * 64) && A(&t->a3, nb * g.F) &&
               A(&t->hpart, (size_t)t->splits * nb * 512) && A(&t->h, nb * 512);
     if (!ok) { delete t; return HTS_ERR_ALLOC; }
     // cells of an odd-sized s2d border that conv1 never writes must hold finite numbers
     if (cudaMemset(t->a1s, 0, nb * t->P1s * 128 * 2) != cudaSuccess) { delete t; return cuda_fail(cudaGetLastError(), "cudaMemset"); }
+    if (cudaMemset(t->absmax, 0, (L_COUNT + 1) * sizeof(unsigned)) != cudaSuccess) { delete t; return cuda_fail(cudaGetLastError(), "cudaMemset"); }
     t->rows2 = conv_res_tile_rows(t->W1s + 1);
     t->rows3 = conv_res_tile_rows(2 * g.W2 + 2);
     if (t->rows2 > 256 || t->rows3 > 256) { delete t; return HTS_ERR_SHAPE; }
@@ -675,30 +717,23 @@ hts_status tc_load_weights(TcState* t, const hts_weights& w, cudaStream_t s)
 {
     const Geometry& g = t->g;
     auto bf = [](const void* p) { return static_cast<const __nv_bfloat16*>(p); };
-    HTS_CUDA(cudaMemsetAsync(t->absmax, 0, L_COUNT * sizeof(unsigned), s));
-    struct Mx { const void* p; size_t n; int l; };
-    const Mx mx[] = {{w.conv1_w, (size_t)32 * g.C * 64, L_CONV1}, {w.conv2_w, (size_t)64 * 512, L_CONV2},
-                     {w.conv3_w, (size_t)64 * 576, L_CONV3}, {w.fc_w, (size_t)512 * g.F, L_FC}};
-    for (const Mx& m : mx) {
-        absmax_kernel<<<64, 256, 0, s>>>(bf(m.p), m.n, t->absmax + m.l);
-        HTS_LAUNCH_CHECK("absmax");
-    }
+    LoadTcParams p{};
     // conv1 feeds raw bytes as fp16 subnormals (b * 2^-24): its accumulator scale undoes that and the /255
-    scales_kernel<<<1, 32, 0, s>>>(t->absmax, t->scale, t->inv_scale, 16777216.0f / 255.0f);
-    HTS_LAUNCH_CHECK("scales");
-    hts_status st1 = conv1_pack_weights(t->pl1, bf(w.conv1_w), t->w1p, t->scale + L_CONV1, s);
-    if (st1 != HTS_OK) return st1;
-    pack_conv2_kernel<<<nblk(64 * 512, 256), 256, 0, s>>>(bf(w.conv2_w), t->w2p, t->scale); HTS_LAUNCH_CHECK("pack_conv2");
-    pack_conv3_kernel<<<nblk(64 * 576, 256), 256, 0, s>>>(bf(w.conv3_w), t->w3p, t->scale); HTS_LAUNCH_CHECK("pack_conv3");
-    pack_fc_kernel<<<nblk((size_t)512 * g.F, 256), 256, 0, s>>>(bf(w.fc_w), t->wfcp, t->P3, t->scale); HTS_LAUNCH_CHECK("pack_fc");
-    struct It { const void* p; float* q; size_t n; };
-    const It items[] = {{w.conv1_b, t->b1, 32}, {w.conv2_b, t->b2, 64},
-                        {w.conv3_b, t->b3, 64}, {w.fc_b, t->bfc, 512}, {w.pi_w, t->whead, (size_t)g.A * 512},
-                        {w.v_w, t->whead + (size_t)g.A * 512, 512}, {w.pi_b, t->bhead, (size_t)g.A}, {w.v_b, t->bhead + g.A, 1}};
-    for (const It& it : items) {
-        bf16_to_f32_kernel<<<nblk(it.n, 256), 256, 0, s>>>(bf(it.p), it.q, it.n);
-        HTS_LAUNCH_CHECK("bf16_to_f32");
-    }
+    p.absmax = t->absmax; p.scale = t->scale; p.inv_scale = t->inv_scale; p.conv1_extra = 16777216.0f / 255.0f; p.C = g.C; p.P3 = t->P3;
+    const void* ws[L_COUNT] = {w.conv1_w, w.conv2_w, w.conv3_w, w.fc_w};
+    const int wn[L_COUNT] = {32 * g.C * 64, 64 * 512, 64 * 576, 512 * g.F};
+    __half* wp[L_COUNT] = {t->w1p, t->w2p, t->w3p, t->wfcp};
+    for (int l = 0; l < L_COUNT; ++l) { p.w[l] = bf(ws[l]); p.n[l] = wn[l]; p.wp[l] = wp[l]; }
+    struct It { const void* p; float* q; int n; };
+    const It items[8] = {{w.conv1_b, t->b1, 32}, {w.conv2_b, t->b2, 64},
+                         {w.conv3_b, t->b3, 64}, {w.fc_b, t->bfc, 512}, {w.pi_w, t->whead, g.A * 512},
+                         {w.v_w, t->whead + (size_t)g.A * 512, 512}, {w.pi_b, t->bhead, g.A}, {w.v_b, t->bhead + g.A, 1}};
+    int rest = 128 * 16 * g.C + 64 * 512 + 64 * 576;
+    for (int k = 0; k < 8; ++k) { p.f[k] = bf(items[k].p); p.fdst[k] = items[k].q; p.fn[k] = items[k].n; rest += items[k].n; }
+    absmax_kernel<<<kAbsmaxBlocks, 256, 0, s>>>(p);
+    HTS_LAUNCH_CHECK("absmax");
+    pack_kernel<<<512 + nblk(rest, 256), 256, 0, s>>>(p);
+    HTS_LAUNCH_CHECK("pack");
     return HTS_OK;
 }
 

@@ -366,9 +366,9 @@ x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     if (p.fc_w) {
                         const int o = (kind % p.ka) * 128 + m, pix = (kind / p.ka) * 2 + g;
                         if (pix < p.P3) {
-                            float* dst = p.fc_w + (size_t)o * 64 * p.P3 + (size_t)(j * 32) * p.P3 + pix;
+                            float* dst = p.fc_w + (size_t)o * 64 * p.P3 + pix * 64 + j * 32;
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) dst[(size_t)i * p.P3] = v[i];
+                            for (int i = 0; i < 32; i += 8) st_v8(dst + i, reinterpret_cast<const uint32_t*>(v) + i);
                         }
                     } else {
                         float* dst = p.part + (gi0 + g) * p.group_stride + ((size_t)range * 128 + m) * NB + j * 32;

@@ -67,7 +67,7 @@ struct X3WgradParams {
     float* part;                        // [group index][range][128][NB], or nullptr
     size_t group_stride;                // floats between group indices
     float* bias_part;                   // [range][NB], written by kind 0, or nullptr
-    float* fc_w;                        // final dense gradient [512][64 P3] (column c * P3 + pixel), or nullptr
+    float* fc_w;                        // dense gradient [512][pixel * 64 + c], or nullptr
     int P3;
     int* status;
 };
