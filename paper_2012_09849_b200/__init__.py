@@ -1,7 +1,8 @@
 """Python binding of the HTS-RL hot-path library (libhts.so, CUDA for sm_100a).
 
 Argument marshalling only: every function here has the name and the meaning of the C
-entry point it forwards to (see include/hts.h).  Tensors are ``torch`` CUDA tensors (torch is
+entry point it forwards to (see include/hts.h).  The calls a training loop makes go through a CPython
+extension (csrc/binding.c), the others through ctypes.  Tensors are ``torch`` CUDA tensors (torch is
 used for device memory and streams, nothing else); the ``*_host`` calls take CPU tensors or
 numpy arrays.  There is no fallback: if the library is missing or a call fails, an exception
 is raised.
@@ -9,6 +10,7 @@ is raised.
 from __future__ import annotations
 
 import ctypes as C
+import importlib
 import os
 
 import numpy as np
@@ -116,6 +118,21 @@ def lib():
     return _lib
 
 
+class _NativeAtFirstUse:
+    """Stands for the extension until it is first called: the package imports before it is built."""
+
+    def __getattr__(self, name):
+        global _native
+        lib()                                            # says how to build it if it is missing
+        module = importlib.import_module("._native", __name__)
+        module.init(HtsError)
+        _native = module
+        return getattr(module, name)
+
+
+_native = _NativeAtFirstUse()
+
+
 def _ptr(x):
     """Address of a torch tensor / numpy array / raw int / None."""
     if x is None:
@@ -151,58 +168,45 @@ def hts_policy_create(C_: int, H: int, W: int, num_actions: int, weight_dtype: i
 
 def hts_policy_load_weights(ctx: int, weights: dict, stream=None) -> None:
     """weights: name -> CUDA tensor (float32, or bfloat16 for a bf16 context), PyTorch layouts."""
-    w = hts_weights(**{n: _ptr(weights[n]) for n in WEIGHT_NAMES})
-    _check(lib().hts_policy_load_weights(ctx, C.byref(w), _stream(stream)), "hts_policy_load_weights")
+    _native.policy_load_weights(ctx, weights, stream)
 
 
 def hts_policy_step(ctx, obs, env_ids, t_per_env, t, seed, n, actions, logp, values, entropy,
                     logits=None, stream=None) -> None:
-    _check(lib().hts_policy_step(ctx, _ptr(obs), _ptr(env_ids), _ptr(t_per_env), int(t), int(seed), int(n),
-                                 _ptr(actions), _ptr(logp), _ptr(values), _ptr(entropy), _ptr(logits),
-                                 _stream(stream)), "hts_policy_step")
+    _native.policy_step(ctx, obs, env_ids, t_per_env, t, seed, n, actions, logp, values, entropy, logits, stream)
 
 
 def hts_policy_step_indexed(ctx, state_buffer, pool, slots, env_ids, t_per_env, t, seed, n, actions_row, logp_row,
                             values_row, entropy_row, stream=None) -> None:
-    _check(lib().hts_policy_step_indexed(ctx, _ptr(state_buffer), int(pool), _ptr(slots), _ptr(env_ids), _ptr(t_per_env),
-                                         int(t), int(seed), int(n), _ptr(actions_row), _ptr(logp_row), _ptr(values_row),
-                                         _ptr(entropy_row), _stream(stream)), "hts_policy_step_indexed")
+    _native.policy_step_indexed(ctx, state_buffer, pool, slots, env_ids, t_per_env, t, seed, n, actions_row, logp_row, values_row,
+                                entropy_row, stream)
 
 
 def hts_policy_evaluate(ctx, obs, actions, n, logp, values, entropy, logits=None, stream=None) -> None:
-    _check(lib().hts_policy_evaluate(ctx, _ptr(obs), _ptr(actions), int(n), _ptr(logp), _ptr(values), _ptr(entropy),
-                                     _ptr(logits), _stream(stream)), "hts_policy_evaluate")
+    _native.policy_evaluate(ctx, obs, actions, n, logp, values, entropy, logits, stream)
 
 
 def hts_policy_gradient(ctx, obs, actions, advantages, returns, logp_old, value_coef, entropy_coef, clip, n, grads: dict,
                         stream=None) -> None:
     """grads: name -> CUDA float32 tensor shaped like the parameter (overwritten)."""
-    g = hts_grads(**{k: _ptr(grads[k]) for k in WEIGHT_NAMES})
-    _check(lib().hts_policy_gradient(ctx, _ptr(obs), _ptr(actions), _ptr(advantages), _ptr(returns), _ptr(logp_old),
-                                     float(value_coef), float(entropy_coef), float(clip), int(n), C.byref(g),
-                                     _stream(stream)), "hts_policy_gradient")
+    _native.policy_gradient(ctx, obs, actions, advantages, returns, logp_old, value_coef, entropy_coef, clip, n, grads, stream)
 
 
 def hts_a2c_terms(logp, values, entropy, returns, count, out3, stream=None) -> None:
-    _check(lib().hts_a2c_terms(_ptr(logp), _ptr(values), _ptr(entropy), _ptr(returns), int(count), _ptr(out3),
-                               _stream(stream)), "hts_a2c_terms")
+    _native.a2c_terms(logp, values, entropy, returns, count, out3, stream)
 
 
 def hts_ppo_terms(logp_new, logp_old, values, entropy, advantages, returns, count, clip, normalize, out4, stream=None) -> None:
-    _check(lib().hts_ppo_terms(_ptr(logp_new), _ptr(logp_old), _ptr(values), _ptr(entropy), _ptr(advantages), _ptr(returns),
-                               int(count), float(clip), int(bool(normalize)), _ptr(out4), _stream(stream)), "hts_ppo_terms")
+    _native.ppo_terms(logp_new, logp_old, values, entropy, advantages, returns, count, clip, normalize, out4, stream)
 
 
 def hts_delayed_update(theta, grad, sq_avg, count, lr, alpha, eps, theta_bf16=None, stream=None) -> None:
-    _check(lib().hts_delayed_update(_ptr(theta), _ptr(grad), _ptr(sq_avg), int(count), float(lr), float(alpha), float(eps),
-                                    _ptr(theta_bf16), _stream(stream)), "hts_delayed_update")
+    _native.delayed_update(theta, grad, sq_avg, count, lr, alpha, eps, theta_bf16, stream)
 
 
 def hts_policy_step_host(ctx, obs, env_ids, t_per_env, t, seed, n, actions, logp, values, entropy,
                          logits=None, stream=None) -> None:
-    _check(lib().hts_policy_step_host(ctx, _ptr(obs), _ptr(env_ids), _ptr(t_per_env), int(t), int(seed), int(n),
-                                      _ptr(actions), _ptr(logp), _ptr(values), _ptr(entropy), _ptr(logits),
-                                      _stream(stream)), "hts_policy_step_host")
+    _native.policy_step_host(ctx, obs, env_ids, t_per_env, t, seed, n, actions, logp, values, entropy, logits, stream)
 
 
 def hts_policy_read_activation(ctx, layer: int, n: int, out, stream=None) -> None:
@@ -243,20 +247,16 @@ def hts_policy_destroy(ctx) -> None:
 
 
 def hts_gae(rewards, values, dones, bootstrap, gamma, lam, T, N, advantages, returns, stream=None) -> None:
-    _check(lib().hts_gae(_ptr(rewards), _ptr(values), _ptr(dones), _ptr(bootstrap), float(gamma), float(lam),
-                         int(T), int(N), _ptr(advantages), _ptr(returns), _stream(stream)), "hts_gae")
+    _native.gae(rewards, values, dones, bootstrap, gamma, lam, T, N, advantages, returns, stream)
 
 
 def hts_gae_host(rewards, values, dones, bootstrap, gamma, lam, T, N, advantages, returns, stream=None) -> None:
-    _check(lib().hts_gae_host(_ptr(rewards), _ptr(values), _ptr(dones), _ptr(bootstrap), float(gamma), float(lam),
-                              int(T), int(N), _ptr(advantages), _ptr(returns), _stream(stream)), "hts_gae_host")
+    _native.gae_host(rewards, values, dones, bootstrap, gamma, lam, T, N, advantages, returns, stream)
 
 
 def hts_vtrace(log_rhos, rewards, values, dones, bootstrap, gamma, lam, rho_bar, c_bar, T, N, vs, pg_advantages,
                stream=None) -> None:
-    _check(lib().hts_vtrace(_ptr(log_rhos), _ptr(rewards), _ptr(values), _ptr(dones), _ptr(bootstrap), float(gamma),
-                            float(lam), float(rho_bar), float(c_bar), int(T), int(N), _ptr(vs), _ptr(pg_advantages),
-                            _stream(stream)), "hts_vtrace")
+    _native.vtrace(log_rhos, rewards, values, dones, bootstrap, gamma, lam, rho_bar, c_bar, T, N, vs, pg_advantages, stream)
 
 
 def hts_gae_host_release() -> None:

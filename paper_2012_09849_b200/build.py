@@ -1,22 +1,25 @@
-"""Builds libhts.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libhts.so (the C-ABI CUDA library) with nvcc for sm_100a and _native.so (its CPython entry points), in-tree."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 LIB = os.path.join(PKG, "libhts.so")
+NATIVE = os.path.join(PKG, "_native.so")
+BINDING = os.path.join(PKG, "csrc", "binding.c")
 SOURCES = sorted(glob.glob(os.path.join(PKG, "csrc", "*.cu")))
 HEADERS = sorted(glob.glob(os.path.join(PKG, "csrc", "*.cuh"))) + [os.path.join(ROOT, "include", "hts.h")]
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
         return True
-    t = os.path.getmtime(LIB)
-    return any(os.path.getmtime(f) > t for f in SOURCES + HEADERS)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
+    return any(os.path.getmtime(f) > t for f in SOURCES + HEADERS + [BINDING])
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -29,6 +32,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if verbose:
         cmd.insert(1, "-Xptxas=-v")
     subprocess.check_call(cmd)
+    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"),
+                           "-I", sysconfig.get_paths()["include"], "-o", NATIVE, BINDING, "-L", PKG, "-l:libhts.so",
+                           "-Wl,-rpath,$ORIGIN"])
     return LIB
 
 
