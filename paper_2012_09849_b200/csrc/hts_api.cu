@@ -31,14 +31,15 @@ struct hts_ctx {
     RefWeights rw{};              // fp32 check path (weight_dtype fp32)
     RefWorkspace rws{};
     TcState* tc = nullptr;        // tensor-core path (weight_dtype bf16)
-    // staging for the host-buffer entry point
+    // staging for the host-buffer entry point: frames, then index words [2][max_batch], result words [4][max_batch] and
+    // logits on the device; the words once more in pinned host memory
     uint8_t* s_obs = nullptr;
-    int32_t *s_ids = nullptr, *s_t = nullptr, *s_act = nullptr;
-    float *s_logp = nullptr, *s_val = nullptr, *s_ent = nullptr, *s_logits = nullptr;
+    int32_t *s_index = nullptr, *s_result = nullptr, *h_words = nullptr;
+    float* s_logits = nullptr;
     X3State* x3 = nullptr;        // packed weights and workspace of the gradient (weight_dtype fp32)
     int* status = nullptr;        // device status word
     Profiler prof;
-    void* allocs[112];
+    void* allocs[8];
     int nalloc = 0;
 };
 
@@ -48,12 +49,32 @@ template <typename T>
 bool dev_alloc(hts_ctx* c, T** p, size_t count)
 {
     void* q = nullptr;
-    if (c->nalloc >= 112) return false;
+    if (c->nalloc >= 8) return false;
     if (cudaMalloc(&q, count * sizeof(T) + 256) != cudaSuccess) { cudaGetLastError(); return false; }
     c->allocs[c->nalloc++] = q;
     *p = static_cast<T*>(q);
     return true;
 }
+
+// Several buffers out of one allocation (an allocation costs tens of microseconds; a context has some thirty buffers).
+struct Carve {
+    struct Item { void** p; size_t bytes; } items[40];
+    int n = 0;
+    size_t total = 0;
+    template <typename T>
+    void add(T** p, size_t count)
+    {
+        items[n++] = {reinterpret_cast<void**>(p), total};
+        total += (count * sizeof(T) + 256 + 255) & ~(size_t)255;
+    }
+    bool alloc(hts_ctx* c)
+    {
+        uint8_t* base = nullptr;
+        if (!dev_alloc(c, &base, total)) return false;
+        for (int i = 0; i < n; ++i) *items[i].p = base + items[i].bytes;
+        return true;
+    }
+};
 
 bool raw_alloc(void* c, void** p, size_t bytes)
 {
@@ -119,6 +140,8 @@ hts_status run_step(hts_ctx* ctx, const uint8_t* obs, const Indexing& ix, const 
 
 }  // namespace
 
+constexpr int kHostDirect = 128;        // rows up to which the kernels use the context's pinned words directly
+
 // staging buffer of hts_gae_host, one per device; grows on demand, freed by hts_gae_host_release
 static char* g_gae_stage[kDeviceSlots] = {};
 static size_t g_gae_stage_bytes[kDeviceSlots] = {};
@@ -154,28 +177,23 @@ hts_status hts_policy_create(const hts_net_desc* d, hts_ctx** out)
     c->desc = *d; c->g = g;
     const size_t nb = (size_t)d->max_batch;
     const int A = g.A;
-    bool ok = dev_alloc(c, &c->status, 1);
-    if (ok && d->weight_dtype == HTS_DTYPE_BF16) {
-        hts_status st = tc_create(g, d->max_batch, c->status, &c->tc, raw_alloc, c);
-        if (st != HTS_OK) { hts_policy_destroy(c); return st; }
-    } else if (ok) {
-        ok = ok && dev_alloc(c, &c->rw.w1, (size_t)32 * g.C * 64) && dev_alloc(c, &c->rw.b1, 32);
-        ok = ok && dev_alloc(c, &c->rw.w2, (size_t)64 * 32 * 16) && dev_alloc(c, &c->rw.b2, 64);
-        ok = ok && dev_alloc(c, &c->rw.w3, (size_t)64 * 64 * 9) && dev_alloc(c, &c->rw.b3, 64);
-        ok = ok && dev_alloc(c, &c->rw.wfc, (size_t)512 * g.F) && dev_alloc(c, &c->rw.bfc, 512);
-        ok = ok && dev_alloc(c, &c->rw.whead, (size_t)(A + 1) * 512) && dev_alloc(c, &c->rw.bhead, (size_t)A + 1);
-        ok = ok && dev_alloc(c, &c->rws.a1, nb * 32 * g.H1 * g.W1) && dev_alloc(c, &c->rws.a2, nb * 64 * g.H2 * g.W2);
-        ok = ok && dev_alloc(c, &c->rws.a3, nb * g.F) && dev_alloc(c, &c->rws.h, nb * 512);
-        if (ok) {
-            const hts_status st = x3_create(g, d->max_batch, c->status, &c->x3);
-            if (st != HTS_OK) { hts_policy_destroy(c); return st; }
-        }
+    Carve cv;
+    cv.add(&c->status, 1);
+    cv.add(&c->s_obs, nb * g.C * g.H * g.W);
+    cv.add(&c->s_index, 2 * nb); cv.add(&c->s_result, 4 * nb); cv.add(&c->s_logits, nb * A);
+    if (d->weight_dtype == HTS_DTYPE_FP32) {
+        cv.add(&c->rw.w1, (size_t)32 * g.C * 64); cv.add(&c->rw.b1, 32);
+        cv.add(&c->rw.w2, (size_t)64 * 32 * 16); cv.add(&c->rw.b2, 64);
+        cv.add(&c->rw.w3, (size_t)64 * 64 * 9); cv.add(&c->rw.b3, 64);
+        cv.add(&c->rw.wfc, (size_t)512 * g.F); cv.add(&c->rw.bfc, 512);
+        cv.add(&c->rw.whead, (size_t)(A + 1) * 512); cv.add(&c->rw.bhead, (size_t)A + 1);
+        cv.add(&c->rws.a1, nb * 32 * g.H1 * g.W1); cv.add(&c->rws.a2, nb * 64 * g.H2 * g.W2);
+        cv.add(&c->rws.a3, nb * g.F); cv.add(&c->rws.h, nb * 512);
     }
-    ok = ok && dev_alloc(c, &c->s_obs, nb * g.C * g.H * g.W);
-    ok = ok && dev_alloc(c, &c->s_ids, nb) && dev_alloc(c, &c->s_t, nb) && dev_alloc(c, &c->s_act, nb);
-    ok = ok && dev_alloc(c, &c->s_logp, nb) && dev_alloc(c, &c->s_val, nb) && dev_alloc(c, &c->s_ent, nb);
-    ok = ok && dev_alloc(c, &c->s_logits, nb * A);
-    if (!ok) { hts_policy_destroy(c); return HTS_ERR_ALLOC; }
+    if (!cv.alloc(c)) { hts_policy_destroy(c); return HTS_ERR_ALLOC; }
+    const hts_status st = d->weight_dtype == HTS_DTYPE_BF16 ? tc_create(g, d->max_batch, c->status, &c->tc, raw_alloc, c)
+                                                            : x3_create(g, d->max_batch, c->status, &c->x3);
+    if (st != HTS_OK) { hts_policy_destroy(c); return st; }
     if (cudaMemset(c->status, 0, sizeof(int)) != cudaSuccess) {
         hts_status st = cuda_fail(cudaGetLastError(), "cudaMemset");
         hts_policy_destroy(c);
@@ -272,20 +290,33 @@ hts_status hts_policy_step_host(hts_ctx* ctx, const uint8_t* obs, const int32_t*
     hts_status st = check_step_args(ctx, obs, env_ids, n, actions, logp, values, entropy, true);
     if (st != HTS_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    const size_t nn = (size_t)n;
+    const size_t nn = (size_t)n, nb = (size_t)ctx->desc.max_batch;
+    // A copy costs about 4 us of the host and 2 of the stream whatever it carries, so the index and result words of a
+    // call pass through the context's pinned words: small batches' kernels read and write those themselves, larger ones
+    // take one copy each way (the heads kernel's 4-byte accesses would each cross the bus).
+    if (!ctx->h_words && cudaHostAlloc(reinterpret_cast<void**>(&ctx->h_words), 6 * nb * 4, cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        return HTS_ERR_ALLOC;
+    }
     HTS_CUDA(cudaMemcpyAsync(ctx->s_obs, obs, nn * ctx->g.C * ctx->g.H * ctx->g.W, cudaMemcpyHostToDevice, s));
-    HTS_CUDA(cudaMemcpyAsync(ctx->s_ids, env_ids, nn * 4, cudaMemcpyHostToDevice, s));
-    if (t_per_env) HTS_CUDA(cudaMemcpyAsync(ctx->s_t, t_per_env, nn * 4, cudaMemcpyHostToDevice, s));
-    st = run_step(ctx, ctx->s_obs, Indexing{}, ctx->s_ids, t_per_env ? ctx->s_t : nullptr, t, seed, n, ctx->s_act,
-                  ctx->s_logp, ctx->s_val, ctx->s_ent, logits_or_null ? ctx->s_logits : nullptr, s);
+    int32_t *h_in = ctx->h_words, *h_out = ctx->h_words + 2 * nb;
+    std::memcpy(h_in, env_ids, nn * 4);
+    if (t_per_env) std::memcpy(h_in + nn, t_per_env, nn * 4);
+    const bool direct = n <= kHostDirect;
+    int32_t *in = direct ? h_in : ctx->s_index, *out = direct ? h_out : ctx->s_result;
+    if (!direct) HTS_CUDA(cudaMemcpyAsync(in, h_in, (t_per_env ? 2 : 1) * nn * 4, cudaMemcpyHostToDevice, s));
+    float* outf = reinterpret_cast<float*>(out);
+    st = run_step(ctx, ctx->s_obs, Indexing{}, in, t_per_env ? in + nn : nullptr, t, seed, n, out, outf + nn, outf + 2 * nn, outf + 3 * nn,
+                  logits_or_null ? ctx->s_logits : nullptr, s);
     if (st != HTS_OK) return st;
-    HTS_CUDA(cudaMemcpyAsync(actions, ctx->s_act, nn * 4, cudaMemcpyDeviceToHost, s));
-    HTS_CUDA(cudaMemcpyAsync(logp, ctx->s_logp, nn * 4, cudaMemcpyDeviceToHost, s));
-    HTS_CUDA(cudaMemcpyAsync(values, ctx->s_val, nn * 4, cudaMemcpyDeviceToHost, s));
-    HTS_CUDA(cudaMemcpyAsync(entropy, ctx->s_ent, nn * 4, cudaMemcpyDeviceToHost, s));
+    if (!direct) HTS_CUDA(cudaMemcpyAsync(h_out, out, 4 * nn * 4, cudaMemcpyDeviceToHost, s));
     if (logits_or_null)
         HTS_CUDA(cudaMemcpyAsync(logits_or_null, ctx->s_logits, nn * ctx->g.A * 4, cudaMemcpyDeviceToHost, s));
     HTS_CUDA(cudaStreamSynchronize(s));
+    std::memcpy(actions, h_out, nn * 4);
+    std::memcpy(logp, h_out + nn, nn * 4);
+    std::memcpy(values, h_out + 2 * nn, nn * 4);
+    std::memcpy(entropy, h_out + 3 * nn, nn * 4);
     return HTS_OK;
 }
 
@@ -380,6 +411,7 @@ void hts_policy_destroy(hts_ctx* ctx)
     if (ctx->tc) tc_destroy(ctx->tc);
     if (ctx->x3) x3_destroy(ctx->x3);
     for (int i = 0; i < ctx->nalloc; ++i) cudaFree(ctx->allocs[i]);
+    if (ctx->h_words) cudaFreeHost(ctx->h_words);
     delete ctx;
 }
 

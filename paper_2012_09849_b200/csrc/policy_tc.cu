@@ -18,6 +18,7 @@
 // Activations are stored as fp16 (clamped at the largest finite value): 11 significant bits
 // instead of bf16's 8, which keeps the logits well inside the 2e-2 parity bound.
 #include <new>
+#include <type_traits>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include "common.cuh"
@@ -688,21 +689,29 @@ hts_status tc_create(const Geometry& g, int max_batch, int* status, TcState** ou
     for (int s = 8; s >= 1; --s) if (chunks % s == 0) { t->splits = s; break; }
     t->cps = chunks / t->splits;
     const size_t nb = (size_t)max_batch;
-    auto A = [&](auto** p, size_t count) { return alloc(alloc_ctx, reinterpret_cast<void**>(p), count * sizeof(**p)); };
-    bool ok = A(&t->w2p, (size_t)64 * 512) && A(&t->w3p, (size_t)64 * 576) && A(&t->wfcp, (size_t)512 * g.F) &&
-              A(&t->w1p, (size_t)128 * 16 * g.C) && A(&t->b1, 32) && A(&t->b2, 64) && A(&t->b3, 64) && A(&t->bfc, 512) &&
-              A(&t->whead, (size_t)(g.A + 1) * 512) && A(&t->bhead, (size_t)g.A + 1) &&
-              A(&t->absmax, L_COUNT + 1) && A(&t->scale, L_COUNT) && A(&t->inv_scale, L_COUNT) &&
-              A(&t->a1s, nb * t->P1s * 128) && A(&t->a2, nb * t->P2 * 64) && A(&t->a3, nb * g.F) &&
-              A(&t->hpart, (size_t)t->splits * nb * 512) && A(&t->h, nb * 512);
-    if (!ok) { delete t; return HTS_ERR_ALLOC; }
+    // one allocation for all buffers: sizes first, then the pointers
+    uint8_t* base = nullptr;
+    for (int pass = 0; pass < 2; ++pass) {
+        size_t total = 0;
+        auto A = [&](auto** p, size_t count) {
+            *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(base + total);
+            total += (count * sizeof(**p) + 256 + 1023) & ~(size_t)1023;
+        };
+        A(&t->w2p, (size_t)64 * 512); A(&t->w3p, (size_t)64 * 576); A(&t->wfcp, (size_t)512 * g.F);
+        A(&t->w1p, (size_t)128 * 16 * g.C); A(&t->b1, 32); A(&t->b2, 64); A(&t->b3, 64); A(&t->bfc, 512);
+        A(&t->whead, (size_t)(g.A + 1) * 512); A(&t->bhead, (size_t)g.A + 1);
+        A(&t->absmax, L_COUNT + 1); A(&t->scale, L_COUNT); A(&t->inv_scale, L_COUNT);
+        A(&t->a1s, nb * t->P1s * 128); A(&t->a2, nb * t->P2 * 64); A(&t->a3, nb * g.F);
+        A(&t->hpart, (size_t)t->splits * nb * 512); A(&t->h, nb * 512);
+        if (pass == 0 && !alloc(alloc_ctx, reinterpret_cast<void**>(&base), total)) { delete t; return HTS_ERR_ALLOC; }
+    }
     // cells of an odd-sized s2d border that conv1 never writes must hold finite numbers
     if (cudaMemset(t->a1s, 0, nb * t->P1s * 128 * 2) != cudaSuccess) { delete t; return cuda_fail(cudaGetLastError(), "cudaMemset"); }
     if (cudaMemset(t->absmax, 0, (L_COUNT + 1) * sizeof(unsigned)) != cudaSuccess) { delete t; return cuda_fail(cudaGetLastError(), "cudaMemset"); }
     t->rows2 = conv_res_tile_rows(t->W1s + 1);
     t->rows3 = conv_res_tile_rows(2 * g.W2 + 2);
     if (t->rows2 > 256 || t->rows3 > 256) { delete t; return HTS_ERR_SHAPE; }
-    ok = make_map(&t->mW1, t->w1p, 128, 16 * g.C, (uint64_t)32 * g.C, 64) &&
+    const bool ok = make_map(&t->mW1, t->w1p, 128, 16 * g.C, (uint64_t)32 * g.C, 64) &&
          make_map(&t->mA2, t->a1s, nb * t->P1s, 128, 256, t->rows2) && make_map(&t->mB2, t->w2p, 64, 512, 1024, 64) &&
          make_map(&t->mA3, t->a2, nb * t->P2, 64, 128, t->rows3) && make_map(&t->mB3, t->w3p, 64, 576, 1152, 64) &&
          make_map(&t->mAfc, t->a3, nb, g.F, (uint64_t)g.F * 2, BM) && make_map(&t->mBfc, t->wfcp, 512, g.F, (uint64_t)g.F * 2, 128);
