@@ -38,7 +38,7 @@ template <> __device__ __forceinline__ float4 pack<4>(const float* o) { return m
 // columns spreads over four times as many SMs.  Chunk boundaries, and with them every rounding, do not depend
 // on CY or W.
 template <int VEC, int L, int CY>
-__global__ void __launch_bounds__(VEC == 4 ? 512 : 1024)
+__global__ void __launch_bounds__(VEC == 4 ? 64 : 1024)
 gae_scan_kernel(const float* __restrict__ rewards, const float* __restrict__ values,
                 const uint8_t* __restrict__ dones, const float* __restrict__ bootstrap,
                 float gamma, float lambda, int T, int N,
@@ -57,6 +57,8 @@ gae_scan_kernel(const float* __restrict__ rewards, const float* __restrict__ val
     float* sS = smem;
     float* sP = smem + NC * cols;
     const float gl = gamma * lambda;
+    pdl_wait();
+    pdl_trigger();
 
     float carry_in[VEC];                             // advantage at the first row after this super-chunk
 #pragma unroll
@@ -152,20 +154,16 @@ gae_scan_kernel(const float* __restrict__ rewards, const float* __restrict__ val
 
 template <int VEC, int L, int CY>
 hts_status launch_t(const float* r, const float* v, const uint8_t* d, const float* b, float gamma,
-                    float lambda, int T, int N, float* adv, float* ret, cudaStream_t s)
+                    float lambda, int T, int N, float* adv, float* ret, int maxW, cudaStream_t s)
 {
-    // Wide problems (VEC == 4) have all the parallelism they need across env: two chunks per block
-    // measured best (86 % of the copy bandwidth at T=128, N=2^20).  Narrow ones cut time as finely
-    // as a block allows.
     const int chunks = (T + L - 1) / L;
     int W = (chunks + CY - 1) / CY;
-    const int maxW = (VEC == 4) ? 2 : 32;
     if (W > maxW) W = maxW;
     const int cols = 32 / CY * VEC;
     const unsigned blocks = (unsigned)((N + cols - 1) / cols);
     const size_t smem = (size_t)2 * W * CY * cols * sizeof(float);
-    gae_scan_kernel<VEC, L, CY><<<blocks, dim3(32, W), smem, s>>>(r, v, d, b, gamma, lambda, T, N, adv, ret);
-    HTS_LAUNCH_CHECK("gae_scan_kernel");
+    HTS_CUDA(launch_pdl(gae_scan_kernel<VEC, L, CY>, dim3(blocks), dim3(32, W), smem, s, r, v, d, b, gamma, lambda, T, N, adv, ret));
+    note_launch();
     return HTS_OK;
 }
 
@@ -181,11 +179,18 @@ hts_status launch_gae(const float* rewards, const float* values, const uint8_t* 
     const bool vec4 = (N % 4 == 0) && aligned(rewards, 16) && aligned(values, 16) && aligned(dones, 4) &&
                       aligned(bootstrap, 16) && aligned(adv, 16) && aligned(ret, 16) &&
                       ((long)N * T >= (1L << 22));
-    if (vec4) return launch_t<4, 2, 1>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, s);
+    const int sms = device_sm_count(device_slot());
+    // Enough blocks of 128 columns: all the parallelism needed is across env, two chunks of two rows per block measured best
+    // (86 % of the copy bandwidth at T=128, N=2^20).  Fewer would walk a long T in many short steps, each waiting for
+    // memory (213 us at 512 x 32768, 60 with the columns of a block cut to 32 and eight chunks of eight rows per step).
+    if (vec4 && N / 128 >= 4 * sms)
+        return launch_t<4, 2, 1>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, 2, s);
     // few columns and many rows: 8-column blocks, four chunks per warp (same chunks, same bits, four times the SMs)
-    if ((N + 31) / 32 < device_sm_count(device_slot()) / 2 && T >= 4 * 8)
-        return launch_t<1, 8, 4>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, s);
-    return launch_t<1, 8, 1>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, s);
+    const int blocks = (N + 31) / 32;
+    if (blocks < sms / 2 && T >= 4 * 8)
+        return launch_t<1, 8, 4>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, 32, s);
+    // several blocks per SM load, chain and store at different times; one per SM takes as many rows as it can
+    return launch_t<1, 8, 1>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, blocks >= 4 * sms ? 8 : 32, s);
 }
 
 }  // namespace hts

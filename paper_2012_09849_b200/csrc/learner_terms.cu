@@ -41,6 +41,8 @@ sums_kernel(const Op op, long long count, long long per_block)
     constexpr int NS = Op::NS;
     __shared__ double s_part[kThreads / 32][NS];
     __shared__ bool s_last;
+    pdl_wait();                               // the partials and the ticket, and the inputs, are the previous kernel's
+    pdl_trigger();
     const long long lo = (long long)blockIdx.x * per_block;               // per_block is a multiple of 4
     long long hi = lo + per_block; hi = hi > count ? count : hi;
     double acc[NS];
@@ -99,15 +101,15 @@ sums_kernel(const Op op, long long count, long long per_block)
 }
 
 template <class Op>
-hts_status launch_sums(const Op& op, long long count, cudaStream_t s, const char* name)
+hts_status launch_sums(const Op& op, long long count, cudaStream_t s)
 {
     long long blocks = (count + (long long)kThreads * kPerThread - 1) / ((long long)kThreads * kPerThread);
     if (blocks > kBlocksMax) blocks = kBlocksMax;
     long long per_block = (count + blocks - 1) / blocks;
     per_block = (per_block + 3) / 4 * 4;
     blocks = (count + per_block - 1) / per_block;
-    sums_kernel<Op><<<(unsigned)blocks, kThreads, 0, s>>>(op, count, per_block);
-    HTS_LAUNCH_CHECK(name);
+    HTS_CUDA(launch_pdl(sums_kernel<Op>, dim3((unsigned)blocks), dim3(kThreads), 0, s, op, count, per_block));
+    note_launch();
     return HTS_OK;
 }
 
@@ -148,33 +150,28 @@ struct A2cOp {
     }
 };
 
-// first and second pass over the advantages: mean, then 1 / (population std + 1e-8)
-struct AdvMeanOp {
-    static constexpr int NS = 1;
+// Mean and 1 / (population std + 1e-8) of the advantages in one pass: sums of a - a_0 and its square in double
+// precision (the shift keeps a mean far from zero from cancelling the variance).
+struct AdvStatsOp {
+    static constexpr int NS = 2;
     const float* adv;
     bool vec;
     using Quad = float4;
     __device__ bool aligned16() const { return vec; }
     __device__ Quad load4(long long q) const { return reinterpret_cast<const float4*>(adv)[q]; }
-    __device__ void add4(const Quad& g, double* acc) const { acc[0] += (double)g.x; acc[0] += (double)g.y; acc[0] += (double)g.z; acc[0] += (double)g.w; }
-    __device__ void add1(long long i, double* acc) const { acc[0] += (double)adv[i]; }
-    __device__ void finish(const double* tot, long long count) const { g_adv_stats[0] = tot[0] / (double)count; }
-};
-struct AdvVarOp {
-    static constexpr int NS = 1;
-    const float* adv;
-    bool vec;
-    using Quad = float4;
-    __device__ bool aligned16() const { return vec; }
-    __device__ Quad load4(long long q) const { return reinterpret_cast<const float4*>(adv)[q]; }
-    __device__ static void one(float a, double mean, double* acc) { const double d = (double)a - mean; acc[0] += d * d; }
+    __device__ static void one(float a, double first, double* acc) { const double d = (double)a - first; acc[0] += d; acc[1] += d * d; }
     __device__ void add4(const Quad& g, double* acc) const
     {
-        const double m = g_adv_stats[0];
-        one(g.x, m, acc); one(g.y, m, acc); one(g.z, m, acc); one(g.w, m, acc);
+        const double f = (double)adv[0];
+        one(g.x, f, acc); one(g.y, f, acc); one(g.z, f, acc); one(g.w, f, acc);
     }
-    __device__ void add1(long long i, double* acc) const { one(adv[i], g_adv_stats[0], acc); }
-    __device__ void finish(const double* tot, long long count) const { g_adv_stats[1] = 1.0 / (sqrt(tot[0] / (double)count) + 1e-8); }
+    __device__ void add1(long long i, double* acc) const { one(adv[i], (double)adv[0], acc); }
+    __device__ void finish(const double* tot, long long count) const
+    {
+        const double d = tot[0] / (double)count, var = tot[1] / (double)count - d * d;
+        g_adv_stats[0] = (double)adv[0] + d;
+        g_adv_stats[1] = 1.0 / (sqrt(var > 0.0 ? var : 0.0) + 1e-8);
+    }
 };
 
 struct PpoOp {
@@ -229,7 +226,7 @@ extern "C" hts_status hts_a2c_terms(const float* logp, const float* values, cons
     using namespace hts;
     if (!logp || !values || !entropy || !returns || !out3 || count < 1) return HTS_ERR_INVALID_ARG;
     const A2cOp op{logp, values, entropy, returns, out3, all_aligned16({logp, values, entropy, returns})};
-    return launch_sums(op, (long long)count, static_cast<cudaStream_t>(cuda_stream), "a2c_terms");
+    return launch_sums(op, (long long)count, static_cast<cudaStream_t>(cuda_stream));
 }
 
 extern "C" hts_status hts_ppo_terms(const float* logp_new, const float* logp_old, const float* values, const float* entropy,
@@ -241,15 +238,12 @@ extern "C" hts_status hts_ppo_terms(const float* logp_new, const float* logp_old
     if (!(clip > 0.f) || std::isinf(clip)) return HTS_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     if (normalize_advantages) {
-        const bool av = all_aligned16({advantages});
-        hts_status st = launch_sums(AdvMeanOp{advantages, av}, (long long)count, s, "adv_mean");
-        if (st != HTS_OK) return st;
-        st = launch_sums(AdvVarOp{advantages, av}, (long long)count, s, "adv_var");
+        const hts_status st = launch_sums(AdvStatsOp{advantages, all_aligned16({advantages})}, (long long)count, s);
         if (st != HTS_OK) return st;
     }
     const PpoOp op{logp_new, logp_old, values, entropy, advantages, returns, out4, (double)clip, normalize_advantages != 0,
                    all_aligned16({logp_new, logp_old, values, entropy, advantages, returns})};
-    return launch_sums(op, (long long)count, s, "ppo_terms");
+    return launch_sums(op, (long long)count, s);
 }
 
 // ---- the learner's parameter update (Section 4.1 "Delayed gradient", Eq. 5) ---------------------------------
@@ -277,6 +271,8 @@ __global__ void __launch_bounds__(256)
 delayed_update_kernel(float* __restrict__ theta, const float* __restrict__ grad, float* __restrict__ sq_avg,
                       long long count, float lr, float alpha, float eps, __nv_bfloat16* __restrict__ theta_bf16)
 {
+    pdl_wait();
+    pdl_trigger();
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long done = 0;
@@ -325,10 +321,9 @@ extern "C" hts_status hts_delayed_update(float* theta, const float* grad, float*
     const bool vec = (((uintptr_t)theta | (uintptr_t)grad | (uintptr_t)sq_avg_or_null) & 15u) == 0 && ((uintptr_t)tb & 7u) == 0;
     const unsigned gb = (unsigned)blocks;
     const long long n = (long long)count;
-    if (sq_avg_or_null && vec) delayed_update_kernel<true, true><<<gb, 256, 0, s>>>(theta, grad, sq_avg_or_null, n, lr, alpha, eps, tb);
-    else if (sq_avg_or_null) delayed_update_kernel<true, false><<<gb, 256, 0, s>>>(theta, grad, sq_avg_or_null, n, lr, alpha, eps, tb);
-    else if (vec) delayed_update_kernel<false, true><<<gb, 256, 0, s>>>(theta, grad, nullptr, n, lr, alpha, eps, tb);
-    else delayed_update_kernel<false, false><<<gb, 256, 0, s>>>(theta, grad, nullptr, n, lr, alpha, eps, tb);
-    HTS_LAUNCH_CHECK("delayed_update_kernel");
+    auto kernel = sq_avg_or_null ? (vec ? delayed_update_kernel<true, true> : delayed_update_kernel<true, false>)
+                                 : (vec ? delayed_update_kernel<false, true> : delayed_update_kernel<false, false>);
+    HTS_CUDA(launch_pdl(kernel, dim3(gb), dim3(256), 0, s, theta, grad, sq_avg_or_null, n, lr, alpha, eps, tb));
+    note_launch();
     return HTS_OK;
 }

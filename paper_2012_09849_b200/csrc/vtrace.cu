@@ -40,24 +40,28 @@ struct VtraceParams {
     float *vs, *pg;
 };
 
-// blockDim = (32, W).  Block b owns columns [b*32*VEC, (b+1)*32*VEC).  Time is walked from the end in
-// super-chunks of W*L rows; warp w owns rows [t0 + w*L, t0 + (w+1)*L) of the super-chunk.
-template <int VEC, int L>
-__global__ void __launch_bounds__(VEC == 4 ? 512 : 1024)
+// blockDim = (32, W).  A warp is CY rows of 32/CY threads, as in the advantage scan: thread (cx, cy) of warp w owns
+// columns [b*cols + cx*VEC, +VEC) (cols = 32/CY*VEC) and chunk w*CY + cy of the super-chunk.  Time is walked from the
+// end in super-chunks of W*CY*L rows.  Chunk boundaries, and with them every rounding, do not depend on CY or W.
+template <int VEC, int L, int CY, int MAXW>
+__global__ void __launch_bounds__(32 * MAXW)
 vtrace_scan_kernel(const VtraceParams p)
 {
     using F = typename VecT<VEC>::F;
     using B = typename VecT<VEC>::B;
     extern __shared__ float smem[];                  // [W][32*VEC] S, then P, then V and vs of each chunk's first row
-    const int W = blockDim.y;
-    const int w = threadIdx.y;
-    const int lane = threadIdx.x;
-    const int cols = 32 * VEC;
+    constexpr int CXW = 32 / CY;                     // threads of a warp along env
+    const int W = blockDim.y * CY;                   // chunks of a super-chunk
+    const int lane = threadIdx.x % CXW;
+    const int w = threadIdx.y * CY + threadIdx.x / CXW;
+    const int cols = CXW * VEC;
     const int T = p.T, N = p.N;
     const long col = (long)blockIdx.x * cols + lane * VEC;
     const bool col_ok = col < N;                     // N % VEC == 0 is guaranteed by the launcher
     float* sS = smem;
     float* sP = smem + W * cols;
+    pdl_wait();
+    pdl_trigger();
 
     float carry_in[VEC];                             // D at the first row after this super-chunk
 #pragma unroll
@@ -156,17 +160,16 @@ vtrace_scan_kernel(const VtraceParams p)
     }
 }
 
-template <int VEC, int L>
+template <int VEC, int L, int CY, int MAXW>
 hts_status launch_t(const VtraceParams& p, cudaStream_t s)
 {
-    int W = (p.T + L - 1) / L;
-    const int maxW = (VEC == 4) ? 2 : 32;
-    if (W > maxW) W = maxW;
-    const int cols = 32 * VEC;
+    int W = ((p.T + L - 1) / L + CY - 1) / CY;
+    if (W > MAXW) W = MAXW;
+    const int cols = 32 / CY * VEC;
     const unsigned blocks = (unsigned)((p.N + cols - 1) / cols);
-    const size_t smem = (size_t)2 * W * cols * sizeof(float);
-    vtrace_scan_kernel<VEC, L><<<blocks, dim3(32, W), smem, s>>>(p);
-    HTS_LAUNCH_CHECK("vtrace_scan_kernel");
+    const size_t smem = (size_t)2 * W * CY * cols * sizeof(float);
+    HTS_CUDA(launch_pdl(vtrace_scan_kernel<VEC, L, CY, MAXW>, dim3(blocks), dim3(32, W), smem, s, p));
+    note_launch();
     return HTS_OK;
 }
 
@@ -182,8 +185,12 @@ hts_status launch_vtrace(const float* log_rhos, const float* rewards, const floa
     const bool vec4 = (N % 4 == 0) && aligned(rewards, 16) && aligned(values, 16) && aligned(log_rhos, 16) &&
                       aligned(dones, 4) && aligned(bootstrap, 16) && aligned(vs, 16) && aligned(pg, 16) &&
                       ((long)N * T >= (1L << 22));
-    if (vec4) return launch_t<4, 2>(p, s);
-    return launch_t<1, 8>(p, s);
+    // the advantage scan's rules, with at most 512 threads (1024 would leave 64 registers: spills)
+    const int sms = device_sm_count(device_slot()), blocks = (N + 31) / 32;
+    if (vec4 && N / 128 >= 4 * sms) return launch_t<4, 2, 1, 2>(p, s);
+    if (blocks < sms / 2 && T >= 4 * 8) return launch_t<1, 8, 4, 16>(p, s);
+    if (blocks >= 8 * sms) return launch_t<1, 8, 1, 4>(p, s);        // 91 us at 256 x 60001; 143 with one 1024-thread block
+    return blocks >= sms ? launch_t<1, 8, 1, 8>(p, s) : launch_t<1, 8, 1, 16>(p, s);
 }
 
 }  // namespace hts
