@@ -73,8 +73,8 @@ struct Conv1Params {
     int pool;               // frames in obs when slots are given
     int n;
     int tiles;              // ceil(n * Ws / 124)
-    int splits;             // equal ranges the H1 output rows of a tile are cut into (a divisor of H1)
-    int su;                 // output rows (steps) per unit: H1 / splits; a unit stages su + 1 grid rows
+    int splits;             // ranges of su output rows a tile is cut into; the last may reach past row H1
+    int su;                 // output rows (steps) per unit; a unit stages su + 1 grid rows
     const float* bias;
     const float* inv_scale;
     __half* out;
@@ -362,7 +362,7 @@ conv1_march_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                         fma2(a0, a1, inv, s_bias[c], s_bias[c + 1]);
                         pk[hh] = relu_pack_h2(a0, a1);
                     }
-                    if (valid)
+                    if (valid && y < pl.H1)
                         asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                                      ::"l"(dst + j), "r"(pk[0]), "r"(pk[1]), "r"(pk[2]), "r"(pk[3]), "r"(pk[4]), "r"(pk[5]),
                                        "r"(pk[6]), "r"(pk[7]) : "memory");
@@ -390,7 +390,7 @@ conv1_march_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                         fma2(a0, a1, inv, s_bias[j + c], s_bias[j + c + 1]);
                         pk[hh] = relu_pack_h2(a0, a1);
                     }
-                    if (valid)
+                    if (valid && y < pl.H1)
                         asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                                      ::"l"(dst + j), "r"(pk[0]), "r"(pk[1]), "r"(pk[2]), "r"(pk[3]), "r"(pk[4]), "r"(pk[5]),
                                        "r"(pk[6]), "r"(pk[7]) : "memory");
@@ -407,19 +407,18 @@ conv1_march_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     if (warp == 1) tmem_dealloc(tmem_slot, S::TMEM);
 }
 
-// output-row ranges per tile: enough units that every CTA of the grid gets several, few enough that the extra
-// grid row each unit converts (a unit of k steps stages k + 1 rows) stays cheap
-int choose_splits(int tiles, int H1, int grid)
+// Output rows per unit: enough units that every CTA of the grid gets several, few enough that the extra grid row each
+// unit converts (a unit of k steps stages k + 1 rows) stays cheap.  The last range of a tile may reach past the last
+// output row (its surplus rows read as zero and are dropped): 17 rows, which nothing divides, kept a small football batch
+// on one CTA per tile (n = 8: conv1 28 -> 11 us).
+int choose_rows(int tiles, int H1, int grid)
 {
-    int best = 1;
+    int best = H1;
     long best_cost = -1;
-    for (int s = 1; s <= H1; ++s) {
-        if (H1 % s) continue;                              // equal ranges only
-        const int steps = H1 / s;
-        if (s > 1 && steps < 2) break;
-        const long rounds = ((long)tiles * s + grid - 1) / grid;
-        const long cost = rounds * (steps + 2);
-        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = s; }
+    for (int su = H1; su >= (H1 > 1 ? 2 : 1); --su) {
+        const long rounds = ((long)tiles * ((H1 + su - 1) / su) + grid - 1) / grid;
+        const long cost = rounds * (su + 2);
+        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = su; }
     }
     return best;
 }
@@ -495,8 +494,8 @@ hts_status conv1_launch(const Conv1Plan& pl, const CUtensorMap& weight_map, Conv
     p.pl = pl; p.obs = obs; p.slots = ix.slots; p.pool = ix.pool; p.n = n;
     p.tiles = (int)((cols + kTileCols - 1) / kTileCols);
     const int max_grid = (pl.CG == 1 ? Shape<1>::PER_SM : 1) * sm_count;
-    p.splits = choose_splits(p.tiles, pl.H1, max_grid);
-    p.su = pl.H1 / p.splits;
+    p.su = choose_rows(p.tiles, pl.H1, max_grid);
+    p.splits = (pl.H1 + p.su - 1) / p.su;
     p.bias = bias; p.inv_scale = inv_scale; p.out = out; p.status = status;
     const long units = (long)p.tiles * p.splits;
     const int grid = units < max_grid ? (int)units : max_grid;
