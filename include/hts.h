@@ -268,7 +268,8 @@ hts_status hts_action_uniforms(const int32_t *env_ids, const int32_t *t_per_env,
  * hts_policy_profile(ctx, 1) starts a fresh collection, (ctx, 0) stops recording.
  * hts_policy_profile_read waits for the recorded events and returns, for kernel index
  * 0..4 (hts_policy_kernel_name gives "conv1","conv2","conv3","fc","heads"), the summed
- * device time in milliseconds and the number of launches recorded.                  */
+ * device time in milliseconds and the number of launches recorded (batches whose three
+ * convolutions run as one kernel are recorded as "conv1").                           */
 hts_status hts_policy_profile(hts_ctx *ctx, int32_t enable);
 hts_status hts_policy_profile_read(hts_ctx *ctx, int32_t kernel, float *total_ms, int32_t *launches);
 const char *hts_policy_kernel_name(int32_t kernel);

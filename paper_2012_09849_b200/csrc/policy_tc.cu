@@ -26,6 +26,7 @@
 #include "tc_host.cuh"
 #include "conv1_tc.cuh"
 #include "conv_res_tc.cuh"
+#include "conv_stack_tc.cuh"
 
 namespace hts {
 using namespace tc;
@@ -659,6 +660,8 @@ struct TcState {
     float *hpart, *h;
     CUtensorMap mW1, mA2, mB2, mA3, mB3, mAfc, mBfc;
     int rows2, rows3;           // activation tile rows of conv2 / conv3
+    bool stacked;               // the frames fit the kernel that runs all three convolutions
+    ConvStackParams stack;
     int* status;
 };
 
@@ -716,6 +719,11 @@ hts_status tc_create(const Geometry& g, int max_batch, int* status, TcState** ou
          make_map(&t->mA3, t->a2, nb * t->P2, 64, 128, t->rows3) && make_map(&t->mB3, t->w3p, 64, 576, 1152, 64) &&
          make_map(&t->mAfc, t->a3, nb, g.F, (uint64_t)g.F * 2, BM) && make_map(&t->mBfc, t->wfcp, 512, g.F, (uint64_t)g.F * 2, 128);
     if (!ok) { delete t; return HTS_ERR_CUDA; }
+    t->stack = ConvStackParams{};
+    t->stacked = conv_stack_plan(g, &t->stack);
+    ConvStackParams& cs = t->stack;
+    cs.b1 = t->b1; cs.b2 = t->b2; cs.b3 = t->b3; cs.inv1 = t->inv_scale + L_CONV1; cs.inv2 = t->inv_scale + L_CONV2; cs.inv3 = t->inv_scale + L_CONV3;
+    cs.a1 = t->a1s; cs.a2 = t->a2; cs.a3 = t->a3; cs.status = status;
     *out = t;
     return HTS_OK;
 }
@@ -749,31 +757,41 @@ hts_status tc_load_weights(TcState* t, const hts_weights& w, cudaStream_t s)
 hts_status tc_forward(TcState* t, const uint8_t* obs, const Indexing& ix, int n, Profiler& prof, cudaStream_t s)
 {
     const Geometry& g = t->g;
-    prof.begin(K_CONV1, s);
-    hts_status st = conv1_launch(t->pl1, t->mW1, t->maps1, obs, ix, n, t->b1, t->inv_scale + L_CONV1, t->a1s, t->status, s);
-    if (st != HTS_OK) return st;
-    prof.end(K_CONV1, s);
+    hts_status st;
+    if (t->stacked && n <= kStackEnvs * device_sm_count(device_slot())) {
+        ConvStackParams c = t->stack;
+        c.obs = obs; c.slots = ix.slots; c.pool = ix.pool; c.n = n;
+        prof.begin(K_CONV1, s);
+        st = conv_stack_launch(t->mW1, t->mB2, t->mB3, c, s);
+        if (st != HTS_OK) return st;
+        prof.end(K_CONV1, s);
+    } else {
+        prof.begin(K_CONV1, s);
+        st = conv1_launch(t->pl1, t->mW1, t->maps1, obs, ix, n, t->b1, t->inv_scale + L_CONV1, t->a1s, t->status, s);
+        if (st != HTS_OK) return st;
+        prof.end(K_CONV1, s);
 
-    // conv2: 2x2 taps on the s2d grid [H1s, W1s] with 128 channels -> [H2, W2] x 64
-    ConvResParams c{};
-    c.status = t->status; c.n_env = n;
-    c.tap_shift[0] = 0; c.tap_shift[1] = 1; c.tap_shift[2] = t->W1s; c.tap_shift[3] = t->W1s + 1;
-    c.tile_rows = t->rows2; c.total_rows = n * t->P1s;
-    c.P_in = t->P1s; c.W_in = t->W1s; c.H_out = g.H2; c.W_out = g.W2; c.P_out = t->P2;
-    c.bias = t->b2; c.out = t->a2; c.inv_scale = t->inv_scale + L_CONV2;
-    prof.begin(K_CONV2, s);
-    st = conv_res_launch<4, 2>(t->mA2, t->mB2, c, s);
-    if (st != HTS_OK) return st;
-    prof.end(K_CONV2, s);
-    // conv3: 3x3 taps on [H2, W2] x 64 -> [H3, W3] x 64
-    for (int dy = 0; dy < 3; ++dy) for (int dx = 0; dx < 3; ++dx) c.tap_shift[dy * 3 + dx] = dy * g.W2 + dx;
-    c.tile_rows = t->rows3; c.total_rows = n * t->P2;
-    c.P_in = t->P2; c.W_in = g.W2; c.H_out = g.H3; c.W_out = g.W3; c.P_out = t->P3;
-    c.bias = t->b3; c.out = t->a3; c.inv_scale = t->inv_scale + L_CONV3;
-    prof.begin(K_CONV3, s);
-    st = conv_res_launch<9, 1>(t->mA3, t->mB3, c, s);
-    if (st != HTS_OK) return st;
-    prof.end(K_CONV3, s);
+        // conv2: 2x2 taps on the s2d grid [H1s, W1s] with 128 channels -> [H2, W2] x 64
+        ConvResParams c{};
+        c.status = t->status; c.n_env = n;
+        c.tap_shift[0] = 0; c.tap_shift[1] = 1; c.tap_shift[2] = t->W1s; c.tap_shift[3] = t->W1s + 1;
+        c.tile_rows = t->rows2; c.total_rows = n * t->P1s;
+        c.P_in = t->P1s; c.W_in = t->W1s; c.H_out = g.H2; c.W_out = g.W2; c.P_out = t->P2;
+        c.bias = t->b2; c.out = t->a2; c.inv_scale = t->inv_scale + L_CONV2;
+        prof.begin(K_CONV2, s);
+        st = conv_res_launch<4, 2>(t->mA2, t->mB2, c, s);
+        if (st != HTS_OK) return st;
+        prof.end(K_CONV2, s);
+        // conv3: 3x3 taps on [H2, W2] x 64 -> [H3, W3] x 64
+        for (int dy = 0; dy < 3; ++dy) for (int dx = 0; dx < 3; ++dx) c.tap_shift[dy * 3 + dx] = dy * g.W2 + dx;
+        c.tile_rows = t->rows3; c.total_rows = n * t->P2;
+        c.P_in = t->P2; c.W_in = g.W2; c.H_out = g.H3; c.W_out = g.W3; c.P_out = t->P3;
+        c.bias = t->b3; c.out = t->a3; c.inv_scale = t->inv_scale + L_CONV3;
+        prof.begin(K_CONV3, s);
+        st = conv_res_launch<9, 1>(t->mA3, t->mB3, c, s);
+        if (st != HTS_OK) return st;
+        prof.end(K_CONV3, s);
+    }
     GemmParams p{};
     p.status = t->status; p.n_env = n;
     // FC: [n, F] x [512, F]^T, K split across blockIdx.z
