@@ -38,6 +38,11 @@ __device__ __forceinline__ float4 load4(const float* p, bool vec)
     return vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
 }
 
+// Where the next kernel may start.  Blocks of a dependent launch that become resident early all settle on the first SMs
+// that have room and stay there, waiting, while the others get none: its work then runs unevenly.  So the convolutions
+// and the wide fully-connected form let it start as they end (no trigger), which costs it no more than its prologue:
+// n = 40 / 160 / 256 / 1024: 96 / 194 / 241 / 587 us per step with triggers after the wait, 81 / 168 / 201 / 549 without.
+// The narrow fully-connected form, before the small heads, still triggers (0.5 us per step).
 struct ConvParams {
     const void* x;                      // [frames][C][H][W], u8 or fp32
     const float *w, *b;                 // [O][C k k], [O]
@@ -101,7 +106,6 @@ conv_tile_kernel(const ConvParams p)
         s_off[u] = (c * p.H + uu) * p.W + (r - uu * p.k);
     }
     pdl_wait();
-    pdl_trigger();
     const TIn* src[NPX];
 #pragma unroll
     for (int q = 0; q < NPX; ++q) {
@@ -270,7 +274,6 @@ conv_small_kernel(const ConvParams p, int ring)
         }
     };
     pdl_wait();
-    pdl_trigger();
     for (int g = 0; g < ring; ++g) fetch_w(g, g);
     if (tid < kSmallPx) {
         int px = px0 + tid;
@@ -400,7 +403,7 @@ fc_chain_kernel(const float* __restrict__ x, const float* __restrict__ w, const 
     const int we = warp % WE, wo = warp / WE;
     const int e0 = (blockIdx.y * WE + we) * TE, o0 = (blockIdx.x * WO + wo) * TO;
     pdl_wait();
-    pdl_trigger();
+    if constexpr (TE < 8) pdl_trigger();
     f32x2 acc[TE][TO / 2];
 #pragma unroll
     for (int i = 0; i < TE; ++i)

@@ -269,8 +269,7 @@ x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_d = tmem_slot;
-    pdl_wait();
-    pdl_trigger();
+    pdl_wait();                                         // no trigger: the next kernel's early blocks would crowd a few SMs (1 %)
 
     if (warp == 0) {
         if (lane == 0) {
