@@ -321,7 +321,7 @@ conv1_march_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
         Walk w;
         w.start(p, g);
         w.i = -1;                                         // forces the per-unit set-up at the first step
-        bool valid = false;
+        int rows = 0;                                     // output rows this thread stores from the unit's first on
         __half* dst0 = nullptr;
         int unit_now = -1;
         w.i = 0;
@@ -332,7 +332,7 @@ conv1_march_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                 w.unit(p);
                 const int q = w.tile * kTileCols + 31 * qq + lane;
                 const int e = q / pl.Ws, X = q - e * pl.Ws;
-                valid = lane < 31 && e < p.n && X < pl.W1;
+                rows = lane < 31 && e < p.n && X < pl.W1 ? pl.H1 - w.y_base : 0;
                 dst0 = p.out + ((size_t)e * pl.P1s + (X >> 1)) * 128 + (X & 1) * 32;
             }
             const int y = w.y_base + w.pos;
@@ -362,7 +362,7 @@ conv1_march_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                         fma2(a0, a1, inv, s_bias[c], s_bias[c + 1]);
                         pk[hh] = relu_pack_h2(a0, a1);
                     }
-                    if (valid && y < pl.H1)
+                    if (w.pos < rows)
                         asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                                      ::"l"(dst + j), "r"(pk[0]), "r"(pk[1]), "r"(pk[2]), "r"(pk[3]), "r"(pk[4]), "r"(pk[5]),
                                        "r"(pk[6]), "r"(pk[7]) : "memory");
@@ -390,7 +390,7 @@ conv1_march_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                         fma2(a0, a1, inv, s_bias[j + c], s_bias[j + c + 1]);
                         pk[hh] = relu_pack_h2(a0, a1);
                     }
-                    if (valid && y < pl.H1)
+                    if (w.pos < rows)
                         asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                                      ::"l"(dst + j), "r"(pk[0]), "r"(pk[1]), "r"(pk[2]), "r"(pk[3]), "r"(pk[4]), "r"(pk[5]),
                                        "r"(pk[6]), "r"(pk[7]) : "memory");
