@@ -626,7 +626,7 @@ def run_ours(args) -> None:
 
     other_configs = config_points(hts, torch, dev, peaks, s_act, l2) if rank == 0 else None
 
-    # ---- the learner's gradient (forward + backward on the fp32 path, CUDA cores, untuned) on one actor batch
+    # ---- the learner's gradient (forward + backward of an fp32 context) on one actor batch
     grad_pt = None
     if rank == 0:
         ctxg = hts.hts_policy_create(cfg.C, cfg.H, cfg.W, A, hts.HTS_DTYPE_FP32, N)
@@ -645,7 +645,7 @@ def run_ours(args) -> None:
         gms = float(np.median(g_ms[1:]))
         gflop = 3 * 2.0 * macs_per_env_step(cfg) * N / 1e9          # forward + data gradient + weight gradient
         grad_pt = {"n": N, "ms": gms, "samples_per_s": N / (gms * 1e-3), "tflops_fp32": gflop / gms,
-                   "arithmetic": "fp32 CUDA cores, fixed-order sums", "flops_counted": "3 x forward"}
+                   "arithmetic": "forward fp32 CUDA cores, backward bf16x3 tensor cores (fp32 accuracy), fixed-order sums", "flops_counted": "3 x forward"}
         del grads
 
     if rank != 0:

@@ -182,8 +182,8 @@ typedef struct {
  *   logp_old DEVICE f32 [n] or NULL; grads: twelve DEVICE f32 buffers, PyTorch layouts, overwritten.
  * Only HTS_DTYPE_FP32 contexts (the learner's master weights are fp32; a bf16 actor context is refreshed
  * from them through hts_delayed_update's bf16 output and hts_policy_load_weights): a bf16 context returns
- * HTS_ERR_UNSUPPORTED.  fp32 CUDA-core arithmetic, every sum in a fixed order; written for a reproducible
- * result, not tuned.  The first call on a context allocates the backward workspace (device memory, freed
+ * HTS_ERR_UNSUPPORTED.  The forward pass is hts_policy_step's own; the backward contractions run on the
+ * tensor cores at fp32 accuracy (each operand as three bf16 pieces), every sum in a fixed order.  The first call on a context allocates the backward workspace (device memory, freed
  * by hts_policy_destroy).  An action outside the range is not used as an index: that sample contributes
  * nothing and hts_last_async_error reports INVALID_ARG.
  * Errors: INVALID_ARG (NULL, n out of range, clip < 0, non-finite coefficient), UNSUPPORTED, ALLOC, CUDA.  */
