@@ -589,7 +589,7 @@ hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, 
     st = ref_forward(g, w, ws, obs, Indexing{}, t->status, n, prof, s, &planes);
     if (st != HTS_OK) return st;
     st = launch_heads(ws.h, 1, 0, nullptr, w.whead, w.bhead, g.A, nullptr, nullptr, 0, 0, n, Indexing{}, t->status, nullptr, t->logp, t->val,
-                      t->ent, t->logits, nullptr, s, actions);
+                      t->ent, t->logits, nullptr, s, actions, false);
     if (st != HTS_OK) return st;
     auto run = [&](X3TapParams p, size_t rows, bf16* dst, size_t dst_plane, const bf16* mask, int mask_pitch) {
         p.m_tiles = tiles_of(rows); p.n = n; p.dst = dst; p.dst_plane = dst_plane; p.mask = mask; p.mask_pitch = mask_pitch;

@@ -140,8 +140,8 @@ hts_status launch_heads(const float* h_partials, int num_splits, size_t split_st
                         const int32_t* env_ids, const int32_t* t_per_env, int32_t t,
                         uint64_t seed, int n, const Indexing& ix, int* status, int32_t* actions, float* logp,
                         float* values, float* entropy, float* logits, float* h_out, cudaStream_t s,
-                        const int32_t* given_actions = nullptr);
-// given_actions != nullptr: no sampling; row e reports log pi(given_actions[e] | s_e) (env_ids, t and seed are
+                        const int32_t* given_actions = nullptr, bool early = true);
+// early: a dependent launch may start before this one ends.  given_actions != nullptr: no sampling; row e reports log pi(given_actions[e] | s_e) (env_ids, t and seed are
 // not read, actions may be nullptr).  An action outside [0, A) sets kStatusBadAction and the row writes nothing.
 
 hts_status launch_uniforms(const int32_t* env_ids, const int32_t* t_per_env, int32_t t, uint64_t seed, int n,

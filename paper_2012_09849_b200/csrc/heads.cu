@@ -96,7 +96,7 @@ heads_kernel(const float* __restrict__ h_partials, int num_splits, size_t split_
              const int32_t* __restrict__ given,
              int32_t* __restrict__ actions, float* __restrict__ logp,
              float* __restrict__ values, float* __restrict__ entropy, float* __restrict__ logits_out,
-             float* __restrict__ h_out)
+             float* __restrict__ h_out, bool early)
 {
     extern __shared__ float4 s_w4[];                   // [(A+1)*512] head weights, staged once per block
     __shared__ float s_out[8][kMaxActions + 1];
@@ -112,7 +112,9 @@ heads_kernel(const float* __restrict__ h_partials, int num_splits, size_t split_
         if (fc_bias && threadIdx.x < kHidden / 4) s_fcb[threadIdx.x] = reinterpret_cast<const float4*>(fc_bias)[threadIdx.x];
     }
     pdl_wait();                                        // the head weights above are older than the previous kernel
-    pdl_trigger();
+    // the next step's first kernel may settle while this one runs: worth 0.3 - 2 us to the tensor-core chain, but blocks of
+    // an fp32 convolution would crowd the SMs that have room first (n = 48 football frames: 134 against 112 us per step)
+    if (early) pdl_trigger();
     __syncthreads();
     const float4* sw4 = s_w4;
     // rows are dealt block-first (row g goes to block g % gridDim.x), so a batch of fewer rows than warps on
@@ -221,7 +223,7 @@ hts_status launch_heads(const float* h_partials, int num_splits, size_t split_st
                         const int32_t* env_ids, const int32_t* t_per_env, int32_t t,
                         uint64_t seed, int n, const Indexing& ix, int* status, int32_t* actions, float* logp,
                         float* values, float* entropy, float* logits, float* h_out, cudaStream_t s,
-                        const int32_t* given_actions)
+                        const int32_t* given_actions, bool early)
 {
     if (num_splits < 1 || num_splits > kMaxSplits) return HTS_ERR_INVALID_ARG;
     const size_t smem = (size_t)(A + 1) * kHidden * sizeof(float);
@@ -248,7 +250,7 @@ hts_status launch_heads(const float* h_partials, int num_splits, size_t split_st
         if (blocks > n) blocks = n;
         HTS_CUDA(launch_pdl(kernel, dim3(blocks), dim3(256), smem, s, h_partials, num_splits, split_stride, fc_bias, whead,
                             bhead, A, env_ids, t_per_env, t, k0, k1, n, ix.slots, ix.pool, status, given_actions, actions,
-                            logp, values, entropy, logits, h_out));
+                            logp, values, entropy, logits, h_out, early));
         note_launch();
         return HTS_OK;
     };

@@ -130,7 +130,7 @@ hts_status run_step(hts_ctx* ctx, const uint8_t* obs, const Indexing& ix, const 
         if (st != HTS_OK) return st;
         ctx->prof.begin(K_HEADS, s);
         st = launch_heads(ctx->rws.h, 1, 0, nullptr, ctx->rw.whead, ctx->rw.bhead, g.A, env_ids, t_per_env, t,
-                          seed, n, ix, ctx->status, actions, logp, values, entropy, logits, nullptr, s, given_actions);
+                          seed, n, ix, ctx->status, actions, logp, values, entropy, logits, nullptr, s, given_actions, false);
     }
     if (st != HTS_OK) return st;
     ctx->prof.end(K_HEADS, s);

@@ -389,16 +389,16 @@ hts_status launch_conv(const ConvParams& p, cudaStream_t s)
 // over the lane number (halves first).  A warp owns TE rows x TO outputs and lane l runs chain l of all of them: both
 // operands are contiguous across the lanes, so neither needs a transposition, and one transposing reduction closes
 // the tree (at each level a lane keeps half of its values and gets its partner's share of them).
-// The block's rows of x and w go through a ring in shared memory, 64 columns at a time.  Bound: large batches by
+// The block's rows of x and w go through a ring in shared memory, COLS columns at a time.  Bound: large batches by
 // shared memory and the fp32 pipes (8 x 8 per warp: one byte per multiply-add, 128 of each per clock; 8 x 16 leaves too
 // few warps, 149 against 115 us at n = 1024), small ones by the latency of the weights: narrow tiles, deep ring.
-template <int TE, int TO, int WE, int WO, int STAGES>
+template <int TE, int TO, int WE, int WO, int STAGES, int COLS>
 __global__ void __launch_bounds__(32 * WE * WO)
 fc_chain_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ b,
                 float* __restrict__ h, int n, int F, bool w_vec)
 {
-    constexpr int NV = TE * TO, RX = TE * WE, RW = TO * WO, NT = 32 * WE * WO, UNITS = (RX + RW) * 16;   // 16-byte pieces of a stage
-    extern __shared__ __align__(16) float s_mem[];      // [STAGES][RX + RW][64]
+    constexpr int NV = TE * TO, RX = TE * WE, RW = TO * WO, NT = 32 * WE * WO, Q = COLS / 4, UNITS = (RX + RW) * Q;   // 16-byte pieces of a row, of a stage
+    extern __shared__ __align__(16) float s_mem[];      // [STAGES][RX + RW][COLS]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int we = warp % WE, wo = warp / WE;
     const int e0 = (blockIdx.y * WE + we) * TE, o0 = (blockIdx.x * WO + wo) * TO;
@@ -410,12 +410,13 @@ fc_chain_kernel(const float* __restrict__ x, const float* __restrict__ w, const 
 #pragma unroll
         for (int j = 0; j < TO / 2; ++j) acc[i][j] = 0;
     auto fetch = [&](int f, int st) {
-        float* dst = s_mem + st * (RX + RW) * 64;
+        float* dst = s_mem + st * (RX + RW) * COLS;
 #pragma unroll
         for (int a = 0; a < (UNITS + NT - 1) / NT; ++a) {
-            const int u = a * NT + threadIdx.x, r = u >> 4, q = (u & 15) * 4;
+            const int u = a * NT + threadIdx.x, r = u / Q, q = u % Q * 4;
             if (UNITS % NT && u >= UNITS) break;
-            const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + r * 64 + q);
+            if (COLS > 64 && f + q >= F) continue;
+            const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + r * COLS + q);
             if (r < RX) cp_async16(d, x + (size_t)min((int)(blockIdx.y * RX) + r, n - 1) * F + f + q);
             else {
                 const float* src = w + (size_t)(blockIdx.x * RW + r - RX) * F + f + q;
@@ -425,35 +426,39 @@ fc_chain_kernel(const float* __restrict__ x, const float* __restrict__ w, const 
             }
         }
     };
-    const int steps = F / 64;
+    const int steps = (F + COLS - 1) / COLS;             // F is a multiple of 64
 #pragma unroll
     for (int s = 0; s < STAGES - 1; ++s) {
-        if (s < steps) fetch(64 * s, s);
+        if (s < steps) fetch(COLS * s, s);
         cp_async_commit();
     }
     for (int s = 0; s < steps; ++s) {
         cp_async_wait<STAGES - 2>();
         __syncthreads();                                // stage s has landed for every thread; stage s - 1 is free
-        if (s + STAGES - 1 < steps) fetch(64 * (s + STAGES - 1), (s + STAGES - 1) % STAGES);
+        if (s + STAGES - 1 < steps) fetch(COLS * (s + STAGES - 1), (s + STAGES - 1) % STAGES);
         cp_async_commit();
-        const float* xr = s_mem + (s % STAGES) * (RX + RW) * 64 + we * TE * 64 + lane;
-        const float* wr = s_mem + (s % STAGES) * (RX + RW) * 64 + (RX + wo * TO) * 64 + lane;
-        float xv[2][TE], wv[2][TO];
+        const float* xr = s_mem + (s % STAGES) * (RX + RW) * COLS + we * TE * COLS + lane;
+        const float* wr = s_mem + (s % STAGES) * (RX + RW) * COLS + (RX + wo * TO) * COLS + lane;
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
+        for (int c = 0; c < COLS; c += 64) {
+            if (c > 0 && COLS * s + c >= F) break;
+            float xv[2][TE], wv[2][TO];
 #pragma unroll
-            for (int j = 0; j < TO; ++j) wv[k][j] = wr[64 * j + 32 * k];
+            for (int k = 0; k < 2; ++k) {
 #pragma unroll
-            for (int i = 0; i < TE; ++i) xv[k][i] = xr[64 * i + 32 * k];
-        }
+                for (int j = 0; j < TO; ++j) wv[k][j] = wr[COLS * j + c + 32 * k];
 #pragma unroll
-        for (int k = 0; k < 2; ++k)
-#pragma unroll
-            for (int i = 0; i < TE; ++i) {
-                const f32x2 xx = both(xv[k][i]);
-#pragma unroll
-                for (int j = 0; j < TO / 2; ++j) fma2(acc[i][j], xx, pair(wv[k][2 * j], wv[k][2 * j + 1]));
+                for (int i = 0; i < TE; ++i) xv[k][i] = xr[COLS * i + c + 32 * k];
             }
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int i = 0; i < TE; ++i) {
+                    const f32x2 xx = both(xv[k][i]);
+#pragma unroll
+                    for (int j = 0; j < TO / 2; ++j) fma2(acc[i][j], xx, pair(wv[k][2 * j], wv[k][2 * j + 1]));
+                }
+        }
     }
     float v[NV];
 #pragma unroll
@@ -483,11 +488,11 @@ fc_chain_kernel(const float* __restrict__ x, const float* __restrict__ w, const 
     }
 }
 
-template <int TE, int TO, int WE, int WO, int STAGES>
+template <int TE, int TO, int WE, int WO, int STAGES, int COLS>
 hts_status launch_fc_chain(const float* x, const float* w, const float* b, float* h, int n, int F, cudaStream_t s)
 {
-    constexpr int smem = STAGES * (TE * WE + TO * WO) * 256;
-    auto kernel = fc_chain_kernel<TE, TO, WE, WO, STAGES>;
+    constexpr int smem = STAGES * (TE * WE + TO * WO) * COLS * 4;
+    auto kernel = fc_chain_kernel<TE, TO, WE, WO, STAGES, COLS>;
     static bool set_by_device[kDeviceSlots] = {};
     bool& set = set_by_device[device_slot()];
     if (!set) {
@@ -502,8 +507,12 @@ hts_status launch_fc_chain(const float* x, const float* w, const float* b, float
 }
 hts_status launch_fc(const float* x, const float* w, const float* b, float* h, int n, int F, cudaStream_t s)
 {
-    if (n > 128) return launch_fc_chain<8, 8, 4, 2, 4>(x, w, b, h, n, F, s);
-    return launch_fc_chain<4, 4, 4, 1, 8>(x, w, b, h, n, F, s);
+    if (n > 128) return launch_fc_chain<8, 8, 4, 2, 4, 64>(x, w, b, h, n, F, s);
+    // 128 blocks per 16 rows.  The fewer of them an SM has, the more each must have in flight and the less often its warps
+    // may meet (64 columns, 8 stages before: n = 8 / 24 / 128: 45 / 57 / 147 us per step; now 41 / 53 / 144).
+    if (n <= 16) return launch_fc_chain<4, 4, 4, 1, 3, 512>(x, w, b, h, n, F, s);
+    if (n <= 32) return launch_fc_chain<4, 4, 4, 1, 2, 512>(x, w, b, h, n, F, s);
+    return launch_fc_chain<4, 4, 4, 1, 4, 128>(x, w, b, h, n, F, s);
 }
 
 }  // namespace
@@ -611,5 +620,5 @@ extern "C" hts_status hts_policy_step_noalloc(const hts_net_desc* d, const hts_w
     hts_status st = ref_forward(g, rw, ws, obs, Indexing{}, nullptr, n, off, s);
     if (st != HTS_OK) return st;
     return launch_heads(ws.h, 1, 0, nullptr, whead, bhead, g.A, env_ids, t_per_env, t, seed, n, Indexing{}, nullptr, actions,
-                        logp, values, entropy, logits_or_null, nullptr, s);
+                        logp, values, entropy, logits_or_null, nullptr, s, nullptr, false);
 }

@@ -12,8 +12,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("C,H,W,sizes", [
-    (4, 84, 84, (1, 15, 17, 96, 97, 384, 385, 700)),     # every tile of the convolutions and of the dense layer
-    (3, 36, 44, (1, 33, 400)),                           # channels not a multiple of four, a dense layer of 256 features
+    (4, 84, 84, (1, 15, 16, 17, 32, 33, 96, 97, 128, 129, 384, 385, 700)),     # every tile of the convolutions and of the dense layer
+    (3, 36, 44, (1, 20, 33, 400)),                       # channels not a multiple of four, a dense layer of 256 features
     (16, 72, 96, (2, 130))])
 def test_rows_do_not_depend_on_the_tile(C, H, W, sizes):
     cfg = dataclasses.replace(wl.CONFIGS[1], C=C, H=H, W=W)
