@@ -109,8 +109,9 @@ conv_tile_kernel(const ConvParams p)
     const TIn* src[NPX];
 #pragma unroll
     for (int q = 0; q < NPX; ++q) {
-        int px = blockIdx.x * PX + (NPX > 1 ? tid + NT * q : tid % PX);
-        px = px < total ? px : total - 1;
+        // past the end of the batch: pixels from its start.  The last one for all would make a warp copy one word to 32
+        // places, which takes 32 passes (conv3, n = 72: 40 us, 26 with distinct words).
+        const int px = (blockIdx.x * PX + (NPX > 1 ? tid + NT * q : tid % PX)) % total;
         const int e = px / P, r = px - e * P, i = r / p.Wo, j = r - i * p.Wo;
         src[q] = static_cast<const TIn*>(p.x) + frame_of(p, e) * p.C * p.H * p.W + (size_t)(i * p.s) * p.W + j * p.s;
     }
@@ -224,9 +225,9 @@ conv_tile_kernel(const ConvParams p)
 }
 
 // The same sums for batches too small to fill the device with tiles: 16 pixels x 32 channels per block of 128 threads,
-// 2 x 2 per thread, K in groups of 64 that are all requested at once (up to kSmallRing of them) and multiplied as they
+// 2 x 2 per thread, K in groups of 64, up to twelve of them requested at once and multiplied as they
 // arrive.  Inputs and weights stay in K order, four of it per load.  Bound: latency, about one warp per scheduler.
-constexpr int kSmallK = 64, kSmallPitch = kSmallK + 4, kSmallPx = 16, kSmallOc = 32, kSmallRing = 12;
+constexpr int kSmallK = 64, kSmallPitch = kSmallK + 4, kSmallPx = 16, kSmallOc = 32;
 template <typename TIn>
 __global__ void __launch_bounds__(128)
 conv_small_kernel(const ConvParams p, int ring)
@@ -337,7 +338,11 @@ conv_small_kernel(const ConvParams p, int ring)
 template <typename TIn>
 hts_status launch_conv_small(const ConvParams& p, cudaStream_t s)
 {
-    const int groups = p.C * p.k * p.k / kSmallK, ring = groups < kSmallRing ? groups : kSmallRing;
+    const size_t px = (size_t)p.n * p.Ho * p.Wo, sms = (size_t)device_sm_count(device_slot());
+    const size_t blocks = (px + kSmallPx - 1) / kSmallPx * (p.O / kSmallOc);
+    // as many groups in flight as let all the blocks be resident at once (conv2, n = 32: 31 us where two blocks fit, 22)
+    const int most = blocks <= sms ? 12 : blocks <= 2 * sms ? 8 : blocks <= 3 * sms ? 5 : blocks <= 4 * sms ? 4 : 3;
+    const int groups = p.C * p.k * p.k / kSmallK, ring = groups < most ? groups : most;
     const int smem = ring * (kSmallPx + kSmallOc) * kSmallPitch * (int)sizeof(float);
     static int smem_set_by_device[kDeviceSlots] = {};
     int& smem_set = smem_set_by_device[device_slot()];
@@ -346,7 +351,6 @@ hts_status launch_conv_small(const ConvParams& p, cudaStream_t s)
         HTS_CUDA(cudaFuncSetAttribute(conv_small_kernel<TIn>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
         smem_set = smem;
     }
-    const size_t px = (size_t)p.n * p.Ho * p.Wo;
     HTS_CUDA(launch_pdl(conv_small_kernel<TIn>, dim3((unsigned)((px + kSmallPx - 1) / kSmallPx), (unsigned)(p.O / kSmallOc)), dim3(128),
                         (size_t)smem, s, p, ring));
     note_launch();
@@ -373,16 +377,19 @@ hts_status launch_conv_tile(const ConvParams& p, cudaStream_t s)
     return HTS_OK;
 }
 
-// 128 x 64 (256 x 32) tiles from two per SM on: they load least per multiply-add.  Below, 64 x 32 tiles of four warps
-// while every second SM gets one (n = 256: 229 us per step, 266 with two warps of 4 x 8 per tile), else the latency form.
+// A form takes a time that steps with the blocks of the SM that has most.  conv2 (us at 1, 2, 3 ... per SM): latency form
+// 15, 19, 23, 27; 64 x 32 tiles 25, 35, 48, 62, 74, 87, 99; 128 x 64 (256 x 32) tiles 50, 80, 109.  So one large tile
+// costs as much as 2.5 small ones and 0.7 more for its start; the latency form pays up to three blocks per SM (two where
+// it converts frames, 17 against 15).
 template <typename TIn>
 hts_status launch_conv(const ConvParams& p, cudaStream_t s)
 {
     const size_t px = (size_t)p.n * p.Ho * p.Wo, sms = (size_t)device_sm_count(device_slot());
-    if (p.O == 64 && px >= 128 * 2 * sms) return launch_conv_tile<TIn, 8, 8, 2, 2, 16, 4>(p, s);
-    if (p.O == 32 && px >= 256 * 2 * sms) return launch_conv_tile<TIn, 8, 8, 4, 1, 16, 4>(p, s);
-    if (px * p.O >= 64 * 16 * sms) return launch_conv_tile<TIn, 4, 4, 2, 2, 32, 5>(p, s);
-    return launch_conv_small<TIn>(p, s);
+    auto per_sm = [&](size_t tile_px, size_t tile_oc) { return ((px + tile_px - 1) / tile_px * (p.O / tile_oc) + sms - 1) / sms; };
+    const size_t small = per_sm(kSmallPx, kSmallOc), medium = per_sm(64, 32), large = p.O == 64 ? per_sm(128, 64) : per_sm(256, 32);
+    if (small <= (std::is_same<TIn, uint8_t>::value ? 2 : 3)) return launch_conv_small<TIn>(p, s);
+    if (2 * medium <= 5 * large + 1) return launch_conv_tile<TIn, 4, 4, 2, 2, 32, 5>(p, s);
+    return p.O == 64 ? launch_conv_tile<TIn, 8, 8, 2, 2, 16, 4>(p, s) : launch_conv_tile<TIn, 8, 8, 4, 1, 16, 4>(p, s);
 }
 
 // h[e,o] = relu(b[o] + sum over lanes l of (chain of f = l, l+32, l+64, ...)), the 32 chains added as a binary tree
