@@ -514,9 +514,10 @@ hts_status launch_fc_chain(const float* x, const float* w, const float* b, float
 }
 hts_status launch_fc(const float* x, const float* w, const float* b, float* h, int n, int F, cudaStream_t s)
 {
-    if (n > 128) return launch_fc_chain<8, 8, 4, 2, 4, 64>(x, w, b, h, n, F, s);
+    // one wide block per SM (n <= 128: 25 us) takes as long as five narrow ones (n = 80; n = 128 with eight: 34)
+    if (n > 80) return launch_fc_chain<8, 8, 4, 2, 4, 64>(x, w, b, h, n, F, s);
     // 128 blocks per 16 rows.  The fewer of them an SM has, the more each must have in flight and the less often its warps
-    // may meet (64 columns, 8 stages before: n = 8 / 24 / 128: 45 / 57 / 147 us per step; now 41 / 53 / 144).
+    // may meet (64 columns, 8 stages before: n = 8 / 24 / 80: 45 / 57 / 125 us per step; now 41 / 53 / 123).
     if (n <= 16) return launch_fc_chain<4, 4, 4, 1, 3, 512>(x, w, b, h, n, F, s);
     if (n <= 32) return launch_fc_chain<4, 4, 4, 1, 2, 512>(x, w, b, h, n, F, s);
     return launch_fc_chain<4, 4, 4, 1, 4, 128>(x, w, b, h, n, F, s);

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("C,H,W,sizes", [
-    (4, 84, 84, (1, 15, 16, 17, 32, 33, 72, 80, 128, 129, 200, 384, 700)),     # every tile of the convolutions and of the dense layer
+    (4, 84, 84, (1, 15, 16, 17, 32, 33, 72, 80, 81, 128, 129, 200, 384, 700)),     # every tile of the convolutions and of the dense layer
     (3, 36, 44, (1, 20, 33, 400)),                       # channels not a multiple of four, a dense layer of 256 features
     (16, 72, 96, (2, 130))])
 def test_rows_do_not_depend_on_the_tile(C, H, W, sizes):
