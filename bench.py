@@ -446,7 +446,7 @@ def run_ours(args) -> None:
         b.record(s_gae); torch.cuda.synchronize()
         t_ms.append(a.elapsed_time(b))
     ppo_wide_ms = float(np.median(t_ms[3:]))
-    ppo_wide_gbs = 32 * T * Nw / (ppo_wide_ms * 1e-3) / 1e9
+    ppo_wide_gbs = 28 * T * Nw / (ppo_wide_ms * 1e-3) / 1e9
     del x1, x2
     # the learner's parameter update (Eq. 5 with RMSProp scaling) over a parameter vector of the widened size
     upd_ms = []
@@ -696,7 +696,7 @@ def run_ours(args) -> None:
                                    "frac_of_hbm": terms_wide_gbs / peaks["hbm_gbs"]},
                           "ppo_wide": {"elems": T * Nw, "ms": ppo_wide_ms, "gbs": ppo_wide_gbs,
                                        "frac_of_hbm": ppo_wide_gbs / peaks["hbm_gbs"],
-                                       "bytes_per_elem": "24 (six arrays) + 2 x 4 (advantage mean and variance passes)"}},
+                                       "bytes_per_elem": "24 (six arrays) + 4 (advantage statistics)"}},
         "learner_gradient": grad_pt,
         "delayed_update": {"elems": T * Nw, "ms": upd_wide_ms, "gbs": upd_gbs, "frac_of_hbm": upd_gbs / peaks["hbm_gbs"]},
         "actor_step_us": 1e3 * ms / (args.steps * T),
