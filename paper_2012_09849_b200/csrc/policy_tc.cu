@@ -498,6 +498,7 @@ constexpr int kAbsmaxBlocks = 4 * 148;
 __global__ void __launch_bounds__(256) absmax_kernel(const LoadTcParams p)
 {
     __shared__ bool s_last;
+    __shared__ unsigned s_max[8][L_COUNT];
     const int tid = blockIdx.x * 256 + threadIdx.x, threads = gridDim.x * 256;
 #pragma unroll
     for (int l = 0; l < L_COUNT; ++l) {
@@ -514,9 +515,16 @@ __global__ void __launch_bounds__(256) absmax_kernel(const LoadTcParams p)
         }
         for (int i = done + tid; i < p.n[l]; i += threads) take(reinterpret_cast<const uint16_t*>(p.w[l])[i]);
         m = __reduce_max_sync(0xffffffffu, m);
-        if ((threadIdx.x & 31) == 0 && m) atomicMax(p.absmax + l, m << 16);
+        if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5][l] = m;
     }
-    __threadfence();
+    __syncthreads();
+    if (threadIdx.x < L_COUNT) {                        // one atomic per block and layer: they all meet at one address
+        unsigned m = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) m = max(m, s_max[w][threadIdx.x]);
+        if (m) atomicMax(p.absmax + threadIdx.x, m << 16);
+        __threadfence();
+    }
     __syncthreads();
     if (threadIdx.x == 0) s_last = atomicAdd(p.absmax + L_COUNT, 1u) == gridDim.x - 1;
     __syncthreads();
@@ -542,7 +550,7 @@ __device__ __forceinline__ __half scaled_h(__nv_bfloat16 w, float s) { return __
 // Blocks 0..511 take one row of the dense layer each and turn it through shared memory (rows of up to 16384 columns;
 // wider ones are read with a stride); the rest one element per thread.
 constexpr int kPackRow = 16384;
-__global__ void __launch_bounds__(256) pack_kernel(const LoadTcParams p)
+__device__ __forceinline__ void pack_share(const LoadTcParams& p)
 {
     __shared__ __nv_bfloat16 s_row[kPackRow];
     if (blockIdx.x < 512) {
@@ -588,6 +596,11 @@ __global__ void __launch_bounds__(256) pack_kernel(const LoadTcParams p)
         }
         i -= p.fn[k];
     }
+}
+__global__ void __launch_bounds__(256) pack_kernel(const LoadTcParams p)
+{
+    pack_share(p);
+    __threadfence();        // the next kernel may load its filter as soon as the last block has left
 }
 
 // ---- parity taps: internal layouts -> fp32 NCHW ----------------------------------------------------
