@@ -480,7 +480,8 @@ fc_ranges_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 // ---- weight scaling and packing ---------------------------------------------------------------
 // Two launches: the largest magnitude of each layer (the last block to finish turns them into scales), then every
 // layer scaled, converted and laid out.  They follow each parameter update, so launches count: 18 separate ones took
-// 125 us (47 of them in a 64-block pass over the dense layer).
+// 125 us (47 of them in a 64-block pass over the dense layer); two are 14, and 9.4 since the second reads its rows while
+// the first runs.
 struct LoadTcParams {
     const __nv_bfloat16* w[L_COUNT];    // conv1, conv2, conv3, dense
     int n[L_COUNT];
@@ -500,6 +501,8 @@ __global__ void __launch_bounds__(256) absmax_kernel(const LoadTcParams p)
     __shared__ bool s_last;
     __shared__ unsigned s_max[8][L_COUNT];
     const int tid = blockIdx.x * 256 + threadIdx.x, threads = gridDim.x * 256;
+    pdl_wait();
+    pdl_trigger();
 #pragma unroll
     for (int l = 0; l < L_COUNT; ++l) {
         unsigned m = 0;                                 // finite magnitudes order like their bits
@@ -556,16 +559,18 @@ __device__ __forceinline__ void pack_share(const LoadTcParams& p)
     if (blockIdx.x < 512) {
         const int o = blockIdx.x, F = 64 * p.P3;
         const __nv_bfloat16* src = p.w[L_FC] + (size_t)o * F;
-        const float s = p.scale[L_FC];
-        if (F <= kPackRow) {
+        if (F <= kPackRow) {                            // the caller's weights are older than the pass over them
             for (int i = threadIdx.x; i < F; i += 256) s_row[i] = src[i];
             __syncthreads();
             src = s_row;
         }
+        pdl_wait();
+        const float s = p.scale[L_FC];
         __half* dst = p.wp[L_FC] + (size_t)o * F;
         for (int k = threadIdx.x; k < F; k += 256) dst[k] = scaled_h(src[(k & 63) * p.P3 + (k >> 6)], s);
         return;
     }
+    pdl_wait();
     int i = (blockIdx.x - 512) * 256 + threadIdx.x;
     const int K = 16 * p.C;
     if (i < 128 * K) {
@@ -760,10 +765,10 @@ hts_status tc_load_weights(TcState* t, const hts_weights& w, cudaStream_t s)
                          {w.v_w, t->whead + (size_t)g.A * 512, 512}, {w.pi_b, t->bhead, g.A}, {w.v_b, t->bhead + g.A, 1}};
     int rest = 128 * 16 * g.C + 64 * 512 + 64 * 576;
     for (int k = 0; k < 8; ++k) { p.f[k] = bf(items[k].p); p.fdst[k] = items[k].q; p.fn[k] = items[k].n; rest += items[k].n; }
-    absmax_kernel<<<kAbsmaxBlocks, 256, 0, s>>>(p);
-    HTS_LAUNCH_CHECK("absmax");
-    pack_kernel<<<512 + nblk(rest, 256), 256, 0, s>>>(p);
-    HTS_LAUNCH_CHECK("pack");
+    HTS_CUDA(launch_pdl(absmax_kernel, dim3(kAbsmaxBlocks), dim3(256), 0, s, p));
+    note_launch();
+    HTS_CUDA(launch_pdl(pack_kernel, dim3(512 + nblk(rest, 256)), dim3(256), 0, s, p));
+    note_launch();
     return HTS_OK;
 }
 
