@@ -1,15 +1,18 @@
 /* CPython entry points of the calls a training loop makes: argument marshalling only, in C because the loop's small
  * calls are bound by it (an advantage scan of 5 us on the device took 10 us to enqueue through ctypes: 3 for the
  * current stream, 2.5 for pointers and conversions, 1.5 for the foreign call).  Every function takes the arguments of
- * the Python function of the same name positionally, the stream last; pointers are torch tensors, C-contiguous
- * buffers (numpy), integers or None.  A non-zero status raises the exception type handed to init(). */
+ * the Python function of the same name positionally, the stream last; pointers are torch tensors, C-contiguous numpy
+ * arrays, integers or None, and contexts integers, c_void_p or None: nothing else that has an address of its own (a
+ * numpy scalar, bytes) is taken for one.  A non-zero status raises the exception type handed to init(). */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include "hts.h"
 
 static PyObject *g_error;                              /* HtsError(status, what) */
 static PyObject *g_raw_stream, *g_get_device;          /* torch._C._cuda_getCurrentRawStream, _cuda_getDevice */
-static PyObject *s_data_ptr, *s_is_contiguous, *s_cuda_stream;
+static PyTypeObject *g_ndarray, *g_void_p;             /* numpy.ndarray, ctypes.c_void_p */
+static PyObject *g_argument_error;                     /* ctypes.ArgumentError */
+static PyObject *s_data_ptr, *s_is_contiguous, *s_cuda_stream, *s_value;
 static PyObject *s_weights[12];
 static const char *const kWeights[12] = {"conv1_w", "conv1_b", "conv2_w", "conv2_b", "conv3_w", "conv3_b",
                                          "fc_w", "fc_b", "pi_w", "pi_b", "v_w", "v_b"};
@@ -21,15 +24,20 @@ static int not_contiguous(void)
     return 0;
 }
 
+static int int_ptr(PyObject *l, void **out)            /* takes the reference */
+{
+    if (!l) return 0;
+    *out = PyLong_AsVoidPtr(l);
+    Py_DECREF(l);
+    return !PyErr_Occurred();
+}
+
 /* address of a tensor, array, integer or None; 0 with an exception set on failure */
 static int to_ptr(PyObject *x, void **out)
 {
     if (x == Py_None) { *out = NULL; return 1; }
-    if (PyLong_Check(x)) {
-        *out = PyLong_AsVoidPtr(x);
-        return !PyErr_Occurred();
-    }
-    if (PyObject_CheckBuffer(x)) {
+    if (PyLong_Check(x)) return int_ptr(Py_NewRef(x), out);
+    if (PyObject_TypeCheck(x, g_ndarray)) {
         Py_buffer b;
         if (PyObject_GetBuffer(x, &b, PyBUF_C_CONTIGUOUS) != 0) return not_contiguous();
         *out = b.buf;
@@ -41,11 +49,23 @@ static int to_ptr(PyObject *x, void **out)
     const int ok = PyObject_IsTrue(c);
     Py_DECREF(c);
     if (ok <= 0) return ok < 0 ? 0 : not_contiguous();
-    PyObject *p = PyObject_CallMethodNoArgs(x, s_data_ptr);
-    if (!p) return 0;
-    *out = PyLong_AsVoidPtr(p);
-    Py_DECREF(p);
-    return !PyErr_Occurred();
+    return int_ptr(PyObject_CallMethodNoArgs(x, s_data_ptr), out);
+}
+
+/* a context: what hts_policy_create returned */
+static int to_ctx(PyObject *x, void **out)
+{
+    if (x == Py_None) { *out = NULL; return 1; }
+    if (PyLong_Check(x)) return int_ptr(Py_NewRef(x), out);
+    if (PyObject_TypeCheck(x, g_void_p)) {
+        PyObject *v = PyObject_GetAttr(x, s_value);
+        if (v != Py_None) return int_ptr(v, out);
+        Py_DECREF(v);
+        *out = NULL;
+        return 1;
+    }
+    PyErr_SetString(g_argument_error, "argument 1: a context is an integer, c_void_p or None");
+    return 0;
 }
 
 static int to_u64(PyObject *x, uint64_t *out)          /* int(x), wrapped to 64 bits */
@@ -66,9 +86,11 @@ static int to_i32(PyObject *x, int32_t *out)
 static int to_i64(PyObject *x, int64_t *out) { return to_u64(x, (uint64_t *)out); }
 static int to_f32(PyObject *x, float *out)
 {
-    const double v = PyFloat_AsDouble(x);
-    *out = (float)v;
-    return !(v == -1.0 && PyErr_Occurred());
+    PyObject *f = PyFloat_Check(x) ? Py_NewRef(x) : PyNumber_Float(x);       /* float(x) */
+    if (!f) return 0;
+    *out = (float)PyFloat_AS_DOUBLE(f);
+    Py_DECREF(f);
+    return 1;
 }
 
 /* None: torch's current stream; else an integer handle or an object with .cuda_stream */
@@ -122,6 +144,7 @@ static PyObject *done(hts_status st, const char *what)
 #define ARGS(count) \
     if (nargs != (count)) { PyErr_SetString(PyExc_TypeError, "wrong number of arguments"); return NULL; }
 #define PTR(name, i) void *name; if (!to_ptr(a[i], &name)) return NULL
+#define CTX() void *ctx; if (!to_ctx(a[0], &ctx)) return NULL
 #define I32(name, i) int32_t name; if (!to_i32(a[i], &name)) return NULL
 #define I64(name, i) int64_t name; if (!to_i64(a[i], &name)) return NULL
 #define U64(name, i) uint64_t name; if (!to_u64(a[i], &name)) return NULL
@@ -134,7 +157,7 @@ static PyObject *done(hts_status st, const char *what)
 static PyObject *step(PyObject *const *a, Py_ssize_t nargs, int host)
 {
     ARGS(13);
-    PTR(ctx, 0); PTR(obs, 1); PTR(ids, 2); PTR(tpe, 3); I32(t, 4); U64(seed, 5); I32(n, 6);
+    CTX(); PTR(obs, 1); PTR(ids, 2); PTR(tpe, 3); I32(t, 4); U64(seed, 5); I32(n, 6);
     PTR(act, 7); PTR(logp, 8); PTR(val, 9); PTR(ent, 10); PTR(logits, 11); STREAM(12);
     CALL((host ? hts_policy_step_host : hts_policy_step)(ctx, obs, ids, tpe, t, seed, n, act, logp, val, ent, logits, stream),
          host ? "hts_policy_step_host" : "hts_policy_step");
@@ -145,7 +168,7 @@ FN(policy_step_indexed)
 {
     (void)self;
     ARGS(14);
-    PTR(ctx, 0); PTR(buf, 1); I32(pool, 2); PTR(slots, 3); PTR(ids, 4); PTR(tpe, 5); I32(t, 6); U64(seed, 7); I32(n, 8);
+    CTX(); PTR(buf, 1); I32(pool, 2); PTR(slots, 3); PTR(ids, 4); PTR(tpe, 5); I32(t, 6); U64(seed, 7); I32(n, 8);
     PTR(act, 9); PTR(logp, 10); PTR(val, 11); PTR(ent, 12); STREAM(13);
     CALL(hts_policy_step_indexed(ctx, buf, pool, slots, ids, tpe, t, seed, n, act, logp, val, ent, stream), "hts_policy_step_indexed");
 }
@@ -153,7 +176,7 @@ FN(policy_evaluate)
 {
     (void)self;
     ARGS(9);
-    PTR(ctx, 0); PTR(obs, 1); PTR(act, 2); I32(n, 3); PTR(logp, 4); PTR(val, 5); PTR(ent, 6); PTR(logits, 7); STREAM(8);
+    CTX(); PTR(obs, 1); PTR(act, 2); I32(n, 3); PTR(logp, 4); PTR(val, 5); PTR(ent, 6); PTR(logits, 7); STREAM(8);
     CALL(hts_policy_evaluate(ctx, obs, act, n, logp, val, ent, logits, stream), "hts_policy_evaluate");
 }
 FN(policy_gradient)
@@ -161,7 +184,7 @@ FN(policy_gradient)
     (void)self;
     ARGS(12);
     hts_grads g;
-    PTR(ctx, 0); PTR(obs, 1); PTR(act, 2); PTR(adv, 3); PTR(ret, 4); PTR(old, 5); F32(vc, 6); F32(ec, 7); F32(clip, 8); I32(n, 9);
+    CTX(); PTR(obs, 1); PTR(act, 2); PTR(adv, 3); PTR(ret, 4); PTR(old, 5); F32(vc, 6); F32(ec, 7); F32(clip, 8); I32(n, 9);
     if (!weights_of(a[10], (void **)&g)) return NULL;
     STREAM(11);
     CALL(hts_policy_gradient(ctx, obs, act, adv, ret, old, vc, ec, clip, n, &g, stream), "hts_policy_gradient");
@@ -171,7 +194,7 @@ FN(policy_load_weights)
     (void)self;
     ARGS(3);
     hts_weights w;
-    PTR(ctx, 0);
+    CTX();
     if (!weights_of(a[1], (void **)&w)) return NULL;
     STREAM(2);
     CALL(hts_policy_load_weights(ctx, &w, stream), "hts_policy_load_weights");
@@ -234,6 +257,14 @@ PyMODINIT_FUNC PyInit__native(void)
     s_data_ptr = PyUnicode_InternFromString("data_ptr");
     s_is_contiguous = PyUnicode_InternFromString("is_contiguous");
     s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
+    s_value = PyUnicode_InternFromString("value");
     for (int i = 0; i < 12; ++i) s_weights[i] = PyUnicode_InternFromString(kWeights[i]);
+    PyObject *np = PyImport_ImportModule("numpy"), *ct = np ? PyImport_ImportModule("ctypes") : NULL;
+    g_ndarray = np ? (PyTypeObject *)PyObject_GetAttrString(np, "ndarray") : NULL;
+    g_void_p = ct ? (PyTypeObject *)PyObject_GetAttrString(ct, "c_void_p") : NULL;
+    g_argument_error = ct ? PyObject_GetAttrString(ct, "ArgumentError") : NULL;
+    Py_XDECREF(np); Py_XDECREF(ct);
+    if (!g_ndarray || !g_void_p || !g_argument_error) return NULL;
+    g_error = Py_NewRef(PyExc_RuntimeError);           /* until init() */
     return PyModule_Create(&kModule);
 }
