@@ -168,7 +168,7 @@ conv1_march_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_d = tmem_slot, tmem_a = tmem_slot + NACC * 64;   // accumulators of 64 columns, then the ring
-    if (threadIdx.x == 0) {                                   // the filter does not depend on the previous kernel
+    if (threadIdx.x == 0) {                                   // not the previous kernel's: see `dependent`
         mbar_arrive_expect_tx(&w_bar, (uint32_t)w_bytes);
         for (int dy = 0; dy < 2; ++dy)
             for (int g = 0; g < CG; ++g) tma_load_2d(sm + (dy * CG + g) * kChunkBytes, &tmW, g * 64, dy * 64, &w_bar);
@@ -425,7 +425,7 @@ int choose_rows(int tiles, int H1, int grid)
 
 template <int CG, int WC>
 hts_status launch_variant(const CUtensorMap& weight_map, const CUtensorMap& frame_map, const Conv1Params& p, int grid,
-                          int smem_bytes, cudaStream_t s)
+                          int smem_bytes, bool dependent, cudaStream_t s)
 {
     static int smem_set_by_device[kDeviceSlots] = {};
     int& smem_set = smem_set_by_device[device_slot()];
@@ -436,7 +436,7 @@ hts_status launch_variant(const CUtensorMap& weight_map, const CUtensorMap& fram
         HTS_CUDA(cudaFuncSetAttribute(conv1_march_kernel<CG, WC>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
         smem_set = smem_bytes;
     }
-    HTS_CUDA(launch_pdl(conv1_march_kernel<CG, WC>, dim3(grid), dim3(threads_of<CG>()), (size_t)smem_bytes, s, weight_map, frame_map, p));
+    HTS_CUDA(launch_chained(dependent, conv1_march_kernel<CG, WC>, dim3(grid), dim3(threads_of<CG>()), (size_t)smem_bytes, s, weight_map, frame_map, p));
     note_launch();
     return HTS_OK;
 }
@@ -471,7 +471,7 @@ bool conv1_plan(const Geometry& g, Conv1Plan* pl)
 
 hts_status conv1_launch(const Conv1Plan& pl, const CUtensorMap& weight_map, Conv1MapCache& maps, const uint8_t* obs,
                         const Indexing& ix, int n, const float* bias, const float* inv_scale, __half* out, int* status,
-                        cudaStream_t s)
+                        bool dependent, cudaStream_t s)
 {
     const int sm_count = device_sm_count(device_slot());
     const long cols = (long)n * pl.Ws;
@@ -501,12 +501,12 @@ hts_status conv1_launch(const Conv1Plan& pl, const CUtensorMap& weight_map, Conv
     const int grid = units < max_grid ? (int)units : max_grid;
     const CUtensorMap& fm = maps.map[slot];
     if (pl.CG == 1) {
-        if (pl.W == 84) return launch_variant<1, 84>(weight_map, fm, p, grid, pl.smem_bytes, s);
-        return launch_variant<1, 0>(weight_map, fm, p, grid, pl.smem_bytes, s);
+        if (pl.W == 84) return launch_variant<1, 84>(weight_map, fm, p, grid, pl.smem_bytes, dependent, s);
+        return launch_variant<1, 0>(weight_map, fm, p, grid, pl.smem_bytes, dependent, s);
     }
-    if (pl.CG == 2) return launch_variant<2, 0>(weight_map, fm, p, grid, pl.smem_bytes, s);
-    if (pl.W == 96) return launch_variant<4, 96>(weight_map, fm, p, grid, pl.smem_bytes, s);
-    return launch_variant<4, 0>(weight_map, fm, p, grid, pl.smem_bytes, s);
+    if (pl.CG == 2) return launch_variant<2, 0>(weight_map, fm, p, grid, pl.smem_bytes, dependent, s);
+    if (pl.W == 96) return launch_variant<4, 96>(weight_map, fm, p, grid, pl.smem_bytes, dependent, s);
+    return launch_variant<4, 0>(weight_map, fm, p, grid, pl.smem_bytes, dependent, s);
 }
 
 }  // namespace hts

@@ -112,7 +112,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tm = tmem_slot;
-    if (threadIdx.x == 0) {                              // the filters do not depend on the previous kernel
+    if (threadIdx.x == 0) {                              // not the previous kernel's: see `dependent`
         mbar_arrive_expect_tx(&w_bar[0], kW1Bytes);
         for (int g = 0; g < 2; ++g) tma_load_2d(sm + g * 8192, &tmW1, 0, g * 64, &w_bar[0]);
         mbar_arrive_expect_tx(&w_bar[1], kW2Bytes);
@@ -339,7 +339,8 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
 }
 
 template <int WC>
-hts_status launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const ConvStackParams& p, int smem, int grid, cudaStream_t s)
+hts_status launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const ConvStackParams& p, int smem, int grid,
+                  bool dependent, cudaStream_t s)
 {
     static int smem_set_by_device[kDeviceSlots] = {};
     int& smem_set = smem_set_by_device[device_slot()];
@@ -348,7 +349,7 @@ hts_status launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMa
         HTS_CUDA(cudaFuncSetAttribute(conv_stack_kernel<WC>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
         smem_set = smem;
     }
-    HTS_CUDA(launch_pdl(conv_stack_kernel<WC>, dim3(grid), dim3(kStackThreads), (size_t)smem, s, w1, w2, w3, p));
+    HTS_CUDA(launch_chained(dependent, conv_stack_kernel<WC>, dim3(grid), dim3(kStackThreads), (size_t)smem, s, w1, w2, w3, p));
     note_launch();
     return HTS_OK;
 }
@@ -375,10 +376,11 @@ bool conv_stack_plan(const Geometry& g, ConvStackParams* p)
     return stack_smem(*p) <= 226 * 1024;
 }
 
-hts_status conv_stack_launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const ConvStackParams& p, cudaStream_t s)
+hts_status conv_stack_launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const ConvStackParams& p,
+                             bool dependent, cudaStream_t s)
 {
     const int sms = device_sm_count(device_slot()), grid = p.n < sms ? p.n : sms, smem = stack_smem(p);
-    return p.W == 84 ? launch<84>(w1, w2, w3, p, smem, grid, s) : launch<0>(w1, w2, w3, p, smem, grid, s);
+    return p.W == 84 ? launch<84>(w1, w2, w3, p, smem, grid, dependent, s) : launch<0>(w1, w2, w3, p, smem, grid, dependent, s);
 }
 
 }  // namespace hts

@@ -27,6 +27,8 @@ bool conv_stack_plan(const Geometry& g, ConvStackParams* p);
 // Batches up to this many environments per SM are faster here than in a kernel per layer.
 constexpr int kStackEnvs = 6;
 // Weight maps: the packed filters of conv1 [128][64], conv2 [64][512] and conv3 [64][576], box 64 x 64.
-hts_status conv_stack_launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const ConvStackParams& p, cudaStream_t s);
+// dependent: as in conv1_launch.
+hts_status conv_stack_launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const ConvStackParams& p,
+                             bool dependent, cudaStream_t s);
 
 }  // namespace hts

@@ -553,7 +553,7 @@ __device__ __forceinline__ __half scaled_h(__nv_bfloat16 w, float s) { return __
 // Blocks 0..511 take one row of the dense layer each and turn it through shared memory (rows of up to 16384 columns;
 // wider ones are read with a stride); the rest one element per thread.
 constexpr int kPackRow = 16384;
-__device__ __forceinline__ void pack_share(const LoadTcParams& p)
+__global__ void __launch_bounds__(256) pack_kernel(const LoadTcParams p)
 {
     __shared__ __nv_bfloat16 s_row[kPackRow];
     if (blockIdx.x < 512) {
@@ -601,11 +601,6 @@ __device__ __forceinline__ void pack_share(const LoadTcParams& p)
         }
         i -= p.fn[k];
     }
-}
-__global__ void __launch_bounds__(256) pack_kernel(const LoadTcParams p)
-{
-    pack_share(p);
-    __threadfence();        // the next kernel may load its filter as soon as the last block has left
 }
 
 // ---- parity taps: internal layouts -> fp32 NCHW ----------------------------------------------------
@@ -665,6 +660,8 @@ struct TcState {
     int H1s, W1s, P1s;          // space-to-depth(2) grid of the conv1 output
     int P2, P3;
     int splits, cps;            // FC split-K
+    bool fresh = false;         // no step has been enqueued since the weights were packed
+    unsigned long long fresh_capture = 0;   // the stream capture that packing belongs to, 0 = none
     bool h_final = false;       // the last forward pass wrote the finished hidden layer (large-batch FC), not partials
     // packed weights
     Conv1Plan pl1;
@@ -748,6 +745,28 @@ hts_status tc_create(const Geometry& g, int max_batch, int* status, TcState** ou
 
 void tc_destroy(TcState* t) { delete t; }
 
+namespace {
+
+unsigned long long capture_of(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(s, &st, &id) != cudaSuccess) { cudaGetLastError(); return 0; }
+    return st == cudaStreamCaptureStatusActive ? id : 0;
+}
+
+// May the first layer of a step start before its predecessor has ended?  Not where that can be the packing of the weights
+// it loads.  A step recorded into a graph does not follow a packing that runs outside of it: the next one may.
+bool first_layer_dependent(TcState* t, cudaStream_t s)
+{
+    if (!t->fresh) return true;
+    const unsigned long long now = capture_of(s);
+    if (now == 0 || now == t->fresh_capture) t->fresh = false;
+    return false;
+}
+
+}  // namespace
+
 hts_status tc_load_weights(TcState* t, const hts_weights& w, cudaStream_t s)
 {
     const Geometry& g = t->g;
@@ -769,6 +788,8 @@ hts_status tc_load_weights(TcState* t, const hts_weights& w, cudaStream_t s)
     note_launch();
     HTS_CUDA(launch_pdl(pack_kernel, dim3(512 + nblk(rest, 256)), dim3(256), 0, s, p));
     note_launch();
+    t->fresh = true;
+    t->fresh_capture = capture_of(s);
     return HTS_OK;
 }
 
@@ -776,16 +797,17 @@ hts_status tc_forward(TcState* t, const uint8_t* obs, const Indexing& ix, int n,
 {
     const Geometry& g = t->g;
     hts_status st;
+    const bool dependent = first_layer_dependent(t, s);
     if (t->stacked && n <= kStackEnvs * device_sm_count(device_slot())) {
         ConvStackParams c = t->stack;
         c.obs = obs; c.slots = ix.slots; c.pool = ix.pool; c.n = n;
         prof.begin(K_CONV1, s);
-        st = conv_stack_launch(t->mW1, t->mB2, t->mB3, c, s);
+        st = conv_stack_launch(t->mW1, t->mB2, t->mB3, c, dependent, s);
         if (st != HTS_OK) return st;
         prof.end(K_CONV1, s);
     } else {
         prof.begin(K_CONV1, s);
-        st = conv1_launch(t->pl1, t->mW1, t->maps1, obs, ix, n, t->b1, t->inv_scale + L_CONV1, t->a1s, t->status, s);
+        st = conv1_launch(t->pl1, t->mW1, t->maps1, obs, ix, n, t->b1, t->inv_scale + L_CONV1, t->a1s, t->status, dependent, s);
         if (st != HTS_OK) return st;
         prof.end(K_CONV1, s);
 
