@@ -421,7 +421,7 @@ bool x3_plan(X3State* t)
     {   // dense layer: kind = (128 outputs, two pixels)
         X3WgradParams& p = t->wfc; p = X3WgradParams{};
         p.n_b = 2;
-        if (!wgrad_rings(&p, 3, 3, 64, 0, 2, 2, &sh)) return false;
+        if (!wgrad_rings(&p, 3, 3, kX3StageRows<64>, 0, 2, 2, &sh)) return false;
         p.ka = 4; p.a_step = 128; p.b_step = 128; p.slab_col[1] = 64;
         p.groups = 2; p.group_cap = 2; p.kinds = 4 * ((t->P3 + 1) / 2); p.ranges = p.last_ranges = 1;
         p.a_lbo[0] = p.a_lbo[1] = slab(p, 3); p.b_off[1] = 3 * p.kr * 128; p.P3 = t->P3;
@@ -429,7 +429,7 @@ bool x3_plan(X3State* t)
     {   // conv3: five pairs of taps (0,1) (2,3) (4,5) (6,7) (7,8)
         X3WgradParams& p = t->wc3; p = X3WgradParams{};
         p.n_b = 1;
-        if (!wgrad_rings(&p, 3, 3, 64, s3[8], 1, 4, &sh)) return false;
+        if (!wgrad_rings(&p, 3, 3, kX3StageRows<64>, s3[8], 1, 4, &sh)) return false;
         p.ka = 1; p.kinds = 3; p.group_mul = 2; p.groups = 2; p.group_cap = 5;
         for (int gi = 0; gi < 5; ++gi) {
             const int t0 = gi < 4 ? 2 * gi : 7;
@@ -442,7 +442,7 @@ bool x3_plan(X3State* t)
     {   // conv2: a group = one tap, its two 64-channel slabs
         X3WgradParams& p = t->wc2; p = X3WgradParams{};
         p.n_b = 1;
-        if (!wgrad_rings(&p, 3, 3, 64, s2[3], 2, 4, &sh)) return false;
+        if (!wgrad_rings(&p, 3, 3, kX3StageRows<64>, s2[3], 2, 4, &sh)) return false;
         p.ka = 1; p.kinds = 2; p.group_mul = 2; p.groups = 2; p.group_cap = 4;
         for (int gi = 0; gi < 4; ++gi) {
             p.a_off[gi] = sh ? s2[gi] * 128 : (gi & 1) * 2 * slab(p, 3);
@@ -454,7 +454,7 @@ bool x3_plan(X3State* t)
     {   // conv1: kind = 64 columns of a cell, groups = the tap pairs (0,1) (2,3)
         X3WgradParams& p = t->wc1; p = X3WgradParams{};
         p.n_b = 2;
-        if (!wgrad_rings(&p, 1, 1, 128, s1[3], 1, 4, &sh)) return false;
+        if (!wgrad_rings(&p, 1, 1, kX3StageRows<32>, s1[3], 1, 4, &sh)) return false;
         p.ka = p.kinds = t->Cp / 4; p.a_step = 64; p.group_mul = 2; p.groups = 2; p.group_cap = 2 * p.kinds;
         for (int gi = 0; gi < p.group_cap; ++gi) {
             p.a_off[gi] = sh ? s1[2 * (gi & 1)] * 128 : (gi & 1) * 2 * slab(p, 1);

@@ -43,37 +43,47 @@ __device__ __forceinline__ void mma_x3(uint32_t d, uint64_t a, uint64_t a_plane,
         mma_f16_ss(d + 2 * NB, a + 2 * a_plane, b, idesc_x3(NB, 0, 0) | (mn_a << 15) | (mn_b << 16), 1);
     }
 }
-template <int NB>
-__device__ __forceinline__ void acc_load32(uint32_t taddr, int c0, float (&v)[32], bool last, uint64_t* empty_bar)
+// Columns [c0, c0 + 32) of an accumulator added to a running sum, its three weight classes smallest first.  WIDE: all
+// three in registers at once, one trip to tensor memory instead of two (where the sums leave room for 96 more).
+template <int NB, bool WIDE>
+__device__ __forceinline__ void acc_add32(uint32_t taddr, int c0, float* sum)
 {
-    uint32_t p0[32], p1[32];
-    tmem_ld_32x32(taddr + NB + c0, p0);
-    tmem_ld_32x32(taddr + 2 * NB + c0, p1);
+    uint32_t p0[32], p1[32], p2[32];
+    tmem_ld_32x32(taddr + NB + c0, p1);
+    tmem_ld_32x32(taddr + 2 * NB + c0, p2);
+    if (WIDE) tmem_ld_32x32(taddr + c0, p0);
     tmem_ld_wait();
 #pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(p0[j]) + __uint_as_float(p1[j]);
-    tmem_ld_32x32(taddr + c0, p0);
-    tmem_ld_wait();
-    if (last && empty_bar) {                            // everything is in registers: hand the accumulator back
-        tc_fence_before();
-        mbar_arrive(empty_bar);
+    for (int j = 0; j < 32; ++j) p1[j] = __float_as_uint(__uint_as_float(p1[j]) + __uint_as_float(p2[j]));
+    if (!WIDE) {
+        tmem_ld_32x32(taddr + c0, p0);
+        tmem_ld_wait();
     }
 #pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(p0[j]) + v[j];
+    for (int j = 0; j < 32; ++j) sum[j] += __uint_as_float(p0[j]) + __uint_as_float(p1[j]);
+}
+// The accumulator is in registers: hand it back.
+__device__ __forceinline__ void acc_release(uint64_t* empty_bar, int lane)
+{
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(empty_bar);
 }
 
 // Persistent: CTA b takes tiles b, b + gridDim.x, ...  Warp 0 copies (A entries and B stages in two rings), warp 1
-// issues, then two groups of four epilogue warps, one accumulator of 192 columns each.
+// issues, then eight epilogue warps, two per lane quarter with 32 columns each.  Two accumulators of 192 columns take
+// pairs of B stages (128 of K) in turn; the epilogue adds each to the tile's sum in registers (see "Accumulation" in
+// x3_gemm.cuh).
 // Bound: the tensor core, which spends (128 + N) / 4 clocks (shared-memory operand fetch) or N / 2 on an
 // instruction: 96 + 64 + 48 = 208 clocks per 16 of K for 64 output columns, against 288 for six separate
 // 128 x 64 instructions.  An A entry (all planes, rows 128 + spread) is loaded once per tile and every tap reads it
 // shifted; B is streamed.
-constexpr int EG = 2, kDgradThreads = 64 + 128 * EG;
-__global__ void __launch_bounds__(kDgradThreads)
+constexpr int kAccs = 2, kPart = 2, kThreads = 64 + 256;
+__global__ void __launch_bounds__(kThreads)
 x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const X3TapParams p)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t a_full[kMaxEntries], a_empty[kMaxEntries], b_full[kMaxStages], b_empty[kMaxStages], d_full[EG], d_empty[EG];
+    __shared__ uint64_t a_full[kMaxEntries], a_empty[kMaxEntries], b_full[kMaxStages], b_empty[kMaxStages], d_full[kAccs], d_empty[kAccs];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     volatile int* abortp = &abort_flag;
@@ -89,7 +99,7 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     if (threadIdx.x == 0) {
         for (int i = 0; i < kMaxEntries; ++i) { mbar_init(&a_full[i], 1); mbar_init(&a_empty[i], 1); }
         for (int i = 0; i < kMaxStages; ++i) { mbar_init(&b_full[i], 1); mbar_init(&b_empty[i], 1); }
-        for (int i = 0; i < EG; ++i) { mbar_init(&d_full[i], 1); mbar_init(&d_empty[i], 128); }
+        for (int i = 0; i < kAccs; ++i) { mbar_init(&d_full[i], 1); mbar_init(&d_empty[i], 8); }
         abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
@@ -130,72 +140,71 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            int ea = 0, sb = 0, it = 0;
+            int ea = 0, sb = 0, it = 0, left = p.chunks * p.taps, in = 0;
             uint32_t pa = 0, pb = 0;
             bool alive = true;
             const uint64_t a_plane = (uint64_t)(plane_bytes >> 4);
-            for (int t = blockIdx.x; alive && t < tiles; t += gridDim.x, ++it) {
-                const int acc = it % EG;
-                if (!mbar_wait(&d_empty[acc], (((uint32_t)(it / EG)) & 1u) ^ 1u, abortp, p.status, 83)) break;
-                tc_fence_after();
-                const uint32_t d = tmem_d + acc * 192;
-                bool first = true;
+            for (int t = blockIdx.x; alive && t < tiles; t += gridDim.x, left = p.chunks * p.taps)
                 for (int c = 0; alive && c < p.chunks; ++c)
                     for (int g = 0; alive && g < groups; ++g) {
                         if (!mbar_wait(&a_full[ea], pa, abortp, p.status, 84)) { alive = false; break; }
                         for (int j = 0; j < p.tpe; ++j) {
+                            const int acc = it % kAccs;
                             if (!mbar_wait(&b_full[sb], pb, abortp, p.status, 85)) { alive = false; break; }
+                            if (in == 0 && !mbar_wait(&d_empty[acc], (((uint32_t)(it / kAccs)) & 1u) ^ 1u, abortp, p.status, 83)) { alive = false; break; }
                             tc_fence_after();
                             const uint32_t row = p.tpe == 1 ? 0 : (uint32_t)(p.shift[j] - p.lo);
                             const uint64_t a = smem_desc_sw128(base + ea * a_pitch + row * 128);
                             const uint64_t b = smem_desc_mn(b_base + sb * BB, BB / 3);
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                mma_x3<3, 64>(d, a + 2 * k, a_plane, b + 128 * k, 0, 1, first);   // 32 bytes along A's rows, 16 rows of B
-                                first = false;
-                            }
+                            for (int k = 0; k < 4; ++k)          // 32 bytes along A's rows, 16 rows of B
+                                mma_x3<3, 64>(tmem_d + acc * 192, a + 2 * k, a_plane, b + 128 * k, 0, 1, (in | k) == 0);
                             mma_commit(&b_empty[sb]);
+                            --left;
+                            if (++in == kPart || left == 0) { mma_commit(&d_full[acc]); ++it; in = 0; }
                             if (++sb == p.b_stages) { sb = 0; pb ^= 1u; }
                         }
                         mma_commit(&a_empty[ea]);
                         if (++ea == p.entries) { ea = 0; pa ^= 1u; }
                     }
-                if (alive) mma_commit(&d_full[acc]);
-            }
         }
     } else {
-        const int grp = (warp - 2) >> 2, q = warp & 3;  // TMEM lane quarter of this warp
-        const int row = q * 32 + lane;
-        int it = grp;
-        for (int t = blockIdx.x + grp * gridDim.x; t < tiles; t += EG * gridDim.x, it += EG) {
+        const int j = (warp - 2) >> 2, q = warp & 3;    // half of the columns; TMEM lane quarter of this warp
+        const int row = q * 32 + lane, parts = (p.chunks * p.taps + kPart - 1) / kPart;
+        int it = 0;
+        bool alive = true;
+        for (int t = blockIdx.x; alive && t < tiles; t += gridDim.x) {
             const int mt = t % p.m_tiles, nt = t / p.m_tiles;
             const int m = mt * 128 + row;
             int env = m / p.P, pix = m - env * p.P;
             int y = pix / p.W, x = pix - y * p.W;
             if (p.mode == X3_DGRAD_FC) { y = nt / p.W_out; x = nt - y * p.W_out; }
-            if (!mbar_wait_warp(&d_full[grp], ((uint32_t)(it / EG)) & 1u, abortp, p.status, 86)) break;
-            tc_fence_after();
-            const uint32_t taddr = tmem_d + grp * 192 + ((uint32_t)(q * 32) << 16);
+            bool ok = env < p.n && y < p.H_out && x < p.W_out;
+            size_t off;
+            if (p.mode == X3_DGRAD_S2D) {
+                const int yy = 2 * y + nt, xx = 2 * x + j;
+                ok = env < p.n && yy < p.H_out && xx < p.W_out;
+                off = ((size_t)env * p.P_dst + (size_t)yy * p.W_dst + xx) * p.dst_pitch;
+            } else
+                off = ((size_t)env * p.P_dst + (size_t)y * p.W_dst + x) * p.dst_pitch + j * 32;
+            uint32_t mk[16];
+            if (ok) {
+                const uint4* src = reinterpret_cast<const uint4*>(p.mask + (size_t)m * p.mask_pitch + nt * 64 + j * 32);
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                __syncwarp();                           // rows without a destination have left the previous half early
-                bool ok = env < p.n && y < p.H_out && x < p.W_out;
-                size_t off;
-                if (p.mode == X3_DGRAD_S2D) {
-                    const int yy = 2 * y + nt, xx = 2 * x + j;
-                    ok = env < p.n && yy < p.H_out && xx < p.W_out;
-                    off = ((size_t)env * p.P_dst + (size_t)yy * p.W_dst + xx) * p.dst_pitch;
-                } else
-                    off = ((size_t)env * p.P_dst + (size_t)y * p.W_dst + x) * p.dst_pitch + j * 32;
-                uint32_t mk[16];
-                if (ok) {
-                    const uint4* src = reinterpret_cast<const uint4*>(p.mask + (size_t)m * p.mask_pitch + nt * 64 + j * 32);
+                for (int i = 0; i < 4; ++i) reinterpret_cast<uint4*>(mk)[i] = src[i];
+            }
+            float v[32];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) reinterpret_cast<uint4*>(mk)[i] = src[i];
-                }
-                float v[32];
-                acc_load32<64>(taddr, j * 32, v, j == 2 - 1, &d_empty[grp]);
-                if (!ok) continue;
+            for (int i = 0; i < 32; ++i) v[i] = 0.f;
+            for (int s = 0; s < parts; ++s, ++it) {
+                const int acc = it % kAccs;
+                alive = mbar_wait_warp(&d_full[acc], ((uint32_t)(it / kAccs)) & 1u, abortp, p.status, 86);
+                if (!alive) break;
+                tc_fence_after();
+                acc_add32<64, true>(tmem_d + acc * 192 + ((uint32_t)(q * 32) << 16), j * 32, v);
+                acc_release(&d_empty[acc], lane);
+            }
+            if (alive && ok) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {           // positive bf16: sign clear, not zero
                     if ((int16_t)(mk[i] & 0xffffu) <= 0) v[2 * i] = 0.f;
@@ -212,6 +221,7 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     st_v8(dst + 2 * p.dst_plane + h, o2);
                 }
             }
+            __syncwarp();                               // rows without a destination are here already
         }
     }
     if (*abortp) {                                      // give copies still in flight time to land
@@ -223,27 +233,35 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     if (warp == 1) tmem_dealloc(tmem_d, 512);
 }
 
-// One CTA = (kind, range of row chunks).  Warp 0 copies, warp 1 issues, warps 2..5 sum the columns of B while the
-// main loop runs (bias gradient) and write the accumulators at the end.
+// One CTA = (kind, range of row chunks).  Warp 0 copies, warps 1 and 2 issue, two sets of four warps (3..6, 7..10) keep
+// the sums in registers (see "Accumulation" in x3_gemm.cuh).  Issuing thread e has accumulators of its own and set e
+// adds them up: with two groups it serves group e, with one group every other pair of stages.  An accumulation covers
+// 128 rows: two stages of 64, or one of 128 (NB = 32, whose narrow products have two accumulators per thread).  The
+// first one of group 0 is a single stage, so that one thread's products run while the other waits for its accumulator
+// to be read.  One thread for both groups leaves the tensor core waiting (its instructions come 55 to 70 clocks apart):
+// weight gradients of conv3 / conv2 / conv1 / dense at n = 1024, 84 x 84: 52 / 48 / 43 / 33 us, 43 / 44 / 38 / 30 with two.
+// The sets of kind 0 also sum the columns of B (bias gradient).
 // Both operands have the contracted index along their rows (pixels), so tiles go from global memory to the tensor
 // core without a transposition; a tap is a row offset into the slab, and the two taps (or slabs) of a group are two
 // 64-row blocks of M at a free distance (the leading byte offset).  Bound: the tensor core, 208 clocks per 16 rows and
 // group (56 for frames).
+constexpr int kWgradThreads = 96 + 256;
 template <int APL, int NB>
-__global__ void __launch_bounds__(192)
+__global__ void __launch_bounds__(kWgradThreads)
 x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const X3WgradParams p)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full[kMaxStages], empty[kMaxStages], done;
-    __shared__ float s_sum[128][2];
+    constexpr int NACC = NB == 64 ? 2 : 4;              // accumulators
+    __shared__ uint64_t full[kMaxStages], empty[kMaxStages], d_full[NACC], d_empty[NACC];
+    __shared__ float s_sum[256][2];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     volatile int* abortp = &abort_flag;
     constexpr int BPL = NB == 64 ? 3 : 1;               // NB = 32: the planes are 32-column blocks of one row
-    constexpr int ACC = 3 * NB;
+    constexpr int ACC = 3 * NB, KR = kX3StageRows<NB>;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint8_t* sm = smem_raw + (base - smem_u32(smem_raw));
-    const int a_slab = (APL * p.a_rows * 128 + 1023) & ~1023, b_plane = p.kr * 128, b_slab = BPL * b_plane;
+    uint8_t* sm = smem_raw + (base - smem_u32(smem_raw));
+    const int a_slab = (APL * p.a_rows * 128 + 1023) & ~1023, b_plane = KR * 128, b_slab = BPL * b_plane;
     const int a_tx = APL * p.a_rows * 128;
     const int stage_bytes = p.n_a * a_slab + p.n_b * b_slab;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -255,10 +273,11 @@ x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int gi0 = kind * p.group_mul;
     int groups = p.groups;
     if (gi0 + groups > p.group_cap) groups = p.group_cap - gi0;
+    const bool biased = p.bias_part && kind == 0;
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kMaxStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], p.bias_part ? 5 : 1); }
-        mbar_init(&done, 1);
+        for (int i = 0; i < kMaxStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], biased ? 10 : 2); }
+        for (int i = 0; i < NACC; ++i) { mbar_init(&d_full[i], 1); mbar_init(&d_empty[i], 4); }
         abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
@@ -282,100 +301,125 @@ x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const uint32_t dst = base + s * stage_bytes;
                 for (int i = 0; i < p.n_a; ++i) {
                     const int k = kind * p.slab_mul + i;
-                    tma_load_3d(dst + i * a_slab, &tmA, a_col + p.slab_col[k], c * p.kr + p.slab_row[k], 0, &full[s]);
+                    tma_load_3d(dst + i * a_slab, &tmA, a_col + p.slab_col[k], c * KR + p.slab_row[k], 0, &full[s]);
                 }
                 for (int i = 0; i < p.n_b; ++i)
-                    tma_load_3d(dst + p.n_a * a_slab + i * b_slab, &tmB, b_col + 64 * i, c * p.kr, 0, &full[s]);
+                    tma_load_3d(dst + p.n_a * a_slab + i * b_slab, &tmB, b_col + 64 * i, c * KR, 0, &full[s]);
                 if (++s == p.stages) { s = 0; ph ^= 1u; }
             }
         }
-    } else if (warp == 1) {
+    } else if (warp <= 2) {
         if (lane == 0) {
-            int s = 0;
+            const int e = warp - 1;
+            int s = 0, k = 0;                           // k: accumulation of this thread
             uint32_t ph = 0;
-            bool alive = true;
             const uint64_t a_plane = (uint64_t)((p.a_rows * 128) >> 4);
             const uint32_t b_lbo = NB == 64 ? (uint32_t)b_plane : (uint32_t)b_slab;
+            const int gi = groups == 2 ? gi0 + e : gi0;
+            const uint32_t a_off = (uint32_t)p.a_off[gi], a_lbo = (uint32_t)p.a_lbo[gi], b_off = (uint32_t)(p.n_a * a_slab + p.b_off[gi - gi0]);
             for (int c = c0; c < c1; ++c) {
-                if (!mbar_wait(&full[s], ph, abortp, p.status, 92)) { alive = false; break; }
-                tc_fence_after();
-                const uint32_t a0 = base + s * stage_bytes, b0 = a0 + p.n_a * a_slab;
-                for (int g = 0; g < groups; ++g) {
-                    const uint64_t a = smem_desc_mn(a0 + p.a_off[gi0 + g], p.a_lbo[gi0 + g]);
-                    const uint64_t b = smem_desc_mn(b0 + p.b_off[g], b_lbo);
-                    for (int k = 0; k < p.kr / 16; ++k)
-                        mma_x3<APL, NB>(tmem_d + g * ACC, a + 128 * k, a_plane, b + 128 * k, 1, 1, c == c0 && k == 0);
-                }
-                mma_commit(&empty[s]);
+                const int i = c - c0;
+                if (!mbar_wait(&full[s], ph, abortp, p.status, 92)) break;
+                if (groups == 2 || ((i >> 1) & 1) == e) {
+                    const int half = groups == 2 ? i + 1 - e : i;          // first stage of an accumulation: even
+                    const bool first = NB == 32 || i == 0 || (half & 1) == 0;
+                    const int acc = NB == 32 ? e + 2 * (k & 1) : e;
+                    if (first && !mbar_wait(&d_empty[acc], ((uint32_t)(NB == 32 ? k >> 1 : k) & 1u) ^ 1u, abortp, p.status, 95)) break;
+                    tc_fence_after();
+                    const uint64_t a = smem_desc_mn(base + s * stage_bytes + a_off, a_lbo);
+                    const uint64_t b = smem_desc_mn(base + s * stage_bytes + b_off, b_lbo);
+                    const uint32_t d = tmem_d + acc * ACC;
+#pragma unroll
+                    for (int kk = 0; kk < KR / 16; ++kk)
+                        mma_x3<APL, NB>(d, a + 128 * kk, a_plane, b + 128 * kk, 1, 1, first && kk == 0);
+                    mma_commit(&empty[s]);
+                    if (NB == 32 || (half & 1) == 1 || c == c1 - 1) { mma_commit(&d_full[acc]); ++k; }
+                } else
+                    mbar_arrive(&empty[s]);
                 if (++s == p.stages) { s = 0; ph ^= 1u; }
             }
-            if (alive) mma_commit(&done);
         }
     } else {
-        const int wt = threadIdx.x - 64;
-        bool ok = true;
-        if (p.bias_part) {                              // all four warps arrive on each stage; those of kind 0 sum
-            int s = 0;
-            uint32_t ph = 0;
-            float s0 = 0.f, s1 = 0.f;
-            constexpr int TC = NB / 2;                  // threads along the columns (two columns each)
-            const int cp = wt % TC, r0 = wt / TC;
-            for (int c = c0; ok && c < c1; ++c) {
-                ok = mbar_wait_warp(&full[s], ph, abortp, p.status, 93);
-                if (ok && kind == 0) {
-                    const uint8_t* b = sm + s * stage_bytes + p.n_a * a_slab;
-                    for (int r = r0; r < p.kr; r += 128 / TC) {
-                        float t0 = 0.f, t1 = 0.f;
+        const int wt = threadIdx.x - 96, set = (warp - 3) >> 2, q = warp & 3, m = q * 32 + lane;
+        const uint32_t taddr = tmem_d + ((uint32_t)(q * 32) << 16);
+        constexpr int TC = NB / 2;                      // threads along the columns of B (two columns each)
+        const int cp = wt % TC, r0 = wt / TC;
+        float sum[NB], s0 = 0.f, s1 = 0.f;
 #pragma unroll
-                        for (int pl = 2; pl >= 0; --pl) {
-                            // byte of the pair inside its 128-byte row, and the row's place (address-based swizzle)
-                            const int col = NB == 64 ? cp * 4 : (pl & 1) * 64 + cp * 4;
-                            const int blk = NB == 64 ? pl : pl >> 1;
-                            const uint32_t off = (uint32_t)(blk * b_plane + r * 128 + (col ^ ((r & 7) << 4)));
-                            const uint32_t w = *reinterpret_cast<const uint32_t*>(b + off);
-                            t0 += __uint_as_float(w << 16); t1 += __uint_as_float(w & 0xffff0000u);
-                        }
-                        s0 += t0; s1 += t1;
+        for (int j = 0; j < NB; ++j) sum[j] = 0.f;
+        bool ok = true;
+        int s = 0;
+        uint32_t ph = 0;
+        int k = 0;                                      // accumulation of this set
+        auto drain = [&]() {
+            const int acc = NB == 32 ? set + 2 * (k & 1) : set;
+            ok = mbar_wait_warp(&d_full[acc], (uint32_t)(NB == 32 ? k >> 1 : k) & 1u, abortp, p.status, 94);
+            if (!ok) return;
+            tc_fence_after();
+#pragma unroll
+            for (int j = 0; j < NB; j += 32) acc_add32<NB, NB == 32>(taddr + acc * ACC, j, sum + j);
+            acc_release(&d_empty[acc], lane);
+            ++k;
+        };
+        const int n_st = c1 - c0;
+        for (int i = 0; ok && i <= n_st; ++i) {         // the columns of stage i, then the accumulations that ended in stage i - 1
+            if (biased && i < n_st) {
+                ok = mbar_wait_warp(&full[s], ph, abortp, p.status, 93);
+                if (!ok) break;
+                const uint8_t* b = sm + s * stage_bytes + p.n_a * a_slab;
+#pragma unroll 4
+                for (int r = r0; r < KR; r += 256 / TC) {
+                    float t0 = 0.f, t1 = 0.f;
+#pragma unroll
+                    for (int pl = 2; pl >= 0; --pl) {
+                        // byte of the pair inside its 128-byte row, and the row's place (address-based swizzle)
+                        const int col = NB == 64 ? cp * 4 : (pl & 1) * 64 + cp * 4;
+                        const int blk = NB == 64 ? pl : pl >> 1;
+                        const uint32_t off = (uint32_t)(blk * b_plane + r * 128 + (col ^ ((r & 7) << 4)));
+                        const uint32_t w = *reinterpret_cast<const uint32_t*>(b + off);
+                        t0 += __uint_as_float(w << 16); t1 += __uint_as_float(w & 0xffff0000u);
                     }
+                    s0 += t0; s1 += t1;
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty[s]);
                 if (++s == p.stages) { s = 0; ph ^= 1u; }
             }
-            if (kind == 0) {
-                s_sum[wt][0] = s0; s_sum[wt][1] = s1;
-                asm volatile("bar.sync 1, 128;" ::: "memory");
-                if (wt < NB) {
-                    float t = 0.f;
-                    for (int r = 0; r < 128 / TC; ++r) t += s_sum[r * TC + wt / 2][wt & 1];
-                    p.bias_part[range * NB + wt] = t;
-                }
+            const int e = i - 1;
+            if (e < 0 || (groups == 1 && ((e >> 1) & 1) != set)) continue;
+            if (NB == 32 || ((groups == 2 ? e + 1 - set : e) & 1) || e == n_st - 1) drain();
+        }
+        if (biased) {
+            s_sum[wt][0] = s0; s_sum[wt][1] = s1;
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            if (wt < NB) {
+                float t = 0.f;
+                for (int r = 0; r < 256 / TC; ++r) t += s_sum[r * TC + wt / 2][wt & 1];
+                p.bias_part[range * NB + wt] = t;
             }
         }
-        const int q = warp & 3, m = q * 32 + lane;
-        ok = ok && mbar_wait_warp(&done, 0, abortp, p.status, 94);
-        tc_fence_after();
-        if (ok) {
-            for (int g = 0; g < groups; ++g) {
-                const uint32_t taddr = tmem_d + g * ACC + ((uint32_t)(q * 32) << 16);
+        if (groups == 1) {                              // the stages' buffers are free once both sets are here
+            float* other = reinterpret_cast<float*>(sm);
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            if (set == 1)
 #pragma unroll
-                for (int j = 0; j < NB / 32; ++j) {
-                    float v[32];
-                    acc_load32<NB>(taddr, j * 32, v, false, nullptr);
-                    if (p.fc_w) {
-                        const int o = (kind % p.ka) * 128 + m, pix = (kind / p.ka) * 2 + g;
-                        if (pix < p.P3) {
-                            float* dst = p.fc_w + (size_t)o * 64 * p.P3 + pix * 64 + j * 32;
+                for (int j = 0; j < NB; ++j) other[j * 128 + m] = sum[j];
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            if (set == 0)
 #pragma unroll
-                            for (int i = 0; i < 32; i += 8) st_v8(dst + i, reinterpret_cast<const uint32_t*>(v) + i);
-                        }
-                    } else {
-                        float* dst = p.part + (gi0 + g) * p.group_stride + ((size_t)range * 128 + m) * NB + j * 32;
+                for (int j = 0; j < NB; ++j) sum[j] += other[j * 128 + m];
+        }
+        if (ok && set < groups) {
+            const uint32_t* v = reinterpret_cast<const uint32_t*>(sum);
+            float* dst = nullptr;
+            if (p.fc_w) {
+                const int o = (kind % p.ka) * 128 + m, pix = (kind / p.ka) * 2 + set;
+                if (pix < p.P3) dst = p.fc_w + (size_t)o * 64 * p.P3 + pix * 64;
+            } else
+                dst = p.part + (gi0 + set) * p.group_stride + ((size_t)range * 128 + m) * NB;
+            if (dst)
 #pragma unroll
-                        for (int i = 0; i < 32; i += 8) st_v8(dst + i, reinterpret_cast<const uint32_t*>(v) + i);
-                    }
-                }
-            }
+                for (int i = 0; i < NB; i += 8) st_v8(dst + i, v + i);
         }
     }
     if (*abortp) {
@@ -437,7 +481,7 @@ hts_status x3_dgrad_launch(const CUtensorMap& a, const CUtensorMap& b, const X3T
     }
     const int smem = 1024 + p.entries * ((3 * p.entry_rows * 128 + 1023) & ~1023) + p.b_stages * 3 * 8192;
     const int tiles = p.m_tiles * p.n_tiles, sms = device_sm_count(dev);
-    HTS_CUDA(launch_pdl(x3_dgrad_kernel, dim3(tiles < sms ? tiles : sms), dim3(kDgradThreads), (size_t)smem, s, a, b, p));
+    HTS_CUDA(launch_pdl(x3_dgrad_kernel, dim3(tiles < sms ? tiles : sms), dim3(kThreads), (size_t)smem, s, a, b, p));
     note_launch();
     return HTS_OK;
 }
@@ -448,15 +492,15 @@ hts_status x3_wgrad_launch(const CUtensorMap& a, const CUtensorMap& b, const X3W
     const int dev = device_slot();
     static bool attr_set[kDeviceSlots] = {};
     if (!attr_set[dev]) {
-        HTS_CUDA(cudaFuncSetAttribute(x3_wgrad_kernel<APL, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 2048));
+        HTS_CUDA(cudaFuncSetAttribute(x3_wgrad_kernel<APL, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 3072));
         HTS_CUDA(cudaFuncSetAttribute(x3_wgrad_kernel<APL, NB>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
         attr_set[dev] = true;
     }
-    const int a_slab = (APL * p.a_rows * 128 + 1023) & ~1023, b_slab = (NB == 64 ? 3 : 1) * p.kr * 128;
+    const int a_slab = (APL * p.a_rows * 128 + 1023) & ~1023, b_slab = (NB == 64 ? 3 : 1) * kX3StageRows<NB> * 128;
     const int smem = 1024 + p.stages * (p.n_a * a_slab + p.n_b * b_slab);
-    if (smem > kSmemMax - 2048) return HTS_ERR_SHAPE;
+    if (smem > kSmemMax - 3072) return HTS_ERR_SHAPE;     // the rest is the kernel's static share
     const int grid = p.ranges * (p.kinds - 1) + p.last_ranges;
-    HTS_CUDA(launch_pdl(x3_wgrad_kernel<APL, NB>, dim3(grid), dim3(192), (size_t)smem, s, a, b, p));
+    HTS_CUDA(launch_pdl(x3_wgrad_kernel<APL, NB>, dim3(grid), dim3(kWgradThreads), (size_t)smem, s, a, b, p));
     note_launch();
     return HTS_OK;
 }

@@ -4,7 +4,15 @@
 // round-to-nearest remainders).  A product of two such sums has nine terms; the six whose weight is at least
 // 2^-16 of the leading one are multiplied by tcgen05.mma (bf16 products are exact, accumulation is fp32) and the
 // three below 2^-24 are dropped: less than one rounding of an fp32 multiply-add.  The terms of weight 1, 2^-8 and
-// 2^-16 go to accumulators of their own, which are added smallest first once a tile is complete.
+// 2^-16 go to accumulators of their own, which are added smallest first.
+//
+// Accumulation.  The tensor core does not round a sum to nearest but cuts it off: a chain of s instructions (16 products
+// each) comes out too small by up to s last places, s / 2 on average, all in one direction.  So a chain is eight
+// instructions, 128 of K, and the epilogue warps add the chains in registers, rounded to nearest, while the next ones
+// run.  Error (2-norm against 64 bits, learner batches of 5 to 1024 of four frame shapes), conv1's weights and the
+// whole gradient: one chain per tile or range of rows (16 to 200 instructions) 5 to 33e-7 and 2 to 13e-7, fp32
+// multiply-adds in order 2 to 11e-7 and 2 to 10e-7, chains of eight 2 to 6e-7 and 1 to 10e-7 (what is left is the forward
+// pass and the heads).  Chains of four are no closer and take 4 % longer; eight cost 2 % of a gradient of 1024 (860 to 876 us).
 //
 // Layouts: activations and gradients are stored as three planes of pixel-major rows [rows][channels] bf16, so
 // that the data gradient of a convolution is a sum over taps of row-shifted products on a flat pixel grid (x3_dgrad)
@@ -53,8 +61,9 @@ bool x3_taps_plan(X3TapParams* p, int chunks, int taps, const int* shift);
 // to two groups of 128 x NB: a group's M = two 64-column blocks at a_off and a_off + lbo (two taps of one slab, or
 // two slabs).
 constexpr int kX3MaxSlabs = 16, kX3MaxGroups = 32;
+template <int NB> constexpr int kX3StageRows = NB == 64 ? 64 : 128;
 struct X3WgradParams {
-    int kr, stages;                     // rows per stage, stages in the ring
+    int kr, stages;                     // rows per stage (kX3StageRows), stages in the ring
     int a_rows;                         // rows of an A slab (kr + spread of the taps)
     int n_a, n_b;                       // slabs per stage
     int ka, a_step, b_step;             // columns: A (kind % ka) * a_step + slab_col, B (kind / ka) * b_step + 64 * slab

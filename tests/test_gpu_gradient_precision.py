@@ -1,0 +1,54 @@
+"""The gradient's tensor-core sums against 64 bits, given the ReLU decisions of the run itself."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+import torch.nn.functional as F
+
+import hts_workloads as wl
+from gpu_util import Policy
+from test_gpu_backward import gpu_gradient, make_batch
+
+pytestmark = pytest.mark.gpu
+# A chain of eight products sums is cut off eight times, each time by less than one last place (2^-23) of what it holds.
+# fp32 roundings of the rest go either way.  One chain for a whole range of rows (190 sums of conv1 at n = 640) is at 2.5 times that.
+CHAIN = 8 * 2.0 ** -23
+
+
+def gradient64(params, obs, actions, adv, ret, cv, ce, masks, chunk=128):
+    """Actor-critic objective's gradient by library operations in 64 bits; masks: which hidden units pass."""
+    w = {k: torch.from_numpy(np.asarray(v, np.float32)).cuda().double().requires_grad_() for k, v in params.items()}
+    n, total = len(obs), {k: torch.zeros_like(v) for k, v in w.items()}
+    f32 = lambda x: float(np.float32(x))
+    for i in range(0, n, chunk):
+        s = slice(i, min(n, i + chunk))
+        x = torch.from_numpy(obs[s]).cuda().double() / 255
+        for layer, stride in ((1, 4), (2, 2), (3, 1)):
+            x = F.conv2d(x, w[f"conv{layer}_w"], w[f"conv{layer}_b"], stride) * masks[layer - 1][s]
+        h = F.linear(x.flatten(1), w["fc_w"], w["fc_b"]) * masks[3][s]
+        logp = F.linear(h, w["pi_w"], w["pi_b"]).log_softmax(1)
+        v = F.linear(h, w["v_w"], w["v_b"])[:, 0]
+        a = torch.from_numpy(np.asarray(actions[s], np.int64)).cuda()
+        term = logp.gather(1, a[:, None])[:, 0] * torch.from_numpy(adv[s]).cuda().double()
+        term = term - f32(cv) * (torch.from_numpy(ret[s]).cuda().double() - v) ** 2 - f32(ce) * (logp.exp() * logp).sum(1)
+        for k, g in zip(w, torch.autograd.grad(term.sum() / n, list(w.values()))):
+            total[k] += g
+    return {k: v.cpu().numpy() for k, v in total.items()}
+
+
+# stages per range of rows: one or two, three or four, and as many as a learner's largest batches have
+@pytest.mark.parametrize("C,H,W,n", [(4, 84, 84, 80), (4, 84, 84, 150), (8, 84, 84, 640), (16, 72, 96, 61)])
+def test_error_stays_within_one_chain(C, H, W, n):
+    cfg = dataclasses.replace(wl.CONFIGS[1], C=C, H=H, W=W)
+    pol = Policy(cfg, max_batch=n)
+    try:
+        obs, actions, adv, ret = make_batch(cfg, n, n)
+        got = gpu_gradient(pol, obs, actions, adv, ret, None, 0.5, 0.01, 0.0)
+        masks = [torch.from_numpy(pol.activation(layer, n) > 0).cuda() for layer in (1, 2, 3, 4)]
+        ref = gradient64(pol.params, obs, actions, adv, ret, 0.5, 0.01, masks)
+        for k in ("conv1_w", "conv1_b", "conv2_w", "conv2_b", "conv3_w", "conv3_b", "fc_w", "fc_b"):
+            e = np.linalg.norm(got[k] - ref[k]) / np.linalg.norm(ref[k])
+            assert e <= CHAIN, (k, e, CHAIN)
+    finally:
+        pol.close()
