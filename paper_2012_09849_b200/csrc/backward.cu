@@ -247,7 +247,7 @@ head_wgrad_kernel(const float* __restrict__ dhead, const float* __restrict__ h, 
             if (o0 + j <= A) acc[j] = fmaf(d[j], x, acc[j]);
             else if (o0 + j == A + 1) {
                 const bf16* g = dh + (size_t)i * 512 + k;
-                acc[j] += __bfloat162float(g[0]) + (__bfloat162float(g[dh_plane]) + __bfloat162float(g[2 * dh_plane]));
+                acc[j] += x3_sum(__bfloat162float(g[0]), __bfloat162float(g[dh_plane]) + __bfloat162float(g[2 * dh_plane]));
             }
         }
     }

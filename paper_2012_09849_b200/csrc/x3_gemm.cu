@@ -45,10 +45,10 @@ __device__ __forceinline__ void mma_x3(uint32_t d, uint64_t a, uint64_t a_plane,
 }
 // Columns [c0, c0 + 32) of an accumulator added to a running sum, its three weight classes smallest first.  WIDE: all
 // three in registers at once, one trip to tensor memory instead of two (where the sums leave room for 96 more).
-template <int NB, bool WIDE>
+template <int NB, bool WIDE, bool GUARD>
 __device__ __forceinline__ void acc_add32(uint32_t taddr, int c0, float* sum)
 {
-    uint32_t p0[32], p1[32], p2[32];
+    uint32_t p0[32], p1[32], p2[32], any = 0;
     tmem_ld_32x32(taddr + NB + c0, p1);
     tmem_ld_32x32(taddr + 2 * NB + c0, p2);
     if (WIDE) tmem_ld_32x32(taddr + c0, p0);
@@ -58,6 +58,12 @@ __device__ __forceinline__ void acc_add32(uint32_t taddr, int c0, float* sum)
     if (!WIDE) {
         tmem_ld_32x32(taddr + c0, p0);
         tmem_ld_wait();
+    }
+#pragma unroll
+    for (int j = 0; j < 32; ++j) any |= p0[j];
+    if (GUARD && (any & 0x7f800000u) == 0x7f800000u) {  // none is infinite or NaN otherwise
+#pragma unroll
+        for (int j = 0; j < 32; ++j) p1[j] = fabsf(__uint_as_float(p0[j])) < INFINITY ? p1[j] : 0;
     }
 #pragma unroll
     for (int j = 0; j < 32; ++j) sum[j] += __uint_as_float(p0[j]) + __uint_as_float(p1[j]);
@@ -201,7 +207,7 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 alive = mbar_wait_warp(&d_full[acc], ((uint32_t)(it / kAccs)) & 1u, abortp, p.status, 86);
                 if (!alive) break;
                 tc_fence_after();
-                acc_add32<64, true>(tmem_d + acc * 192 + ((uint32_t)(q * 32) << 16), j * 32, v);
+                acc_add32<64, true, true>(tmem_d + acc * 192 + ((uint32_t)(q * 32) << 16), j * 32, v);
                 acc_release(&d_empty[acc], lane);
             }
             if (alive && ok) {
@@ -215,7 +221,7 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 for (int h = 0; h < 32; h += 16) {
                     uint32_t o0[8], o1[8], o2[8];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) x3_split2(v[h + 2 * i], v[h + 2 * i + 1], o0[i], o1[i], o2[i]);
+                    for (int i = 0; i < 8; ++i) x3_split2<true>(v[h + 2 * i], v[h + 2 * i + 1], o0[i], o1[i], o2[i]);
                     st_v8(dst + h, o0);
                     st_v8(dst + p.dst_plane + h, o1);
                     st_v8(dst + 2 * p.dst_plane + h, o2);
@@ -344,7 +350,7 @@ x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         const uint32_t taddr = tmem_d + ((uint32_t)(q * 32) << 16);
         constexpr int TC = NB / 2;                      // threads along the columns of B (two columns each)
         const int cp = wt % TC, r0 = wt / TC;
-        float sum[NB], s0 = 0.f, s1 = 0.f;
+        float sum[NB], s0 = 0.f, s1 = 0.f, l0 = 0.f, l1 = 0.f;      // first pieces and lower ones of two columns
 #pragma unroll
         for (int j = 0; j < NB; ++j) sum[j] = 0.f;
         bool ok = true;
@@ -357,7 +363,7 @@ x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             if (!ok) return;
             tc_fence_after();
 #pragma unroll
-            for (int j = 0; j < NB; j += 32) acc_add32<NB, NB == 32>(taddr + acc * ACC, j, sum + j);
+            for (int j = 0; j < NB; j += 32) acc_add32<NB, NB == 32, APL == 3>(taddr + acc * ACC, j, sum + j);
             acc_release(&d_empty[acc], lane);
             ++k;
         };
@@ -369,17 +375,18 @@ x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const uint8_t* b = sm + s * stage_bytes + p.n_a * a_slab;
 #pragma unroll 4
                 for (int r = r0; r < KR; r += 256 / TC) {
-                    float t0 = 0.f, t1 = 0.f;
+                    uint32_t w[3];
 #pragma unroll
-                    for (int pl = 2; pl >= 0; --pl) {
+                    for (int pl = 0; pl < 3; ++pl) {
                         // byte of the pair inside its 128-byte row, and the row's place (address-based swizzle)
                         const int col = NB == 64 ? cp * 4 : (pl & 1) * 64 + cp * 4;
                         const int blk = NB == 64 ? pl : pl >> 1;
                         const uint32_t off = (uint32_t)(blk * b_plane + r * 128 + (col ^ ((r & 7) << 4)));
-                        const uint32_t w = *reinterpret_cast<const uint32_t*>(b + off);
-                        t0 += __uint_as_float(w << 16); t1 += __uint_as_float(w & 0xffff0000u);
+                        w[pl] = *reinterpret_cast<const uint32_t*>(b + off);
                     }
-                    s0 += t0; s1 += t1;
+                    s0 += __uint_as_float(w[0] << 16); s1 += __uint_as_float(w[0] & 0xffff0000u);
+                    l0 += __uint_as_float(w[2] << 16) + __uint_as_float(w[1] << 16);
+                    l1 += __uint_as_float(w[2] & 0xffff0000u) + __uint_as_float(w[1] & 0xffff0000u);
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty[s]);
@@ -390,7 +397,7 @@ x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             if (NB == 32 || ((groups == 2 ? e + 1 - set : e) & 1) || e == n_st - 1) drain();
         }
         if (biased) {
-            s_sum[wt][0] = s0; s_sum[wt][1] = s1;
+            s_sum[wt][0] = x3_sum(s0, l0); s_sum[wt][1] = x3_sum(s1, l1);
             asm volatile("bar.sync 1, 256;" ::: "memory");
             if (wt < NB) {
                 float t = 0.f;

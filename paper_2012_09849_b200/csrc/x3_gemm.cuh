@@ -88,15 +88,22 @@ bool x3_make_map(CUtensorMap* m, const void* ptr, uint64_t cols, uint64_t rows, 
                  uint64_t plane_elems, uint32_t box_rows, uint32_t box_planes);
 
 #ifdef __CUDACC__
-// Two fp32 values -> three packed bf16 pairs whose sums are the values.
+// Two fp32 values -> three packed bf16 pairs whose sums are the values.  Where a first piece is infinite (a magnitude
+// above 3.39e38 rounds to that too) the lower ones mean nothing, or are zero with ZERO_LOW: a sum of first pieces, or of
+// products of first pieces, that is not finite is the value by itself (x3_sum), so that a sum is infinite or NaN where
+// its fp32 form is.  The frames' gradient has one finite piece on its other side: zero lower pieces are enough there.
+template <bool ZERO_LOW = false>
 __device__ __forceinline__ void x3_split2(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2)
 {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p0) : "f"(b), "f"(a));
-    const float ra = a - __uint_as_float(p0 << 16), rb = b - __uint_as_float(p0 & 0xffff0000u);
+    const float ha = __uint_as_float(p0 << 16), hb = __uint_as_float(p0 & 0xffff0000u);
+    const float ra = !ZERO_LOW || fabsf(ha) < INFINITY ? a - ha : 0.f, rb = !ZERO_LOW || fabsf(hb) < INFINITY ? b - hb : 0.f;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p1) : "f"(rb), "f"(ra));
     const float sa = ra - __uint_as_float(p1 << 16), sb = rb - __uint_as_float(p1 & 0xffff0000u);
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p2) : "f"(sb), "f"(sa));
 }
+// A sum of first pieces (or of products of them) and what the lower ones add to it.
+__device__ __forceinline__ float x3_sum(float first, float low) { return first + (fabsf(first) < INFINITY ? low : 0.f); }
 #endif
 
 }  // namespace hts
