@@ -512,14 +512,19 @@ hts_status launch_fc_chain(const float* x, const float* w, const float* b, float
     note_launch();
     return HTS_OK;
 }
+// The form goes by the narrow blocks (128 per 16 rows) of the SM that has most of them, k.  One wide block per SM takes as
+// long as five narrow ones, at every width of the layer: step with k = 5 (80 rows) and 6 (81) on 148 SMs, narrow / wide, us:
+// 98.1 / 98.0 and 104.2 / 98.1 with 3136 features, 143.8 / 144.0 and 149.3 / 144.6 with 2560, 36.6 / 37.1 and 37.4 / 37.2
+// with 256.  The fewer narrow blocks an SM has, the more each must have in flight and the less often its warps may meet:
+// stages of 512 columns, three deep at k = 1 and two at k = 2 (both fill the shared memory), of 128 columns above (k = 1 / 2 / 3,
+// 3136 features: 45.4 / 52.4 / 71.5 us with the first, 45.8 / 48.1 / 69.4 with the second, 47.7 / 50.7 / 64.3 with the third).
 hts_status launch_fc(const float* x, const float* w, const float* b, float* h, int n, int F, cudaStream_t s)
 {
-    // one wide block per SM (n <= 128: 25 us) takes as long as five narrow ones (n = 80; n = 128 with eight: 34)
-    if (n > 80) return launch_fc_chain<8, 8, 4, 2, 4, 64>(x, w, b, h, n, F, s);
-    // 128 blocks per 16 rows.  The fewer of them an SM has, the more each must have in flight and the less often its warps
-    // may meet (64 columns, 8 stages before: n = 8 / 24 / 80: 45 / 57 / 125 us per step; now 41 / 53 / 123).
-    if (n <= 16) return launch_fc_chain<4, 4, 4, 1, 3, 512>(x, w, b, h, n, F, s);
-    if (n <= 32) return launch_fc_chain<4, 4, 4, 1, 2, 512>(x, w, b, h, n, F, s);
+    const int sms = device_sm_count(device_slot());
+    const long k = (128L * ((n + 15) / 16) + sms - 1) / sms;
+    if (k > 5) return launch_fc_chain<8, 8, 4, 2, 4, 64>(x, w, b, h, n, F, s);
+    if (k == 1) return launch_fc_chain<4, 4, 4, 1, 3, 512>(x, w, b, h, n, F, s);
+    if (k == 2) return launch_fc_chain<4, 4, 4, 1, 2, 512>(x, w, b, h, n, F, s);
     return launch_fc_chain<4, 4, 4, 1, 4, 128>(x, w, b, h, n, F, s);
 }
 

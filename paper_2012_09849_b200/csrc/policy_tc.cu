@@ -494,7 +494,7 @@ struct LoadTcParams {
     float* fdst[8];
     int fn[8];
 };
-constexpr int kAbsmaxBlocks = 4 * 148;
+constexpr int kAbsmaxPerSm = 4;         // blocks of the first
 
 __global__ void __launch_bounds__(256) absmax_kernel(const LoadTcParams p)
 {
@@ -784,7 +784,7 @@ hts_status tc_load_weights(TcState* t, const hts_weights& w, cudaStream_t s)
                          {w.v_w, t->whead + (size_t)g.A * 512, 512}, {w.pi_b, t->bhead, g.A}, {w.v_b, t->bhead + g.A, 1}};
     int rest = 128 * 16 * g.C + 64 * 512 + 64 * 576;
     for (int k = 0; k < 8; ++k) { p.f[k] = bf(items[k].p); p.fdst[k] = items[k].q; p.fn[k] = items[k].n; rest += items[k].n; }
-    HTS_CUDA(launch_pdl(absmax_kernel, dim3(kAbsmaxBlocks), dim3(256), 0, s, p));
+    HTS_CUDA(launch_pdl(absmax_kernel, dim3(kAbsmaxPerSm * device_sm_count(device_slot())), dim3(256), 0, s, p));
     note_launch();
     HTS_CUDA(launch_pdl(pack_kernel, dim3(512 + nblk(rest, 256)), dim3(256), 0, s, p));
     note_launch();
