@@ -183,8 +183,9 @@ typedef struct {
  * Only HTS_DTYPE_FP32 contexts (the learner's master weights are fp32; a bf16 actor context is refreshed
  * from them through hts_delayed_update's bf16 output and hts_policy_load_weights): a bf16 context returns
  * HTS_ERR_UNSUPPORTED.  The forward pass is hts_policy_step's own; the backward contractions run on the
- * tensor cores at fp32 accuracy (each operand as three bf16 pieces), every sum in a fixed order.  The first call on a context allocates the backward workspace (device memory, freed
- * by hts_policy_destroy).  An action outside the range is not used as an index: that sample contributes
+ * tensor cores at fp32 accuracy (each operand as three bf16 pieces), every sum in a fixed order; infinite inputs
+ * give infinities and NaN where fp32 sums do.
+ * The first call on a context allocates the backward workspace (device memory, freed by hts_policy_destroy).  An action outside the range is not used as an index: that sample contributes
  * nothing and hts_last_async_error reports INVALID_ARG.
  * Errors: INVALID_ARG (NULL, n out of range, clip < 0, non-finite coefficient), UNSUPPORTED, ALLOC, CUDA.  */
 hts_status hts_policy_gradient(hts_ctx *ctx, const uint8_t *obs, const int32_t *actions,

@@ -67,6 +67,8 @@ def lib():
         if not os.path.exists(path):
             raise ImportError(f"{path} is missing: run `python -m paper_2012_09849_b200.build`")
         L = C.CDLL(path)
+        # every entry point has its signature, also those that the functions below reach through the extension: a program
+        # may call the library object itself, and without one a pointer would be cut to 32 bits
         vp, i32, u64, f32 = C.c_void_p, C.c_int32, C.c_uint64, C.c_float
         L.hts_policy_create.argtypes = [C.POINTER(hts_net_desc), C.POINTER(vp)]
         L.hts_policy_load_weights.argtypes = [vp, C.POINTER(hts_weights), vp]

@@ -180,16 +180,20 @@ hts_status launch_gae(const float* rewards, const float* values, const uint8_t* 
                       aligned(bootstrap, 16) && aligned(adv, 16) && aligned(ret, 16) &&
                       ((long)N * T >= (1L << 22));
     const int sms = device_sm_count(device_slot());
-    // Enough blocks of 128 columns: all the parallelism needed is across env, two chunks of two rows per block measured best
-    // (86 % of the copy bandwidth at T=128, N=2^20).  Fewer would walk a long T in many short steps, each waiting for
-    // memory (213 us at 512 x 32768, 60 with the columns of a block cut to 32 and eight chunks of eight rows per step).
+    // Enough blocks of 128 columns: all the parallelism needed is across env, two chunks of two rows per block (6.3 TB/s,
+    // 97 % of the copy rate, at T=128, N=2^20).  Fewer would walk a long T in many short steps, each waiting for memory
+    // (213 us at 512 x 32768, 60 with the columns of a block cut to 32 and eight chunks of eight rows per step).  This form
+    // against the last one below, us at T=128: 50 / 34 (N = 75776), 62 / 57 (2^17), 91 / 109 (2^18), 356 / 427 (2^20);
+    // at T=512: 186 / 130, 234 / 222, 366 / 436: the line at four blocks per SM is low, they cross near 2^17 columns.
     if (vec4 && N / 128 >= 4 * sms)
         return launch_t<4, 2, 1>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, 2, s);
-    // few columns and many rows: 8-column blocks, four chunks per warp (same chunks, same bits, four times the SMs)
+    // few columns and many rows: 8-column blocks, four chunks per warp (same chunks, same bits, four times the SMs).
+    // Against 32 columns: 4.3 / 8.9 us at 512 x 512, 7.9 / 11.4 at 512 x 2048, 14.8 / 13.0 at 512 x 4096
     const int blocks = (N + 31) / 32;
     if (blocks < sms / 2 && T >= 4 * 8)
         return launch_t<1, 8, 4>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, 32, s);
-    // several blocks per SM load, chain and store at different times; one per SM takes as many rows as it can
+    // several blocks per SM load, chain and store at different times; one per SM takes as many rows as it can: 8 / 32 chunk
+    // rows per step at 512 x 4096 (128 blocks) 17.9 / 13.0 us, 128 x 18976 (593) 11.3 / 12.5, 128 x 75648 34 / 39
     return launch_t<1, 8, 1>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, blocks >= 4 * sms ? 8 : 32, s);
 }
 

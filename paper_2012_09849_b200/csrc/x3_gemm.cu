@@ -80,10 +80,11 @@ __device__ __forceinline__ void acc_release(uint64_t* empty_bar, int lane)
 // issues, then eight epilogue warps, two per lane quarter with 32 columns each.  Two accumulators of 192 columns take
 // pairs of B stages (128 of K) in turn; the epilogue adds each to the tile's sum in registers (see "Accumulation" in
 // x3_gemm.cuh).
-// Bound: the tensor core, which spends (128 + N) / 4 clocks (shared-memory operand fetch) or N / 2 on an
-// instruction: 96 + 64 + 48 = 208 clocks per 16 of K for 64 output columns, against 288 for six separate
-// 128 x 64 instructions.  An A entry (all planes, rows 128 + spread) is loaded once per tile and every tap reads it
-// shifted; B is streamed.
+// The tensor core spends (128 + N) / 4 clocks (shared-memory operand fetch) or N / 2 on an instruction:
+// 96 + 64 + 48 = 208 clocks per 16 of K for 64 output columns, against 288 for six separate 128 x 64 instructions.
+// It is busy for 33 / 44 / 42 % of the time (gradients of conv3's / conv2's / conv1's output, n = 1024, 84 x 84: 34 / 49 /
+// 51 us alone) and no other unit for more than half: one thread issues, an instruction every 55 to 70 clocks at best.
+// An A entry (all planes, rows 128 + spread) is loaded once per tile and every tap reads it shifted; B is streamed.
 constexpr int kAccs = 2, kPart = 2, kThreads = 64 + 256;
 __global__ void __launch_bounds__(kThreads)
 x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const X3TapParams p)
@@ -249,8 +250,9 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 // The sets of kind 0 also sum the columns of B (bias gradient).
 // Both operands have the contracted index along their rows (pixels), so tiles go from global memory to the tensor
 // core without a transposition; a tap is a row offset into the slab, and the two taps (or slabs) of a group are two
-// 64-row blocks of M at a free distance (the leading byte offset).  Bound: the tensor core, 208 clocks per 16 rows and
-// group (56 for frames).
+// 64-row blocks of M at a free distance (the leading byte offset).  Tensor core: 208 clocks per 16 rows and group (56 for
+// frames); busy for 51 / 54 / 50 % of the time (dense, conv3, conv2 at n = 1024: 32 / 45 / 48 us alone), shared memory
+// for as much, DRAM 9 / 19 / 31 %.
 constexpr int kWgradThreads = 96 + 256;
 template <int APL, int NB>
 __global__ void __launch_bounds__(kWgradThreads)
