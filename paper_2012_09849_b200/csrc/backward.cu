@@ -600,12 +600,8 @@ hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, 
     const int sms = t->sms;
     {
         const size_t smem = (size_t)(g.A + 1) * 2048;
-        static size_t smem_set_by_device[kDeviceSlots] = {};
-        size_t& smem_set = smem_set_by_device[device_slot()];
-        if (smem > 40 * 1024 && smem > smem_set) {
-            HTS_CUDA(cudaFuncSetAttribute(head_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            smem_set = smem;
-        }
+        static OncePerDevice allowed;
+        HTS_CUDA(allow_shared(head_backward_kernel, allowed, false));
         const int blocks = n < sms ? n : (int)nblk(N, 8) < sms ? sms : (int)nblk(N, 8) < 4 * sms ? (int)nblk(N, 8) : 4 * sms;
         HTS_CUDA(launch_pdl(head_backward_kernel, dim3(blocks), dim3(256), smem, s, t->logits, t->val, actions, adv, ret, logp_old, w.whead, ws.h,
                             value_coef, entropy_coef, clip, n, g.A, t->status, t->dhead, t->dh, ph));

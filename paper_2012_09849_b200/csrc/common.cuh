@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
+#include <atomic>
 #include <stdint.h>
 #include <utility>
 #include "hts.h"
@@ -69,6 +70,24 @@ inline int device_sm_count(int slot)
         else cudaGetLastError();
     }
     return count[slot] > 0 ? count[slot] : 1;
+}
+// Dynamic shared memory and carve-out of a kernel, once per device.  Always as much as the kernel can have: contexts in
+// several threads launch it with sizes of their own, and a limit set to one's size could lower what another relies on.
+using OncePerDevice = std::atomic<bool>[kDeviceSlots];
+template <typename K>
+inline cudaError_t allow_shared(K* kernel, OncePerDevice& done, bool carveout = true)
+{
+    std::atomic<bool>& d = done[device_slot()];
+    if (d.load(std::memory_order_acquire)) return cudaSuccess;
+    int dev = 0, most = 0;
+    cudaFuncAttributes own;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&own, kernel);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)own.sharedSizeBytes);
+    if (e == cudaSuccess && carveout) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e == cudaSuccess) d.store(true, std::memory_order_release);
+    return e;
 }
 
 // Executor-facing addressing of a step (state buffer -> actors -> storage row, Section 4.1): row e of the

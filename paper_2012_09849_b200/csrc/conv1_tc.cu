@@ -427,15 +427,10 @@ template <int CG, int WC>
 hts_status launch_variant(const CUtensorMap& weight_map, const CUtensorMap& frame_map, const Conv1Params& p, int grid,
                           int smem_bytes, bool dependent, cudaStream_t s)
 {
-    static int smem_set_by_device[kDeviceSlots] = {};
-    int& smem_set = smem_set_by_device[device_slot()];
-    if (smem_set < smem_bytes) {
-        HTS_CUDA(cudaFuncSetAttribute(conv1_march_kernel<CG, WC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes));
-        // every kernel of the step asks for the largest shared-memory carve-out, so that the SMs are not
-        // re-partitioned between consecutive kernels
-        HTS_CUDA(cudaFuncSetAttribute(conv1_march_kernel<CG, WC>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        smem_set = smem_bytes;
-    }
+    // every kernel of the step asks for the largest shared-memory carve-out, so that the SMs are not
+    // re-partitioned between consecutive kernels
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(conv1_march_kernel<CG, WC>, allowed));
     HTS_CUDA(launch_chained(dependent, conv1_march_kernel<CG, WC>, dim3(grid), dim3(threads_of<CG>()), (size_t)smem_bytes, s, weight_map, frame_map, p));
     note_launch();
     return HTS_OK;

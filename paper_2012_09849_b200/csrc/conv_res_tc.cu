@@ -183,17 +183,12 @@ hts_status conv_res_launch(const CUtensorMap& act_map, const CUtensorMap& weight
 {
     const int dev = device_slot();
     const int sm_count = device_sm_count(dev);
-    static int smem_set_by_device[kDeviceSlots] = {};
-    int& smem_set = smem_set_by_device[dev];
     constexpr int NST = CPT == 2 ? 4 : 6;        // activation tiles in the ring: two being multiplied, the rest in flight
     const int smem = conv_res_smem_bytes(TAPS, CPT, p.tile_rows);
     if (smem > 227 * 1024) return HTS_ERR_SHAPE;
     if (p.P_in < 1 || p.P_in > 2048 || p.W_in < 1 || p.W_in > 64) return HTS_ERR_SHAPE;   // the epilogue's row arithmetic
-    if (smem > smem_set) {
-        HTS_CUDA(cudaFuncSetAttribute(conv_res_kernel<TAPS, CPT, NST>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        HTS_CUDA(cudaFuncSetAttribute(conv_res_kernel<TAPS, CPT, NST>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        smem_set = smem;
-    }
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(conv_res_kernel<TAPS, CPT, NST>, allowed));
     const int tiles = (p.total_rows + 127) / 128;
     const int grid = tiles < sm_count ? tiles : sm_count;
     HTS_CUDA(launch_pdl(conv_res_kernel<TAPS, CPT, NST>, dim3(grid), dim3(kThreads), (size_t)smem, s, act_map, weight_map, p));

@@ -346,13 +346,8 @@ template <int WC>
 hts_status launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const ConvStackParams& p, int smem, int grid,
                   bool dependent, cudaStream_t s)
 {
-    static int smem_set_by_device[kDeviceSlots] = {};
-    int& smem_set = smem_set_by_device[device_slot()];
-    if (smem > smem_set) {
-        HTS_CUDA(cudaFuncSetAttribute(conv_stack_kernel<WC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        HTS_CUDA(cudaFuncSetAttribute(conv_stack_kernel<WC>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        smem_set = smem;
-    }
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(conv_stack_kernel<WC>, allowed));
     HTS_CUDA(launch_chained(dependent, conv_stack_kernel<WC>, dim3(grid), dim3(kStackThreads), (size_t)smem, s, w1, w2, w3, p));
     note_launch();
     return HTS_OK;

@@ -231,19 +231,8 @@ hts_status launch_heads(const float* h_partials, int num_splits, size_t split_st
     const int sm_count = device_sm_count(dev);
     const uint32_t k0 = (uint32_t)(seed & 0xffffffffu), k1 = (uint32_t)(seed >> 32);
     auto launch = [&](auto kernel, int which, int per_sm) -> hts_status {
-        static size_t smem_set_by_device[3][kDeviceSlots] = {};
-        static bool carveout_set_by_device[3][kDeviceSlots] = {};
-        size_t& smem_set = smem_set_by_device[which][dev];
-        bool& carveout_set = carveout_set_by_device[which][dev];
-        if (smem_set == 0) smem_set = 48 * 1024;        // what a kernel may use without asking
-        if (!carveout_set) {
-            HTS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-            carveout_set = true;
-        }
-        if (smem > smem_set) {
-            HTS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            smem_set = smem;
-        }
+        static OncePerDevice allowed[3];
+        HTS_CUDA(allow_shared(kernel, allowed[which]));
         // one block per SM until every warp has a row, then as many as are resident together
         int blocks = sm_count;
         while (blocks < per_sm * sm_count && n > 8 * blocks) blocks += sm_count;

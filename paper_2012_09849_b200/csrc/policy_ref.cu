@@ -346,13 +346,8 @@ hts_status launch_conv_small(const ConvParams& p, cudaStream_t s)
     const int most = blocks <= sms ? 12 : blocks <= 2 * sms ? 8 : blocks <= 3 * sms ? 5 : blocks <= 4 * sms ? 4 : 3;
     const int groups = p.C * p.k * p.k / kSmallK, ring = groups < most ? groups : most;
     const int smem = ring * (kSmallPx + kSmallOc) * kSmallPitch * (int)sizeof(float);
-    static int smem_set_by_device[kDeviceSlots] = {};
-    int& smem_set = smem_set_by_device[device_slot()];
-    if (smem > smem_set) {
-        HTS_CUDA(cudaFuncSetAttribute(conv_small_kernel<TIn>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        HTS_CUDA(cudaFuncSetAttribute(conv_small_kernel<TIn>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        smem_set = smem;
-    }
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(conv_small_kernel<TIn>, allowed));
     HTS_CUDA(launch_pdl(conv_small_kernel<TIn>, dim3((unsigned)((px + kSmallPx - 1) / kSmallPx), (unsigned)(p.O / kSmallOc)), dim3(128),
                         (size_t)smem, s, p, ring));
     note_launch();
@@ -366,13 +361,8 @@ hts_status launch_conv_tile(const ConvParams& p, cudaStream_t s)
     const int K = p.C * p.k * p.k;
     const size_t smem = sizeof(float) * (2 * KC * PX + 2 * KC * OC) + sizeof(int) * (size_t)(K / (std::is_same<TIn, uint8_t>::value ? 4 : 1));
     auto kernel = conv_tile_kernel<TIn, PXT, OT, WPX, WO, KC, PER_SM>;
-    static size_t smem_set_by_device[kDeviceSlots] = {};
-    size_t& smem_set = smem_set_by_device[device_slot()];
-    if (smem > smem_set) {
-        HTS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        HTS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        smem_set = smem;
-    }
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(kernel, allowed));
     const size_t px = (size_t)p.n * p.Ho * p.Wo;
     HTS_CUDA(launch_pdl(kernel, dim3((unsigned)((px + PX - 1) / PX), (unsigned)(p.O / OC)), dim3(NT), smem, s, p));
     note_launch();
@@ -502,13 +492,8 @@ hts_status launch_fc_chain(const float* x, const float* w, const float* b, float
 {
     constexpr int smem = STAGES * (TE * WE + TO * WO) * COLS * 4;
     auto kernel = fc_chain_kernel<TE, TO, WE, WO, STAGES, COLS>;
-    static bool set_by_device[kDeviceSlots] = {};
-    bool& set = set_by_device[device_slot()];
-    if (!set) {
-        HTS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        HTS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        set = true;
-    }
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(kernel, allowed));
     HTS_CUDA(launch_pdl(kernel, dim3(512 / (TO * WO), (unsigned)((n + TE * WE - 1) / (TE * WE))), dim3(32 * WE * WO), (size_t)smem, s,
                         x, w, b, h, n, F, ((uintptr_t)w & 15) == 0));
     note_launch();

@@ -624,13 +624,8 @@ template <int BN, int EPI>
 hts_status launch_gemm(const CUtensorMap& a, const CUtensorMap& b, const GemmParams& p, dim3 grid, cudaStream_t s)
 {
     constexpr int smem = STAGES * (A_BYTES + BN * BK * 2) + 1024;
-    static bool attr_set_by_device[kDeviceSlots] = {};
-    bool& attr_set = attr_set_by_device[device_slot()];
-    if (!attr_set) {
-        HTS_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        HTS_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        attr_set = true;
-    }
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(gemm_tc_kernel<BN, EPI>, allowed));
     HTS_CUDA(launch_pdl(gemm_tc_kernel<BN, EPI>, grid, dim3(192), (size_t)smem, s, a, b, p));
     note_launch();
     return HTS_OK;
@@ -640,13 +635,8 @@ hts_status launch_fc_resident(const CUtensorMap& a, const CUtensorMap& b, const 
                               cudaStream_t s)
 {
     constexpr int smem = FCB_MAX_NK * 128 * BK * 2 + FCB_STAGES * A_BYTES + FCB_STAGE_FLOATS * 4 + 1024;
-    static bool attr_set_by_device[kDeviceSlots] = {};
-    bool& attr_set = attr_set_by_device[device_slot()];
-    if (!attr_set) {
-        HTS_CUDA(cudaFuncSetAttribute(fc_resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        HTS_CUDA(cudaFuncSetAttribute(fc_resident_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        attr_set = true;
-    }
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(fc_resident_kernel, allowed));
     HTS_CUDA(launch_pdl(fc_resident_kernel, dim3(4, ranges, slots), dim3(192), (size_t)smem, s, a, b, p));
     note_launch();
     return HTS_OK;
@@ -844,13 +834,8 @@ hts_status tc_forward(TcState* t, const uint8_t* obs, const Indexing& ix, int n,
     t->h_final = (long)nblk(n, BM) * 4 >= 64;
     if (t->h_final) {
         constexpr int smem = FCL_STAGES * (A_BYTES + 128 * BK * 2) + 1024;
-        static bool attr_set_by_device[kDeviceSlots] = {};
-        bool& attr_set = attr_set_by_device[device_slot()];
-        if (!attr_set) {
-            HTS_CUDA(cudaFuncSetAttribute(fc_ranges_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-            HTS_CUDA(cudaFuncSetAttribute(fc_ranges_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-            attr_set = true;
-        }
+        static OncePerDevice allowed;
+        HTS_CUDA(allow_shared(fc_ranges_kernel, allowed));
         const FclParams fp{t->splits, t->cps, n, t->bfc, t->inv_scale + L_FC, t->h, t->status};
         HTS_CUDA(launch_pdl(fc_ranges_kernel, dim3(nblk(n, BM), 4), dim3(FCL_THREADS), (size_t)smem, s, t->mAfc, t->mBfc, fp));
         note_launch();

@@ -481,15 +481,10 @@ bool x3_taps_plan(X3TapParams* p, int chunks, int taps, const int* shift)
 
 hts_status x3_dgrad_launch(const CUtensorMap& a, const CUtensorMap& b, const X3TapParams& p, cudaStream_t s)
 {
-    const int dev = device_slot();
-    static bool attr_set[kDeviceSlots] = {};
-    if (!attr_set[dev]) {
-        HTS_CUDA(cudaFuncSetAttribute(x3_dgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 2048));
-        HTS_CUDA(cudaFuncSetAttribute(x3_dgrad_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        attr_set[dev] = true;
-    }
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(x3_dgrad_kernel, allowed));
     const int smem = 1024 + p.entries * ((3 * p.entry_rows * 128 + 1023) & ~1023) + p.b_stages * 3 * 8192;
-    const int tiles = p.m_tiles * p.n_tiles, sms = device_sm_count(dev);
+    const int tiles = p.m_tiles * p.n_tiles, sms = device_sm_count(device_slot());
     HTS_CUDA(launch_pdl(x3_dgrad_kernel, dim3(tiles < sms ? tiles : sms), dim3(kThreads), (size_t)smem, s, a, b, p));
     note_launch();
     return HTS_OK;
@@ -498,13 +493,8 @@ hts_status x3_dgrad_launch(const CUtensorMap& a, const CUtensorMap& b, const X3T
 template <int APL, int NB>
 hts_status x3_wgrad_launch(const CUtensorMap& a, const CUtensorMap& b, const X3WgradParams& p, cudaStream_t s)
 {
-    const int dev = device_slot();
-    static bool attr_set[kDeviceSlots] = {};
-    if (!attr_set[dev]) {
-        HTS_CUDA(cudaFuncSetAttribute(x3_wgrad_kernel<APL, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 3072));
-        HTS_CUDA(cudaFuncSetAttribute(x3_wgrad_kernel<APL, NB>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        attr_set[dev] = true;
-    }
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(x3_wgrad_kernel<APL, NB>, allowed));
     const int a_slab = (APL * p.a_rows * 128 + 1023) & ~1023, b_slab = (NB == 64 ? 3 : 1) * kX3StageRows<NB> * 128;
     const int smem = 1024 + p.stages * (p.n_a * a_slab + p.n_b * b_slab);
     if (smem > kSmemMax - 3072) return HTS_ERR_SHAPE;     // the rest is the kernel's static share
