@@ -78,6 +78,7 @@ struct Conv1Params {
     const float* bias;
     const float* inv_scale;
     __half* out;
+    size_t out_row;         // elements of out from one of its grid rows to the next
     int* status;
 };
 
@@ -333,14 +334,14 @@ conv1_march_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                 const int q = w.tile * kTileCols + 31 * qq + lane;
                 const int e = q / pl.Ws, X = q - e * pl.Ws;
                 rows = lane < 31 && e < p.n && X < pl.W1 ? pl.H1 - w.y_base : 0;
-                dst0 = p.out + ((size_t)e * pl.P1s + (X >> 1)) * 128 + (X & 1) * 32;
+                dst0 = p.out + ((size_t)e * pl.W1s + (X >> 1)) * 128 + (X & 1) * 32;
             }
             const int y = w.y_base + w.pos;
             const int acc = k % NACC;
             if (!mbar_wait_warp(&d_full[acc], ((uint32_t)(k / NACC)) & 1u, abortp, p.status, 37)) break;
             tc_fence_after();
             const uint32_t taddr = tmem_d + acc * 64 + ((uint32_t)(qq * 32) << 16);
-            __half* dst = dst0 + ((size_t)(y >> 1) * pl.W1s) * 128 + (y & 1) * 64;
+            __half* dst = dst0 + (size_t)(y >> 1) * p.out_row + (y & 1) * 64;
             if constexpr (kThreads * S::PER_SM <= 768) {
                 // registers allow it: the whole accumulator row in one round trip to tensor memory
                 uint32_t v0[32], v1[32];
@@ -465,7 +466,7 @@ bool conv1_plan(const Geometry& g, Conv1Plan* pl)
 }
 
 hts_status conv1_launch(const Conv1Plan& pl, const CUtensorMap& weight_map, Conv1MapCache& maps, const uint8_t* obs,
-                        const Indexing& ix, int n, const float* bias, const float* inv_scale, __half* out, int* status,
+                        const Indexing& ix, int n, const float* bias, const float* inv_scale, __half* out, int env_rows, int* status,
                         bool dependent, cudaStream_t s)
 {
     const int sm_count = device_sm_count(device_slot());
@@ -491,7 +492,7 @@ hts_status conv1_launch(const Conv1Plan& pl, const CUtensorMap& weight_map, Conv
     const int max_grid = (pl.CG == 1 ? Shape<1>::PER_SM : 1) * sm_count;
     p.su = choose_rows(p.tiles, pl.H1, max_grid);
     p.splits = (pl.H1 + p.su - 1) / p.su;
-    p.bias = bias; p.inv_scale = inv_scale; p.out = out; p.status = status;
+    p.bias = bias; p.inv_scale = inv_scale; p.out = out; p.out_row = (size_t)env_rows * pl.W1s * 128; p.status = status;
     const long units = (long)p.tiles * p.splits;
     const int grid = units < max_grid ? (int)units : max_grid;
     const CUtensorMap& fm = maps.map[slot];

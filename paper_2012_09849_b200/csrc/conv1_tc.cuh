@@ -39,12 +39,12 @@ struct Conv1MapCache {
 bool conv1_plan(const Geometry& g, Conv1Plan* plan);
 
 // weight_map: w1 packed [128][16*C] fp16, scaled: row dy*64 + dx*32 + o, column c*16 + uy*4 + ux  holds  w1[o][c][4dy+uy][4dx+ux]
-// out: fp16 rows [env*P1s + (y/2)*W1s + x/2][128], column ((y%2)*2 + x%2)*32 + o
+// out: fp16 rows [((y/2)*env_rows + env)*W1s + x/2][128], column ((y%2)*2 + x%2)*32 + o; env_rows: environments of the workspace
 // ix: dense frames (row e = frame e of obs) or frames gathered by slot from a pool (see Indexing)
 // dependent: the kernel loads the filter and biases before it waits for its predecessor, so it may start early only
 // where that is not the one that packed them
 hts_status conv1_launch(const Conv1Plan& pl, const CUtensorMap& weight_map, Conv1MapCache& maps, const uint8_t* obs,
-                        const Indexing& ix, int n, const float* bias, const float* inv_scale, __half* out, int* status,
+                        const Indexing& ix, int n, const float* bias, const float* inv_scale, __half* out, int env_rows, int* status,
                         bool dependent, cudaStream_t s);
 
 }  // namespace hts

@@ -1,20 +1,24 @@
 // conv2 / conv3 of the policy-value network as a persistent tcgen05 kernel.
 //
-// A stride-1 convolution on the flat pixel grid is a sum over filter taps of row-shifted GEMMs
-//     D[m, o] = sum_tap sum_c X[m + dy*W_in + dx, c] * W[o, tap, c].
-// Each CTA keeps the whole packed filter in shared memory and walks over 128-row tiles of the
-// activation matrix.  For a tile it loads rows [m0, m0 + 128 + largest shift) ONCE (one TMA box
-// per 64-channel plane, 128-byte swizzle) and every tap reads the same tile through a shared-
-// memory descriptor whose start address is moved by `shift` rows: the swizzle is a function of
-// the address bits, so a start that is a multiple of 128 bytes keeps the pattern intact.
-// Activation tiles sit in a ring; four accumulators live in tensor memory.  Two warps issue MMAs,
-// warp g for the CTA's tiles g, g+2, ... into accumulators g and g+2 in turn, and each accumulator
-// has its own four epilogue warps, so copies, MMAs and epilogues of different tiles overlap.
-// Measured: a 128x64x16 MMA occupies the tensor core for 48 clocks (128 + 64 operand rows of 32
-// bytes from shared memory at 128 bytes per clock), one thread issues one every 70 to 100 clocks,
-// and one epilogue takes about 2300 clocks per tile; two issuers keep the tensor core busy and
-// four epilogue groups keep the issuers from waiting for an accumulator.  Rows whose pixel lies
-// outside the output extent are computed and dropped by the epilogue.
+// Activations are rows of 64 channels (128 bytes) in the order (y, environment, x).  An M tile is 128 consecutive columns
+// (environment, x) of the batch, and the kernel marches down the grid rows: input row y of a tile is loaded once (one TMA box
+// per 64-channel plane, 128-byte swizzle, KX - 1 columns wider) and contributes to the KY output rows y - KY + 1 .. y.  The
+// filter sits in shared memory with the vertical taps stacked along N, so ONE instruction multiplies the input row by KY taps
+// into KY accumulators that lie side by side in tensor memory; the horizontal taps read the same tile through a descriptor
+// moved by dx rows (128 bytes each; the swizzle follows the address bits).
+//
+// Why: a 128 x 64 x 16 instruction with both operands in shared memory takes 48 clocks (128 + 64 operand rows of 32 bytes at
+// 128 bytes a clock) where its products need 32; with N = 128 fetch and products take 64 clocks each, with N = 192 the
+// products' 96 exceed the fetch.  And no grid row is multiplied that no output needs (conv3: 7 of 9 columns are outputs instead
+// of 49 of 81 grid points).  A sum still runs over (dy, dx, plane, channel) in that order: the bits are those of one tap
+// after the other.  Against one instruction per tap on flat tiles: step of 1024 observations 51.9 -> 48.1 us, of 1733 76.9 ->
+// 71.5, of 8192 243 -> 224 (conv3 46 -> 29; conv2 52 -> 49, where 210 MB of input and 85 of output at 6 TB/s are the bound), of
+// 512 football frames 51.6 -> 51.1.  conv2's instructions take 80 clocks instead of 64 while copies write the same shared memory.
+//
+// Work: output rows of all tiles in a line, cut into one stretch per CTA; a stretch enters each tile it touches with KY - 1
+// rows more than it puts out.  Eight accumulators of 64 columns form a ring over the CTA's output rows; a group of rows that
+// crosses the ring's end takes two instructions.  One thread issues all MMAs (two would have to order their sums), four
+// groups of four warps drain accumulators c, c + 4.
 #include "conv_res_tc.cuh"
 #include "tc_ptx.cuh"
 
@@ -23,9 +27,18 @@ using namespace tc;
 
 namespace {
 
-constexpr int kAcc = 4;                         // accumulators in tensor memory (64 columns each)
-constexpr int kThreads = 128 + kAcc * 128;      // warp 0 copies, warps 1 and 2 issue MMAs, warp 3 idle, then four epilogue warps per accumulator
-constexpr int kChunkBytes = 64 * 128;           // one filter K chunk: 64 output channels x 128 bytes
+constexpr int kRing = 8;                        // accumulators in tensor memory (64 columns each)
+constexpr int kGroups = 4;                      // epilogue groups of four warps
+constexpr int kThreads = 128 + kGroups * 128;   // warp 0 copies, warp 1 issues MMAs, warps 2 and 3 idle, then the epilogues
+constexpr int kPlaneBytes = 17 * 1024;          // one plane of an input row: at most 136 rows of 128 bytes
+
+template <int KY, int KX, int CPT> struct RowsShape {
+    static constexpr int kFilter = KY * KX * CPT * 64 * 128;
+    static constexpr int kStage = CPT * kPlaneBytes;
+    static constexpr int kStages = (226 * 1024 - kFilter) / kStage;
+    static constexpr int kSmem = 1024 + kFilter + kStages * kStage;
+    static_assert(kConvRowsBox<KX> * 128 <= kPlaneBytes && kStages >= 2, "an input row does not fit its stage");
+};
 
 // 256-bit store of eight packed half2 (one 32-byte sector)
 __device__ __forceinline__ void st_global_v8(void* ptr, const uint32_t (&v)[8])
@@ -34,12 +47,14 @@ __device__ __forceinline__ void st_global_v8(void* ptr, const uint32_t (&v)[8])
                  ::"l"(ptr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
 }
 
-template <int TAPS, int CPT, int NST>
+template <int KY, int KX, int CPT>
 __global__ void __launch_bounds__(kThreads)
-conv_res_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, const ConvResParams p)
+conv_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, const ConvRowsParams p)
 {
+    using S = RowsShape<KY, KX, CPT>;
+    constexpr int NST = S::kStages;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t w_bar, a_full[NST], a_empty[NST], d_full[kAcc], d_empty[kAcc];
+    __shared__ uint64_t w_bar, a_full[NST], a_empty[NST], d_full[kRing], d_empty[kRing];
     __shared__ float s_bias[64];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
@@ -47,106 +62,145 @@ conv_res_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* sm = smem_raw + (base - smem_u32(smem_raw));
-    constexpr int w_bytes = TAPS * CPT * kChunkBytes;
-    const int plane_bytes = p.tile_rows * 128;
-    const int a_bytes = CPT * plane_bytes;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles = (p.total_rows + 127) / 128;
+    // this CTA's stretch of output rows (tile, y)
+    const int H = p.H_out, share = p.tiles * H / (int)gridDim.x, extra = p.tiles * H - share * (int)gridDim.x;
+    const int r0 = (int)blockIdx.x * share + min((int)blockIdx.x, extra), total = share + ((int)blockIdx.x < extra);
+    const int tile0 = r0 / H, y0 = r0 - tile0 * H;
 
     if (threadIdx.x == 0) {
         mbar_init(&w_bar, 1);
         for (int b = 0; b < NST; ++b) { mbar_init(&a_full[b], 1); mbar_init(&a_empty[b], 1); }
-        for (int b = 0; b < kAcc; ++b) { mbar_init(&d_full[b], 1); mbar_init(&d_empty[b], 128); }
+        for (int b = 0; b < kRing; ++b) { mbar_init(&d_full[b], 1); mbar_init(&d_empty[b], 4); }
         abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmW);
     }
     if (threadIdx.x >= 64 && threadIdx.x < 128) s_bias[threadIdx.x - 64] = p.bias[threadIdx.x - 64];
-    if (warp == 1) tmem_alloc(&tmem_slot, kAcc * 64);
+    if (warp == 1) tmem_alloc(&tmem_slot, kRing * 64);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_d = tmem_slot;
 
     if (warp == 0 && lane == 0) {                        // the filter does not depend on the previous kernel
-        mbar_arrive_expect_tx(&w_bar, w_bytes);
-        for (int g = 0; g < TAPS * CPT; ++g) tma_load_2d(sm + g * kChunkBytes, &tmW, g * 64, 0, &w_bar);
+        mbar_arrive_expect_tx(&w_bar, S::kFilter);
+        for (int dx = 0; dx < KX; ++dx)
+            for (int pl = 0; pl < CPT; ++pl)
+                for (int dy = 0; dy < KY; ++dy)          // the last filter row first: it belongs to the earliest output row
+                    tma_load_2d(sm + ((dx * CPT + pl) * KY + KY - 1 - dy) * 8192, &tmW, ((dy * KX + dx) * CPT + pl) * 64, 0, &w_bar);
     }
     pdl_wait();
     pdl_trigger();
 
     if (warp == 0) {
         if (lane == 0) {
-            int it = 0;
-            for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
-                const int b = it % NST;
-                if (!mbar_wait(&a_empty[b], (((uint32_t)(it / NST)) & 1u) ^ 1u, abortp, p.status, 21)) break;
-                uint8_t* dst = sm + w_bytes + b * a_bytes;
-                mbar_arrive_expect_tx(&a_full[b], (uint32_t)a_bytes);
-                for (int pl = 0; pl < CPT; ++pl) tma_load_2d(dst + pl * plane_bytes, &tmA, pl * 64, tile * 128, &a_full[b]);
+            int st = 0, tile = tile0, y = y0;            // input row y of the tile
+            uint32_t ph = 1;
+            for (int left = total; left > 0;) {
+                const int cnt = min(left, H - y);        // output rows in this tile
+                int row = y * p.in_plane + tile * 128;
+                for (int i = 0; i < cnt + KY - 1; ++i, row += p.in_plane) {
+                    if (!mbar_wait(&a_empty[st], ph, abortp, p.status, 21)) { left = 0; break; }
+                    uint8_t* dst = sm + S::kFilter + st * S::kStage;
+                    mbar_arrive_expect_tx(&a_full[st], (uint32_t)(CPT * kConvRowsBox<KX> * 128));
+                    for (int pl = 0; pl < CPT; ++pl) tma_load_2d(dst + pl * kPlaneBytes, &tmA, pl * 64, row, &a_full[st]);
+                    if (++st == NST) { st = 0; ph ^= 1u; }
+                }
+                left -= cnt;
+                ++tile;
+                y = 0;
             }
         }
-    } else if (warp <= 2) {
-        if (lane == 0) {
-            // issuing thread g: tiles g, g+2, ... of this CTA, accumulator it % 4 (g, g+2, g, ...)
-            const int g = warp - 1;
-            constexpr uint32_t idesc = instr_desc_f16(0, 128, 64);
-            bool alive = mbar_wait(&w_bar, 0, abortp, p.status, 22);
-            int it = g;
-            for (int tile = blockIdx.x + g * gridDim.x; alive && tile < tiles; tile += 2 * gridDim.x, it += 2) {
-                const int b = it % NST, db = it % kAcc;
-                if (!mbar_wait(&a_full[b], ((uint32_t)(it / NST)) & 1u, abortp, p.status, 23)) break;
-                if (!mbar_wait(&d_empty[db], (((uint32_t)(it / kAcc)) & 1u) ^ 1u, abortp, p.status, 24)) break;
+    } else if (warp == 1) {
+        if (elect_one()) {
+            constexpr uint32_t idesc0 = instr_desc_f16(0, 128, 0);
+            constexpr int KS = KX * CPT * 4;             // K steps of an input row: (dx, plane, 16 channels)
+            // an input row: stage and its phase; its place i in the tile's stretch of cnt output rows, c0 of them before
+            int st = 0, i = 0, c0 = 0, cnt = min(total, H - y0);
+            uint32_t ph = 0;
+            auto start_wait = [&](bool a_there, bool d_there) {
+                if (!a_there && !mbar_wait(&a_full[st], ph, abortp, p.status, 23)) return false;
+                const int cy = c0 + i;
+                return d_there || i >= cnt || mbar_wait(&d_empty[cy % kRing], (((uint32_t)(cy / kRing)) & 1u) ^ 1u, abortp, p.status, 24);
+            };
+            bool alive = mbar_wait(&w_bar, 0, abortp, p.status, 22) && start_wait(false, false);
+            while (alive) {                              // input row i feeds outputs i - KY + 1 .. i
+                const int lo = i - KY + 1 > 0 ? i - KY + 1 : 0, hi = i < cnt ? i : cnt - 1, m = hi - lo + 1;
+                const int slot = (c0 + lo) % kRing;
+                const int m1 = m < kRing - slot ? m : kRing - slot, m2 = m - m1;   // accumulators up to the ring's end, and past it
+                const uint64_t a = smem_desc_sw128(base + S::kFilter + st * S::kStage);
+                const uint64_t b = smem_desc_sw128(base + (KY - 1 - (i - lo)) * 8192);
+                const uint32_t d = tmem_d + slot * 64;
+                auto issue = [&](int kk, uint32_t dd, int skip, int count, uint32_t acc) {
+                    const int g = kk >> 2;
+                    mma_f16_ss(dd, a + (uint32_t)((g % CPT) * (kPlaneBytes >> 4) + (g / CPT) * 8 + 2 * (kk & 3)),
+                               b + (uint32_t)(g * KY * 512 + 2 * (kk & 3)) + (uint64_t)(skip * 512), idesc0 + ((uint32_t)count << 20), acc);
+                };
                 tc_fence_after();
-                const uint32_t a_addr = base + w_bytes + b * a_bytes;
-                const uint32_t d_addr = tmem_d + db * 64;
-#pragma unroll
-                for (int tap = 0; tap < TAPS; ++tap) {
-#pragma unroll
-                    for (int pl = 0; pl < CPT; ++pl) {
-                        const uint64_t adesc = smem_desc_sw128(a_addr + pl * plane_bytes + p.tap_shift[tap] * 128);
-                        const uint64_t bdesc = smem_desc_sw128(base + (tap * CPT + pl) * kChunkBytes);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) mma_f16_ss(d_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (tap | pl | k) != 0);
-                    }
+                if (i < cnt) {                           // output row i starts here: its accumulator takes its first product by itself
+                    const int o1 = m - 1 < m1 ? m - 1 : m1;
+                    if (o1 > 0) issue(0, d, 0, o1, 1);
+                    if (m - 1 > o1) issue(0, tmem_d, o1, m - 1 - o1, 1);
+                    issue(0, tmem_d + ((c0 + i) % kRing) * 64, m - 1, 1, 0);
+                } else {
+                    issue(0, d, 0, m1, 1);
+                    if (m2 > 0) issue(0, tmem_d, m1, m2, 1);
                 }
-                mma_commit(&a_empty[b]);
-                mma_commit(&d_full[db]);
+                if (m2 > 0) {
+#pragma unroll 1                                    // seldom taken: unrolled, its code cost a small batch 0.3 us
+                    for (int kk = 1; kk < KS; ++kk) issue(kk, tmem_d, m1, m2, 1);
+                }
+#pragma unroll
+                for (int kk = 1; kk < KS / 2; ++kk) issue(kk, d, 0, m1, 1);
+                // The next row's barriers are polled while this row's instructions execute: the tensor core takes about four
+                // ahead, and a poll lasts over 100 clocks in the shared memory that it fetches its operands from.
+                const int stage = st, done = i - KY + 1 >= 0 ? (c0 + i - KY + 1) % kRing : -1;
+                if (++st == NST) { st = 0; ph ^= 1u; }
+                if (++i == cnt + KY - 1) { c0 += cnt; i = 0; cnt = min(total - c0, H); }
+                const bool more = c0 < total;
+                bool a_there = false, d_there = false;
+                if (more) {
+                    a_there = mbar_try_wait(&a_full[st], ph);
+                    const int cy = c0 + i;
+                    if (i < cnt) d_there = mbar_try_wait(&d_empty[cy % kRing], (((uint32_t)(cy / kRing)) & 1u) ^ 1u);
+                }
+#pragma unroll
+                for (int kk = KS / 2; kk < KS; ++kk) issue(kk, d, 0, m1, 1);
+                mma_commit(&a_empty[stage]);
+                if (done >= 0) mma_commit(&d_full[done]);
+                alive = more && start_wait(a_there, d_there);
             }
         }
     } else if (warp >= 4) {
-        // four warps per accumulator: group j drains accumulator j, i.e. tiles j, j+4, ... of the CTA
         const int grp = (warp - 4) >> 2;
         const int q = warp & 3;                         // TMEM lane quarter this warp may read
-        const int r = q * 32 + lane;
         const float inv = *p.inv_scale;
-        int it = grp;
-        // Row m of the flat grid = (env, y, x).  The row of this thread advances by the same amount from one of its
-        // tiles to the next, so (env, pix) are carried along with one conditional subtraction per tile instead of
-        // two divisions, and y = pix / W_in is a multiply: with pix < 2048 and W_in <= 64,
-        // (pix * ceil(2^20 / W_in)) >> 20 is exact and the product fits 32 bits (the launcher checks both bounds).
-        const uint32_t first = (uint32_t)(blockIdx.x + grp * gridDim.x) * 128u + (uint32_t)r;
-        const uint32_t stride = (uint32_t)kAcc * gridDim.x * 128u;
-        const int d_env = (int)(stride / (uint32_t)p.P_in), d_pix = (int)(stride - (uint32_t)d_env * (uint32_t)p.P_in);
-        int env = (int)(first / (uint32_t)p.P_in), pix = (int)(first - (uint32_t)env * (uint32_t)p.P_in);
-        const uint32_t w_magic = ((1u << 20) + (uint32_t)p.W_in - 1u) / (uint32_t)p.W_in;
-        for (int tile = blockIdx.x + grp * gridDim.x; tile < tiles; tile += kAcc * gridDim.x, it += kAcc) {
-            if (!mbar_wait_warp(&d_full[grp], ((uint32_t)(it / kAcc)) & 1u, abortp, p.status, 25)) break;
+        int tile = tile0, y = y0 + grp, at = -1;
+        bool valid = false;
+        __half* dst = nullptr;
+        for (int c = grp; c < total; c += kGroups, y += kGroups) {
+            while (y >= H) { y -= H; ++tile; }
+            if (at != tile) {                           // this thread's column of the new tile
+                at = tile;
+                const int col = tile * 128 + q * 32 + lane, env = col / p.W_in, x = col - env * p.W_in;
+                valid = env < p.n_env && x < p.W_out;
+                dst = p.out + (size_t)env * p.out_env + (size_t)x * 64;
+            }
+            const int slot = c % kRing;
+            if (!mbar_wait_warp(&d_full[slot], ((uint32_t)(c / kRing)) & 1u, abortp, p.status, 25)) break;
             tc_fence_after();
-            const int y = (int)(((uint32_t)pix * w_magic) >> 20), x = pix - y * p.W_in;
-            const bool valid = env < p.n_env && y < p.H_out && x < p.W_out;
-            __half* dst = p.out + ((size_t)env * p.P_out + (size_t)y * p.W_out + x) * 64;
-            env += d_env; pix += d_pix;
-            if (pix >= p.P_in) { pix -= p.P_in; ++env; }
             uint32_t v0[32], v1[32];
-            const uint32_t taddr = tmem_d + grp * 64 + ((uint32_t)(q * 32) << 16);
+            const uint32_t taddr = tmem_d + slot * 64 + ((uint32_t)(q * 32) << 16);
             tmem_ld_32x32(taddr, v0);
             tmem_ld_32x32(taddr + 32, v1);
             tmem_ld_wait();
             tc_fence_before();
-            mbar_arrive(&d_empty[grp]);                 // accumulator is in registers: hand it back
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&d_empty[slot]);  // accumulator is in registers: hand it back
             if (valid) {
+                __half* o = dst + (size_t)y * p.out_y;
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
 #pragma unroll
@@ -154,13 +208,13 @@ conv_res_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         uint32_t pk[8];
 #pragma unroll
                         for (int h = 0; h < 8; ++h) {
-                            const int c = j + 2 * h;
-                            float x0 = __uint_as_float(half ? v1[c] : v0[c]);
-                            float x1 = __uint_as_float(half ? v1[c + 1] : v0[c + 1]);
-                            fma2(x0, x1, inv, s_bias[half * 32 + c], s_bias[half * 32 + c + 1]);
+                            const int k = j + 2 * h;
+                            float x0 = __uint_as_float(half ? v1[k] : v0[k]);
+                            float x1 = __uint_as_float(half ? v1[k + 1] : v0[k + 1]);
+                            fma2(x0, x1, inv, s_bias[half * 32 + k], s_bias[half * 32 + k + 1]);
                             pk[h] = relu_pack_h2(x0, x1);     // ReLU, round to fp16, clamp at the largest finite value
                         }
-                        st_global_v8(dst + half * 32 + j, pk);
+                        st_global_v8(o + half * 32 + j, pk);
                     }
                 }
             }
@@ -172,31 +226,25 @@ conv_res_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_d, kAcc * 64);
+    if (warp == 1) tmem_dealloc(tmem_d, kRing * 64);
 }
 
 }  // namespace
 
-template <int TAPS, int CPT>
-hts_status conv_res_launch(const CUtensorMap& act_map, const CUtensorMap& weight_map, const ConvResParams& p,
-                           cudaStream_t s)
+template <int KY, int KX, int CPT>
+hts_status conv_rows_launch(const CUtensorMap& act_map, const CUtensorMap& weight_map, const ConvRowsParams& p, cudaStream_t s)
 {
-    const int dev = device_slot();
-    const int sm_count = device_sm_count(dev);
-    constexpr int NST = CPT == 2 ? 4 : 6;        // activation tiles in the ring: two being multiplied, the rest in flight
-    const int smem = conv_res_smem_bytes(TAPS, CPT, p.tile_rows);
-    if (smem > 227 * 1024) return HTS_ERR_SHAPE;
-    if (p.P_in < 1 || p.P_in > 2048 || p.W_in < 1 || p.W_in > 64) return HTS_ERR_SHAPE;   // the epilogue's row arithmetic
+    using S = RowsShape<KY, KX, CPT>;
+    const int sm_count = device_sm_count(device_slot());
     static OncePerDevice allowed;
-    HTS_CUDA(allow_shared(conv_res_kernel<TAPS, CPT, NST>, allowed));
-    const int tiles = (p.total_rows + 127) / 128;
-    const int grid = tiles < sm_count ? tiles : sm_count;
-    HTS_CUDA(launch_pdl(conv_res_kernel<TAPS, CPT, NST>, dim3(grid), dim3(kThreads), (size_t)smem, s, act_map, weight_map, p));
+    HTS_CUDA(allow_shared(conv_rows_kernel<KY, KX, CPT>, allowed));
+    const int rows = p.tiles * p.H_out, grid = rows < sm_count ? rows : sm_count;
+    HTS_CUDA(launch_pdl(conv_rows_kernel<KY, KX, CPT>, dim3(grid), dim3(kThreads), (size_t)S::kSmem, s, act_map, weight_map, p));
     note_launch();
     return HTS_OK;
 }
 
-template hts_status conv_res_launch<4, 2>(const CUtensorMap&, const CUtensorMap&, const ConvResParams&, cudaStream_t);
-template hts_status conv_res_launch<9, 1>(const CUtensorMap&, const CUtensorMap&, const ConvResParams&, cudaStream_t);
+template hts_status conv_rows_launch<2, 2, 2>(const CUtensorMap&, const CUtensorMap&, const ConvRowsParams&, cudaStream_t);
+template hts_status conv_rows_launch<3, 3, 1>(const CUtensorMap&, const CUtensorMap&, const ConvRowsParams&, cudaStream_t);
 
 }  // namespace hts

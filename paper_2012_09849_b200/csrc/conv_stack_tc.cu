@@ -251,7 +251,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             const bool valid = lane < 31 && y < p.H1 && x < p.W1;
             const int row = (y >> 1) * p.W1s + (x >> 1);
             const uint32_t dst = a1_addr + (y & 1) * p.a1_plane + row * 128, swz = (uint32_t)(row & 7), ch = (uint32_t)((x & 1) * 4 + 2 * h);
-            __half* out = p.a1 + ((size_t)(blockIdx.x + i * gridDim.x) * p.P1s + row) * 128 + (y & 1) * 64 + (x & 1) * 32 + 16 * h;
+            __half* out = p.a1 + ((y >> 1) * p.a1_plane_rows + (size_t)(blockIdx.x + i * gridDim.x) * p.W1s + (x >> 1)) * 128 + (y & 1) * 64 + (x & 1) * 32 + 16 * h;
             const uint32_t taddr = tm + kAcc1 + acc * 64 + lanes;
             if (!mbar_wait_warp(&acc1_full[acc], (uint32_t)(k / kNAcc1) & 1u, abortp, p.status, 53)) break;
             tc_fence_after();
@@ -316,7 +316,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             fence_async_proxy();
             __syncwarp();
             if (lane == 0) mbar_arrive(&a2_full);
-            __half* out = p.a2 + (e * p.P2 + r2) * 64 + 32 * h;
+            __half* out = p.a2 + (y2 * p.a2_plane_rows + e * p.W2 + x2) * 64 + 32 * h;
             if (ok2) { st_global_v8(out, pk[0]); st_global_v8(out + 16, pk[1]); }     // parity tap: after the hand-over
             if (!mbar_wait_warp(&acc3_full, ph, abortp, p.status, 56)) break;
             tc_fence_after();

@@ -19,6 +19,7 @@ struct ConvStackParams {
     const float *b1, *b2, *b3;
     const float *inv1, *inv2, *inv3;    // device scalars undoing the weight scaling (and conv1's /255)
     __half *a1, *a2, *a3;               // workspaces: a3 is the dense layer's input, the others the parity taps
+    size_t a1_plane_rows, a2_plane_rows;    // rows of a1 / a2 from one grid row to the next (all environments of the workspace)
     int* status;
 };
 

@@ -604,8 +604,11 @@ __global__ void __launch_bounds__(256) pack_kernel(const LoadTcParams p)
 }
 
 // ---- parity taps: internal layouts -> fp32 NCHW ----------------------------------------------------
+// Rows of conv1's output (s2d) and conv2's are ordered (y, env, x), `W_rows` to an environment and grid row and env_rows
+// environments to a grid row; conv3's (env, y, x).
+enum { TAP_S2D, TAP_ROWS, TAP_PIXELS };
 __global__ void tap_rows_kernel(const __half* __restrict__ src, float* __restrict__ dst, int n, int Cc,
-                                int Ho, int Wo, int s2d, int P_rows, int W_rows)
+                                int Ho, int Wo, int form, size_t env_rows, int W_rows)
 {
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t total = (size_t)n * Cc * Ho * Wo;
@@ -613,8 +616,9 @@ __global__ void tap_rows_kernel(const __half* __restrict__ src, float* __restric
     const int x = (int)(idx % Wo), y = (int)((idx / Wo) % Ho), c = (int)((idx / ((size_t)Wo * Ho)) % Cc);
     const size_t e = idx / ((size_t)Wo * Ho * Cc);
     size_t off;
-    if (s2d) off = (e * P_rows + (size_t)(y >> 1) * W_rows + (x >> 1)) * (4 * Cc) + ((y & 1) * 2 + (x & 1)) * Cc + c;
-    else off = (e * P_rows + (size_t)y * W_rows + x) * Cc + c;
+    if (form == TAP_S2D) off = (((size_t)(y >> 1) * env_rows + e) * W_rows + (x >> 1)) * (4 * Cc) + ((y & 1) * 2 + (x & 1)) * Cc + c;
+    else if (form == TAP_ROWS) off = (((size_t)y * env_rows + e) * W_rows + x) * Cc + c;
+    else off = ((e * Ho + y) * Wo + x) * Cc + c;
     dst[idx] = __half2float(src[off]);
 }
 
@@ -664,7 +668,6 @@ struct TcState {
     __half *a1s, *a2, *a3;
     float *hpart, *h;
     CUtensorMap mW1, mA2, mB2, mA3, mB3, mAfc, mBfc;
-    int rows2, rows3;           // activation tile rows of conv2 / conv3
     bool stacked;               // the frames fit the kernel that runs all three convolutions
     ConvStackParams stack;
     int* status;
@@ -674,12 +677,9 @@ hts_status tc_check_geometry(const Geometry& g)
 {
     Conv1Plan pl;
     if (!conv1_plan(g, &pl)) return HTS_ERR_SHAPE;
-    const int rows2 = conv_res_tile_rows(pl.W1s + 1), rows3 = conv_res_tile_rows(2 * g.W2 + 2);
-    if (rows2 > 256 || rows3 > 256) return HTS_ERR_SHAPE;                    // TMA box height
-    if (conv_res_smem_bytes(4, 2, rows2) > 227 * 1024 || conv_res_smem_bytes(9, 1, rows3) > 227 * 1024) return HTS_ERR_SHAPE;
     if (g.F % BK) return HTS_ERR_SHAPE;
-    // row arithmetic of the conv2 / conv3 epilogues: grids of at most 2048 pixels, at most 64 wide
-    if (pl.P1s > 2048 || pl.W1s > 64 || g.H2 * g.W2 > 2048 || g.W2 > 64) return HTS_ERR_SHAPE;
+    // the frames this path has been made for: conv2's input grid at most 31 wide (frames of 252 columns) and of 2048 pixels
+    if (pl.P1s > 2048 || pl.W1s > 31) return HTS_ERR_SHAPE;
     return HTS_OK;
 }
 
@@ -716,18 +716,16 @@ hts_status tc_create(const Geometry& g, int max_batch, int* status, TcState** ou
     // cells of an odd-sized s2d border that conv1 never writes must hold finite numbers
     if (cudaMemset(t->a1s, 0, nb * t->P1s * 128 * 2) != cudaSuccess) { delete t; return cuda_fail(cudaGetLastError(), "cudaMemset"); }
     if (cudaMemset(t->absmax, 0, (L_COUNT + 1) * sizeof(unsigned)) != cudaSuccess) { delete t; return cuda_fail(cudaGetLastError(), "cudaMemset"); }
-    t->rows2 = conv_res_tile_rows(t->W1s + 1);
-    t->rows3 = conv_res_tile_rows(2 * g.W2 + 2);
-    if (t->rows2 > 256 || t->rows3 > 256) { delete t; return HTS_ERR_SHAPE; }
     const bool ok = make_map(&t->mW1, t->w1p, 128, 16 * g.C, (uint64_t)32 * g.C, 64) &&
-         make_map(&t->mA2, t->a1s, nb * t->P1s, 128, 256, t->rows2) && make_map(&t->mB2, t->w2p, 64, 512, 1024, 64) &&
-         make_map(&t->mA3, t->a2, nb * t->P2, 64, 128, t->rows3) && make_map(&t->mB3, t->w3p, 64, 576, 1152, 64) &&
+         make_map(&t->mA2, t->a1s, nb * t->P1s, 128, 256, kConvRowsBox<2>) && make_map(&t->mB2, t->w2p, 64, 512, 1024, 64) &&
+         make_map(&t->mA3, t->a2, nb * t->P2, 64, 128, kConvRowsBox<3>) && make_map(&t->mB3, t->w3p, 64, 576, 1152, 64) &&
          make_map(&t->mAfc, t->a3, nb, g.F, (uint64_t)g.F * 2, BM) && make_map(&t->mBfc, t->wfcp, 512, g.F, (uint64_t)g.F * 2, 128);
     if (!ok) { delete t; return HTS_ERR_CUDA; }
     t->stack = ConvStackParams{};
     t->stacked = conv_stack_plan(g, &t->stack);
     ConvStackParams& cs = t->stack;
     cs.b1 = t->b1; cs.b2 = t->b2; cs.b3 = t->b3; cs.inv1 = t->inv_scale + L_CONV1; cs.inv2 = t->inv_scale + L_CONV2; cs.inv3 = t->inv_scale + L_CONV3;
+    cs.a1_plane_rows = nb * t->W1s; cs.a2_plane_rows = nb * g.W2;
     cs.a1 = t->a1s; cs.a2 = t->a2; cs.a3 = t->a3; cs.status = status;
     *out = t;
     return HTS_OK;
@@ -797,28 +795,29 @@ hts_status tc_forward(TcState* t, const uint8_t* obs, const Indexing& ix, int n,
         prof.end(K_CONV1, s);
     } else {
         prof.begin(K_CONV1, s);
-        st = conv1_launch(t->pl1, t->mW1, t->maps1, obs, ix, n, t->b1, t->inv_scale + L_CONV1, t->a1s, t->status, dependent, s);
+        st = conv1_launch(t->pl1, t->mW1, t->maps1, obs, ix, n, t->b1, t->inv_scale + L_CONV1, t->a1s, t->max_batch, t->status, dependent, s);
         if (st != HTS_OK) return st;
         prof.end(K_CONV1, s);
 
-        // conv2: 2x2 taps on the s2d grid [H1s, W1s] with 128 channels -> [H2, W2] x 64
-        ConvResParams c{};
+        // conv2: 2x2 taps on the s2d grid [H1s, W1s] with 128 channels -> [H2, W2] x 64, rows (y, env, x) again
+        const size_t nb = (size_t)t->max_batch;
+        ConvRowsParams c{};
         c.status = t->status; c.n_env = n;
-        c.tap_shift[0] = 0; c.tap_shift[1] = 1; c.tap_shift[2] = t->W1s; c.tap_shift[3] = t->W1s + 1;
-        c.tile_rows = t->rows2; c.total_rows = n * t->P1s;
-        c.P_in = t->P1s; c.W_in = t->W1s; c.H_out = g.H2; c.W_out = g.W2; c.P_out = t->P2;
-        c.bias = t->b2; c.out = t->a2; c.inv_scale = t->inv_scale + L_CONV2;
+        c.W_in = t->W1s; c.H_out = g.H2; c.W_out = g.W2; c.in_plane = (int)(nb * t->W1s);
+        c.tiles = (int)nblk((size_t)n * c.W_in, BM);
+        c.bias = t->b2; c.inv_scale = t->inv_scale + L_CONV2;
+        c.out = t->a2; c.out_env = (size_t)g.W2 * 64; c.out_y = nb * g.W2 * 64;
         prof.begin(K_CONV2, s);
-        st = conv_res_launch<4, 2>(t->mA2, t->mB2, c, s);
+        st = conv_rows_launch<2, 2, 2>(t->mA2, t->mB2, c, s);
         if (st != HTS_OK) return st;
         prof.end(K_CONV2, s);
-        // conv3: 3x3 taps on [H2, W2] x 64 -> [H3, W3] x 64
-        for (int dy = 0; dy < 3; ++dy) for (int dx = 0; dx < 3; ++dx) c.tap_shift[dy * 3 + dx] = dy * g.W2 + dx;
-        c.tile_rows = t->rows3; c.total_rows = n * t->P2;
-        c.P_in = t->P2; c.W_in = g.W2; c.H_out = g.H3; c.W_out = g.W3; c.P_out = t->P3;
-        c.bias = t->b3; c.out = t->a3; c.inv_scale = t->inv_scale + L_CONV3;
+        // conv3: 3x3 taps on [H2, W2] x 64 -> [H3, W3] x 64, an environment's pixels together: a row of the dense layer's input
+        c.W_in = g.W2; c.H_out = g.H3; c.W_out = g.W3; c.in_plane = (int)(nb * g.W2);
+        c.tiles = (int)nblk((size_t)n * c.W_in, BM);
+        c.bias = t->b3; c.inv_scale = t->inv_scale + L_CONV3;
+        c.out = t->a3; c.out_env = (size_t)g.F; c.out_y = (size_t)g.W3 * 64;
         prof.begin(K_CONV3, s);
-        st = conv_res_launch<9, 1>(t->mA3, t->mB3, c, s);
+        st = conv_rows_launch<3, 3, 1>(t->mA3, t->mB3, c, s);
         if (st != HTS_OK) return st;
         prof.end(K_CONV3, s);
     }
@@ -874,11 +873,11 @@ hts_status tc_read_activation(TcState* t, int layer, int n, float* out, cudaStre
         return HTS_OK;
     }
     if (layer == 1)
-        tap_rows_kernel<<<nblk((size_t)n * 32 * g.H1 * g.W1, 256), 256, 0, s>>>(t->a1s, out, n, 32, g.H1, g.W1, 1, t->P1s, t->W1s);
+        tap_rows_kernel<<<nblk((size_t)n * 32 * g.H1 * g.W1, 256), 256, 0, s>>>(t->a1s, out, n, 32, g.H1, g.W1, TAP_S2D, t->max_batch, t->W1s);
     else if (layer == 2)
-        tap_rows_kernel<<<nblk((size_t)n * 64 * g.H2 * g.W2, 256), 256, 0, s>>>(t->a2, out, n, 64, g.H2, g.W2, 0, t->P2, g.W2);
+        tap_rows_kernel<<<nblk((size_t)n * 64 * g.H2 * g.W2, 256), 256, 0, s>>>(t->a2, out, n, 64, g.H2, g.W2, TAP_ROWS, t->max_batch, g.W2);
     else
-        tap_rows_kernel<<<nblk((size_t)n * 64 * g.H3 * g.W3, 256), 256, 0, s>>>(t->a3, out, n, 64, g.H3, g.W3, 0, t->P3, g.W3);
+        tap_rows_kernel<<<nblk((size_t)n * 64 * g.H3 * g.W3, 256), 256, 0, s>>>(t->a3, out, n, 64, g.H3, g.W3, TAP_PIXELS, 0, 0);
     HTS_LAUNCH_CHECK("tap_rows_kernel");
     return HTS_OK;
 }
