@@ -6,10 +6,9 @@
 // A k x k / s convolution with k = 2s is a 2x2/1 convolution on the space-to-depth(s) image,
 // and a stride-1 convolution on a flat pixel grid is a sum over taps of row-shifted GEMMs:
 //     D[m, o] = sum_tap sum_c X[m + dy*W_in + dx, c] * W[o, tap, c]
-// computed for every row m of the input grid; rows whose (y, x) fall outside the output extent
-// are discarded by the epilogue.  Every K chunk (64 channels of one tap) is one dense TMA box.
-// The FC layer is the same kernel with one tap and a fixed split of K across CTAs; the split
-// partials are summed in index order by the heads kernel, so nothing depends on the batch size.
+// computed for whole grid rows (conv_res_tc.cu); columns whose x falls outside the output extent are discarded by the epilogue.
+// The FC layer is a GEMM with a fixed split of K into ranges, whose sums are added in index order here, in fc_tc.cu or by
+// the heads kernel, so nothing depends on the batch size.
 //
 // Operand type.  Both MMA operands are fp16 (kind::f16, fp32 accumulation).  The caller's bf16
 // weights are multiplied by a per-layer power of two that brings the largest magnitude just
@@ -26,6 +25,7 @@
 #include "tc_host.cuh"
 #include "conv1_tc.cuh"
 #include "conv_res_tc.cuh"
+#include "fc_tc.cuh"
 #include "conv_stack_tc.cuh"
 
 namespace hts {
@@ -35,157 +35,17 @@ namespace {
 
 constexpr int BM = 128;                 // rows per tile = TMEM lanes
 constexpr int BK = 64;                  // 16-bit elements per K chunk = one 128-byte swizzle row
-constexpr int STAGES = 3;                 // 3 x 32 KiB: two CTAs per SM, so the 224 FC tiles run in one wave
 constexpr int A_BYTES = BM * BK * 2;    // 16 KiB
-enum { EPI_SPLITK = 1 };
 enum { L_CONV1 = 0, L_CONV2, L_CONV3, L_FC, L_COUNT };
-
-struct GemmParams {
-    int taps, cpt;                      // filter taps, K chunks per tap
-    int tap_shift[9];                   // row shift of each tap on the flat input grid
-    int nk;                             // K chunks handled by one CTA (all of them, or one split)
-    int n_env;                          // valid environments (conv) / valid rows (FC)
-    int P_in, W_in, H_out, W_out, P_out;   // conv epilogue geometry (pixels per env, grid widths)
-    const float* bias;
-    const float* inv_scale;             // device scalar: undoes the weight scaling of this layer
-    __half* out_h;                      // conv: rows [env*P_out + y*W_out + x][64]
-    float* out_f32;                     // split-K partials [split][rows][ldo]
-    size_t split_stride;
-    int ldo;
-    int* status;
-};
-
-template <int BN, int EPI>
-__global__ void __launch_bounds__(192)
-gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmParams p)
-{
-    constexpr int B_BYTES = BN * BK * 2;
-    constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    constexpr uint32_t TMEM_COLS = BN < 32 ? 32 : BN;
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[STAGES], empty_bar[STAGES], accum_bar;
-    __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag;
-
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    uint8_t* tiles = smem_raw + (base - smem_u32(smem_raw));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    volatile int* abortp = &abort_flag;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        mbar_init(&accum_bar, 1);
-        abort_flag = 0;
-        fence_barrier_init();
-        tma_prefetch_desc(&tmA);
-        tma_prefetch_desc(&tmB);
-    }
-    if (warp == 1) tmem_alloc(&tmem_base_slot, TMEM_COLS);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_d = tmem_base_slot;
-    // The weight halves of the first stages do not depend on the previous kernel: they are on their way while
-    // this one still waits for it.
-    if (warp == 0 && lane == 0) {
-        for (int kc = 0; kc < p.nk && kc < STAGES; ++kc) {
-            mbar_arrive_expect_tx(&full_bar[kc], STAGE_BYTES);
-            tma_load_2d(tiles + kc * STAGE_BYTES + A_BYTES, &tmB, (blockIdx.z * p.nk + kc) * BK, n0, &full_bar[kc]);
-        }
-    }
-    pdl_wait();
-    pdl_trigger();
-
-    if (warp == 0) {
-        if (lane == 0) {
-            for (int kc = 0; kc < p.nk; ++kc) {
-                const int s = kc % STAGES;
-                const uint32_t ph = (uint32_t)(kc / STAGES) & 1u;
-                if (!mbar_wait(&empty_bar[s], ph ^ 1u, abortp, p.status, 1)) break;
-                const int g = blockIdx.z * p.nk + kc;
-                const int tap = g / p.cpt, sub = g - tap * p.cpt;
-                uint8_t* a_dst = tiles + s * STAGE_BYTES;
-                if (kc >= STAGES) {
-                    mbar_arrive_expect_tx(&full_bar[s], STAGE_BYTES);
-                    tma_load_2d(a_dst + A_BYTES, &tmB, g * BK, n0, &full_bar[s]);
-                }
-                tma_load_2d(a_dst, &tmA, sub * BK, m0 + p.tap_shift[tap], &full_bar[s]);
-            }
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = instr_desc_f16(0, BM, BN);
-            for (int kc = 0; kc < p.nk; ++kc) {
-                const int s = kc % STAGES;
-                const uint32_t ph = (uint32_t)(kc / STAGES) & 1u;
-                if (!mbar_wait(&full_bar[s], ph, abortp, p.status, 2)) break;
-                tc_fence_after();
-                const uint32_t a_addr = base + s * STAGE_BYTES;
-                const uint64_t adesc = smem_desc_sw128(a_addr);
-                const uint64_t bdesc = smem_desc_sw128(a_addr + A_BYTES);
-#pragma unroll
-                for (int k = 0; k < BK / 16; ++k)       // 32 bytes further along the swizzled row per K step
-                    mma_f16_ss(tmem_d, adesc + 2 * k, bdesc + 2 * k, idesc, (kc | k) != 0);
-                mma_commit(&empty_bar[s]);
-            }
-            mma_commit(&accum_bar);
-        }
-    } else {
-        // epilogue warps 2..5: warp w may touch TMEM lanes [32*(w%4), 32*(w%4)+32)
-        const int q = warp & 3;
-        const bool ok = mbar_wait_warp(&accum_bar, 0, abortp, p.status, 3);
-        tc_fence_after();
-        if (ok) {
-            const float inv = *p.inv_scale;
-            {
-                // The accumulator arrives one row per thread; a row-per-thread store would touch 32
-                // lines per instruction.  Each warp turns its 32x32 block through shared memory (the
-                // pipeline stages are free by now) so that eight lanes write one full 128-byte line.
-                float* stage = reinterpret_cast<float*>(tiles) + (warp - 2) * (32 * 36);
-                float* dst = p.out_f32 + blockIdx.z * p.split_stride + (size_t)(m0 + q * 32) * p.ldo + n0;
-                const int rl = lane >> 3, c4 = (lane & 7) * 4;
-#pragma unroll
-                for (int c = 0; c < BN; c += 32) {
-                    uint32_t v[32];
-                    tmem_ld_32x32(tmem_d + ((uint32_t)(q * 32) << 16) + c, v);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int j = 0; j < 32; j += 4)
-                        *reinterpret_cast<float4*>(stage + lane * 36 + j) =
-                            make_float4(__uint_as_float(v[j]) * inv, __uint_as_float(v[j + 1]) * inv,
-                                        __uint_as_float(v[j + 2]) * inv, __uint_as_float(v[j + 3]) * inv);
-                    __syncwarp();
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int rr = 4 * i + rl;
-                        const float4 val = *reinterpret_cast<const float4*>(stage + rr * 36 + c4);
-                        if (m0 + q * 32 + rr < p.n_env) *reinterpret_cast<float4*>(dst + (size_t)rr * p.ldo + c + c4) = val;
-                    }
-                    __syncwarp();
-                }
-            }
-        }
-    }
-    if (*abortp) {                                      // give copies still in flight time to land
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000) { }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_d, TMEM_COLS);
-}
-
 
 // ---- FC for small batches with the weights resident: one CTA per (column tile, K range) and slot of row tiles.
 // A CTA asks for its whole weight slice (nk chunks of 128 x 64) before it waits for the previous kernel; a CTA of
 // this kernel cannot start before the previous kernel's CTA has left its SM, but the hand-over from the last of
 // those to the release of the wait (about 1.4 us) is enough for most of the slice.  After the wait only
 // activations cross the SM's L2 port: 112 KB per row tile instead of 224 KB.  Used while every CTA has one row
-// tile (n <= 640 for 4 x 84 x 84 frames: 31.0 against 31.5 us per step at n = 256, 51.2 against 52.7 us for 512
-// football frames); with two tiles per CTA it only equals the kernel above (one CTA per SM streams less from L2
-// than two do).  K ranges, the order inside them and the partial planes are those of the kernel above: the same
-// bits.
+// tile (n <= 640 for 4 x 84 x 84 frames: 31.0 us per step at n = 256, 31.5 with weights and activations copied together);
+// from there on pairs of SMs (fc_tc.cu) are faster.  K ranges, the order inside them and the partial planes are the same
+// there: the same bits.
 constexpr int FCB_STAGES = 5;                   // activation chunks in flight (16 KiB each)
 constexpr int FCB_MAX_NK = 7;                   // weight chunks a CTA can keep: 7 x 16 KiB
 constexpr int FCB_MAX_TILES = 1;                // row tiles of a CTA (accumulators of 128 columns)
@@ -319,162 +179,6 @@ fc_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_d, FCB_MAX_TILES * BN);
-}
-
-// ---- FC for large batches: all K ranges of a tile in one CTA -----------------------------------------
-// The FC result is defined as  h = relu(bias + p_0 + p_1 + ... + p_{S-1}),  p_s = inv * (sum over the K chunks of
-// range s, accumulated in tensor memory in chunk order), the p_s added in index order in fp32.  Small batches
-// spread the S ranges over S CTAs (gemm_tc_kernel writes the p_s, the heads kernel adds them), which fills the
-// SMs.  Once there are enough 128 x 128 tiles to fill them anyway, one CTA runs the S ranges of its tile back to
-// back, alternating between two accumulators, and its epilogue warps keep the running sum in registers: the same
-// operations in the same order (explicitly rounded multiplies and adds, no fused forms), hence the same bits, but
-// the hidden layer leaves the chip once (2 KB per observation instead of S x 2 KB) and the copy pipeline never
-// drains between ranges.
-constexpr int FCL_STAGES = 6;
-constexpr int FCL_THREADS = 320;          // warp 0 copies, warp 1 issues, warps 2..9 epilogue (two per lane quarter, 64 columns each)
-
-struct FclParams {
-    int splits, cps;                      // K ranges and chunks per range
-    int n;                                // valid rows
-    const float* bias;                    // [512]
-    const float* inv_scale;
-    float* h;                             // [n][512]
-    int* status;
-};
-
-__global__ void __launch_bounds__(FCL_THREADS)
-fc_ranges_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const FclParams p)
-{
-    constexpr int BN = 128;
-    constexpr int B_BYTES = BN * BK * 2;
-    constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[FCL_STAGES], empty_bar[FCL_STAGES], acc_full[2], acc_empty[2];
-    __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag;
-    __shared__ float s_bias[BN];
-
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    uint8_t* tiles = smem_raw + (base - smem_u32(smem_raw));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    volatile int* abortp = &abort_flag;
-    const int total_chunks = p.splits * p.cps;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < FCL_STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&acc_full[a], 1); mbar_init(&acc_empty[a], 8); }
-        abort_flag = 0;
-        fence_barrier_init();
-        tma_prefetch_desc(&tmA);
-        tma_prefetch_desc(&tmB);
-    }
-    if (threadIdx.x >= 64 && threadIdx.x < 64 + BN) s_bias[threadIdx.x - 64] = p.bias[n0 + threadIdx.x - 64];
-    if (warp == 1) tmem_alloc(&tmem_base_slot, 2 * BN);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_d = tmem_base_slot;
-    pdl_wait();
-    pdl_trigger();
-
-    if (warp == 0) {
-        if (lane == 0) {
-            for (int kc = 0; kc < total_chunks; ++kc) {
-                const int s = kc % FCL_STAGES;
-                const uint32_t ph = (uint32_t)(kc / FCL_STAGES) & 1u;
-                if (!mbar_wait(&empty_bar[s], ph ^ 1u, abortp, p.status, 51)) break;
-                uint8_t* a_dst = tiles + s * STAGE_BYTES;
-                mbar_arrive_expect_tx(&full_bar[s], STAGE_BYTES);
-                tma_load_2d(a_dst, &tmA, kc * BK, m0, &full_bar[s]);
-                tma_load_2d(a_dst + A_BYTES, &tmB, kc * BK, n0, &full_bar[s]);
-            }
-        }
-    } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = instr_desc_f16(0, BM, BN);
-            int kc = 0;
-            bool alive = true;
-            for (int sp = 0; alive && sp < p.splits; ++sp) {
-                const int acc = sp & 1;
-                if (!mbar_wait(&acc_empty[acc], (((uint32_t)(sp >> 1)) & 1u) ^ 1u, abortp, p.status, 52)) break;
-                tc_fence_after();
-                for (int c = 0; c < p.cps; ++c, ++kc) {
-                    const int s = kc % FCL_STAGES;
-                    if (!mbar_wait(&full_bar[s], (uint32_t)(kc / FCL_STAGES) & 1u, abortp, p.status, 53)) { alive = false; break; }
-                    tc_fence_after();
-                    const uint32_t a_addr = base + s * STAGE_BYTES;
-                    const uint64_t adesc = smem_desc_sw128(a_addr), bdesc = smem_desc_sw128(a_addr + A_BYTES);
-#pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        mma_f16_ss(tmem_d + acc * BN, adesc + 2 * k, bdesc + 2 * k, idesc, (c | k) != 0);
-                    mma_commit(&empty_bar[s]);
-                }
-                if (alive) mma_commit(&acc_full[acc]);
-            }
-        }
-    } else {
-        // epilogue warps 2..9: lane quarter warp % 4, columns [64 half, 64 half + 64) of the tile
-        const int q = warp & 3, half = (warp - 2) >> 2;
-        const float inv = *p.inv_scale;
-        float sum[64];
-        bool ok = true;
-        for (int sp = 0; ok && sp < p.splits; ++sp) {
-            const int acc = sp & 1;
-            ok = mbar_wait_warp(&acc_full[acc], ((uint32_t)(sp >> 1)) & 1u, abortp, p.status, 54);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t taddr = tmem_d + acc * BN + half * 64 + ((uint32_t)(q * 32) << 16);
-#pragma unroll
-            for (int c = 0; c < 64; c += 32) {
-                uint32_t v[32];
-                tmem_ld_32x32(taddr + c, v);
-                tmem_ld_wait();
-                if (c == 32) {                            // the accumulator is in registers: hand it back
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&acc_empty[acc]);
-                }
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float t = __fmul_rn(__uint_as_float(v[j]), inv);           // p_s, as the split kernel stores it
-                    sum[c + j] = sp == 0 ? t : __fadd_rn(sum[c + j], t);              // added in index order, as the heads kernel does
-                }
-            }
-        }
-        if (ok) {
-            // bias, ReLU, and the block turned through shared memory (the pipeline stages are free by now) so that
-            // eight lanes write one full 128-byte line
-            float* stage = reinterpret_cast<float*>(tiles) + (warp - 2) * (32 * 36);
-            float* dst = p.h + (size_t)(m0 + q * 32) * 512 + n0 + half * 64;
-            const int rl = lane >> 3, c4 = (lane & 7) * 4;
-#pragma unroll
-            for (int c = 0; c < 64; c += 32) {
-#pragma unroll
-                for (int j = 0; j < 32; j += 4)
-                    *reinterpret_cast<float4*>(stage + lane * 36 + j) =
-                        make_float4(fmaxf(__fadd_rn(sum[c + j], s_bias[half * 64 + c + j]), 0.f),
-                                    fmaxf(__fadd_rn(sum[c + j + 1], s_bias[half * 64 + c + j + 1]), 0.f),
-                                    fmaxf(__fadd_rn(sum[c + j + 2], s_bias[half * 64 + c + j + 2]), 0.f),
-                                    fmaxf(__fadd_rn(sum[c + j + 3], s_bias[half * 64 + c + j + 3]), 0.f));
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int rr = 4 * i + rl;
-                    const float4 val = *reinterpret_cast<const float4*>(stage + rr * 36 + c4);
-                    if (m0 + q * 32 + rr < p.n) *reinterpret_cast<float4*>(dst + (size_t)rr * 512 + c + c4) = val;
-                }
-                __syncwarp();
-            }
-        }
-    }
-    if (*abortp) {                                      // give copies still in flight time to land
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000) { }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_d, 2 * BN);
 }
 
 // ---- weight scaling and packing ---------------------------------------------------------------
@@ -624,17 +328,6 @@ __global__ void tap_rows_kernel(const __half* __restrict__ src, float* __restric
 
 inline unsigned nblk(size_t total, int th) { return (unsigned)((total + th - 1) / th); }
 
-template <int BN, int EPI>
-hts_status launch_gemm(const CUtensorMap& a, const CUtensorMap& b, const GemmParams& p, dim3 grid, cudaStream_t s)
-{
-    constexpr int smem = STAGES * (A_BYTES + BN * BK * 2) + 1024;
-    static OncePerDevice allowed;
-    HTS_CUDA(allow_shared(gemm_tc_kernel<BN, EPI>, allowed));
-    HTS_CUDA(launch_pdl(gemm_tc_kernel<BN, EPI>, grid, dim3(192), (size_t)smem, s, a, b, p));
-    note_launch();
-    return HTS_OK;
-}
-
 hts_status launch_fc_resident(const CUtensorMap& a, const CUtensorMap& b, const FcbParams& p, int ranges, int slots,
                               cudaStream_t s)
 {
@@ -656,7 +349,8 @@ struct TcState {
     int splits, cps;            // FC split-K
     bool fresh = false;         // no step has been enqueued since the weights were packed
     unsigned long long fresh_capture = 0;   // the stream capture that packing belongs to, 0 = none
-    bool h_final = false;       // the last forward pass wrote the finished hidden layer (large-batch FC), not partials
+    bool h_final = false;       // the last forward pass wrote the finished hidden layer, not planes to be added up
+    int planes = 0;             // how many of those
     // packed weights
     Conv1Plan pl1;
     Conv1MapCache maps1;
@@ -667,7 +361,7 @@ struct TcState {
     // workspace
     __half *a1s, *a2, *a3;
     float *hpart, *h;
-    CUtensorMap mW1, mA2, mB2, mA3, mB3, mAfc, mBfc;
+    CUtensorMap mW1, mA2, mB2, mA3, mB3, mAfc, mBfc, mBfcPair;
     bool stacked;               // the frames fit the kernel that runs all three convolutions
     ConvStackParams stack;
     int* status;
@@ -719,7 +413,8 @@ hts_status tc_create(const Geometry& g, int max_batch, int* status, TcState** ou
     const bool ok = make_map(&t->mW1, t->w1p, 128, 16 * g.C, (uint64_t)32 * g.C, 64) &&
          make_map(&t->mA2, t->a1s, nb * t->P1s, 128, 256, kConvRowsBox<2>) && make_map(&t->mB2, t->w2p, 64, 512, 1024, 64) &&
          make_map(&t->mA3, t->a2, nb * t->P2, 64, 128, kConvRowsBox<3>) && make_map(&t->mB3, t->w3p, 64, 576, 1152, 64) &&
-         make_map(&t->mAfc, t->a3, nb, g.F, (uint64_t)g.F * 2, BM) && make_map(&t->mBfc, t->wfcp, 512, g.F, (uint64_t)g.F * 2, 128);
+         make_map(&t->mAfc, t->a3, nb, g.F, (uint64_t)g.F * 2, BM) && make_map(&t->mBfc, t->wfcp, 512, g.F, (uint64_t)g.F * 2, 128) &&
+         make_map(&t->mBfcPair, t->wfcp, 512, g.F, (uint64_t)g.F * 2, 64);
     if (!ok) { delete t; return HTS_ERR_CUDA; }
     t->stack = ConvStackParams{};
     t->stacked = conv_stack_plan(g, &t->stack);
@@ -821,35 +516,25 @@ hts_status tc_forward(TcState* t, const uint8_t* obs, const Indexing& ix, int n,
         if (st != HTS_OK) return st;
         prof.end(K_CONV3, s);
     }
-    GemmParams p{};
-    p.status = t->status; p.n_env = n;
-    // FC: [n, F] x [512, F]^T, K split across blockIdx.z
-    p.taps = 1; p.cpt = g.F / BK; p.nk = t->cps; p.tap_shift[0] = 0;
-    p.out_f32 = t->hpart; p.split_stride = (size_t)t->max_batch * 512; p.ldo = 512; p.inv_scale = t->inv_scale + L_FC;
+    // FC: [n, F] x [512, F]^T, K split into ranges.  Weights resident per CTA when a range is at most seven chunks and every
+    // CTA gets one row tile, pairs of SMs otherwise.
     prof.begin(K_FC, s);
-    // From 64 tiles on (n > 1920) one CTA per tile running all K ranges beats spreading the ranges over CTAs
-    // (measured: 89 against 91 us per step at n = 2048, 139 against 166 at n = 4096, 254 against 298 at n = 8192;
-    // at n = 1024 its 32 CTAs would each pull 1.6 MB through one SM's L2 port)
-    t->h_final = (long)nblk(n, BM) * 4 >= 64;
-    if (t->h_final) {
-        constexpr int smem = FCL_STAGES * (A_BYTES + 128 * BK * 2) + 1024;
-        static OncePerDevice allowed;
-        HTS_CUDA(allow_shared(fc_ranges_kernel, allowed));
-        const FclParams fp{t->splits, t->cps, n, t->bfc, t->inv_scale + L_FC, t->h, t->status};
-        HTS_CUDA(launch_pdl(fc_ranges_kernel, dim3(nblk(n, BM), 4), dim3(FCL_THREADS), (size_t)smem, s, t->mAfc, t->mBfc, fp));
-        note_launch();
+    const int m_tiles = (int)nblk(n, BM);
+    int slots = device_sm_count(device_slot()) / (4 * t->splits);
+    if (slots > m_tiles) slots = m_tiles;
+    if (t->cps <= FCB_MAX_NK && slots >= 1 && (m_tiles + slots - 1) / slots <= FCB_MAX_TILES) {
+        const FcbParams fp{t->cps, n, m_tiles, t->inv_scale + L_FC, t->hpart, (size_t)t->max_batch * 512, t->status};
+        t->planes = t->splits;
+        t->h_final = false;
+        st = launch_fc_resident(t->mAfc, t->mBfc, fp, t->splits, slots, s);
     } else {
-        // Weights resident per CTA when a K range is at most seven chunks and every CTA gets one row tile
-        const int m_tiles = (int)nblk(n, BM);
-        int slots = device_sm_count(device_slot()) / (4 * t->splits);
-        if (slots > m_tiles) slots = m_tiles;
-        if (t->cps <= FCB_MAX_NK && slots >= 1 && (m_tiles + slots - 1) / slots <= FCB_MAX_TILES) {
-            const FcbParams fp{t->cps, n, m_tiles, t->inv_scale + L_FC, t->hpart, (size_t)t->max_batch * 512, t->status};
-            st = launch_fc_resident(t->mAfc, t->mBfc, fp, t->splits, slots, s);
-        } else
-            st = launch_gemm<128, EPI_SPLITK>(t->mAfc, t->mBfc, p, dim3(nblk(n, BM), 4, t->splits), s);
-        if (st != HTS_OK) return st;
+        const FcPairPlan plan = fc_pair_plan(n, t->splits);
+        const FcPairParams fp{t->splits, t->cps, plan.group, n, t->bfc, t->inv_scale + L_FC, t->h, t->hpart, (size_t)t->max_batch * 512, t->status};
+        t->planes = plan.planes;
+        t->h_final = plan.planes == 1;
+        st = fc_pair_launch(t->mAfc, t->mBfcPair, fp, plan.wide, s);
     }
+    if (st != HTS_OK) return st;
     prof.end(K_FC, s);
     return HTS_OK;
 }
@@ -861,7 +546,7 @@ hts_status tc_heads(TcState* t, const int32_t* env_ids, const int32_t* t_per_env
     if (t->h_final)        // the FC kernel wrote relu(bias + sum of the K ranges) itself
         return launch_heads(t->h, 1, 0, nullptr, t->whead, t->bhead, t->g.A, env_ids, t_per_env, tt, seed, n, ix, t->status,
                             actions, logp, values, entropy, logits, nullptr, s, given_actions);
-    return launch_heads(t->hpart, t->splits, (size_t)t->max_batch * 512, t->bfc, t->whead, t->bhead, t->g.A, env_ids,
+    return launch_heads(t->hpart, t->planes, (size_t)t->max_batch * 512, t->bfc, t->whead, t->bhead, t->g.A, env_ids,
                         t_per_env, tt, seed, n, ix, t->status, actions, logp, values, entropy, logits, t->h, s, given_actions);
 }
 
