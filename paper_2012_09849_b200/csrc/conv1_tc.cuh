@@ -10,19 +10,11 @@ namespace hts {
 
 struct Conv1Plan {
     int C, H, W;            // observation
-    int CG;                 // groups of four channels (C / 4): 64 K values = 32 tensor-memory columns each
     int Hs, Ws;             // space-to-depth(4) grid
     int H1, W1;             // conv1 output extent (Hs-1, Ws-1)
     int H1s, W1s, P1s;      // space-to-depth(2) grid of the output (input layout of conv2)
-    int env_max;            // environments one tile of 125 grid columns can touch
-    int group_rows;         // grid rows per staged group (one TMA box per environment)
-    int env_bytes;          // bytes of one environment's box: C x group_rows x 4 W
-    int env_pitch;          // its pitch in the staged group (boxes start on 128-byte boundaries)
-    int stage_bytes;        // one staged group: env_max boxes
-    int stages;             // staged groups in the ring
-    int ring;               // operand rows resident in tensor memory
-    int accs;               // accumulators in tensor memory (64 columns each)
-    int smem_bytes;         // dynamic shared memory of the kernel
+    int env_pitch;              // bytes of a box: what a staged entry holds of one environment
+    int stage_bytes, stages;    // a staged entry, and how many of them shared memory holds for each of the kernel's two pipes
 };
 
 // Tensor maps over the caller's frame buffers, keyed by (address, frames): encoding one costs about a

@@ -162,9 +162,9 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const bool more = c0 < total;
                 bool a_there = false, d_there = false;
                 if (more) {
-                    a_there = mbar_try_wait(&a_full[st], ph);
+                    a_there = mbar_test(&a_full[st], ph);
                     const int cy = c0 + i;
-                    if (i < cnt) d_there = mbar_try_wait(&d_empty[cy % kRing], (((uint32_t)(cy / kRing)) & 1u) ^ 1u);
+                    if (i < cnt) d_there = mbar_test(&d_empty[cy % kRing], (((uint32_t)(cy / kRing)) & 1u) ^ 1u);
                 }
 #pragma unroll
                 for (int kk = KS / 2; kk < KS; ++kk) issue(kk, d, 0, m1, 1);
