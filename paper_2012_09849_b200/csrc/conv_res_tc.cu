@@ -54,7 +54,8 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     using S = RowsShape<KY, KX, CPT>;
     constexpr int NST = S::kStages;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t w_bar, a_full[NST], a_empty[NST], d_full[kRing], d_empty[kRing];
+    __shared__ uint64_t bars[1 + 2 * NST + 2 * kRing];
+    uint64_t *w_bar = bars, *a_full = bars + 1, *a_empty = a_full + NST, *d_full = a_empty + NST, *d_empty = d_full + kRing;
     __shared__ float s_bias[64];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
@@ -68,29 +69,28 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const int r0 = (int)blockIdx.x * share + min((int)blockIdx.x, extra), total = share + ((int)blockIdx.x < extra);
     const int tile0 = r0 / H, y0 = r0 - tile0 * H;
 
-    if (threadIdx.x == 0) {
-        mbar_init(&w_bar, 1);
-        for (int b = 0; b < NST; ++b) { mbar_init(&a_full[b], 1); mbar_init(&a_empty[b], 1); }
-        for (int b = 0; b < kRing; ++b) { mbar_init(&d_full[b], 1); mbar_init(&d_empty[b], 4); }
-        abort_flag = 0;
+    // The prologue is on the step's critical path: this CTA gets the SM when the previous kernel's last one leaves it.
+    if (warp == 0) {
+        for (int i = lane; i < 1 + 2 * NST + 2 * kRing; i += 32) mbar_init(&bars[i], i < 1 + 2 * NST + kRing ? 1 : 4);
         fence_barrier_init();
+        __syncwarp();
+        if (lane == 0) {                                 // the filter does not depend on the previous kernel
+            mbar_arrive_expect_tx(w_bar, S::kFilter);
+            for (int dx = 0; dx < KX; ++dx)
+                for (int pl = 0; pl < CPT; ++pl)
+                    for (int dy = 0; dy < KY; ++dy)      // the last filter row first: it belongs to the earliest output row
+                        tma_load_2d(sm + ((dx * CPT + pl) * KY + KY - 1 - dy) * 8192, &tmW, ((dy * KX + dx) * CPT + pl) * 64, 0, w_bar);
+        }
+    } else if (warp == 1) {
+        tmem_alloc(&tmem_slot, kRing * 64);
+    } else if (warp == 2 && lane == 0) {
+        abort_flag = 0;
         tma_prefetch_desc(&tmA);
-        tma_prefetch_desc(&tmW);
     }
-    if (threadIdx.x >= 64 && threadIdx.x < 128) s_bias[threadIdx.x - 64] = p.bias[threadIdx.x - 64];
-    if (warp == 1) tmem_alloc(&tmem_slot, kRing * 64);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_d = tmem_slot;
-
-    if (warp == 0 && lane == 0) {                        // the filter does not depend on the previous kernel
-        mbar_arrive_expect_tx(&w_bar, S::kFilter);
-        for (int dx = 0; dx < KX; ++dx)
-            for (int pl = 0; pl < CPT; ++pl)
-                for (int dy = 0; dy < KY; ++dy)          // the last filter row first: it belongs to the earliest output row
-                    tma_load_2d(sm + ((dx * CPT + pl) * KY + KY - 1 - dy) * 8192, &tmW, ((dy * KX + dx) * CPT + pl) * 64, 0, &w_bar);
-    }
     pdl_wait();
     pdl_trigger();
 
@@ -125,7 +125,7 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const int cy = c0 + i;
                 return d_there || i >= cnt || mbar_wait(&d_empty[cy % kRing], (((uint32_t)(cy / kRing)) & 1u) ^ 1u, abortp, p.status, 24);
             };
-            bool alive = mbar_wait(&w_bar, 0, abortp, p.status, 22) && start_wait(false, false);
+            bool alive = mbar_wait(w_bar, 0, abortp, p.status, 22) && start_wait(false, false);
             while (alive) {                              // input row i feeds outputs i - KY + 1 .. i
                 const int lo = i - KY + 1 > 0 ? i - KY + 1 : 0, hi = i < cnt ? i : cnt - 1, m = hi - lo + 1;
                 const int slot = (c0 + lo) % kRing;
@@ -177,6 +177,9 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int grp = (warp - 4) >> 2;
         const int q = warp & 3;                         // TMEM lane quarter this warp may read
         const float inv = *p.inv_scale;
+        s_bias[lane] = p.bias[lane];                    // every epilogue warp writes the same
+        s_bias[32 + lane] = p.bias[32 + lane];
+        __syncwarp();
         int tile = tile0, y = y0 + grp, at = -1;
         bool valid = false;
         __half* dst = nullptr;

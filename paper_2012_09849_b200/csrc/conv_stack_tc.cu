@@ -78,8 +78,11 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
                   const __grid_constant__ CUtensorMap tmW3, const ConvStackParams p)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t w_bar[3], raw_full, raw_empty, op_full[2], op_empty[2], acc1_full[kNAcc1], acc1_empty[kNAcc1], a1_full, a1_empty,
-        acc2_full, acc2_empty, a2_full, acc3_full, acc3_empty;
+    constexpr int kStackBars = 3 + 2 + 4 + 2 * kNAcc1 + 7;
+    __shared__ uint64_t bars[kStackBars];
+    uint64_t *w_bar = bars, *raw_full = w_bar + 3, *raw_empty = raw_full + 1, *op_full = raw_empty + 1, *op_empty = op_full + 2,
+             *acc1_full = op_empty + 2, *acc1_empty = acc1_full + kNAcc1, *a1_full = acc1_empty + kNAcc1, *a1_empty = a1_full + 1,
+             *acc2_full = a1_empty + 1, *acc2_empty = acc2_full + 1, *a2_full = acc2_empty + 1, *acc3_full = a2_full + 1, *acc3_empty = acc3_full + 1;
     __shared__ __align__(16) float s_b1[32], s_b2[64], s_b3[64];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
@@ -94,21 +97,26 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
     const int envs = blockIdx.x < p.n ? (p.n - blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;   // of this CTA
     const int total = envs * p.tiles;                   // conv1 tiles of this CTA
 
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < 3; ++i) mbar_init(&w_bar[i], 1);
-        mbar_init(&raw_full, 1); mbar_init(&raw_empty, 8);
-        for (int i = 0; i < 2; ++i) { mbar_init(&op_full[i], 8); mbar_init(&op_empty[i], 1); }
-        for (int i = 0; i < kNAcc1; ++i) { mbar_init(&acc1_full[i], 1); mbar_init(&acc1_empty[i], 8); }
-        mbar_init(&a1_full, 8); mbar_init(&a1_empty, 1);
-        mbar_init(&acc2_full, 1); mbar_init(&acc2_empty, 8); mbar_init(&a2_full, 8);
-        mbar_init(&acc3_full, 1); mbar_init(&acc3_empty, 8);
-        abort_flag = 0;
+    if (warp == 0) {
+        // one barrier a lane; eight warps arrive at raw_empty, op_full, acc1_empty, a1_full, acc2_empty, a2_full and acc3_empty
+        static_assert(kStackBars == 24 && kNAcc1 == 4, "the mask");
+        constexpr uint32_t eight = 1u << 4 | 3u << 5 | 15u << 13 | 1u << 17 | 1u << 20 | 1u << 21 | 1u << 23;
+        if (lane < kStackBars) mbar_init(&bars[lane], eight >> lane & 1 ? 8 : 1);
         fence_barrier_init();
-        tma_prefetch_desc(&tmW1); tma_prefetch_desc(&tmW2); tma_prefetch_desc(&tmW3);
+        __syncwarp();
+        if (lane == 0) {                                 // the filters: not the previous kernel's, see `dependent`
+            mbar_arrive_expect_tx(&w_bar[0], kW1Bytes);
+            for (int g = 0; g < 2; ++g) tma_load_2d(sm + g * 8192, &tmW1, 0, g * 64, &w_bar[0]);
+            mbar_arrive_expect_tx(&w_bar[1], kW2Bytes);
+            for (int g = 0; g < 8; ++g) tma_load_2d(sm + kW1Bytes + g * 8192, &tmW2, g * 64, 0, &w_bar[1]);
+            mbar_arrive_expect_tx(&w_bar[2], kW3Bytes);
+            for (int g = 0; g < 9; ++g) tma_load_2d(sm + kW1Bytes + kW2Bytes + g * 8192, &tmW3, g * 64, 0, &w_bar[2]);
+        }
+    } else if (warp == 1) {
+        tmem_alloc(&tmem_slot, 512);
+    } else if (warp == 2 && lane == 0) {
+        abort_flag = 0;
     }
-    if (warp == 1) tmem_alloc(&tmem_slot, 512);
-    if (warp == 2) s_b1[lane] = p.b1[lane];
-    if (warp == 3) for (int i = lane; i < 64; i += 32) { s_b2[i] = p.b2[i]; s_b3[i] = p.b3[i]; }
     // positions of an odd-sized grid's border are never written: they must hold finite numbers
     for (int i = threadIdx.x; i < (2 * p.a1_plane + p.a2_bytes) / 16; i += kStackThreads) st_shared_v4(a1_addr + 16 * i, 0, 0, 0, 0);
     fence_async_proxy();
@@ -116,14 +124,6 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tm = tmem_slot;
-    if (threadIdx.x == 0) {                              // not the previous kernel's: see `dependent`
-        mbar_arrive_expect_tx(&w_bar[0], kW1Bytes);
-        for (int g = 0; g < 2; ++g) tma_load_2d(sm + g * 8192, &tmW1, 0, g * 64, &w_bar[0]);
-        mbar_arrive_expect_tx(&w_bar[1], kW2Bytes);
-        for (int g = 0; g < 8; ++g) tma_load_2d(sm + kW1Bytes + g * 8192, &tmW2, g * 64, 0, &w_bar[1]);
-        mbar_arrive_expect_tx(&w_bar[2], kW3Bytes);
-        for (int g = 0; g < 9; ++g) tma_load_2d(sm + kW1Bytes + kW2Bytes + g * 8192, &tmW3, g * 64, 0, &w_bar[2]);
-    }
     pdl_wait();
     pdl_trigger();
 
@@ -135,9 +135,9 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             const uint32_t bytes = 4u * (uint32_t)(p.H * W);
             size_t frame = envs ? frame_of(p, blockIdx.x) : 0;
             for (int i = 0; i < envs; ++i) {
-                if (!mbar_wait(&raw_empty, ((uint32_t)i & 1u) ^ 1u, abortp, p.status, 41)) break;
-                mbar_arrive_expect_tx(&raw_full, bytes);
-                bulk_load(s_raw, p.obs + frame * bytes, bytes, &raw_full);
+                if (!mbar_wait(raw_empty, ((uint32_t)i & 1u) ^ 1u, abortp, p.status, 41)) break;
+                mbar_arrive_expect_tx(raw_full, bytes);
+                bulk_load(s_raw, p.obs + frame * bytes, bytes, raw_full);
                 if (i + 1 < envs) {                      // the next frame at least as far as L2
                     frame = frame_of(p, blockIdx.x + (i + 1) * gridDim.x);
                     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.obs + frame * bytes), "r"(bytes) : "memory");
@@ -170,8 +170,8 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             bool alive = mbar_wait(&w_bar[1], 0, abortp, p.status, 42);
             for (int i = 0; alive && i < envs; ++i) {
                 const uint32_t ph = (uint32_t)i & 1u;
-                if (!mbar_wait(&a1_full, ph, abortp, p.status, 45)) break;
-                if (!mbar_wait(&acc2_empty, ph ^ 1u, abortp, p.status, 46)) break;
+                if (!mbar_wait(a1_full, ph, abortp, p.status, 45)) break;
+                if (!mbar_wait(acc2_empty, ph ^ 1u, abortp, p.status, 46)) break;
                 tc_fence_after();
 #pragma unroll
                 for (int tap = 0; tap < 4; ++tap) {
@@ -183,8 +183,8 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
                         for (int k = 0; k < 4; ++k) mma_f16_ss(tm + kAcc2, a + 2 * k, b + 2 * k, idesc, (tap | pl | k) != 0);
                     }
                 }
-                mma_commit(&a1_empty);
-                mma_commit(&acc2_full);
+                mma_commit(a1_empty);
+                mma_commit(acc2_full);
             }
         }
     } else if (warp == 3) {
@@ -194,8 +194,8 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             bool alive = mbar_wait(&w_bar[2], 0, abortp, p.status, 42);
             for (int i = 0; alive && i < envs; ++i) {
                 const uint32_t ph = (uint32_t)i & 1u;
-                if (!mbar_wait(&a2_full, ph, abortp, p.status, 47)) break;
-                if (!mbar_wait(&acc3_empty, ph ^ 1u, abortp, p.status, 48)) break;
+                if (!mbar_wait(a2_full, ph, abortp, p.status, 47)) break;
+                if (!mbar_wait(acc3_empty, ph ^ 1u, abortp, p.status, 48)) break;
                 tc_fence_after();
 #pragma unroll
                 for (int tap = 0; tap < 9; ++tap) {
@@ -204,7 +204,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
 #pragma unroll
                     for (int k = 0; k < 4; ++k) mma_f16_ss(tm + kAcc3, a + 2 * k, b + 2 * k, idesc, (tap | k) != 0);
                 }
-                mma_commit(&acc3_full);                  // also says that conv2's output has been read: it is written after this wait
+                mma_commit(acc3_full);                  // also says that conv2's output has been read: it is written after this wait
             }
         }
     } else if (warp >= kConvWarp && warp < kEpi1Warp) {
@@ -217,7 +217,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             q = q < cells ? q : 0;                       // past the last position: results are never stored
             const int Y = q / Ws, X = q - Y * Ws;
             const uint8_t* src = s_raw + (4 * Y) * W + 4 * X;
-            if (t == 0 && !mbar_wait_warp(&raw_full, (uint32_t)i & 1u, abortp, p.status, 51)) break;
+            if (t == 0 && !mbar_wait_warp(raw_full, (uint32_t)i & 1u, abortp, p.status, 51)) break;
             uint32_t v[32];
 #pragma unroll
             for (int c = 0; c < 4; ++c)
@@ -231,7 +231,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
                 t = 0;
                 ++i;
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&raw_empty);
+                if (lane == 0) mbar_arrive(raw_empty);
             }
             if (!mbar_wait_warp(&op_empty[b], ((uint32_t)(k >> 1) & 1u) ^ 1u, abortp, p.status, 52)) break;
             tc_fence_after();
@@ -245,6 +245,8 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
         // ---- conv1 epilogue: warps of group h take output channels [16 h, 16 h + 16)
         const int h = (warp - kEpi1Warp) >> 2, qq = warp & 3;
         const float inv = *p.inv1;
+        s_b1[lane] = p.b1[lane];                         // every warp of the role writes the same
+        __syncwarp();
         const uint32_t lanes = ((uint32_t)(qq * 32) << 16) + 16 * h;
         for (int k = 0, t = 0, i = 0; k < total; ++k) {
             const int q = t * kTile + 31 * qq + lane, y = q / Ws, x = q - y * Ws, acc = k % kNAcc1;
@@ -270,7 +272,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             }
             finish16(v0, inv, s_b1 + 16 * h, pk);
             // finished in registers: conv2 has until here to read the previous environment's rows
-            if (t == 0 && i > 0 && !mbar_wait_warp(&a1_empty, (uint32_t)(i - 1) & 1u, abortp, p.status, 54)) break;
+            if (t == 0 && i > 0 && !mbar_wait_warp(a1_empty, (uint32_t)(i - 1) & 1u, abortp, p.status, 54)) break;
             if (valid) {
                 st_shared_v4(dst + ((ch ^ swz) << 4), pk[0], pk[1], pk[2], pk[3]);
                 st_shared_v4(dst + (((ch + 1) ^ swz) << 4), pk[4], pk[5], pk[6], pk[7]);
@@ -280,7 +282,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
                 ++i;
                 fence_async_proxy();                     // the tensor core reads these rows through the asynchronous proxy
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&a1_full);
+                if (lane == 0) mbar_arrive(a1_full);
             }
             if (valid) st_global_v8(out, pk);            // parity tap: after the hand-over
         }
@@ -288,6 +290,8 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
         // ---- conv2 and conv3 epilogues: thread = row of the input grid, warps of group h take channels [32 h, 32 h + 32)
         const int h = (warp - kEpi2Warp) >> 2, qq = warp & 3, m = qq * 32 + lane;
         const float inv2 = *p.inv2, inv3 = *p.inv3;
+        for (int i = lane; i < 64; i += 32) { s_b2[i] = p.b2[i]; s_b3[i] = p.b3[i]; }      // every warp of the role writes the same
+        __syncwarp();
         const uint32_t lanes = ((uint32_t)(qq * 32) << 16) + 32 * h;
         const int y2 = m / p.W1s, x2 = m - y2 * p.W1s, y3 = m / p.W2, x3 = m - y3 * p.W2;
         const bool ok2 = y2 < p.H2 && x2 < p.W2, ok3 = y3 < p.H3 && x3 < p.W3;
@@ -297,13 +301,13 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             const uint32_t ph = (uint32_t)i & 1u;
             const size_t e = (size_t)blockIdx.x + (size_t)i * gridDim.x;
             uint32_t v[32], pk[2][8];
-            if (!mbar_wait_warp(&acc2_full, ph, abortp, p.status, 55)) break;
+            if (!mbar_wait_warp(acc2_full, ph, abortp, p.status, 55)) break;
             tc_fence_after();
             tmem_ld_32x32(tm + kAcc2 + lanes, v);
             tmem_ld_wait();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acc2_empty);
+            if (lane == 0) mbar_arrive(acc2_empty);
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 finish16(v + 16 * j, inv2, s_b2 + 32 * h + 16 * j, pk[j]);
@@ -315,16 +319,16 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             }
             fence_async_proxy();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&a2_full);
+            if (lane == 0) mbar_arrive(a2_full);
             __half* out = p.a2 + (y2 * p.a2_plane_rows + e * p.W2 + x2) * 64 + 32 * h;
             if (ok2) { st_global_v8(out, pk[0]); st_global_v8(out + 16, pk[1]); }     // parity tap: after the hand-over
-            if (!mbar_wait_warp(&acc3_full, ph, abortp, p.status, 56)) break;
+            if (!mbar_wait_warp(acc3_full, ph, abortp, p.status, 56)) break;
             tc_fence_after();
             tmem_ld_32x32(tm + kAcc3 + lanes, v);
             tmem_ld_wait();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acc3_empty);
+            if (lane == 0) mbar_arrive(acc3_empty);
             out = p.a3 + (e * p.P3 + (size_t)(y3 * p.W3 + x3)) * 64 + 32 * h;
 #pragma unroll
             for (int j = 0; j < 2; ++j) {

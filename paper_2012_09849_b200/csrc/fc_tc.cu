@@ -89,7 +89,8 @@ fc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     using S = PairShape<BN>;
     constexpr int NST = S::kStages, HALF = BN / 2;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[NST], empty_bar[NST], acc_full[2], acc_empty[2];
+    __shared__ uint64_t bars[2 * NST + 4];
+    uint64_t *full_bar = bars, *empty_bar = bars + NST, *acc_full = empty_bar + NST, *acc_empty = acc_full + 2;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ float s_bias[BN];
@@ -103,22 +104,19 @@ fc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int s0 = blockIdx.z * p.group, ns = min(p.group, p.splits - s0);
     const int k0 = s0 * p.cps, chunks = ns * p.cps;
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < NST; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&acc_full[a], 1); mbar_init(&acc_empty[a], 16); }
-        abort_flag = 0;
+    if (warp == 0) {
+        if (lane < 2 * NST + 4) mbar_init(&bars[lane], lane < 2 * NST + 2 ? 1 : 16);
         fence_barrier_init();
-        tma_prefetch_desc(&tmA);
-        tma_prefetch_desc(&tmB);
-    }
-    if (threadIdx.x >= 64) for (int i = threadIdx.x - 64; i < BN; i += kThreads - 64) s_bias[i] = p.bias[n0 + i];
-    if (warp == 1) {
+    } else if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(2 * BN) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else if (warp == 2 && lane == 0) {
+        abort_flag = 0;
+        tma_prefetch_desc(&tmA);
     }
+    static_assert(2 * NST + 4 <= 32, "a lane initialises one barrier");
     tc_fence_before();
-    __syncthreads();
-    cluster_sync();                                      // the partner's barriers exist
+    cluster_sync();                                      // of both CTAs' threads: the partner's barriers exist
     tc_fence_after();
     const uint32_t tmem_d = tmem_slot;
 
@@ -173,6 +171,10 @@ fc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // epilogue warps 2..9: lane quarter warp % 4, columns [HALF half, HALF half + HALF) of the tile
         const int q = warp & 3, half = (warp - 2) >> 2;
         const float inv = *p.inv_scale;
+        if constexpr (!ONE) {                            // the two to four warps that share a column write the same
+            for (int i = lane; i < HALF; i += 32) s_bias[half * HALF + i] = p.bias[n0 + half * HALF + i];
+            __syncwarp();
+        }
         const bool running = !ONE && (BN == 256 || blockIdx.z == 0);      // a wide tile has one range or all of them
         float* turn = reinterpret_cast<float*>(sm + NST * S::kStage) + (warp - 2) * kTurn;
         const int row0 = m0 + q * 32, col0 = n0 + half * HALF, rl = lane >> 3, c4 = (lane & 7) * 4;

@@ -67,7 +67,9 @@ fc_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     constexpr int BN = 128;
     constexpr int B_BYTES = BN * BK * 2;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t b_full[FCB_MAX_NK], a_full[FCB_STAGES], a_empty[FCB_STAGES], acc_full[FCB_MAX_TILES];
+    constexpr int kBars = FCB_MAX_NK + 2 * FCB_STAGES + FCB_MAX_TILES;
+    __shared__ uint64_t bars[kBars];
+    uint64_t *b_full = bars, *a_full = bars + FCB_MAX_NK, *a_empty = a_full + FCB_STAGES, *acc_full = a_empty + FCB_STAGES;
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
@@ -81,26 +83,27 @@ fc_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     const int my_tiles = slot < p.m_tiles ? (p.m_tiles - slot + slots - 1) / slots : 0;   // <= FCB_MAX_TILES (launcher)
     volatile int* abortp = &abort_flag;
 
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < FCB_MAX_NK; ++i) mbar_init(&b_full[i], 1);
-        for (int i = 0; i < FCB_STAGES; ++i) { mbar_init(&a_full[i], 1); mbar_init(&a_empty[i], 1); }
-        for (int i = 0; i < FCB_MAX_TILES; ++i) mbar_init(&acc_full[i], 1);
-        abort_flag = 0;
+    if (warp == 0) {
+        static_assert(kBars <= 32, "a lane initialises one barrier");
+        if (lane < kBars) mbar_init(&bars[lane], 1);
         fence_barrier_init();
+        __syncwarp();
+        if (lane == 0) {                                 // the weights do not depend on the previous kernel
+            for (int kc = 0; kc < p.nk; ++kc) {
+                mbar_arrive_expect_tx(&b_full[kc], B_BYTES);
+                tma_load_2d(sm + kc * B_BYTES, &tmB, (range * p.nk + kc) * BK, n0, &b_full[kc]);
+            }
+        }
+    } else if (warp == 1) {
+        tmem_alloc(&tmem_base_slot, FCB_MAX_TILES * BN);
+    } else if (warp == 2 && lane == 0) {
+        abort_flag = 0;
         tma_prefetch_desc(&tmA);
-        tma_prefetch_desc(&tmB);
     }
-    if (warp == 1) tmem_alloc(&tmem_base_slot, FCB_MAX_TILES * BN);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_d = tmem_base_slot;
-    if (warp == 0 && lane == 0) {                        // the weights do not depend on the previous kernel
-        for (int kc = 0; kc < p.nk; ++kc) {
-            mbar_arrive_expect_tx(&b_full[kc], B_BYTES);
-            tma_load_2d(sm + kc * B_BYTES, &tmB, (range * p.nk + kc) * BK, n0, &b_full[kc]);
-        }
-    }
     pdl_wait();
     pdl_trigger();
 
