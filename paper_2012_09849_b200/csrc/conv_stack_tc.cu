@@ -2,9 +2,9 @@
 // environment at a time per CTA with every filter resident in shared memory (152 KB).
 //
 // For batches of a few environments per SM, where three kernels spend their time between them: each starts 1.3 us after
-// the last CTA of the one before and needs 2 us to its first finished tile.  Step of n = 8: 22.7 -> 18.2 us, of 256: 31.0 ->
-// 26.1, of 512: 37.2 -> 35.1; equal at seven environments per SM (n = 1024: 51.7).  From there on the three kernels win
-// (n = 8192: 198 us of convolutions against 240): one environment here takes about 7800 clocks where its MMAs need 4288,
+// the last CTA of the one before and needs 2 us to its first finished tile.  Step of 16 observations: 20.5 -> 16.9 us, of 256: 27.3
+// -> 24.5, of 444: 31.6 -> 29.1; five to six environments per SM are equal (conv_stack_envs).  From there on the three
+// kernels win: one environment here takes about 7800 clocks where its MMAs need 4288,
 // because those fetch their operands from the same shared memory (128 bytes per clock, 68 x 6 KB per environment) that the
 // converters and epilogues work in.  The activations never leave the SM between layers: a CTA keeps one frame (raw bytes), conv1's output (K-major 128-byte-swizzled rows, two
 // planes of 64 channels of the space-to-depth(2) grid) and conv2's output (one plane) in shared memory, and
@@ -18,12 +18,12 @@
 //   * conv2 and conv3 are sums over taps of row-shifted 128 x 64 products on their input grids; both grids of an
 //     environment fit one tile.  Rows outside the output extent are computed from whatever lies there and dropped.
 //
-// conv1's and conv2's outputs are also written to global memory, after their hand-overs: hts_policy_read_activation may ask
-// for any step's hidden layers and nothing else reads them.  36 KB per observation: 18.0 against 17.7 us without (n = 8),
-// 25.9 / 25.0 (256), 34.6 / 32.6 (592), 46.9 / 41.6 (888).
+// conv1's and conv2's outputs are also written to global memory: hts_policy_read_activation may ask for any step's hidden
+// layers and nothing else reads them.  36 KB per observation, which a thread each stores by TMA from where they lie (as
+// 32-byte stores of the epilogue warps they cost 0.3 us at n = 8, 0.9 at 256, 5 at 888).
 //
-// Roles: warp 0 copies, warps 1 and 4 issue the MMAs of conv1 (alternate tiles), 2 and 3 those of conv2 and conv3 (warps
-// 5..7 are idle), then eight converter warps (four per filter
+// Roles: warp 0 copies, warps 1 and 4 issue the MMAs of conv1 (alternate tiles), 2 and 3 those of conv2 and conv3, 5 and 6
+// store the parity taps (warp 7 is idle), then eight converter warps (four per filter
 // row), eight epilogue warps for conv1 and eight for conv2 and conv3 in turn (four per half of the channels).  A tile takes
 // all warps of a role: what bounds small batches, and the hand-overs of large ones, is the latency of one tile.
 // Tensor clocks per environment: conv1 4 tiles x 8 x 32, conv2 32 x 48, conv3 36 x 48 = 4288 (84 x 84 frames).
@@ -75,14 +75,15 @@ __device__ __forceinline__ void finish16(const uint32_t* v, float inv, const flo
 template <int WC>
 __global__ void __launch_bounds__(kStackThreads)
 conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,
-                  const __grid_constant__ CUtensorMap tmW3, const ConvStackParams p)
+                  const __grid_constant__ CUtensorMap tmW3, const __grid_constant__ CUtensorMap tmT1, const __grid_constant__ CUtensorMap tmT2,
+                  const ConvStackParams p)
 {
     extern __shared__ uint8_t smem_raw[];
-    constexpr int kStackBars = 3 + 2 + 4 + 2 * kNAcc1 + 7;
+    constexpr int kStackBars = 3 + 2 + 4 + 2 * kNAcc1 + 8;
     __shared__ uint64_t bars[kStackBars];
     uint64_t *w_bar = bars, *raw_full = w_bar + 3, *raw_empty = raw_full + 1, *op_full = raw_empty + 1, *op_empty = op_full + 2,
              *acc1_full = op_empty + 2, *acc1_empty = acc1_full + kNAcc1, *a1_full = acc1_empty + kNAcc1, *a1_empty = a1_full + 1,
-             *acc2_full = a1_empty + 1, *acc2_empty = acc2_full + 1, *a2_full = acc2_empty + 1, *acc3_full = a2_full + 1, *acc3_empty = acc3_full + 1;
+             *acc2_full = a1_empty + 1, *acc2_empty = acc2_full + 1, *a2_full = acc2_empty + 1, *acc3_full = a2_full + 1, *acc3_empty = acc3_full + 1, *a2_stored = acc3_empty + 1;
     __shared__ __align__(16) float s_b1[32], s_b2[64], s_b3[64];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
@@ -98,10 +99,11 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
     const int total = envs * p.tiles;                   // conv1 tiles of this CTA
 
     if (warp == 0) {
-        // one barrier a lane; eight warps arrive at raw_empty, op_full, acc1_empty, a1_full, acc2_empty, a2_full and acc3_empty
-        static_assert(kStackBars == 24 && kNAcc1 == 4, "the mask");
+        // one barrier a lane; eight warps arrive at raw_empty, op_full, acc1_empty, a1_full, acc2_empty, a2_full and acc3_empty,
+        // and at a1_empty both who reads conv1's output: the tensor core and the store
+        static_assert(kStackBars == 25 && kNAcc1 == 4, "the mask");
         constexpr uint32_t eight = 1u << 4 | 3u << 5 | 15u << 13 | 1u << 17 | 1u << 20 | 1u << 21 | 1u << 23;
-        if (lane < kStackBars) mbar_init(&bars[lane], eight >> lane & 1 ? 8 : 1);
+        if (lane < kStackBars) mbar_init(&bars[lane], eight >> lane & 1 ? 8 : lane == 18 ? 2 : 1);
         fence_barrier_init();
         __syncwarp();
         if (lane == 0) {                                 // the filters: not the previous kernel's, see `dependent`
@@ -145,7 +147,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             }
         }
     } else if (warp == 1 || warp == 4) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = instr_desc_f16(0, 128, 64);
             const uint64_t b0 = smem_desc_sw128(base), b1 = smem_desc_sw128(base + 8192);
             bool alive = mbar_wait(&w_bar[0], 0, abortp, p.status, 42);
@@ -164,7 +166,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             }
         }
     } else if (warp == 2) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = instr_desc_f16(0, 128, 64);
             const uint32_t w2 = base + kW1Bytes;
             bool alive = mbar_wait(&w_bar[1], 0, abortp, p.status, 42);
@@ -188,7 +190,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             }
         }
     } else if (warp == 3) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = instr_desc_f16(0, 128, 64);
             const uint32_t w3 = base + kW1Bytes + kW2Bytes;
             bool alive = mbar_wait(&w_bar[2], 0, abortp, p.status, 42);
@@ -206,6 +208,23 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
                 }
                 mma_commit(acc3_full);                  // also says that conv2's output has been read: it is written after this wait
             }
+        }
+    } else if (warp == 5 || warp == 6) {
+        // ---- parity taps: the SM's copy of a layer, as it lies there
+        if (lane == 0) {
+            for (int i = 0; i < envs; ++i) {
+                const int e = (int)(blockIdx.x + i * gridDim.x);
+                if (!mbar_wait(warp == 5 ? a1_full : a2_full, (uint32_t)i & 1u, abortp, p.status, 57)) break;
+                if (warp == 5) {
+                    for (int pl = 0; pl < 2; ++pl) tma_store_4d(&tmT1, a1_addr + pl * p.a1_plane, pl * 64, 0, e, 0);
+                } else {
+                    tma_store_4d(&tmT2, a2_addr, 0, 0, e, 0);
+                }
+                tma_store_commit();
+                tma_store_wait_read();
+                mbar_arrive(warp == 5 ? a1_empty : a2_stored);
+            }
+            tma_store_wait();
         }
     } else if (warp >= kConvWarp && warp < kEpi1Warp) {
         // ---- converters: warps of group dy write the operand of that filter row
@@ -253,7 +272,6 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             const bool valid = lane < 31 && y < p.H1 && x < p.W1;
             const int row = (y >> 1) * p.W1s + (x >> 1);
             const uint32_t dst = a1_addr + (y & 1) * p.a1_plane + row * 128, swz = (uint32_t)(row & 7), ch = (uint32_t)((x & 1) * 4 + 2 * h);
-            __half* out = p.a1 + ((y >> 1) * p.a1_plane_rows + (size_t)(blockIdx.x + i * gridDim.x) * p.W1s + (x >> 1)) * 128 + (y & 1) * 64 + (x & 1) * 32 + 16 * h;
             const uint32_t taddr = tm + kAcc1 + acc * 64 + lanes;
             if (!mbar_wait_warp(&acc1_full[acc], (uint32_t)(k / kNAcc1) & 1u, abortp, p.status, 53)) break;
             tc_fence_after();
@@ -271,7 +289,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
                 v0[c] = __float_as_uint(a0); v0[c + 1] = __float_as_uint(a1);
             }
             finish16(v0, inv, s_b1 + 16 * h, pk);
-            // finished in registers: conv2 has until here to read the previous environment's rows
+            // finished in registers: conv2 and the store have until here to read the previous environment's rows
             if (t == 0 && i > 0 && !mbar_wait_warp(a1_empty, (uint32_t)(i - 1) & 1u, abortp, p.status, 54)) break;
             if (valid) {
                 st_shared_v4(dst + ((ch ^ swz) << 4), pk[0], pk[1], pk[2], pk[3]);
@@ -284,7 +302,6 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
                 __syncwarp();
                 if (lane == 0) mbar_arrive(a1_full);
             }
-            if (valid) st_global_v8(out, pk);            // parity tap: after the hand-over
         }
     } else if (warp >= kEpi2Warp) {
         // ---- conv2 and conv3 epilogues: thread = row of the input grid, warps of group h take channels [32 h, 32 h + 32)
@@ -308,6 +325,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(acc2_empty);
+            if (i > 0 && !mbar_wait_warp(a2_stored, (uint32_t)(i - 1) & 1u, abortp, p.status, 58)) break;
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 finish16(v + 16 * j, inv2, s_b2 + 32 * h + 16 * j, pk[j]);
@@ -320,8 +338,6 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             fence_async_proxy();
             __syncwarp();
             if (lane == 0) mbar_arrive(a2_full);
-            __half* out = p.a2 + (y2 * p.a2_plane_rows + e * p.W2 + x2) * 64 + 32 * h;
-            if (ok2) { st_global_v8(out, pk[0]); st_global_v8(out + 16, pk[1]); }     // parity tap: after the hand-over
             if (!mbar_wait_warp(acc3_full, ph, abortp, p.status, 56)) break;
             tc_fence_after();
             tmem_ld_32x32(tm + kAcc3 + lanes, v);
@@ -329,7 +345,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(acc3_empty);
-            out = p.a3 + (e * p.P3 + (size_t)(y3 * p.W3 + x3)) * 64 + 32 * h;
+            __half* out = p.a3 + (e * p.P3 + (size_t)(y3 * p.W3 + x3)) * 64 + 32 * h;
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 finish16(v + 16 * j, inv3, s_b3 + 32 * h + 16 * j, pk[0]);
@@ -347,12 +363,12 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
 }
 
 template <int WC>
-hts_status launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const ConvStackParams& p, int smem, int grid,
+hts_status launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const CUtensorMap& t1, const CUtensorMap& t2, const ConvStackParams& p, int smem, int grid,
                   bool dependent, cudaStream_t s)
 {
     static OncePerDevice allowed;
     HTS_CUDA(allow_shared(conv_stack_kernel<WC>, allowed));
-    HTS_CUDA(launch_chained(dependent, conv_stack_kernel<WC>, dim3(grid), dim3(kStackThreads), (size_t)smem, s, w1, w2, w3, p));
+    HTS_CUDA(launch_chained(dependent, conv_stack_kernel<WC>, dim3(grid), dim3(kStackThreads), (size_t)smem, s, w1, w2, w3, t1, t2, p));
     note_launch();
     return HTS_OK;
 }
@@ -379,11 +395,11 @@ bool conv_stack_plan(const Geometry& g, ConvStackParams* p)
     return stack_smem(*p) <= 226 * 1024;
 }
 
-hts_status conv_stack_launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const ConvStackParams& p,
-                             bool dependent, cudaStream_t s)
+hts_status conv_stack_launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const CUtensorMap& t1, const CUtensorMap& t2,
+                             const ConvStackParams& p, bool dependent, cudaStream_t s)
 {
     const int sms = device_sm_count(device_slot()), grid = p.n < sms ? p.n : sms, smem = stack_smem(p);
-    return p.W == 84 ? launch<84>(w1, w2, w3, p, smem, grid, dependent, s) : launch<0>(w1, w2, w3, p, smem, grid, dependent, s);
+    return p.W == 84 ? launch<84>(w1, w2, w3, t1, t2, p, smem, grid, dependent, s) : launch<0>(w1, w2, w3, t1, t2, p, smem, grid, dependent, s);
 }
 
 }  // namespace hts

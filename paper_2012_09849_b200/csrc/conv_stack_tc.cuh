@@ -18,18 +18,25 @@ struct ConvStackParams {
     int a1_plane, a2_bytes, raw_bytes;  // shared memory: one 64-channel plane of conv1's output, conv2's output, one frame
     const float *b1, *b2, *b3;
     const float *inv1, *inv2, *inv3;    // device scalars undoing the weight scaling (and conv1's /255)
-    __half *a1, *a2, *a3;               // workspaces: a3 is the dense layer's input, the others the parity taps
-    size_t a1_plane_rows, a2_plane_rows;    // rows of a1 / a2 from one grid row to the next (all environments of the workspace)
+    __half* a3;                         // the dense layer's input
     int* status;
 };
 
 // false if the frames do not fit the kernel (four channels; one 128-row tile must hold conv2's and conv3's grids)
 bool conv_stack_plan(const Geometry& g, ConvStackParams* p);
-// Batches up to this many environments per SM are faster here than in a kernel per layer.
-constexpr int kStackEnvs = 6;
+// Batches up to this many environments per SM are faster here than in a kernel per layer.  A kernel per layer fills its tiles
+// from several environments; here an environment's conv2 and conv3 take a tile of 128 rows each, however few of them its grids
+// fill.  Measured, here / there, us per step: 84 x 84 (100 and 81 rows) 33.2 / 33.9 at four per SM, 38.4 / 39.3 at five, 42.6 /
+// 42.1 at six; 64 x 96 (96 and 60 rows) 32.5 / 32.7 at four, 36.6 / 34.6 at five.
+inline int conv_stack_envs(const ConvStackParams& p)
+{
+    const int per_sm = (p.P1s + p.P2) / 36;
+    return per_sm < 2 ? 2 : per_sm < 6 ? per_sm : 6;
+}
 // Weight maps: the packed filters of conv1 [128][64], conv2 [64][512] and conv3 [64][576], box 64 x 64.
+// t1, t2: where conv1's and conv2's outputs go, as (channel, x, environment, y), box 64 channels x one environment's grid.
 // dependent: as in conv1_launch.
-hts_status conv_stack_launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const ConvStackParams& p,
-                             bool dependent, cudaStream_t s);
+hts_status conv_stack_launch(const CUtensorMap& w1, const CUtensorMap& w2, const CUtensorMap& w3, const CUtensorMap& t1, const CUtensorMap& t2,
+                             const ConvStackParams& p, bool dependent, cudaStream_t s);
 
 }  // namespace hts

@@ -364,7 +364,7 @@ struct TcState {
     // workspace
     __half *a1s, *a2, *a3;
     float *hpart, *h;
-    CUtensorMap mW1, mA2, mB2, mA3, mB3, mAfc, mBfc, mBfcPair;
+    CUtensorMap mW1, mA2, mB2, mA3, mB3, mAfc, mBfc, mBfcPair, mT1, mT2;
     bool stacked;               // the frames fit the kernel that runs all three convolutions
     ConvStackParams stack;
     int* status;
@@ -423,8 +423,8 @@ hts_status tc_create(const Geometry& g, int max_batch, int* status, TcState** ou
     t->stacked = conv_stack_plan(g, &t->stack);
     ConvStackParams& cs = t->stack;
     cs.b1 = t->b1; cs.b2 = t->b2; cs.b3 = t->b3; cs.inv1 = t->inv_scale + L_CONV1; cs.inv2 = t->inv_scale + L_CONV2; cs.inv3 = t->inv_scale + L_CONV3;
-    cs.a1_plane_rows = nb * t->W1s; cs.a2_plane_rows = nb * g.W2;
-    cs.a1 = t->a1s; cs.a2 = t->a2; cs.a3 = t->a3; cs.status = status;
+    cs.a3 = t->a3; cs.status = status;
+    if (t->stacked && !(make_grid_map(&t->mT1, t->a1s, 128, t->W1s, nb, t->H1s) && make_grid_map(&t->mT2, t->a2, 64, g.W2, nb, g.H2))) { delete t; return HTS_ERR_CUDA; }
     *out = t;
     return HTS_OK;
 }
@@ -484,11 +484,11 @@ hts_status tc_forward(TcState* t, const uint8_t* obs, const Indexing& ix, int n,
     const Geometry& g = t->g;
     hts_status st;
     const bool dependent = first_layer_dependent(t, s);
-    if (t->stacked && n <= kStackEnvs * device_sm_count(device_slot())) {
+    if (t->stacked && n <= conv_stack_envs(t->stack) * device_sm_count(device_slot())) {
         ConvStackParams c = t->stack;
         c.obs = obs; c.slots = ix.slots; c.pool = ix.pool; c.n = n;
         prof.begin(K_CONV1, s);
-        st = conv_stack_launch(t->mW1, t->mB2, t->mB3, c, dependent, s);
+        st = conv_stack_launch(t->mW1, t->mB2, t->mB3, t->mT1, t->mT2, c, dependent, s);
         if (st != HTS_OK) return st;
         prof.end(K_CONV1, s);
     } else {

@@ -39,6 +39,22 @@ inline bool make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t co
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// fp16 rows of `channels` in the order (y, environment, x), seen as (channel, x, environment, y); box = 64 channels of one
+// environment's grid, 128-byte swizzle.
+inline bool make_grid_map(CUtensorMap* m, const void* ptr, int channels, int W, uint64_t envs, int H)
+{
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t row = (cuuint64_t)channels * 2;
+    const cuuint64_t dims[4] = {(cuuint64_t)channels, (cuuint64_t)W, envs, (cuuint64_t)H};
+    const cuuint64_t strides[3] = {row, row * W, row * W * envs};
+    const cuuint32_t box[4] = {64, (cuuint32_t)W, 1, (cuuint32_t)H};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // uint8 frames [frames, C, H, W] seen as 32-bit words [frames][C][H/4 grid rows][W words]: the four input
 // rows under one grid row are W contiguous words.  Box = `group_rows` grid rows of `channels` channels of one frame.
 inline bool make_frames_map(CUtensorMap* m, const void* ptr, int W, int H, int C, uint64_t frames, int group_rows, int channels)
