@@ -78,11 +78,14 @@ __device__ __forceinline__ size_t plane_row(const ConvParams& p, int e, int r)
 // y[e,o,i,j] = relu(b[o] + in_scale * sum_{c,u,v} w[o,c,u,v] x[e,c,i s+u,j s+v]), summed over (c, u, v) in ascending
 // order.  Implicit GEMM: a block owns PX consecutive output pixels of the batch and OC channels and gathers PX x KC
 // inputs and OC x KC weights per step into shared memory, one step ahead; a thread owns PXT pixels x OT channels.
-// Bound: the 128 bytes per clock at which shared memory reaches registers (a thread loads 4 (PXT + OT) bytes per
-// PXT x OT multiply-adds) and the fp32 pipes alike.  Packed multiply-adds (two channels each, the input in both lanes)
-// reach 64 TFLOP/s in this pattern where scalar ones stop at 49 (three distinct registers per operation).  8 x 16 per
-// thread loads less but leaves two warps per scheduler: 206 against 171 us (conv2, n = 1024); copying input rows
-// instead of gathering per tap makes the reads scattered: 278 us.
+// Bound: issue slots and the 128 bytes per clock at which shared memory reaches registers (a thread loads 4 (PXT + OT)
+// bytes per PXT x OT multiply-adds), both close to the fp32 pipes' own time.  Packed multiply-adds (two channels each, the input
+// in both lanes) reach 64 TFLOP/s in this pattern where scalar ones stop at 49 (three distinct registers per operation).  A
+// thread's pixels are runs of four, so a step's inputs are two 16-byte loads instead of eight of 4: conv1 / conv2 / conv3 at n =
+// 1024 162 / 171 / 114 -> 153 / 154 / 103 us (a 16-byte load takes 4 clocks of shared memory where the eight lanes of a
+// quarter differ, 2 where they agree; pairs of pixels, with the weights in both lanes, take 16 clocks a step instead of 12:
+// 193 / 181 / 119).  8 x 16 per thread loads less but leaves two warps per scheduler: 206 against 171 us (conv2, n = 1024);
+// copying input rows instead of gathering per tap makes the reads scattered: 278 us.
 template <typename TIn, int PXT, int OT, int WPX, int WO, int KC, int PER_SM>
 __global__ void __launch_bounds__(32 * WPX * WO, PER_SM)
 conv_tile_kernel(const ConvParams p)
@@ -160,7 +163,8 @@ conv_tile_kernel(const ConvParams p)
         }
     };
     const int wp = warp % WPX, wo = warp / WPX, g = lane & 7, og = lane >> 3;
-    const int px_t = wp * 8 * PXT + g, o_t = wo * 4 * OT + og * OT;              // pixels px_t + 8 q
+    static_assert(PXT % 4 == 0, "16-byte loads");
+    const int px_t = wp * 8 * PXT + 4 * g, o_t = wo * 4 * OT + og * OT;          // pixels px_t + 32 (q / 4) + q % 4
     f32x2 acc[PXT][OT / 2];
 #pragma unroll
     for (int q = 0; q < PXT; ++q)
@@ -184,9 +188,13 @@ conv_tile_kernel(const ConvParams p)
                 const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(w + 2 * j);
                 wv[j] = t.x; wv[j + 1] = t.y;
             }
+            float4 xv[PXT / 4];
+#pragma unroll
+            for (int q = 0; q < PXT / 4; ++q) xv[q] = *reinterpret_cast<const float4*>(a + 32 * q);
 #pragma unroll
             for (int q = 0; q < PXT; ++q) {
-                const f32x2 xx = both(a[8 * q]);
+                const float4 x4 = xv[q / 4];
+                const f32x2 xx = both(q % 4 == 0 ? x4.x : q % 4 == 1 ? x4.y : q % 4 == 2 ? x4.z : x4.w);
 #pragma unroll
                 for (int j = 0; j < OT / 2; ++j) fma2(acc[q][j], xx, wv[j]);
             }
@@ -199,7 +207,7 @@ conv_tile_kernel(const ConvParams p)
     }
 #pragma unroll
     for (int q = 0; q < PXT; ++q) {
-        const int px = blockIdx.x * PX + px_t + 8 * q;
+        const int px = blockIdx.x * PX + px_t + 32 * (q / 4) + q % 4;
         if (px >= total) continue;
         const int e = px / P, r = px - e * P;
         float v[OT];
