@@ -34,15 +34,16 @@ __device__ __forceinline__ double warp_sum_d(double v)
 
 // An Op names NS sums, how four consecutive elements (float4 group q) or one element i add to them, whether
 // its arrays allow float4 loads, and what the last block does with the totals.
-template <class Op>
+// CHAINED: the kernel before this one is one of these as well, over the same inputs.  It has waited for whatever wrote them, so
+// the first loads need not wait for it: they are under way while it runs (means of 131072 transitions 9.5 -> 8.7 us).
+template <class Op, bool CHAINED>
 __global__ void __launch_bounds__(kThreads)
 sums_kernel(const Op op, long long count, long long per_block)
 {
     constexpr int NS = Op::NS;
     __shared__ double s_part[kThreads / 32][NS];
     __shared__ bool s_last;
-    pdl_wait();                               // the partials and the ticket, and the inputs, are the previous kernel's
-    pdl_trigger();
+    if constexpr (!CHAINED) { pdl_wait(); pdl_trigger(); }                // the partials, the ticket and the inputs are the previous kernel's
     const long long lo = (long long)blockIdx.x * per_block;               // per_block is a multiple of 4
     long long hi = lo + per_block; hi = hi > count ? count : hi;
     double acc[NS];
@@ -51,6 +52,16 @@ sums_kernel(const Op op, long long count, long long per_block)
     if (op.aligned16()) {
         const long long q_lo = lo >> 2, q_hi = hi >> 2;                    // whole float4 groups of the range
         long long q = q_lo + threadIdx.x;
+        if constexpr (CHAINED) {
+            typename Op::Quad g[2];                                        // two groups are all that a thread of a small problem has
+#pragma unroll
+            for (int u = 0; u < 2; ++u) if (q + u * kThreads < q_hi) g[u] = op.load4(q + u * kThreads);
+            pdl_wait();
+            pdl_trigger();
+#pragma unroll
+            for (int u = 0; u < 2; ++u) if (q + u * kThreads < q_hi) op.add4(g[u], acc);
+            q += 2 * kThreads;
+        }
         for (; q + 3 * kThreads < q_hi; q += 4 * kThreads) {               // four groups per array in flight per thread
             typename Op::Quad g[4];
 #pragma unroll
@@ -61,6 +72,7 @@ sums_kernel(const Op op, long long count, long long per_block)
         for (; q < q_hi; q += kThreads) op.add4(op.load4(q), acc);
         for (long long i = (q_hi << 2) + threadIdx.x; i < hi; i += kThreads) op.add1(i, acc);   // the last block's ragged tail
     } else {
+        if constexpr (CHAINED) { pdl_wait(); pdl_trigger(); }
         for (long long i = lo + threadIdx.x; i < hi; i += kThreads) op.add1(i, acc);
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -100,7 +112,7 @@ sums_kernel(const Op op, long long count, long long per_block)
     }
 }
 
-template <class Op>
+template <bool CHAINED = false, class Op>
 hts_status launch_sums(const Op& op, long long count, cudaStream_t s)
 {
     long long blocks = (count + (long long)kThreads * kPerThread - 1) / ((long long)kThreads * kPerThread);
@@ -108,7 +120,7 @@ hts_status launch_sums(const Op& op, long long count, cudaStream_t s)
     long long per_block = (count + blocks - 1) / blocks;
     per_block = (per_block + 3) / 4 * 4;
     blocks = (count + per_block - 1) / per_block;
-    HTS_CUDA(launch_pdl(sums_kernel<Op>, dim3((unsigned)blocks), dim3(kThreads), 0, s, op, count, per_block));
+    HTS_CUDA(launch_pdl(sums_kernel<Op, CHAINED>, dim3((unsigned)blocks), dim3(kThreads), 0, s, op, count, per_block));
     note_launch();
     return HTS_OK;
 }
@@ -243,7 +255,7 @@ extern "C" hts_status hts_ppo_terms(const float* logp_new, const float* logp_old
     }
     const PpoOp op{logp_new, logp_old, values, entropy, advantages, returns, out4, (double)clip, normalize_advantages != 0,
                    all_aligned16({logp_new, logp_old, values, entropy, advantages, returns})};
-    return launch_sums(op, (long long)count, s);
+    return normalize_advantages ? launch_sums<true>(op, (long long)count, s) : launch_sums(op, (long long)count, s);
 }
 
 // ---- the learner's parameter update (Section 4.1 "Delayed gradient", Eq. 5) ---------------------------------
