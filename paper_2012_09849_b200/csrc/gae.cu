@@ -184,8 +184,9 @@ hts_status launch_gae(const float* rewards, const float* values, const uint8_t* 
     // 97 % of the copy rate, at T=128, N=2^20).  Fewer would walk a long T in many short steps, each waiting for memory
     // (213 us at 512 x 32768, 60 with the columns of a block cut to 32 and eight chunks of eight rows per step).  This form
     // against the last one below, us at T=128: 50 / 34 (N = 75776), 62 / 57 (2^17), 91 / 109 (2^18), 356 / 427 (2^20);
-    // at T=512: 186 / 130, 234 / 222, 366 / 436: the line at four blocks per SM is low, they cross near 2^17 columns.
-    if (vec4 && N / 128 >= 4 * sms)
+    // at T=512: 186 / 130, 234 / 222, 366 / 436: they cross between 2^17 and 2^18 columns, 7 and 14 blocks per SM;
+    // short columns walk few steps: 11.3 / 12.3 at 32 x 2^17, but 20.9 / 16.6 at 64 x 80000.
+    if (vec4 && N / 128 >= (T < 64 ? 4 : 8) * sms)
         return launch_t<4, 2, 1>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, 2, s);
     // few columns and many rows: 8-column blocks, four chunks per warp (same chunks, same bits, four times the SMs).
     // Against 32 columns: 4.3 / 8.9 us at 512 x 512, 7.9 / 11.4 at 512 x 2048, 14.8 / 13.0 at 512 x 4096

@@ -186,12 +186,13 @@ hts_status launch_vtrace(const float* log_rhos, const float* rewards, const floa
                       aligned(dones, 4) && aligned(bootstrap, 16) && aligned(vs, 16) && aligned(pg, 16) &&
                       ((long)N * T >= (1L << 22));
     // the advantage scan's rules, with at most 512 threads (1024 would leave 64 registers: spills).  us, T x N:
-    //   128 against 32 columns per block: 68.4 / 61.5 at 128 x 75776, 85.7 / 96.5 at 128 x 2^17, 538 / 703 at 128 x 2^20
+    //   128 against 32 columns per block: 68.4 / 60.9 at 128 x 75776, 80.8 / 75.4 at 128 x 98304, 83.3 / 81.6 at 128 x 112000,
+    //   85.7 / 96.5 at 128 x 2^17, 538 / 703 at 128 x 2^20; 34.8 / 31.1 at 64 x 80000, 23.1 / 26.6 at 48 x 90000
     //   8 against 32 columns: 5.1 / 11.8 at 512 x 512, 11.7 / 15.0 at 512 x 2048, 22.7 / 16.9 at 512 x 4096
     //   4 against 8 warps: 30.2 / 32.3 at 128 x 37856, 92 / 96 at 256 x 60001, 46.6 / 29.4 at 512 x 8192
     //   8 against 16 warps: 7.7 / 8.6 at 128 x 4768 (149 blocks), 7.6 / 5.4 at 128 x 4704 (147)
     const int sms = device_sm_count(device_slot()), blocks = (N + 31) / 32;
-    if (vec4 && N / 128 >= 4 * sms) return launch_t<4, 2, 1, 2>(p, s);
+    if (vec4 && N / 128 >= (T < 64 ? 4 : 6) * sms) return launch_t<4, 2, 1, 2>(p, s);
     if (blocks < sms / 2 && T >= 4 * 8) return launch_t<1, 8, 4, 16>(p, s);
     if (blocks >= 8 * sms) return launch_t<1, 8, 1, 4>(p, s);
     return blocks >= sms ? launch_t<1, 8, 1, 8>(p, s) : launch_t<1, 8, 1, 16>(p, s);
