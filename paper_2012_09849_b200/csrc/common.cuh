@@ -97,6 +97,7 @@ inline cudaError_t allow_shared(K* kernel, OncePerDevice& done, bool carveout = 
 struct Indexing {
     const int32_t* slots = nullptr;
     int pool = 0;
+    int row0 = 0;                      // the batch's rows of the context's workspaces start here
 };
 constexpr int kStatusBadSlot = 100;
 constexpr int kStatusBadAction = 101;     // a stored action outside [0, A) met by the re-evaluation of given actions

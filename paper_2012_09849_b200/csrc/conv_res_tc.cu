@@ -100,7 +100,7 @@ conv_rows_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             uint32_t ph = 1;
             for (int left = total; left > 0;) {
                 const int cnt = min(left, H - y);        // output rows in this tile
-                int row = y * p.in_plane + tile * 128;
+                int row = y * p.in_plane + p.col0 + tile * 128;
                 for (int i = 0; i < cnt + KY - 1; ++i, row += p.in_plane) {
                     if (!mbar_wait(&a_empty[st], ph, abortp, p.status, 21)) { left = 0; break; }
                     uint8_t* dst = sm + S::kFilter + st * S::kStage;

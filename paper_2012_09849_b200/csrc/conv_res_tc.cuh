@@ -13,6 +13,7 @@ struct ConvRowsParams {
     int H_out, W_out;
     int in_plane;           // input rows of one grid row: environments of the workspace x W_in
     int tiles;              // 128-column tiles of n_env * W_in
+    int col0;               // the batch's first column (environment, x)
     const float* bias;      // [64]
     const float* inv_scale; // device scalar undoing the weight scaling
     __half* out;            // [64] per output pixel, at env * out_env + y * out_y + x * 64

@@ -213,7 +213,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
         // ---- parity taps: the SM's copy of a layer, as it lies there
         if (lane == 0) {
             for (int i = 0; i < envs; ++i) {
-                const int e = (int)(blockIdx.x + i * gridDim.x);
+                const int e = p.row0 + (int)(blockIdx.x + i * gridDim.x);
                 if (!mbar_wait(warp == 5 ? a1_full : a2_full, (uint32_t)i & 1u, abortp, p.status, 57)) break;
                 if (warp == 5) {
                     for (int pl = 0; pl < 2; ++pl) tma_store_4d(&tmT1, a1_addr + pl * p.a1_plane, pl * 64, 0, e, 0);
@@ -316,7 +316,7 @@ conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constan
         const uint32_t dst2 = a2_addr + r2 * 128, swz = (uint32_t)(r2 & 7);
         for (int i = 0; i < envs; ++i) {
             const uint32_t ph = (uint32_t)i & 1u;
-            const size_t e = (size_t)blockIdx.x + (size_t)i * gridDim.x;
+            const size_t e = (size_t)p.row0 + blockIdx.x + (size_t)i * gridDim.x;
             uint32_t v[32], pk[2][8];
             if (!mbar_wait_warp(acc2_full, ph, abortp, p.status, 55)) break;
             tc_fence_after();

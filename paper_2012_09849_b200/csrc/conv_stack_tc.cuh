@@ -11,6 +11,7 @@ struct ConvStackParams {
     const int32_t* slots;               // frame of each row in obs, or nullptr: row e is frame e
     int pool;                           // frames in obs when slots are given
     int n;
+    int row0;                           // the batch's first row of the workspaces
     int H, W, Ws;                       // frame, and width of its space-to-depth(4) grid
     int H1, W1, W1s, P1s;               // conv1 output; width and positions of its space-to-depth(2) grid
     int H2, W2, P2, H3, W3, P3;

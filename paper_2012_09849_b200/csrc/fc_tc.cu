@@ -141,7 +141,7 @@ fc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     if (!mbar_wait(&empty_bar[st], ((uint32_t)(kc / NST) & 1u) ^ 1u, abortp, p.status, 51)) break;
                     load_b(kc, st);
                 }
-                tma_load_2d_pair(sm + st * S::kStage, &tmA, (k0 + kc) * kChunk, m0, in_first(&full_bar[st]));
+                tma_load_2d_pair(sm + st * S::kStage, &tmA, (k0 + kc) * kChunk, p.row0 + m0, in_first(&full_bar[st]));
             }
         }
     } else if (warp == 1) {

@@ -9,6 +9,7 @@ struct FcPairParams {
     int splits, cps;                    // K ranges, 64-column chunks of a range
     int group;                          // ranges of one pair of SMs (the last pair of a tile may have fewer)
     int n;                              // valid rows
+    int row0;                           // the first one's row of the activations
     const float* bias;                  // [512]
     const float* inv_scale;             // device scalar undoing the weight scaling
     float* h;                           // [n][512]: written where one pair has all ranges

@@ -36,6 +36,8 @@ struct hts_ctx {
     uint8_t* s_obs = nullptr;
     int32_t *s_index = nullptr, *s_result = nullptr, *h_words = nullptr;
     float* s_logits = nullptr;
+    cudaStream_t h_stream = nullptr;    // its frames' copies, where they are cut in two
+    cudaEvent_t h_start = nullptr, h_copied[2] = {nullptr, nullptr};
     X3State* x3 = nullptr;        // packed weights and workspace of the gradient (weight_dtype fp32)
     int* status = nullptr;        // device status word
     Profiler prof;
@@ -126,15 +128,17 @@ hts_status run_step(hts_ctx* ctx, const uint8_t* obs, const Indexing& ix, const 
         ctx->prof.begin(K_HEADS, s);
         st = tc_heads(ctx->tc, env_ids, t_per_env, t, seed, n, ix, actions, logp, values, entropy, logits, s, given_actions);
     } else {
-        st = ref_forward(g, ctx->rw, ctx->rws, obs, ix, ctx->status, n, ctx->prof, s);
+        const size_t r = (size_t)ix.row0;
+        const RefWorkspace ws{ctx->rws.a1 + r * 32 * g.H1 * g.W1, ctx->rws.a2 + r * 64 * g.H2 * g.W2, ctx->rws.a3 + r * g.F, ctx->rws.h + r * 512};
+        st = ref_forward(g, ctx->rw, ws, obs, ix, ctx->status, n, ctx->prof, s);
         if (st != HTS_OK) return st;
         ctx->prof.begin(K_HEADS, s);
-        st = launch_heads(ctx->rws.h, 1, 0, nullptr, ctx->rw.whead, ctx->rw.bhead, g.A, env_ids, t_per_env, t,
+        st = launch_heads(ws.h, 1, 0, nullptr, ctx->rw.whead, ctx->rw.bhead, g.A, env_ids, t_per_env, t,
                           seed, n, ix, ctx->status, actions, logp, values, entropy, logits, nullptr, s, given_actions, false);
     }
     if (st != HTS_OK) return st;
     ctx->prof.end(K_HEADS, s);
-    ctx->last_n = n;
+    ctx->last_n = ix.row0 + n;
     return HTS_OK;
 }
 
@@ -144,6 +148,26 @@ hts_status run_step(hts_ctx* ctx, const uint8_t* obs, const Indexing& ix, const 
 // 55.4 / 58.4 (32), 108.6 / 114.5 (128), 149.0 / 153.7 (192), 320.7 / 330.2 (512), 601 / 609 (1024), 1165 / 1169 (2048),
 // 2265 / 2258 (4096), 4484 / 4461 (8192): the two cross between 2048 and 4096 rows, so the line could lie higher.
 constexpr int kHostDirect = 128;
+
+// The frames of a host step are copied in two parts, so that the step of the first runs while the second is copied.  Rows of the
+// first part: all but as many as leave a short step at the end and whose copy outlasts the first step (bf16: a step of 64 or
+// 128 observations takes 18 or 20 us, their copy 33 or 66 us); fp32 steps take as long as their copies: halves.
+namespace {
+int host_first_rows(const hts_ctx* ctx, int n)
+{
+    if (ctx->tc) return n >= 512 ? n - 128 : n >= 192 ? n - 64 : n;
+    return n >= 512 ? n / 2 : n;
+}
+// Stream and events of the copies, made by the first call that needs them.
+bool host_copies_ready(hts_ctx* c)
+{
+    if (!c->h_stream && cudaStreamCreateWithFlags(&c->h_stream, cudaStreamNonBlocking) != cudaSuccess) c->h_stream = nullptr;
+    for (cudaEvent_t* e : {&c->h_start, &c->h_copied[0], &c->h_copied[1]})
+        if (!*e && cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) *e = nullptr;
+    cudaGetLastError();
+    return c->h_stream && c->h_start && c->h_copied[0] && c->h_copied[1];
+}
+}  // namespace
 
 // staging buffer of hts_gae_host, one per device; grows on demand, freed by hts_gae_host_release
 static char* g_gae_stage[kDeviceSlots] = {};
@@ -301,7 +325,6 @@ hts_status hts_policy_step_host(hts_ctx* ctx, const uint8_t* obs, const int32_t*
         cudaGetLastError();
         return HTS_ERR_ALLOC;
     }
-    HTS_CUDA(cudaMemcpyAsync(ctx->s_obs, obs, nn * ctx->g.C * ctx->g.H * ctx->g.W, cudaMemcpyHostToDevice, s));
     int32_t *h_in = ctx->h_words, *h_out = ctx->h_words + 2 * nb;
     std::memcpy(h_in, env_ids, nn * 4);
     if (t_per_env) std::memcpy(h_in + nn, t_per_env, nn * 4);
@@ -309,9 +332,35 @@ hts_status hts_policy_step_host(hts_ctx* ctx, const uint8_t* obs, const int32_t*
     int32_t *in = direct ? h_in : ctx->s_index, *out = direct ? h_out : ctx->s_result;
     if (!direct) HTS_CUDA(cudaMemcpyAsync(in, h_in, (t_per_env ? 2 : 1) * nn * 4, cudaMemcpyHostToDevice, s));
     float* outf = reinterpret_cast<float*>(out);
-    st = run_step(ctx, ctx->s_obs, Indexing{}, in, t_per_env ? in + nn : nullptr, t, seed, n, out, outf + nn, outf + 2 * nn, outf + 3 * nn,
-                  logits_or_null ? ctx->s_logits : nullptr, s);
-    if (st != HTS_OK) return st;
+    const size_t frame = (size_t)ctx->g.C * ctx->g.H * ctx->g.W;
+    auto step = [&](int row0, int rows) {
+        Indexing ix;
+        ix.row0 = row0;
+        return run_step(ctx, ctx->s_obs + row0 * frame, ix, in + row0, t_per_env ? in + nn + row0 : nullptr, t, seed, rows, out + row0,
+                        outf + nn + row0, outf + 2 * nn + row0, outf + 3 * nn + row0,
+                        logits_or_null ? ctx->s_logits + (size_t)row0 * ctx->g.A : nullptr, s);
+    };
+    const int first = host_first_rows(ctx, n);
+    if (first < n && host_copies_ready(ctx)) {
+        HTS_CUDA(cudaEventRecord(ctx->h_start, s));        // what the stream still does to the caller's frames comes first
+        HTS_CUDA(cudaStreamWaitEvent(ctx->h_stream, ctx->h_start, 0));
+        cudaError_t e = cudaSuccess;
+        for (int part = 0; part < 2 && st == HTS_OK && e == cudaSuccess; ++part) {
+            const int row0 = part ? first : 0, rows = part ? n - first : first;
+            e = cudaMemcpyAsync(ctx->s_obs + row0 * frame, obs + row0 * frame, rows * frame, cudaMemcpyHostToDevice, ctx->h_stream);
+            if (e == cudaSuccess) e = cudaEventRecord(ctx->h_copied[part], ctx->h_stream);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ctx->h_copied[part], 0);
+            if (e == cudaSuccess) st = step(row0, rows);
+        }
+        if (st != HTS_OK || e != cudaSuccess) {
+            cudaStreamSynchronize(ctx->h_stream);          // the caller's buffer is free again
+            return st != HTS_OK ? st : cuda_fail(e, "hts_policy_step_host");
+        }
+    } else {
+        HTS_CUDA(cudaMemcpyAsync(ctx->s_obs, obs, nn * frame, cudaMemcpyHostToDevice, s));
+        st = step(0, n);
+        if (st != HTS_OK) return st;
+    }
     if (!direct) HTS_CUDA(cudaMemcpyAsync(h_out, out, 4 * nn * 4, cudaMemcpyDeviceToHost, s));
     if (logits_or_null)
         HTS_CUDA(cudaMemcpyAsync(logits_or_null, ctx->s_logits, nn * ctx->g.A * 4, cudaMemcpyDeviceToHost, s));
@@ -415,6 +464,8 @@ void hts_policy_destroy(hts_ctx* ctx)
     if (ctx->x3) x3_destroy(ctx->x3);
     for (int i = 0; i < ctx->nalloc; ++i) cudaFree(ctx->allocs[i]);
     if (ctx->h_words) cudaFreeHost(ctx->h_words);
+    for (cudaEvent_t e : {ctx->h_start, ctx->h_copied[0], ctx->h_copied[1]}) if (e) cudaEventDestroy(e);
+    if (ctx->h_stream) cudaStreamDestroy(ctx->h_stream);
     delete ctx;
 }
 

@@ -54,6 +54,7 @@ constexpr int FCB_STAGE_FLOATS = 4 * 32 * 36;   // the epilogue warps' transposi
 struct FcbParams {
     int nk;                             // K chunks of one range
     int n_env;                          // valid rows
+    int row0;                           // the first one's row of the activations
     int m_tiles;                        // row tiles of the batch
     const float* inv_scale;
     float* out_f32;                     // partial planes [range][rows][512]
@@ -116,7 +117,7 @@ fc_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                     const int s = it % FCB_STAGES;
                     if (!mbar_wait(&a_empty[s], (((uint32_t)(it / FCB_STAGES)) & 1u) ^ 1u, abortp, p.status, 71)) { t = my_tiles; break; }
                     mbar_arrive_expect_tx(&a_full[s], A_BYTES);
-                    tma_load_2d(sm_a + s * A_BYTES, &tmA, (range * p.nk + kc) * BK, m0, &a_full[s]);
+                    tma_load_2d(sm_a + s * A_BYTES, &tmA, (range * p.nk + kc) * BK, p.row0 + m0, &a_full[s]);
                 }
             }
         }
@@ -484,16 +485,17 @@ hts_status tc_forward(TcState* t, const uint8_t* obs, const Indexing& ix, int n,
     const Geometry& g = t->g;
     hts_status st;
     const bool dependent = first_layer_dependent(t, s);
+    const size_t row0 = (size_t)ix.row0;
     if (t->stacked && n <= conv_stack_envs(t->stack) * device_sm_count(device_slot())) {
         ConvStackParams c = t->stack;
-        c.obs = obs; c.slots = ix.slots; c.pool = ix.pool; c.n = n;
+        c.obs = obs; c.slots = ix.slots; c.pool = ix.pool; c.n = n; c.row0 = ix.row0;
         prof.begin(K_CONV1, s);
         st = conv_stack_launch(t->mW1, t->mB2, t->mB3, t->mT1, t->mT2, c, dependent, s);
         if (st != HTS_OK) return st;
         prof.end(K_CONV1, s);
     } else {
         prof.begin(K_CONV1, s);
-        st = conv1_launch(t->pl1, t->mW1, t->maps1, obs, ix, n, t->b1, t->inv_scale + L_CONV1, t->a1s, t->max_batch, t->status, dependent, s);
+        st = conv1_launch(t->pl1, t->mW1, t->maps1, obs, ix, n, t->b1, t->inv_scale + L_CONV1, t->a1s + row0 * t->W1s * 128, t->max_batch, t->status, dependent, s);
         if (st != HTS_OK) return st;
         prof.end(K_CONV1, s);
 
@@ -501,19 +503,19 @@ hts_status tc_forward(TcState* t, const uint8_t* obs, const Indexing& ix, int n,
         const size_t nb = (size_t)t->max_batch;
         ConvRowsParams c{};
         c.status = t->status; c.n_env = n;
-        c.W_in = t->W1s; c.H_out = g.H2; c.W_out = g.W2; c.in_plane = (int)(nb * t->W1s);
+        c.W_in = t->W1s; c.H_out = g.H2; c.W_out = g.W2; c.in_plane = (int)(nb * t->W1s); c.col0 = ix.row0 * t->W1s;
         c.tiles = (int)nblk((size_t)n * c.W_in, BM);
         c.bias = t->b2; c.inv_scale = t->inv_scale + L_CONV2;
-        c.out = t->a2; c.out_env = (size_t)g.W2 * 64; c.out_y = nb * g.W2 * 64;
+        c.out_env = (size_t)g.W2 * 64; c.out_y = nb * g.W2 * 64; c.out = t->a2 + row0 * c.out_env;
         prof.begin(K_CONV2, s);
         st = conv_rows_launch<2, 2, 2>(t->mA2, t->mB2, c, s);
         if (st != HTS_OK) return st;
         prof.end(K_CONV2, s);
         // conv3: 3x3 taps on [H2, W2] x 64 -> [H3, W3] x 64, an environment's pixels together: a row of the dense layer's input
-        c.W_in = g.W2; c.H_out = g.H3; c.W_out = g.W3; c.in_plane = (int)(nb * g.W2);
+        c.W_in = g.W2; c.H_out = g.H3; c.W_out = g.W3; c.in_plane = (int)(nb * g.W2); c.col0 = ix.row0 * g.W2;
         c.tiles = (int)nblk((size_t)n * c.W_in, BM);
         c.bias = t->b3; c.inv_scale = t->inv_scale + L_CONV3;
-        c.out = t->a3; c.out_env = (size_t)g.F; c.out_y = (size_t)g.W3 * 64;
+        c.out_env = (size_t)g.F; c.out_y = (size_t)g.W3 * 64; c.out = t->a3 + row0 * c.out_env;
         prof.begin(K_CONV3, s);
         st = conv_rows_launch<3, 3, 1>(t->mA3, t->mB3, c, s);
         if (st != HTS_OK) return st;
@@ -526,13 +528,13 @@ hts_status tc_forward(TcState* t, const uint8_t* obs, const Indexing& ix, int n,
     int slots = device_sm_count(device_slot()) / (4 * t->splits);
     if (slots > m_tiles) slots = m_tiles;
     if (t->cps <= FCB_MAX_NK && slots >= 1 && (m_tiles + slots - 1) / slots <= FCB_MAX_TILES) {
-        const FcbParams fp{t->cps, n, m_tiles, t->inv_scale + L_FC, t->hpart, (size_t)t->max_batch * 512, t->status};
+        const FcbParams fp{t->cps, n, ix.row0, m_tiles, t->inv_scale + L_FC, t->hpart + row0 * 512, (size_t)t->max_batch * 512, t->status};
         t->planes = t->splits;
         t->h_final = false;
         st = launch_fc_resident(t->mAfc, t->mBfc, fp, t->splits, slots, s);
     } else {
         const FcPairPlan plan = fc_pair_plan(n, t->splits);
-        const FcPairParams fp{t->splits, t->cps, plan.group, n, t->bfc, t->inv_scale + L_FC, t->h, t->hpart, (size_t)t->max_batch * 512, t->status};
+        const FcPairParams fp{t->splits, t->cps, plan.group, n, ix.row0, t->bfc, t->inv_scale + L_FC, t->h + row0 * 512, t->hpart + row0 * 512, (size_t)t->max_batch * 512, t->status};
         t->planes = plan.planes;
         t->h_final = plan.planes == 1;
         st = fc_pair_launch(t->mAfc, t->mBfcPair, fp, plan.wide, s);
@@ -546,11 +548,12 @@ hts_status tc_heads(TcState* t, const int32_t* env_ids, const int32_t* t_per_env
                     const Indexing& ix, int32_t* actions, float* logp, float* values, float* entropy, float* logits,
                     cudaStream_t s, const int32_t* given_actions)
 {
+    float *h = t->h + (size_t)ix.row0 * 512, *planes = t->hpart + (size_t)ix.row0 * 512;
     if (t->h_final)        // the FC kernel wrote relu(bias + sum of the K ranges) itself
-        return launch_heads(t->h, 1, 0, nullptr, t->whead, t->bhead, t->g.A, env_ids, t_per_env, tt, seed, n, ix, t->status,
+        return launch_heads(h, 1, 0, nullptr, t->whead, t->bhead, t->g.A, env_ids, t_per_env, tt, seed, n, ix, t->status,
                             actions, logp, values, entropy, logits, nullptr, s, given_actions);
-    return launch_heads(t->hpart, t->planes, (size_t)t->max_batch * 512, t->bfc, t->whead, t->bhead, t->g.A, env_ids,
-                        t_per_env, tt, seed, n, ix, t->status, actions, logp, values, entropy, logits, t->h, s, given_actions);
+    return launch_heads(planes, t->planes, (size_t)t->max_batch * 512, t->bfc, t->whead, t->bhead, t->g.A, env_ids,
+                        t_per_env, tt, seed, n, ix, t->status, actions, logp, values, entropy, logits, h, s, given_actions);
 }
 
 hts_status tc_read_activation(TcState* t, int layer, int n, float* out, cudaStream_t s)

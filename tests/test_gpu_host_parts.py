@@ -1,0 +1,37 @@
+"""Host steps whose frames are copied in two parts: outputs and hidden layers are those of the device step, bit for bit."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import hts_workloads as wl
+import paper_2012_09849_b200 as hts
+from gpu_util import Policy
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("C,H,W,dtype,sizes", [
+    (4, 84, 84, "bf16", (191, 192, 511, 512, 1024, 2500)),        # parts in different kernels: stack and layers, forms of the dense layer
+    (16, 72, 96, "bf16", (193, 530)),
+    (4, 36, 44, "fp32", (511, 512, 901))])
+def test_outputs_and_layers(C, H, W, dtype, sizes):
+    cfg = dataclasses.replace(wl.CONFIGS[2], C=C, H=H, W=W, weight_dtype=dtype)
+    pol = Policy(cfg, max_batch=max(sizes) + 5)
+    try:
+        for n in sizes:
+            obs = wl.make_obs(cfg, n, batch_index=n)
+            ids, t = np.arange(7, 7 + n, dtype=np.int32), (np.arange(n, dtype=np.int32) * 3) % 11
+            dev = pol.step(obs, ids, 2, 5, t_per_env=t)
+            layers = [pol.activation(k, n) for k in (1, 2, 3, 4)]
+            pol.step(obs[::-1], ids, 2, 5, t_per_env=t)            # other contents in the workspaces
+            out = {"actions": np.full(n, -1, np.int32), "logits": np.full((n, cfg.A), np.nan, np.float32),
+                   **{k: np.full(n, np.nan, np.float32) for k in ("logp", "values", "entropy")}}
+            hts.hts_policy_step_host(pol.ctx, obs, ids, t, 2, 5, n, out["actions"], out["logp"], out["values"], out["entropy"], out["logits"])
+            assert hts.hts_last_async_error(pol.ctx) == 0
+            for k, v in out.items():
+                assert np.array_equal(v.view(np.int32), dev[k].view(np.int32)), (n, k)
+            for k, ref in enumerate(layers):
+                assert np.array_equal(pol.activation(k + 1, n).view(np.int32), ref.view(np.int32)), (n, "layer", k + 1)
+    finally:
+        pol.close()
