@@ -151,11 +151,13 @@ constexpr int kHostDirect = 128;
 
 // The frames of a host step are copied in two parts, so that the step of the first runs while the second is copied.  Rows of the
 // first part: all but as many as leave a short step at the end and whose copy outlasts the first step (bf16: a step of 64 or
-// 128 observations takes 18 or 20 us, their copy 33 or 66 us); fp32 steps take as long as their copies: halves.
+// 128 observations takes 18 or 20 us, their copy 33 or 66 us); fp32 steps take as long as their copies: halves.  In two / in one
+// part, us, 84 x 84: 155.8 / 147.2 (192 rows), 179.9 / 183.2 (256), 310 / 325 (512), 576 / 599 (1024), 1102 / 1149 (2048); fp32
+// 551 / 621 (512), 935 / 1093 (1024).
 namespace {
 int host_first_rows(const hts_ctx* ctx, int n)
 {
-    if (ctx->tc) return n >= 512 ? n - 128 : n >= 192 ? n - 64 : n;
+    if (ctx->tc) return n >= 512 ? n - 128 : n >= 256 ? n - 64 : n;
     return n >= 512 ? n / 2 : n;
 }
 // Stream and events of the copies, made by the first call that needs them.

@@ -12,8 +12,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("C,H,W,dtype,sizes", [
-    (4, 84, 84, "bf16", (191, 192, 511, 512, 1024, 2500)),        # parts in different kernels: stack and layers, forms of the dense layer
-    (16, 72, 96, "bf16", (193, 530)),
+    (4, 84, 84, "bf16", (255, 256, 511, 512, 1024, 2500)),        # parts in different kernels: stack and layers, forms of the dense layer
+    (16, 72, 96, "bf16", (257, 530)),
     (4, 36, 44, "fp32", (511, 512, 901))])
 def test_outputs_and_layers(C, H, W, dtype, sizes):
     cfg = dataclasses.replace(wl.CONFIGS[2], C=C, H=H, W=W, weight_dtype=dtype)
