@@ -32,14 +32,25 @@ __device__ __forceinline__ double warp_sum_d(double v)
     return v;
 }
 
+// How a kernel of sums follows the one before it.  Not Alone: that one is a kernel of sums as well, over the same inputs.  It has
+// waited for whatever wrote them, so the first loads (two groups of a thread, all that it has up to kThreads * kPerThread elements
+// to a block) need not wait for it: they are under way while it runs.  Its 48 registers of inputs decide how many blocks an SM
+// holds, so there are two forms.  Standardised means, us, inputs not in cache (both launches):
+//   transitions            131072  300000  600000 | 640000  768000  900000  1000000  2000000  4000000  16000000
+//   Alone, 70 registers       9.6    12.3    14.1 |   13.7    16.2    15.4     20.2     29.0     47.7     116.2
+//   EarlyTwo, 102             8.3     9.7    11.7 |   13.8    16.3    16.0     18.1     28.5     50.3
+//   EarlyThree, 80            8.7     9.9    12.3 |   12.6    14.9    13.9     17.7     26.6     43.8      96.8
+// EarlyTwo while all blocks are on the device at two per SM (606208 transitions on 148 SMs); above that, a third block per SM saves
+// a wave (up to 909312) or covers more latency.
+enum class Form { Alone, EarlyTwo, EarlyThree };
+
 // An Op names NS sums, how four consecutive elements (float4 group q) or one element i add to them, whether
 // its arrays allow float4 loads, and what the last block does with the totals.
-// CHAINED: the kernel before this one is one of these as well, over the same inputs.  It has waited for whatever wrote them, so
-// the first loads need not wait for it: they are under way while it runs (means of 131072 transitions 9.5 -> 8.7 us).
-template <class Op, bool CHAINED>
-__global__ void __launch_bounds__(kThreads)
+template <class Op, Form FORM>
+__global__ void __launch_bounds__(kThreads, FORM == Form::EarlyThree ? 3 : 0)
 sums_kernel(const Op op, long long count, long long per_block)
 {
+    constexpr bool CHAINED = FORM != Form::Alone;
     constexpr int NS = Op::NS;
     __shared__ double s_part[kThreads / 32][NS];
     __shared__ bool s_last;
@@ -53,7 +64,8 @@ sums_kernel(const Op op, long long count, long long per_block)
         const long long q_lo = lo >> 2, q_hi = hi >> 2;                    // whole float4 groups of the range
         long long q = q_lo + threadIdx.x;
         if constexpr (CHAINED) {
-            typename Op::Quad g[2];                                        // two groups are all that a thread of a small problem has
+            static_assert(kPerThread == 8, "two groups are all that a thread of an EarlyTwo block has");
+            typename Op::Quad g[2];
 #pragma unroll
             for (int u = 0; u < 2; ++u) if (q + u * kThreads < q_hi) g[u] = op.load4(q + u * kThreads);
             pdl_wait();
@@ -62,14 +74,17 @@ sums_kernel(const Op op, long long count, long long per_block)
             for (int u = 0; u < 2; ++u) if (q + u * kThreads < q_hi) op.add4(g[u], acc);
             q += 2 * kThreads;
         }
-        for (; q + 3 * kThreads < q_hi; q += 4 * kThreads) {               // four groups per array in flight per thread
-            typename Op::Quad g[4];
+        if constexpr (FORM != Form::EarlyTwo) {
+            constexpr int U = FORM == Form::Alone ? 4 : 2;                 // groups per array in flight per thread
+            for (; q + (U - 1) * kThreads < q_hi; q += U * kThreads) {
+                typename Op::Quad g[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) g[u] = op.load4(q + u * kThreads);
+                for (int u = 0; u < U; ++u) g[u] = op.load4(q + u * kThreads);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) op.add4(g[u], acc);
+                for (int u = 0; u < U; ++u) op.add4(g[u], acc);
+            }
+            for (; q < q_hi; q += kThreads) op.add4(op.load4(q), acc);
         }
-        for (; q < q_hi; q += kThreads) op.add4(op.load4(q), acc);
         for (long long i = (q_hi << 2) + threadIdx.x; i < hi; i += kThreads) op.add1(i, acc);   // the last block's ragged tail
     } else {
         if constexpr (CHAINED) { pdl_wait(); pdl_trigger(); }
@@ -112,15 +127,21 @@ sums_kernel(const Op op, long long count, long long per_block)
     }
 }
 
-template <bool CHAINED = false, class Op>
-hts_status launch_sums(const Op& op, long long count, cudaStream_t s)
+struct SumsGrid { long long blocks, per_block; };
+inline SumsGrid sums_grid(long long count)
 {
     long long blocks = (count + (long long)kThreads * kPerThread - 1) / ((long long)kThreads * kPerThread);
     if (blocks > kBlocksMax) blocks = kBlocksMax;
     long long per_block = (count + blocks - 1) / blocks;
     per_block = (per_block + 3) / 4 * 4;
-    blocks = (count + per_block - 1) / per_block;
-    HTS_CUDA(launch_pdl(sums_kernel<Op, CHAINED>, dim3((unsigned)blocks), dim3(kThreads), 0, s, op, count, per_block));
+    return {(count + per_block - 1) / per_block, per_block};
+}
+
+template <Form FORM = Form::Alone, class Op>
+hts_status launch_sums(const Op& op, long long count, cudaStream_t s)
+{
+    const SumsGrid g = sums_grid(count);
+    HTS_CUDA(launch_pdl(sums_kernel<Op, FORM>, dim3((unsigned)g.blocks), dim3(kThreads), 0, s, op, count, g.per_block));
     note_launch();
     return HTS_OK;
 }
@@ -186,6 +207,9 @@ struct AdvStatsOp {
     }
 };
 
+// IN_TURN: an element's sums are finished before the next one's are begun (the compiler otherwise works on all eight of two groups
+// at once, 110 registers).
+template <bool IN_TURN>
 struct PpoOp {
     static constexpr int NS = 4;
     const float *logp_new, *logp_old, *values, *entropy, *adv, *returns;
@@ -211,11 +235,18 @@ struct PpoOp {
         acc[2] += (double)h;
         acc[3] += fabs(rho - 1.0) > clip ? 1.0 : 0.0;
     }
-    __device__ void add4(const Quad& g, double* acc) const
+    __device__ static void in_turn(float& ln, float& lo, float& v, float& a, float& r, double* acc)
+    {
+        if constexpr (IN_TURN)
+            asm volatile("" : "+f"(ln), "+f"(lo), "+f"(v), "+f"(a), "+f"(r), "+d"(acc[0]), "+d"(acc[1]), "+d"(acc[2]), "+d"(acc[3]));
+    }
+    __device__ void add4(Quad g, double* acc) const
     {
         const double m = normalize ? g_adv_stats[0] : 0.0, is = normalize ? g_adv_stats[1] : 1.0;
-        one(g.ln.x, g.lo.x, g.v.x, g.h.x, g.a.x, g.r.x, m, is, acc); one(g.ln.y, g.lo.y, g.v.y, g.h.y, g.a.y, g.r.y, m, is, acc);
-        one(g.ln.z, g.lo.z, g.v.z, g.h.z, g.a.z, g.r.z, m, is, acc); one(g.ln.w, g.lo.w, g.v.w, g.h.w, g.a.w, g.r.w, m, is, acc);
+        in_turn(g.ln.x, g.lo.x, g.v.x, g.a.x, g.r.x, acc); one(g.ln.x, g.lo.x, g.v.x, g.h.x, g.a.x, g.r.x, m, is, acc);
+        in_turn(g.ln.y, g.lo.y, g.v.y, g.a.y, g.r.y, acc); one(g.ln.y, g.lo.y, g.v.y, g.h.y, g.a.y, g.r.y, m, is, acc);
+        in_turn(g.ln.z, g.lo.z, g.v.z, g.a.z, g.r.z, acc); one(g.ln.z, g.lo.z, g.v.z, g.h.z, g.a.z, g.r.z, m, is, acc);
+        in_turn(g.ln.w, g.lo.w, g.v.w, g.a.w, g.r.w, acc); one(g.ln.w, g.lo.w, g.v.w, g.h.w, g.a.w, g.r.w, m, is, acc);
     }
     __device__ void add1(long long i, double* acc) const
     {
@@ -253,9 +284,14 @@ extern "C" hts_status hts_ppo_terms(const float* logp_new, const float* logp_old
         const hts_status st = launch_sums(AdvStatsOp{advantages, all_aligned16({advantages})}, (long long)count, s);
         if (st != HTS_OK) return st;
     }
-    const PpoOp op{logp_new, logp_old, values, entropy, advantages, returns, out4, (double)clip, normalize_advantages != 0,
-                   all_aligned16({logp_new, logp_old, values, entropy, advantages, returns})};
-    return normalize_advantages ? launch_sums<true>(op, (long long)count, s) : launch_sums(op, (long long)count, s);
+    const bool vec = all_aligned16({logp_new, logp_old, values, entropy, advantages, returns});
+    const PpoOp<false> op{logp_new, logp_old, values, entropy, advantages, returns, out4, (double)clip, normalize_advantages != 0, vec};
+    if (!normalize_advantages) return launch_sums(op, (long long)count, s);
+    const SumsGrid grid = sums_grid((long long)count);
+    if (grid.blocks <= 2LL * device_sm_count(device_slot()) && grid.per_block <= kThreads * kPerThread)
+        return launch_sums<Form::EarlyTwo>(op, (long long)count, s);
+    return launch_sums<Form::EarlyThree>(PpoOp<true>{logp_new, logp_old, values, entropy, advantages, returns, out4, (double)clip, true, vec},
+                                         (long long)count, s);
 }
 
 // ---- the learner's parameter update (Section 4.1 "Delayed gradient", Eq. 5) ---------------------------------
