@@ -149,16 +149,31 @@ hts_status run_step(hts_ctx* ctx, const uint8_t* obs, const Indexing& ix, const 
 // 2265 / 2258 (4096), 4484 / 4461 (8192): the two cross between 2048 and 4096 rows, so the line could lie higher.
 constexpr int kHostDirect = 128;
 
-// The frames of a host step are copied in two parts, so that the step of the first runs while the second is copied.  Rows of the
-// first part: all but as many as leave a short step at the end and whose copy outlasts the first step (bf16: a step of 64 or
-// 128 observations takes 18 or 20 us, their copy 33 or 66 us); fp32 steps take as long as their copies: halves.  In two / in one
-// part, us, 84 x 84: 155.8 / 147.2 (192 rows), 179.9 / 183.2 (256), 310 / 325 (512), 576 / 599 (1024), 1102 / 1149 (2048); fp32
-// 551 / 621 (512), 935 / 1093 (1024).
+// The frames of a host step are copied in two parts, so that the step of the first runs while the second is copied.  It pays if
+// the second part's copy outlasts the first part's step, and if what then remains, the second part's step, is shorter than the
+// whole one by more than another copy and chain of launches cost.
+// bf16: a step of n rows takes 16 to 20 us and a sixteenth (60 x 60) to a forty-fifth (72 x 96, 16 channels) of what the n frames'
+// copy takes (55 bytes per ns), so the second part is 2 MB and an eighteenth of all bytes.  Host step with second parts of fewer rows /
+// about as many / more, us: 1024 of 84 x 84 x 4 593.8 (48 rows) / 575 (96 to 128) / 577.6 (144); 512 of 72 x 96 x 16 1082.1 (16) / 1079.6
+// (48) / 1082.3 (128); 512 of 84 x 84 x 8 579.7 (32) / 577.6 (64) / 579.2 (128); 2048 of 36 x 44 299.3 (128) / 287.7 (448) / 291.4 (640).
+// Small frames' steps save less than their share of the bytes: the line is 5.2 MB and 4 KB for each row.  One part / two, us:
+//   36 x 44 x 4   6 MB 158.9 / 164.8   7 MB 177.5 / 187.1   10 MB 236.4 / 236.0   14 MB 315.3 / 315.2   20 MB 433.2 / 427.5   51 MB 1021 / 993
+//   60 x 60 x 4   6 MB 158.3 / 161.4   7 MB 176.5 / 181.8   8 MB 201.4 / 198.5    12 MB 274.3 / 273.6   16 MB 354.8 / 339.5   40 MB 810 / 780
+//   64 x 96 x 4   6.3 MB 165.8 / 162.8   8 MB 198.5 / 194.0   12 MB 274.1 / 265.3   24 MB 502.5 / 487.9
+//   84 x 84 x 4   7.2 MB 182.6 / 181.9   8 MB 197.8 / 193.9   12 MB 273.1 / 266.6   28.9 MB 595.9 / 575.7   57.8 MB 1141 / 1104
+//   84 x 84 x 8   14.5 MB 316.8 / 314.3   29 MB 584.7 / 578.2   57 MB 1107 / 1086
+//   72 x 96 x 16   28.4 MB 570.7 / 567.0   57 MB 1097 / 1086   110 MB 2071 / 2042
+// and 256 rows: below two per SM the step is one observation's latency, whatever it is cut into (159 of 84 x 84 x 8 216.0 / 216.3, 124
+// of them 174.9 / 186.4; 144 of 72 x 96 x 16 343.1 / 342.7).
+// fp32 steps take as long as their copies: halves, from 512 rows.  513 of 84 x 84 x 4 618.8 / 557.1, 631 of 36 x 44 191.4 / 183.3 (394 of
+// them 139.3 / 144.8), 515 of 72 x 96 x 16 1567 / 1346.
 namespace {
 int host_first_rows(const hts_ctx* ctx, int n)
 {
-    if (ctx->tc) return n >= 512 ? n - 128 : n >= 256 ? n - 64 : n;
-    return n >= 512 ? n / 2 : n;
+    if (!ctx->tc) return n >= 512 ? n / 2 : n;
+    const long long frame = (long long)ctx->g.C * ctx->g.H * ctx->g.W, bytes = n * frame;
+    if (n < 256 || bytes < 5200000 + 4000LL * n) return n;
+    return n - (int)((2000000 + bytes / 18 + frame - 1) / frame);
 }
 // Stream and events of the copies, made by the first call that needs them.
 bool host_copies_ready(hts_ctx* c)

@@ -14,6 +14,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("C,H,W,dtype,sizes", [
     (4, 84, 84, "bf16", (255, 256, 511, 512, 1024, 2500)),        # parts in different kernels: stack and layers, forms of the dense layer
     (16, 72, 96, "bf16", (257, 530)),
+    (4, 36, 44, "bf16", (2226, 2227, 2600)),                      # the line lies between the first two
     (4, 36, 44, "fp32", (511, 512, 901))])
 def test_outputs_and_layers(C, H, W, dtype, sizes):
     cfg = dataclasses.replace(wl.CONFIGS[2], C=C, H=H, W=W, weight_dtype=dtype)
@@ -33,5 +34,25 @@ def test_outputs_and_layers(C, H, W, dtype, sizes):
                 assert np.array_equal(v.view(np.int32), dev[k].view(np.int32)), (n, k)
             for k, ref in enumerate(layers):
                 assert np.array_equal(pol.activation(k + 1, n).view(np.int32), ref.view(np.int32)), (n, "layer", k + 1)
+    finally:
+        pol.close()
+
+
+@pytest.mark.parametrize("C,H,W,cut,whole", [
+    (4, 36, 44, (2227, 2600), (256, 512, 1105, 2226)),            # few bytes: no step hides behind the second part's copy
+    (4, 84, 84, (256, 512), (248, 255)),
+    (16, 72, 96, (256,), (64, 255))])                             # few rows: their step is one observation's latency
+def test_parts_by_bytes_and_rows(C, H, W, cut, whole):
+    """Frames are copied in two parts, each with a step of its own, from 256 rows and 5.2 MB and 4 KB a row on."""
+    cfg = dataclasses.replace(wl.CONFIGS[2], C=C, H=H, W=W)
+    pol = Policy(cfg, max_batch=max(cut))
+    try:
+        for n in cut + whole:
+            obs = np.zeros((n, C, H, W), np.uint8)
+            ids = np.arange(n, dtype=np.int32)
+            out = [np.empty(n, d) for d in (np.int32, np.float32, np.float32, np.float32)]
+            before = hts.hts_launch_count()
+            hts.hts_policy_step_host(pol.ctx, obs, ids, None, 0, 5, n, *out)
+            assert (hts.hts_launch_count() - before > 5) == (n in cut), n      # a step is three or five kernels
     finally:
         pol.close()
