@@ -36,7 +36,7 @@ struct hts_ctx {
     uint8_t* s_obs = nullptr;
     int32_t *s_index = nullptr, *s_result = nullptr, *h_words = nullptr;
     float* s_logits = nullptr;
-    cudaStream_t h_stream = nullptr;    // its frames' copies, where they are cut in two
+    cudaStream_t h_stream = nullptr;    // its frames' copies, where they are cut in two; null if no batch of the context is
     cudaEvent_t h_start = nullptr, h_copied[2] = {nullptr, nullptr};
     X3State* x3 = nullptr;        // packed weights and workspace of the gradient (weight_dtype fp32)
     int* status = nullptr;        // device status word
@@ -175,14 +175,17 @@ int host_first_rows(const hts_ctx* ctx, int n)
     if (n < 256 || bytes < 5200000 + 4000LL * n) return n;
     return n - (int)((2000000 + bytes / 18 + frame - 1) / frame);
 }
-// Stream and events of the copies, made by the first call that needs them.
-bool host_copies_ready(hts_ctx* c)
+// Stream and events of the copies.  A stream takes 56 to 66 us to make, more than a cut saves: it is made with the context, if the
+// context's largest batch is cut.  Without them frames are copied in one part.
+void make_host_copies(hts_ctx* c)
 {
-    if (!c->h_stream && cudaStreamCreateWithFlags(&c->h_stream, cudaStreamNonBlocking) != cudaSuccess) c->h_stream = nullptr;
-    for (cudaEvent_t* e : {&c->h_start, &c->h_copied[0], &c->h_copied[1]})
-        if (!*e && cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) *e = nullptr;
-    cudaGetLastError();
-    return c->h_stream && c->h_start && c->h_copied[0] && c->h_copied[1];
+    if (host_first_rows(c, c->desc.max_batch) == c->desc.max_batch) return;
+    bool ok = true;
+    for (cudaEvent_t* e : {&c->h_start, &c->h_copied[0], &c->h_copied[1]}) ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+    if (!ok || cudaStreamCreateWithFlags(&c->h_stream, cudaStreamNonBlocking) != cudaSuccess) {
+        c->h_stream = nullptr;
+        cudaGetLastError();
+    }
 }
 }  // namespace
 
@@ -243,6 +246,7 @@ hts_status hts_policy_create(const hts_net_desc* d, hts_ctx** out)
         hts_policy_destroy(c);
         return st;
     }
+    make_host_copies(c);
     *out = c;
     return HTS_OK;
 }
@@ -358,7 +362,7 @@ hts_status hts_policy_step_host(hts_ctx* ctx, const uint8_t* obs, const int32_t*
                         logits_or_null ? ctx->s_logits + (size_t)row0 * ctx->g.A : nullptr, s);
     };
     const int first = host_first_rows(ctx, n);
-    if (first < n && host_copies_ready(ctx)) {
+    if (first < n && ctx->h_stream) {
         HTS_CUDA(cudaEventRecord(ctx->h_start, s));        // what the stream still does to the caller's frames comes first
         HTS_CUDA(cudaStreamWaitEvent(ctx->h_stream, ctx->h_start, 0));
         cudaError_t e = cudaSuccess;

@@ -1,4 +1,5 @@
 """Host steps whose frames are copied in two parts: outputs and hidden layers are those of the device step, bit for bit."""
+import ctypes
 import dataclasses
 
 import numpy as np
@@ -54,5 +55,31 @@ def test_parts_by_bytes_and_rows(C, H, W, cut, whole):
             before = hts.hts_launch_count()
             hts.hts_policy_step_host(pol.ctx, obs, ids, None, 0, 5, n, *out)
             assert (hts.hts_launch_count() - before > 5) == (n in cut), n      # a step is three or five kernels
+    finally:
+        pol.close()
+
+
+def _next_stream_id():
+    """Streams of a process are numbered as they are made."""
+    cuda, s, i = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(), ctypes.c_ulonglong()
+    assert cuda.cuStreamCreate(ctypes.byref(s), 1) == 0 and cuda.cuStreamGetId(s, ctypes.byref(i)) == 0
+    assert cuda.cuStreamDestroy_v2(s) == 0
+    return i.value
+
+
+@pytest.mark.parametrize("dtype,max_batch,made", [("bf16", 256, 1), ("bf16", 255, 0), ("fp32", 512, 1), ("fp32", 511, 0)])
+def test_no_call_makes_a_stream(dtype, max_batch, made):
+    """The stream of the copies is made with the context, and only if its batches can be cut."""
+    cfg = dataclasses.replace(wl.CONFIGS[2], weight_dtype=dtype)
+    assert _next_stream_id() + 1 == _next_stream_id()
+    before = _next_stream_id()
+    pol = Policy(cfg, max_batch=max_batch)
+    try:
+        created = _next_stream_id()
+        assert created - before == 1 + made
+        out = [np.empty(max_batch, d) for d in (np.int32, np.float32, np.float32, np.float32)]
+        hts.hts_policy_step_host(pol.ctx, np.zeros((max_batch, cfg.C, cfg.H, cfg.W), np.uint8), np.arange(max_batch, dtype=np.int32), None, 0, 5,
+                                 max_batch, *out)
+        assert _next_stream_id() - created == 1
     finally:
         pol.close()
