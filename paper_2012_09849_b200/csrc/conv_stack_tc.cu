@@ -3,7 +3,7 @@
 //
 // For batches of a few environments per SM, where three kernels spend their time between them: each starts 1.3 us after
 // the last CTA of the one before and needs 2 us to its first finished tile.  Step of 16 observations: 20.5 -> 16.9 us, of 256: 27.3
-// -> 24.5, of 444: 31.6 -> 29.1; five to six environments per SM are equal (conv_stack_envs).  From there on the three
+// -> 24.5, of 444: 31.6 -> 29.1; at five environments per SM they are equal (conv_stack_envs).  From there on the three
 // kernels win: one environment here takes about 7800 clocks where its MMAs need 4288,
 // because those fetch their operands from the same shared memory (128 bytes per clock, 68 x 6 KB per environment) that the
 // converters and epilogues work in.  The activations never leave the SM between layers: a CTA keeps one frame (raw bytes), conv1's output (K-major 128-byte-swizzled rows, two
