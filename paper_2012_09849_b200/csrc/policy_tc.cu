@@ -38,7 +38,7 @@ constexpr int BK = 64;                  // 16-bit elements per K chunk = one 128
 constexpr int A_BYTES = BM * BK * 2;    // 16 KiB
 enum { L_CONV1 = 0, L_CONV2, L_CONV3, L_FC, L_COUNT };
 
-// ---- FC for small batches with the weights resident: one CTA per (column tile, K range) and slot of row tiles.
+// ---- FC for small batches with the weights resident: one CTA per (column tile, K range, row tile).
 // A CTA asks for its whole weight slice (nk chunks of 128 x 64) before it waits for the previous kernel; a CTA of
 // this kernel cannot start before the previous kernel's CTA has left its SM, but the hand-over from the last of
 // those to the release of the wait (about 1.4 us) is enough for most of the slice.  After the wait only
@@ -48,14 +48,12 @@ enum { L_CONV1 = 0, L_CONV2, L_CONV3, L_FC, L_COUNT };
 // there: the same bits.
 constexpr int FCB_STAGES = 5;                   // activation chunks in flight (16 KiB each)
 constexpr int FCB_MAX_NK = 7;                   // weight chunks a CTA can keep: 7 x 16 KiB
-constexpr int FCB_MAX_TILES = 1;                // row tiles of a CTA (accumulators of 128 columns)
 constexpr int FCB_STAGE_FLOATS = 4 * 32 * 36;   // the epilogue warps' transposing buffers
 
 struct FcbParams {
     int nk;                             // K chunks of one range
     int n_env;                          // valid rows
     int row0;                           // the first one's row of the activations
-    int m_tiles;                        // row tiles of the batch
     const float* inv_scale;
     float* out_f32;                     // partial planes [range][rows][512]
     size_t split_stride;
@@ -68,7 +66,7 @@ fc_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     constexpr int BN = 128;
     constexpr int B_BYTES = BN * BK * 2;
     extern __shared__ uint8_t smem_raw[];
-    constexpr int kBars = FCB_MAX_NK + 2 * FCB_STAGES + FCB_MAX_TILES;
+    constexpr int kBars = FCB_MAX_NK + 2 * FCB_STAGES + 1;
     __shared__ uint64_t bars[kBars];
     uint64_t *b_full = bars, *a_full = bars + FCB_MAX_NK, *a_empty = a_full + FCB_STAGES, *acc_full = a_empty + FCB_STAGES;
     __shared__ uint32_t tmem_base_slot;
@@ -80,8 +78,7 @@ fc_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     const uint32_t a_base = base + FCB_MAX_NK * B_BYTES;
     float* sm_stage = reinterpret_cast<float*>(sm_a + FCB_STAGES * A_BYTES);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n0 = blockIdx.x * BN, range = blockIdx.y, slot = blockIdx.z, slots = gridDim.z;
-    const int my_tiles = slot < p.m_tiles ? (p.m_tiles - slot + slots - 1) / slots : 0;   // <= FCB_MAX_TILES (launcher)
+    const int n0 = blockIdx.x * BN, range = blockIdx.y, m0 = blockIdx.z * BM;
     volatile int* abortp = &abort_flag;
 
     if (warp == 0) {
@@ -96,7 +93,7 @@ fc_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             }
         }
     } else if (warp == 1) {
-        tmem_alloc(&tmem_base_slot, FCB_MAX_TILES * BN);
+        tmem_alloc(&tmem_base_slot, BN);
     } else if (warp == 2 && lane == 0) {
         abort_flag = 0;
         tma_prefetch_desc(&tmA);
@@ -110,37 +107,30 @@ fc_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
 
     if (warp == 0) {
         if (lane == 0) {
-            int it = 0;
-            for (int t = 0; t < my_tiles; ++t) {
-                const int m0 = (slot + t * slots) * BM;
-                for (int kc = 0; kc < p.nk; ++kc, ++it) {
-                    const int s = it % FCB_STAGES;
-                    if (!mbar_wait(&a_empty[s], (((uint32_t)(it / FCB_STAGES)) & 1u) ^ 1u, abortp, p.status, 71)) { t = my_tiles; break; }
-                    mbar_arrive_expect_tx(&a_full[s], A_BYTES);
-                    tma_load_2d(sm_a + s * A_BYTES, &tmA, (range * p.nk + kc) * BK, p.row0 + m0, &a_full[s]);
-                }
+            for (int kc = 0; kc < p.nk; ++kc) {
+                const int s = kc % FCB_STAGES;
+                if (!mbar_wait(&a_empty[s], (((uint32_t)(kc / FCB_STAGES)) & 1u) ^ 1u, abortp, p.status, 71)) break;
+                mbar_arrive_expect_tx(&a_full[s], A_BYTES);
+                tma_load_2d(sm_a + s * A_BYTES, &tmA, (range * p.nk + kc) * BK, p.row0 + m0, &a_full[s]);
             }
         }
     } else if (warp == 1) {
         if (lane == 0) {
             constexpr uint32_t idesc = instr_desc_f16(0, BM, BN);
-            int it = 0;
             bool alive = true;
-            for (int t = 0; alive && t < my_tiles; ++t) {
-                for (int kc = 0; kc < p.nk; ++kc, ++it) {
-                    const int s = it % FCB_STAGES;
-                    if (t == 0 && !mbar_wait(&b_full[kc], 0, abortp, p.status, 72)) { alive = false; break; }
-                    if (!mbar_wait(&a_full[s], ((uint32_t)(it / FCB_STAGES)) & 1u, abortp, p.status, 73)) { alive = false; break; }
-                    tc_fence_after();
-                    const uint64_t adesc = smem_desc_sw128(a_base + s * A_BYTES);
-                    const uint64_t bdesc = smem_desc_sw128(base + kc * B_BYTES);
+            for (int kc = 0; kc < p.nk; ++kc) {
+                const int s = kc % FCB_STAGES;
+                if (!mbar_wait(&b_full[kc], 0, abortp, p.status, 72)) { alive = false; break; }
+                if (!mbar_wait(&a_full[s], ((uint32_t)(kc / FCB_STAGES)) & 1u, abortp, p.status, 73)) { alive = false; break; }
+                tc_fence_after();
+                const uint64_t adesc = smem_desc_sw128(a_base + s * A_BYTES);
+                const uint64_t bdesc = smem_desc_sw128(base + kc * B_BYTES);
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        mma_f16_ss(tmem_d + t * BN, adesc + 2 * k, bdesc + 2 * k, idesc, (kc | k) != 0);
-                    mma_commit(&a_empty[s]);
-                }
-                if (alive) mma_commit(&acc_full[t]);
+                for (int k = 0; k < BK / 16; ++k)
+                    mma_f16_ss(tmem_d, adesc + 2 * k, bdesc + 2 * k, idesc, (kc | k) != 0);
+                mma_commit(&a_empty[s]);
             }
+            if (alive) mma_commit(acc_full);
         }
     } else {
         // epilogue warps 2..5: warp w may touch TMEM lanes [32*(w%4), 32*(w%4)+32)
@@ -148,17 +138,15 @@ fc_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         const float inv = *p.inv_scale;
         float* stage = sm_stage + (warp - 2) * (32 * 36);
         const int rl = lane >> 3, c4 = (lane & 7) * 4;
-        for (int t = 0; t < my_tiles; ++t) {
-            if (!mbar_wait_warp(&acc_full[t], 0, abortp, p.status, 74)) break;
+        if (mbar_wait_warp(acc_full, 0, abortp, p.status, 74)) {
             tc_fence_after();
-            const int m0 = (slot + t * slots) * BM;
             // one row per thread arrives; each warp turns its 32 x 32 blocks through shared memory so that eight
             // lanes write one full 128-byte line
             float* dst = p.out_f32 + range * p.split_stride + (size_t)(m0 + q * 32) * 512 + n0;
 #pragma unroll
             for (int c = 0; c < BN; c += 32) {
                 uint32_t v[32];
-                tmem_ld_32x32(tmem_d + ((uint32_t)(q * 32) << 16) + t * BN + c, v);
+                tmem_ld_32x32(tmem_d + ((uint32_t)(q * 32) << 16) + c, v);
                 tmem_ld_wait();
 #pragma unroll
                 for (int j = 0; j < 32; j += 4)
@@ -182,7 +170,7 @@ fc_resident_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_d, FCB_MAX_TILES * BN);
+    if (warp == 1) tmem_dealloc(tmem_d, BN);
 }
 
 // ---- weight scaling and packing ---------------------------------------------------------------
@@ -332,13 +320,13 @@ __global__ void tap_rows_kernel(const __half* __restrict__ src, float* __restric
 
 inline unsigned nblk(size_t total, int th) { return (unsigned)((total + th - 1) / th); }
 
-hts_status launch_fc_resident(const CUtensorMap& a, const CUtensorMap& b, const FcbParams& p, int ranges, int slots,
+hts_status launch_fc_resident(const CUtensorMap& a, const CUtensorMap& b, const FcbParams& p, int ranges, int m_tiles,
                               cudaStream_t s)
 {
     constexpr int smem = FCB_MAX_NK * 128 * BK * 2 + FCB_STAGES * A_BYTES + FCB_STAGE_FLOATS * 4 + 1024;
     static OncePerDevice allowed;
     HTS_CUDA(allow_shared(fc_resident_kernel, allowed));
-    HTS_CUDA(launch_pdl(fc_resident_kernel, dim3(4, ranges, slots), dim3(192), (size_t)smem, s, a, b, p));
+    HTS_CUDA(launch_pdl(fc_resident_kernel, dim3(4, ranges, m_tiles), dim3(192), (size_t)smem, s, a, b, p));
     note_launch();
     return HTS_OK;
 }
@@ -525,13 +513,11 @@ hts_status tc_forward(TcState* t, const uint8_t* obs, const Indexing& ix, int n,
     // CTA gets one row tile, pairs of SMs otherwise.
     prof.begin(K_FC, s);
     const int m_tiles = (int)nblk(n, BM);
-    int slots = device_sm_count(device_slot()) / (4 * t->splits);
-    if (slots > m_tiles) slots = m_tiles;
-    if (t->cps <= FCB_MAX_NK && slots >= 1 && (m_tiles + slots - 1) / slots <= FCB_MAX_TILES) {
-        const FcbParams fp{t->cps, n, ix.row0, m_tiles, t->inv_scale + L_FC, t->hpart + row0 * 512, (size_t)t->max_batch * 512, t->status};
+    if (t->cps <= FCB_MAX_NK && m_tiles <= device_sm_count(device_slot()) / (4 * t->splits)) {
+        const FcbParams fp{t->cps, n, ix.row0, t->inv_scale + L_FC, t->hpart + row0 * 512, (size_t)t->max_batch * 512, t->status};
         t->planes = t->splits;
         t->h_final = false;
-        st = launch_fc_resident(t->mAfc, t->mBfc, fp, t->splits, slots, s);
+        st = launch_fc_resident(t->mAfc, t->mBfc, fp, t->splits, m_tiles, s);
     } else {
         const FcPairPlan plan = fc_pair_plan(n, t->splits);
         const FcPairParams fp{t->splits, t->cps, plan.group, n, ix.row0, t->bfc, t->inv_scale + L_FC, t->h + row0 * 512, t->hpart + row0 * 512, (size_t)t->max_batch * 512, t->status};
