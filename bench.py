@@ -15,8 +15,10 @@ its own range of environment ids; there is no data-path collective.
 from __future__ import annotations
 
 import argparse
+import hashlib
 import json
 import os
+import re
 import subprocess
 import sys
 import threading
@@ -31,13 +33,29 @@ if ROOT not in sys.path:
 import hts_workloads as wl  # noqa: E402
 
 WORKLOAD = 3                       # hts_workloads.CONFIGS index
-# dram__bytes_read.sum + dram__bytes_write.sum of one launch of a kernel at this workload (n = 1024), from one ncu
-# capture of that kernel; None once the kernel has changed since its counters were taken
-DRAM_TRAFFIC_BYTES = {"conv1": 28953344 + 242432, "conv2": None, "conv3": None, "fc": None, "heads": None}
+# dram__bytes_read.sum + dram__bytes_write.sum of one launch of a kernel at this workload (n = 1024), from one ncu capture of the
+# five (profiles/actor_step_rows_pairs.md), the kernel's source and that one's digest when they were taken
+DRAM_TRAFFIC = {"conv1": (28956416 + 313344, "conv1_tc.cu", "493a8205d6e7"), "conv2": (26305024, "conv_res_tc.cu", "c91b7de800dc"),
+                "conv3": (10714624, "conv_res_tc.cu", "c91b7de800dc"), "fc": (9659392, "fc_tc.cu", "db09713381ee"),
+                "heads": (14763776, "heads.cu", "533d268a2788")}
+CSRC = os.path.join(ROOT, "paper_2012_09849_b200", "csrc")
 DTYPE = "bf16 weights, fp16 operands, fp32 accumulate"
 METRIC = "actor env-steps/s (whole rollout: T actor steps + GAE)"
 UNIT = "env-steps/s"
 SEED = 0x5EED
+
+
+def source_digest(path) -> str:
+    """Digest of a C++ source without its comments."""
+    with open(path, encoding="utf-8") as f:
+        code = re.sub(r"//[^\n]*|/\*.*?\*/", " ", f.read(), flags=re.S)
+    return hashlib.sha256(" ".join(code.split()).encode()).hexdigest()[:12]
+
+
+def dram_traffic(kernel):
+    """Counted bytes of a launch; None once the kernel's source has changed since they were counted."""
+    count, source, digest = DRAM_TRAFFIC[kernel]
+    return count if source_digest(os.path.join(CSRC, source)) == digest else None
 
 
 def macs_per_env_step(cfg) -> int:
@@ -472,7 +490,7 @@ def run_ours(args) -> None:
                 "frac": achieved_tf / peak_burst, "frac_burst": achieved_tf / peak_burst,
                 "frac_sustained": achieved_tf / peak_tf, "peak_sustained": peak_tf,
                 "peak_kind": peak_kind + " burst (the timed region is a fraction of a second at full clocks)",
-                "traffic": DRAM_TRAFFIC_BYTES.get(top),
+                "traffic": dram_traffic(top),
                 "algorithmic_bytes": N * obs_bytes if top == "conv1" else None,
                 "us_per_launch": top_us}
     for name, kk in kern.items():
