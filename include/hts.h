@@ -241,7 +241,8 @@ hts_status hts_delayed_update(float *theta, const float *grad, float *sq_avg_or_
  * runs the step, copies the four outputs (and logits if asked) back and waits for
  * them.  Uses staging buffers owned by the context (24 max_batch bytes of pinned host
  * memory among them, allocated by the first call), so calls on one context must not
- * overlap.
+ * overlap.  Larger batches' frames are copied in two parts on a stream of the context's,
+ * between what cuda_stream does before and after.
  * Pinned host memory makes the copies asynchronous but is not required.           */
 hts_status hts_policy_step_host(hts_ctx *ctx, const uint8_t *obs, const int32_t *env_ids,
                                 const int32_t *t_per_env, int32_t t, uint64_t seed, int32_t n,

@@ -72,6 +72,7 @@ __device__ __forceinline__ void finish16(const uint32_t* v, float inv, const flo
 }
 
 // WC: the frame width when known at compile time (the converter's loads then use immediate offsets), 0 = any.
+// 1024 threads leave 64 registers to each: the compiler spills 8 bytes.
 template <int WC>
 __global__ void __launch_bounds__(kStackThreads)
 conv_stack_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,

@@ -81,7 +81,7 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar)
                  ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
 }
 
-// ONE: each pair has one range and hands it on as it is.
+// ONE: each pair has one range and hands it on as it is.  <256, true> takes 64 registers and spills 16 bytes.
 template <int BN, bool ONE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads)
 fc_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const FcPairParams p)

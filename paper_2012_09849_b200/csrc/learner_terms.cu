@@ -4,7 +4,7 @@
 //   hts_ppo_terms  the clipped surrogate of proximal policy optimisation (Schulman et al. 2017, Eq. 7), the
 //                  algorithm the football runs of Section 5 use, with the same value loss and entropy.
 //
-// HBM-bound (16 to 24 bytes per transition).  Each block sums a contiguous range in double precision in a
+// HBM-bound (16 to 28 bytes per transition).  Each block sums a contiguous range in double precision in a
 // fixed order (thread-strided float4 loads, shuffle tree, warp order), writes its partial and takes a
 // ticket; the block that draws the last ticket adds the partials in a fixed order.  The grid is a
 // function of the count alone, so the result does not depend on timing or on the device's load.

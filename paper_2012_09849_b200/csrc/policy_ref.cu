@@ -86,6 +86,9 @@ __device__ __forceinline__ size_t plane_row(const ConvParams& p, int e, int r)
 // quarter differ, 2 where they agree; pairs of pixels, with the weights in both lanes, take 16 clocks a step instead of 12:
 // 193 / 181 / 119).  8 x 16 per thread loads less but leaves two warps per scheduler: 206 against 171 us (conv2, n = 1024);
 // copying input rows instead of gathering per tap makes the reads scattered: 278 us.
+// What keeps it from 64 TFLOP/s (28 to 44 are reached, and no unit is busy for more than 81 % of the time): inputs are gathered four bytes
+// at a time; weights are turned through eight registers a thread in every block and chunk, under a cap of 128 (the conv2 / conv3 form
+// spills 4 bytes); two to four warps per scheduler cover the rest.
 template <typename TIn, int PXT, int OT, int WPX, int WO, int KC, int PER_SM>
 __global__ void __launch_bounds__(32 * WPX * WO, PER_SM)
 conv_tile_kernel(const ConvParams p)
