@@ -72,6 +72,8 @@ struct LoadParams {
     float* wf_dst;
     LoadItem conv[2];                   // conv2, conv3: copied and packed
     LoadItem rest[9];                   // copied
+    LoadItem turned[3];                 // conv1, conv2, conv3: [O][K] as [K][O]
+    int turned_k[3];
     int P3;
     bf16 *w2p, *w3p, *wfp;              // nullptr: only copied
 };
@@ -129,6 +131,15 @@ __global__ void __launch_bounds__(256) load_fp32_kernel(const LoadParams p)
             return;
         }
         i -= p.rest[k].n;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (i < p.turned[k].n) {
+            const int O = k == 0 ? 32 : 64;
+            p.turned[k].dst[i] = p.turned[k].src[i % O * p.turned_k[k] + i / O];
+            return;
+        }
+        i -= p.turned[k].n;
     }
 }
 
@@ -492,10 +503,12 @@ hts_status x3_load_weights(X3State* t, const hts_weights& w, const RefWeights& d
                        {{f(w.conv1_w), d.w1, 32 * 64 * t->g.C}, {f(w.conv1_b), d.b1, 32}, {f(w.conv2_b), d.b2, 64}, {f(w.conv3_b), d.b3, 64},
                         {f(w.fc_b), d.bfc, 512}, {f(w.pi_w), d.whead, A * 512}, {f(w.v_w), d.whead + A * 512, 512}, {f(w.pi_b), d.bhead, A},
                         {f(w.v_b), d.bhead + A, 1}},
-                       t->P3, t->w2p, t->w3p, t->wfp};
+                       {{f(w.conv1_w), d.w1k, 32 * 64 * t->g.C}, {f(w.conv2_w), d.w2k, 64 * 512}, {f(w.conv3_w), d.w3k, 64 * 576}},
+                       {64 * t->g.C, 512, 576}, t->P3, t->w2p, t->w3p, t->wfp};
     t->packed = t->wfp != nullptr;
     int n = 64 * 512 + 64 * 576;
     for (const LoadItem& it : p.rest) n += it.n;
+    for (const LoadItem& it : p.turned) n += it.n;
     load_fp32_kernel<<<512 + nblk(n, 256), 256, 0, s>>>(p);
     HTS_LAUNCH_CHECK("load_fp32");
     return HTS_OK;

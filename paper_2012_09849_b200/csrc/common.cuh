@@ -124,8 +124,25 @@ struct Profiler {
 struct RefWeights {            // fp32 device copies in PyTorch layouts
     float *w1, *b1, *w2, *b2, *w3, *b3, *wfc, *bfc;
     float *whead, *bhead;      // [A+1,512], [A+1]: policy rows then the value row
+    float *w1k, *w2k, *w3k;    // the convolutions' weights once more as [C k k][O], or nullptr
 };
-struct RefWorkspace { float *a1, *a2, *a3, *h; };   // NCHW fp32 activations, [n,512]
+// Rows of one channel: row y is at (y % phases) * phase + (y / phases) * pitch.  A convolution of stride s reads inputs of
+// one phase or of s of them.
+struct RowLayout { int pitch, phases, phase, chan; };    // elements; chan: between channels
+inline RowLayout rows_dense(int H, int W) { return {W, 1, 0, H * W}; }
+// Rows of an odd number of 16-byte pieces: eight of them start in eight different sixteenths of the shared-memory banks.
+inline RowLayout rows_strips(int H, int W, int phases)
+{
+    RowLayout l{((W + 3) / 4 | 1) * 4, phases, 0, 0};
+    l.phase = (H + phases - 1) / phases * l.pitch; l.chan = phases * l.phase;
+    return l;
+}
+struct RefWorkspace {          // fp32 activations [n][channels][rows], [n,512]
+    float *a1, *a2, *a3, *h;   // a3 is dense
+    RowLayout l1, l2;
+};
+inline RowLayout rows_a1(const Geometry& g) { return rows_strips(g.H1, g.W1, 2); }
+inline RowLayout rows_a2(const Geometry& g) { return rows_strips(g.H2, g.W2, 1); }
 struct RefPlanes {             // the hidden convolution outputs once more, as three bf16 planes of pixel-major rows
     __nv_bfloat16 *a1, *a2, *a3;
     size_t p1, p2, p3;         // elements between planes
@@ -134,6 +151,8 @@ struct RefPlanes {             // the hidden convolution outputs once more, as t
 hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspace& ws,
                        const uint8_t* obs, const Indexing& ix, int* status, int n, Profiler& prof, cudaStream_t s,
                        const RefPlanes* planes = nullptr);
+// n frames of activations in rows of a layout as [n][channels][H][W].
+hts_status launch_dense_rows(const float* x, const RowLayout& l, int channels, int H, int W, int n, float* out, cudaStream_t s);
 
 // ---- gradient of the learner objective: fp32-accurate passes on the tensor cores (backward.cu) -------
 struct X3State;

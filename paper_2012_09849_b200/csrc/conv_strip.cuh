@@ -1,0 +1,50 @@
+// fp32 convolutions of the actor step in strips: a thread owns PX consecutive pixels of one output row and OT channels.
+#pragma once
+#include "common.cuh"
+
+namespace hts {
+
+// One convolution of the fp32 path, whichever kernel computes it.
+struct ConvParams {
+    const void* x;                      // [frames][C][rows], u8 or fp32
+    const float *w, *b;                 // [O][C k k], [O]
+    const float* wk;                    // the same weights as [C k k][O], 16-byte aligned, or nullptr
+    float* y;                           // [n][O][rows]
+    int n, C, H, W, O, k, s, Ho, Wo;
+    RowLayout xl, yl;
+    float in_scale;
+    const int32_t* slots;               // frame of each row, or nullptr
+    int pool;
+    int* status;
+    bool w_vec, words;                  // weights 16-byte aligned; frames 4-byte aligned
+    __nv_bfloat16* planes;              // optional second output: three bf16 planes of pixel-major rows (x3_gemm.cuh)
+    size_t plane;
+    int W_rows, P_rows;                 // its grid; 2 x 2 pixels per row when s2d
+    bool s2d;
+};
+
+#ifdef __CUDACC__
+// Frame of batch row e: e itself, or its slot in the pool (a slot outside it is reported and reads frame 0).
+__device__ __forceinline__ size_t frame_of(const ConvParams& p, int e)
+{
+    if (!p.slots) return (size_t)e;
+    const int sl = p.slots[e];
+    if ((unsigned)sl >= (unsigned)p.pool) { atomicCAS(p.status, 0, kStatusBadSlot); return 0; }
+    return (size_t)sl;
+}
+// Where the inputs of output row i start, and its filter row u relative to that; where output row i is.
+__device__ __forceinline__ int x_row(const ConvParams& p, int i) { return i * (p.s / p.xl.phases) * p.xl.pitch; }
+__device__ __forceinline__ int x_tap(const ConvParams& p, int u) { return u % p.xl.phases * p.xl.phase + u / p.xl.phases * p.xl.pitch; }
+__device__ __forceinline__ int y_row(const ConvParams& p, int i) { return i % p.yl.phases * p.yl.phase + i / p.yl.phases * p.yl.pitch; }
+// Where pixel (i, x) of row e starts in the planes.
+__device__ __forceinline__ size_t plane_row(const ConvParams& p, int e, int i, int x)
+{
+    return p.s2d ? ((size_t)e * p.P_rows + (size_t)(i >> 1) * p.W_rows + (x >> 1)) * 128 + ((i & 1) * 2 + (x & 1)) * 32
+                 : ((size_t)e * p.P_rows + i * p.Wo + x) * 64;
+}
+#endif
+
+// HTS_ERR_UNSUPPORTED: not a shape for strips (nothing was launched).
+hts_status launch_conv_strip(const ConvParams& p, cudaStream_t s);
+
+}  // namespace hts

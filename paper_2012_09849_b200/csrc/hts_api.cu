@@ -129,7 +129,8 @@ hts_status run_step(hts_ctx* ctx, const uint8_t* obs, const Indexing& ix, const 
         st = tc_heads(ctx->tc, env_ids, t_per_env, t, seed, n, ix, actions, logp, values, entropy, logits, s, given_actions);
     } else {
         const size_t r = (size_t)ix.row0;
-        const RefWorkspace ws{ctx->rws.a1 + r * 32 * g.H1 * g.W1, ctx->rws.a2 + r * 64 * g.H2 * g.W2, ctx->rws.a3 + r * g.F, ctx->rws.h + r * 512};
+        RefWorkspace ws = ctx->rws;
+        ws.a1 += r * 32 * ws.l1.chan; ws.a2 += r * 64 * ws.l2.chan; ws.a3 += r * g.F; ws.h += r * 512;
         st = ref_forward(g, ctx->rw, ws, obs, ix, ctx->status, n, ctx->prof, s);
         if (st != HTS_OK) return st;
         ctx->prof.begin(K_HEADS, s);
@@ -234,7 +235,9 @@ hts_status hts_policy_create(const hts_net_desc* d, hts_ctx** out)
         cv.add(&c->rw.w3, (size_t)64 * 64 * 9); cv.add(&c->rw.b3, 64);
         cv.add(&c->rw.wfc, (size_t)512 * g.F); cv.add(&c->rw.bfc, 512);
         cv.add(&c->rw.whead, (size_t)(A + 1) * 512); cv.add(&c->rw.bhead, (size_t)A + 1);
-        cv.add(&c->rws.a1, nb * 32 * g.H1 * g.W1); cv.add(&c->rws.a2, nb * 64 * g.H2 * g.W2);
+        cv.add(&c->rw.w1k, (size_t)32 * g.C * 64); cv.add(&c->rw.w2k, (size_t)64 * 32 * 16); cv.add(&c->rw.w3k, (size_t)64 * 64 * 9);
+        c->rws.l1 = rows_a1(g); c->rws.l2 = rows_a2(g);
+        cv.add(&c->rws.a1, nb * 32 * c->rws.l1.chan); cv.add(&c->rws.a2, nb * 64 * c->rws.l2.chan);
         cv.add(&c->rws.a3, nb * g.F); cv.add(&c->rws.h, nb * 512);
     }
     if (!cv.alloc(c)) { hts_policy_destroy(c); return HTS_ERR_ALLOC; }
@@ -400,9 +403,10 @@ hts_status hts_policy_read_activation(hts_ctx* ctx, int32_t layer, int32_t n, fl
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     if (ctx->tc) return tc_read_activation(ctx->tc, layer, n, out, s);
     const Geometry& g = ctx->g;
-    const float* src = layer == 1 ? ctx->rws.a1 : layer == 2 ? ctx->rws.a2 : layer == 3 ? ctx->rws.a3 : ctx->rws.h;
-    const size_t per = layer == 1 ? (size_t)32 * g.H1 * g.W1 : layer == 2 ? (size_t)64 * g.H2 * g.W2
-                     : layer == 3 ? (size_t)g.F : 512;
+    if (layer == 1) return launch_dense_rows(ctx->rws.a1, ctx->rws.l1, 32, g.H1, g.W1, n, out, s);
+    if (layer == 2) return launch_dense_rows(ctx->rws.a2, ctx->rws.l2, 64, g.H2, g.W2, n, out, s);
+    const float* src = layer == 3 ? ctx->rws.a3 : ctx->rws.h;
+    const size_t per = layer == 3 ? (size_t)g.F : 512;
     HTS_CUDA(cudaMemcpyAsync(out, src, per * n * sizeof(float), cudaMemcpyDeviceToDevice, s));
     return HTS_OK;
 }

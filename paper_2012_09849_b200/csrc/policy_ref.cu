@@ -1,38 +1,17 @@
 // fp32 CUDA-core path of the actor step: the check path (fp32 weights) of the policy-value
 // network of Appendix F.1 / F.2.  Every output is one chain of fp32 multiply-adds in a fixed order, whatever the
-// tile that computes it, so a row's bits do not depend on the batch around it.
+// tile that computes it, so a row's bits do not depend on the batch around it.  A context's convolutions run in strips
+// (conv_strip.cu); the tiles here take what those do not: weights in the caller's layout (the step that allocates nothing),
+// frames that are not 16-byte aligned, rows too wide for shared memory.
 #include <type_traits>
 #include "common.cuh"
+#include "conv_strip.cuh"
+#include "f32x2.cuh"
 #include "x3_gemm.cuh"
 
 namespace hts {
 namespace {
 
-typedef unsigned long long f32x2;                       // two fp32 lanes of a packed multiply-add
-__device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b)
-{
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
-}
-__device__ __forceinline__ f32x2 pair(float lo, float hi)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ f32x2 both(float v) { return pair(v, v); }
-__device__ __forceinline__ float lane_of(f32x2 v, int i) { return __uint_as_float(i ? (uint32_t)(v >> 32) : (uint32_t)v); }
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-template <int PENDING>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
 __device__ __forceinline__ float4 load4(const float* p, bool vec)
 {
     return vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
@@ -43,52 +22,13 @@ __device__ __forceinline__ float4 load4(const float* p, bool vec)
 // and the wide fully-connected form let it start as they end (no trigger), which costs it no more than its prologue:
 // n = 40 / 160 / 256 / 1024: 96 / 194 / 241 / 587 us per step with triggers after the wait, 81 / 168 / 201 / 549 without.
 // The narrow fully-connected form, before the small heads, still triggers (0.5 us per step).
-struct ConvParams {
-    const void* x;                      // [frames][C][H][W], u8 or fp32
-    const float *w, *b;                 // [O][C k k], [O]
-    float* y;                           // [n][O][Ho][Wo]
-    int n, C, H, W, O, k, s, Ho, Wo;
-    float in_scale;
-    const int32_t* slots;               // frame of each row, or nullptr
-    int pool;
-    int* status;
-    bool w_vec, words;                  // weights 16-byte aligned; frames 4-byte aligned
-    __nv_bfloat16* planes;              // optional second output: three bf16 planes of pixel-major rows (x3_gemm.cuh)
-    size_t plane;
-    int W_rows, P_rows;                 // its grid; 2 x 2 pixels per row when s2d
-    bool s2d;
-};
-
-// Frame of batch row e: e itself, or its slot in the pool (a slot outside it is reported and reads frame 0).
-__device__ __forceinline__ size_t frame_of(const ConvParams& p, int e)
-{
-    if (!p.slots) return (size_t)e;
-    const int sl = p.slots[e];
-    if ((unsigned)sl >= (unsigned)p.pool) { atomicCAS(p.status, 0, kStatusBadSlot); return 0; }
-    return (size_t)sl;
-}
-// Where pixel r of row e starts in the planes.
-__device__ __forceinline__ size_t plane_row(const ConvParams& p, int e, int r)
-{
-    const int i = r / p.Wo, x = r - i * p.Wo;
-    return p.s2d ? ((size_t)e * p.P_rows + (size_t)(i >> 1) * p.W_rows + (x >> 1)) * 128 + ((i & 1) * 2 + (x & 1)) * 32
-                 : ((size_t)e * p.P_rows + r) * 64;
-}
-
 // y[e,o,i,j] = relu(b[o] + in_scale * sum_{c,u,v} w[o,c,u,v] x[e,c,i s+u,j s+v]), summed over (c, u, v) in ascending
 // order.  Implicit GEMM: a block owns PX consecutive output pixels of the batch and OC channels and gathers PX x KC
 // inputs and OC x KC weights per step into shared memory, one step ahead; a thread owns PXT pixels x OT channels.
-// Bound: issue slots and the 128 bytes per clock at which shared memory reaches registers (a thread loads 4 (PXT + OT)
-// bytes per PXT x OT multiply-adds), both close to the fp32 pipes' own time.  Packed multiply-adds (two channels each, the input
-// in both lanes) reach 64 TFLOP/s in this pattern where scalar ones stop at 49 (three distinct registers per operation).  A
-// thread's pixels are runs of four, so a step's inputs are two 16-byte loads instead of eight of 4: conv1 / conv2 / conv3 at n =
-// 1024 162 / 171 / 114 -> 153 / 154 / 103 us (a 16-byte load takes 4 clocks of shared memory where the eight lanes of a
-// quarter differ, 2 where they agree; pairs of pixels, with the weights in both lanes, take 16 clocks a step instead of 12:
-// 193 / 181 / 119).  8 x 16 per thread loads less but leaves two warps per scheduler: 206 against 171 us (conv2, n = 1024);
-// copying input rows instead of gathering per tap makes the reads scattered: 278 us.
-// What keeps it from 64 TFLOP/s (28 to 44 are reached, and no unit is busy for more than 81 % of the time): inputs are gathered four bytes
-// at a time; weights are turned through eight registers a thread in every block and chunk, under a cap of 128 (the conv2 / conv3 form
-// spills 4 bytes); two to four warps per scheduler cover the rest.
+// Bound: no unit alone.  Inputs are gathered four bytes at a time, weights turned through registers in every block and chunk, and
+// shared memory reaches registers at 128 bytes per clock (a thread loads 4 (PXT + OT) bytes per PXT x OT multiply-adds): 28 to 44
+// TFLOP/s where strips reach 45 to 53 (first / second / third layer of 1024 observations 150 / 151 / 101 us, 134 / 104 / 83 in strips).
+// A thread's pixels are runs of four, so a step's inputs are two 16-byte loads.
 template <typename TIn, int PXT, int OT, int WPX, int WO, int KC, int PER_SM>
 __global__ void __launch_bounds__(32 * WPX * WO, PER_SM)
 conv_tile_kernel(const ConvParams p)
@@ -109,7 +49,7 @@ conv_tile_kernel(const ConvParams p)
     const int total = p.n * P, o_base = blockIdx.y * OC;
     for (int u = tid; u < K / UNIT; u += NT) {
         const int kk = u * UNIT, c = kk / (p.k * p.k), r = kk - c * p.k * p.k, uu = r / p.k;
-        s_off[u] = (c * p.H + uu) * p.W + (r - uu * p.k);
+        s_off[u] = c * p.xl.chan + x_tap(p, uu) + (r - uu * p.k);
     }
     pdl_wait();
     const TIn* src[NPX];
@@ -119,7 +59,7 @@ conv_tile_kernel(const ConvParams p)
         // places, which takes 32 passes (conv3, n = 72: 40 us, 26 with distinct words).
         const int px = (blockIdx.x * PX + (NPX > 1 ? tid + NT * q : tid % PX)) % total;
         const int e = px / P, r = px - e * P, i = r / p.Wo, j = r - i * p.Wo;
-        src[q] = static_cast<const TIn*>(p.x) + frame_of(p, e) * p.C * p.H * p.W + (size_t)(i * p.s) * p.W + j * p.s;
+        src[q] = static_cast<const TIn*>(p.x) + frame_of(p, e) * p.C * p.xl.chan + x_row(p, i) + j * p.s;
     }
     __syncthreads();
     const int kl = NPX > 1 ? 0 : tid / PX, pl = NPX > 1 ? tid : tid % PX;
@@ -212,16 +152,16 @@ conv_tile_kernel(const ConvParams p)
     for (int q = 0; q < PXT; ++q) {
         const int px = blockIdx.x * PX + px_t + 32 * (q / 4) + q % 4;
         if (px >= total) continue;
-        const int e = px / P, r = px - e * P;
+        const int e = px / P, r = px - e * P, i = r / p.Wo, x = r - i * p.Wo;
         float v[OT];
 #pragma unroll
         for (int j = 0; j < OT; ++j) {
             const float t = fmaf(lane_of(acc[q][j / 2], j & 1), p.in_scale, p.b[o_base + o_t + j]);
             v[j] = t > 0.f ? t : 0.f;
-            p.y[((size_t)e * p.O + o_base + o_t + j) * P + r] = v[j];
+            p.y[((size_t)e * p.O + o_base + o_t + j) * p.yl.chan + y_row(p, i) + x] = v[j];
         }
         if (p.planes) {
-            __nv_bfloat16* d = p.planes + plane_row(p, e, r) + o_base + o_t;
+            __nv_bfloat16* d = p.planes + plane_row(p, e, i, x) + o_base + o_t;
 #pragma unroll
             for (int j = 0; j < OT; j += 4) {
                 uint2 o0, o1, o2;
@@ -270,7 +210,7 @@ conv_small_kernel(const ConvParams p, int ring)
             for (int a = 0; a < kSmallPx * kSmallK / 4 / 128; ++a) {
                 const int u = a * 128 + tid, px = u >> 4, k = gr * kSmallK + (u & 15) * 4;
                 const int c = k / kk2, r = k - c * kk2, uu = r / p.k;
-                const TIn* s = s_src[px] + (c * p.H + uu) * p.W + (r - uu * p.k);
+                const TIn* s = s_src[px] + c * p.xl.chan + x_tap(p, uu) + (r - uu * p.k);
                 uint32_t w;
                 if (p.words) w = *reinterpret_cast<const uint32_t*>(s);
                 else w = s[0] | (uint32_t)s[1] << 8 | (uint32_t)s[2] << 16 | (uint32_t)s[3] << 24;
@@ -279,7 +219,7 @@ conv_small_kernel(const ConvParams p, int ring)
             }
         } else {
             const int k = gr * kSmallK + (tid & 63), c = k / kk2, r = k - c * kk2, uu = r / p.k;
-            const int off = (c * p.H + uu) * p.W + (r - uu * p.k);
+            const int off = c * p.xl.chan + x_tap(p, uu) + (r - uu * p.k);
 #pragma unroll
             for (int a = 0; a < kSmallPx / 2; ++a) {
                 const int px = 2 * a + (tid >> 6);
@@ -293,7 +233,7 @@ conv_small_kernel(const ConvParams p, int ring)
         int px = px0 + tid;
         px = px < total ? px : total - 1;
         const int e = px / P, r = px - e * P, i = r / p.Wo, j = r - i * p.Wo;
-        s_src[tid] = static_cast<const TIn*>(p.x) + frame_of(p, e) * p.C * p.H * p.W + (size_t)(i * p.s) * p.W + j * p.s;
+        s_src[tid] = static_cast<const TIn*>(p.x) + frame_of(p, e) * p.C * p.xl.chan + x_row(p, i) + j * p.s;
     }
     __syncthreads();
     for (int g = 0; g < ring; ++g) {
@@ -331,18 +271,18 @@ conv_small_kernel(const ConvParams p, int ring)
     for (int q = 0; q < 2; ++q) {
         const int px = px0 + g8 + 8 * q;
         if (px >= total) continue;
-        const int e = px / P, r = px - e * P, o = o_base + o_t;
+        const int e = px / P, r = px - e * P, i = r / p.Wo, x = r - i * p.Wo, o = o_base + o_t;
         float v[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const float t = fmaf(q ? (j ? a11 : a10) : (j ? a01 : a00), p.in_scale, p.b[o + j]);
             v[j] = t > 0.f ? t : 0.f;
-            p.y[((size_t)e * p.O + o + j) * P + r] = v[j];
+            p.y[((size_t)e * p.O + o + j) * p.yl.chan + y_row(p, i) + x] = v[j];
         }
         if (p.planes) {
             uint32_t o0, o1, o2;
             x3_split2(v[0], v[1], o0, o1, o2);
-            uint32_t* d = reinterpret_cast<uint32_t*>(p.planes + plane_row(p, e, r) + o);
+            uint32_t* d = reinterpret_cast<uint32_t*>(p.planes + plane_row(p, e, i, x) + o);
             d[0] = o0; d[p.plane / 2] = o1; d[p.plane] = o2;
         }
     }
@@ -380,19 +320,21 @@ hts_status launch_conv_tile(const ConvParams& p, cudaStream_t s)
     return HTS_OK;
 }
 
-// A form takes a time that steps with the blocks of the SM that has most.  conv2 (us at 1, 2, 3 ... per SM): latency form
-// 15, 19, 23, 27; 64 x 32 tiles 25, 35, 48, 62, 74, 87, 99; 128 x 64 (256 x 32) tiles 50, 80, 109.  So one large tile
-// costs as much as 2.5 small ones and 0.7 more for its start; the latency form pays up to three blocks per SM (two where
-// it converts frames, 17 against 15).
+// A form takes a time that steps with the blocks of the SM that has most (conv2, us at 1, 2, 3 ... per SM: latency form 15, 19, 23,
+// 27; 64 x 32 tiles 25, 35, 48, 62, 74).  The latency form pays up to three blocks per SM, two where it converts frames (17 against
+// 15).  Large tiles (256 x 32) only take many unaligned frames: one costs as much as 2.5 small ones and 0.7 more for its start.
 template <typename TIn>
 hts_status launch_conv(const ConvParams& p, cudaStream_t s)
 {
+    const hts_status strips = launch_conv_strip(p, s);
+    if (strips != HTS_ERR_UNSUPPORTED) return strips;
+    constexpr bool U8 = std::is_same<TIn, uint8_t>::value;
     const size_t px = (size_t)p.n * p.Ho * p.Wo, sms = (size_t)device_sm_count(device_slot());
     auto per_sm = [&](size_t tile_px, size_t tile_oc) { return ((px + tile_px - 1) / tile_px * (p.O / tile_oc) + sms - 1) / sms; };
-    const size_t small = per_sm(kSmallPx, kSmallOc), medium = per_sm(64, 32), large = p.O == 64 ? per_sm(128, 64) : per_sm(256, 32);
-    if (small <= (std::is_same<TIn, uint8_t>::value ? 2 : 3)) return launch_conv_small<TIn>(p, s);
-    if (2 * medium <= 5 * large + 1) return launch_conv_tile<TIn, 4, 4, 2, 2, 32, 5>(p, s);
-    return p.O == 64 ? launch_conv_tile<TIn, 8, 8, 2, 2, 16, 4>(p, s) : launch_conv_tile<TIn, 8, 8, 4, 1, 16, 4>(p, s);
+    if (per_sm(kSmallPx, kSmallOc) <= (U8 ? 2 : 3)) return launch_conv_small<TIn>(p, s);
+    if constexpr (U8)
+        if (2 * per_sm(64, 32) > 5 * per_sm(256, 32) + 1) return launch_conv_tile<TIn, 8, 8, 4, 1, 16, 4>(p, s);
+    return launch_conv_tile<TIn, 4, 4, 2, 2, 32, 5>(p, s);
 }
 
 // h[e,o] = relu(b[o] + sum over lanes l of (chain of f = l, l+32, l+64, ...)), the 32 chains added as a binary tree
@@ -526,7 +468,24 @@ hts_status launch_fc(const float* x, const float* w, const float* b, float* h, i
     return launch_fc_chain<4, 4, 4, 1, 4, 128>(x, w, b, h, n, F, s);
 }
 
+__global__ void __launch_bounds__(256) dense_rows_kernel(const float* __restrict__ x, const RowLayout l, int H, int W, size_t total, float* __restrict__ out)
+{
+    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= total) return;
+    const size_t row = i / W, c = row / H;
+    const int y = (int)(row - c * H);
+    out[i] = x[c * l.chan + y % l.phases * l.phase + y / l.phases * l.pitch + (int)(i - row * W)];
+}
+
 }  // namespace
+
+hts_status launch_dense_rows(const float* x, const RowLayout& l, int channels, int H, int W, int n, float* out, cudaStream_t s)
+{
+    const size_t total = (size_t)n * channels * H * W;
+    dense_rows_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(x, l, H, W, total, out);
+    HTS_LAUNCH_CHECK("dense_rows");
+    return HTS_OK;
+}
 
 // `planes`: also leave the three hidden convolution outputs as bf16 planes for the gradient.
 hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspace& ws,
@@ -534,27 +493,28 @@ hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspac
                        const RefPlanes* planes)
 {
     hts_status st;
-    auto layer = [&](const void* x, const float* wt, const float* b, float* y, int C, int H, int W, int O, int k, int stride, int Ho, int Wo) {
+    auto layer = [&](const void* x, const RowLayout& xl, const float* wt, const float* wk, const float* b, float* y, const RowLayout& yl, int C, int H,
+                     int W, int O, int k, int stride, int Ho, int Wo) {
         ConvParams p{};
-        p.x = x; p.w = wt; p.b = b; p.y = y; p.n = n; p.C = C; p.H = H; p.W = W; p.O = O; p.k = k; p.s = stride; p.Ho = Ho; p.Wo = Wo;
-        p.in_scale = 1.f; p.w_vec = ((uintptr_t)wt & 15) == 0; p.words = ((uintptr_t)x & 3) == 0;
+        p.x = x; p.xl = xl; p.w = wt; p.wk = wk; p.b = b; p.y = y; p.yl = yl; p.n = n; p.C = C; p.H = H; p.W = W; p.O = O; p.k = k; p.s = stride; p.Ho = Ho; p.Wo = Wo;
+        p.status = status; p.in_scale = 1.f; p.w_vec = ((uintptr_t)wt & 15) == 0; p.words = ((uintptr_t)x & 3) == 0;
         return p;
     };
     prof.begin(K_CONV1, s);
-    ConvParams c1 = layer(obs, w.w1, w.b1, ws.a1, g.C, g.H, g.W, 32, 8, 4, g.H1, g.W1);
-    c1.in_scale = 1.0f / 255.0f; c1.slots = ix.slots; c1.pool = ix.pool; c1.status = status;
+    ConvParams c1 = layer(obs, rows_dense(g.H, g.W), w.w1, w.w1k, w.b1, ws.a1, ws.l1, g.C, g.H, g.W, 32, 8, 4, g.H1, g.W1);
+    c1.in_scale = 1.0f / 255.0f; c1.slots = ix.slots; c1.pool = ix.pool;
     if (planes) { c1.planes = planes->a1; c1.plane = planes->p1; c1.s2d = true; c1.W_rows = (g.W1 + 1) / 2; c1.P_rows = (g.H1 + 1) / 2 * c1.W_rows; }
     st = launch_conv<uint8_t>(c1, s);
     if (st != HTS_OK) return st;
     prof.end(K_CONV1, s);
     prof.begin(K_CONV2, s);
-    ConvParams c2 = layer(ws.a1, w.w2, w.b2, ws.a2, 32, g.H1, g.W1, 64, 4, 2, g.H2, g.W2);
+    ConvParams c2 = layer(ws.a1, ws.l1, w.w2, w.w2k, w.b2, ws.a2, ws.l2, 32, g.H1, g.W1, 64, 4, 2, g.H2, g.W2);
     if (planes) { c2.planes = planes->a2; c2.plane = planes->p2; c2.P_rows = g.H2 * g.W2; }
     st = launch_conv<float>(c2, s);
     if (st != HTS_OK) return st;
     prof.end(K_CONV2, s);
     prof.begin(K_CONV3, s);
-    ConvParams c3 = layer(ws.a2, w.w3, w.b3, ws.a3, 64, g.H2, g.W2, 64, 3, 1, g.H3, g.W3);
+    ConvParams c3 = layer(ws.a2, ws.l2, w.w3, w.w3k, w.b3, ws.a3, rows_dense(g.H3, g.W3), 64, g.H2, g.W2, 64, 3, 1, g.H3, g.W3);
     if (planes) { c3.planes = planes->a3; c3.plane = planes->p3; c3.P_rows = g.H3 * g.W3; }
     st = launch_conv<float>(c3, s);
     if (st != HTS_OK) return st;
@@ -616,7 +576,7 @@ extern "C" hts_status hts_policy_step_noalloc(const hts_net_desc* d, const hts_w
     }
     float* base = g_noalloc_ptr[dev];
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    RefWorkspace ws{base, base + f_a1, base + f_a1 + f_a2, base + f_a1 + f_a2 + f_a3};
+    const RefWorkspace ws{base, base + f_a1, base + f_a1 + f_a2, base + f_a1 + f_a2 + f_a3, rows_dense(g.H1, g.W1), rows_dense(g.H2, g.W2)};
     float* whead = ws.h + f_h;
     float* bhead = whead + f_wh;
     // every scratch float is written before it is read, so nothing has to start at zero
@@ -626,7 +586,7 @@ extern "C" hts_status hts_policy_step_noalloc(const hts_net_desc* d, const hts_w
     HTS_CUDA(cudaMemcpyAsync(bhead + g.A, w->v_b, sizeof(float), cudaMemcpyDeviceToDevice, s));
     auto f = [](const void* p) { return const_cast<float*>(static_cast<const float*>(p)); };
     const RefWeights rw{f(w->conv1_w), f(w->conv1_b), f(w->conv2_w), f(w->conv2_b), f(w->conv3_w), f(w->conv3_b),
-                        f(w->fc_w), f(w->fc_b), whead, bhead};
+                        f(w->fc_w), f(w->fc_b), whead, bhead, nullptr, nullptr, nullptr};
     Profiler off;
     hts_status st = ref_forward(g, rw, ws, obs, Indexing{}, nullptr, n, off, s);
     if (st != HTS_OK) return st;
