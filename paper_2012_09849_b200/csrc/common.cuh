@@ -137,9 +137,12 @@ inline RowLayout rows_strips(int H, int W, int phases)
     l.phase = (H + phases - 1) / phases * l.pitch; l.chan = phases * l.phase;
     return l;
 }
+struct RefMaps;                // tensor maps of a context's activations and dense weights (policy_ref.cu)
 struct RefWorkspace {          // fp32 activations [n][channels][rows], [n,512]
     float *a1, *a2, *a3, *h;   // a3 is dense
     RowLayout l1, l2;
+    const RefMaps* maps;       // or nullptr
+    int row0;                  // frame of the maps that is this workspace's first
 };
 inline RowLayout rows_a1(const Geometry& g) { return rows_strips(g.H1, g.W1, 2); }
 inline RowLayout rows_a2(const Geometry& g) { return rows_strips(g.H2, g.W2, 1); }
@@ -148,6 +151,9 @@ struct RefPlanes {             // the hidden convolution outputs once more, as t
     size_t p1, p2, p3;         // elements between planes
 };
 
+// The maps of a workspace for `frames` frames; nullptr if there is no memory or driver for them (its kernels then take other forms).
+RefMaps* ref_maps_create(const Geometry& g, const RefWeights& w, const RefWorkspace& ws, size_t frames);
+void ref_maps_destroy(RefMaps* maps);
 hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspace& ws,
                        const uint8_t* obs, const Indexing& ix, int* status, int n, Profiler& prof, cudaStream_t s,
                        const RefPlanes* planes = nullptr);

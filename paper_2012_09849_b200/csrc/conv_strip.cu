@@ -6,7 +6,7 @@
 // mbarrier per stage; all waits are bounded), and a thread reads 20 inputs and 16 weights for 144 multiply-adds (second layer)
 // where 8 x 8 tiles read 32 and 32 for 128.  Bound: the fp32 pipes (80 % busy while the sums run; 60 TFLOP/s of the 70 that packed
 // multiply-adds reach), then what a block spends on its first copies and its stores.  At 1024 observations of 84 x 84 x 4 the
-// three layers take 134 / 104 / 83 us, in gathered tiles 150 / 151 / 101; at 80 15 / 17 / 11.5 against 26 / 31 / 22.
+// three layers take 133 / 107 / 80 us, in gathered tiles 150 / 151 / 101; at 80 15 / 17 / 10.5 against 26 / 31 / 22.
 // Rows have an odd number of 16-byte pieces and, for stride 2, even and odd rows lie apart: eight output rows' inputs are in eight
 // different sixteenths of the banks.  Copies issued by the computing warps cost 20 % (their address chains come before every
 // stage's first sums), one copying warp with 16-byte asynchronous copies 10 to 20 us a layer (40 of them per stage and lane).
@@ -14,6 +14,7 @@
 #include "common.cuh"
 #include "conv_strip.cuh"
 #include "f32x2.cuh"
+#include "tc_host.cuh"
 #include "tc_ptx.cuh"
 #include "x3_gemm.cuh"
 
@@ -22,19 +23,17 @@ namespace {
 
 struct StripPlan {
     int segs;                           // strips per output row
-    int pch, X, GP;                     // 16-byte pieces: row pitch, extra between frames, a phase of rows
+    int rows;                           // rows of a phase (bytes: of four input rows each) that a tile reads of a frame at most
+    int pch, slot;                      // 16-byte pieces: of a row, of a frame's part of a stage
+    int frames;                         // of a tile, at most
+    int X;                              // pieces between the rows of two frames of a tile, besides
     int o_pitch;                        // floats between channels of the outputs in shared memory; 0: stored from registers
+    int frame0;                         // frame of the map that is the batch's first
 };
 struct Strip { int q, rr, sx, e, i; };  // of a thread: strip and row of the batch, strip of the row, frame, row of the frame
 
 // A named barrier among the computing warps.
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(tc::smem_u32(dst)), "l"(src), "r"(bytes), "r"(tc::smem_u32(bar)) : "memory");
-}
-
 // One filter row of one channel: a strip's inputs x times the row's weights w[tap][OC].  A packed multiply-add takes 2 clocks
 // of its scheduler if it shares an operand with the one before it and 3 if not (three pairs of registers, two banks), so the
 // weights stay while the pixels pass, there and back: 64 to 70 TFLOP/s, 58 to 62 with the input kept and the weights passing.
@@ -159,20 +158,24 @@ __device__ __forceinline__ void strip_store(const ConvParams& p, const StripPlan
     }
 }
 
-// The rows of a frame, a channel and a phase that a tile reads follow one another in memory as they do in shared memory (bytes
-// of frames: four rows make one), so a stage (CK channels) is a few bulk copies, one lane each, and one for its weights.
+// A stage is CK channels of the inputs and their weights.  fp32: one box per frame of the tile, whose row r holds what the tile's
+// output row r reads (of a second frame rows start before its first: those are filled with zeros).  Bytes: the rows of a frame and
+// a channel that a tile reads follow one another in memory, four of them make a row here, a bulk copy each.  (A copy takes the
+// copying unit 70 clocks, whatever its size: with one per channel, phase and frame the third layer took 11.5 / 83 us at 80 / 1024
+// observations, with boxes 10.5 / 80.)
 template <typename TIn, int KS, int S, int PX, int OT, int LG, int WS, int CK, int NST, int PER_SM>
 __global__ void __launch_bounds__(32 * (WS * (S == 4 ? 32 : 64) / (32 / LG * OT) + 1), PER_SM)
-conv_strip_kernel(const ConvParams p, const StripPlan t)
+conv_strip_kernel(const ConvParams p, const StripPlan t, const __grid_constant__ CUtensorMap map)
 {
     constexpr bool U8 = sizeof(TIn) == 1;
     constexpr int OC = S == 4 ? 32 : 64, WO = OC / (32 / LG * OT), NC = WS * WO, SEGS = LG * WS, KK = KS * KS, HALO = (KS - 1) / S;
     constexpr int PH = U8 ? 1 : S, RW = (PX - 1) * S + KS;
     constexpr int WCH = CK * KK * OC / 4;                // 16-byte pieces of weights per stage
-    extern __shared__ __align__(16) float4 s4[];         // [NST][inputs of CK channels | weights]
+    extern __shared__ float4 s_dyn[];
     __shared__ uint64_t full[NST], freed[NST];
     __shared__ int abort_flag;
-    const int CP = PH * t.GP, XCH = CK * CP;
+    float4* s4 = s_dyn + (-tc::smem_u32(s_dyn) & 127) / 16;                      // [NST][inputs of CK channels | weights]
+    const int XCH = t.slot, GP = t.rows * t.pch, CP = PH * GP, STAGE = ((U8 ? CK * XCH : XCH) + WCH + 7) / 8 * 8;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int total = p.n * p.Ho * t.segs, q0 = blockIdx.x * SEGS;
     const int rr0 = q0 / t.segs, last = min(q0 + SEGS, total) - 1, rr1 = last / t.segs;
@@ -185,31 +188,37 @@ conv_strip_kernel(const ConvParams p, const StripPlan t)
     __syncthreads();
     if (warp == NC) {
         pdl_wait();
-        const int frames = rr1 / p.Ho - e0 + 1, copies = frames * CK * PH;
-        const size_t row = U8 ? 4 * p.W : p.xl.pitch;    // a row of t.pch pieces
+        const int frames = rr1 / p.Ho - e0 + 1;
         auto rows_of = [&](int f, int* lo) {
             *lo = f == 0 ? rr0 - e0 * p.Ho : 0;
             return (f == frames - 1 ? rr1 - (e0 + f) * p.Ho : p.Ho - 1) - *lo + 1 + HALO;
         };
         uint32_t bytes = WCH * 16;                       // of a stage
         int lo;
-        for (int f = 0; f < frames; ++f) bytes += CK * PH * rows_of(f, &lo) * t.pch * 16;
+        if constexpr (U8)
+            for (int f = 0; f < frames; ++f) bytes += CK * rows_of(f, &lo) * t.pch * 16;
+        else
+            bytes += frames * CK * CP * 16;
         int st = 0;
 #pragma unroll 1
         for (; st < stages; ++st) {
             const int slot = st % NST;
             if (st >= NST && !tc::mbar_wait_warp(freed + slot, (st / NST - 1) & 1, &abort_flag, p.status, 40)) break;
-            float4* dst = s4 + slot * (XCH + WCH);
+            float4* dst = s4 + slot * STAGE;
             if (lane == 0) {
                 tc::mbar_arrive_expect_tx(full + slot, bytes);
-                bulk_load(dst + XCH, p.wk + (size_t)st * CK * KK * OC, WCH * 16, full + slot);
+                tc::bulk_load(dst + STAGE - WCH, p.wk + (size_t)st * CK * KK * OC, WCH * 16, full + slot);
             }
             __syncwarp();
-            for (int u = lane; u < copies; u += 32) {
-                const int ph = u % PH, cc = u / PH % CK, f = u / (PH * CK), rows = rows_of(f, &lo);
-                const TIn* x = static_cast<const TIn*>(p.x) + (frame_of(p, e0 + f) * p.C + st * CK + cc) * p.xl.chan + ph * p.xl.phase + lo * row;
-                bulk_load(dst + cc * CP + ph * t.GP + ((e0 + f) * p.Ho + lo - rr0) * t.pch + f * t.X, x, rows * t.pch * 16, full + slot);
-            }
+            if constexpr (U8) {
+                for (int u = lane; u < frames * CK; u += 32) {
+                    const int cc = u % CK, f = u / CK, rows = rows_of(f, &lo);
+                    const TIn* x = static_cast<const TIn*>(p.x) + (frame_of(p, e0 + f) * p.C + st * CK + cc) * p.xl.chan + (size_t)lo * 4 * p.W;
+                    tc::bulk_load(dst + cc * XCH + ((e0 + f) * p.Ho + lo - rr0) * t.pch + f * t.X, x, rows * t.pch * 16, full + slot);
+                }
+            } else
+                for (int f = lane; f < frames; f += 32)
+                    tc::tma_load_5d(dst + f * t.X, &map, 0, rr0 - (e0 + f) * p.Ho, 0, st * CK, t.frame0 + e0 + f, full + slot);
         }
         if (st < stages)                                 // given up: the copies in flight end before the block does
             for (int i = st < NST ? 0 : st - NST; i < st; ++i) tc::mbar_wait_warp(full + i % NST, (i / NST) & 1, &abort_flag, p.status, 41);
@@ -228,13 +237,13 @@ conv_strip_kernel(const ConvParams p, const StripPlan t)
     for (int st = 0; st < stages; ++st) {
         const int slot = st % NST;
         if (!tc::mbar_wait_warp(full + slot, (st / NST) & 1, &abort_flag, p.status, 42)) break;    // the barriers below are met all the same
-        const float4* in = s4 + slot * (XCH + WCH);
-        const float* w = reinterpret_cast<const float*>(in + XCH) + o_t;
+        const float4* in = s4 + slot * STAGE;
+        const float* w = reinterpret_cast<const float*>(in + STAGE - WCH) + o_t;
 #pragma unroll 1
         for (int cc = 0; cc < CK; ++cc) {
             float x[(RW + 3) / 4 * 4];
             if constexpr (U8) {
-                const uint32_t* x4 = reinterpret_cast<const uint32_t*>(in + cc * CP) + x_at;
+                const uint32_t* x4 = reinterpret_cast<const uint32_t*>(in + cc * XCH) + x_at;
 #pragma unroll 1
                 for (int u = 0; u < KS; ++u) {
                     strip_load<RW>(x, x4);
@@ -246,7 +255,7 @@ conv_strip_kernel(const ConvParams p, const StripPlan t)
                 const float4* x4 = in + cc * CP + x_at;
 #pragma unroll
                 for (int u = 0; u < KS; ++u) {
-                    strip_load<RW>(x, x4 + u % S * t.GP + u / S * t.pch);
+                    strip_load<RW>(x, x4 + u % S * GP + u / S * t.pch);
                     strip_row<KS, S, PX, OT, OC>(acc, x, w + u * KS * OC);
                 }
                 w += KK * OC;
@@ -259,34 +268,66 @@ conv_strip_kernel(const ConvParams p, const StripPlan t)
     strip_store<PX, OT, NC>(p, t, acc, k, q0 + ws * LG + g <= last, o_t, q0, last, OC, reinterpret_cast<float*>(s4));
 }
 
-constexpr size_t kSharedPerSm = 227 * 1024;
-// The tile's place in shared memory.  HTS_ERR_UNSUPPORTED: not a shape for these strips.
-template <typename TIn, int KS, int S, int PX, int OT, int LG, int WS, int CK, int NST, int PER_SM>
-hts_status launch_strip(const ConvParams& p, cudaStream_t s)
+constexpr int kSharedPerSm = 227 * 1024;
+
+// A form of strips: its tile, and where that lies in shared memory for one geometry.
+template <typename TIn_, int KS_, int S_, int PX_, int OT_, int LG_, int WS_, int CK_, int NST_, int PER_SM_>
+struct StripForm {
+    typedef TIn_ TIn;
+    static constexpr int KS = KS_, S = S_, PX = PX_, OT = OT_, LG = LG_, WS = WS_, CK = CK_, NST = NST_, PER_SM = PER_SM_;
+    static constexpr bool U8 = sizeof(TIn) == 1;
+    static constexpr int OC = S == 4 ? 32 : 64, NC = WS * OC / (32 / LG * OT), SEGS = LG * WS, HALO = (KS - 1) / S, PH = U8 ? 1 : S;
+    // C channels of rows of `pch` pieces, outputs of Ho x Wo.  Shared memory without the stored outputs; 0: not a shape for it.
+    static int plan(int C, int pch, int Ho, int Wo, StripPlan* t)
+    {
+        t->segs = (Wo + PX - 1) / PX;
+        if (C % CK || (t->segs > 1 && PX * S % 4)) return 0;
+        const int rt = t->segs == 1 ? SEGS : (SEGS - 1) / t->segs + 2;
+        t->frames = (rt + Ho - 2) / Ho + 1;
+        t->pch = pch; t->rows = rt + HALO; t->X = 0;
+        long long stage;
+        if (U8) {
+            t->X = (HALO * pch + 7) / 8 * 8;
+            // a last strip that ends past its row reads on into what follows
+            const int reach = ((t->segs - 1) * PX * 4 + (PX - 1) * S + KS + (KS - 1) * pch * 4 + 15) / 16;
+            t->slot = (rt - 1) * pch + (t->frames - 1) * t->X + (reach > (1 + HALO) * pch ? reach : (1 + HALO) * pch);
+            stage = (long long)CK * t->slot;
+        } else {
+            if (pch > 64 || t->rows > 256) return 0;     // a box
+            const int box = (CK * PH * t->rows * pch + 7) / 8 * 8;                // a copy lands on 128 bytes
+            t->X = box;
+            stage = t->slot = t->frames * box;
+        }
+        const long long smem = NST * 16 * ((stage + CK * KS * KS * OC / 4 + 7) / 8 * 8) + 128;
+        return smem <= kSharedPerSm / PER_SM - 1024 - 128 ? (int)smem : 0;
+    }
+};
+
+template <typename Form>
+bool strip_map(const RowLayout& l, const float* x, int C, int H, int Ho, int Wo, size_t frames, CUtensorMap* map)
 {
-    constexpr bool U8 = sizeof(TIn) == 1;
-    constexpr int OC = S == 4 ? 32 : 64, NC = WS * OC / (32 / LG * OT), SEGS = LG * WS, HALO = (KS - 1) / S, RW = (PX - 1) * S + KS, PH = U8 ? 1 : S;
     StripPlan t{};
-    t.segs = (p.Wo + PX - 1) / PX;
-    if (p.C % CK || (t.segs > 1 && PX * S % 4)) return HTS_ERR_UNSUPPORTED;
+    return !Form::plan(C, l.pitch / 4, Ho, Wo, &t) ||
+           tc::make_rows_map(map, x, l.pitch, l.phase / l.pitch, l.phases, C, frames, t.rows, Form::CK);
+}
+
+template <typename Form>
+hts_status launch_strip(const ConvParams& p, const CUtensorMap* map, cudaStream_t s)
+{
+    StripPlan t{};
+    int smem = Form::plan(p.C, Form::U8 ? p.W / 4 : p.xl.pitch / 4, p.Ho, p.Wo, &t);
     const long long total = (long long)p.n * p.Ho * t.segs;
-    if (total > INT_MAX / 4) return HTS_ERR_UNSUPPORTED;
-    t.pch = U8 ? p.W / 4 : p.xl.pitch / 4;
-    t.X = (HALO * t.pch + 7) / 8 * 8;
-    const int rt = t.segs == 1 ? SEGS : (SEGS - 1) / t.segs + 2, frames = (rt + p.Ho - 2) / p.Ho + 1;
-    // a last strip that ends past its row reads on into what follows
-    const int reach = U8 ? ((t.segs - 1) * PX * 4 + RW + (KS - 1) * p.W + 15) / 16 : ((t.segs - 1) * PX * S + RW + 3) / 4 + HALO * t.pch;
-    t.GP = (rt - 1) * t.pch + (frames - 1) * t.X + (reach > (1 + HALO) * t.pch ? reach : (1 + HALO) * t.pch);
-    const bool direct = p.yl.pitch % 4 == 0 && p.yl.phase % 4 == 0 && p.yl.chan % 4 == 0 && (PX % 4 == 0 || t.segs == 1);
-    t.o_pitch = direct ? 0 : rt * p.Wo;
-    size_t smem = 16 * NST * ((size_t)CK * KS * KS * OC / 4 + (size_t)CK * PH * t.GP);
-    const size_t out = 4 * (size_t)t.o_pitch * OC;
-    if (out > smem) smem = out;
-    if (smem > kSharedPerSm / PER_SM - 1024 - 128) return HTS_ERR_UNSUPPORTED;
-    auto kernel = conv_strip_kernel<TIn, KS, S, PX, OT, LG, WS, CK, NST, PER_SM>;
+    if (!smem || total > INT_MAX / 4) return HTS_ERR_UNSUPPORTED;
+    t.frame0 = p.frame0;
+    const bool direct = p.yl.pitch % 4 == 0 && p.yl.phase % 4 == 0 && p.yl.chan % 4 == 0 && (Form::PX % 4 == 0 || t.segs == 1);
+    t.o_pitch = direct ? 0 : (t.rows - Form::HALO) * p.Wo;
+    if (4 * t.o_pitch * Form::OC + 128 > smem) smem = 4 * t.o_pitch * Form::OC + 128;
+    if (smem > kSharedPerSm / Form::PER_SM - 1024 - 128) return HTS_ERR_UNSUPPORTED;
+    auto kernel = conv_strip_kernel<typename Form::TIn, Form::KS, Form::S, Form::PX, Form::OT, Form::LG, Form::WS, Form::CK, Form::NST, Form::PER_SM>;
     static OncePerDevice allowed;
     HTS_CUDA(allow_shared(kernel, allowed));
-    HTS_CUDA(launch_pdl(kernel, dim3((unsigned)((total + SEGS - 1) / SEGS)), dim3(32 * (NC + 1)), smem, s, p, t));
+    HTS_CUDA(launch_pdl(kernel, dim3((unsigned)((total + Form::SEGS - 1) / Form::SEGS)), dim3(32 * (Form::NC + 1)), (size_t)smem, s, p, t,
+                        map ? *map : CUtensorMap{}));
     note_launch();
     return HTS_OK;
 }
@@ -301,35 +342,63 @@ static int strip_blocks(const ConvParams& p, int px, int tile)
     return (int)((blocks + sms - 1) / sms);
 }
 
+template <int PX, int OT, int LG, int WS, int CK, int NST, int PER_SM>
+using Form1 = StripForm<uint8_t, 8, 4, PX, OT, LG, WS, CK, NST, PER_SM>;
+template <int PX, int OT, int LG, int CK, int NST, int PER_SM>
+using Form2 = StripForm<float, 4, 2, PX, OT, LG, 1, CK, NST, PER_SM>;
+template <int PX, int OT, int LG, int CK, int NST, int PER_SM>
+using Form3 = StripForm<float, 3, 1, PX, OT, LG, 1, CK, NST, PER_SM>;
+typedef Form1<2, 4, 8, 2, 2, 2, 4> Few1;
+typedef Form1<4, 8, 8, 4, 2, 2, 3> Many1;
+typedef Form1<4, 8, 8, 4, 1, 2, 3> Odd1;                // an odd number of channels
+typedef Form2<4, 2, 4, 4, 2, 4> Few2;
+typedef Form2<9, 2, 4, 4, 2, 4> Some2n;                 // rows up to 9 pixels; else of strips of 10
+typedef Form2<10, 2, 4, 4, 2, 4> Some2w;
+typedef Form2<9, 4, 8, 4, 2, 3> Many2n;
+typedef Form2<10, 4, 8, 2, 3, 3> Many2w;                // (four channels of three frames' boxes are too much for three blocks per SM)
+typedef Form3<4, 2, 4, 8, 3, 2> Few3;
+typedef Form3<7, 2, 4, 8, 2, 3> Some3n;                 // rows up to 7 pixels; else of strips of 8
+typedef Form3<8, 2, 4, 8, 2, 3> Some3w;
+
+bool make_strip_maps(const Geometry& g, const RefWorkspace& ws, size_t frames, StripMaps* m)
+{
+    auto two = [&](auto form, CUtensorMap* map) { return strip_map<decltype(form)>(ws.l1, ws.a1, 32, g.H1, g.H2, g.W2, frames, map); };
+    auto three = [&](auto form, CUtensorMap* map) { return strip_map<decltype(form)>(ws.l2, ws.a2, 64, g.H2, g.H3, g.W3, frames, map); };
+    return two(Few2{}, &m->few2) && three(Few3{}, &m->few3) &&
+           (g.W2 <= 9 ? two(Some2n{}, &m->some2) && two(Many2n{}, &m->many2) : two(Some2w{}, &m->some2) && two(Many2w{}, &m->many2)) &&
+           (g.W3 <= 7 ? three(Some3n{}, &m->some3) : three(Some3w{}, &m->some3));
+}
+
 // A form takes a time that steps with the blocks of the fullest SM.  84 x 84 x 4, us at 1, 2, 3, 4 ... blocks, and what that is
 // about (first + each more):
 //   first layer    2 pixels x 4 channels 5.9, 7.7, 10.0, .. 17.0 (6): 5.6 + 2.2      4 x 8  9.1, 15.0, .. 27 (4), 38.8 (6), 134 (22): 9.1 + 6
-//   second   4 x 2  9.2, 11.1, 15.1: 9.2 + 3.7     a row x 2  11.6, 18.1, 25.0, 32.5: 11.6 + 6.8     a row x 4  17.1, 29.1, .. 55.4, .. 104 (8): 17.1 + 12.5
-//   third    4 x 2  9.7, 12.6, .. 22.6 (4): 9.7 + 4.3     a row x 2  11.4, 16.7, .. 28.6 (4), 46.7 (7), 83 (13): 11.4 + 5.9
+//   second   4 x 2  7.4, 10.9, 14.9: 7.4 + 3.7     a row x 2  11.3, 18.0, 25.5, 32.9: 11.3 + 7.0     a row x 4  16.7, 29.5, .. 56 (4), .. 107 (8): 16.7 + 12.5
+//   third    4 x 2  8.6, 11.8, .. 21.2 (4): 8.6 + 4.2     a row x 2  10.2, 15.6, .. 27.2 (4), 44.7 (7), 80 (13): 10.1 + 5.8
 // (the tiles of policy_ref.cu: 12 to 16 at 16 frames, 26 / 31 / 22 at 80, 150 / 151 / 101 at 1024).  A small tile's block has a short
 // chain of sums, a large one more of them for each load.
-hts_status launch_conv_strip(const ConvParams& p, cudaStream_t s)
+hts_status launch_conv_strip(const ConvParams& p, const StripMaps* maps, cudaStream_t s)
 {
-    if (!p.wk || ((uintptr_t)p.x & 15) || p.xl.pitch % 4) return HTS_ERR_UNSUPPORTED;
+    if (!p.wk || ((uintptr_t)p.x & 15)) return HTS_ERR_UNSUPPORTED;
     hts_status st = HTS_ERR_UNSUPPORTED;
     if (p.s == 4) {
-        if (p.C % 2 == 0 && 56 + 22 * (strip_blocks(p, 2, 16) - 1) < 91 + 60 * (strip_blocks(p, 4, 32) - 1))
-            st = launch_strip<uint8_t, 8, 4, 2, 4, 8, 2, 2, 2, 4>(p, s);
-        if (st == HTS_ERR_UNSUPPORTED) st = launch_strip<uint8_t, 8, 4, 4, 8, 8, 4, 2, 2, 3>(p, s);
-        if (st == HTS_ERR_UNSUPPORTED) st = launch_strip<uint8_t, 8, 4, 4, 8, 8, 4, 1, 2, 3>(p, s);
+        if (56 + 22 * (strip_blocks(p, Few1::PX, Few1::SEGS) - 1) < 91 + 60 * (strip_blocks(p, Many1::PX, Many1::SEGS) - 1)) st = launch_strip<Few1>(p, nullptr, s);
+        if (st == HTS_ERR_UNSUPPORTED) st = launch_strip<Many1>(p, nullptr, s);
+        if (st == HTS_ERR_UNSUPPORTED) st = launch_strip<Odd1>(p, nullptr, s);
         return st;
     }
+    if (!maps) return HTS_ERR_UNSUPPORTED;
     if (p.s == 2) {
-        const int px = p.Wo <= 9 ? 9 : 10;
-        const int few = 92 + 37 * (strip_blocks(p, 4, 4) - 1), some = 116 + 68 * (strip_blocks(p, px, 4) - 1), many = 171 + 125 * (strip_blocks(p, px, 8) - 1);
-        if (few < some && few < many) st = launch_strip<float, 4, 2, 4, 2, 4, 1, 4, 3, 3>(p, s);
-        else if (some < many) st = px == 9 ? launch_strip<float, 4, 2, 9, 2, 4, 1, 4, 2, 4>(p, s) : launch_strip<float, 4, 2, 10, 2, 4, 1, 4, 2, 4>(p, s);
-        if (st == HTS_ERR_UNSUPPORTED) st = px == 9 ? launch_strip<float, 4, 2, 9, 4, 8, 1, 2, 3, 3>(p, s) : launch_strip<float, 4, 2, 10, 4, 8, 1, 2, 3, 3>(p, s);
-        return st;
+        const bool narrow = p.Wo <= 9;
+        const int px = narrow ? 9 : 10;
+        const int few = 74 + 37 * (strip_blocks(p, 4, 4) - 1), some = 113 + 70 * (strip_blocks(p, px, 4) - 1), many = 167 + 125 * (strip_blocks(p, px, 8) - 1);
+        if (few >= many && some >= many) st = narrow ? launch_strip<Many2n>(p, &maps->many2, s) : launch_strip<Many2w>(p, &maps->many2, s);
+        if (st == HTS_ERR_UNSUPPORTED && few >= some) st = narrow ? launch_strip<Some2n>(p, &maps->some2, s) : launch_strip<Some2w>(p, &maps->some2, s);
+        return st == HTS_ERR_UNSUPPORTED ? launch_strip<Few2>(p, &maps->few2, s) : st;
     }
-    if (97 + 43 * (strip_blocks(p, 4, 4) - 1) < 114 + 59 * (strip_blocks(p, p.Wo <= 7 ? 7 : 8, 4) - 1)) st = launch_strip<float, 3, 1, 4, 2, 4, 1, 8, 3, 2>(p, s);
-    if (st == HTS_ERR_UNSUPPORTED) st = p.Wo <= 7 ? launch_strip<float, 3, 1, 7, 2, 4, 1, 8, 2, 3>(p, s) : launch_strip<float, 3, 1, 8, 2, 4, 1, 8, 2, 3>(p, s);
-    return st;
+    const bool narrow = p.Wo <= 7;
+    if (86 + 42 * (strip_blocks(p, 4, 4) - 1) >= 101 + 58 * (strip_blocks(p, narrow ? 7 : 8, 4) - 1))
+        st = narrow ? launch_strip<Some3n>(p, &maps->some3, s) : launch_strip<Some3w>(p, &maps->some3, s);
+    return st == HTS_ERR_UNSUPPORTED ? launch_strip<Few3>(p, &maps->few3, s) : st;
 }
 
 }  // namespace hts

@@ -1,5 +1,6 @@
 // fp32 convolutions of the actor step in strips: a thread owns PX consecutive pixels of one output row and OT channels.
 #pragma once
+#include <cuda.h>
 #include "common.cuh"
 
 namespace hts {
@@ -13,6 +14,7 @@ struct ConvParams {
     int n, C, H, W, O, k, s, Ho, Wo;
     RowLayout xl, yl;
     float in_scale;
+    int frame0;                         // fp32: frame of the layer's map that is x
     const int32_t* slots;               // frame of each row, or nullptr
     int pool;
     int* status;
@@ -44,7 +46,11 @@ __device__ __forceinline__ size_t plane_row(const ConvParams& p, int e, int i, i
 }
 #endif
 
+// Boxes of a context's activations, as the forms of the second and third layer read them.
+struct StripMaps { CUtensorMap few2, some2, many2, few3, some3; };
+bool make_strip_maps(const Geometry& g, const RefWorkspace& ws, size_t frames, StripMaps* maps);
+
 // HTS_ERR_UNSUPPORTED: not a shape for strips (nothing was launched).
-hts_status launch_conv_strip(const ConvParams& p, cudaStream_t s);
+hts_status launch_conv_strip(const ConvParams& p, const StripMaps* maps, cudaStream_t s);
 
 }  // namespace hts

@@ -1,0 +1,157 @@
+// fp32 dense layer of the actor step for batches that fill the device.
+//
+// Lane l of a warp runs chain l of TE rows x TO outputs, so both operands are contiguous across the lanes; one transposing
+// reduction closes the tree (at each level a lane keeps half of its values and gets its partner's share of them).  Stages of 128
+// columns arrive as boxes of 16 rows, asked for by a warp of their own (all waits are bounded); the next 32 columns are loaded
+// while these are multiplied.  Bound: loads from shared memory, a clock for each of the 16 words that 64 multiply-adds take, and as
+// much time in the fp32 pipes (with the moves that put a weight into both lanes); 61 % of the one and 60 % of the other are reached.
+// 3136 features, us at 40 / 80 / 160 / 256 / 512 / 1024 rows: 12.3 / 16.7 / 22.7 / 29.9 / 48.5 / 92; copied by the multiplying warps,
+// 32 x 16 outputs per block of eight of them: 16 / 22 / 36 / 36 / 67 / 114.  16 x 8 per warp reads less (24 words for 128) but leaves
+// two warps per scheduler: 29 / 29 / 29 / 29 / 56 / 108.  Pairs of chains in 8-byte loads, without the moves: 99 to 102 at 1024.  A copy
+// per row instead of a box: 163 (70 clocks each).
+#include "common.cuh"
+#include "f32x2.cuh"
+#include "fc_f32.cuh"
+#include "tc_host.cuh"
+#include "tc_ptx.cuh"
+
+namespace hts {
+namespace {
+
+template <int TE, int TO, int WE, int WO, int NST, int PER_SM>
+__global__ void __launch_bounds__(32 * (WE * WO + 1), PER_SM)
+fc_lanes_kernel(const FcParams p, const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mw)
+{
+    constexpr int COLS = kFcBoxCols, BOX = kFcBoxRows, NC = WE * WO, RX = TE * WE, RW = TO * WO, STAGE = (RX + RW) * COLS, NV = TE * TO;
+    static_assert(RX % BOX == 0 && RW % BOX == 0, "whole boxes");
+    extern __shared__ float s_dyn[];
+    float* s_ring = s_dyn + (-tc::smem_u32(s_dyn) & 127) / 4;                    // [NST][RX + RW][COLS]
+    __shared__ uint64_t full[NST], freed[NST];
+    __shared__ int abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < NST; ++i) { tc::mbar_init(full + i, 1); tc::mbar_init(freed + i, NC); }
+        abort_flag = 0;
+        tc::fence_barrier_init();
+    }
+    __syncthreads();
+    const int stages = (p.F + COLS - 1) / COLS, e_base = blockIdx.y * RX, o_base = blockIdx.x * RW;
+    if (warp == NC) {
+        pdl_wait();
+        int st = 0;
+#pragma unroll 1
+        for (; st < stages; ++st) {
+            const int slot = st % NST;
+            if (st >= NST && !tc::mbar_wait_warp(freed + slot, (st / NST - 1) & 1, &abort_flag, p.status, 50)) break;
+            if (lane == 0) tc::mbar_arrive_expect_tx(full + slot, STAGE * 4);
+            __syncwarp();
+            if (lane < (RX + RW) / BOX) {
+                const int r = lane * BOX;
+                if (r < RX) tc::tma_load_2d(s_ring + slot * STAGE + r * COLS, &mx, st * COLS, p.row0 + e_base + r, full + slot);
+                else tc::tma_load_2d(s_ring + slot * STAGE + r * COLS, &mw, st * COLS, o_base + r - RX, full + slot);
+            }
+        }
+        if (st < stages)                                 // given up: the copies in flight end before the block does
+            for (int i = st < NST ? 0 : st - NST; i < st; ++i) tc::mbar_wait_warp(full + i % NST, (i / NST) & 1, &abort_flag, p.status, 51);
+        return;
+    }
+    const int we = warp % WE, wo = warp / WE;
+    f32x2 acc[TE / 2][TO];
+#pragma unroll
+    for (int i = 0; i < TE / 2; ++i)
+#pragma unroll
+        for (int j = 0; j < TO; ++j) acc[i][j] = 0;
+#pragma unroll 1
+    for (int st = 0; st < stages; ++st) {
+        const int slot = st % NST;
+        if (!tc::mbar_wait_warp(full + slot, (st / NST) & 1, &abort_flag, p.status, 52)) break;
+        const float* xr = s_ring + slot * STAGE + we * TE * COLS + lane;
+        const float* wr = s_ring + slot * STAGE + (RX + wo * TO) * COLS + lane;
+        auto load = [&](int c, float (&xv)[TE], float (&wv)[TO]) {
+#pragma unroll
+            for (int j = 0; j < TO; ++j) wv[j] = wr[j * COLS + c];
+#pragma unroll
+            for (int i = 0; i < TE; ++i) xv[i] = xr[i * COLS + c];
+        };
+        auto step = [&](const float (&xv)[TE], const float (&wv)[TO]) {
+            f32x2 xx[TE / 2];
+#pragma unroll
+            for (int i = 0; i < TE / 2; ++i) xx[i] = pair(xv[2 * i], xv[2 * i + 1]);
+#pragma unroll
+            for (int j = 0; j < TO; ++j) {
+                const f32x2 ww = both(wv[j]);
+#pragma unroll
+                for (int a = 0; a < TE / 2; ++a) {
+                    const int i = j & 1 ? TE / 2 - 1 - a : a;
+                    fma2(acc[i][j], xx[i], ww);
+                }
+            }
+        };
+        const int cols = min(COLS, p.F - st * COLS);     // a multiple of 64
+        float xv[2][TE], wv[2][TO];
+        load(0, xv[0], wv[0]);
+#pragma unroll 1
+        for (int c = 0; c < cols; c += 64) {
+            load(c + 32, xv[1], wv[1]);
+            step(xv[0], wv[0]);
+            load(c + 64 < cols ? c + 64 : c, xv[0], wv[0]);
+            step(xv[1], wv[1]);
+        }
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(freed + slot);
+    }
+    float v[NV];
+#pragma unroll
+    for (int i = 0; i < TE; ++i)
+#pragma unroll
+        for (int j = 0; j < TO; ++j) v[i * TO + j] = lane_of(acc[i / 2][j], i & 1);
+    int id = 0;                                          // (row, output) of v[0]
+#pragma unroll
+    for (int m = 16, len = NV / 2; m > 0; m >>= 1, len >>= 1) {
+        const bool up = lane & m;
+#pragma unroll
+        for (int k = 0; k < len; ++k) {
+            const float send = up ? v[k] : v[k + len], keep = up ? v[k + len] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+        }
+        id += up ? len : 0;
+    }
+    pdl_wait();                                          // the kernel before may still read what this one writes
+    constexpr int LEFT = NV / 32;
+    static_assert(LEFT >= 1 && TO % LEFT == 0, "a lane's results are of one row");
+    const int e = e_base + we * TE + id / TO, o = o_base + wo * TO + id % TO;
+    if (e < p.n)
+#pragma unroll
+        for (int k = 0; k < LEFT; ++k) {
+            const float r = v[k] + p.b[o + k];
+            p.h[(size_t)e * 512 + o + k] = r > 0.f ? r : 0.f;
+        }
+}
+
+template <int TE, int TO, int WE, int WO, int NST, int PER_SM>
+hts_status launch_lanes(const FcParams& p, const FcMaps& m, cudaStream_t s)
+{
+    constexpr int smem = NST * (TE * WE + TO * WO) * kFcBoxCols * 4 + 128;
+    static_assert(smem <= 227 * 1024 / PER_SM - 1024 - 128, "shared memory");
+    auto kernel = fc_lanes_kernel<TE, TO, WE, WO, NST, PER_SM>;
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(kernel, allowed));
+    HTS_CUDA(launch_pdl(kernel, dim3(512 / (TO * WO), (unsigned)((p.n + TE * WE - 1) / (TE * WE))), dim3(32 * (WE * WO + 1)), (size_t)smem, s, p, m.x, m.w));
+    note_launch();
+    return HTS_OK;
+}
+
+}  // namespace
+
+bool make_fc_maps(const float* x, const float* w, int F, size_t frames, FcMaps* m)
+{
+    m->ok = F >= kFcBoxCols;
+    return !m->ok || (tc::make_f32_map(&m->x, x, frames, F, kFcBoxRows, kFcBoxCols) && tc::make_f32_map(&m->w, w, 512, F, kFcBoxRows, kFcBoxCols));
+}
+
+hts_status launch_fc_lanes(const FcParams& p, const FcMaps& m, cudaStream_t s)
+{
+    return m.ok ? launch_lanes<8, 8, 2, 2, 2, 3>(p, m, s) : HTS_ERR_UNSUPPORTED;
+}
+
+}  // namespace hts

@@ -30,6 +30,7 @@ struct hts_ctx {
     int last_n = 0;
     RefWeights rw{};              // fp32 check path (weight_dtype fp32)
     RefWorkspace rws{};
+    RefMaps* maps = nullptr;
     TcState* tc = nullptr;        // tensor-core path (weight_dtype bf16)
     // staging for the host-buffer entry point: frames, then index words [2][max_batch], result words [4][max_batch] and
     // logits on the device; the words once more in pinned host memory
@@ -130,7 +131,7 @@ hts_status run_step(hts_ctx* ctx, const uint8_t* obs, const Indexing& ix, const 
     } else {
         const size_t r = (size_t)ix.row0;
         RefWorkspace ws = ctx->rws;
-        ws.a1 += r * 32 * ws.l1.chan; ws.a2 += r * 64 * ws.l2.chan; ws.a3 += r * g.F; ws.h += r * 512;
+        ws.row0 = ix.row0; ws.a1 += r * 32 * ws.l1.chan; ws.a2 += r * 64 * ws.l2.chan; ws.a3 += r * g.F; ws.h += r * 512;
         st = ref_forward(g, ctx->rw, ws, obs, ix, ctx->status, n, ctx->prof, s);
         if (st != HTS_OK) return st;
         ctx->prof.begin(K_HEADS, s);
@@ -244,6 +245,7 @@ hts_status hts_policy_create(const hts_net_desc* d, hts_ctx** out)
     const hts_status st = d->weight_dtype == HTS_DTYPE_BF16 ? tc_create(g, d->max_batch, c->status, &c->tc, raw_alloc, c)
                                                             : x3_create(g, d->max_batch, c->status, &c->x3);
     if (st != HTS_OK) { hts_policy_destroy(c); return st; }
+    if (!c->tc) c->rws.maps = c->maps = ref_maps_create(g, c->rw, c->rws, nb);
     if (cudaMemset(c->status, 0, sizeof(int)) != cudaSuccess) {
         hts_status st = cuda_fail(cudaGetLastError(), "cudaMemset");
         hts_policy_destroy(c);
@@ -487,6 +489,7 @@ void hts_policy_destroy(hts_ctx* ctx)
     }
     if (ctx->tc) tc_destroy(ctx->tc);
     if (ctx->x3) x3_destroy(ctx->x3);
+    if (ctx->maps) ref_maps_destroy(ctx->maps);
     for (int i = 0; i < ctx->nalloc; ++i) cudaFree(ctx->allocs[i]);
     if (ctx->h_words) cudaFreeHost(ctx->h_words);
     for (cudaEvent_t e : {ctx->h_start, ctx->h_copied[0], ctx->h_copied[1]}) if (e) cudaEventDestroy(e);

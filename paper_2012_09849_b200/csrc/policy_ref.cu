@@ -3,13 +3,27 @@
 // tile that computes it, so a row's bits do not depend on the batch around it.  A context's convolutions run in strips
 // (conv_strip.cu); the tiles here take what those do not: weights in the caller's layout (the step that allocates nothing),
 // frames that are not 16-byte aligned, rows too wide for shared memory.
+#include <new>
 #include <type_traits>
 #include "common.cuh"
 #include "conv_strip.cuh"
 #include "f32x2.cuh"
+#include "fc_f32.cuh"
 #include "x3_gemm.cuh"
 
 namespace hts {
+
+struct RefMaps { StripMaps strips; FcMaps fc; };
+
+RefMaps* ref_maps_create(const Geometry& g, const RefWeights& w, const RefWorkspace& ws, size_t frames)
+{
+    RefMaps* m = new (std::nothrow) RefMaps();
+    if (m && make_strip_maps(g, ws, frames, &m->strips) && make_fc_maps(ws.a3, w.wfc, g.F, frames, &m->fc)) return m;
+    delete m;
+    return nullptr;
+}
+void ref_maps_destroy(RefMaps* maps) { delete maps; }
+
 namespace {
 
 __device__ __forceinline__ float4 load4(const float* p, bool vec)
@@ -19,15 +33,15 @@ __device__ __forceinline__ float4 load4(const float* p, bool vec)
 
 // Where the next kernel may start.  Blocks of a dependent launch that become resident early all settle on the first SMs
 // that have room and stay there, waiting, while the others get none: its work then runs unevenly.  So the convolutions
-// and the wide fully-connected form let it start as they end (no trigger), which costs it no more than its prologue:
-// n = 40 / 160 / 256 / 1024: 96 / 194 / 241 / 587 us per step with triggers after the wait, 81 / 168 / 201 / 549 without.
-// The narrow fully-connected form, before the small heads, still triggers (0.5 us per step).
+// and the dense layer of many rows let it start as they end (no trigger), which costs it no more than its prologue (with
+// gathered tiles n = 40 / 160 / 256 / 1024: 96 / 194 / 241 / 587 us per step with triggers after the wait, 81 / 168 / 201 / 549 without).
+// The dense layer of few rows, before the small heads, still triggers (0.5 us per step).
 // y[e,o,i,j] = relu(b[o] + in_scale * sum_{c,u,v} w[o,c,u,v] x[e,c,i s+u,j s+v]), summed over (c, u, v) in ascending
 // order.  Implicit GEMM: a block owns PX consecutive output pixels of the batch and OC channels and gathers PX x KC
 // inputs and OC x KC weights per step into shared memory, one step ahead; a thread owns PXT pixels x OT channels.
 // Bound: no unit alone.  Inputs are gathered four bytes at a time, weights turned through registers in every block and chunk, and
 // shared memory reaches registers at 128 bytes per clock (a thread loads 4 (PXT + OT) bytes per PXT x OT multiply-adds): 28 to 44
-// TFLOP/s where strips reach 45 to 53 (first / second / third layer of 1024 observations 150 / 151 / 101 us, 134 / 104 / 83 in strips).
+// TFLOP/s where strips reach 45 to 53 (first / second / third layer of 1024 observations 150 / 151 / 101 us, 133 / 107 / 80 in strips).
 // A thread's pixels are runs of four, so a step's inputs are two 16-byte loads.
 template <typename TIn, int PXT, int OT, int WPX, int WO, int KC, int PER_SM>
 __global__ void __launch_bounds__(32 * WPX * WO, PER_SM)
@@ -324,9 +338,9 @@ hts_status launch_conv_tile(const ConvParams& p, cudaStream_t s)
 // 27; 64 x 32 tiles 25, 35, 48, 62, 74).  The latency form pays up to three blocks per SM, two where it converts frames (17 against
 // 15).  Large tiles (256 x 32) only take many unaligned frames: one costs as much as 2.5 small ones and 0.7 more for its start.
 template <typename TIn>
-hts_status launch_conv(const ConvParams& p, cudaStream_t s)
+hts_status launch_conv(const ConvParams& p, const StripMaps* maps, cudaStream_t s)
 {
-    const hts_status strips = launch_conv_strip(p, s);
+    const hts_status strips = launch_conv_strip(p, maps, s);
     if (strips != HTS_ERR_UNSUPPORTED) return strips;
     constexpr bool U8 = std::is_same<TIn, uint8_t>::value;
     const size_t px = (size_t)p.n * p.Ho * p.Wo, sms = (size_t)device_sm_count(device_slot());
@@ -338,12 +352,11 @@ hts_status launch_conv(const ConvParams& p, cudaStream_t s)
 }
 
 // h[e,o] = relu(b[o] + sum over lanes l of (chain of f = l, l+32, l+64, ...)), the 32 chains added as a binary tree
-// over the lane number (halves first).  A warp owns TE rows x TO outputs and lane l runs chain l of all of them: both
-// operands are contiguous across the lanes, so neither needs a transposition, and one transposing reduction closes
-// the tree (at each level a lane keeps half of its values and gets its partner's share of them).
-// The block's rows of x and w go through a ring in shared memory, COLS columns at a time.  Bound: large batches by
-// shared memory and the fp32 pipes (8 x 8 per warp: one byte per multiply-add, 128 of each per clock; 8 x 16 leaves too
-// few warps, 149 against 115 us at n = 1024), small ones by the latency of the weights: narrow tiles, deep ring.
+// over the lane number (halves first), for few rows (and callers without tensor maps; fc_f32.cu takes the others).  A warp owns
+// TE rows x TO outputs and lane l runs chain l of all of them: both operands are contiguous across the lanes, so neither needs a
+// transposition, and one transposing reduction closes the tree (at each level a lane keeps half of its values and gets its partner's
+// share of them).  The block's rows of x and w go through a ring in shared memory, COLS columns at a time.  Bound: the latency of the
+// weights: narrow tiles, deep ring.
 template <int TE, int TO, int WE, int WO, int STAGES, int COLS>
 __global__ void __launch_bounds__(32 * WE * WO)
 fc_chain_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ b,
@@ -355,7 +368,7 @@ fc_chain_kernel(const float* __restrict__ x, const float* __restrict__ w, const 
     const int we = warp % WE, wo = warp / WE;
     const int e0 = (blockIdx.y * WE + we) * TE, o0 = (blockIdx.x * WO + wo) * TO;
     pdl_wait();
-    if constexpr (TE < 8) pdl_trigger();
+    pdl_trigger();
     f32x2 acc[TE][TO / 2];
 #pragma unroll
     for (int i = 0; i < TE; ++i)
@@ -452,20 +465,19 @@ hts_status launch_fc_chain(const float* x, const float* w, const float* b, float
     note_launch();
     return HTS_OK;
 }
-// The form goes by the narrow blocks (128 per 16 rows) of the SM that has most of them, k.  One wide block per SM takes as
-// long as five narrow ones, at every width of the layer: step with k = 5 (80 rows) and 6 (81) on 148 SMs, narrow / wide, us:
-// 98.1 / 98.0 and 104.2 / 98.1 with 3136 features, 143.8 / 144.0 and 149.3 / 144.6 with 2560, 36.6 / 37.1 and 37.4 / 37.2
-// with 256.  The fewer narrow blocks an SM has, the more each must have in flight and the less often its warps may meet:
-// stages of 512 columns, three deep at k = 1 and two at k = 2 (both fill the shared memory), of 128 columns above (k = 1 / 2 / 3,
-// 3136 features: 45.4 / 52.4 / 71.5 us with the first, 45.8 / 48.1 / 69.4 with the second, 47.7 / 50.7 / 64.3 with the third).
-hts_status launch_fc(const float* x, const float* w, const float* b, float* h, int n, int F, cudaStream_t s)
+// The form goes by the blocks (128 per 16 rows) of the SM that has most of them, k.  The fewer it has, the more each must have in
+// flight and the less often its warps may meet: stages of 512 columns, three deep at k = 1 and two at k = 2 (both fill the shared
+// memory), of 128 columns above (step at k = 1 / 2 / 3, 3136 features: 45.4 / 52.4 / 71.5 us with the first, 45.8 / 48.1 / 69.4 with the second,
+// 47.7 / 50.7 / 64.3 with the third).  From k = 3 on boxes are faster (the layer alone, this / boxes: 16 rows 9.8 / 12.1 us, 32 rows
+// 11.7 / 12.2, 40 rows 15.8 / 12.3).
+hts_status launch_fc(const float* x, const float* w, const float* b, float* h, int n, int F, const RefWorkspace& ws, int* status, cudaStream_t s)
 {
     const int sms = device_sm_count(device_slot());
     const long k = (128L * ((n + 15) / 16) + sms - 1) / sms;
-    if (k > 5) return launch_fc_chain<8, 8, 4, 2, 4, 64>(x, w, b, h, n, F, s);
     if (k == 1) return launch_fc_chain<4, 4, 4, 1, 3, 512>(x, w, b, h, n, F, s);
     if (k == 2) return launch_fc_chain<4, 4, 4, 1, 2, 512>(x, w, b, h, n, F, s);
-    return launch_fc_chain<4, 4, 4, 1, 4, 128>(x, w, b, h, n, F, s);
+    const hts_status st = ws.maps ? launch_fc_lanes({b, h, n, F, ws.row0, status}, ws.maps->fc, s) : HTS_ERR_UNSUPPORTED;
+    return st != HTS_ERR_UNSUPPORTED ? st : launch_fc_chain<4, 4, 4, 1, 4, 128>(x, w, b, h, n, F, s);
 }
 
 __global__ void __launch_bounds__(256) dense_rows_kernel(const float* __restrict__ x, const RowLayout l, int H, int W, size_t total, float* __restrict__ out)
@@ -493,10 +505,11 @@ hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspac
                        const RefPlanes* planes)
 {
     hts_status st;
+    const StripMaps* maps = ws.maps ? &ws.maps->strips : nullptr;
     auto layer = [&](const void* x, const RowLayout& xl, const float* wt, const float* wk, const float* b, float* y, const RowLayout& yl, int C, int H,
                      int W, int O, int k, int stride, int Ho, int Wo) {
         ConvParams p{};
-        p.x = x; p.xl = xl; p.w = wt; p.wk = wk; p.b = b; p.y = y; p.yl = yl; p.n = n; p.C = C; p.H = H; p.W = W; p.O = O; p.k = k; p.s = stride; p.Ho = Ho; p.Wo = Wo;
+        p.x = x; p.xl = xl; p.w = wt; p.wk = wk; p.b = b; p.y = y; p.yl = yl; p.n = n; p.frame0 = ws.row0; p.C = C; p.H = H; p.W = W; p.O = O; p.k = k; p.s = stride; p.Ho = Ho; p.Wo = Wo;
         p.status = status; p.in_scale = 1.f; p.w_vec = ((uintptr_t)wt & 15) == 0; p.words = ((uintptr_t)x & 3) == 0;
         return p;
     };
@@ -504,23 +517,23 @@ hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspac
     ConvParams c1 = layer(obs, rows_dense(g.H, g.W), w.w1, w.w1k, w.b1, ws.a1, ws.l1, g.C, g.H, g.W, 32, 8, 4, g.H1, g.W1);
     c1.in_scale = 1.0f / 255.0f; c1.slots = ix.slots; c1.pool = ix.pool;
     if (planes) { c1.planes = planes->a1; c1.plane = planes->p1; c1.s2d = true; c1.W_rows = (g.W1 + 1) / 2; c1.P_rows = (g.H1 + 1) / 2 * c1.W_rows; }
-    st = launch_conv<uint8_t>(c1, s);
+    st = launch_conv<uint8_t>(c1, nullptr, s);
     if (st != HTS_OK) return st;
     prof.end(K_CONV1, s);
     prof.begin(K_CONV2, s);
     ConvParams c2 = layer(ws.a1, ws.l1, w.w2, w.w2k, w.b2, ws.a2, ws.l2, 32, g.H1, g.W1, 64, 4, 2, g.H2, g.W2);
     if (planes) { c2.planes = planes->a2; c2.plane = planes->p2; c2.P_rows = g.H2 * g.W2; }
-    st = launch_conv<float>(c2, s);
+    st = launch_conv<float>(c2, maps, s);
     if (st != HTS_OK) return st;
     prof.end(K_CONV2, s);
     prof.begin(K_CONV3, s);
     ConvParams c3 = layer(ws.a2, ws.l2, w.w3, w.w3k, w.b3, ws.a3, rows_dense(g.H3, g.W3), 64, g.H2, g.W2, 64, 3, 1, g.H3, g.W3);
     if (planes) { c3.planes = planes->a3; c3.plane = planes->p3; c3.P_rows = g.H3 * g.W3; }
-    st = launch_conv<float>(c3, s);
+    st = launch_conv<float>(c3, maps, s);
     if (st != HTS_OK) return st;
     prof.end(K_CONV3, s);
     prof.begin(K_FC, s);
-    st = launch_fc(ws.a3, w.wfc, w.bfc, ws.h, n, g.F, s);
+    st = launch_fc(ws.a3, w.wfc, w.bfc, ws.h, n, g.F, ws, status, s);
     if (st != HTS_OK) return st;
     prof.end(K_FC, s);
     return HTS_OK;
@@ -576,7 +589,7 @@ extern "C" hts_status hts_policy_step_noalloc(const hts_net_desc* d, const hts_w
     }
     float* base = g_noalloc_ptr[dev];
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    const RefWorkspace ws{base, base + f_a1, base + f_a1 + f_a2, base + f_a1 + f_a2 + f_a3, rows_dense(g.H1, g.W1), rows_dense(g.H2, g.W2)};
+    const RefWorkspace ws{base, base + f_a1, base + f_a1 + f_a2, base + f_a1 + f_a2 + f_a3, rows_dense(g.H1, g.W1), rows_dense(g.H2, g.W2), nullptr, 0};
     float* whead = ws.h + f_h;
     float* bhead = whead + f_wh;
     // every scratch float is written before it is read, so nothing has to start at zero

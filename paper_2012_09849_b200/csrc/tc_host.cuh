@@ -70,5 +70,35 @@ inline bool make_frames_map(CUtensorMap* m, const void* ptr, int W, int H, int C
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// fp32 row-major [rows, cols], box [box_rows x box_cols], no swizzle, zero fill.
+inline bool make_f32_map(CUtensorMap* m, const float* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_cols)
+{
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[2] = {cols, rows};
+    const cuuint64_t strides[1] = {cols * 4};
+    const cuuint32_t box[2] = {box_cols, box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// fp32 activations seen as (x, row of a phase, phase, channel, frame); box = whole rows, `rows` of them in every phase of `channels`
+// channels of one frame.
+inline bool make_rows_map(CUtensorMap* m, const float* ptr, int pitch, int phase_rows, int phases, int C, uint64_t frames, int rows, int channels)
+{
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t row = (cuuint64_t)pitch * 4, phase = row * phase_rows, chan = phase * phases;
+    const cuuint64_t dims[5] = {(cuuint64_t)pitch, (cuuint64_t)phase_rows, (cuuint64_t)phases, (cuuint64_t)C, frames};
+    const cuuint64_t strides[4] = {row, phase, chan, chan * C};
+    const cuuint32_t box[5] = {(cuuint32_t)pitch, (cuuint32_t)rows, (cuuint32_t)phases, (cuuint32_t)channels, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<float*>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace tc
 }  // namespace hts
