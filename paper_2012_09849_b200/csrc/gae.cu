@@ -11,6 +11,7 @@
 // 17 bytes per element.  The replay uses the same operation order as the sequential
 // recurrence, so only the incoming carry differs from it, by rounding.
 #include "common.cuh"
+#include "scan_chain.cuh"
 
 namespace hts {
 namespace {
@@ -37,8 +38,10 @@ template <> __device__ __forceinline__ float4 pack<4>(const float* o) { return m
 // blocks four times narrower (8 columns: still whole 32-byte sectors per row) so that a problem with few
 // columns spreads over four times as many SMs.  Chunk boundaries, and with them every rounding, do not depend
 // on CY or W.
-template <int VEC, int L, int CY>
-__global__ void __launch_bounds__(VEC == 4 ? 64 : 1024)
+// ROOMY: as many registers as a block alone on its SM can have, so that all of a chunk's loads are in flight together (110 instead of
+// 64; 4.02 -> 3.80 us at 512 x 512).  It pays while no SM has a second block: 128 x 5000 4.6 / 5.4 us, 512 x 20000 43 / 59.
+template <int VEC, int L, int CY, bool MANY, bool ROOMY>
+__global__ void __launch_bounds__(VEC == 4 ? 64 : ROOMY ? 512 : 1024, ROOMY ? 1 : 0)
 gae_scan_kernel(const float* __restrict__ rewards, const float* __restrict__ values,
                 const uint8_t* __restrict__ dones, const float* __restrict__ bootstrap,
                 float gamma, float lambda, int T, int N,
@@ -120,11 +123,18 @@ gae_scan_kernel(const float* __restrict__ rewards, const float* __restrict__ val
         float c[VEC], mine[VEC];
 #pragma unroll
         for (int k = 0; k < VEC; ++k) { c[k] = carry_in[k]; mine[k] = 0.f; }
-        for (int ww = NC - 1; ww >= 0; --ww) {
+        if constexpr (MANY) {
+            if (threadIdx.y == 0 && threadIdx.x < CXW) walk_chunks(sS + cx, sP + cx, cols, NC, c[0]);
+            __syncthreads();
+            mine[0] = sS[w * cols + cx];
+            c[0] = sP[cx];
+        } else {
+            for (int ww = NC - 1; ww >= 0; --ww) {
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) {
-                if (ww == w) mine[k] = c[k];
-                c[k] = sS[ww * cols + cx * VEC + k] + sP[ww * cols + cx * VEC + k] * c[k];
+                for (int k = 0; k < VEC; ++k) {
+                    if (ww == w) mine[k] = c[k];
+                    c[k] = sS[ww * cols + cx * VEC + k] + sP[ww * cols + cx * VEC + k] * c[k];
+                }
             }
         }
 #pragma unroll
@@ -162,7 +172,11 @@ hts_status launch_t(const float* r, const float* v, const uint8_t* d, const floa
     const int cols = 32 / CY * VEC;
     const unsigned blocks = (unsigned)((N + cols - 1) / cols);
     const size_t smem = (size_t)2 * W * CY * cols * sizeof(float);
-    HTS_CUDA(launch_pdl(gae_scan_kernel<VEC, L, CY>, dim3(blocks), dim3(32, W), smem, s, r, v, d, b, gamma, lambda, T, N, adv, ret));
+    constexpr bool V1 = VEC == 1;
+    const bool many = V1 && W * CY >= kManyChunks, roomy = V1 && W <= 16 && (int)blocks <= device_sm_count(device_slot());
+    auto kernel = many ? (roomy ? gae_scan_kernel<VEC, L, CY, V1, V1> : gae_scan_kernel<VEC, L, CY, V1, false>)
+                       : (roomy ? gae_scan_kernel<VEC, L, CY, false, V1> : gae_scan_kernel<VEC, L, CY, false, false>);
+    HTS_CUDA(launch_pdl(kernel, dim3(blocks), dim3(32, W), smem, s, r, v, d, b, gamma, lambda, T, N, adv, ret));
     note_launch();
     return HTS_OK;
 }

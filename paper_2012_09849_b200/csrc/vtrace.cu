@@ -12,6 +12,7 @@
 // affine map, the block chains the chunk maps through shared memory, and each thread replays its chunk with
 // the true incoming D.  One pass over HBM: 21 bytes per element.
 #include "common.cuh"
+#include "scan_chain.cuh"
 
 namespace hts {
 namespace {
@@ -43,8 +44,10 @@ struct VtraceParams {
 // blockDim = (32, W).  A warp is CY rows of 32/CY threads, as in the advantage scan: thread (cx, cy) of warp w owns
 // columns [b*cols + cx*VEC, +VEC) (cols = 32/CY*VEC) and chunk w*CY + cy of the super-chunk.  Time is walked from the
 // end in super-chunks of W*CY*L rows.  Chunk boundaries, and with them every rounding, do not depend on CY or W.
-template <int VEC, int L, int CY, int MAXW>
-__global__ void __launch_bounds__(32 * MAXW)
+// ROOMY: as many registers as a block alone on its SM can have, so that all of a chunk's loads are in flight together (115 instead of
+// 93; 3.29 -> 2.73 us at 128 x 1024).  It pays while no SM has a second block: 512 x 8000 (two per SM) 28.9 / 29.3 us.
+template <int VEC, int L, int CY, int MAXW, bool MANY, bool ROOMY>
+__global__ void __launch_bounds__(32 * MAXW, ROOMY ? 1 : 0)
 vtrace_scan_kernel(const VtraceParams p)
 {
     using F = typename VecT<VEC>::F;
@@ -127,11 +130,31 @@ vtrace_scan_kernel(const VtraceParams p)
         float c[VEC], mine[VEC];
 #pragma unroll
         for (int k = 0; k < VEC; ++k) { c[k] = carry_in[k]; mine[k] = 0.f; }
-        for (int ww = W - 1; ww >= 0; --ww) {
+        if constexpr (MANY) {
+            if (threadIdx.y == 0 && threadIdx.x < CXW) walk_chunks(sS + lane, sP + lane, cols, W, c[0]);
+            __syncthreads();
+            mine[0] = sS[w * cols + lane];
+            c[0] = sP[lane];
+        } else {
+            int ww = W - 1;
+            if constexpr (ROOMY) {                       // four maps loaded at a time
+                for (; ww >= 3; ww -= 4) {
+                    float S4[4], P4[4];
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) {
-                if (ww == w) mine[k] = c[k];
-                c[k] = sS[ww * cols + lane * VEC + k] + sP[ww * cols + lane * VEC + k] * c[k];
+                    for (int i = 0; i < 4; ++i) { S4[i] = sS[(ww - i) * cols + lane]; P4[i] = sP[(ww - i) * cols + lane]; }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (ww - i == w) mine[0] = c[0];
+                        c[0] = S4[i] + P4[i] * c[0];
+                    }
+                }
+            }
+            for (; ww >= 0; --ww) {
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) {
+                    if (ww == w) mine[k] = c[k];
+                    c[k] = sS[ww * cols + lane * VEC + k] + sP[ww * cols + lane * VEC + k] * c[k];
+                }
             }
         }
 #pragma unroll
@@ -168,7 +191,11 @@ hts_status launch_t(const VtraceParams& p, cudaStream_t s)
     const int cols = 32 / CY * VEC;
     const unsigned blocks = (unsigned)((p.N + cols - 1) / cols);
     const size_t smem = (size_t)2 * W * CY * cols * sizeof(float);
-    HTS_CUDA(launch_pdl(vtrace_scan_kernel<VEC, L, CY, MAXW>, dim3(blocks), dim3(32, W), smem, s, p));
+    constexpr bool V1 = VEC == 1, M = V1 && MAXW * CY >= kManyChunks;
+    const bool many = M && W * CY >= kManyChunks, roomy = V1 && (int)blocks <= device_sm_count(device_slot());
+    auto kernel = many ? (roomy ? vtrace_scan_kernel<VEC, L, CY, MAXW, M, V1> : vtrace_scan_kernel<VEC, L, CY, MAXW, M, false>)
+                       : (roomy ? vtrace_scan_kernel<VEC, L, CY, MAXW, false, V1> : vtrace_scan_kernel<VEC, L, CY, MAXW, false, false>);
+    HTS_CUDA(launch_pdl(kernel, dim3(blocks), dim3(32, W), smem, s, p));
     note_launch();
     return HTS_OK;
 }
