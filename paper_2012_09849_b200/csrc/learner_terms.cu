@@ -10,6 +10,8 @@
 // function of the count alone, so the result does not depend on timing or on the device's load.
 #include <cmath>
 #include "common.cuh"
+#include "f32x2.cuh"
+#include "tc_ptx.cuh"
 
 namespace hts {
 namespace {
@@ -199,12 +201,13 @@ struct AdvStatsOp {
         one(g.x, f, acc); one(g.y, f, acc); one(g.z, f, acc); one(g.w, f, acc);
     }
     __device__ void add1(long long i, double* acc) const { one(adv[i], (double)adv[0], acc); }
-    __device__ void finish(const double* tot, long long count) const
+    __device__ static void standardise(double sum, double squares, double first, long long count, double* stats)
     {
-        const double d = tot[0] / (double)count, var = tot[1] / (double)count - d * d;
-        g_adv_stats[0] = (double)adv[0] + d;
-        g_adv_stats[1] = 1.0 / (sqrt(var > 0.0 ? var : 0.0) + 1e-8);
+        const double d = sum / (double)count, var = squares / (double)count - d * d;
+        stats[0] = first + d;
+        stats[1] = 1.0 / (sqrt(var > 0.0 ? var : 0.0) + 1e-8);
     }
+    __device__ void finish(const double* tot, long long count) const { standardise(tot[0], tot[1], (double)adv[0], count, g_adv_stats); }
 };
 
 // IN_TURN: an element's sums are finished before the next one's are begun (the compiler otherwise works on all eight of two groups
@@ -240,25 +243,148 @@ struct PpoOp {
         if constexpr (IN_TURN)
             asm volatile("" : "+f"(ln), "+f"(lo), "+f"(v), "+f"(a), "+f"(r), "+d"(acc[0]), "+d"(acc[1]), "+d"(acc[2]), "+d"(acc[3]));
     }
-    __device__ void add4(Quad g, double* acc) const
+    __device__ void add4(Quad g, double m, double is, double* acc) const
     {
-        const double m = normalize ? g_adv_stats[0] : 0.0, is = normalize ? g_adv_stats[1] : 1.0;
         in_turn(g.ln.x, g.lo.x, g.v.x, g.a.x, g.r.x, acc); one(g.ln.x, g.lo.x, g.v.x, g.h.x, g.a.x, g.r.x, m, is, acc);
         in_turn(g.ln.y, g.lo.y, g.v.y, g.a.y, g.r.y, acc); one(g.ln.y, g.lo.y, g.v.y, g.h.y, g.a.y, g.r.y, m, is, acc);
         in_turn(g.ln.z, g.lo.z, g.v.z, g.a.z, g.r.z, acc); one(g.ln.z, g.lo.z, g.v.z, g.h.z, g.a.z, g.r.z, m, is, acc);
         in_turn(g.ln.w, g.lo.w, g.v.w, g.a.w, g.r.w, acc); one(g.ln.w, g.lo.w, g.v.w, g.h.w, g.a.w, g.r.w, m, is, acc);
     }
-    __device__ void add1(long long i, double* acc) const
+    __device__ void add1(long long i, double m, double is, double* acc) const
     {
-        const double m = normalize ? g_adv_stats[0] : 0.0, is = normalize ? g_adv_stats[1] : 1.0;
         one(logp_new[i], logp_old[i], values[i], entropy[i], adv[i], returns[i], m, is, acc);
     }
+    __device__ void add4(const Quad& g, double* acc) const { add4(g, normalize ? g_adv_stats[0] : 0.0, normalize ? g_adv_stats[1] : 1.0, acc); }
+    __device__ void add1(long long i, double* acc) const { add1(i, normalize ? g_adv_stats[0] : 0.0, normalize ? g_adv_stats[1] : 1.0, acc); }
     __device__ void finish(const double* tot, long long count) const
     {
         const double inv = 1.0 / (double)count;
         for (int k = 0; k < 4; ++k) out[k] = (float)(tot[k] * inv);
     }
 };
+
+// Standardised terms of few transitions in one launch: a cluster of up to 16 blocks whose shared memory holds all inputs, so that
+// the advantages' statistics and the terms are two passes over it, with the blocks' sums exchanged through each other's shared
+// memory in between.  The sums' order is fixed by the count; nothing global is written but the results.  Bound: one launch (4.3 us
+// for the host, where two take 6.5), then copies into at most 16 SMs.  Standardised means, us, calls in a row:
+//   transitions        64   2048  16384  50000  131072  147455
+//   two launches     7.67   8.26   8.13   8.52    9.06    9.93
+//   one              4.67   4.61   5.15   6.08    7.95    8.30
+// so it is taken as long as the inputs fit.  512 transitions to a block (2048: 5.42 at 2048; 256: the same).  A cooperative launch
+// of sums_kernel's blocks with a barrier across the grid: 8.2 whatever the count, 9.3 at 131072.  The terms without the advantages
+// summed while the statistics cross the cluster: 8.24 at 131072 (the ratios pass through shared memory once more).
+constexpr int kClusterMost = 16, kClusterThreads = 512, kClusterHolds = 9216;      // transitions of a block: 24 bytes each
+constexpr int kClusterEach = 512;                        // transitions before another block is worth its place
+constexpr int kClusterWarps = kClusterThreads / 32;
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void store_to_rank(double* here, unsigned rank, double v)
+{
+    uint32_t there;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(tc::smem_u32(here)), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there), "d"(v) : "memory");
+}
+
+__global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const PpoOp<false> op, int count, int per_block)
+{
+    constexpr int NS = PpoOp<false>::NS;
+    extern __shared__ float4 s_in[];                     // [6][per_block / 4]: advantages first
+    __shared__ double s_warp[kClusterWarps][NS], s_stat[kClusterMost][2], s_all[kClusterMost][NS];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const unsigned rank = blockIdx.x, ranks = gridDim.x;
+    pdl_wait();
+    pdl_trigger();
+    const int lo = rank * per_block, n = max(0, min(per_block, count - lo)), quads = n >> 2, pitch = per_block >> 2;
+    const float* const arrays[6] = {op.adv, op.logp_new, op.logp_old, op.values, op.entropy, op.returns};
+    const double first = (double)op.adv[0];
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+        for (int q = tid; q < quads; q += kClusterThreads) cp_async16(tc::smem_u32(s_in + a * pitch + q), reinterpret_cast<const float4*>(arrays[a] + lo) + q);
+        if (a == 0) cp_async_commit();
+    }
+    cp_async_commit();
+    // A thread reads what it copied itself.  The last block's ragged transitions are read where they are.
+    const int i = lo + 4 * quads + tid;
+    const bool ragged = tid < (n & 3);
+    double st[2] = {0.0, 0.0};
+    cp_async_wait<1>();
+    for (int q = tid; q < quads; q += kClusterThreads) {
+        const float4 a = s_in[q];
+        AdvStatsOp::one(a.x, first, st); AdvStatsOp::one(a.y, first, st); AdvStatsOp::one(a.z, first, st); AdvStatsOp::one(a.w, first, st);
+    }
+    if (ragged) AdvStatsOp::one(op.adv[i], first, st);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        st[k] = warp_sum_d(st[k]);
+        if (lane == 0) s_warp[warp][k] = st[k];
+    }
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const double v = warp_sum_d(lane < kClusterWarps ? s_warp[lane][k] : 0.0);
+            if (lane < ranks) store_to_rank(&s_stat[rank][k], lane, v);
+        }
+    }
+    cluster_sync();
+    double stats[2], tot[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) tot[k] = warp_sum_d(lane < ranks ? s_stat[lane][k] : 0.0);
+    AdvStatsOp::standardise(tot[0], tot[1], first, count, stats);
+    double acc[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) acc[k] = 0.0;
+    cp_async_wait_all();
+    for (int q = tid; q < quads; q += kClusterThreads)
+        op.add4(PpoOp<false>::Quad{s_in[pitch + q], s_in[2 * pitch + q], s_in[3 * pitch + q], s_in[4 * pitch + q], s_in[q], s_in[5 * pitch + q]},
+                stats[0], stats[1], acc);
+    if (ragged) op.add1(i, stats[0], stats[1], acc);
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+        acc[k] = warp_sum_d(acc[k]);
+        if (lane == 0) s_warp[warp][k] = acc[k];         // the statistics in it were read before the cluster's barrier
+    }
+    __syncthreads();
+    if (warp == 0)
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            const double v = warp_sum_d(lane < kClusterWarps ? s_warp[lane][k] : 0.0);
+            if (lane == 0) store_to_rank(&s_all[rank][k], 0, v);
+        }
+    cluster_sync();
+    if (rank == 0 && warp == 0) {
+#pragma unroll
+        for (int k = 0; k < NS; ++k) acc[k] = warp_sum_d(lane < ranks ? s_all[lane][k] : 0.0);
+        if (lane == 0) op.finish(acc, count);
+    }
+}
+
+cudaError_t launch_terms_cluster(const PpoOp<false>& op, int count, cudaStream_t s)
+{
+    int ranks = 1;
+    while (ranks < kClusterMost && ranks * kClusterEach < count) ranks *= 2;
+    const int per_block = ((count + ranks - 1) / ranks + 3) / 4 * 4;
+    static OncePerDevice allowed, sized;
+    cudaError_t e = allow_shared(terms_cluster_kernel, allowed);
+    std::atomic<bool>& done = sized[device_slot()];
+    if (e == cudaSuccess && !done.load(std::memory_order_acquire)) {
+        e = cudaFuncSetAttribute(terms_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e == cudaSuccess) done.store(true, std::memory_order_release);
+    }
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ranks); cfg.blockDim = dim3(kClusterThreads); cfg.dynamicSmemBytes = (size_t)per_block * 24; cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)ranks; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, terms_cluster_kernel, op, count, per_block);
+}
 
 }  // namespace
 }  // namespace hts
@@ -280,13 +406,17 @@ extern "C" hts_status hts_ppo_terms(const float* logp_new, const float* logp_old
     if (!logp_new || !logp_old || !values || !entropy || !advantages || !returns || !out4 || count < 1) return HTS_ERR_INVALID_ARG;
     if (!(clip > 0.f) || std::isinf(clip)) return HTS_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    if (normalize_advantages) {
-        const hts_status st = launch_sums(AdvStatsOp{advantages, all_aligned16({advantages})}, (long long)count, s);
-        if (st != HTS_OK) return st;
-    }
     const bool vec = all_aligned16({logp_new, logp_old, values, entropy, advantages, returns});
     const PpoOp<false> op{logp_new, logp_old, values, entropy, advantages, returns, out4, (double)clip, normalize_advantages != 0, vec};
     if (!normalize_advantages) return launch_sums(op, (long long)count, s);
+    if (vec && count <= kClusterMost * kClusterHolds) {
+        const cudaError_t e = launch_terms_cluster(op, (int)count, s);
+        if (e == cudaSuccess) { note_launch(); return HTS_OK; }
+        if (e != cudaErrorInvalidClusterSize) return cuda_fail(e, "terms_cluster_kernel");
+        cudaGetLastError();                              // a part of a device that has no room for the cluster: two launches
+    }
+    const hts_status st = launch_sums(AdvStatsOp{advantages, all_aligned16({advantages})}, (long long)count, s);
+    if (st != HTS_OK) return st;
     const SumsGrid grid = sums_grid((long long)count);
     if (grid.blocks <= 2LL * device_sm_count(device_slot()) && grid.per_block <= kThreads * kPerThread)
         return launch_sums<Form::EarlyTwo>(op, (long long)count, s);

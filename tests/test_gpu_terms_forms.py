@@ -8,12 +8,7 @@ import paper_2012_09849_b200 as hts
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("aligned", [True, False])
-@pytest.mark.parametrize("blocks_per_sm,blocks", [(2, 0), (3, 0), (0, 2048)])
-@pytest.mark.parametrize("more", [-3, 0, 1, 2053])
-def test_against_64_bits(blocks_per_sm, blocks, more, aligned):
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
-    count = (blocks or blocks_per_sm * sms) * 2048 + more
+def check(count, aligned):
     g = torch.Generator(device="cuda").manual_seed(count)
     x = [torch.randn(count + 1, device="cuda", generator=g) for _ in range(6)]
     x[1] = x[0] + 0.2 * x[1]
@@ -31,3 +26,18 @@ def test_against_64_bits(blocks_per_sm, blocks, more, aligned):
         assert abs(out[0, k].item() - ref[k].item()) <= 2.0 ** -20 * scale[k].item(), k
     # of the ratios, that exponential moves about one in a million across the edge of the clip range
     assert abs(out[0, 3].item() - ((rho - 1).abs() > clip).double().mean().item()) <= 2e-6 + 2.0 / count
+
+
+@pytest.mark.parametrize("aligned", [True, False])
+@pytest.mark.parametrize("blocks_per_sm,blocks", [(2, 0), (3, 0), (0, 2048)])
+@pytest.mark.parametrize("more", [-3, 0, 1, 2053])
+def test_against_64_bits(blocks_per_sm, blocks, more, aligned):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    check((blocks or blocks_per_sm * sms) * 2048 + more, aligned)
+
+
+# one block, more blocks, ragged ends and blocks without a transition, as many as the blocks' shared memory holds, and one more
+@pytest.mark.parametrize("aligned", [True, False])
+@pytest.mark.parametrize("count", [1, 3, 4, 7, 512, 513, 2047, 2049, 8191, 8193, 70001, 147453, 147456, 147457])
+def test_few_transitions_against_64_bits(count, aligned):
+    check(count, aligned)
