@@ -626,38 +626,47 @@ hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, 
     HTS_CUDA(launch_pdl(head_wgrad_kernel, dim3(8, rh, nblk(g.A + 2, kHeadTile)), dim3(256), 0, s, t->dhead, ws.h, t->dh, ph, n, g.A, per_range,
                         t->headp));
     note_launch();
-    st = x3_dgrad_launch(t->mDh, t->mWf, run(t->bfc, N, t->dz3, p2, t->a3, g.F), s);
-    if (st != HTS_OK) return st;
-    st = x3_dgrad_launch(t->mDz3, t->mW3, run(t->bc3, N * t->P2, t->dz2, pz2, t->a2, 64), s);
-    if (st != HTS_OK) return st;
-    st = x3_dgrad_launch(t->mDz2, t->mW2, run(t->bc2, N * t->P1s, t->dz1, 32, t->a1, 128), s);
-    if (st != HTS_OK) return st;
 
-    // ---- weight gradients: as many ranges of rows as SMs, each with at least one stage of rows
+    // ---- data and weight gradients: ranges of at least one stage of rows
     auto cut = [&](X3WgradParams p, size_t rows, int ranges, int last) {
         p.row_chunks = (int)((rows + p.kr - 1) / p.kr);
+        ranges = ranges < 1 ? 1 : ranges; last = last < 1 ? 1 : last;
         p.ranges = ranges < p.row_chunks ? ranges : p.row_chunks;
         p.last_ranges = last < p.row_chunks ? last : p.row_chunks;
         return p;
     };
+    // Passes that do not wait for each other share a launch.  Blocks, one to an SM: of the dense layer's data gradient two thirds of
+    // the SMs' at most, then its weight gradient's 128 x 128 outputs follow as SMs become free; conv3's data gradient gets its share of
+    // the work (58 %: 45 to 58 % are the same within 2 % where tiles do not quantise, 256 and 512 rows gain 4 and 2 % from it), in
+    // equal rounds; conv1's and conv2's weight gradients share by rows x their cost per row.  Gradient without its forward pass, us,
+    // one launch per pass / now: 84 x 84 x 4 at 5 rows 75 / 57, 80 98 / 73, 256 147 / 125, 512 221 / 184, 1024 341 / 318; 72 x 96 x 16 at
+    // 40 93 / 71, 512 283 / 261.
     X3WgradParams q = cut(t->wfc, N, 1, 1);
     q.fc_w = t->partf;
-    st = x3_wgrad_launch<3, 64>(t->vDh, t->vA3, q, s);
+    const X3TapParams df = run(t->bfc, N, t->dz3, p2, t->a3, g.F);
+    const int tiles_f = df.m_tiles * df.n_tiles, share_f = sms * 2 / 3 < 1 ? 1 : sms * 2 / 3;
+    st = x3_data_weights_launch(t->mDh, t->mWf, df, tiles_f < share_f ? tiles_f : share_f, t->vDh, t->vA3, q, s);
     if (st != HTS_OK) return st;
-    ReduceParams r{};
-    X3WgradParams q3 = cut(t->wc3, N * t->P2, sms * 2 / 5 < 1 ? 1 : sms * 2 / 5, sms / 5 < 1 ? 1 : sms / 5);   // the last kind has one group of five
+    const X3TapParams d3 = run(t->bc3, N * t->P2, t->dz2, pz2, t->a2, 64);
+    const int share_3 = sms * 58 / 100 < 1 ? 1 : sms * 58 / 100, rounds = (d3.m_tiles + share_3 - 1) / share_3;
+    const int blocks_3 = (d3.m_tiles + rounds - 1) / rounds, left = sms - blocks_3;
+    X3WgradParams q3 = cut(t->wc3, N * t->P2, left * 2 / 5, left / 5);          // the last kind has one group of five
     q3.part = t->part3; q3.group_stride = (size_t)q3.ranges * 8192; q3.bias_part = t->bias3;
-    st = x3_wgrad_launch<3, 64>(t->vA2, t->vDz3, q3, s);
+    st = x3_data_weights_launch(t->mDz3, t->mW3, d3, blocks_3, t->vA2, t->vDz3, q3, s);
     if (st != HTS_OK) return st;
-    X3WgradParams q2 = cut(t->wc2, N * t->P1s, sms / 2 < 1 ? 1 : sms / 2, sms / 2 < 1 ? 1 : sms / 2);
+    st = x3_dgrad_launch(t->mDz2, t->mW2, run(t->bc2, N * t->P1s, t->dz1, 32, t->a1, 128), s);
+    if (st != HTS_OK) return st;
+    const double cost2 = 5.4 * t->P1s, cost1 = (double)t->wc1.kinds * t->G0;    // 0.44 and 0.082 ns a row
+    int n2 = (int)(sms * cost2 / (cost1 + cost2) + 0.5);
+    X3WgradParams q2 = cut(t->wc2, N * t->P1s, n2 / 2, n2 / 2);
     q2.part = t->part2; q2.group_stride = (size_t)q2.ranges * 8192; q2.bias_part = t->bias2;
-    st = x3_wgrad_launch<3, 64>(t->vA1, t->vDz2, q2, s);
-    if (st != HTS_OK) return st;
-    const int r1 = sms / t->wc1.kinds < 1 ? 1 : sms / t->wc1.kinds;
+    n2 = 2 * q2.ranges;
+    const int r1 = (sms - n2) / t->wc1.kinds;
     X3WgradParams q1 = cut(t->wc1, N * t->G0, r1, r1);
     q1.part = t->part1; q1.group_stride = (size_t)q1.ranges * 4096; q1.bias_part = t->bias1;
-    st = x3_wgrad_launch<1, 32>(t->vX0, t->vDz1, q1, s);
+    st = x3_weights_launch(t->vA1, t->vDz2, q2, t->vX0, t->vDz1, q1, s);
     if (st != HTS_OK) return st;
+    ReduceParams r{};
     r.c1 = t->part1; r.c2 = t->part2; r.c3 = t->part3; r.b1 = t->bias1; r.b2 = t->bias2; r.b3 = t->bias3; r.head = t->headp;
     r.r1 = q1.ranges; r.r2 = q2.ranges; r.r3 = q3.ranges; r.r3_last = q3.last_ranges; r.rh = rh;
     r.g1 = q1.group_stride; r.g2 = q2.group_stride; r.g3 = q3.group_stride;

@@ -86,14 +86,17 @@ __device__ __forceinline__ void acc_release(uint64_t* empty_bar, int lane)
 // 51 us alone) and no other unit for more than half: one thread issues, an instruction every 55 to 70 clocks at best.
 // An A entry (all planes, rows 128 + spread) is loaded once per tile and every tap reads it shifted; B is streamed.
 constexpr int kAccs = 2, kPart = 2, kThreads = 64 + 256;
-__global__ void __launch_bounds__(kThreads)
-x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const X3TapParams p)
+struct DgradShared {
+    uint64_t a_full[kMaxEntries], a_empty[kMaxEntries], b_full[kMaxStages], b_empty[kMaxStages], d_full[kAccs], d_empty[kAccs];
+    uint32_t tmem_slot;
+    int abort_flag;
+};
+// Block `first` of `blocks`.
+__device__ __forceinline__ void x3_dgrad(const CUtensorMap& tmA, const CUtensorMap& tmB, const X3TapParams& p, uint8_t* smem_raw, DgradShared& sh,
+                                         int first, int blocks)
 {
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t a_full[kMaxEntries], a_empty[kMaxEntries], b_full[kMaxStages], b_empty[kMaxStages], d_full[kAccs], d_empty[kAccs];
-    __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
-    volatile int* abortp = &abort_flag;
+    uint64_t *a_full = sh.a_full, *a_empty = sh.a_empty, *b_full = sh.b_full, *b_empty = sh.b_empty, *d_full = sh.d_full, *d_empty = sh.d_empty;
+    volatile int* abortp = &sh.abort_flag;
     constexpr int BB = 3 * 8192;                        // bytes of a B stage: [plane][64 K rows][64 columns]
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const int plane_bytes = p.entry_rows * 128;
@@ -107,16 +110,16 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         for (int i = 0; i < kMaxEntries; ++i) { mbar_init(&a_full[i], 1); mbar_init(&a_empty[i], 1); }
         for (int i = 0; i < kMaxStages; ++i) { mbar_init(&b_full[i], 1); mbar_init(&b_empty[i], 1); }
         for (int i = 0; i < kAccs; ++i) { mbar_init(&d_full[i], 1); mbar_init(&d_empty[i], 8); }
-        abort_flag = 0;
+        sh.abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
     }
-    if (warp == 1) tmem_alloc(&tmem_slot, 512);
+    if (warp == 1) tmem_alloc(&sh.tmem_slot, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_d = tmem_slot;
+    const uint32_t tmem_d = sh.tmem_slot;
     pdl_wait();
     pdl_trigger();
 
@@ -126,7 +129,7 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             int ea = 0, sb = 0;
             uint32_t pa = 1, pb = 1;                    // parity of the "empty" phase waited for
             bool alive = true;
-            for (int t = blockIdx.x; alive && t < tiles; t += gridDim.x) {
+            for (int t = first; alive && t < tiles; t += blocks) {
                 const int mt = t % p.m_tiles, nt = t / p.m_tiles;
                 for (int c = 0; alive && c < p.chunks; ++c) {
                     const int kc = c * 64;
@@ -151,7 +154,7 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             uint32_t pa = 0, pb = 0;
             bool alive = true;
             const uint64_t a_plane = (uint64_t)(plane_bytes >> 4);
-            for (int t = blockIdx.x; alive && t < tiles; t += gridDim.x, left = p.chunks * p.taps)
+            for (int t = first; alive && t < tiles; t += blocks, left = p.chunks * p.taps)
                 for (int c = 0; alive && c < p.chunks; ++c)
                     for (int g = 0; alive && g < groups; ++g) {
                         if (!mbar_wait(&a_full[ea], pa, abortp, p.status, 84)) { alive = false; break; }
@@ -175,12 +178,12 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         if (++ea == p.entries) { ea = 0; pa ^= 1u; }
                     }
         }
-    } else {
+    } else if (warp < kThreads / 32) {
         const int j = (warp - 2) >> 2, q = warp & 3;    // half of the columns; TMEM lane quarter of this warp
         const int row = q * 32 + lane, parts = (p.chunks * p.taps + kPart - 1) / kPart;
         int it = 0;
         bool alive = true;
-        for (int t = blockIdx.x; alive && t < tiles; t += gridDim.x) {
+        for (int t = first; alive && t < tiles; t += blocks) {
             const int mt = t % p.m_tiles, nt = t / p.m_tiles;
             const int m = mt * 128 + row;
             int env = m / p.P, pix = m - env * p.P;
@@ -239,6 +242,13 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_d, 512);
 }
+__global__ void __launch_bounds__(kThreads)
+x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const X3TapParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ DgradShared sh;
+    x3_dgrad(tmA, tmB, p, smem_raw, sh, blockIdx.x, gridDim.x);
+}
 
 // One CTA = (kind, range of row chunks).  Warp 0 copies, warps 1 and 2 issue, two sets of four warps (3..6, 7..10) keep
 // the sums in registers (see "Accumulation" in x3_gemm.cuh).  Issuing thread e has accumulators of its own and set e
@@ -251,20 +261,23 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 // Both operands have the contracted index along their rows (pixels), so tiles go from global memory to the tensor
 // core without a transposition; a tap is a row offset into the slab, and the two taps (or slabs) of a group are two
 // 64-row blocks of M at a free distance (the leading byte offset).  Tensor core: 208 clocks per 16 rows and group (56 for
-// frames); busy for 51 / 54 / 50 % of the time (dense, conv3, conv2 at n = 1024: 32 / 45 / 48 us alone), shared memory
+// frames); busy for 51 / 54 / 50 % of the time (dense, conv3, conv2 at n = 1024: 32 / 45 / 48 us in launches of their own), shared memory
 // for as much, DRAM 9 / 19 / 31 %.
 constexpr int kWgradThreads = 96 + 256;
+struct WgradShared {
+    uint64_t full[kMaxStages], empty[kMaxStages], d_full[4], d_empty[4];
+    float sum[256][2];
+    uint32_t tmem_slot;
+    int abort_flag;
+};
 template <int APL, int NB>
-__global__ void __launch_bounds__(kWgradThreads)
-x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const X3WgradParams p)
+__device__ __forceinline__ void x3_wgrad(const CUtensorMap& tmA, const CUtensorMap& tmB, const X3WgradParams& p, uint8_t* smem_raw, WgradShared& sh,
+                                         int block)
 {
-    extern __shared__ uint8_t smem_raw[];
     constexpr int NACC = NB == 64 ? 2 : 4;              // accumulators
-    __shared__ uint64_t full[kMaxStages], empty[kMaxStages], d_full[NACC], d_empty[NACC];
-    __shared__ float s_sum[256][2];
-    __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
-    volatile int* abortp = &abort_flag;
+    uint64_t *full = sh.full, *empty = sh.empty, *d_full = sh.d_full, *d_empty = sh.d_empty;
+    float (*s_sum)[2] = sh.sum;
+    volatile int* abortp = &sh.abort_flag;
     constexpr int BPL = NB == 64 ? 3 : 1;               // NB = 32: the planes are 32-column blocks of one row
     constexpr int ACC = 3 * NB, KR = kX3StageRows<NB>;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -273,9 +286,9 @@ x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int a_tx = APL * p.a_rows * 128;
     const int stage_bytes = p.n_a * a_slab + p.n_b * b_slab;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int kind = (int)blockIdx.x / p.ranges;
+    int kind = block / p.ranges;
     if (kind > p.kinds - 1) kind = p.kinds - 1;
-    const int range = (int)blockIdx.x - kind * p.ranges;
+    const int range = block - kind * p.ranges;
     const int nr = kind == p.kinds - 1 ? p.last_ranges : p.ranges;
     const int c0 = (int)((long)p.row_chunks * range / nr), c1 = (int)((long)p.row_chunks * (range + 1) / nr);
     const int gi0 = kind * p.group_mul;
@@ -286,16 +299,16 @@ x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     if (threadIdx.x == 0) {
         for (int i = 0; i < kMaxStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], biased ? 10 : 2); }
         for (int i = 0; i < NACC; ++i) { mbar_init(&d_full[i], 1); mbar_init(&d_empty[i], 4); }
-        abort_flag = 0;
+        sh.abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
     }
-    if (warp == 1) tmem_alloc(&tmem_slot, 512);
+    if (warp == 1) tmem_alloc(&sh.tmem_slot, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_d = tmem_slot;
+    const uint32_t tmem_d = sh.tmem_slot;
     pdl_wait();                                         // no trigger: the next kernel's early blocks would crowd a few SMs (1 %)
 
     if (warp == 0) {
@@ -440,6 +453,25 @@ x3_wgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     if (warp == 1) tmem_dealloc(tmem_d, 512);
 }
 
+// Two independent passes of the gradient in one launch, each on blocks of its own (one per SM).
+__global__ void __launch_bounds__(kWgradThreads)
+x3_data_weights_kernel(const __grid_constant__ CUtensorMap dA, const __grid_constant__ CUtensorMap dB, const X3TapParams d, int d_blocks,
+                       const __grid_constant__ CUtensorMap wA, const __grid_constant__ CUtensorMap wB, const X3WgradParams w)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ union { DgradShared d; WgradShared w; } sh;
+    if ((int)blockIdx.x < d_blocks) x3_dgrad(dA, dB, d, smem_raw, sh.d, blockIdx.x, d_blocks);
+    else x3_wgrad<3, 64>(wA, wB, w, smem_raw, sh.w, (int)blockIdx.x - d_blocks);
+}
+__global__ void __launch_bounds__(kWgradThreads)
+x3_weights_kernel(const __grid_constant__ CUtensorMap A2, const __grid_constant__ CUtensorMap B2, const X3WgradParams w2, int blocks2,
+                  const __grid_constant__ CUtensorMap A1, const __grid_constant__ CUtensorMap B1, const X3WgradParams w1)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ WgradShared sh;
+    if ((int)blockIdx.x < blocks2) x3_wgrad<3, 64>(A2, B2, w2, smem_raw, sh, blockIdx.x);
+    else x3_wgrad<1, 32>(A1, B1, w1, smem_raw, sh, (int)blockIdx.x - blocks2);
+}
 }  // namespace
 
 bool x3_make_map(CUtensorMap* m, const void* ptr, uint64_t cols, uint64_t rows, uint64_t planes, uint64_t pitch_elems,
@@ -470,8 +502,8 @@ bool x3_taps_plan(X3TapParams* p, int chunks, int taps, const int* shift)
         if (p->entry_rows > 256) continue;
         const int a = (3 * p->entry_rows * 128 + 1023) & ~1023;
         p->entries = taps == 1 ? 3 : 2;
-        int room = kSmemMax - 3 * 1024 - p->entries * a;
-        if (room < 2 * bb) { p->entries = 2; room = kSmemMax - 3 * 1024 - p->entries * a; }
+        int room = kSmemMax - 4 * 1024 - p->entries * a;
+        if (room < 2 * bb) { p->entries = 2; room = kSmemMax - 4 * 1024 - p->entries * a; }
         if (room < 2 * bb) continue;
         p->b_stages = room / bb > kMaxStages ? kMaxStages : room / bb;
         return true;
@@ -479,31 +511,49 @@ bool x3_taps_plan(X3TapParams* p, int chunks, int taps, const int* shift)
     return false;
 }
 
+namespace {
+int dgrad_smem(const X3TapParams& p) { return 1024 + p.entries * ((3 * p.entry_rows * 128 + 1023) & ~1023) + p.b_stages * 3 * 8192; }
+template <int APL, int NB>
+int wgrad_smem(const X3WgradParams& p)
+{
+    return 1024 + p.stages * (p.n_a * ((APL * p.a_rows * 128 + 1023) & ~1023) + p.n_b * (NB == 64 ? 3 : 1) * kX3StageRows<NB> * 128);
+}
+int wgrad_blocks(const X3WgradParams& p) { return p.ranges * (p.kinds - 1) + p.last_ranges; }
+constexpr int kRoom = kSmemMax - 3072;                   // the rest is the kernels' static share
+}  // namespace
+
 hts_status x3_dgrad_launch(const CUtensorMap& a, const CUtensorMap& b, const X3TapParams& p, cudaStream_t s)
 {
     static OncePerDevice allowed;
     HTS_CUDA(allow_shared(x3_dgrad_kernel, allowed));
-    const int smem = 1024 + p.entries * ((3 * p.entry_rows * 128 + 1023) & ~1023) + p.b_stages * 3 * 8192;
     const int tiles = p.m_tiles * p.n_tiles, sms = device_sm_count(device_slot());
-    HTS_CUDA(launch_pdl(x3_dgrad_kernel, dim3(tiles < sms ? tiles : sms), dim3(kThreads), (size_t)smem, s, a, b, p));
+    HTS_CUDA(launch_pdl(x3_dgrad_kernel, dim3(tiles < sms ? tiles : sms), dim3(kThreads), (size_t)dgrad_smem(p), s, a, b, p));
     note_launch();
     return HTS_OK;
 }
 
-template <int APL, int NB>
-hts_status x3_wgrad_launch(const CUtensorMap& a, const CUtensorMap& b, const X3WgradParams& p, cudaStream_t s)
+hts_status x3_data_weights_launch(const CUtensorMap& da, const CUtensorMap& db, const X3TapParams& d, int d_blocks, const CUtensorMap& wa,
+                                  const CUtensorMap& wb, const X3WgradParams& w, cudaStream_t s)
 {
     static OncePerDevice allowed;
-    HTS_CUDA(allow_shared(x3_wgrad_kernel<APL, NB>, allowed));
-    const int a_slab = (APL * p.a_rows * 128 + 1023) & ~1023, b_slab = (NB == 64 ? 3 : 1) * kX3StageRows<NB> * 128;
-    const int smem = 1024 + p.stages * (p.n_a * a_slab + p.n_b * b_slab);
-    if (smem > kSmemMax - 3072) return HTS_ERR_SHAPE;     // the rest is the kernel's static share
-    const int grid = p.ranges * (p.kinds - 1) + p.last_ranges;
-    HTS_CUDA(launch_pdl(x3_wgrad_kernel<APL, NB>, dim3(grid), dim3(kWgradThreads), (size_t)smem, s, a, b, p));
+    HTS_CUDA(allow_shared(x3_data_weights_kernel, allowed));
+    const int sd = dgrad_smem(d), sw = wgrad_smem<3, 64>(w), smem = sd > sw ? sd : sw;
+    if (smem > kRoom) return HTS_ERR_SHAPE;
+    HTS_CUDA(launch_pdl(x3_data_weights_kernel, dim3(d_blocks + wgrad_blocks(w)), dim3(kWgradThreads), (size_t)smem, s, da, db, d, d_blocks, wa, wb, w));
     note_launch();
     return HTS_OK;
 }
-template hts_status x3_wgrad_launch<3, 64>(const CUtensorMap&, const CUtensorMap&, const X3WgradParams&, cudaStream_t);
-template hts_status x3_wgrad_launch<1, 32>(const CUtensorMap&, const CUtensorMap&, const X3WgradParams&, cudaStream_t);
+
+hts_status x3_weights_launch(const CUtensorMap& a2, const CUtensorMap& b2, const X3WgradParams& w2, const CUtensorMap& a1, const CUtensorMap& b1,
+                             const X3WgradParams& w1, cudaStream_t s)
+{
+    static OncePerDevice allowed;
+    HTS_CUDA(allow_shared(x3_weights_kernel, allowed));
+    const int s2 = wgrad_smem<3, 64>(w2), s1 = wgrad_smem<1, 32>(w1), smem = s2 > s1 ? s2 : s1, blocks2 = wgrad_blocks(w2);
+    if (smem > kRoom) return HTS_ERR_SHAPE;
+    HTS_CUDA(launch_pdl(x3_weights_kernel, dim3(blocks2 + wgrad_blocks(w1)), dim3(kWgradThreads), (size_t)smem, s, a2, b2, w2, blocks2, a1, b1, w1));
+    note_launch();
+    return HTS_OK;
+}
 
 }  // namespace hts

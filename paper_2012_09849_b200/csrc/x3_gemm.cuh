@@ -80,8 +80,12 @@ struct X3WgradParams {
     int P3;
     int* status;
 };
-template <int APL, int NB>
-hts_status x3_wgrad_launch(const CUtensorMap& a, const CUtensorMap& b, const X3WgradParams& p, cudaStream_t s);
+// A data gradient on d_blocks blocks and, beside it, a weight gradient that does not need it.
+hts_status x3_data_weights_launch(const CUtensorMap& da, const CUtensorMap& db, const X3TapParams& d, int d_blocks, const CUtensorMap& wa,
+                                  const CUtensorMap& wb, const X3WgradParams& w, cudaStream_t s);
+// The weight gradients of the second and the first convolution side by side.
+hts_status x3_weights_launch(const CUtensorMap& a2, const CUtensorMap& b2, const X3WgradParams& w2, const CUtensorMap& a1, const CUtensorMap& b1,
+                             const X3WgradParams& w1, cudaStream_t s);
 
 // bf16 [planes][rows][cols], box 64 columns x box_rows x box_planes, 128-byte swizzle, zero fill
 bool x3_make_map(CUtensorMap* m, const void* ptr, uint64_t cols, uint64_t rows, uint64_t planes, uint64_t pitch_elems,

@@ -80,3 +80,9 @@ def test_an_infinite_return_gives_infinities_where_fp32_sums_do(positive):
             assert set(np.unique(kind(got["fc_w"]))) == {-1, 0, 1, 2}
     finally:
         pol.close()
+
+
+# the passes that share a launch: more data-gradient tiles than blocks of them, row counts on both sides of a tile, one row
+@pytest.mark.parametrize("C,H,W,n", [(4, 84, 84, 1), (4, 84, 84, 128), (4, 84, 84, 129), (4, 84, 84, 300), (16, 72, 96, 133), (4, 36, 44, 500)])
+def test_passes_that_share_a_launch(C, H, W, n):
+    test_error_stays_within_one_chain(C, H, W, n)
