@@ -76,16 +76,17 @@ __device__ __forceinline__ void acc_release(uint64_t* empty_bar, int lane)
     if (lane == 0) mbar_arrive(empty_bar);
 }
 
-// Persistent: CTA b takes tiles b, b + gridDim.x, ...  Warp 0 copies (A entries and B stages in two rings), warp 1
-// issues, then eight epilogue warps, two per lane quarter with 32 columns each.  Two accumulators of 192 columns take
-// pairs of B stages (128 of K) in turn; the epilogue adds each to the tile's sum in registers (see "Accumulation" in
-// x3_gemm.cuh).
-// The tensor core spends (128 + N) / 4 clocks (shared-memory operand fetch) or N / 2 on an instruction:
-// 96 + 64 + 48 = 208 clocks per 16 of K for 64 output columns, against 288 for six separate 128 x 64 instructions.
-// It is busy for 33 / 44 / 42 % of the time (gradients of conv3's / conv2's / conv1's output, n = 1024, 84 x 84: 34 / 49 /
-// 51 us alone) and no other unit for more than half: one thread issues, an instruction every 55 to 70 clocks at best.
-// An A entry (all planes, rows 128 + spread) is loaded once per tile and every tap reads it shifted; B is streamed.
-constexpr int kAccs = 2, kPart = 2, kThreads = 64 + 256;
+// Persistent: block b takes tiles b, b + blocks, ...  Warp 0 copies (A entries and B stages in two rings), warps 1 and 2
+// issue, then eight epilogue warps, two per lane quarter with 32 columns each.  Two accumulators of 192 columns, one for
+// each issuing thread, take pairs of B stages (128 of K) in turn; the epilogue adds each to the tile's sum in registers
+// (see "Accumulation" in x3_gemm.cuh).
+// Bound: shared memory.  An instruction fetches (128 + N) * 32 bytes of operands, 192 clocks per 16 of K (the tensor core
+// needs 192, an N of 64 at least 48: 208), and the copies write 4 to 18 KB of A and B meanwhile (30 to 140 clocks): 265 to 310
+// clocks are what the issuing threads see (n = 1024, 84 x 84).  So an A entry (all planes, rows 128 + spread) is loaded once
+// per tile and every tap reads it shifted, and the weights of an N tile stay in the ring while its M tiles pass, if they
+// fit (conv2's 96 KB: gradient of 1024 323 -> 317 us without its forward pass).  One issuing thread: 2 to 3 us more at 5 to 40
+// rows, where a tile is a chain of its own, the same at 1024.
+constexpr int kAccs = 2, kPart = 2, kThreads = 96 + 256;
 struct DgradShared {
     uint64_t a_full[kMaxEntries], a_empty[kMaxEntries], b_full[kMaxStages], b_empty[kMaxStages], d_full[kAccs], d_empty[kAccs];
     uint32_t tmem_slot;
@@ -105,10 +106,11 @@ __device__ __forceinline__ void x3_dgrad(const CUtensorMap& tmA, const CUtensorM
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles = p.m_tiles * p.n_tiles;
     const int groups = p.taps / p.tpe;                  // A entries per chunk
+    const bool stay = p.chunks * p.taps <= p.b_stages;  // the weights of an N tile stay while its M tiles pass
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < kMaxEntries; ++i) { mbar_init(&a_full[i], 1); mbar_init(&a_empty[i], 1); }
-        for (int i = 0; i < kMaxStages; ++i) { mbar_init(&b_full[i], 1); mbar_init(&b_empty[i], 1); }
+        for (int i = 0; i < kMaxEntries; ++i) { mbar_init(&a_full[i], 1); mbar_init(&a_empty[i], 2); }
+        for (int i = 0; i < kMaxStages; ++i) { mbar_init(&b_full[i], 1); mbar_init(&b_empty[i], stay ? 2 : 1); }
         for (int i = 0; i < kAccs; ++i) { mbar_init(&d_full[i], 1); mbar_init(&d_empty[i], 8); }
         sh.abort_flag = 0;
         fence_barrier_init();
@@ -126,11 +128,14 @@ __device__ __forceinline__ void x3_dgrad(const CUtensorMap& tmA, const CUtensorM
     // tile -> (M tile, N tile): M fastest, so that CTAs running together share B through L2
     if (warp == 0) {
         if (lane == 0) {
-            int ea = 0, sb = 0;
+            int ea = 0, sb = 0, held = -1;
             uint32_t pa = 1, pb = 1;                    // parity of the "empty" phase waited for
             bool alive = true;
             for (int t = first; alive && t < tiles; t += blocks) {
                 const int mt = t % p.m_tiles, nt = t / p.m_tiles;
+                const bool load = !stay || nt != held;
+                if (stay) { sb = 0; if (load && held >= 0) pb ^= 1u; }
+                held = nt;
                 for (int c = 0; alive && c < p.chunks; ++c) {
                     const int kc = c * 64;
                     for (int g = 0; alive && g < groups; ++g) {
@@ -138,48 +143,66 @@ __device__ __forceinline__ void x3_dgrad(const CUtensorMap& tmA, const CUtensorM
                         mbar_arrive_expect_tx(&a_full[ea], (uint32_t)a_bytes);
                         tma_load_3d(base + ea * a_pitch, &tmA, kc, mt * 128 + (p.tpe == 1 ? p.shift[g] : p.lo), 0, &a_full[ea]);
                         if (++ea == p.entries) { ea = 0; pa ^= 1u; }
-                        for (int j = 0; j < p.tpe; ++j) {
+                        for (int j = 0; load && j < p.tpe; ++j) {
                             if (!mbar_wait(&b_empty[sb], pb, abortp, p.status, 82)) { alive = false; break; }
                             mbar_arrive_expect_tx(&b_full[sb], BB);
                             tma_load_3d(b_base + sb * BB, &tmB, (g + j) * p.tap_cols + nt * 64, kc, 0, &b_full[sb]);
-                            if (++sb == p.b_stages) { sb = 0; pb ^= 1u; }
+                            if (++sb == p.b_stages && !stay) { sb = 0; pb ^= 1u; }
                         }
                     }
                 }
             }
         }
-    } else if (warp == 1) {
+    } else if (warp <= 2) {
         if (lane == 0) {
+            const int e = warp - 1;                     // this thread's accumulator: every other accumulation
             int ea = 0, sb = 0, it = 0, left = p.chunks * p.taps, in = 0;
             uint32_t pa = 0, pb = 0;
             bool alive = true;
             const uint64_t a_plane = (uint64_t)(plane_bytes >> 4);
-            for (int t = first; alive && t < tiles; t += blocks, left = p.chunks * p.taps)
+            int end = p.m_tiles;                        // of the N tile's tiles
+            while (stay && end <= first) end += p.m_tiles;
+            for (int t = first; alive && t < tiles; t += blocks, left = p.chunks * p.taps) {
+                if (stay) {
+                    sb = 0;
+                    if (t >= end) pb ^= 1u;
+                    while (end <= t) end += p.m_tiles;
+                }
+                const bool give = !stay || t + blocks >= end;            // the last to read them
                 for (int c = 0; alive && c < p.chunks; ++c)
                     for (int g = 0; alive && g < groups; ++g) {
-                        if (!mbar_wait(&a_full[ea], pa, abortp, p.status, 84)) { alive = false; break; }
+                        bool used = false;
                         for (int j = 0; j < p.tpe; ++j) {
-                            const int acc = it % kAccs;
-                            if (!mbar_wait(&b_full[sb], pb, abortp, p.status, 85)) { alive = false; break; }
-                            if (in == 0 && !mbar_wait(&d_empty[acc], (((uint32_t)(it / kAccs)) & 1u) ^ 1u, abortp, p.status, 83)) { alive = false; break; }
-                            tc_fence_after();
-                            const uint32_t row = p.tpe == 1 ? 0 : (uint32_t)(p.shift[j] - p.lo);
-                            const uint64_t a = smem_desc_sw128(base + ea * a_pitch + row * 128);
-                            const uint64_t b = smem_desc_mn(b_base + sb * BB, BB / 3);
+                            if ((it & 1) == e) {
+                                if (!used && !mbar_wait(&a_full[ea], pa, abortp, p.status, 84)) { alive = false; break; }
+                                used = true;
+                                if (!mbar_wait(&b_full[sb], pb, abortp, p.status, 85)) { alive = false; break; }
+                                if (in == 0 && !mbar_wait(&d_empty[e], (((uint32_t)(it / kAccs)) & 1u) ^ 1u, abortp, p.status, 83)) { alive = false; break; }
+                                tc_fence_after();
+                                const uint32_t row = p.tpe == 1 ? 0 : (uint32_t)(p.shift[j] - p.lo);
+                                const uint64_t a = smem_desc_sw128(base + ea * a_pitch + row * 128);
+                                const uint64_t b = smem_desc_mn(b_base + sb * BB, BB / 3);
 #pragma unroll
-                            for (int k = 0; k < 4; ++k)          // 32 bytes along A's rows, 16 rows of B
-                                mma_x3<3, 64>(tmem_d + acc * 192, a + 2 * k, a_plane, b + 128 * k, 0, 1, (in | k) == 0);
-                            mma_commit(&b_empty[sb]);
+                                for (int k = 0; k < 4; ++k)      // 32 bytes along A's rows, 16 rows of B
+                                    mma_x3<3, 64>(tmem_d + e * 192, a + 2 * k, a_plane, b + 128 * k, 0, 1, (in | k) == 0);
+                                if (give) mma_commit(&b_empty[sb]);
+                            } else if (stay && give)
+                                mbar_arrive(&b_empty[sb]);
                             --left;
-                            if (++in == kPart || left == 0) { mma_commit(&d_full[acc]); ++it; in = 0; }
-                            if (++sb == p.b_stages) { sb = 0; pb ^= 1u; }
+                            if (++in == kPart || left == 0) {
+                                if ((it & 1) == e) mma_commit(&d_full[e]);
+                                ++it; in = 0;
+                            }
+                            if (++sb == p.b_stages && !stay) { sb = 0; pb ^= 1u; }
                         }
-                        mma_commit(&a_empty[ea]);
+                        if (used) mma_commit(&a_empty[ea]);
+                        else mbar_arrive(&a_empty[ea]);
                         if (++ea == p.entries) { ea = 0; pa ^= 1u; }
                     }
+            }
         }
-    } else if (warp < kThreads / 32) {
-        const int j = (warp - 2) >> 2, q = warp & 3;    // half of the columns; TMEM lane quarter of this warp
+    } else {
+        const int j = (warp - 3) >> 2, q = warp & 3;    // half of the columns; TMEM lane quarter of this warp
         const int row = q * 32 + lane, parts = (p.chunks * p.taps + kPart - 1) / kPart;
         int it = 0;
         bool alive = true;
