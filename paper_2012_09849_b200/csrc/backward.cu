@@ -168,7 +168,7 @@ head_backward_kernel(const float* __restrict__ logits, const float* __restrict__
     pdl_trigger();
     __syncthreads();
     const float inv_n = 1.0f / (float)n;
-    for (int i = blockIdx.x * 8 + wib; i < n; i += gridDim.x * 8) {
+    for (int i = blockIdx.x + wib * gridDim.x; i < n; i += gridDim.x * 8) {      // few rows: a block each
         const int a = actions[i];
         const bool bad = (unsigned)a >= (unsigned)A;     // not used as an index: the row contributes nothing
         if (bad && lane == 0 && status) atomicCAS(status, 0, kStatusBadAction);
@@ -285,34 +285,44 @@ struct ReduceParams {
     size_t g1, g2, g3;                                   // floats between group indices
     const float* fc;                                     // [512][pixel * 64 + c]
     int C, Cp, A, P3;
+    const float *dhead, *h;                              // few samples: the heads' sums are taken here (n > 0), else from `head`
+    const bf16* dh;
+    size_t dh_plane;
+    int n;
     hts_grads out;
 };
-__device__ __forceinline__ float sum_ranges(const float* p, int ranges, size_t stride)
+// One kernel less while there are few samples.  Gradient without its forward pass, us, here / in a kernel of their own: 5 samples
+// 52.4 / 55.1, 40 60.9 / 64.6, 64 66.1 / 69.3, 80 71.3 / 72.6, 100 79.7 / 78.5, 160 111 / 100.
+constexpr int kHeadsInReduce = 80;
+constexpr int kTurnFloats = 4096;                        // eight blocks on an SM
+// Sixteen terms in flight.
+template <class Term>
+__device__ __forceinline__ float sum_terms(int lo, int hi, Term term)
 {
     float acc = 0.f;
-    int r = 0;
-    for (; r + 16 <= ranges; r += 16) {
+    for (int r = lo; r < hi; r += 16) {
         float v[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = p[(size_t)(r + i) * stride];
+        for (int i = 0; i < 16; ++i) v[i] = r + i < hi ? term(r + i) : 0.f;
 #pragma unroll
         for (int i = 0; i < 16; ++i) acc += v[i];
     }
-    for (; r < ranges; ++r) acc += p[(size_t)r * stride];
     return acc;
 }
 // Blocks 0..511 turn one row of the dense gradient each into the caller's column order (c * P3 + pixel): written by the
-// contraction itself, 4-byte pieces P3 apart cost it 20 us.  The others sum.
+// contraction itself, 4-byte pieces P3 apart cost it 20 us.  The others sum, four threads of a block (64 apart) to a sum: a quarter
+// of the ranges each, then the quarters in order: gradient of 512 frames of 72 x 96 x 16 260 -> 244 us, of 40 68 -> 64, of 80 of 84 x 84 x 4
+// 72.3 -> 71.3 (one thread to a sum waited for up to 148 ranges, sixteen at a time).
 __global__ void __launch_bounds__(256) reduce_kernel(const ReduceParams p)
 {
-    __shared__ float s_row[kPackFloats];
+    __shared__ float s_row[kTurnFloats];
     pdl_wait();
     pdl_trigger();
     if (blockIdx.x < 512) {
         const int F = 64 * p.P3;
         const float* src = p.fc + (size_t)blockIdx.x * F;
         float* dst = p.out.fc_w + (size_t)blockIdx.x * F;
-        const int pstep = kPackFloats / 65;              // pixels per pass, rows of 65 against bank conflicts
+        const int pstep = kTurnFloats / 65;              // pixels per pass, rows of 65 against bank conflicts
         for (int q0 = 0; q0 < p.P3; q0 += pstep) {
             const int nq = p.P3 - q0 < pstep ? p.P3 - q0 : pstep;
             for (int i = threadIdx.x; i < nq * 64; i += 256) s_row[(i >> 6) * 65 + (i & 63)] = src[(size_t)q0 * 64 + i];
@@ -325,46 +335,56 @@ __global__ void __launch_bounds__(256) reduce_kernel(const ReduceParams p)
         }
         return;
     }
-    int i = (blockIdx.x - 512) * 256 + threadIdx.x;
+    int i = (blockIdx.x - 512) * 64 + (threadIdx.x & 63);
     const int n3 = 5 * 8192, n2 = 4 * 8192, n1 = p.Cp / 2 * 4096, nh = (p.A + 2) * 513;
+    const float* src = nullptr;                          // what this thread's sum adds up, and where it goes
+    float* dst = nullptr;
+    int ranges = 0, ho = -1, hk = 0;
+    size_t stride = 0;
+    float scale = 1.f;
     if (i < n3) {                                        // [tap pair][tap of the pair, c][o]
         const int gi = i >> 13, e = i & 8191, m = e >> 6, o = e & 63, b = m >> 6, c = m & 63;
         const int tap = gi < 4 ? 2 * gi + b : 7 + b;
-        if (gi == 4 && b == 0) return;                   // tap 7 belongs to pair 3
-        p.out.conv3_w[(o * 64 + c) * 9 + tap] = sum_ranges(p.c3 + gi * p.g3 + e, gi == 4 ? p.r3_last : p.r3, 8192);
-        return;
-    }
-    i -= n3;
-    if (i < n2) {                                        // [tap][(uy, ux, c)][o]
+        src = p.c3 + gi * p.g3 + e; ranges = gi == 4 ? p.r3_last : p.r3; stride = 8192;
+        if (gi < 4 || b != 0) dst = p.out.conv3_w + (o * 64 + c) * 9 + tap;      // tap 7 belongs to pair 3
+    } else if ((i -= n3) < n2) {                         // [tap][(uy, ux, c)][o]
         const int tap = i >> 13, e = i & 8191, cp = e >> 6, o = e & 63;
         const int dy = tap >> 1, dx = tap & 1, uy = cp >> 6, ux = (cp >> 5) & 1, c = cp & 31;
-        p.out.conv2_w[((o * 32 + c) * 4 + 2 * dy + uy) * 4 + 2 * dx + ux] = sum_ranges(p.c2 + tap * p.g2 + e, p.r2, 8192);
-        return;
-    }
-    i -= n2;
-    if (i < n1) {                                        // [64 columns of the cell, tap pair][tap, column][o]
+        src = p.c2 + tap * p.g2 + e; ranges = p.r2; stride = 8192;
+        dst = p.out.conv2_w + ((o * 32 + c) * 4 + 2 * dy + uy) * 4 + 2 * dx + ux;
+    } else if ((i -= n2) < n1) {                         // [64 columns of the cell, tap pair][tap, column][o]
         const int gi = i >> 12, e = i & 4095, m = e >> 5, o = e & 31;
         const int tap = (gi & 1) * 2 + (m >> 6), k = (gi >> 1) * 64 + (m & 63);
         const int c = k >> 4, uy = (k >> 2) & 3, ux = k & 3, dy = tap >> 1, dx = tap & 1;
-        if (c < p.C)
-            p.out.conv1_w[((o * p.C + c) * 8 + 4 * dy + uy) * 8 + 4 * dx + ux] =
-                sum_ranges(p.c1 + gi * p.g1 + e, p.r1, 4096) * (1.0f / 255.0f);
-        return;
+        src = p.c1 + gi * p.g1 + e; ranges = p.r1; stride = 4096; scale = 1.0f / 255.0f;
+        if (c < p.C) dst = p.out.conv1_w + ((o * p.C + c) * 8 + 4 * dy + uy) * 8 + 4 * dx + ux;
+    } else if ((i -= n1) < nh) {
+        ho = i / 513; hk = i - ho * 513;
+        src = p.head + i; ranges = p.n > 0 ? p.n : p.rh; stride = (size_t)nh;
+        if (ho == p.A + 1) dst = hk < 512 ? p.out.fc_b + hk : nullptr;
+        else if (hk == 512) dst = ho < p.A ? p.out.pi_b + ho : p.out.v_b;
+        else dst = ho < p.A ? p.out.pi_w + ho * 512 + hk : p.out.v_w + hk;
+    } else if ((i -= nh) < 64) {
+        src = p.b3 + i; ranges = p.r3; stride = 64; dst = p.out.conv3_b + i;
+    } else if (i < 128) {
+        src = p.b2 + i - 64; ranges = p.r2; stride = 64; dst = p.out.conv2_b + i - 64;
+    } else if (i < 160) {
+        src = p.b1 + i - 128; ranges = p.r1; stride = 32; dst = p.out.conv1_b + i - 128;
     }
-    i -= n1;
-    if (i < nh) {
-        const int o = i / 513, k = i - o * 513;
-        if (o == p.A + 1 && k == 512) return;
-        const float v = sum_ranges(p.head + i, p.rh, (size_t)nh);
-        if (o == p.A + 1) p.out.fc_b[k] = v;
-        else if (k == 512) *(o < p.A ? p.out.pi_b + o : p.out.v_b) = v;
-        else *(o < p.A ? p.out.pi_w + o * 512 + k : p.out.v_w + k) = v;
-        return;
+    const int part = threadIdx.x >> 6, lo = ranges * part / 4, hi = ranges * (part + 1) / 4;
+    float acc = 0.f;
+    if (dst) {
+        if (ho < 0 || p.n == 0) acc = sum_terms(lo, hi, [&](int r) { return src[(size_t)r * stride]; });
+        else if (ho == p.A + 1) acc = sum_terms(lo, hi, [&](int r) {
+            const bf16* g = p.dh + (size_t)r * 512 + hk;
+            return x3_sum(__bfloat162float(g[0]), __bfloat162float(g[p.dh_plane]) + __bfloat162float(g[2 * p.dh_plane]));
+        });
+        else if (hk == 512) acc = sum_terms(lo, hi, [&](int r) { return p.dhead[(size_t)r * (p.A + 1) + ho]; });
+        else acc = sum_terms(lo, hi, [&](int r) { return p.dhead[(size_t)r * (p.A + 1) + ho] * p.h[(size_t)r * 512 + hk]; });
     }
-    i -= nh;
-    if (i < 64) p.out.conv3_b[i] = sum_ranges(p.b3 + i, p.r3, 64);
-    else if (i < 128) p.out.conv2_b[i - 64] = sum_ranges(p.b2 + i - 64, p.r2, 64);
-    else if (i < 160) p.out.conv1_b[i - 128] = sum_ranges(p.b1 + i - 128, p.r1, 32);
+    s_row[threadIdx.x] = acc;
+    __syncthreads();
+    if (dst && threadIdx.x < 64) *dst = ((s_row[threadIdx.x] + s_row[64 + threadIdx.x]) + (s_row[128 + threadIdx.x] + s_row[192 + threadIdx.x])) * scale;
 }
 
 inline unsigned nblk(size_t total, int th) { return (unsigned)((total + th - 1) / th); }
@@ -623,9 +643,11 @@ hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, 
     int per_range = (n + (int)kHeadRanges - 1) / (int)kHeadRanges;
     if (per_range < 16) per_range = 16;
     const int rh = (n + per_range - 1) / per_range;
-    HTS_CUDA(launch_pdl(head_wgrad_kernel, dim3(8, rh, nblk(g.A + 2, kHeadTile)), dim3(256), 0, s, t->dhead, ws.h, t->dh, ph, n, g.A, per_range,
-                        t->headp));
-    note_launch();
+    if (n > kHeadsInReduce) {
+        HTS_CUDA(launch_pdl(head_wgrad_kernel, dim3(8, rh, nblk(g.A + 2, kHeadTile)), dim3(256), 0, s, t->dhead, ws.h, t->dh, ph, n, g.A, per_range,
+                            t->headp));
+        note_launch();
+    }
 
     // ---- data and weight gradients: ranges of at least one stage of rows
     auto cut = [&](X3WgradParams p, size_t rows, int ranges, int last) {
@@ -670,9 +692,10 @@ hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, 
     r.c1 = t->part1; r.c2 = t->part2; r.c3 = t->part3; r.b1 = t->bias1; r.b2 = t->bias2; r.b3 = t->bias3; r.head = t->headp;
     r.r1 = q1.ranges; r.r2 = q2.ranges; r.r3 = q3.ranges; r.r3_last = q3.last_ranges; r.rh = rh;
     r.g1 = q1.group_stride; r.g2 = q2.group_stride; r.g3 = q3.group_stride;
+    r.dhead = t->dhead; r.h = ws.h; r.dh = t->dh; r.dh_plane = ph; r.n = n > kHeadsInReduce ? 0 : n;
     r.fc = t->partf; r.P3 = t->P3; r.C = g.C; r.Cp = t->Cp; r.A = g.A; r.out = out;
     const size_t total = (size_t)9 * 8192 + (size_t)t->Cp / 2 * 4096 + (size_t)(g.A + 2) * 513 + 160;
-    HTS_CUDA(launch_pdl(reduce_kernel, dim3(512 + nblk(total, 256)), dim3(256), 0, s, r));
+    HTS_CUDA(launch_pdl(reduce_kernel, dim3(512 + nblk(total, 64)), dim3(256), 0, s, r));
     note_launch();
     return HTS_OK;
 }
