@@ -1,14 +1,15 @@
 // fp32 dense layer of the actor step for batches that fill the device.
 //
 // Lane l of a warp runs chain l of TE rows x TO outputs, so both operands are contiguous across the lanes; one transposing
-// reduction closes the tree (at each level a lane keeps half of its values and gets its partner's share of them).  Stages of 128
-// columns arrive as boxes of 16 rows, asked for by a warp of their own (all waits are bounded); the next 32 columns are loaded
-// while these are multiplied.  Bound: loads from shared memory, a clock for each of the 16 words that 64 multiply-adds take, and as
-// much time in the fp32 pipes (with the moves that put a weight into both lanes); 61 % of the one and 60 % of the other are reached.
-// 3136 features, us at 40 / 80 / 160 / 256 / 512 / 1024 rows: 12.3 / 16.7 / 22.7 / 29.9 / 48.5 / 92; copied by the multiplying warps,
-// 32 x 16 outputs per block of eight of them: 16 / 22 / 36 / 36 / 67 / 114.  16 x 8 per warp reads less (24 words for 128) but leaves
-// two warps per scheduler: 29 / 29 / 29 / 29 / 56 / 108.  Pairs of chains in 8-byte loads, without the moves: 99 to 102 at 1024.  A copy
-// per row instead of a box: 163 (70 clocks each).
+// reduction closes the tree (at each level a lane keeps half of its values and gets its partner's share of them).  Stages of 256
+// columns arrive as boxes of 16 rows x 128, asked for by a warp of their own (all waits are bounded).  A stage's eight steps are one
+// straight run of instructions, so that a step's loads are under way during the products before it; what remains is the first
+// step of each stage, and loads from shared memory, a clock for each of the 16 words that 64 multiply-adds take, beside as much time
+// in the fp32 pipes.  Whole fp32 step of 84 x 84 x 4, us at 40 / 80 / 160 / 256 / 512 / 1024 rows: 42.3 / 60.3 / 91.3 / 124 / 216 / 406; with
+// stages of 128 columns and the next step's loads written out before a step's products 45.3 / 62.6 / 94.3 / 129 / 223 / 421 (straight
+// runs of 128: 44.6 / 62.3 / 93.6 / 128 / 221 / 417; the next stage's first loads before a stage's last products: 44.2 / 61.0 / 92.5 /
+// 126 / 218 / 412; 8 x 4 per warp and eight warps: 43.3 / 62.0 / 95.3 / 129 / 225 / 426; 16 x 8, two warps per scheduler: 52 / 66 / 101 /
+// 128 / 230 / 423).  A copy per row instead of a box: 70 clocks each.
 #include "common.cuh"
 #include "f32x2.cuh"
 #include "fc_f32.cuh"
@@ -18,14 +19,14 @@
 namespace hts {
 namespace {
 
-template <int TE, int TO, int WE, int WO, int NST, int PER_SM>
+template <int TE, int TO, int WE, int WO, int SUB, int NST, int PER_SM>
 __global__ void __launch_bounds__(32 * (WE * WO + 1), PER_SM)
 fc_lanes_kernel(const FcParams p, const __grid_constant__ CUtensorMap mx, const __grid_constant__ CUtensorMap mw)
 {
-    constexpr int COLS = kFcBoxCols, BOX = kFcBoxRows, NC = WE * WO, RX = TE * WE, RW = TO * WO, STAGE = (RX + RW) * COLS, NV = TE * TO;
+    constexpr int COLS = kFcBoxCols, BOX = kFcBoxRows, NC = WE * WO, RX = TE * WE, RW = TO * WO, BOXES = (RX + RW) * COLS, STAGE = SUB * BOXES, NV = TE * TO;
     static_assert(RX % BOX == 0 && RW % BOX == 0, "whole boxes");
     extern __shared__ float s_dyn[];
-    float* s_ring = s_dyn + (-tc::smem_u32(s_dyn) & 127) / 4;                    // [NST][RX + RW][COLS]
+    float* s_ring = s_dyn + (-tc::smem_u32(s_dyn) & 127) / 4;                    // [NST][SUB][RX + RW][COLS]
     __shared__ uint64_t full[NST], freed[NST];
     __shared__ int abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -35,7 +36,7 @@ fc_lanes_kernel(const FcParams p, const __grid_constant__ CUtensorMap mx, const 
         tc::fence_barrier_init();
     }
     __syncthreads();
-    const int stages = (p.F + COLS - 1) / COLS, e_base = blockIdx.y * RX, o_base = blockIdx.x * RW;
+    const int stages = (p.F + SUB * COLS - 1) / (SUB * COLS), e_base = blockIdx.y * RX, o_base = blockIdx.x * RW;
     if (warp == NC) {
         pdl_wait();
         int st = 0;
@@ -45,10 +46,11 @@ fc_lanes_kernel(const FcParams p, const __grid_constant__ CUtensorMap mx, const 
             if (st >= NST && !tc::mbar_wait_warp(freed + slot, (st / NST - 1) & 1, &abort_flag, p.status, 50)) break;
             if (lane == 0) tc::mbar_arrive_expect_tx(full + slot, STAGE * 4);
             __syncwarp();
-            if (lane < (RX + RW) / BOX) {
-                const int r = lane * BOX;
-                if (r < RX) tc::tma_load_2d(s_ring + slot * STAGE + r * COLS, &mx, st * COLS, p.row0 + e_base + r, full + slot);
-                else tc::tma_load_2d(s_ring + slot * STAGE + r * COLS, &mw, st * COLS, o_base + r - RX, full + slot);
+            if (lane < SUB * (RX + RW) / BOX) {         // columns past the last are zeros
+                const int r = lane / SUB * BOX, sub = lane % SUB, c = (st * SUB + sub) * COLS;
+                float* dst = s_ring + slot * STAGE + sub * BOXES + r * COLS;
+                if (r < RX) tc::tma_load_2d(dst, &mx, c, p.row0 + e_base + r, full + slot);
+                else tc::tma_load_2d(dst, &mw, c, o_base + r - RX, full + slot);
             }
         }
         if (st < stages)                                 // given up: the copies in flight end before the block does
@@ -67,16 +69,13 @@ fc_lanes_kernel(const FcParams p, const __grid_constant__ CUtensorMap mx, const 
         if (!tc::mbar_wait_warp(full + slot, (st / NST) & 1, &abort_flag, p.status, 52)) break;
         const float* xr = s_ring + slot * STAGE + we * TE * COLS + lane;
         const float* wr = s_ring + slot * STAGE + (RX + wo * TO) * COLS + lane;
-        auto load = [&](int c, float (&xv)[TE], float (&wv)[TO]) {
+        auto step = [&](int c) {
+            f32x2 xx[TE / 2];
+            float wv[TO];
 #pragma unroll
             for (int j = 0; j < TO; ++j) wv[j] = wr[j * COLS + c];
 #pragma unroll
-            for (int i = 0; i < TE; ++i) xv[i] = xr[i * COLS + c];
-        };
-        auto step = [&](const float (&xv)[TE], const float (&wv)[TO]) {
-            f32x2 xx[TE / 2];
-#pragma unroll
-            for (int i = 0; i < TE / 2; ++i) xx[i] = pair(xv[2 * i], xv[2 * i + 1]);
+            for (int i = 0; i < TE / 2; ++i) xx[i] = pair(xr[2 * i * COLS + c], xr[(2 * i + 1) * COLS + c]);
 #pragma unroll
             for (int j = 0; j < TO; ++j) {
                 const f32x2 ww = both(wv[j]);
@@ -87,16 +86,13 @@ fc_lanes_kernel(const FcParams p, const __grid_constant__ CUtensorMap mx, const 
                 }
             }
         };
-        const int cols = min(COLS, p.F - st * COLS);     // a multiple of 64
-        float xv[2][TE], wv[2][TO];
-        load(0, xv[0], wv[0]);
+        const int cols = p.F - st * SUB * COLS;          // a multiple of 64
+        if (cols >= SUB * COLS) {
+#pragma unroll
+            for (int c = 0; c < SUB * COLS; c += 32) step(c / COLS * BOXES + c % COLS);
+        } else
 #pragma unroll 1
-        for (int c = 0; c < cols; c += 64) {
-            load(c + 32, xv[1], wv[1]);
-            step(xv[0], wv[0]);
-            load(c + 64 < cols ? c + 64 : c, xv[0], wv[0]);
-            step(xv[1], wv[1]);
-        }
+            for (int c = 0; c < cols; c += 32) step(c / COLS * BOXES + c % COLS);
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(freed + slot);
     }
@@ -128,12 +124,12 @@ fc_lanes_kernel(const FcParams p, const __grid_constant__ CUtensorMap mx, const 
         }
 }
 
-template <int TE, int TO, int WE, int WO, int NST, int PER_SM>
+template <int TE, int TO, int WE, int WO, int SUB, int NST, int PER_SM>
 hts_status launch_lanes(const FcParams& p, const FcMaps& m, cudaStream_t s)
 {
-    constexpr int smem = NST * (TE * WE + TO * WO) * kFcBoxCols * 4 + 128;
+    constexpr int smem = NST * SUB * (TE * WE + TO * WO) * kFcBoxCols * 4 + 128;
     static_assert(smem <= 227 * 1024 / PER_SM - 1024 - 128, "shared memory");
-    auto kernel = fc_lanes_kernel<TE, TO, WE, WO, NST, PER_SM>;
+    auto kernel = fc_lanes_kernel<TE, TO, WE, WO, SUB, NST, PER_SM>;
     static OncePerDevice allowed;
     HTS_CUDA(allow_shared(kernel, allowed));
     HTS_CUDA(launch_pdl(kernel, dim3(512 / (TO * WO), (unsigned)((p.n + TE * WE - 1) / (TE * WE))), dim3(32 * (WE * WO + 1)), (size_t)smem, s, p, m.x, m.w));
@@ -151,7 +147,7 @@ bool make_fc_maps(const float* x, const float* w, int F, size_t frames, FcMaps* 
 
 hts_status launch_fc_lanes(const FcParams& p, const FcMaps& m, cudaStream_t s)
 {
-    return m.ok ? launch_lanes<8, 8, 2, 2, 2, 3>(p, m, s) : HTS_ERR_UNSUPPORTED;
+    return m.ok ? launch_lanes<8, 8, 2, 2, 2, 2, 3>(p, m, s) : HTS_ERR_UNSUPPORTED;
 }
 
 }  // namespace hts
