@@ -239,12 +239,12 @@ conv_strip_kernel(const ConvParams p, const StripPlan t, const __grid_constant__
         if (!tc::mbar_wait_warp(full + slot, (st / NST) & 1, &abort_flag, p.status, 42)) break;    // the barriers below are met all the same
         const float4* in = s4 + slot * STAGE;
         const float* w = reinterpret_cast<const float*>(in + STAGE - WCH) + o_t;
-#pragma unroll 1
+#pragma unroll (U8 ? 1 : CK)
         for (int cc = 0; cc < CK; ++cc) {
             float x[(RW + 3) / 4 * 4];
             if constexpr (U8) {
                 const uint32_t* x4 = reinterpret_cast<const uint32_t*>(in + cc * XCH) + x_at;
-#pragma unroll 1
+#pragma unroll 4
                 for (int u = 0; u < KS; ++u) {
                     strip_load<RW>(x, x4);
                     strip_row<KS, S, PX, OT, OC>(acc, x, w);
