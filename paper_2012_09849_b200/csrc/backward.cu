@@ -23,24 +23,36 @@ typedef __nv_bfloat16 bf16;
 // ---- frames as the first convolution's operand -----------------------------------------------------------------
 // uint8 [n,C,H,W] -> bf16 [n * (H/4)(W/4)][16 Cp], column c*16 + uy*4 + ux = x[c][4Y+uy][4X+ux] (a byte is exact);
 // Cp = C rounded up to a multiple of 4, the added channels are zero.
-__global__ void __launch_bounds__(256)
-frames_kernel(const uint8_t* __restrict__ obs, int C, int Cp, int H, int W, size_t items, bool words, bf16* __restrict__ x0)
+// Bound by memory (87 MB for 1024 frames of 84 x 84 x 4, 18 us), where conv1 is bound by its multiply-adds.  Where conv1 has blocks
+// of 32 strips for more than three to an SM, this runs beside its last ones: it begins when they have all begun (its inputs are
+// ready then) and waits for them with its last block only, so that its own end means theirs.  Gradient without the forward pass, us,
+// before conv1 / beside it: 160 of 84 x 84 x 4 99.1 / 96.5, 1024 316 / 312, 512 of 72 x 96 x 16 238 / 221; where all of conv1's blocks are on
+// the device at once the two crowd each other: 80 of 84 x 84 x 4 71.5 / 83.5, 40 of 72 x 96 x 16 64 / 105.
+struct FramesParams {
+    const uint8_t* obs;
+    int C, Cp, H, W;
+    size_t items;                       // (position, channel), channel fastest
+    bool words;                         // frames 4-byte aligned
+    bf16* x0;
+    bool beside;                        // launched behind conv1
+};
+__global__ void __launch_bounds__(256) frames_kernel(const FramesParams p)
 {
-    pdl_wait();                                         // no trigger: early blocks of the forward would settle unevenly (5 us of 383)
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;       // (position, channel), channel fastest
-    if (idx >= items) return;
-    const int c = (int)(idx % Cp);
-    const size_t pos = idx / Cp;
-    const int W0 = W / 4, G0 = W0 * (H / 4);
+    if (!p.beside || blockIdx.x == gridDim.x - 1) pdl_wait();
+    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= p.items) return;
+    const int c = (int)(idx % p.Cp);
+    const size_t pos = idx / p.Cp;
+    const int W0 = p.W / 4, G0 = W0 * (p.H / 4);
     const size_t e = pos / G0;
     const int cell = (int)(pos - e * G0), Y = cell / W0, X = cell - Y * W0;
     uint32_t out[8];
 #pragma unroll
     for (int uy = 0; uy < 4; ++uy) {
         uint32_t w = 0;
-        if (c < C) {
-            const uint8_t* src = obs + ((e * C + c) * H + 4 * Y + uy) * W + 4 * X;
-            if (words) w = *reinterpret_cast<const uint32_t*>(src);
+        if (c < p.C) {
+            const uint8_t* src = p.obs + ((e * p.C + c) * p.H + 4 * Y + uy) * p.W + 4 * X;
+            if (p.words) w = *reinterpret_cast<const uint32_t*>(src);
             else w = src[0] | (uint32_t)src[1] << 8 | (uint32_t)src[2] << 16 | (uint32_t)src[3] << 24;
         }
 #pragma unroll
@@ -49,7 +61,7 @@ frames_kernel(const uint8_t* __restrict__ obs, int C, int Cp, int H, int W, size
             out[2 * uy + h] = (__float_as_uint(lo) >> 16) | (__float_as_uint(hi) & 0xffff0000u);
         }
     }
-    uint4* dst = reinterpret_cast<uint4*>(x0 + idx * 16);
+    uint4* dst = reinterpret_cast<uint4*>(p.x0 + idx * 16);
     dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
     dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
 }
@@ -605,6 +617,14 @@ bool x3_map_batch(X3State* t, int n)
     return ok;
 }
 
+hts_status launch_frames(const void* arg, cudaStream_t s)
+{
+    const FramesParams& p = *static_cast<const FramesParams*>(arg);
+    HTS_CUDA(launch_pdl(frames_kernel, dim3(nblk(p.items, 256)), dim3(256), 0, s, p));
+    note_launch();
+    return HTS_OK;
+}
+
 inline int tiles_of(size_t rows) { return (int)((rows + 127) / 128); }
 
 }  // namespace
@@ -625,11 +645,11 @@ hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, 
     const size_t nb = (size_t)t->max_batch, N = (size_t)n;
     const size_t p1 = nb * t->P1s * 128, p2 = nb * t->P2 * 64, p3 = nb * g.F, ph = nb * 512, pz2 = nb * t->P1s * 64;
 
-    const size_t items = N * t->G0 * t->Cp;
-    HTS_CUDA(launch_pdl(frames_kernel, dim3(nblk(items, 256)), dim3(256), 0, s, obs, g.C, t->Cp, g.H, g.W, items, ((uintptr_t)obs & 3) == 0,
-                        t->x0));
-    note_launch();
-    const RefPlanes planes{t->a1, t->a2, t->a3, p1, p2, p3};
+    const FramesParams fp{obs, g.C, t->Cp, g.H, g.W, N * t->G0 * t->Cp, ((uintptr_t)obs & 3) == 0, t->x0,
+                          N * g.H1 * ((g.W1 + 3) / 4) > (size_t)96 * t->sms};
+    const RefPlanes planes{t->a1, t->a2, t->a3, p1, p2, p3, fp.beside ? launch_frames : nullptr, &fp};
+    if (!fp.beside) st = launch_frames(&fp, s);
+    if (st != HTS_OK) return st;
     st = ref_forward(g, w, ws, obs, Indexing{}, t->status, n, prof, s, &planes);
     if (st != HTS_OK) return st;
     st = launch_heads(ws.h, 1, 0, nullptr, w.whead, w.bhead, g.A, nullptr, nullptr, 0, 0, n, Indexing{}, t->status, nullptr, t->logp, t->val,

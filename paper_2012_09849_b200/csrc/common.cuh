@@ -149,6 +149,9 @@ inline RowLayout rows_a2(const Geometry& g) { return rows_strips(g.H2, g.W2, 1);
 struct RefPlanes {             // the hidden convolution outputs once more, as three bf16 planes of pixel-major rows
     __nv_bfloat16 *a1, *a2, *a3;
     size_t p1, p2, p3;         // elements between planes
+    // Launched behind conv1 if not null: a kernel that needs nothing of it and whose end means conv1's (frames_kernel).
+    hts_status (*beside_conv1)(const void* arg, cudaStream_t s);
+    const void* arg;
 };
 
 // The maps of a workspace for `frames` frames; nullptr if there is no memory or driver for them (its kernels then take other forms).

@@ -188,6 +188,7 @@ conv_strip_kernel(const ConvParams p, const StripPlan t, const __grid_constant__
     __syncthreads();
     if (warp == NC) {
         pdl_wait();
+        if (p.early) pdl_trigger();
         const int frames = rr1 / p.Ho - e0 + 1;
         auto rows_of = [&](int f, int* lo) {
             *lo = f == 0 ? rr0 - e0 * p.Ho : 0;

@@ -23,6 +23,7 @@ struct ConvParams {
     size_t plane;
     int W_rows, P_rows;                 // its grid; 2 x 2 pixels per row when s2d
     bool s2d;
+    bool early;                         // the next kernel is beside_conv1: its blocks may settle while the last ones of this run
 };
 
 #ifdef __CUDACC__

@@ -516,10 +516,14 @@ hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspac
     prof.begin(K_CONV1, s);
     ConvParams c1 = layer(obs, rows_dense(g.H, g.W), w.w1, w.w1k, w.b1, ws.a1, ws.l1, g.C, g.H, g.W, 32, 8, 4, g.H1, g.W1);
     c1.in_scale = 1.0f / 255.0f; c1.slots = ix.slots; c1.pool = ix.pool;
-    if (planes) { c1.planes = planes->a1; c1.plane = planes->p1; c1.s2d = true; c1.W_rows = (g.W1 + 1) / 2; c1.P_rows = (g.H1 + 1) / 2 * c1.W_rows; }
+    if (planes) { c1.planes = planes->a1; c1.plane = planes->p1; c1.s2d = true; c1.W_rows = (g.W1 + 1) / 2; c1.P_rows = (g.H1 + 1) / 2 * c1.W_rows; c1.early = planes->beside_conv1; }
     st = launch_conv<uint8_t>(c1, nullptr, s);
     if (st != HTS_OK) return st;
     prof.end(K_CONV1, s);
+    if (planes && planes->beside_conv1) {
+        st = planes->beside_conv1(planes->arg, s);
+        if (st != HTS_OK) return st;
+    }
     prof.begin(K_CONV2, s);
     ConvParams c2 = layer(ws.a1, ws.l1, w.w2, w.w2k, w.b2, ws.a2, ws.l2, 32, g.H1, g.W1, 64, 4, 2, g.H2, g.W2);
     if (planes) { c2.planes = planes->a2; c2.plane = planes->p2; c2.P_rows = g.H2 * g.W2; }
