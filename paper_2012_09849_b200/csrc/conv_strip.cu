@@ -351,6 +351,7 @@ template <int PX, int OT, int LG, int CK, int NST, int PER_SM>
 using Form3 = StripForm<float, 3, 1, PX, OT, LG, 1, CK, NST, PER_SM>;
 typedef Form1<2, 4, 8, 2, 2, 2, 4> Few1;
 typedef Form1<4, 8, 8, 4, 2, 2, 3> Many1;
+typedef Form1<5, 8, 8, 4, 2, 2, 3> Five1;
 typedef Form1<4, 8, 8, 4, 1, 2, 3> Odd1;                // an odd number of channels
 typedef Form2<4, 2, 4, 4, 2, 4> Few2;
 typedef Form2<9, 2, 4, 4, 2, 4> Some2n;                 // rows up to 9 pixels; else of strips of 10
@@ -373,6 +374,7 @@ bool make_strip_maps(const Geometry& g, const RefWorkspace& ws, size_t frames, S
 // A form takes a time that steps with the blocks of the fullest SM.  84 x 84 x 4, us at 1, 2, 3, 4 ... blocks, and what that is
 // about (first + each more):
 //   first layer    2 pixels x 4 channels 5.9, 7.7, 10.0, .. 17.0 (6): 5.6 + 2.2      4 x 8  9.1, 15.0, .. 27 (4), 38.8 (6), 134 (22): 9.1 + 6
+//     5 x 8: 11.5 + 8.2, where that saves a round (step of 50 frames of 72 x 96 x 16 73 -> 63 us, of 100 116 -> 106; 80: 85 / 98)
 //   second   4 x 2  7.4, 10.9, 14.9: 7.4 + 3.7     a row x 2  11.3, 18.0, 25.5, 32.9: 11.3 + 7.0     a row x 4  16.7, 29.5, .. 56 (4), .. 107 (8): 16.7 + 12.5
 //   third    4 x 2  8.6, 11.8, .. 21.2 (4): 8.6 + 4.2     a row x 2  10.2, 15.6, .. 27.2 (4), 44.7 (7), 80 (13): 10.1 + 5.8
 // (the tiles of policy_ref.cu: 12 to 16 at 16 frames, 26 / 31 / 22 at 80, 150 / 151 / 101 at 1024).  A small tile's block has a short
@@ -382,7 +384,10 @@ hts_status launch_conv_strip(const ConvParams& p, const StripMaps* maps, cudaStr
     if (!p.wk || ((uintptr_t)p.x & 15)) return HTS_ERR_UNSUPPORTED;
     hts_status st = HTS_ERR_UNSUPPORTED;
     if (p.s == 4) {
-        if (56 + 22 * (strip_blocks(p, Few1::PX, Few1::SEGS) - 1) < 91 + 60 * (strip_blocks(p, Many1::PX, Many1::SEGS) - 1)) st = launch_strip<Few1>(p, nullptr, s);
+        const int few = 56 + 22 * (strip_blocks(p, Few1::PX, Few1::SEGS) - 1), many = 91 + 60 * (strip_blocks(p, Many1::PX, Many1::SEGS) - 1),
+                  five = 115 + 82 * (strip_blocks(p, Five1::PX, Five1::SEGS) - 1);
+        if (few < many && few < five) st = launch_strip<Few1>(p, nullptr, s);
+        if (st == HTS_ERR_UNSUPPORTED && five < many) st = launch_strip<Five1>(p, nullptr, s);
         if (st == HTS_ERR_UNSUPPORTED) st = launch_strip<Many1>(p, nullptr, s);
         if (st == HTS_ERR_UNSUPPORTED) st = launch_strip<Odd1>(p, nullptr, s);
         return st;

@@ -63,3 +63,22 @@ def test_frames_at_any_address(n, offset):
         assert np.array_equal(act.cpu().numpy(), want["actions"])
     finally:
         pol.close()
+
+
+@pytest.mark.parametrize("C,H,W,sizes", [(4, 84, 84, (30, 50, 100)), (16, 72, 96, (30, 50, 100)), (2, 40, 128, (40, 150))])
+def test_strips_of_five_pixels(C, H, W, sizes):
+    """Batches of which the first layer's blocks of four-pixel strips take one round more than those of five."""
+    cfg = dataclasses.replace(wl.CONFIGS[1], C=C, H=H, W=W)
+    n = max(sizes)
+    pol = Policy(cfg, max_batch=n)
+    try:
+        obs, ids = wl.make_obs(cfg, n), np.arange(n, dtype=np.int32)
+        few = [pol.step(obs[i:i + 8], ids[i:i + 8], 3, 17) for i in (0, n - 8)]
+        for m in sizes:
+            part = pol.step(obs[n - m:], ids[n - m:], 3, 17)
+            for k in part:
+                assert np.array_equal(part[k][-8:].view(np.int32), few[1][k].view(np.int32)), (m, k)
+                if m == n:
+                    assert np.array_equal(part[k][:8].view(np.int32), few[0][k].view(np.int32)), (m, k)
+    finally:
+        pol.close()
