@@ -10,7 +10,6 @@
 // function of the count alone, so the result does not depend on timing or on the device's load.
 #include <cmath>
 #include "common.cuh"
-#include "f32x2.cuh"
 #include "tc_ptx.cuh"
 
 namespace hts {
@@ -269,8 +268,8 @@ struct PpoOp {
 // for the host, where two take 6.5), then copies into at most 16 SMs.  Standardised means, us, calls in a row:
 //   transitions        64   2048  16384  50000  131072  147455
 //   two launches     7.67   8.26   8.13   8.52    9.06    9.93
-//   one              4.67   4.61   5.15   6.08    7.95    8.30
-// so it is taken as long as the inputs fit.  512 transitions to a block (2048: 5.42 at 2048; 256: the same).  A cooperative launch
+//   one              4.67   4.54   5.20   6.07    7.69    8.32
+// (16-byte asynchronous copies of the threads instead of bulk copies: 8.2 at 131072), so it is taken as long as the inputs fit.  512 transitions to a block (2048: 5.42 at 2048; 256: the same).  A cooperative launch
 // of sums_kernel's blocks with a barrier across the grid: 8.2 whatever the count, 9.3 at 131072.  The terms without the advantages
 // summed while the statistics cross the cluster: 8.24 at 131072 (the ratios pass through shared memory once more).
 constexpr int kClusterMost = 16, kClusterThreads = 512, kClusterHolds = 9216;      // transitions of a block: 24 bytes each
@@ -291,26 +290,34 @@ __device__ __forceinline__ void store_to_rank(double* here, unsigned rank, doubl
 __global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const PpoOp<false> op, int count, int per_block)
 {
     constexpr int NS = PpoOp<false>::NS;
-    extern __shared__ float4 s_in[];                     // [6][per_block / 4]: advantages first
+    extern __shared__ __align__(16) float4 s_in[];       // [6][per_block / 4]: advantages first
+    __shared__ uint64_t landed[2];                       // advantages; the others
+    __shared__ int gave_up;
     __shared__ double s_warp[kClusterWarps][NS], s_stat[kClusterMost][2], s_all[kClusterMost][NS];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const unsigned rank = blockIdx.x, ranks = gridDim.x;
+    if (tid == 0) {
+        tc::mbar_init(landed, 1); tc::mbar_init(landed + 1, 1);
+        gave_up = 0;
+        tc::fence_barrier_init();
+    }
+    __syncthreads();
     pdl_wait();
     pdl_trigger();
     const int lo = rank * per_block, n = max(0, min(per_block, count - lo)), quads = n >> 2, pitch = per_block >> 2;
-    const float* const arrays[6] = {op.adv, op.logp_new, op.logp_old, op.values, op.entropy, op.returns};
     const double first = (double)op.adv[0];
+    if (tid == 0 && quads > 0) {
+        const float* const arrays[6] = {op.adv, op.logp_new, op.logp_old, op.values, op.entropy, op.returns};
+        tc::mbar_arrive_expect_tx(landed, quads * 16);
+        tc::mbar_arrive_expect_tx(landed + 1, 5 * quads * 16);
 #pragma unroll
-    for (int a = 0; a < 6; ++a) {
-        for (int q = tid; q < quads; q += kClusterThreads) cp_async16(tc::smem_u32(s_in + a * pitch + q), reinterpret_cast<const float4*>(arrays[a] + lo) + q);
-        if (a == 0) cp_async_commit();
+        for (int a = 0; a < 6; ++a) tc::bulk_load(s_in + a * pitch, arrays[a] + lo, quads * 16, landed + (a > 0));
     }
-    cp_async_commit();
-    // A thread reads what it copied itself.  The last block's ragged transitions are read where they are.
+    // The last block's ragged transitions are read where they are.
     const int i = lo + 4 * quads + tid;
     const bool ragged = tid < (n & 3);
     double st[2] = {0.0, 0.0};
-    cp_async_wait<1>();
+    if (quads > 0) tc::mbar_wait_warp(landed, 0, &gave_up, nullptr, 0);
     for (int q = tid; q < quads; q += kClusterThreads) {
         const float4 a = s_in[q];
         AdvStatsOp::one(a.x, first, st); AdvStatsOp::one(a.y, first, st); AdvStatsOp::one(a.z, first, st); AdvStatsOp::one(a.w, first, st);
@@ -337,7 +344,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const
     double acc[NS];
 #pragma unroll
     for (int k = 0; k < NS; ++k) acc[k] = 0.0;
-    cp_async_wait_all();
+    if (quads > 0) tc::mbar_wait_warp(landed + 1, 0, &gave_up, nullptr, 0);
     for (int q = tid; q < quads; q += kClusterThreads)
         op.add4(PpoOp<false>::Quad{s_in[pitch + q], s_in[2 * pitch + q], s_in[3 * pitch + q], s_in[4 * pitch + q], s_in[q], s_in[5 * pitch + q]},
                 stats[0], stats[1], acc);
@@ -352,13 +359,17 @@ __global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const
 #pragma unroll
         for (int k = 0; k < NS; ++k) {
             const double v = warp_sum_d(lane < kClusterWarps ? s_warp[lane][k] : 0.0);
-            if (lane == 0) store_to_rank(&s_all[rank][k], 0, v);
+            if (lane == 0) store_to_rank(&s_all[rank][k], 0, *(volatile int*)&gave_up ? nan("") : v);
         }
     cluster_sync();
     if (rank == 0 && warp == 0) {
 #pragma unroll
         for (int k = 0; k < NS; ++k) acc[k] = warp_sum_d(lane < ranks ? s_all[lane][k] : 0.0);
         if (lane == 0) op.finish(acc, count);
+    }
+    if (*(volatile int*)&gave_up) {                      // give copies still in flight time to land
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000) { }
     }
 }
 
