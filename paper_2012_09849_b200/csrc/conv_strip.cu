@@ -353,12 +353,14 @@ typedef Form1<2, 4, 8, 2, 2, 2, 4> Few1;
 typedef Form1<4, 8, 8, 4, 2, 2, 3> Many1;
 typedef Form1<5, 8, 8, 4, 2, 2, 3> Five1;
 typedef Form1<4, 8, 8, 4, 1, 2, 3> Odd1;                // an odd number of channels
-typedef Form2<4, 2, 4, 4, 2, 4> Few2;
+typedef Form2<4, 2, 4, 8, 2, 2> Few2;
+typedef Form2<4, 2, 4, 4, 2, 4> Thin2;                 // wide rows: Few2's stages do not fit
 typedef Form2<9, 2, 4, 4, 2, 4> Some2n;                 // rows up to 9 pixels; else of strips of 10
 typedef Form2<10, 2, 4, 4, 2, 4> Some2w;
 typedef Form2<9, 4, 8, 4, 2, 3> Many2n;
 typedef Form2<10, 4, 8, 2, 3, 3> Many2w;                // (four channels of three frames' boxes are too much for three blocks per SM)
-typedef Form3<4, 2, 4, 8, 3, 2> Few3;
+typedef Form3<4, 2, 4, 16, 2, 2> Few3;
+typedef Form3<4, 2, 4, 8, 3, 2> Thin3;
 typedef Form3<7, 2, 4, 8, 2, 3> Some3n;                 // rows up to 7 pixels; else of strips of 8
 typedef Form3<8, 2, 4, 8, 2, 3> Some3w;
 
@@ -366,7 +368,7 @@ bool make_strip_maps(const Geometry& g, const RefWorkspace& ws, size_t frames, S
 {
     auto two = [&](auto form, CUtensorMap* map) { return strip_map<decltype(form)>(ws.l1, ws.a1, 32, g.H1, g.H2, g.W2, frames, map); };
     auto three = [&](auto form, CUtensorMap* map) { return strip_map<decltype(form)>(ws.l2, ws.a2, 64, g.H2, g.H3, g.W3, frames, map); };
-    return two(Few2{}, &m->few2) && three(Few3{}, &m->few3) &&
+    return two(Few2{}, &m->few2) && two(Thin2{}, &m->thin2) && three(Few3{}, &m->few3) && three(Thin3{}, &m->thin3) &&
            (g.W2 <= 9 ? two(Some2n{}, &m->some2) && two(Many2n{}, &m->many2) : two(Some2w{}, &m->some2) && two(Many2w{}, &m->many2)) &&
            (g.W3 <= 7 ? three(Some3n{}, &m->some3) : three(Some3w{}, &m->some3));
 }
@@ -377,6 +379,7 @@ bool make_strip_maps(const Geometry& g, const RefWorkspace& ws, size_t frames, S
 //     5 x 8: 11.5 + 8.2, where that saves a round (step of 50 frames of 72 x 96 x 16 73 -> 63 us, of 100 116 -> 106; 80: 85 / 98)
 //   second   4 x 2  7.4, 10.9, 14.9: 7.4 + 3.7     a row x 2  11.3, 18.0, 25.5, 32.9: 11.3 + 7.0     a row x 4  16.7, 29.5, .. 56 (4), .. 107 (8): 16.7 + 12.5
 //   third    4 x 2  8.6, 11.8, .. 21.2 (4): 8.6 + 4.2     a row x 2  10.2, 15.6, .. 27.2 (4), 44.7 (7), 80 (13): 10.1 + 5.8
+// Few2 and Few3 have four stages of 8 and 16 channels (eight of 4 and 8 before: step of 16 32.9 us, now 32.3).
 // (the tiles of policy_ref.cu: 12 to 16 at 16 frames, 26 / 31 / 22 at 80, 150 / 151 / 101 at 1024).  A small tile's block has a short
 // chain of sums, a large one more of them for each load.
 hts_status launch_conv_strip(const ConvParams& p, const StripMaps* maps, cudaStream_t s)
@@ -399,12 +402,14 @@ hts_status launch_conv_strip(const ConvParams& p, const StripMaps* maps, cudaStr
         const int few = 74 + 37 * (strip_blocks(p, 4, 4) - 1), some = 113 + 70 * (strip_blocks(p, px, 4) - 1), many = 167 + 125 * (strip_blocks(p, px, 8) - 1);
         if (few >= many && some >= many) st = narrow ? launch_strip<Many2n>(p, &maps->many2, s) : launch_strip<Many2w>(p, &maps->many2, s);
         if (st == HTS_ERR_UNSUPPORTED && few >= some) st = narrow ? launch_strip<Some2n>(p, &maps->some2, s) : launch_strip<Some2w>(p, &maps->some2, s);
-        return st == HTS_ERR_UNSUPPORTED ? launch_strip<Few2>(p, &maps->few2, s) : st;
+        if (st == HTS_ERR_UNSUPPORTED) st = launch_strip<Few2>(p, &maps->few2, s);
+        return st == HTS_ERR_UNSUPPORTED ? launch_strip<Thin2>(p, &maps->thin2, s) : st;
     }
     const bool narrow = p.Wo <= 7;
     if (86 + 42 * (strip_blocks(p, 4, 4) - 1) >= 101 + 58 * (strip_blocks(p, narrow ? 7 : 8, 4) - 1))
         st = narrow ? launch_strip<Some3n>(p, &maps->some3, s) : launch_strip<Some3w>(p, &maps->some3, s);
-    return st == HTS_ERR_UNSUPPORTED ? launch_strip<Few3>(p, &maps->few3, s) : st;
+    if (st == HTS_ERR_UNSUPPORTED) st = launch_strip<Few3>(p, &maps->few3, s);
+    return st == HTS_ERR_UNSUPPORTED ? launch_strip<Thin3>(p, &maps->thin3, s) : st;
 }
 
 }  // namespace hts

@@ -48,7 +48,7 @@ __device__ __forceinline__ size_t plane_row(const ConvParams& p, int e, int i, i
 #endif
 
 // Boxes of a context's activations, as the forms of the second and third layer read them.
-struct StripMaps { CUtensorMap few2, some2, many2, few3, some3; };
+struct StripMaps { CUtensorMap few2, thin2, some2, many2, few3, thin3, some3; };
 bool make_strip_maps(const Geometry& g, const RefWorkspace& ws, size_t frames, StripMaps* maps);
 
 // HTS_ERR_UNSUPPORTED: not a shape for strips (nothing was launched).
