@@ -164,7 +164,7 @@ gae_scan_kernel(const float* __restrict__ rewards, const float* __restrict__ val
 
 template <int VEC, int L, int CY>
 hts_status launch_t(const float* r, const float* v, const uint8_t* d, const float* b, float gamma,
-                    float lambda, int T, int N, float* adv, float* ret, int maxW, cudaStream_t s)
+                    float lambda, int T, int N, float* adv, float* ret, int maxW, int sms, cudaStream_t s)
 {
     const int chunks = (T + L - 1) / L;
     int W = (chunks + CY - 1) / CY;
@@ -173,7 +173,7 @@ hts_status launch_t(const float* r, const float* v, const uint8_t* d, const floa
     const unsigned blocks = (unsigned)((N + cols - 1) / cols);
     const size_t smem = (size_t)2 * W * CY * cols * sizeof(float);
     constexpr bool V1 = VEC == 1;
-    const bool many = V1 && W * CY >= kManyChunks, roomy = V1 && W <= 16 && (int)blocks <= device_sm_count(device_slot());
+    const bool many = V1 && W * CY >= kManyChunks, roomy = V1 && W <= 16 && (int)blocks <= sms;
     auto kernel = many ? (roomy ? gae_scan_kernel<VEC, L, CY, V1, V1> : gae_scan_kernel<VEC, L, CY, V1, false>)
                        : (roomy ? gae_scan_kernel<VEC, L, CY, false, V1> : gae_scan_kernel<VEC, L, CY, false, false>);
     HTS_CUDA(launch_pdl(kernel, dim3(blocks), dim3(32, W), smem, s, r, v, d, b, gamma, lambda, T, N, adv, ret));
@@ -201,15 +201,15 @@ hts_status launch_gae(const float* rewards, const float* values, const uint8_t* 
     // at T=512: 186 / 130, 234 / 222, 366 / 436: they cross between 2^17 and 2^18 columns, 7 and 14 blocks per SM;
     // short columns walk few steps: 11.3 / 12.3 at 32 x 2^17, but 20.9 / 16.6 at 64 x 80000.
     if (vec4 && N / 128 >= (T < 64 ? 4 : 8) * sms)
-        return launch_t<4, 2, 1>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, 2, s);
+        return launch_t<4, 2, 1>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, 2, sms, s);
     // few columns and many rows: 8-column blocks, four chunks per warp (same chunks, same bits, four times the SMs).
     // Against 32 columns: 4.3 / 8.9 us at 512 x 512, 7.9 / 11.4 at 512 x 2048, 14.8 / 13.0 at 512 x 4096
     const int blocks = (N + 31) / 32;
     if (blocks < sms / 2 && T >= 4 * 8)
-        return launch_t<1, 8, 4>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, 32, s);
+        return launch_t<1, 8, 4>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, 32, sms, s);
     // several blocks per SM load, chain and store at different times; one per SM takes as many rows as it can: 8 / 32 chunk
     // rows per step at 512 x 4096 (128 blocks) 17.9 / 13.0 us, 128 x 18976 (593) 11.3 / 12.5, 128 x 75648 34 / 39
-    return launch_t<1, 8, 1>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, blocks >= 4 * sms ? 8 : 32, s);
+    return launch_t<1, 8, 1>(rewards, values, dones, bootstrap, gamma, lambda, T, N, adv, ret, blocks >= 4 * sms ? 8 : 32, sms, s);
 }
 
 }  // namespace hts

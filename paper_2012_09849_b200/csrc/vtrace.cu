@@ -184,7 +184,7 @@ vtrace_scan_kernel(const VtraceParams p)
 }
 
 template <int VEC, int L, int CY, int MAXW>
-hts_status launch_t(const VtraceParams& p, cudaStream_t s)
+hts_status launch_t(const VtraceParams& p, int sms, cudaStream_t s)
 {
     int W = ((p.T + L - 1) / L + CY - 1) / CY;
     if (W > MAXW) W = MAXW;
@@ -192,7 +192,7 @@ hts_status launch_t(const VtraceParams& p, cudaStream_t s)
     const unsigned blocks = (unsigned)((p.N + cols - 1) / cols);
     const size_t smem = (size_t)2 * W * CY * cols * sizeof(float);
     constexpr bool V1 = VEC == 1, M = V1 && MAXW * CY >= kManyChunks;
-    const bool many = M && W * CY >= kManyChunks, roomy = V1 && (int)blocks <= device_sm_count(device_slot());
+    const bool many = M && W * CY >= kManyChunks, roomy = V1 && (int)blocks <= sms;
     auto kernel = many ? (roomy ? vtrace_scan_kernel<VEC, L, CY, MAXW, M, V1> : vtrace_scan_kernel<VEC, L, CY, MAXW, M, false>)
                        : (roomy ? vtrace_scan_kernel<VEC, L, CY, MAXW, false, V1> : vtrace_scan_kernel<VEC, L, CY, MAXW, false, false>);
     HTS_CUDA(launch_pdl(kernel, dim3(blocks), dim3(32, W), smem, s, p));
@@ -219,10 +219,10 @@ hts_status launch_vtrace(const float* log_rhos, const float* rewards, const floa
     //   4 against 8 warps: 30.2 / 32.3 at 128 x 37856, 92 / 96 at 256 x 60001, 46.6 / 29.4 at 512 x 8192
     //   8 against 16 warps: 7.7 / 8.6 at 128 x 4768 (149 blocks), 7.6 / 5.4 at 128 x 4704 (147)
     const int sms = device_sm_count(device_slot()), blocks = (N + 31) / 32;
-    if (vec4 && N / 128 >= (T < 64 ? 4 : 6) * sms) return launch_t<4, 2, 1, 2>(p, s);
-    if (blocks < sms / 2 && T >= 4 * 8) return launch_t<1, 8, 4, 16>(p, s);
-    if (blocks >= 8 * sms) return launch_t<1, 8, 1, 4>(p, s);
-    return blocks >= sms ? launch_t<1, 8, 1, 8>(p, s) : launch_t<1, 8, 1, 16>(p, s);
+    if (vec4 && N / 128 >= (T < 64 ? 4 : 6) * sms) return launch_t<4, 2, 1, 2>(p, sms, s);
+    if (blocks < sms / 2 && T >= 4 * 8) return launch_t<1, 8, 4, 16>(p, sms, s);
+    if (blocks >= 8 * sms) return launch_t<1, 8, 1, 4>(p, sms, s);
+    return blocks >= sms ? launch_t<1, 8, 1, 8>(p, sms, s) : launch_t<1, 8, 1, 16>(p, sms, s);
 }
 
 }  // namespace hts
