@@ -6,7 +6,9 @@
 // mbarrier per stage; all waits are bounded), and a thread reads 20 inputs and 16 weights for 144 multiply-adds (second layer)
 // where 8 x 8 tiles read 32 and 32 for 128.  Bound: the fp32 pipes (80 % busy while the sums run; 60 TFLOP/s of the 70 that packed
 // multiply-adds reach), then what a block spends on its first copies and its stores.  At 1024 observations of 84 x 84 x 4 the
-// three layers take 133 / 107 / 80 us, in gathered tiles 150 / 151 / 101; at 80 15 / 17 / 10.5 against 26 / 31 / 22.
+// three layers take 131 / 100 / 78 us, in gathered tiles 150 / 151 / 101.  All channels of a stage are one straight run of instructions,
+// so that the next channel's loads are under way during a channel's sums: with a loop over channels (first layer: filter rows) 133 /
+// 107 / 80, and 60.3 instead of 57.1 us for a step of 80.
 // Rows have an odd number of 16-byte pieces and, for stride 2, even and odd rows lie apart: eight output rows' inputs are in eight
 // different sixteenths of the banks.  Copies issued by the computing warps cost 20 % (their address chains come before every
 // stage's first sums), one copying warp with 16-byte asynchronous copies 10 to 20 us a layer (40 of them per stage and lane).

@@ -265,13 +265,14 @@ struct PpoOp {
 // Standardised terms of few transitions in one launch: a cluster of up to 16 blocks whose shared memory holds all inputs, so that
 // the advantages' statistics and the terms are two passes over it, with the blocks' sums exchanged through each other's shared
 // memory in between.  The sums' order is fixed by the count; nothing global is written but the results.  Bound: one launch (4.3 us
-// for the host, where two take 6.5), then copies into at most 16 SMs.  Standardised means, us, calls in a row:
+// for the host, where two take 6.5), then copies into at most 16 SMs and fp64 conversions and sums there.  Standardised means, us, calls in a row:
 //   transitions        64   2048  16384  50000  131072  147455
 //   two launches     7.67   8.26   8.13   8.52    9.06    9.93
 //   one              4.67   4.54   5.20   6.07    7.69    8.32
-// (16-byte asynchronous copies of the threads instead of bulk copies: 8.2 at 131072), so it is taken as long as the inputs fit.  512 transitions to a block (2048: 5.42 at 2048; 256: the same).  A cooperative launch
-// of sums_kernel's blocks with a barrier across the grid: 8.2 whatever the count, 9.3 at 131072.  The terms without the advantages
-// summed while the statistics cross the cluster: 8.24 at 131072 (the ratios pass through shared memory once more).
+// so it is taken as long as the inputs fit.  512 transitions to a block (2048: 5.42 at 2048; 256: the same); 256 or 1024 threads: 8.0
+// and 9.0 at 131072, 4.3 and 5.6 at 2048.  16-byte asynchronous copies of the threads instead of bulk copies: 8.2 at 131072.  The terms
+// without the advantages summed while the statistics cross the cluster: 8.24 (the ratios pass through shared memory once more).  A
+// cooperative launch of sums_kernel's blocks with a barrier across the grid: 8.2 whatever the count, 9.3 at 131072.
 constexpr int kClusterMost = 16, kClusterThreads = 512, kClusterHolds = 9216;      // transitions of a block: 24 bytes each
 constexpr int kClusterEach = 512;                        // transitions before another block is worth its place
 constexpr int kClusterWarps = kClusterThreads / 32;
