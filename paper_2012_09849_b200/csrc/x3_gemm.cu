@@ -1,5 +1,6 @@
 // The two tensor-core kernels of the fp32-accurate path (see x3_gemm.cuh for the arithmetic and the layouts).
 #include "x3_gemm.cuh"
+#include "x3_ring.cuh"
 #include "tc_ptx.cuh"
 #include "tc_host.cuh"
 
@@ -86,7 +87,8 @@ __device__ __forceinline__ void acc_release(uint64_t* empty_bar, int lane)
 // per tile and every tap reads it shifted, and the weights of an N tile stay in the ring while its M tiles pass, if they
 // fit (conv2's 96 KB: gradient of 1024 323 -> 317 us without its forward pass).  One issuing thread: 2 to 3 us more at 5 to 40
 // rows, where a tile is a chain of its own, the same at 1024.
-constexpr int kAccs = 2, kPart = 2, kThreads = 96 + 256;
+// The slots' hand-over is in x3_ring.cuh.
+constexpr int kAccs = 2, kThreads = 96 + 256;
 struct DgradShared {
     uint64_t a_full[kMaxEntries], a_empty[kMaxEntries], b_full[kMaxStages], b_empty[kMaxStages], d_full[kAccs], d_empty[kAccs];
     uint32_t tmem_slot;
@@ -105,12 +107,10 @@ __device__ __forceinline__ void x3_dgrad(const CUtensorMap& tmA, const CUtensorM
     const uint32_t b_base = base + p.entries * a_pitch;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles = p.m_tiles * p.n_tiles;
-    const int groups = p.taps / p.tpe;                  // A entries per chunk
-    const bool stay = p.chunks * p.taps <= p.b_stages;  // the weights of an N tile stay while its M tiles pass
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kMaxEntries; ++i) { mbar_init(&a_full[i], 1); mbar_init(&a_empty[i], 2); }
-        for (int i = 0; i < kMaxStages; ++i) { mbar_init(&b_full[i], 1); mbar_init(&b_empty[i], stay ? 2 : 1); }
+        for (int i = 0; i < kMaxStages; ++i) { mbar_init(&b_full[i], 1); mbar_init(&b_empty[i], 2); }
         for (int i = 0; i < kAccs; ++i) { mbar_init(&d_full[i], 1); mbar_init(&d_empty[i], 8); }
         sh.abort_flag = 0;
         fence_barrier_init();
@@ -125,85 +125,64 @@ __device__ __forceinline__ void x3_dgrad(const CUtensorMap& tmA, const CUtensorM
     pdl_wait();
     pdl_trigger();
 
-    // tile -> (M tile, N tile): M fastest, so that CTAs running together share B through L2
+    const X3Ring ring{p.m_tiles, p.n_tiles, p.chunks, p.taps, p.tpe, p.entries, p.b_stages, first, blocks};
     if (warp == 0) {
         if (lane == 0) {
-            int ea = 0, sb = 0, held = -1;
-            uint32_t pa = 1, pb = 1;                    // parity of the "empty" phase waited for
-            bool alive = true;
-            for (int t = first; alive && t < tiles; t += blocks) {
-                const int mt = t % p.m_tiles, nt = t / p.m_tiles;
-                const bool load = !stay || nt != held;
-                if (stay) { sb = 0; if (load && held >= 0) pb ^= 1u; }
-                held = nt;
-                for (int c = 0; alive && c < p.chunks; ++c) {
-                    const int kc = c * 64;
-                    for (int g = 0; alive && g < groups; ++g) {
-                        if (!mbar_wait(&a_empty[ea], pa, abortp, p.status, 81)) { alive = false; break; }
-                        mbar_arrive_expect_tx(&a_full[ea], (uint32_t)a_bytes);
-                        tma_load_3d(base + ea * a_pitch, &tmA, kc, mt * 128 + (p.tpe == 1 ? p.shift[g] : p.lo), 0, &a_full[ea]);
-                        if (++ea == p.entries) { ea = 0; pa ^= 1u; }
-                        for (int j = 0; load && j < p.tpe; ++j) {
-                            if (!mbar_wait(&b_empty[sb], pb, abortp, p.status, 82)) { alive = false; break; }
-                            mbar_arrive_expect_tx(&b_full[sb], BB);
-                            tma_load_3d(b_base + sb * BB, &tmB, (g + j) * p.tap_cols + nt * 64, kc, 0, &b_full[sb]);
-                            if (++sb == p.b_stages && !stay) { sb = 0; pb ^= 1u; }
-                        }
-                    }
+            struct {
+                const CUtensorMap &tmA, &tmB;
+                const X3TapParams& p;
+                uint64_t *a_full, *a_empty, *b_full, *b_empty;
+                volatile int* abortp;
+                uint32_t base, b_base;
+                int a_bytes, a_pitch;
+                __device__ __forceinline__ bool wait_a_empty(int ea, uint32_t par) { return mbar_wait(&a_empty[ea], par, abortp, p.status, 81); }
+                __device__ __forceinline__ bool wait_b_empty(int sb, uint32_t par) { return mbar_wait(&b_empty[sb], par, abortp, p.status, 82); }
+                __device__ __forceinline__ void load_a(int ea, int mt, int c, int g)
+                {
+                    mbar_arrive_expect_tx(&a_full[ea], (uint32_t)a_bytes);
+                    tma_load_3d(base + ea * a_pitch, &tmA, c * 64, mt * 128 + (p.tpe == 1 ? p.shift[g] : p.lo), 0, &a_full[ea]);
                 }
-            }
+                __device__ __forceinline__ void load_b(int sb, int nt, int c, int tap)
+                {
+                    mbar_arrive_expect_tx(&b_full[sb], BB);
+                    tma_load_3d(b_base + sb * BB, &tmB, tap * p.tap_cols + nt * 64, c * 64, 0, &b_full[sb]);
+                }
+            } io{tmA, tmB, p, a_full, a_empty, b_full, b_empty, abortp, base, b_base, a_bytes, a_pitch};
+            x3_ring_copy(ring, io);
         }
     } else if (warp <= 2) {
         if (lane == 0) {
             const int e = warp - 1;                     // this thread's accumulator: every other accumulation
-            int ea = 0, sb = 0, it = 0, left = p.chunks * p.taps, in = 0;
-            uint32_t pa = 0, pb = 0;
-            bool alive = true;
-            const uint64_t a_plane = (uint64_t)(plane_bytes >> 4);
-            int end = p.m_tiles;                        // of the N tile's tiles
-            while (stay && end <= first) end += p.m_tiles;
-            for (int t = first; alive && t < tiles; t += blocks, left = p.chunks * p.taps) {
-                if (stay) {
-                    sb = 0;
-                    if (t >= end) pb ^= 1u;
-                    while (end <= t) end += p.m_tiles;
-                }
-                const bool give = !stay || t + blocks >= end;            // the last to read them
-                for (int c = 0; alive && c < p.chunks; ++c)
-                    for (int g = 0; alive && g < groups; ++g) {
-                        bool used = false;
-                        for (int j = 0; j < p.tpe; ++j) {
-                            if ((it & 1) == e) {
-                                if (!used && !mbar_wait(&a_full[ea], pa, abortp, p.status, 84)) { alive = false; break; }
-                                used = true;
-                                if (!mbar_wait(&b_full[sb], pb, abortp, p.status, 85)) { alive = false; break; }
-                                if (in == 0 && !mbar_wait(&d_empty[e], (((uint32_t)(it / kAccs)) & 1u) ^ 1u, abortp, p.status, 83)) { alive = false; break; }
-                                tc_fence_after();
-                                const uint32_t row = p.tpe == 1 ? 0 : (uint32_t)(p.shift[j] - p.lo);
-                                const uint64_t a = smem_desc_sw128(base + ea * a_pitch + row * 128);
-                                const uint64_t b = smem_desc_mn(b_base + sb * BB, BB / 3);
+            struct {
+                const X3TapParams& p;
+                uint64_t *a_full, *a_empty, *b_full, *b_empty, *d_full, *d_empty;
+                volatile int* abortp;
+                uint32_t base, b_base, tmem;
+                int a_pitch, plane_bytes;
+                __device__ __forceinline__ bool wait_a_full(int ea, uint32_t par) { return mbar_wait(&a_full[ea], par, abortp, p.status, 84); }
+                __device__ __forceinline__ bool wait_b_full(int sb, uint32_t par) { return mbar_wait(&b_full[sb], par, abortp, p.status, 85); }
+                __device__ __forceinline__ bool wait_d_empty(uint32_t par) { return mbar_wait(d_empty, par, abortp, p.status, 83); }
+                __device__ __forceinline__ void commit_a_empty(int ea) { mma_commit(&a_empty[ea]); }
+                __device__ __forceinline__ void commit_b_empty(int sb) { mma_commit(&b_empty[sb]); }
+                __device__ __forceinline__ void commit_d_full() { mma_commit(d_full); }
+                __device__ __forceinline__ void arrive_a_empty(int ea) { mbar_arrive(&a_empty[ea]); }
+                __device__ __forceinline__ void arrive_b_empty(int sb) { mbar_arrive(&b_empty[sb]); }
+                __device__ __forceinline__ void multiply(int ea, int sb, int j, bool start)
+                {
+                    tc_fence_after();
+                    const uint32_t row = p.tpe == 1 ? 0 : (uint32_t)(p.shift[j] - p.lo);
+                    const uint64_t a_plane = (uint64_t)(plane_bytes >> 4), a = smem_desc_sw128(base + ea * a_pitch + row * 128);
+                    const uint64_t b = smem_desc_mn(b_base + sb * BB, BB / 3);
 #pragma unroll
-                                for (int k = 0; k < 4; ++k)      // 32 bytes along A's rows, 16 rows of B
-                                    mma_x3<3, 64>(tmem_d + e * 192, a + 2 * k, a_plane, b + 128 * k, 0, 1, (in | k) == 0);
-                                if (give) mma_commit(&b_empty[sb]);
-                            } else if (stay && give)
-                                mbar_arrive(&b_empty[sb]);
-                            --left;
-                            if (++in == kPart || left == 0) {
-                                if ((it & 1) == e) mma_commit(&d_full[e]);
-                                ++it; in = 0;
-                            }
-                            if (++sb == p.b_stages && !stay) { sb = 0; pb ^= 1u; }
-                        }
-                        if (used) mma_commit(&a_empty[ea]);
-                        else mbar_arrive(&a_empty[ea]);
-                        if (++ea == p.entries) { ea = 0; pa ^= 1u; }
-                    }
-            }
+                    for (int k = 0; k < 4; ++k)          // 32 bytes along A's rows, 16 rows of B
+                        mma_x3<3, 64>(tmem, a + 2 * k, a_plane, b + 128 * k, 0, 1, start && k == 0);
+                }
+            } io{p, a_full, a_empty, b_full, b_empty, d_full + e, d_empty + e, abortp, base, b_base, tmem_d + e * 192, a_pitch, plane_bytes};
+            x3_ring_issue(ring, e, io);
         }
     } else {
         const int j = (warp - 3) >> 2, q = warp & 3;    // half of the columns; TMEM lane quarter of this warp
-        const int row = q * 32 + lane, parts = (p.chunks * p.taps + kPart - 1) / kPart;
+        const int row = q * 32 + lane, parts = (p.chunks * p.taps + kX3Part - 1) / kX3Part;
         int it = 0;
         bool alive = true;
         for (int t = first; alive && t < tiles; t += blocks) {
