@@ -268,8 +268,9 @@ struct PpoOp {
 // for the host, where two take 6.5), then copies into at most 16 SMs and fp64 conversions and sums there.  Standardised means, us, calls in a row:
 //   transitions        64   2048  16384  50000  131072  147455
 //   two launches     7.67   8.26   8.13   8.52    9.06    9.93
-//   one              4.67   4.54   5.20   6.07    7.69    8.32
-// so it is taken as long as the inputs fit.  512 transitions to a block (2048: 5.42 at 2048; 256: the same); 256 or 1024 threads: 8.0
+//   one              4.22   4.50   5.30   6.18    7.79    8.39
+// so it is taken as long as the inputs fit.  Beside actor steps of 1024 on another stream, which leave few SMs free, the median call takes
+// 20, 16, 23, 24, 27 and 26 us (at 147456), two launches 30, 31, 28, 32, 32 and 32; the steps take as long beside either.  512 transitions to a block (2048: 5.42 at 2048; 256: the same); 256 or 1024 threads: 8.0
 // and 9.0 at 131072, 4.3 and 5.6 at 2048.  16-byte asynchronous copies of the threads instead of bulk copies: 8.2 at 131072.  The terms
 // without the advantages summed while the statistics cross the cluster: 8.24 (the ratios pass through shared memory once more).  A
 // cooperative launch of sums_kernel's blocks with a barrier across the grid: 8.2 whatever the count, 9.3 at 131072.
@@ -277,9 +278,12 @@ constexpr int kClusterMost = 16, kClusterThreads = 512, kClusterHolds = 9216;   
 constexpr int kClusterEach = 512;                        // transitions before another block is worth its place
 constexpr int kClusterWarps = kClusterThreads / 32;
 
+__device__ __forceinline__ void cluster_started() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync()
 {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    cluster_wait();
 }
 __device__ __forceinline__ void store_to_rank(double* here, unsigned rank, double v)
 {
@@ -303,6 +307,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const
         tc::fence_barrier_init();
     }
     __syncthreads();
+    cluster_started();
     pdl_wait();
     pdl_trigger();
     const int lo = rank * per_block, n = max(0, min(per_block, count - lo)), quads = n >> 2, pitch = per_block >> 2;
@@ -330,6 +335,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const
         if (lane == 0) s_warp[warp][k] = st[k];
     }
     __syncthreads();
+    cluster_wait();                                      // every block has started: its shared memory may be written from here on
     if (warp == 0) {
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
