@@ -269,11 +269,12 @@ struct PpoOp {
 //   transitions        64   2048  16384  50000  131072  147455
 //   two launches     7.67   8.26   8.13   8.52    9.06    9.93
 //   one              4.22   4.50   5.30   6.18    7.79    8.39
-// so it is taken as long as the inputs fit.  Beside actor steps of 1024 on another stream, which leave few SMs free, the median call takes
-// 20, 16, 23, 24, 27 and 26 us (at 147456), two launches 30, 31, 28, 32, 32 and 32; the steps take as long beside either.  512 transitions to a block (2048: 5.42 at 2048; 256: the same); 256 or 1024 threads: 8.0
-// and 9.0 at 131072, 4.3 and 5.6 at 2048.  16-byte asynchronous copies of the threads instead of bulk copies: 8.2 at 131072.  The terms
-// without the advantages summed while the statistics cross the cluster: 8.24 (the ratios pass through shared memory once more).  A
-// cooperative launch of sums_kernel's blocks with a barrier across the grid: 8.2 whatever the count, 9.3 at 131072.
+// so it is taken as long as the inputs fit.  Beside actor steps of 1024 on another stream, which leave few SMs free, the median call
+// takes 20, 16, 23, 24, 27 and 26 us (at 147456), two launches 30, 31, 28, 32, 32 and 32; the steps take as long beside either.  512
+// transitions to a block (2048: 5.42 at 2048; 256: the same); 256 or 1024 threads: 8.0 and 9.0 at 131072, 4.3 and 5.6 at 2048.  16-byte
+// asynchronous copies of the threads instead of bulk copies: 8.2 at 131072.  The terms without the advantages summed while the
+// statistics cross the cluster: 8.24 (the ratios pass through shared memory once more).  A cooperative launch of sums_kernel's blocks
+// with a barrier across the grid: 8.2 whatever the count, 9.3 at 131072.
 constexpr int kClusterMost = 16, kClusterThreads = 512, kClusterHolds = 9216;      // transitions of a block: 24 bytes each
 constexpr int kClusterEach = 512;                        // transitions before another block is worth its place
 constexpr int kClusterWarps = kClusterThreads / 32;
@@ -292,7 +293,7 @@ __device__ __forceinline__ void store_to_rank(double* here, unsigned rank, doubl
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there), "d"(v) : "memory");
 }
 
-__global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const PpoOp<false> op, int count, int per_block)
+__global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const PpoOp<false> op, int count, int per_block, bool lost)
 {
     constexpr int NS = PpoOp<false>::NS;
     extern __shared__ __align__(16) float4 s_in[];       // [6][per_block / 4]: advantages first
@@ -312,7 +313,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const
     pdl_trigger();
     const int lo = rank * per_block, n = max(0, min(per_block, count - lo)), quads = n >> 2, pitch = per_block >> 2;
     const double first = (double)op.adv[0];
-    if (tid == 0 && quads > 0) {
+    if (tid == 0 && quads > 0 && !lost) {
         const float* const arrays[6] = {op.adv, op.logp_new, op.logp_old, op.values, op.entropy, op.returns};
         tc::mbar_arrive_expect_tx(landed, quads * 16);
         tc::mbar_arrive_expect_tx(landed + 1, 5 * quads * 16);
@@ -323,10 +324,19 @@ __global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const
     const int i = lo + 4 * quads + tid;
     const bool ragged = tid < (n & 3);
     double st[2] = {0.0, 0.0};
-    if (quads > 0) tc::mbar_wait_warp(landed, 0, &gave_up, nullptr, 0);
-    for (int q = tid; q < quads; q += kClusterThreads) {
-        const float4 a = s_in[q];
-        AdvStatsOp::one(a.x, first, st); AdvStatsOp::one(a.y, first, st); AdvStatsOp::one(a.z, first, st); AdvStatsOp::one(a.w, first, st);
+    const long long limit = lost ? 100000 : tc::kWaitLimitTicks;
+    auto copied = [&](int a, const float*, int q) { return s_in[a * pitch + q]; };
+    // Where copies do not land, a warp reads the same inputs where they are.
+    auto global = [&](int, const float* from, int q) { return reinterpret_cast<const float4*>(from + lo)[q]; };
+    auto add_stats = [&](auto input) {
+        for (int q = tid; q < quads; q += kClusterThreads) {
+            const float4 a = input(0, op.adv, q);
+            AdvStatsOp::one(a.x, first, st); AdvStatsOp::one(a.y, first, st); AdvStatsOp::one(a.z, first, st); AdvStatsOp::one(a.w, first, st);
+        }
+    };
+    if (quads > 0) {
+        if (tc::mbar_wait_warp(landed, 0, &gave_up, nullptr, 0, limit)) add_stats(copied);
+        else add_stats(global);
     }
     if (ragged) AdvStatsOp::one(op.adv[i], first, st);
 #pragma unroll
@@ -351,10 +361,15 @@ __global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const
     double acc[NS];
 #pragma unroll
     for (int k = 0; k < NS; ++k) acc[k] = 0.0;
-    if (quads > 0) tc::mbar_wait_warp(landed + 1, 0, &gave_up, nullptr, 0);
-    for (int q = tid; q < quads; q += kClusterThreads)
-        op.add4(PpoOp<false>::Quad{s_in[pitch + q], s_in[2 * pitch + q], s_in[3 * pitch + q], s_in[4 * pitch + q], s_in[q], s_in[5 * pitch + q]},
-                stats[0], stats[1], acc);
+    auto add_terms = [&](auto input) {
+        for (int q = tid; q < quads; q += kClusterThreads)
+            op.add4(PpoOp<false>::Quad{input(1, op.logp_new, q), input(2, op.logp_old, q), input(3, op.values, q), input(4, op.entropy, q),
+                                       input(0, op.adv, q), input(5, op.returns, q)}, stats[0], stats[1], acc);
+    };
+    if (quads > 0) {
+        if (tc::mbar_wait_warp(landed, 0, &gave_up, nullptr, 0, limit) && tc::mbar_wait_warp(landed + 1, 0, &gave_up, nullptr, 0, limit)) add_terms(copied);
+        else add_terms(global);
+    }
     if (ragged) op.add1(i, stats[0], stats[1], acc);
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
@@ -366,7 +381,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const
 #pragma unroll
         for (int k = 0; k < NS; ++k) {
             const double v = warp_sum_d(lane < kClusterWarps ? s_warp[lane][k] : 0.0);
-            if (lane == 0) store_to_rank(&s_all[rank][k], 0, *(volatile int*)&gave_up ? nan("") : v);
+            if (lane == 0) store_to_rank(&s_all[rank][k], 0, v);
         }
     cluster_sync();
     if (rank == 0 && warp == 0) {
@@ -380,7 +395,8 @@ __global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const
     }
 }
 
-cudaError_t launch_terms_cluster(const PpoOp<false>& op, int count, cudaStream_t s)
+// lost: without the copies, as if none of them landed (self-test).
+cudaError_t launch_terms_cluster(const PpoOp<false>& op, int count, cudaStream_t s, bool lost = false)
 {
     int ranks = 1;
     while (ranks < kClusterMost && ranks * kClusterEach < count) ranks *= 2;
@@ -401,7 +417,7 @@ cudaError_t launch_terms_cluster(const PpoOp<false>& op, int count, cudaStream_t
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, terms_cluster_kernel, op, count, per_block);
+    return cudaLaunchKernelEx(&cfg, terms_cluster_kernel, op, count, per_block, lost);
 }
 
 }  // namespace
@@ -416,11 +432,14 @@ extern "C" hts_status hts_a2c_terms(const float* logp, const float* values, cons
     return launch_sums(op, (long long)count, static_cast<cudaStream_t>(cuda_stream));
 }
 
-extern "C" hts_status hts_ppo_terms(const float* logp_new, const float* logp_old, const float* values, const float* entropy,
-                                    const float* advantages, const float* returns, int64_t count, float clip,
-                                    int32_t normalize_advantages, float* out4, void* cuda_stream)
+namespace hts {
+namespace {
+
+enum class TermsForm { ByCount, ClusterLost };
+
+hts_status ppo_terms(const float* logp_new, const float* logp_old, const float* values, const float* entropy, const float* advantages,
+                     const float* returns, int64_t count, float clip, int32_t normalize_advantages, float* out4, void* cuda_stream, TermsForm form)
 {
-    using namespace hts;
     if (!logp_new || !logp_old || !values || !entropy || !advantages || !returns || !out4 || count < 1) return HTS_ERR_INVALID_ARG;
     if (!(clip > 0.f) || std::isinf(clip)) return HTS_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
@@ -428,7 +447,7 @@ extern "C" hts_status hts_ppo_terms(const float* logp_new, const float* logp_old
     const PpoOp<false> op{logp_new, logp_old, values, entropy, advantages, returns, out4, (double)clip, normalize_advantages != 0, vec};
     if (!normalize_advantages) return launch_sums(op, (long long)count, s);
     if (vec && count <= kClusterMost * kClusterHolds) {
-        if (launch_terms_cluster(op, (int)count, s) == cudaSuccess) { note_launch(); return HTS_OK; }
+        if (launch_terms_cluster(op, (int)count, s, form == TermsForm::ClusterLost) == cudaSuccess) { note_launch(); return HTS_OK; }
         cudaGetLastError();                              // a part of a device may have no room for the cluster: two launches
     }
     const hts_status st = launch_sums(AdvStatsOp{advantages, all_aligned16({advantages})}, (long long)count, s);
@@ -438,6 +457,24 @@ extern "C" hts_status hts_ppo_terms(const float* logp_new, const float* logp_old
         return launch_sums<Form::EarlyTwo>(op, (long long)count, s);
     return launch_sums<Form::EarlyThree>(PpoOp<true>{logp_new, logp_old, values, entropy, advantages, returns, out4, (double)clip, true, vec},
                                          (long long)count, s);
+}
+
+}  // namespace
+}  // namespace hts
+
+extern "C" hts_status hts_ppo_terms(const float* logp_new, const float* logp_old, const float* values, const float* entropy,
+                                    const float* advantages, const float* returns, int64_t count, float clip,
+                                    int32_t normalize_advantages, float* out4, void* cuda_stream)
+{
+    return hts::ppo_terms(logp_new, logp_old, values, entropy, advantages, returns, count, clip, normalize_advantages, out4, cuda_stream,
+                          hts::TermsForm::ByCount);
+}
+
+// The standardised means by the cluster without its copies, for tests; not declared in hts.h.
+extern "C" hts_status hts_ppo_terms_selftest(const float* logp_new, const float* logp_old, const float* values, const float* entropy,
+                                             const float* advantages, const float* returns, int64_t count, float clip, float* out4, void* cuda_stream)
+{
+    return hts::ppo_terms(logp_new, logp_old, values, entropy, advantages, returns, count, clip, 1, out4, cuda_stream, hts::TermsForm::ClusterLost);
 }
 
 // ---- the learner's parameter update (Section 4.1 "Delayed gradient", Eq. 5) ---------------------------------

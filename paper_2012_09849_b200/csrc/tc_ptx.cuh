@@ -90,11 +90,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 }
 // The same for a whole warp (all 32 lanes must call it together): lane 0 polls, the others
 // join once the phase has completed, so a waiting warp costs one poller instead of 32.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status, int code)
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status, int code,
+                                               long long limit_ticks = kWaitLimitTicks)
 {
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;      // already complete: one poll, one vote
     bool ok = true;
-    if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort_flag, status, code);
+    if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort_flag, status, code, limit_ticks);
     ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
     if (ok) {
         while (!mbar_try_wait(bar, parity)) { }         // completes at once: the phase is already over

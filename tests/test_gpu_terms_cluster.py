@@ -37,3 +37,16 @@ def test_the_same_bits_beside_actor_steps(count):
     finally:
         pol.close()
     assert np.array_equal(beside.cpu().numpy().view(np.int32), np.tile(alone.cpu().numpy().view(np.int32), (50, 1)))
+
+
+def test_copies_that_never_land_are_read_where_they_are():
+    """The wait for them runs out after a moment; the result is the same, to the bit."""
+    import ctypes
+    selftest = hts.lib().hts_ppo_terms_selftest
+    selftest.restype, selftest.argtypes = ctypes.c_int, [ctypes.c_void_p] * 6 + [ctypes.c_int64, ctypes.c_float] + [ctypes.c_void_p] * 2
+    for count in (3, 700, 9217, 131071):
+        x, out = inputs(count), torch.zeros(2, 4, device="cuda")
+        hts.hts_ppo_terms(*x, count, 0.2, True, out[0])
+        assert selftest(*(a.data_ptr() for a in x), count, 0.2, out[1].data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+        torch.cuda.synchronize()
+        assert np.array_equal(out[0].cpu().numpy().view(np.int32), out[1].cpu().numpy().view(np.int32)), count
