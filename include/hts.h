@@ -200,9 +200,10 @@ hts_status hts_policy_gradient(hts_ctx *ctx, const uint8_t *obs, const int32_t *
  *   out3[1] = (1/count) sum (returns_i - values_i)^2         value loss J_V
  *   out3[2] = (1/count) sum entropy_i                        the term Eq. 4 weights by alpha
  *   logp, values, entropy, returns  DEVICE f32 [count];  out3 DEVICE f32 [3]
- * Summed in double precision in an order that depends on count alone.  Uses a small
- * table inside the library: calls on one device must be ordered (one stream, or
- * events between streams), not concurrent.  Errors: INVALID_ARG, CUDA.            */
+ * Summed in double precision in an order that depends on count and on whether all
+ * inputs are 16-byte aligned.  Uses a small table inside the library: calls on one
+ * device must be ordered (one stream, or events between streams), not concurrent.
+ * Errors: INVALID_ARG, CUDA.                                                       */
 hts_status hts_a2c_terms(const float *logp, const float *values, const float *entropy,
                          const float *returns, int64_t count, float *out3, void *cuda_stream);
 
@@ -216,7 +217,8 @@ hts_status hts_a2c_terms(const float *logp, const float *values, const float *en
  *   out4[2] = (1/count) sum entropy_i
  *   out4[3] = fraction of samples with |rho_i - 1| > clip
  *   all inputs DEVICE f32 [count]; out4 DEVICE f32 [4]; clip > 0.
- * Summation, ordering and the non-concurrency rule as for hts_a2c_terms.            */
+ * Summation and the non-concurrency rule as for hts_a2c_terms; with normalize_advantages
+ * the order also depends on whether the device has room for a cluster of 16 blocks.  */
 hts_status hts_ppo_terms(const float *logp_new, const float *logp_old, const float *values,
                          const float *entropy, const float *advantages, const float *returns,
                          int64_t count, float clip, int32_t normalize_advantages, float *out4,

@@ -7,7 +7,8 @@
 // HBM-bound (16 to 28 bytes per transition).  Each block sums a contiguous range in double precision in a
 // fixed order (thread-strided float4 loads, shuffle tree, warp order), writes its partial and takes a
 // ticket; the block that draws the last ticket adds the partials in a fixed order.  The grid is a
-// function of the count alone, so the result does not depend on timing or on the device's load.
+// function of the count alone; the order of the sums depends besides on whether the inputs are 16-byte aligned and, for
+// standardised terms, on whether the device has room for a cluster.  It depends neither on timing nor on the device's load.
 #include <cmath>
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -395,20 +396,38 @@ __global__ void __launch_bounds__(kClusterThreads, 1) terms_cluster_kernel(const
     }
 }
 
+// A part of a device may have no room for the largest cluster.  Asked once per device.
+cudaError_t terms_cluster_fits(bool* fits)
+{
+    static std::atomic<int> known[kDeviceSlots];         // 1: it fits, 2: it does not
+    std::atomic<int>& k = known[device_slot()];
+    if (!k.load(std::memory_order_acquire)) {
+        static OncePerDevice allowed;
+        cudaError_t e = allow_shared(terms_cluster_kernel, allowed);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(terms_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kClusterMost); cfg.blockDim = dim3(kClusterThreads); cfg.dynamicSmemBytes = (size_t)kClusterHolds * 24;
+        cudaLaunchAttribute size;
+        size.id = cudaLaunchAttributeClusterDimension;
+        size.val.clusterDim.x = kClusterMost; size.val.clusterDim.y = size.val.clusterDim.z = 1;
+        cfg.attrs = &size; cfg.numAttrs = 1;
+        int clusters = 0;
+        e = cudaOccupancyMaxActiveClusters(&clusters, terms_cluster_kernel, &cfg);
+        if (e != cudaSuccess && e != cudaErrorInvalidClusterSize && e != cudaErrorLaunchOutOfResources) return e;
+        if (e != cudaSuccess) cudaGetLastError();
+        k.store(e == cudaSuccess && clusters > 0 ? 1 : 2, std::memory_order_release);
+    }
+    *fits = k.load(std::memory_order_acquire) == 1;
+    return cudaSuccess;
+}
+
 // lost: without the copies, as if none of them landed (self-test).
 cudaError_t launch_terms_cluster(const PpoOp<false>& op, int count, cudaStream_t s, bool lost = false)
 {
     int ranks = 1;
     while (ranks < kClusterMost && ranks * kClusterEach < count) ranks *= 2;
     const int per_block = ((count + ranks - 1) / ranks + 3) / 4 * 4;
-    static OncePerDevice allowed, sized;
-    cudaError_t e = allow_shared(terms_cluster_kernel, allowed);
-    std::atomic<bool>& done = sized[device_slot()];
-    if (e == cudaSuccess && !done.load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(terms_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e == cudaSuccess) done.store(true, std::memory_order_release);
-    }
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)ranks); cfg.blockDim = dim3(kClusterThreads); cfg.dynamicSmemBytes = (size_t)per_block * 24; cfg.stream = s;
     cudaLaunchAttribute attr[2];
@@ -435,7 +454,7 @@ extern "C" hts_status hts_a2c_terms(const float* logp, const float* values, cons
 namespace hts {
 namespace {
 
-enum class TermsForm { ByCount, ClusterLost };
+enum class TermsForm { ByCount, TwoLaunches, ClusterLost };
 
 hts_status ppo_terms(const float* logp_new, const float* logp_old, const float* values, const float* entropy, const float* advantages,
                      const float* returns, int64_t count, float clip, int32_t normalize_advantages, float* out4, void* cuda_stream, TermsForm form)
@@ -446,9 +465,16 @@ hts_status ppo_terms(const float* logp_new, const float* logp_old, const float* 
     const bool vec = all_aligned16({logp_new, logp_old, values, entropy, advantages, returns});
     const PpoOp<false> op{logp_new, logp_old, values, entropy, advantages, returns, out4, (double)clip, normalize_advantages != 0, vec};
     if (!normalize_advantages) return launch_sums(op, (long long)count, s);
-    if (vec && count <= kClusterMost * kClusterHolds) {
-        if (launch_terms_cluster(op, (int)count, s, form == TermsForm::ClusterLost) == cudaSuccess) { note_launch(); return HTS_OK; }
-        cudaGetLastError();                              // a part of a device may have no room for the cluster: two launches
+    if (vec && count <= kClusterMost * kClusterHolds && form != TermsForm::TwoLaunches) {
+        bool fits = false;
+        HTS_CUDA(terms_cluster_fits(&fits));
+        if (fits) {
+            const cudaError_t e = launch_terms_cluster(op, (int)count, s, form == TermsForm::ClusterLost);
+            if (e == cudaSuccess) { note_launch(); return HTS_OK; }
+            // the current context may hold less of the device than the one that was asked
+            if (e != cudaErrorInvalidClusterSize && e != cudaErrorLaunchOutOfResources) return cuda_fail(e, "terms_cluster_kernel");
+            cudaGetLastError();
+        }
     }
     const hts_status st = launch_sums(AdvStatsOp{advantages, all_aligned16({advantages})}, (long long)count, s);
     if (st != HTS_OK) return st;
@@ -470,11 +496,14 @@ extern "C" hts_status hts_ppo_terms(const float* logp_new, const float* logp_old
                           hts::TermsForm::ByCount);
 }
 
-// The standardised means by the cluster without its copies, for tests; not declared in hts.h.
+// For tests, not declared in hts.h.  The standardised means by two launches, as where the cluster does not fit, or (`lost`) by the
+// cluster without its copies.
 extern "C" hts_status hts_ppo_terms_selftest(const float* logp_new, const float* logp_old, const float* values, const float* entropy,
-                                             const float* advantages, const float* returns, int64_t count, float clip, float* out4, void* cuda_stream)
+                                             const float* advantages, const float* returns, int64_t count, float clip, int32_t lost, float* out4,
+                                             void* cuda_stream)
 {
-    return hts::ppo_terms(logp_new, logp_old, values, entropy, advantages, returns, count, clip, 1, out4, cuda_stream, hts::TermsForm::ClusterLost);
+    return hts::ppo_terms(logp_new, logp_old, values, entropy, advantages, returns, count, clip, 1, out4, cuda_stream,
+                          lost ? hts::TermsForm::ClusterLost : hts::TermsForm::TwoLaunches);
 }
 
 // ---- the learner's parameter update (Section 4.1 "Delayed gradient", Eq. 5) ---------------------------------
