@@ -260,6 +260,7 @@ head_backward_kernel(const float* __restrict__ logits, const float* __restrict__
 //   part [range][A + 2][513]
 constexpr size_t kHeadRanges = 40;
 constexpr int kHeadTile = 11;                            // outputs per block
+constexpr int kHeadLeast = 16;                           // samples of a range, at least
 __global__ void __launch_bounds__(256)
 head_wgrad_kernel(const float* __restrict__ dhead, const float* __restrict__ h, const bf16* __restrict__ dh, size_t dh_plane,
                   int n, int A, int per_range, float* __restrict__ part)
@@ -314,10 +315,12 @@ struct ReduceParams {
     int n;
     hts_grads out;
 };
-// One kernel less while there are few samples.  Gradient without its forward pass, us, here / in a kernel of their own: 5 samples
-// 52.4 / 55.1, 40 60.9 / 64.6, 64 66.1 / 69.3, 80 71.3 / 72.6, 100 79.7 / 78.5, 160 111 / 100.
+// One kernel less while there are few samples.  Gradient of 84 x 84 x 4 frames, us, here / in a kernel of their own, with 2, 6, 18 and 32
+// actions: 40 samples 97 / 101, 97 / 102, 99 / 105, 100 / 106; 80 samples 125 / 128, 126 / 129, 126 / 131, 127 / 131; 88 134 / 134, 134 / 136,
+// 135 / 137, 136 / 137; 112 the same within 1 %; 128 160 / 153, 161 / 155, 162 / 156, 163 / 156.
 constexpr int kHeadsInReduce = 80;
-constexpr int kTurnFloats = 4096;                        // eight blocks on an SM
+constexpr int kTurnFloats = 4096;
+static_assert((kHeadsInReduce + 3 * kHeadLeast) / kHeadLeast * 256 <= kTurnFloats, "a sum's chains");
 // Sixteen terms in flight.
 template <class Term>
 __device__ __forceinline__ float sum_terms(int lo, int hi, Term term)
@@ -334,8 +337,9 @@ __device__ __forceinline__ float sum_terms(int lo, int hi, Term term)
 }
 // Blocks 0..511 turn one row of the dense gradient each into the caller's column order (c * P3 + pixel): written by the
 // contraction itself, 4-byte pieces P3 apart cost it 20 us.  The others sum, four threads of a block (64 apart) to a sum: a quarter
-// of the ranges each, then the quarters in order: gradient of 512 frames of 72 x 96 x 16 260 -> 244 us, of 40 68 -> 64, of 80 of 84 x 84 x 4
-// 72.3 -> 71.3 (one thread to a sum waited for up to 148 ranges, sixteen at a time).
+// of the ranges each, then the quarters in order: gradient without its forward pass of 512 frames of 72 x 96 x 16 260 -> 241 us, of 40 68 -> 64,
+// of 80 of 84 x 84 x 4 72.3 -> 71.3 (one thread to a sum waited for up to 148 ranges, sixteen at a time).  The heads' sums come first:
+// with their blocks last a gradient of 80 takes 131.5 us instead of 129.2.
 __global__ void __launch_bounds__(256) reduce_kernel(const ReduceParams p)
 {
     __shared__ float s_row[kTurnFloats];
@@ -365,7 +369,13 @@ __global__ void __launch_bounds__(256) reduce_kernel(const ReduceParams p)
     int ranges = 0, ho = -1, hk = 0;
     size_t stride = 0;
     float scale = 1.f;
-    if (i < n3) {                                        // [tap pair][tap of the pair, c][o]
+    if (i < nh) {                                        // first: with the longest chains of loads
+        ho = i / 513; hk = i - ho * 513;
+        src = p.head + i; ranges = p.rh; stride = (size_t)nh;
+        if (ho == p.A + 1) dst = hk < 512 ? p.out.fc_b + hk : nullptr;
+        else if (hk == 512) dst = ho < p.A ? p.out.pi_b + ho : p.out.v_b;
+        else dst = ho < p.A ? p.out.pi_w + ho * 512 + hk : p.out.v_w + hk;
+    } else if ((i -= nh) < n3) {                         // [tap pair][tap of the pair, c][o]
         const int gi = i >> 13, e = i & 8191, m = e >> 6, o = e & 63, b = m >> 6, c = m & 63;
         const int tap = gi < 4 ? 2 * gi + b : 7 + b;
         src = p.c3 + gi * p.g3 + e; ranges = gi == 4 ? p.r3_last : p.r3; stride = 8192;
@@ -381,33 +391,57 @@ __global__ void __launch_bounds__(256) reduce_kernel(const ReduceParams p)
         const int c = k >> 4, uy = (k >> 2) & 3, ux = k & 3, dy = tap >> 1, dx = tap & 1;
         src = p.c1 + gi * p.g1 + e; ranges = p.r1; stride = 4096; scale = 1.0f / 255.0f;
         if (c < p.C) dst = p.out.conv1_w + ((o * p.C + c) * 8 + 4 * dy + uy) * 8 + 4 * dx + ux;
-    } else if ((i -= n1) < nh) {
-        ho = i / 513; hk = i - ho * 513;
-        src = p.head + i; ranges = p.n > 0 ? p.n : p.rh; stride = (size_t)nh;
-        if (ho == p.A + 1) dst = hk < 512 ? p.out.fc_b + hk : nullptr;
-        else if (hk == 512) dst = ho < p.A ? p.out.pi_b + ho : p.out.v_b;
-        else dst = ho < p.A ? p.out.pi_w + ho * 512 + hk : p.out.v_w + hk;
-    } else if ((i -= nh) < 64) {
+    } else if ((i -= n1) < 64) {
         src = p.b3 + i; ranges = p.r3; stride = 64; dst = p.out.conv3_b + i;
     } else if (i < 128) {
         src = p.b2 + i - 64; ranges = p.r2; stride = 64; dst = p.out.conv2_b + i - 64;
     } else if (i < 160) {
         src = p.b1 + i - 128; ranges = p.r1; stride = 32; dst = p.out.conv1_b + i - 128;
     }
-    const int part = threadIdx.x >> 6, lo = ranges * part / 4, hi = ranges * (part + 1) / 4;
-    float acc = 0.f;
-    if (dst) {
-        if (ho < 0 || p.n == 0) acc = sum_terms(lo, hi, [&](int r) { return src[(size_t)r * stride]; });
-        else if (ho == p.A + 1) acc = sum_terms(lo, hi, [&](int r) {
-            const bf16* g = p.dh + (size_t)r * 512 + hk;
-            return x3_sum(__bfloat162float(g[0]), __bfloat162float(g[p.dh_plane]) + __bfloat162float(g[2 * p.dh_plane]));
-        });
-        else if (hk == 512) acc = sum_terms(lo, hi, [&](int r) { return p.dhead[(size_t)r * (p.A + 1) + ho]; });
-        else acc = sum_terms(lo, hi, [&](int r) { return p.dhead[(size_t)r * (p.A + 1) + ho] * p.h[(size_t)r * 512 + hk]; });
-    }
-    s_row[threadIdx.x] = acc;
+    const int part = threadIdx.x >> 6, t = threadIdx.x & 63;
+    const bool samples = ho >= 0 && p.n > 0;             // of this sum, not of its block
+    if (dst && samples) {
+        // As head_wgrad_kernel adds: chains of every fourth sample of kHeadLeast, products not rounded before they are added.
+        constexpr int IN_FLIGHT = 2, EACH = kHeadLeast / 4;      // ranges; a chain's samples
+#pragma unroll 1
+        for (int q = 0; q * kHeadLeast < p.n; q += IN_FLIGHT) {
+            float2 v[IN_FLIGHT * EACH];
+#pragma unroll
+            for (int k = 0; k < IN_FLIGHT * EACH; ++k) {
+                const int r = q * kHeadLeast + 4 * k + part;
+                v[k] = make_float2(0.f, 0.f);
+                if (r >= p.n) continue;
+                if (ho == p.A + 1) {
+                    const bf16* g = p.dh + (size_t)r * 512 + hk;
+                    v[k] = make_float2(1.f, x3_sum(__bfloat162float(g[0]), __bfloat162float(g[p.dh_plane]) + __bfloat162float(g[2 * p.dh_plane])));
+                } else
+                    v[k] = make_float2(p.dhead[(size_t)r * (p.A + 1) + ho], hk == 512 ? 1.f : p.h[(size_t)r * 512 + hk]);
+            }
+#pragma unroll
+            for (int j = 0; j < IN_FLIGHT; ++j) {
+                float acc = 0.f;
+#pragma unroll
+                for (int k = 0; k < EACH; ++k) acc = fmaf(v[j * EACH + k].x, v[j * EACH + k].y, acc);
+                s_row[(q + j) * 256 + threadIdx.x] = acc;
+            }
+        }
+    } else
+        s_row[threadIdx.x] = dst ? sum_terms(ranges * part / 4, ranges * (part + 1) / 4, [&](int r) { return src[(size_t)r * stride]; }) : 0.f;
     __syncthreads();
-    if (dst && threadIdx.x < 64) *dst = ((s_row[threadIdx.x] + s_row[64 + threadIdx.x]) + (s_row[128 + threadIdx.x] + s_row[192 + threadIdx.x])) * scale;
+    if (!dst || threadIdx.x >= 64) return;
+    auto four = [&](int q) { const float* a = s_row + q * 256 + t; return (a[0] + a[64]) + (a[128] + a[192]); };
+    float sum = four(0);
+    if (samples) {                                       // the same quarters as of partial sums of kHeadLeast samples
+        const int chains = (p.n + kHeadLeast - 1) / kHeadLeast;
+        float q4[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            q4[q] = 0.f;
+            for (int r = chains * q / 4; r < chains * (q + 1) / 4; ++r) q4[q] += four(r);
+        }
+        sum = (q4[0] + q4[1]) + (q4[2] + q4[3]);
+    }
+    *dst = sum * scale;
 }
 
 inline unsigned nblk(size_t total, int th) { return (unsigned)((total + th - 1) / th); }
@@ -672,7 +706,7 @@ hts_status x3_gradient(X3State* t, const RefWeights& w, const RefWorkspace& ws, 
         note_launch();
     }
     int per_range = (n + (int)kHeadRanges - 1) / (int)kHeadRanges;
-    if (per_range < 16) per_range = 16;
+    if (per_range < kHeadLeast) per_range = kHeadLeast;
     const int rh = (n + per_range - 1) / per_range;
     if (n > kHeadsInReduce) {
         HTS_CUDA(launch_pdl(head_wgrad_kernel, dim3(8, rh, nblk(g.A + 2, kHeadTile)), dim3(256), 0, s, t->dhead, ws.h, t->dh, ph, n, g.A, per_range,
