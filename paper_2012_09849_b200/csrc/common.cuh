@@ -128,7 +128,7 @@ struct RefWeights {            // fp32 device copies in PyTorch layouts
 };
 // Rows of one channel: row y is at (y % phases) * phase + (y / phases) * pitch.  A convolution of stride s reads inputs of
 // one phase or of s of them.
-struct RowLayout { int pitch, phases, phase, chan; };    // elements; chan: between channels
+struct RowLayout { int pitch, phases, phase, chan; };    // one or two phases; the others in elements; chan: between channels
 inline RowLayout rows_dense(int H, int W) { return {W, 1, 0, H * W}; }
 // Rows of an odd number of 16-byte pieces: eight of them start in eight different sixteenths of the shared-memory banks.
 inline RowLayout rows_strips(int H, int W, int phases)

@@ -35,10 +35,13 @@ __device__ __forceinline__ size_t frame_of(const ConvParams& p, int e)
     if ((unsigned)sl >= (unsigned)p.pool) { atomicCAS(p.status, 0, kStatusBadSlot); return 0; }
     return (size_t)sl;
 }
-// Where the inputs of output row i start, and its filter row u relative to that; where output row i is.
-__device__ __forceinline__ int x_row(const ConvParams& p, int i) { return i * (p.s / p.xl.phases) * p.xl.pitch; }
-__device__ __forceinline__ int x_tap(const ConvParams& p, int u) { return u % p.xl.phases * p.xl.phase + u / p.xl.phases * p.xl.pitch; }
-__device__ __forceinline__ int y_row(const ConvParams& p, int i) { return i % p.yl.phases * p.yl.phase + i / p.yl.phases * p.yl.pitch; }
+// Where the inputs of output row i start, and its filter row u relative to that; where output row i is.  Divisions by one or two
+// phases as shifts: a tile's block does them for every input that it looks up (step of one 84 x 84 x 4 frame that allocates nothing 47.3 us
+// with divisions, 45.3).
+__device__ __forceinline__ int x_row(const ConvParams& p, int i) { return i * (p.s >> (p.xl.phases - 1)) * p.xl.pitch; }
+__device__ __forceinline__ int row_at(const RowLayout& l, int y) { return (y & (l.phases - 1)) * l.phase + (y >> (l.phases - 1)) * l.pitch; }
+__device__ __forceinline__ int x_tap(const ConvParams& p, int u) { return row_at(p.xl, u); }
+__device__ __forceinline__ int y_row(const ConvParams& p, int i) { return row_at(p.yl, i); }
 // Where pixel (i, x) of row e starts in the planes.
 __device__ __forceinline__ size_t plane_row(const ConvParams& p, int e, int i, int x)
 {
