@@ -352,11 +352,11 @@ hts_status launch_conv(const ConvParams& p, const StripMaps* maps, cudaStream_t 
 }
 
 // h[e,o] = relu(b[o] + sum over lanes l of (chain of f = l, l+32, l+64, ...)), the 32 chains added as a binary tree
-// over the lane number (halves first), for few rows (and callers without tensor maps; fc_f32.cu takes the others).  A warp owns
+// over the lane number (halves first), for few rows (and callers without tensor maps, layers of 64 features; fc_f32.cu takes the others).  A warp owns
 // TE rows x TO outputs and lane l runs chain l of all of them: both operands are contiguous across the lanes, so neither needs a
 // transposition, and one transposing reduction closes the tree (at each level a lane keeps half of its values and gets its partner's
-// share of them).  The block's rows of x and w go through a ring in shared memory, COLS columns at a time.  Bound: the latency of the
-// weights: narrow tiles, deep ring.
+// share of them).  The block's rows of x and w go through a ring in shared memory, COLS columns at a time.  Bound: few rows by the latency
+// of the weights: narrow tiles, deep ring; many by shared memory and the fp32 pipes: 8 x 8 per warp.
 template <int TE, int TO, int WE, int WO, int STAGES, int COLS>
 __global__ void __launch_bounds__(32 * WE * WO)
 fc_chain_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ b,
@@ -368,7 +368,7 @@ fc_chain_kernel(const float* __restrict__ x, const float* __restrict__ w, const 
     const int we = warp % WE, wo = warp / WE;
     const int e0 = (blockIdx.y * WE + we) * TE, o0 = (blockIdx.x * WO + wo) * TO;
     pdl_wait();
-    pdl_trigger();
+    if constexpr (TE < 8) pdl_trigger();
     f32x2 acc[TE][TO / 2];
 #pragma unroll
     for (int i = 0; i < TE; ++i)
@@ -468,7 +468,8 @@ hts_status launch_fc_chain(const float* x, const float* w, const float* b, float
 // The form goes by the blocks (128 per 16 rows) of the SM that has most of them, k.  The fewer it has, the more each must have in
 // flight and the less often its warps may meet: stages of 512 columns, three deep at k = 1 and two at k = 2 (both fill the shared
 // memory), of 128 columns above (step at k = 1 / 2 / 3, 3136 features: 45.4 / 52.4 / 71.5 us with the first, 45.8 / 48.1 / 69.4 with the second,
-// 47.7 / 50.7 / 64.3 with the third).  From k = 3 on boxes are faster (the layer alone, this / boxes: 16 rows 9.8 / 12.1 us, 32 rows
+// 47.7 / 50.7 / 64.3 with the third).  Where there are no boxes, one wide block per SM takes as long as five narrow ones (64 features, the
+// layer of 2048 rows: 35 us narrow, 21 wide).  From k = 3 on boxes are faster (the layer alone, this / boxes: 16 rows 9.8 / 12.1 us, 32 rows
 // 11.7 / 12.2, 40 rows 15.8 / 12.3).
 hts_status launch_fc(const float* x, const float* w, const float* b, float* h, int n, int F, const RefWorkspace& ws, int* status, cudaStream_t s)
 {
@@ -477,7 +478,8 @@ hts_status launch_fc(const float* x, const float* w, const float* b, float* h, i
     if (k == 1) return launch_fc_chain<4, 4, 4, 1, 3, 512>(x, w, b, h, n, F, s);
     if (k == 2) return launch_fc_chain<4, 4, 4, 1, 2, 512>(x, w, b, h, n, F, s);
     const hts_status st = ws.maps ? launch_fc_lanes({b, h, n, F, ws.row0, status}, ws.maps->fc, s) : HTS_ERR_UNSUPPORTED;
-    return st != HTS_ERR_UNSUPPORTED ? st : launch_fc_chain<4, 4, 4, 1, 4, 128>(x, w, b, h, n, F, s);
+    if (st != HTS_ERR_UNSUPPORTED) return st;
+    return k > 5 ? launch_fc_chain<8, 8, 4, 2, 4, 64>(x, w, b, h, n, F, s) : launch_fc_chain<4, 4, 4, 1, 4, 128>(x, w, b, h, n, F, s);
 }
 
 __global__ void __launch_bounds__(256) dense_rows_kernel(const float* __restrict__ x, const RowLayout l, int H, int W, size_t total, float* __restrict__ out)
