@@ -381,6 +381,10 @@ bool make_strip_maps(const Geometry& g, const RefWorkspace& ws, size_t frames, S
 //     5 x 8: 11.5 + 8.2, where that saves a round (step of 50 frames of 72 x 96 x 16 73 -> 63 us, of 100 116 -> 106; 80: 85 / 98)
 //   second   4 x 2  7.4, 10.9, 14.9: 7.4 + 3.7     a row x 2  11.3, 18.0, 25.5, 32.9: 11.3 + 7.0     a row x 4  16.7, 29.5, .. 56 (4), .. 107 (8): 16.7 + 12.5
 //   third    4 x 2  8.6, 11.8, .. 21.2 (4): 8.6 + 4.2     a row x 2  10.2, 15.6, .. 27.2 (4), 44.7 (7), 80 (13): 10.1 + 5.8
+// Rows that leave strips half empty are faster in 128 x 64 tiles once there are many: 49 + 26.5 us for each more per SM in the second
+// layer, 51 + 28 in the third.  The lines above are of full strips; of the forms for wider rows and of many blocks 18.5 + 15.2 (row x 4), 12.5 + 7.8 and 11 + 7.1
+// (row x 2), 7.4 + 4.6 and 8.6 + 5.2 (4 x 2).  Second / third layer, us, tiles / strips: 2048 frames of 52 x 52 x 4 (rows of 5 and 3
+// pixels) 99 / 118, 52 / 60; 512 of 128 x 128 x 4 (14 and 12) 177 / 202, 132 / 148; of 144 x 144 x 4 (16 and 14) 200 / 224, 191 / 178.
 // Few2 and Few3 have four stages of 8 and 16 channels (eight of 4 and 8 before: step of 16 32.9 us, now 32.3).
 // (the tiles of policy_ref.cu: 12 to 16 at 16 frames, 26 / 31 / 22 at 80, 150 / 151 / 101 at 1024).  A small tile's block has a short
 // chain of sums, a large one more of them for each load.
@@ -402,13 +406,19 @@ hts_status launch_conv_strip(const ConvParams& p, const StripMaps* maps, cudaStr
         const bool narrow = p.Wo <= 9;
         const int px = narrow ? 9 : 10;
         const int few = 74 + 37 * (strip_blocks(p, 4, 4) - 1), some = 113 + 70 * (strip_blocks(p, px, 4) - 1), many = 167 + 125 * (strip_blocks(p, px, 8) - 1);
+        const int strips = few >= many && some >= many ? (narrow ? many : 185 + 152 * (strip_blocks(p, px, 8) - 1))
+                         : few >= some ? (narrow ? some : 125 + 78 * (strip_blocks(p, px, 4) - 1)) : 74 + 46 * (strip_blocks(p, 4, 4) - 1);
+        if (conv_tiles_large(p) && 490 + 265 * (conv_large_tiles(p) - 1) < strips) return HTS_ERR_UNSUPPORTED;
         if (few >= many && some >= many) st = narrow ? launch_strip<Many2n>(p, &maps->many2, s) : launch_strip<Many2w>(p, &maps->many2, s);
         if (st == HTS_ERR_UNSUPPORTED && few >= some) st = narrow ? launch_strip<Some2n>(p, &maps->some2, s) : launch_strip<Some2w>(p, &maps->some2, s);
         if (st == HTS_ERR_UNSUPPORTED) st = launch_strip<Few2>(p, &maps->few2, s);
         return st == HTS_ERR_UNSUPPORTED ? launch_strip<Thin2>(p, &maps->thin2, s) : st;
     }
     const bool narrow = p.Wo <= 7;
-    if (86 + 42 * (strip_blocks(p, 4, 4) - 1) >= 101 + 58 * (strip_blocks(p, narrow ? 7 : 8, 4) - 1))
+    const int few = 86 + 42 * (strip_blocks(p, 4, 4) - 1), row_blocks = strip_blocks(p, narrow ? 7 : 8, 4), some = 101 + 58 * (row_blocks - 1);
+    const int strips = few < some ? 86 + 52 * (strip_blocks(p, 4, 4) - 1) : narrow ? some : 110 + 71 * (row_blocks - 1);
+    if (conv_tiles_large(p) && 510 + 280 * (conv_large_tiles(p) - 1) < strips) return HTS_ERR_UNSUPPORTED;
+    if (few >= some)
         st = narrow ? launch_strip<Some3n>(p, &maps->some3, s) : launch_strip<Some3w>(p, &maps->some3, s);
     if (st == HTS_ERR_UNSUPPORTED) st = launch_strip<Few3>(p, &maps->few3, s);
     return st == HTS_ERR_UNSUPPORTED ? launch_strip<Thin3>(p, &maps->thin3, s) : st;

@@ -335,20 +335,19 @@ hts_status launch_conv_tile(const ConvParams& p, cudaStream_t s)
 }
 
 // A form takes a time that steps with the blocks of the SM that has most (conv2, us at 1, 2, 3 ... per SM: latency form 15, 19, 23,
-// 27; 64 x 32 tiles 25, 35, 48, 62, 74).  The latency form pays up to three blocks per SM, two where it converts frames (17 against
-// 15).  Large tiles (256 x 32) only take many unaligned frames: one costs as much as 2.5 small ones and 0.7 more for its start.
+// 27; 64 x 32 tiles 25, 35, 48, 62, 74; 128 x 64 49, 75, 101).  The latency form pays up to three blocks per SM, two where it converts
+// frames (17 against 15).  Large tiles: where rows leave strips half empty or do not fit (second / third layer of 200 frames of
+// 48 x 1024 x 4 175 / 103 us, 259 / 144 in 64 x 32 tiles), and many unaligned frames.
 template <typename TIn>
 hts_status launch_conv(const ConvParams& p, const StripMaps* maps, cudaStream_t s)
 {
     const hts_status strips = launch_conv_strip(p, maps, s);
     if (strips != HTS_ERR_UNSUPPORTED) return strips;
     constexpr bool U8 = std::is_same<TIn, uint8_t>::value;
-    const size_t px = (size_t)p.n * p.Ho * p.Wo, sms = (size_t)device_sm_count(device_slot());
-    auto per_sm = [&](size_t tile_px, size_t tile_oc) { return ((px + tile_px - 1) / tile_px * (p.O / tile_oc) + sms - 1) / sms; };
-    if (per_sm(kSmallPx, kSmallOc) <= (U8 ? 2 : 3)) return launch_conv_small<TIn>(p, s);
-    if constexpr (U8)
-        if (2 * per_sm(64, 32) > 5 * per_sm(256, 32) + 1) return launch_conv_tile<TIn, 8, 8, 4, 1, 16, 4>(p, s);
-    return launch_conv_tile<TIn, 4, 4, 2, 2, 32, 5>(p, s);
+    if (conv_tiles(p, kSmallPx, kSmallOc) <= (U8 ? 2 : 3)) return launch_conv_small<TIn>(p, s);
+    if (!conv_tiles_large(p)) return launch_conv_tile<TIn, 4, 4, 2, 2, 32, 5>(p, s);
+    if constexpr (U8) return launch_conv_tile<TIn, 8, 8, 4, 1, 16, 4>(p, s);
+    else return launch_conv_tile<TIn, 8, 8, 2, 2, 16, 4>(p, s);
 }
 
 // h[e,o] = relu(b[o] + sum over lanes l of (chain of f = l, l+32, l+64, ...)), the 32 chains added as a binary tree

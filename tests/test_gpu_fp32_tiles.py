@@ -1,4 +1,4 @@
-"""fp32 dense layers of few features, which run in tiles."""
+"""fp32 layers in tiles: where rows leave strips half empty or are too wide for them, and dense layers of few features."""
 import dataclasses
 
 import numpy as np
@@ -58,3 +58,15 @@ def test_a_dense_layer_of_few_features(n):
 
 def test_a_quarter_of_the_features_takes_no_longer():
     assert layers_us(36, 36, 2048)["fc"] <= 1.1 * layers_us(44, 44, 2048)["fc"]
+
+
+# the second layer's rows of 5 pixels in strips of 9, of 12, 14 and 16 in strips of 10, the third's of 3 in 4 and of 12 in 8; rows too wide; ragged ends
+@pytest.mark.parametrize("C,H,W,n", [(4, 52, 52, 2047), (1, 112, 112, 515), (4, 128, 128, 512), (1, 144, 144, 509), (4, 48, 1024, 200)])
+def test_layers_whose_strips_are_half_empty_or_do_not_fit(C, H, W, n):
+    check_bits(C, H, W, n)
+
+
+def test_rows_too_wide_for_strips_take_no_longer_for_their_outputs():
+    """504 outputs of each channel a frame in rows of 126 pixels, 372 in rows of 62."""
+    wide, fits = layers_us(48, 1024, 200)["conv2"], layers_us(64, 512, 256)["conv2"]
+    assert wide / (200 * 504) <= 1.25 * fits / (256 * 372)
