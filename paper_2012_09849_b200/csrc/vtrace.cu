@@ -45,7 +45,9 @@ struct VtraceParams {
 // columns [b*cols + cx*VEC, +VEC) (cols = 32/CY*VEC) and chunk w*CY + cy of the super-chunk.  Time is walked from the
 // end in super-chunks of W*CY*L rows.  Chunk boundaries, and with them every rounding, do not depend on CY or W.
 // ROOMY: as many registers as a block alone on its SM can have, so that all of a chunk's loads are in flight together (115 instead of
-// 93; 3.29 -> 2.73 us at 128 x 1024).  It pays while no SM has a second block: 512 x 8000 (two per SM) 28.9 / 29.3 us.
+// 93; 3.29 -> 2.73 us at 128 x 1024).  It pays for blocks of up to 16 warps while no SM has a second one: 512 x 8000 (two per SM)
+// 28.9 / 29.3 us.  Not for those of 8 warps, one to an SM at 4705 to 4736 columns (148 SMs): 256 / 1024 / 5000 x 4736 7.9 / 43.2 /
+// 227 us, ROOMY 8.2 / 44.1 / 231.
 template <int VEC, int L, int CY, int MAXW, bool MANY, bool ROOMY>
 __global__ void __launch_bounds__(32 * MAXW, ROOMY ? 1 : 0)
 vtrace_scan_kernel(const VtraceParams p)
@@ -191,10 +193,10 @@ hts_status launch_t(const VtraceParams& p, int sms, cudaStream_t s)
     const int cols = 32 / CY * VEC;
     const unsigned blocks = (unsigned)((p.N + cols - 1) / cols);
     const size_t smem = (size_t)2 * W * CY * cols * sizeof(float);
-    constexpr bool V1 = VEC == 1, M = V1 && MAXW * CY >= kManyChunks;
-    const bool many = M && W * CY >= kManyChunks, roomy = V1 && (int)blocks <= sms;
-    auto kernel = many ? (roomy ? vtrace_scan_kernel<VEC, L, CY, MAXW, M, V1> : vtrace_scan_kernel<VEC, L, CY, MAXW, M, false>)
-                       : (roomy ? vtrace_scan_kernel<VEC, L, CY, MAXW, false, V1> : vtrace_scan_kernel<VEC, L, CY, MAXW, false, false>);
+    constexpr bool M = VEC == 1 && MAXW * CY >= kManyChunks, R = VEC == 1 && MAXW >= 16;
+    const bool many = M && W * CY >= kManyChunks, roomy = R && (int)blocks <= sms;
+    auto kernel = many ? (roomy ? vtrace_scan_kernel<VEC, L, CY, MAXW, M, R> : vtrace_scan_kernel<VEC, L, CY, MAXW, M, false>)
+                       : (roomy ? vtrace_scan_kernel<VEC, L, CY, MAXW, false, R> : vtrace_scan_kernel<VEC, L, CY, MAXW, false, false>);
     HTS_CUDA(launch_pdl(kernel, dim3(blocks), dim3(32, W), smem, s, p));
     note_launch();
     return HTS_OK;
