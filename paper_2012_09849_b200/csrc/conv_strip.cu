@@ -236,6 +236,7 @@ conv_strip_kernel(const ConvParams p, const StripPlan t, const __grid_constant__
     for (int j = 0; j < PX; ++j)
 #pragma unroll
         for (int o = 0; o < OT / 2; ++o) acc[j][o] = 0;
+    pdl_wait();                                          // here, so that the waits' limit does not count the kernel before
 #pragma unroll 1
     for (int st = 0; st < stages; ++st) {
         const int slot = st % NST;
@@ -267,7 +268,6 @@ conv_strip_kernel(const ConvParams p, const StripPlan t, const __grid_constant__
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(freed + slot);
     }
-    pdl_wait();                                          // the kernel before may still read what this one writes
     strip_store<PX, OT, NC>(p, t, acc, k, q0 + ws * LG + g <= last, o_t, q0, last, OC, reinterpret_cast<float*>(s4));
 }
 

@@ -63,6 +63,7 @@ fc_lanes_kernel(const FcParams p, const __grid_constant__ CUtensorMap mx, const 
     for (int i = 0; i < TE / 2; ++i)
 #pragma unroll
         for (int j = 0; j < TO; ++j) acc[i][j] = 0;
+    pdl_wait();                                          // here, so that the waits' limit does not count the kernel before
 #pragma unroll 1
     for (int st = 0; st < stages; ++st) {
         const int slot = st % NST;
@@ -112,7 +113,6 @@ fc_lanes_kernel(const FcParams p, const __grid_constant__ CUtensorMap mx, const 
         }
         id += up ? len : 0;
     }
-    pdl_wait();                                          // the kernel before may still read what this one writes
     constexpr int LEFT = NV / 32;
     static_assert(LEFT >= 1 && TO % LEFT == 0, "a lane's results are of one row");
     const int e = e_base + we * TE + id / TO, o = o_base + wo * TO + id % TO;
