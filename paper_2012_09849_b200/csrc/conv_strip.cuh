@@ -19,6 +19,7 @@ struct ConvParams {
     int pool;
     int* status;
     bool w_vec, words;                  // weights 16-byte aligned; frames 4-byte aligned
+    bool y_rows;                        // outputs (or planes) are not one dense run of pixels per channel: a pixel's row is needed
     __nv_bfloat16* planes;              // optional second output: three bf16 planes of pixel-major rows (x3_gemm.cuh)
     size_t plane;
     int W_rows, P_rows;                 // its grid; 2 x 2 pixels per row when s2d

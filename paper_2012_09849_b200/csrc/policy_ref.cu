@@ -166,7 +166,7 @@ conv_tile_kernel(const ConvParams p)
     for (int q = 0; q < PXT; ++q) {
         const int px = blockIdx.x * PX + px_t + 32 * (q / 4) + q % 4;
         if (px >= total) continue;
-        const int e = px / P, r = px - e * P, i = r / p.Wo, x = r - i * p.Wo;
+        const int e = px / P, r = px - e * P, i = p.y_rows ? r / p.Wo : 0, x = r - i * p.Wo;
         float v[OT];
 #pragma unroll
         for (int j = 0; j < OT; ++j) {
@@ -285,7 +285,7 @@ conv_small_kernel(const ConvParams p, int ring)
     for (int q = 0; q < 2; ++q) {
         const int px = px0 + g8 + 8 * q;
         if (px >= total) continue;
-        const int e = px / P, r = px - e * P, i = r / p.Wo, x = r - i * p.Wo, o = o_base + o_t;
+        const int e = px / P, r = px - e * P, i = p.y_rows ? r / p.Wo : 0, x = r - i * p.Wo, o = o_base + o_t;
         float v[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -511,13 +511,13 @@ hts_status ref_forward(const Geometry& g, const RefWeights& w, const RefWorkspac
                      int W, int O, int k, int stride, int Ho, int Wo) {
         ConvParams p{};
         p.x = x; p.xl = xl; p.w = wt; p.wk = wk; p.b = b; p.y = y; p.yl = yl; p.n = n; p.frame0 = ws.row0; p.C = C; p.H = H; p.W = W; p.O = O; p.k = k; p.s = stride; p.Ho = Ho; p.Wo = Wo;
-        p.status = status; p.in_scale = 1.f; p.w_vec = ((uintptr_t)wt & 15) == 0; p.words = ((uintptr_t)x & 3) == 0;
+        p.status = status; p.in_scale = 1.f; p.w_vec = ((uintptr_t)wt & 15) == 0; p.y_rows = yl.pitch != Wo || yl.phases != 1; p.words = ((uintptr_t)x & 3) == 0;
         return p;
     };
     prof.begin(K_CONV1, s);
     ConvParams c1 = layer(obs, rows_dense(g.H, g.W), w.w1, w.w1k, w.b1, ws.a1, ws.l1, g.C, g.H, g.W, 32, 8, 4, g.H1, g.W1);
     c1.in_scale = 1.0f / 255.0f; c1.slots = ix.slots; c1.pool = ix.pool;
-    if (planes) { c1.planes = planes->a1; c1.plane = planes->p1; c1.s2d = true; c1.W_rows = (g.W1 + 1) / 2; c1.P_rows = (g.H1 + 1) / 2 * c1.W_rows; c1.early = planes->beside_conv1; }
+    if (planes) { c1.planes = planes->a1; c1.plane = planes->p1; c1.s2d = c1.y_rows = true; c1.W_rows = (g.W1 + 1) / 2; c1.P_rows = (g.H1 + 1) / 2 * c1.W_rows; c1.early = planes->beside_conv1; }
     st = launch_conv<uint8_t>(c1, nullptr, s);
     if (st != HTS_OK) return st;
     prof.end(K_CONV1, s);
