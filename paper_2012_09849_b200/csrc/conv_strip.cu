@@ -417,6 +417,8 @@ hts_status launch_conv_strip(const ConvParams& p, const StripMaps* maps, cudaStr
     const bool narrow = p.Wo <= 7;
     const int few = 86 + 42 * (strip_blocks(p, 4, 4) - 1), row_blocks = strip_blocks(p, narrow ? 7 : 8, 4), some = 101 + 58 * (row_blocks - 1);
     const int strips = few < some ? 86 + 52 * (strip_blocks(p, 4, 4) - 1) : narrow ? some : 110 + 71 * (row_blocks - 1);
+    // Rows of one pixel leave three quarters of a strip idle: 12.6, 16.8, 21, 25.5 us at 1, 2, 3, 4 blocks per SM, in 64 x 32 tiles 16.3 (2), 18.9 (3 and 4).
+    if (p.Wo == 1 && strip_blocks(p, 4, 4) >= 3) return HTS_ERR_UNSUPPORTED;
     if (conv_tiles_large(p) && 510 + 280 * (conv_large_tiles(p) - 1) < strips) return HTS_ERR_UNSUPPORTED;
     if (few >= some)
         st = narrow ? launch_strip<Some3n>(p, &maps->some3, s) : launch_strip<Some3w>(p, &maps->some3, s);

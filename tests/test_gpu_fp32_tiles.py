@@ -61,7 +61,8 @@ def test_a_quarter_of_the_features_takes_no_longer():
 
 
 # the second layer's rows of 5 pixels in strips of 9, of 12, 14 and 16 in strips of 10, the third's of 3 in 4 and of 12 in 8; rows too wide; ragged ends
-@pytest.mark.parametrize("C,H,W,n", [(4, 52, 52, 2047), (1, 112, 112, 515), (4, 128, 128, 512), (1, 144, 144, 509), (4, 48, 1024, 200)])
+@pytest.mark.parametrize("C,H,W,n", [(4, 52, 52, 2047), (1, 112, 112, 515), (4, 128, 128, 512), (1, 144, 144, 509), (4, 48, 1024, 200),
+                                     (4, 36, 36, 1183), (4, 36, 36, 1185), (1, 84, 36, 255)])      # the third's of one pixel: strips, tiles
 def test_layers_whose_strips_are_half_empty_or_do_not_fit(C, H, W, n):
     check_bits(C, H, W, n)
 
