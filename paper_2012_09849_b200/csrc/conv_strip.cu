@@ -223,8 +223,7 @@ conv_strip_kernel(const ConvParams p, const StripPlan t, const __grid_constant__
                 for (int f = lane; f < frames; f += 32)
                     tc::tma_load_5d(dst + f * t.X, &map, 0, rr0 - (e0 + f) * p.Ho, 0, st * CK, t.frame0 + e0 + f, full + slot);
         }
-        if (st < stages)                                 // given up: the copies in flight end before the block does
-            for (int i = st < NST ? 0 : st - NST; i < st; ++i) tc::mbar_wait_warp(full + i % NST, (i / NST) & 1, &abort_flag, p.status, 41);
+        if (st < stages) tc::let_copies_land();
         return;
     }
     const int ws = warp % WS, wo = warp / WS, g = lane % LG, o_t = (wo * (32 / LG) + lane / LG) * OT;
@@ -240,7 +239,10 @@ conv_strip_kernel(const ConvParams p, const StripPlan t, const __grid_constant__
 #pragma unroll 1
     for (int st = 0; st < stages; ++st) {
         const int slot = st % NST;
-        if (!tc::mbar_wait_warp(full + slot, (st / NST) & 1, &abort_flag, p.status, 42)) break;    // the barriers below are met all the same
+        if (!tc::mbar_wait_warp(full + slot, (st / NST) & 1, &abort_flag, p.status, 42)) {
+            tc::let_copies_land();                       // the outputs pass through the ring
+            break;                                       // strip_store's barriers are met all the same
+        }
         const float4* in = s4 + slot * STAGE;
         const float* w = reinterpret_cast<const float*>(in + STAGE - WCH) + o_t;
 #pragma unroll (U8 ? 1 : CK)

@@ -53,8 +53,7 @@ fc_lanes_kernel(const FcParams p, const __grid_constant__ CUtensorMap mx, const 
                 else tc::tma_load_2d(dst, &mw, c, o_base + r - RX, full + slot);
             }
         }
-        if (st < stages)                                 // given up: the copies in flight end before the block does
-            for (int i = st < NST ? 0 : st - NST; i < st; ++i) tc::mbar_wait_warp(full + i % NST, (i / NST) & 1, &abort_flag, p.status, 51);
+        if (st < stages) tc::let_copies_land();
         return;
     }
     const int we = warp % WE, wo = warp / WE;
@@ -67,7 +66,10 @@ fc_lanes_kernel(const FcParams p, const __grid_constant__ CUtensorMap mx, const 
 #pragma unroll 1
     for (int st = 0; st < stages; ++st) {
         const int slot = st % NST;
-        if (!tc::mbar_wait_warp(full + slot, (st / NST) & 1, &abort_flag, p.status, 52)) break;
+        if (!tc::mbar_wait_warp(full + slot, (st / NST) & 1, &abort_flag, p.status, 52)) {
+            tc::let_copies_land();
+            break;
+        }
         const float* xr = s_ring + slot * STAGE + we * TE * COLS + lane;
         const float* wr = s_ring + slot * STAGE + (RX + wo * TO) * COLS + lane;
         auto step = [&](int c) {

@@ -103,6 +103,14 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
     return ok;
 }
 
+// After a wait that gave up: copies that are still in flight get time to land (about a millisecond) before their shared memory is used
+// for something else, by this block or by the next.
+__device__ __forceinline__ void let_copies_land()
+{
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000) { }
+}
+
 // ---- TMA (tiled, 2-D, shared::cta destination of this CTA, completion on an mbarrier) ---------
 __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* map, int x, int y, uint64_t* bar)
 {

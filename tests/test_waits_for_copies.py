@@ -23,3 +23,13 @@ def branches(source, kernel):
 def test_the_limit_of_a_wait_does_not_count_the_kernel_before(source, kernel):
     for part in branches(source, kernel):
         assert 0 <= part.find("pdl_wait()") < part.find("mbar_wait_warp(")
+
+
+@pytest.mark.parametrize("source,kernel", KERNELS, ids=[k[1] for k in KERNELS])
+def test_copies_in_flight_land_before_a_warp_that_gave_up_goes_on(source, kernel):
+    """A wait after one that gave up ends at once, landed or not: what follows must be time, not a wait."""
+    copies, computes = branches(source, kernel)
+    assert "mbar_wait_warp(full" not in copies
+    assert copies.rstrip().endswith("if (st < stages) tc::let_copies_land();\n        return;")
+    gives_up = re.search(r"if \(!tc::mbar_wait_warp\(full[^{;]*\{\s*tc::let_copies_land\(\);\s*break;", computes)
+    assert gives_up and computes.count("mbar_wait_warp(") == 1
