@@ -91,7 +91,8 @@ struct LoadParams {
 };
 // One launch for all twelve tensors (a parameter update ends in one, so launches count: twelve copies and a packing pass
 // took 45 us).  Blocks 0..511 take one row of the dense layer each and turn it through shared memory, sixteen bytes in and two
-// channels of a pixel out at a time (10.3 -> 5.2 us for 84 x 84 x 4; four and two bytes before); the rest one element per thread.
+// channels of a pixel out at a time (four and two bytes before: 6.2 us for 84 x 84 x 4 and 10.3 for 128 x 128 x 4, calls in a row, now 4.1 and
+// 5.6); the rest one element per thread.
 __global__ void __launch_bounds__(256) load_fp32_kernel(const LoadParams p)
 {
     __shared__ __align__(16) float s_row[kPackFloats];

@@ -4,8 +4,8 @@
 // channels each.  The sums are those of the plain loop: one chain over (c, u, v) per output.  Of a filter row a strip needs
 // (PX - 1) s + k inputs instead of k PX gathered ones, so shared memory holds raw rows, filled by bulk copies of one warp (an
 // mbarrier per stage; all waits are bounded), and a thread reads 20 inputs and 16 weights for 144 multiply-adds (second layer)
-// where 8 x 8 tiles read 32 and 32 for 128.  Bound: the fp32 pipes (80 % busy while the sums run; 60 TFLOP/s of the 70 that packed
-// multiply-adds reach), then what a block spends on its first copies and its stores.  At 1024 observations of 84 x 84 x 4 the
+// where 8 x 8 tiles read 32 and 32 for 128.  Bound: the fp32 pipes (80 % busy while the sums run: 57 to 62 TFLOP/s of
+// the pipes' 72), then what a block spends on its first copies and its stores.  At 1024 observations of 84 x 84 x 4 the
 // three layers take 131 / 100 / 78 us, in gathered tiles 150 / 151 / 101.  All channels of a stage are one straight run of instructions,
 // so that the next channel's loads are under way during a channel's sums: with a loop over channels (first layer: filter rows) 133 /
 // 107 / 80, and 60.3 instead of 57.1 us for a step of 80.
@@ -38,7 +38,8 @@ struct Strip { int q, rr, sx, e, i; };  // of a thread: strip and row of the bat
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 // One filter row of one channel: a strip's inputs x times the row's weights w[tap][OC].  A packed multiply-add takes 2 clocks
 // of its scheduler if it shares an operand with the one before it and 3 if not (three pairs of registers, two banks), so the
-// weights stay while the pixels pass, there and back: 64 to 70 TFLOP/s, 58 to 62 with the input kept and the weights passing.
+// weights stay while the pixels pass, there and back: 64 to 70 TFLOP/s of multiply-adds
+// alone, 58 to 62 with the input kept and the weights passing.
 template <int KS, int S, int PX, int OT, int OC>
 __device__ __forceinline__ void strip_row(f32x2 (&acc)[PX][OT / 2], const float (&x)[((PX - 1) * S + KS + 3) / 4 * 4], const float* w)
 {

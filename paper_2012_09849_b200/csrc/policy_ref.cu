@@ -2,7 +2,7 @@
 // network of Appendix F.1 / F.2.  Every output is one chain of fp32 multiply-adds in a fixed order, whatever the
 // tile that computes it, so a row's bits do not depend on the batch around it.  A context's convolutions run in strips
 // (conv_strip.cu); the tiles here take what those do not: weights in the caller's layout (the step that allocates nothing),
-// frames that are not 16-byte aligned, rows too wide for shared memory.
+// frames that are not 16-byte aligned, rows too wide for shared memory or of a length that leaves strips half empty.
 #include <new>
 #include <type_traits>
 #include "common.cuh"
@@ -41,7 +41,7 @@ __device__ __forceinline__ float4 load4(const float* p, bool vec)
 // inputs and OC x KC weights per step into shared memory, one step ahead; a thread owns PXT pixels x OT channels.
 // Bound: no unit alone.  Inputs are gathered four bytes at a time, weights turned through registers in every block and chunk, and
 // shared memory reaches registers at 128 bytes per clock (a thread loads 4 (PXT + OT) bytes per PXT x OT multiply-adds): 28 to 44
-// TFLOP/s where strips reach 45 to 53 (first / second / third layer of 1024 observations 150 / 151 / 101 us, 133 / 107 / 80 in strips).
+// TFLOP/s where strips reach 47 to 54 (first / second / third layer of 1024 observations 150 / 151 / 101 us, 131 / 100 / 78 in strips).
 // A thread's pixels are runs of four, so a step's inputs are two 16-byte loads.
 template <typename TIn, int PXT, int OT, int WPX, int WO, int KC, int PER_SM>
 __global__ void __launch_bounds__(32 * WPX * WO, PER_SM)

@@ -258,12 +258,13 @@ x3_dgrad_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 // 128 rows: two stages of 64, or one of 128 (NB = 32, whose narrow products have two accumulators per thread).  The
 // first one of group 0 is a single stage, so that one thread's products run while the other waits for its accumulator
 // to be read.  One thread for both groups leaves the tensor core waiting (its instructions come 55 to 70 clocks apart):
-// weight gradients of conv3 / conv2 / conv1 / dense at n = 1024, 84 x 84: 52 / 48 / 43 / 33 us, 43 / 44 / 38 / 30 with two.
+// weight gradients of conv3 / conv2 / conv1 / dense at n = 1024, 84 x 84, in launches of their own: 52 / 48 / 43 / 33 us, 43 / 44 / 38 / 30
+// with two.
 // The sets of kind 0 also sum the columns of B (bias gradient).
 // Both operands have the contracted index along their rows (pixels), so tiles go from global memory to the tensor
 // core without a transposition; a tap is a row offset into the slab, and the two taps (or slabs) of a group are two
 // 64-row blocks of M at a free distance (the leading byte offset).  Tensor core: 208 clocks per 16 rows and group (56 for
-// frames); busy for 51 / 54 / 50 % of the time (dense, conv3, conv2 at n = 1024: 32 / 45 / 48 us in launches of their own), shared memory
+// frames); busy for 51 / 54 / 50 % of the time (dense, conv3, conv2 at n = 1024 under ncu, in launches of their own), shared memory
 // for as much, DRAM 9 / 19 / 31 %.
 constexpr int kWgradThreads = 96 + 256;
 struct WgradShared {
